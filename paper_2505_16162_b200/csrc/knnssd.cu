@@ -92,6 +92,8 @@ struct knnssd_ctx {
     float *pf_rinv = nullptr;                                // RMSNorm scale of the chunk's rows [cap]
     bf16_t *pf_ad = nullptr, *pf_aq = nullptr, *pf_af = nullptr;   // hi / lo planes [2][cap][d], [2][cap][nq], [2][cap][d_ff]
     CUtensorMap pf_map_d{}, pf_map_q{}, pf_map_f{};
+    float *pf_part = nullptr;                                // sums of the pieces of tiles that several CTAs share
+    int *pf_cnt = nullptr;                                   // pieces done so far, zero between launches
 
     // instrumentation
     long long launches = 0;
@@ -365,6 +367,7 @@ void reset_mega_state(knnssd_ctx *c) {
     cudaMemset(c->gabort, 0, sizeof(int));
     cudaMemset(c->attn_cnt, 0, sizeof(int) * pass::MAXM * c->cfg.n_heads);
     cudaMemset(c->amax_cnt, 0, sizeof(int));
+    if (c->pf_cnt) cudaMemset(c->pf_cnt, 0, prefill::PIECE_COUNTERS * sizeof(int));
     c->bar_total = 0;
 }
 
@@ -478,7 +481,7 @@ void free_all(knnssd_ctx *c) {
                     c->anchor_inv_norm, c->cosines, c->amax_v, c->part_ml, c->rope_cs, c->pool_sum, c->inv_freq, c->chain,
                     c->target, c->prompt, c->out_tokens, c->accept_log, c->amax_i, c->flag, c->knn_out, c->state,
                     c->ops_full, c->ops_draft, c->bar, c->gabort, c->attn_cnt, c->amax_cnt, c->mpart_o, c->mamax_v, c->mpart_ml,
-                    c->mamax_i, c->trace, c->xs_x, c->xs_attn, c->xs_act, c->ssp, c->pf_x, c->pf_qkv, c->pf_ad, c->pf_aq, c->pf_af, c->pf_cs, c->pf_rinv,
+                    c->mamax_i, c->trace, c->xs_x, c->xs_attn, c->xs_act, c->ssp, c->pf_x, c->pf_qkv, c->pf_ad, c->pf_aq, c->pf_af, c->pf_cs, c->pf_rinv, c->pf_part, c->pf_cnt,
                     c->samp_p, c->samp_q, c->samp_res};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -512,10 +515,17 @@ bool prefill_tensor(knnssd_ctx *c, int n) {
     cudaStream_t s = c->stream;
     int *err = c->err_word;
     const size_t layer_stride = (size_t)Hkv * g.max_seq * HD;
+    const prefill::GemmScratch scratch{c->pf_part, c->pf_cnt};
     bool ok = true;
     for (int t0 = 0; t0 < n && ok; t0 += cap) {
         const int T = n - t0 < cap ? n - t0 : cap;
         const bool last = t0 + T == n;
+        CUtensorMap map_d = c->pf_map_d, map_q = c->pf_map_q, map_f = c->pf_map_f;
+        if (T < prefill::BM) {               // fewer rows than a tile: boxes of the live rows only
+            const int box = prefill::act_box_rows(T);
+            ok = prefill::make_map(&map_d, c->pf_ad, 2 * (size_t)cap, (size_t)d, box) && prefill::make_map(&map_q, c->pf_aq, 2 * (size_t)cap, (size_t)nq, box) &&
+                 prefill::make_map(&map_f, c->pf_af, 2 * (size_t)cap, (size_t)F, box);
+        }
         prefill::embed_rows_kernel<<<T, 256, 0, s>>>(reinterpret_cast<const bf16_t *>(c->tok_embed), c->prompt + t0, d, c->pf_x);
         prefill::rope_table_kernel<<<T, HD / 2, 0, s>>>(c->inv_freq, t0, c->pf_cs);
         c->launches += 2;
@@ -528,25 +538,25 @@ bool prefill_tensor(knnssd_ctx *c, int n) {
             if (nq % prefill::BOX_N == 0 && nkv % prefill::BOX_N == 0) {
                 // q, k and v in one launch over the stacked units (their columns of the projection buffer are adjacent)
                 const prefill::QkvFuse fuse{c->pf_cs, kc, vc, g.max_seq, t0, HD};
-                ok = ok && prefill::launch_gemm(c->pf_map_d, cap, ly.wq, ly.wk, ldq, d, T, prefill::PF_STORE, c->pf_qkv, ldq, 0, nullptr,
+                ok = ok && prefill::launch_gemm(map_d, scratch, cap, ly.wq, ly.wk, ldq, d, T, prefill::PF_STORE, c->pf_qkv, ldq, 0, nullptr,
                                                 nullptr, 0, err, c->n_sms, s, ly.wv, nq, nkv, &fuse, &heads_done, c->pf_rinv);
             } else {
-                ok = ok && prefill::launch_gemm(c->pf_map_d, cap, ly.wq, nullptr, nq, d, T, prefill::PF_STORE, c->pf_qkv, ldq, 0, nullptr,
+                ok = ok && prefill::launch_gemm(map_d, scratch, cap, ly.wq, nullptr, nq, d, T, prefill::PF_STORE, c->pf_qkv, ldq, 0, nullptr,
                                                 nullptr, 0, err, c->n_sms, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
-                ok = ok && prefill::launch_gemm(c->pf_map_d, cap, ly.wk, nullptr, nkv, d, T, prefill::PF_STORE, c->pf_qkv, ldq, nq, nullptr,
+                ok = ok && prefill::launch_gemm(map_d, scratch, cap, ly.wk, nullptr, nkv, d, T, prefill::PF_STORE, c->pf_qkv, ldq, nq, nullptr,
                                                 nullptr, 0, err, c->n_sms, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
-                ok = ok && prefill::launch_gemm(c->pf_map_d, cap, ly.wv, nullptr, nkv, d, T, prefill::PF_STORE, c->pf_qkv, ldq, nq + nkv,
+                ok = ok && prefill::launch_gemm(map_d, scratch, cap, ly.wv, nullptr, nkv, d, T, prefill::PF_STORE, c->pf_qkv, ldq, nq + nkv,
                                                 nullptr, nullptr, 0, err, c->n_sms, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
             }
             if (!heads_done) prefill::rope_kv_rows_kernel<<<T, 256, 0, s>>>(c->pf_qkv, H, Hkv, HD, c->pf_cs, kc, vc, g.max_seq, t0);
             prefill::attn_prompt_kernel<HD><<<dim3(H, (T + 63) / 64), 128, prefill::attn_smem_bytes<HD>(), s>>>(
                 c->pf_qkv, H, Hkv, kc, vc, g.max_seq, t0, T, c->pf_aq, c->pf_aq + (size_t)cap * nq);
-            ok = ok && prefill::launch_gemm(c->pf_map_q, cap, ly.wo, nullptr, d, nq, T, prefill::PF_ADD, c->pf_x, d, 0, nullptr, nullptr, 0,
+            ok = ok && prefill::launch_gemm(map_q, scratch, cap, ly.wo, nullptr, d, nq, T, prefill::PF_ADD, c->pf_x, d, 0, nullptr, nullptr, 0,
                                             err, c->n_sms, s);
             prefill::norm_split_kernel<<<T, 256, 0, s>>>(c->pf_x, d, ly.mlp_norm, g.rms_eps, c->pf_ad, c->pf_ad + (size_t)cap * d, c->pf_rinv);
-            ok = ok && prefill::launch_gemm(c->pf_map_d, cap, ly.w_gate, ly.w_up, F, d, T, prefill::PF_SWIGLU, nullptr, 0, 0, c->pf_af,
+            ok = ok && prefill::launch_gemm(map_d, scratch, cap, ly.w_gate, ly.w_up, F, d, T, prefill::PF_SWIGLU, nullptr, 0, 0, c->pf_af,
                                             c->pf_af + (size_t)cap * F, F, err, c->n_sms, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
-            ok = ok && prefill::launch_gemm(c->pf_map_f, cap, ly.w_down, nullptr, d, F, T, prefill::PF_ADD, c->pf_x, d, 0, nullptr, nullptr,
+            ok = ok && prefill::launch_gemm(map_f, scratch, cap, ly.w_down, nullptr, d, F, T, prefill::PF_ADD, c->pf_x, d, 0, nullptr, nullptr,
                                             0, err, c->n_sms, s);
             c->launches += ((nq % prefill::BOX_N == 0 && nkv % prefill::BOX_N == 0) ? 9 : 11) - (heads_done ? 1 : 0);
         }
@@ -801,7 +811,10 @@ knnssd_status knnssd_init(const knnssd_config *cfg, const knnssd_weights *w, con
             ok3 &= dev_alloc(&c->pf_ad, 2 * cap * d) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_aq, 2 * cap * nq) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_af, 2 * cap * g.d_ff) == cudaSuccess;
+            ok3 &= dev_alloc(&c->pf_part, (size_t)prefill::MAX_PIECES * prefill::PIECE_FLOATS) == cudaSuccess;
+            ok3 &= dev_alloc(&c->pf_cnt, (size_t)prefill::PIECE_COUNTERS) == cudaSuccess;
             if (!ok3) { cudaGetLastError(); return bail(KNNSSD_ERR_CUDA); }
+            cudaMemsetAsync(c->pf_cnt, 0, prefill::PIECE_COUNTERS * sizeof(int), c->stream);
             cudaMemsetAsync(c->pf_ad, 0, 2 * cap * d * sizeof(bf16_t), c->stream);
             cudaMemsetAsync(c->pf_aq, 0, 2 * cap * nq * sizeof(bf16_t), c->stream);
             cudaMemsetAsync(c->pf_af, 0, 2 * cap * g.d_ff * sizeof(bf16_t), c->stream);
@@ -1347,15 +1360,26 @@ knnssd_status knnssd_gemm_split(const void *W0_dev, const void *W1_dev, int n_ou
     cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev);
     const int cap = (T + prefill::BM - 1) / prefill::BM * prefill::BM;
     bf16_t *planes = nullptr, *outp = nullptr;
+    prefill::GemmScratch scratch{};
     const size_t plane = (size_t)cap * n_in, oplane = (size_t)T * n_out;
-    if (dev_alloc(&planes, 2 * plane) != cudaSuccess) { cudaGetLastError(); return KNNSSD_ERR_CUDA; }
-    if (mode == 2 && dev_alloc(&outp, 2 * oplane) != cudaSuccess) { cudaGetLastError(); cudaFree(planes); return KNNSSD_ERR_CUDA; }
+    auto cleanup = [&]() {
+        void *ptrs[] = {planes, outp, scratch.part, scratch.piece_cnt};
+        for (void *p : ptrs)
+            if (p) cudaFree(p);
+    };
+    if (dev_alloc(&planes, 2 * plane) != cudaSuccess || (mode == 2 && dev_alloc(&outp, 2 * oplane) != cudaSuccess) ||
+        dev_alloc(&scratch.part, (size_t)prefill::MAX_PIECES * prefill::PIECE_FLOATS) != cudaSuccess || dev_alloc(&scratch.piece_cnt, (size_t)prefill::PIECE_COUNTERS) != cudaSuccess) {
+        cudaGetLastError();
+        cleanup();
+        return KNNSSD_ERR_CUDA;
+    }
+    cudaMemsetAsync(scratch.piece_cnt, 0, prefill::PIECE_COUNTERS * sizeof(int), s);
     knnssd_status st = KNNSSD_OK;
     cudaMemsetAsync(planes, 0, 2 * plane * sizeof(bf16_t), s);
     prefill::split_rows_kernel<<<T, 256, 0, s>>>(x_dev, n_in, planes, planes + plane);
     CUtensorMap ta;
-    if (!prefill::make_map(&ta, planes, (size_t)2 * cap, (size_t)n_in, prefill::BM) ||
-        !prefill::launch_gemm(ta, cap, W0_dev, W1_dev, n_out, n_in, T, mode, y_dev, n_out, 0, outp, outp ? outp + oplane : nullptr,
+    if (!prefill::make_map(&ta, planes, (size_t)2 * cap, (size_t)n_in, prefill::act_box_rows(T)) ||
+        !prefill::launch_gemm(ta, scratch, cap, W0_dev, W1_dev, n_out, n_in, T, mode, y_dev, n_out, 0, outp, outp ? outp + oplane : nullptr,
                               n_out, stream_err_ptr(), n_sms, s))
         st = KNNSSD_ERR_CUDA;
     if (st == KNNSSD_OK && mode == 2) prefill::join_planes_kernel<<<T, 256, 0, s>>>(outp, outp + oplane, n_out, y_dev);
@@ -1367,8 +1391,7 @@ knnssd_status knnssd_gemm_split(const void *W0_dev, const void *W1_dev, int n_ou
         if (cudaMemcpy(&code, stream_err_ptr(), sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) st = KNNSSD_ERR_CUDA;
         else if (code) { cudaMemset(stream_err_ptr(), 0, sizeof(int)); st = KNNSSD_ERR_TIMEOUT; }
     }
-    cudaFree(planes);
-    if (outp) cudaFree(outp);
+    cleanup();
     return st;
 }
 

@@ -34,14 +34,20 @@ constexpr int BM = 128;                               // tokens per tile: rows o
 constexpr int BN_MAX = 256;                           // most accumulator columns per tile (a launch picks 64, 128, 192 or 256)
 constexpr int BOX_N = 64;                             // weight rows per TMA box
 constexpr int BK = 64;                                // input columns per stage: 128 bytes of bf16 = one swizzle row
-constexpr int STAGES = 3;
-constexpr int A_BYTES = BM * BK * 2;                  // one term of the activation tile
-constexpr int B_BYTES = BN_MAX * BK * 2;
-constexpr int STAGE_BYTES = 2 * A_BYTES + B_BYTES;    // hi plane, lo plane, weights
+// The ring of stages.  A stage is what a k-block of the launch needs: two boxes of a_rows activation rows (hi and lo plane)
+// and bn weight rows, 64 KB at 128 rows and 256 columns (three stages), 56 KB at 192 columns (four).  A launch takes no
+// more shared memory than its stages: the add epilogue reads 32 bytes of a row at a time and lives on what is left as L1.
+constexpr int RING_BYTES = 224 * 1024;
+constexpr int MAX_STAGES = 10;
+__host__ __device__ constexpr int ring_stages(int a_rows, int bn) {
+    return RING_BYTES / ((2 * a_rows + bn) * BK * 2) < MAX_STAGES ? RING_BYTES / ((2 * a_rows + bn) * BK * 2) : MAX_STAGES;
+}
 constexpr int TMEM_COLS = 512;                        // columns of tensor memory a CTA takes: two accumulators of BN_MAX columns
 constexpr int CHUNK_KB = 8;                           // k-blocks accumulated in tensor memory before the sum moves to registers
 constexpr int GEMM_THREADS = 320;                     // warp 0: TMA; warp 1: MMA issue + tensor-memory owner; warps 2..9: epilogue
-constexpr int GEMM_SMEM = STAGES * STAGE_BYTES + 1024 + 128;   // + slack to align the tiles to 1024 bytes + barriers
+__host__ __device__ constexpr int gemm_smem(int a_rows, int bn) {     // + slack to align the tiles to 1024 bytes + barriers
+    return ring_stages(a_rows, bn) * (2 * a_rows + bn) * BK * 2 + 1024 + 256;
+}
 constexpr unsigned WAIT_LIMIT = 4000000u;           // polls of one wait (a whole tile takes well under a millisecond)
 
 enum { PF_STORE = 0, PF_ADD = 1, PF_SWIGLU = 2, PF_QKV = 3 };
@@ -57,7 +63,13 @@ struct GemmArgs {
     bf16_t *out_lo;
     int ldo;
     int *err;          // set non-zero if a bounded wait gave up
-    int tiles_x, tiles_y;   // gemm_split_kernel: row tiles and column tiles of the launch (its CTAs walk tile = ty tiles_x + tx)
+    int tiles_x, tiles_y;   // row tiles and column tiles of the launch (tile = ty tiles_x + tx)
+    int box;           // weight rows per box: BOX_N, or 128 where tiles and matrices allow it (a box costs the copy engine ~0.13 us
+                       // whatever its height: 0.75 -> 0.6 us per k-block of 256 columns for the copies alone)
+    int a_rows;        // rows of an activation box (the maps' box height): BM, or T rounded up to 8 where T < BM
+    int whole;         // tiles [0, whole) are done whole by one CTA each, the others in pieces (see Jobs below)
+    float *part;       // the chunk sums of the tiles done in pieces, [tiles_x tiles_y - whole][chunks][PIECE_FLOATS]
+    int *piece_cnt;    // [tiles done in pieces][8 epilogue warps], zero between launches
     int nA, nB;        // STORE over stacked matrices (q, k, v in one launch): units [0, nA) are rows of map tb0,
                        // [nA, nA + nB) rows of tb1, the rest rows of tb2; all multiples of BOX_N.  One matrix: nA = N
     // PF_QKV (stacked q, k, v; head dimension 128, bn = 256: an epilogue thread holds one head of its token): the q
@@ -139,9 +151,72 @@ __device__ __forceinline__ bool pf_wait(uint64_t *b, uint32_t parity, volatile i
     return true;
 }
 
+__device__ __forceinline__ int ld_acquire_int(const int *p) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// 32 bytes, a sector: in one access at a 32-byte boundary (whole), else in two at a 16-byte boundary.
+__device__ __forceinline__ void ld_sector(const float *p, float (&v)[8], bool whole) {
+    if (whole) {
+        asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]) : "l"(p) : "memory");
+    } else {
+        const float4 a = *reinterpret_cast<const float4 *>(p), b = *reinterpret_cast<const float4 *>(p + 4);
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    }
+}
+__device__ __forceinline__ void st_sector(float *p, const float (&v)[8], bool whole) {
+    if (whole) {
+        asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]),
+                     "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]) : "memory");
+    } else {
+        *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+        *reinterpret_cast<float4 *>(p + 4) = make_float4(v[4], v[5], v[6], v[7]);
+    }
+}
+
 __device__ __forceinline__ uint32_t pack_bf16(uint32_t lo16, uint32_t hi16) { return lo16 | (hi16 << 16); }
 
-// One CTA per tile of 128 tokens x bn accumulator columns.  EPI = PF_SWIGLU: columns [0, bn / 2) are units n0 .. of
+// How a launch's work is dealt out to its CTAs (one per SM).  Tiles [0, whole) go round: CTA c takes tiles c, c + G, ..,
+// so that all CTAs are at the same k-blocks of neighbouring tiles and share them through L2 (walking a contiguous run of
+// tiles each instead cost 1.05 us per k-block against 0.81: the weights of all column tiles in flight at once).  The
+// chunks (CHUNK_KB k-blocks) of the tiles that are left, fewer than the CTAs, are dealt out evenly, CTA c of P getting
+// chunks [c U / P, (c + 1) U / P): a last round that would leave most of the chip idle takes the time its work takes.
+// A piece's chunk sums go to `part` one by one; once all of a tile's are there (every CTA has left all of its
+// own before it waits for others, and nothing it waits for waits for it; the wait is bounded) the tile's CTAs take an eighth
+// of its columns each and add them up from the first chunk to the last, the order of a tile done whole: a row's
+// numbers do not depend on how the launch was dealt out.  Epilogue warp w of every CTA has the same 32 rows x half of
+// the columns of a tile, so counting and waiting are per warp.
+struct Jobs {
+    int G, P, cta, whole, nchunks, n_whole, r0;      // P: the CTAs that get pieces, one chunk each at least
+    long long units, u0, u1;
+    __device__ __forceinline__ Jobs(const GemmArgs &g) : G(gridDim.x), cta(blockIdx.x), whole(g.whole) {
+        nchunks = (g.K / BK + CHUNK_KB - 1) / CHUNK_KB;
+        n_whole = cta < whole ? (whole - cta + G - 1) / G : 0;
+        units = (long long)(g.tiles_x * g.tiles_y - whole) * nchunks;
+        P = (int)min((long long)G, units);
+        u0 = cta < P ? units * cta / P : 0;
+        u1 = cta < P ? units * (cta + 1) / P : 0;
+        r0 = (int)(u0 / nchunks);
+    }
+    // job i of this CTA: chunks [c0, c1) of a tile; false when there is none
+    __device__ __forceinline__ bool get(int i, int &tile, int &c0, int &c1) const {
+        if (i < n_whole) { tile = cta + i * G; c0 = 0; c1 = nchunks; return true; }
+        const int r = r0 + i - n_whole;
+        const long long first = (long long)r * nchunks;
+        if (first >= u1 || u0 >= u1) return false;
+        tile = whole + r;
+        c0 = first < u0 ? (int)(u0 - first) : 0;
+        c1 = (int)min((long long)nchunks, u1 - first);
+        return true;
+    }
+    __device__ __forceinline__ int cta_of(long long u) const { return (int)(((u + 1) * P - 1) / units); }   // the CTA that has unit u
+};
+constexpr int PIECE_FLOATS = BM * BN_MAX;      // a chunk's sums, by register group and thread (coalesced): 32 x 256 float4
+
+// Tiles of 128 tokens x bn accumulator columns, dealt out to one CTA per SM (Jobs).  EPI = PF_SWIGLU: columns [0, bn / 2) are units n0 .. of
 // the gate matrix (map tb0) and columns [bn / 2, bn) the same units of the up matrix (map tb1); otherwise the columns
 // are units n0 .. n0 + bn - 1 of one matrix (tb0 = tb1).  ta covers both activation planes: rows [0, Tpad) the hi
 // terms, rows [Tpad, 2 Tpad) the lo terms.  The weight maps are read in boxes of BOX_N rows.
@@ -158,23 +233,23 @@ template <int EPI>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb0,
                   const __grid_constant__ CUtensorMap tb1, const __grid_constant__ CUtensorMap tb2, GemmArgs g, int Tpad) {
+    const int bn = g.bn, per = EPI == PF_SWIGLU ? bn / 2 : bn;      // units of a matrix per tile
+    const int a_bytes = g.a_rows * BK * 2, stage_bytes = 2 * a_bytes + bn * BK * 2, stages = ring_stages(g.a_rows, bn);
     extern __shared__ unsigned char pf_smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(pf_smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem + STAGES * STAGE_BYTES);
-    uint64_t *empty = full + STAGES;
-    uint64_t *acc_full = empty + STAGES;          // [2]: a chunk's sum is complete in accumulator b
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem + stages * stage_bytes);
+    uint64_t *empty = full + MAX_STAGES;
+    uint64_t *acc_full = empty + MAX_STAGES;      // [2]: a chunk's sum is complete in accumulator b
     uint64_t *acc_empty = acc_full + 2;           // [2]: the epilogue warps have moved accumulator b's sum out
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + 2);
     volatile int *cta_abort = reinterpret_cast<volatile int *>(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int bn = g.bn, per = EPI == PF_SWIGLU ? bn / 2 : bn;      // units of a matrix per tile
-    // tiles: row tile fastest (tile = ty * tiles_x + tx); this CTA takes tiles blockIdx.x, + gridDim.x, ..
-    const int n_tiles = g.tiles_x * g.tiles_y;
-    const int nkb = g.K / BK, nchunks = (nkb + CHUNK_KB - 1) / CHUNK_KB;
+    const Jobs jobs(g);                                              // tiles: row tile fastest (tile = ty * tiles_x + tx)
+    const int nkb = g.K / BK, nchunks = jobs.nchunks;
     constexpr int EPI_WARPS = GEMM_THREADS / 32 - 2;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+        for (int s = 0; s < stages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], EPI_WARPS); }
         *cta_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -192,20 +267,18 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant_
     if (warp == 0) {
         if (lane == 0) {
             // ---- TMA producer: a stage is refilled once the MMAs that read it have finished ----
-            int armed = 0;                   // k-blocks armed so far, over all of this CTA's tiles: stage and phase follow it
+            int armed = 0, s = 0;            // k-blocks armed so far, over all of this CTA's jobs; the next one's stage and phase
+            uint32_t ph = 0;
             bool ok = true;
-            for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
-            const int t0 = (tile % g.tiles_x) * BM, n0 = (tile / g.tiles_x) * per;
-            for (int kb = 0; kb < nkb; ++kb) {
-                const int s = armed % STAGES;
-                const uint32_t ph = (uint32_t)(armed / STAGES) & 1u;
+            for (int i = 0, tile, c_begin, c_end; ok && jobs.get(i, tile, c_begin, c_end); ++i) {
+            const int t0 = (tile % g.tiles_x) * BM, n0 = (tile / g.tiles_x) * per, kb1 = min(nkb, c_end * CHUNK_KB);
+            for (int kb = c_begin * CHUNK_KB; kb < kb1; ++kb) {
                 if (!pf_wait(&empty[s], ph ^ 1u, cta_abort, g.err, 21)) { ok = false; break; }
-                unsigned char *st = smem + s * STAGE_BYTES;
-                stream::mbar_expect_tx(&full[s], 2 * A_BYTES + bn * BK * 2);
+                unsigned char *st = smem + s * stage_bytes;
+                stream::mbar_expect_tx(&full[s], stage_bytes);
                 tma_load_2d(st, &ta, kb * BK, t0, &full[s]);
-                tma_load_2d(st + A_BYTES, &ta, kb * BK, Tpad + t0, &full[s]);
-                for (int j = 0; j < bn / BOX_N; ++j) {
-                    const int r = j * BOX_N;                 // accumulator column the box starts at
+                tma_load_2d(st + a_bytes, &ta, kb * BK, Tpad + t0, &full[s]);
+                for (int r = 0; r < bn; r += g.box) {        // accumulator column the box starts at
                     const bool second = EPI == PF_SWIGLU && r >= per;
                     const CUtensorMap *wm = second ? &tb1 : &tb0;
                     int wrow = n0 + (second ? r - per : r);
@@ -213,16 +286,17 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant_
                         wm = &tb1; wrow -= g.nA;
                         if (wrow >= g.nB) { wm = &tb2; wrow -= g.nB; }
                     }
-                    tma_load_2d(st + 2 * A_BYTES + r * BK * 2, wm, kb * BK, wrow, &full[s]);
+                    tma_load_2d(st + 2 * a_bytes + r * BK * 2, wm, kb * BK, wrow, &full[s]);
                 }
                 ++armed;
+                if (++s == stages) { s = 0; ph ^= 1u; }
             }
             }
             if (*cta_abort) {
                 // copies in flight land in this CTA's shared memory: let them finish before the CTA goes away
-                for (int kb = (armed > STAGES ? armed - STAGES : 0); kb < armed; ++kb) {
+                for (int kb = (armed > stages ? armed - stages : 0); kb < armed; ++kb) {
                     unsigned spins = 0;
-                    while (!mbar_try_wait(&full[kb % STAGES], (uint32_t)(kb / STAGES) & 1u) && ++spins < WAIT_LIMIT) {}
+                    while (!mbar_try_wait(&full[kb % stages], (uint32_t)(kb / stages) & 1u) && ++spins < WAIT_LIMIT) {}
                 }
             }
         }
@@ -231,22 +305,21 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant_
             // ---- MMA issue: chunk c goes to accumulator c & 1; per stage 4 k-steps of 16 columns, hi and lo term ----
             bool ok = true;
             const uint32_t idesc = umma_idesc(bn);
-            int kbg = 0, cg = 0;             // k-blocks and chunks issued so far, over all of this CTA's tiles
-            for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x)
-            for (int c = 0; c < nchunks && ok; ++c, ++cg) {
+            int cg = 0, s = 0;               // chunks issued so far, over all of this CTA's jobs; stage and phase of the next k-block
+            uint32_t ph = 0;
+            for (int i = 0, tile, c_begin, c_end; ok && jobs.get(i, tile, c_begin, c_end); ++i)
+            for (int c = c_begin; c < c_end && ok; ++c, ++cg) {
                 const int b = cg & 1;
                 ok = pf_wait(&acc_empty[b], ((uint32_t)(cg >> 1) & 1u) ^ 1u, cta_abort, g.err, 24);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t acc_addr = tmem + (uint32_t)(b * BN_MAX);
                 const int kb1 = min(nkb, (c + 1) * CHUNK_KB);
-                for (int kb = c * CHUNK_KB; kb < kb1 && ok; ++kb, ++kbg) {
-                    const int s = kbg % STAGES;
-                    const uint32_t ph = (uint32_t)(kbg / STAGES) & 1u;
+                for (int kb = c * CHUNK_KB; kb < kb1 && ok; ++kb) {
                     ok = pf_wait(&full[s], ph, cta_abort, g.err, 22);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t a_hi = smem_u32(smem + s * STAGE_BYTES), a_lo = a_hi + A_BYTES, bw = a_hi + 2 * A_BYTES;
+                    const uint32_t a_hi = smem_u32(smem + s * stage_bytes), a_lo = a_hi + a_bytes, bw = a_hi + 2 * a_bytes;   // fewer rows than a tile's: the rest of its rows is what follows, and meets no live token
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k) {
                         const uint32_t accum = (kb != c * CHUNK_KB || k != 0) ? 1u : 0u;
@@ -255,6 +328,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant_
                         umma_bf16(acc_addr, umma_desc(a_lo + 32 * k), db, idesc, 1u);
                     }
                     umma_commit(&empty[s]);
+                    if (++s == stages) { s = 0; ph ^= 1u; }
                 }
                 umma_commit(&acc_full[b]);     // on the abort path too: it releases the epilogue warps' wait
             }
@@ -268,6 +342,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant_
         const int q = warp & 3, hsel = (warp - 2) >> 2;
         const uint32_t trow = tmem + ((uint32_t)(32 * q) << 16);
         const int half = bn / 2, qtr = bn / 4;
+        const bool y32 = (reinterpret_cast<uintptr_t>(g.y) & 31u) == 0;      // ldy, col0 and the columns are multiples of 8
         // tile column of register group gi (32 columns), or -1 if the group is not in use
         auto group_col = [&](int gi) -> int {
             if (EPI == PF_SWIGLU) {
@@ -279,13 +354,91 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant_
         };
         bool ok = true;
         int cg = 0;                          // chunks taken so far, over all of this CTA's tiles
-        for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
-        const int t0 = (tile % g.tiles_x) * BM, n0 = (tile / g.tiles_x) * per;
-        const int t = t0 + 32 * q + lane;
+        const int et = threadIdx.x - 64;     // this thread among the epilogue threads
+        // the sums of piece r's chunk c as this thread's float4s, 256 apart; its counter
+        auto part_of = [&](int r, int c) { return reinterpret_cast<float4 *>(g.part + ((size_t)r * nchunks + c) * PIECE_FLOATS) + et; };
+        auto counter = [&](int r) { return g.piece_cnt + (size_t)r * EPI_WARPS + (warp - 2); };
+        // What becomes of 16 sums of token t of a tile: register k8 .. k8 + 7 in v[0 .. 7], 64 + k8 .. in v[8 .. 15] (k8 = 8 k).
+        // SwiGLU: gate and up columns of eight units; q / k / v heads: eight pairs (j, j + 64) of one head; else columns.
+        auto finish = [&](int tile, int t, int k8, float (&v)[16]) {
+            const int n0 = (tile / g.tiles_x) * per;
+            if (g.row_scale) {
+                const float rs = g.row_scale[t];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) v[i] *= rs;
+            }
+            if (EPI == PF_SWIGLU) {
+                const int u = n0 + hsel * qtr + k8;
+                if (k8 >= qtr || u >= g.N) return;
+                uint32_t hi[4], lo[4];
+#pragma unroll
+                for (int i = 0; i < 8; i += 2) {
+                    uint32_t h2[2], l2[2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const float gt = v[i + e], up = v[8 + i + e];
+                        const float a = gt / (1.0f + expf(-gt)) * up;
+                        h2[e] = float_to_bf16_rne(a);
+                        l2[e] = float_to_bf16_rne(a - __uint_as_float(h2[e] << 16));
+                    }
+                    hi[i >> 1] = pack_bf16(h2[0], h2[1]);
+                    lo[i >> 1] = pack_bf16(l2[0], l2[1]);
+                }
+                *reinterpret_cast<uint4 *>(g.out_hi + (size_t)t * g.ldo + u) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                *reinterpret_cast<uint4 *>(g.out_lo + (size_t)t * g.ldo + u) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+            } else if (EPI == PF_QKV) {
+                const int u0 = n0 + hsel * 128;                  // the head's first unit of the stacked q / k / v units
+                if (u0 >= g.N) return;
+                if (u0 < g.nA + g.nB) {                          // a q or a k head: rotary embedding
+                    const float2 *cs = g.rope + (size_t)t * 64 + k8;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const float2 c = cs[i];
+                        const float a = v[i], b = v[8 + i];
+                        v[i] = a * c.x - b * c.y;
+                        v[8 + i] = b * c.x + a * c.y;
+                    }
+                }
+                const bool is_k = u0 < g.nA + g.nB;
+                const int kvh = (u0 - g.nA - (is_k ? 0 : g.nB)) >> 7;
+#pragma unroll
+                for (int e = 0; e < 16; e += 8) {
+                    if (u0 < g.nA) {
+                        float *yp = g.y + (size_t)t * g.ldy + g.col0 + u0 + 8 * e + k8;
+                        float o[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) o[i] = v[e + i];
+                        st_sector(yp, o, y32);
+                    } else {
+                        bf16_t *dst = (is_k ? g.kc : g.vc) + ((size_t)kvh * g.max_seq + g.pos0 + t) * 128 + 8 * e + k8;
+                        uint32_t w[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) w[i] = pack_bf16(float_to_bf16_rne(v[e + 2 * i]), float_to_bf16_rne(v[e + 2 * i + 1]));
+                        *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int e = 0; e < 16; e += 8) {
+                    const int r = 8 * e + k8, n = n0 + hsel * half + r;
+                    if (r >= half || n >= g.N) continue;         // N is a multiple of 8
+                    float *yp = g.y + (size_t)t * g.ldy + g.col0 + n;
+                    float o[8], x[8];
+                    if (EPI == PF_ADD) ld_sector(yp, x, y32);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) o[i] = EPI == PF_ADD ? v[e + i] + x[i] : v[e + i];
+                    st_sector(yp, o, y32);
+                }
+            }
+        };
+        int tile, c_begin, c_end, i = 0;
+        for (; ok && jobs.get(i, tile, c_begin, c_end); ++i) {
+        const int t = (tile % g.tiles_x) * BM + 32 * q + lane;
+        const bool piece = c_end - c_begin < nchunks;
         float acc[128];
 #pragma unroll
         for (int i = 0; i < 128; ++i) acc[i] = 0.f;
-        for (int c = 0; c < nchunks && ok; ++c, ++cg) {
+        for (int c = c_begin; c < c_end && ok; ++c, ++cg) {
             const int b = cg & 1;
             // the loads from tensor memory are warp-wide: the warp goes on only if all of its threads saw the accumulator
             ok = __all_sync(0xffffffffu, pf_wait(&acc_full[b], (uint32_t)(cg >> 1) & 1u, cta_abort, g.err, 23) && !*cta_abort);
@@ -297,324 +450,94 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant_
                 if (col >= 0) {                          // warp-uniform
                     float v[32];
                     tmem_ld32(trow + (uint32_t)(b * BN_MAX + col), v);
+                    if (piece) {                         // warp-uniform
+                        if (t < g.T) {
+                            float4 *dst = part_of(tile - g.whole, c) + 8 * gi * 256;
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) acc[32 * gi + i] += v[i];
+                            for (int i = 0; i < 8; ++i) __stcg(dst + i * 256, make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
+                        }
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) acc[32 * gi + i] += v[i];
+                    }
                 }
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) stream::mbar_arrive(&acc_empty[b]);
         }
-        if (ok && t < g.T && g.row_scale) {
-            const float rs = g.row_scale[t];
-#pragma unroll
-            for (int i = 0; i < 128; ++i) acc[i] *= rs;
-        }
-        if (ok && t < g.T) {
-            if (EPI == PF_SWIGLU) {
-#pragma unroll
-                for (int gg = 0; gg < 2; ++gg) {
-                    const int c0 = hsel * qtr + 32 * gg;         // unit offset within the tile
-                    if (32 * gg >= qtr || n0 + c0 >= g.N) continue;
-                    uint32_t hi[16], lo[16];
-#pragma unroll
-                    for (int i = 0; i < 32; i += 2) {
-                        uint32_t h2[2], l2[2];
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const float gt = acc[32 * gg + i + e], up = acc[64 + 32 * gg + i + e];
-                            const float a = gt / (1.0f + expf(-gt)) * up;
-                            h2[e] = float_to_bf16_rne(a);
-                            l2[e] = float_to_bf16_rne(a - __uint_as_float(h2[e] << 16));
-                        }
-                        hi[i >> 1] = pack_bf16(h2[0], h2[1]);
-                        lo[i >> 1] = pack_bf16(l2[0], l2[1]);
-                    }
-                    bf16_t *ph = g.out_hi + (size_t)t * g.ldo + n0 + c0, *pl = g.out_lo + (size_t)t * g.ldo + n0 + c0;
-                    if (n0 + c0 + 32 <= g.N) {
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            reinterpret_cast<uint4 *>(ph)[i] = make_uint4(hi[4 * i], hi[4 * i + 1], hi[4 * i + 2], hi[4 * i + 3]);
-                            reinterpret_cast<uint4 *>(pl)[i] = make_uint4(lo[4 * i], lo[4 * i + 1], lo[4 * i + 2], lo[4 * i + 3]);
-                        }
-                    } else {
-                        for (int i = 0; n0 + c0 + i < g.N; ++i) {
-                            ph[i] = (bf16_t)((hi[i >> 1] >> (16 * (i & 1))) & 0xFFFFu);
-                            pl[i] = (bf16_t)((lo[i >> 1] >> (16 * (i & 1))) & 0xFFFFu);
-                        }
-                    }
-                }
-            } else if (EPI == PF_QKV) {
-                // acc[j] = unit u0 + j of the stacked q / k / v units: one head of token t
-                const int u0 = n0 + hsel * 128;
-                if (u0 < g.N) {
-                    if (u0 < g.nA + g.nB) {                     // a q or a k head: rotary embedding, pairs (i, i + 64)
-                        const float2 *cs = g.rope + (size_t)t * 64;
-#pragma unroll
-                        for (int i = 0; i < 64; ++i) {
-                            const float2 c = cs[i];
-                            const float a = acc[i], b = acc[64 + i];
-                            acc[i] = a * c.x - b * c.y;
-                            acc[64 + i] = b * c.x + a * c.y;
-                        }
-                    }
-                    if (u0 < g.nA) {
-                        float *yp = g.y + (size_t)t * g.ldy + g.col0 + u0;
-#pragma unroll
-                        for (int i = 0; i < 128; i += 4)
-                            *reinterpret_cast<float4 *>(yp + i) = make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
-                    } else {
-                        const bool is_k = u0 < g.nA + g.nB;
-                        const int kvh = (u0 - g.nA - (is_k ? 0 : g.nB)) >> 7;
-                        bf16_t *dst = (is_k ? g.kc : g.vc) + ((size_t)kvh * g.max_seq + g.pos0 + t) * 128;
-#pragma unroll
-                        for (int i = 0; i < 128; i += 8) {
-                            uint32_t w[4];
-#pragma unroll
-                            for (int e = 0; e < 4; ++e)
-                                w[e] = pack_bf16(float_to_bf16_rne(acc[i + 2 * e]), float_to_bf16_rne(acc[i + 2 * e + 1]));
-                            *reinterpret_cast<uint4 *>(dst + i) = make_uint4(w[0], w[1], w[2], w[3]);
-                        }
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int gi = 0; gi < 4; ++gi) {
-                    const int c0 = hsel * half + 32 * gi;
-                    if (32 * gi >= half || n0 + c0 >= g.N) continue;
-                    float *yp = g.y + (size_t)t * g.ldy + g.col0 + n0 + c0;
-                    if (n0 + c0 + 32 <= g.N) {
-#pragma unroll
-                        for (int i = 0; i < 32; i += 4) {
-                            float4 o = make_float4(acc[32 * gi + i], acc[32 * gi + i + 1], acc[32 * gi + i + 2], acc[32 * gi + i + 3]);
-                            if (EPI == PF_ADD) {
-                                const float4 x = *reinterpret_cast<const float4 *>(yp + i);
-                                o.x += x.x; o.y += x.y; o.z += x.z; o.w += x.w;
-                            }
-                            *reinterpret_cast<float4 *>(yp + i) = o;
-                        }
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < 32; ++i)
-                            if (n0 + c0 + i < g.N) yp[i] = EPI == PF_ADD ? yp[i] + acc[32 * gi + i] : acc[32 * gi + i];
-                    }
-                }
-            }
-        }
-        }                                    // next tile: its first chunks are already accumulating in tensor memory
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) {
-        tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
-    }
-}
-
-// 16 consecutive accumulator columns of this thread's lane.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
-          "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// The same contraction on tiles of 128 tokens x 320 units (store and add epilogues), for the maps whose unit count
-// makes 320-wide tiles fill the SMs better (5120 units x 1024 rows: 128 tiles = one round, where 216 tiles of 192 columns
-// take two).  Two double-buffered accumulators of 320 columns do not fit the 512 columns of tensor memory, so the tile
-// is cut into two halves of 160 columns whose chunks are staggered by half a chunk, and three accumulators of 160
-// columns rotate between them: half A's chunk i covers k-blocks [8 i, 8 i + 8) in accumulator i mod 3, half B's chunk j
-// covers [8 j - 4, 8 j + 4) (its first one [0, 4)) in accumulator (j + 1) mod 3.  When a chunk ends, its half goes on
-// in the accumulator the other half left four k-blocks earlier (moved out by then), and the four epilogue warps of
-// the half move the finished sum into their registers while both halves keep the tensor core busy.
-// Same operand staging, maps and arguments as gemm_split_kernel with bn = 320.
-constexpr int WIDE_BN = 320, WIDE_HALF = 160;
-constexpr int WIDE_STAGE = 2 * A_BYTES + WIDE_BN * BK * 2;
-constexpr int WIDE_SMEM = STAGES * WIDE_STAGE + 1024 + 128;
-
-// Accumulator and how many times it was used before: half 0 chunk i / half 1 chunk j (see above).
-__device__ __forceinline__ void wide_slot(int half, int i, int &buf, int &use) {
-    if (half == 0) { buf = i % 3; use = 2 * (i / 3) + (buf == 0 ? 0 : 1); }
-    else { buf = (i + 1) % 3; use = 2 * (i / 3) + (buf == 0 ? 1 : 0); }
-}
-
-template <int EPI>
-__global__ void __launch_bounds__(GEMM_THREADS, 1)
-gemm_wide_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb0,
-                 const __grid_constant__ CUtensorMap tb1, const __grid_constant__ CUtensorMap tb2, GemmArgs g, int Tpad) {
-    static_assert(EPI == PF_STORE || EPI == PF_ADD, "wide tiles: store and add epilogues");
-    extern __shared__ unsigned char pf_smem_raw[];
-    unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(pf_smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem + STAGES * WIDE_STAGE);
-    uint64_t *empty = full + STAGES;
-    uint64_t *acc_full = empty + STAGES;          // [3]: a chunk's sum is complete in accumulator b
-    uint64_t *acc_empty = acc_full + 3;           // [3]: the half's epilogue warps have moved accumulator b's sum out
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + 3);
-    volatile int *cta_abort = reinterpret_cast<volatile int *>(tmem_slot + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int t0 = blockIdx.x * BM;
-    const int n0 = blockIdx.y * WIDE_BN;
-    const int nkb = g.K / BK;
-    // chunks per half: A [0, 8), [8, 16), ..; B [0, 4), [4, 12), ..
-    const int n_chunks[2] = {(nkb + CHUNK_KB - 1) / CHUNK_KB, nkb <= CHUNK_KB / 2 ? 1 : 1 + (nkb - CHUNK_KB / 2 + CHUNK_KB - 1) / CHUNK_KB};
-    constexpr int HALF_WARPS = (GEMM_THREADS / 32 - 2) / 2;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-        for (int b = 0; b < 3; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], HALF_WARPS); }
-        *cta_abort = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(TMEM_COLS) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
-
-    if (warp == 0) {
-        if (lane == 0) {
-            // ---- TMA producer ----
-            int armed = 0;
-            for (int kb = 0; kb < nkb; ++kb) {
-                const int s = kb % STAGES;
-                const uint32_t ph = (uint32_t)(kb / STAGES) & 1u;
-                if (!pf_wait(&empty[s], ph ^ 1u, cta_abort, g.err, 31)) break;
-                unsigned char *st = smem + s * WIDE_STAGE;
-                stream::mbar_expect_tx(&full[s], WIDE_STAGE);
-                tma_load_2d(st, &ta, kb * BK, t0, &full[s]);
-                tma_load_2d(st + A_BYTES, &ta, kb * BK, Tpad + t0, &full[s]);
-#pragma unroll
-                for (int j = 0; j < WIDE_BN / BOX_N; ++j) {
-                    const CUtensorMap *wm = &tb0;
-                    int wrow = n0 + j * BOX_N;
-                    if (wrow >= g.nA) {                              // stacked matrices: the box lies in the second or third one
-                        wm = &tb1; wrow -= g.nA;
-                        if (wrow >= g.nB) { wm = &tb2; wrow -= g.nB; }
-                    }
-                    tma_load_2d(st + 2 * A_BYTES + j * BOX_N * BK * 2, wm, kb * BK, wrow, &full[s]);
-                }
-                armed = kb + 1;
-            }
-            if (*cta_abort) {
-                for (int kb = (armed > STAGES ? armed - STAGES : 0); kb < armed; ++kb) {
-                    unsigned spins = 0;
-                    while (!mbar_try_wait(&full[kb % STAGES], (uint32_t)(kb / STAGES) & 1u) && ++spins < WAIT_LIMIT) {}
-                }
-            }
-        }
-    } else if (warp == 1) {
-        if (lane == 0) {
-            // ---- MMA issue: per stage 4 k-steps x (hi, lo) x (half A, half B) ----
-            bool ok = true;
-            const uint32_t idesc = umma_idesc(WIDE_HALF);
-            int cur[2] = {-1, -1};                 // chunk each half is in
-            uint32_t acc_addr[2] = {0u, 0u};
-            int cur_buf[2] = {0, 0};
-            for (int kb = 0; kb < nkb && ok; ++kb) {
-                // chunk boundaries: A at kb = 0, 8, 16, ..; B at kb = 0, 4, 12, 20, ..
-                bool fresh[2] = {false, false};
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const bool boundary = h == 0 ? (kb % CHUNK_KB == 0) : (kb == 0 || kb % CHUNK_KB == CHUNK_KB / 2);
-                    if (!boundary || !ok) continue;
-                    if (cur[h] >= 0) umma_commit(&acc_full[cur_buf[h]]);
-                    ++cur[h];
-                    int buf, use;
-                    wide_slot(h, cur[h], buf, use);
-                    ok = pf_wait(&acc_empty[buf], ((uint32_t)use & 1u) ^ 1u, cta_abort, g.err, 34);
-                    cur_buf[h] = buf;
-                    acc_addr[h] = tmem + (uint32_t)(buf * WIDE_HALF);
-                    fresh[h] = true;
-                }
-                if (!ok) break;
-                tc_fence_after();
-                const int s = kb % STAGES;
-                const uint32_t ph = (uint32_t)(kb / STAGES) & 1u;
-                ok = pf_wait(&full[s], ph, cta_abort, g.err, 32);
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t a_hi = smem_u32(smem + s * WIDE_STAGE), a_lo = a_hi + A_BYTES, bw = a_hi + 2 * A_BYTES;
-#pragma unroll
-                for (int k = 0; k < BK / 16; ++k) {
-                    const uint64_t dah = umma_desc(a_hi + 32 * k), dal = umma_desc(a_lo + 32 * k);
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const uint64_t db = umma_desc(bw + h * (WIDE_HALF * BK * 2) + 32 * k);
-                        umma_bf16(acc_addr[h], dah, db, idesc, (fresh[h] && k == 0) ? 0u : 1u);
-                        umma_bf16(acc_addr[h], dal, db, idesc, 1u);
-                    }
-                }
-                umma_commit(&empty[s]);
-            }
-            // the last chunks; on the abort path every accumulator is signalled so that no epilogue warp keeps waiting
-            if (ok) { umma_commit(&acc_full[cur_buf[0]]); umma_commit(&acc_full[cur_buf[1]]); }
-            else { umma_commit(&acc_full[0]); umma_commit(&acc_full[1]); umma_commit(&acc_full[2]); }
-        }
-    } else {
-        // ---- epilogue warps: warp w reads lanes 32 (w % 4) .. + 31 = tokens t0 + 32 (w % 4) + lane; warps 2..5 own half A
-        //      (tile columns 0 .. 159), warps 6..9 half B; acc[] = this thread's running sums over its half's chunks (the
-        //      compiler keeps a few dozen of the 160 in local memory: touched once per chunk) ----
-        const int q = warp & 3, hsel = (warp - 2) >> 2;
-        const int t = t0 + 32 * q + lane;
-        const uint32_t trow = tmem + ((uint32_t)(32 * q) << 16);
-        float acc[WIDE_HALF];
-#pragma unroll
-        for (int i = 0; i < WIDE_HALF; ++i) acc[i] = 0.f;
-        bool ok = true;
-        for (int c = 0; c < n_chunks[hsel] && ok; ++c) {
-            int buf, use;
-            wide_slot(hsel, c, buf, use);
-            ok = __all_sync(0xffffffffu, pf_wait(&acc_full[buf], (uint32_t)use & 1u, cta_abort, g.err, 33) && !*cta_abort);
-            if (!ok) break;
-            tc_fence_after();
-#pragma unroll
-            for (int gi = 0; gi < WIDE_HALF / 16; ++gi) {
-                float v[16];
-                tmem_ld16(trow + (uint32_t)(buf * WIDE_HALF + 16 * gi), v);
-#pragma unroll
-                for (int i = 0; i < 16; ++i) acc[16 * gi + i] += v[i];
-            }
-            tc_fence_before();
+        if (!ok) break;
+        if (piece) {
+            __threadfence();
             __syncwarp();
-            if (lane == 0) stream::mbar_arrive(&acc_empty[buf]);
-        }
-        if (ok && t < g.T && g.row_scale) {
-            const float rs = g.row_scale[t];
+            if (lane == 0) atomicAdd(counter(tile - g.whole), c_end - c_begin);
+        } else if (t < g.T && (EPI == PF_STORE || EPI == PF_ADD)) {
+            // columns: 32 at a time, in 32-byte accesses (a sector each), the old values of a group fetched together
+            const float rs = g.row_scale ? g.row_scale[t] : 1.0f;
 #pragma unroll
-            for (int i = 0; i < WIDE_HALF; ++i) acc[i] *= rs;
-        }
-        if (ok && t < g.T) {
+            for (int gi = 0; gi < 4; ++gi) {
+                const int n = (tile / g.tiles_x) * per + hsel * half + 32 * gi;
+                if (32 * gi >= half || n >= g.N) continue;
+                float *yp = g.y + (size_t)t * g.ldy + g.col0 + n;
+                const int live = min(4, (g.N - n) >> 3);         // N is a multiple of 8
+                float x[4][8];
 #pragma unroll
-            for (int gi = 0; gi < WIDE_HALF / 16; ++gi) {
-                const int c0 = hsel * WIDE_HALF + 16 * gi;
-                if (n0 + c0 >= g.N) continue;
-                float *yp = g.y + (size_t)t * g.ldy + g.col0 + n0 + c0;
-                if (n0 + c0 + 16 <= g.N) {
+                for (int e = 0; e < 4; ++e)
+                    if (EPI == PF_ADD && e < live) ld_sector(yp + 8 * e, x[e], y32);
 #pragma unroll
-                    for (int i = 0; i < 16; i += 4) {
-                        float4 o = make_float4(acc[16 * gi + i], acc[16 * gi + i + 1], acc[16 * gi + i + 2], acc[16 * gi + i + 3]);
-                        if (EPI == PF_ADD) {
-                            const float4 x = *reinterpret_cast<const float4 *>(yp + i);
-                            o.x += x.x; o.y += x.y; o.z += x.z; o.w += x.w;
-                        }
-                        *reinterpret_cast<float4 *>(yp + i) = o;
+                for (int e = 0; e < 4; ++e) {
+                    float o[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        o[j] = acc[32 * gi + 8 * e + j] * rs;
+                        if (EPI == PF_ADD) o[j] += x[e][j];
                     }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        if (n0 + c0 + i < g.N) yp[i] = EPI == PF_ADD ? yp[i] + acc[16 * gi + i] : acc[16 * gi + i];
+                    if (e < live) st_sector(yp + 8 * e, o, y32);
                 }
             }
+        } else if (t < g.T) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                float v[16];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) { v[e] = acc[8 * k + e]; v[8 + e] = acc[64 + 8 * k + e]; }
+                finish(tile, t, 8 * k, v);
+            }
+        }
+        }                                    // next job: its first chunks are already accumulating in tensor memory
+        // ---- this CTA's share of the tiles it has a piece of (at most two: its range is no longer than a tile's) ----
+        for (i = jobs.n_whole; ok && jobs.get(i, tile, c_begin, c_end); ++i) {
+            if (c_end - c_begin == nchunks) continue;
+            const int r = tile - g.whole, t = (tile % g.tiles_x) * BM + 32 * q + lane;
+            const int first = jobs.cta_of((long long)r * nchunks), n_ctas = min(8, jobs.cta_of((long long)(r + 1) * nchunks - 1) - first + 1);
+            if (jobs.cta - first >= n_ctas) continue;
+            int *cnt = counter(r), seen = 0;
+            unsigned spins = 0;
+            while (((seen = ld_acquire_int(cnt)) & 0xFFFF) < nchunks && !*cta_abort)
+                if (++spins > WAIT_LIMIT) { *cta_abort = 1; atomicExch(g.err, 25); }
+            ok = __all_sync(0xffffffffu, (seen & 0xFFFF) >= nchunks);
+            if (!ok) break;
+            for (int k = jobs.cta - first; k < 8; k += n_ctas) {
+                // registers 8 k .. and 64 + 8 k ..: not all are in use in tiles of fewer columns
+                const bool two = group_col(2 + (k >> 2)) >= 0;
+                if (group_col(k >> 2) < 0 || t >= g.T) continue;
+                float v[16];
+#pragma unroll
+                for (int e = 0; e < 16; ++e) v[e] = 0.f;
+#pragma unroll 8
+                for (int c = 0; c < nchunks; ++c) {
+                    const float4 *src = part_of(r, c) + 2 * k * 256;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        if (e >= 2 && !two) continue;
+                        const float4 x = __ldcg(src + ((e & 1) + 16 * (e >> 1)) * 256);
+                        v[4 * e] += x.x; v[4 * e + 1] += x.y; v[4 * e + 2] += x.z; v[4 * e + 3] += x.w;
+                    }
+                }
+                finish(tile, t, 8 * k, v);
+            }
+            __syncwarp();
+            if (lane == 0 && (atomicAdd(cnt, 0x10000) >> 16) == n_ctas - 1) *cnt = 0;      // the last of them: idle again
         }
     }
     tc_fence_before();

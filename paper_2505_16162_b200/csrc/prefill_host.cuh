@@ -48,43 +48,69 @@ inline bool gemm_attrs_once() {
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
     if (done[dev]) return true;
     const bool ok =
-        cudaFuncSetAttribute(gemm_split_kernel<PF_STORE>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM) == cudaSuccess &&
-        cudaFuncSetAttribute(gemm_split_kernel<PF_ADD>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM) == cudaSuccess &&
-        cudaFuncSetAttribute(gemm_split_kernel<PF_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM) == cudaSuccess &&
-        cudaFuncSetAttribute(gemm_split_kernel<PF_QKV>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM) == cudaSuccess &&
-        cudaFuncSetAttribute(gemm_wide_kernel<PF_STORE>, cudaFuncAttributeMaxDynamicSharedMemorySize, WIDE_SMEM) == cudaSuccess &&
-        cudaFuncSetAttribute(gemm_wide_kernel<PF_ADD>, cudaFuncAttributeMaxDynamicSharedMemorySize, WIDE_SMEM) == cudaSuccess &&
+        cudaFuncSetAttribute(gemm_split_kernel<PF_STORE>, cudaFuncAttributeMaxDynamicSharedMemorySize, RING_BYTES + 1280) == cudaSuccess &&
+        cudaFuncSetAttribute(gemm_split_kernel<PF_ADD>, cudaFuncAttributeMaxDynamicSharedMemorySize, RING_BYTES + 1280) == cudaSuccess &&
+        cudaFuncSetAttribute(gemm_split_kernel<PF_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, RING_BYTES + 1280) == cudaSuccess &&
+        cudaFuncSetAttribute(gemm_split_kernel<PF_QKV>, cudaFuncAttributeMaxDynamicSharedMemorySize, RING_BYTES + 1280) == cudaSuccess &&
         cudaFuncSetAttribute(attn_prompt_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn_smem_bytes<128>()) == cudaSuccess &&
         cudaFuncSetAttribute(attn_prompt_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn_smem_bytes<64>()) == cudaSuccess;
     done[dev] = ok;
     return ok;
 }
 
-// Accumulator columns per tile.  gemm_split_kernel runs one CTA per SM that walks the tiles round after round;
-// gemm_wide_kernel one CTA per tile.  The main loop is bound by shared-memory traffic (measured per k-block and CTA:
-// 0.57 / 0.69 / 0.81 us at 128 / 192 / 256 columns, 1.1 - 1.4 at 2 x 160): per k-block TMA writes the two activation
-// planes (32 KB) and bn / 8 KB of weights, and the tensor core reads the planes once and the weights twice (hi and lo
-// products), 64 + 3 bn / 8 KB in all; the 320-column tiles of gemm_wide_kernel (returned as WIDE_BN; store and add
-// epilogues only) read the planes once per half and are charged 15 % on top, as measured, plus ~10 us per round for the
-// prologue and epilogue that nothing overlaps there (1960 KB at that rate; the walking kernel pays ~3 us once).  The
-// width with the lowest rounds x traffic x k-blocks + fixed cost wins (ties: the wider tile).
-inline int pick_bn(int T, int N, int K, bool swiglu, int n_sms) {
-    const int row_tiles = (T + BM - 1) / BM;
-    const long nkb = K / BK;
-    int best = 0;
-    long best_cost = 0;
-    for (int bn = BOX_N; bn <= (swiglu ? BN_MAX : WIDE_BN); bn += BOX_N) {
-        if (bn > BN_MAX && bn != WIDE_BN) continue;
+// Most chunk sums a launch may leave in the scratch of the pieces (PIECE_FLOATS each, 72 MB in all: they have to stay in
+// L2 to be worth it).  20 tiles of 27 chunks - 5120 units at 13824 input columns, up to 128 rows - are 540.
+constexpr int MAX_PIECES = 576;
+
+// Columns per tile, CTAs, and how many tiles are done whole (the rest in pieces).
+struct Deal { int bn, grid, whole; };
+
+// The cheapest of 128, 192 and 256 columns, tiles all whole or the last, incomplete round of them in pieces, by times measured
+// on the 13B widths (5120 / 13824 columns in, 77 .. 1024 rows):
+//   whole tiles: 8 us + rounds x k-blocks x 0.5 / 0.62 / 0.73 us - the products of a k-block take that long (both terms'
+//     operands leave shared memory at ~64 bytes per clock), copies and sums run under them.  5120 units x 1024 rows, 256
+//     columns: two rounds 144 us, of which the second has 12 tiles.
+//   pieces: 14 us for the two meetings and the last sums, 1.3 x the products' time (pieces are not in step, so they share
+//     less through L2), and per chunk sum 0.012 us + 0.036 us per 128 KB to write and read it.  The same launch: one
+//     round + 12 tiles in 120 pieces, 93 us; at 77 rows, 20 tiles in 200 pieces 33 us against 63 us.
+// `heads`: 256 columns let the launch finish the heads itself; else a kernel of its own does.
+inline Deal deal_out(int T, int N, int K, bool swiglu, bool heads, int n_sms) {
+    const int row_tiles = (T + BM - 1) / BM, nkb = K / BK, nchunks = (nkb + CHUNK_KB - 1) / CHUNK_KB;
+    Deal best{0, 0, 0};
+    double best_us = 0.0;
+    for (int bn = 128; bn <= BN_MAX; bn += 64) {
         if (swiglu && bn % 128) continue;
         const int per = swiglu ? bn / 2 : bn;
-        const long ctas = (long)row_tiles * ((N + per - 1) / per);
-        const long traffic = bn == WIDE_BN ? 248 : 64 + 3 * bn / 8;
-        const long rounds = (ctas + n_sms - 1) / n_sms;
-        const long cost = bn == WIDE_BN ? rounds * (traffic * nkb + 1960) : rounds * traffic * nkb + 600;
-        if (!best || cost <= best_cost) { best = bn; best_cost = cost; }
+        const long long tiles = (long long)row_tiles * ((N + per - 1) / per), last_round = tiles % n_sms, units = last_round * nchunks;
+        const double kb_us = bn == 256 ? 0.73 : bn == 192 ? 0.62 : 0.5, heads_us = heads && bn != 256 ? 12.0 + T * 0.02 : 0.0;
+        const double round_us = nkb * kb_us;
+        for (int pieces = 0; pieces < 2; ++pieces) {
+            Deal d{bn, (int)(tiles < n_sms ? tiles : n_sms), (int)tiles};
+            double us = heads_us + 8.0 + (double)((tiles + n_sms - 1) / n_sms) * round_us;
+            if (pieces) {
+                if (last_round == 0 || units > MAX_PIECES) continue;
+                d.whole = (int)(tiles - last_round);
+                d.grid = d.whole == 0 && units < n_sms ? (int)units : n_sms;
+                const long long most = (units + d.grid - 1) / d.grid;
+                us = heads_us + 14.0 + (double)(d.whole / n_sms) * round_us + most * 1.3 * CHUNK_KB * kb_us +
+                     units * (0.012 + 0.036 * (T < BM ? T : BM) * bn / (double)PIECE_FLOATS);
+            }
+            if (!best.bn || us <= best_us) { best = d; best_us = us; }
+        }
     }
     return best;
 }
+
+// Rows of an activation box: a tile's worth, or what a launch of fewer rows needs (the rows a box leaves out of a tile hold
+// whatever the stage held before; they meet no live row).
+inline int act_box_rows(int T) { return T >= BM ? BM : (T + 7) / 8 * 8; }
+
+// Scratch of one launch: a launch finds the counters at zero and leaves them at zero.
+struct GemmScratch {
+    float *part;           // MAX_PIECES * PIECE_FLOATS
+    int *piece_cnt;        // PIECE_COUNTERS
+};
+constexpr int PIECE_COUNTERS = MAX_PIECES * (GEMM_THREADS / 32 - 2);
 
 // One contraction over T rows.  `planes` = the activation map (hi rows [0, cap), lo rows [cap, 2 cap)); W0 (and W1 for
 // SwiGLU: W0 = gate, W1 = up) are [N][K] bf16.  STORE with W1 and W2 given: the three matrices (nA, nB and nC rows, all
@@ -100,42 +126,42 @@ struct QkvFuse {
 // `fuse` (stacked q, k, v only): if the head dimension is 128 and the launch takes 256-column tiles, the epilogue does
 // the rotary embedding and writes K / V to the cache itself; *fused says whether it did (otherwise the caller runs
 // rope_kv_rows_kernel on y).
-inline bool launch_gemm(const CUtensorMap &planes, int cap, const void *W0, const void *W1, int N, int K, int T, int epi, float *y,
+inline bool launch_gemm(const CUtensorMap &planes, const GemmScratch &scratch, int cap, const void *W0, const void *W1, int N, int K, int T, int epi, float *y,
                         int ldy, int col0, bf16_t *out_hi, bf16_t *out_lo, int ldo, int *err, int n_sms, cudaStream_t s,
                         const void *W2 = nullptr, int nA = 0, int nB = 0, const QkvFuse *fuse = nullptr, bool *fused = nullptr,
                         const float *row_scale = nullptr) {
     if (fused) *fused = false;
     if (!gemm_attrs_once()) return false;
-    CUtensorMap tb0, tb1, tb2;
     const bool stacked = epi == PF_STORE && W1 && W2;
-    if (!make_map(&tb0, W0, (size_t)(stacked ? nA : N), (size_t)K, BOX_N)) return false;
+    const bool heads = stacked && fuse && fuse->head_dim == 128 && nA % 128 == 0 && nB % 128 == 0 && N % 128 == 0;
+    const Deal deal = deal_out(T, N, K, epi == PF_SWIGLU, heads, n_sms);
+    const int bn = deal.bn;
+    const int per = epi == PF_SWIGLU ? bn / 2 : bn;
+    const int box = per % 128 == 0 && (!stacked || (nA % 128 == 0 && nB % 128 == 0)) ? 128 : BOX_N;
+    CUtensorMap tb0, tb1, tb2;
+    if (!make_map(&tb0, W0, (size_t)(stacked ? nA : N), (size_t)K, box)) return false;
     if (epi == PF_SWIGLU) {
-        if (!make_map(&tb1, W1, (size_t)N, (size_t)K, BOX_N)) return false;
+        if (!make_map(&tb1, W1, (size_t)N, (size_t)K, box)) return false;
         tb2 = tb1;
     } else if (stacked) {
-        if (!make_map(&tb1, W1, (size_t)nB, (size_t)K, BOX_N) || !make_map(&tb2, W2, (size_t)(N - nA - nB), (size_t)K, BOX_N)) return false;
+        if (!make_map(&tb1, W1, (size_t)nB, (size_t)K, box) || !make_map(&tb2, W2, (size_t)(N - nA - nB), (size_t)K, box)) return false;
     } else {
         tb1 = tb0;
         tb2 = tb0;
     }
-    const int bn = pick_bn(T, N, K, epi == PF_SWIGLU, n_sms);
-    const int per = epi == PF_SWIGLU ? bn / 2 : bn;
-    const dim3 grid((T + BM - 1) / BM, (N + per - 1) / per);
-    GemmArgs g{T, K, N, bn, y, ldy, col0, out_hi, out_lo, ldo, err, (int)grid.x, (int)grid.y, stacked ? nA : N, stacked ? nB : 0,
-               row_scale, nullptr, nullptr, nullptr, 0, 0};
-    // gemm_split_kernel: one CTA per SM walks the tiles (the epilogue of a tile runs under the next tile's products)
-    const int n_tiles = (int)(grid.x * grid.y);
-    const dim3 pgrid(n_tiles < n_sms ? n_tiles : n_sms);
-    const bool fuse_heads = stacked && fuse && fuse->head_dim == 128 && bn == 256 && nA % 128 == 0 && nB % 128 == 0 && N % 128 == 0;
-    if (fuse_heads) { g.rope = fuse->rope; g.kc = fuse->kc; g.vc = fuse->vc; g.max_seq = fuse->max_seq; g.pos0 = fuse->pos0; }
+    const int tiles_x = (T + BM - 1) / BM, tiles_y = (N + per - 1) / per;
+    GemmArgs g{T, K, N, bn, y, ldy, col0, out_hi, out_lo, ldo, err, tiles_x, tiles_y, box, act_box_rows(T), deal.whole, scratch.part, scratch.piece_cnt,
+               stacked ? nA : N, stacked ? nB : 0, row_scale, nullptr, nullptr, nullptr, 0, 0};
+    const dim3 grid(deal.grid);
+    const int smem = gemm_smem(g.a_rows, bn);
+    const bool fuse_heads = heads && bn == 256;
     if (fuse_heads) {
-        gemm_split_kernel<PF_QKV><<<pgrid, GEMM_THREADS, GEMM_SMEM, s>>>(planes, tb0, tb1, tb2, g, cap);
+        g.rope = fuse->rope; g.kc = fuse->kc; g.vc = fuse->vc; g.max_seq = fuse->max_seq; g.pos0 = fuse->pos0;
+        gemm_split_kernel<PF_QKV><<<grid, GEMM_THREADS, smem, s>>>(planes, tb0, tb1, tb2, g, cap);
         if (fused) *fused = true;
-    } else if (bn == WIDE_BN && epi == PF_STORE) gemm_wide_kernel<PF_STORE><<<grid, GEMM_THREADS, WIDE_SMEM, s>>>(planes, tb0, tb1, tb2, g, cap);
-    else if (bn == WIDE_BN) gemm_wide_kernel<PF_ADD><<<grid, GEMM_THREADS, WIDE_SMEM, s>>>(planes, tb0, tb1, tb2, g, cap);
-    else if (epi == PF_STORE) gemm_split_kernel<PF_STORE><<<pgrid, GEMM_THREADS, GEMM_SMEM, s>>>(planes, tb0, tb1, tb2, g, cap);
-    else if (epi == PF_ADD) gemm_split_kernel<PF_ADD><<<pgrid, GEMM_THREADS, GEMM_SMEM, s>>>(planes, tb0, tb1, tb2, g, cap);
-    else gemm_split_kernel<PF_SWIGLU><<<pgrid, GEMM_THREADS, GEMM_SMEM, s>>>(planes, tb0, tb1, tb2, g, cap);
+    } else if (epi == PF_STORE) gemm_split_kernel<PF_STORE><<<grid, GEMM_THREADS, smem, s>>>(planes, tb0, tb1, tb2, g, cap);
+    else if (epi == PF_ADD) gemm_split_kernel<PF_ADD><<<grid, GEMM_THREADS, smem, s>>>(planes, tb0, tb1, tb2, g, cap);
+    else gemm_split_kernel<PF_SWIGLU><<<grid, GEMM_THREADS, smem, s>>>(planes, tb0, tb1, tb2, g, cap);
     return true;
 }
 

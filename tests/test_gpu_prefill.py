@@ -47,14 +47,11 @@ def _inputs(n_out, n_in, T, seed=3):
 # several row tiles; the 13B-shaped widths; one row
 GEMM_CASES = [(512, 256, 128), (1000, 320, 77), (136, 64, 5), (640, 1024, 300), (5120, 5120, 260), (264, 13824, 130),
               (15360, 5120, 1),
-              # tile widths other than 128 columns (the launch picks the width with the fewest column-rounds on the
-              # GPU's SMs): 192, 320 and 256 on a 148-SM part
+              # tile widths other than 128 columns (the launch picks the cheapest)
               (5120, 256, 520), (5120, 256, 900), (4608, 256, 1024),
               # more tiles than SMs (a CTA walks several tiles); a ragged last tile
               (5120, 2176, 900), (4936, 512, 1000),
-              # 320-column tiles on three rotating accumulators (picked where they save a round and the input is long
-              # enough to pay for their one-tile CTAs): staggered chunks with short last ones (69 k-blocks), a ragged
-              # last tile (136 of 320 columns, a weight box partly past the end)
+              # a short last chunk (69 k-blocks), a ragged last column tile, a weight box partly past the end
               (4936, 4416, 900)]
 
 
