@@ -214,6 +214,21 @@ void ctx_linear(knnssd_ctx *c, const LinearArgs &a) {
     c->launches++;
 }
 
+// Rows are y blocks of the grid, at most 65535 per launch.
+void launch_filter(const float *logits, int rows, int V, float inv_t, float top_p, float *probs, cudaStream_t s) {
+    static bool configured[kMaxDevices] = {};          // function attributes are per device
+    const int dev = current_device_slot();
+    if (!configured[dev]) {
+        cudaFuncSetAttribute(sampling::filtered_probs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(float) * sampling::SLICE_MAX);
+        configured[dev] = true;
+    }
+    for (int r = 0; r < rows; r += 65535) {
+        const int n = rows - r < 65535 ? rows - r : 65535;
+        sampling::filtered_probs_kernel<<<dim3(sampling::CL, n), sampling::NT, sampling::probs_smem(V), s>>>(
+            logits + (size_t)r * V, V, inv_t, top_p, probs + (size_t)r * V);
+    }
+}
+
 LinearArgs make_args(const void *W0, int rows0, int n_in, const float *x, const float *gain, float eps, float *y,
                      int epi, int M) {
     LinearArgs a{};
@@ -1053,14 +1068,14 @@ knnssd_status knnssd_decode_sampled(knnssd_ctx *c, int max_new, int k, float tem
         for (int j = 0; j < keff; ++j) {
             // draft step j: the draft model's logits of the row, filtered into q_j, the draft drawn from it
             run_pass(c, 1, c->chain + j, j, c->active_mask.data(), 0, c->target, false);
-            sampling::filtered_probs_kernel<<<1, sampling::NT, 0, s>>>(c->logits, g.vocab, inv_t, top_p, c->samp_q + (size_t)j * V);
-            sampling::sample_kernel<<<1, sampling::NT, 0, s>>>(c->samp_q + (size_t)j * V, g.vocab, u + j, 0.f, c->chain + j + 1);
+            launch_filter(c->logits, 1, g.vocab, inv_t, top_p, c->samp_q + (size_t)j * V, s);
+            sampling::sample_kernel<<<sampling::CL, sampling::NT, 0, s>>>(c->samp_q + (size_t)j * V, g.vocab, u + j, 0.f, c->chain + j + 1);
             c->launches += 2;
         }
         cudaEventRecord(c->ev1, s);
         run_pass(c, keff + 1, c->chain, 0, nullptr, 0, c->target, false);
-        sampling::filtered_probs_kernel<<<keff + 1, sampling::NT, 0, s>>>(c->logits, g.vocab, inv_t, top_p, c->samp_p);
-        sampling::spec_accept_kernel<<<1, sampling::NT, 0, s>>>(c->samp_p, c->samp_q, c->chain + 1, keff, g.vocab, u + k, u + 2 * k, 0.f,
+        launch_filter(c->logits, keff + 1, g.vocab, inv_t, top_p, c->samp_p, s);
+        sampling::spec_accept_kernel<<<sampling::CL, sampling::NT, 0, s>>>(c->samp_p, c->samp_q, c->chain + 1, keff, g.vocab, u + k, u + 2 * k, 0.f,
                                                                 c->samp_res);
         sampling::commit_sampled_kernel<<<1, 32, 0, s>>>(c->chain, c->samp_res, c->state, c->out_tokens, g.max_seq, c->accept_log, round);
         c->launches += 3;
@@ -1554,7 +1569,7 @@ knnssd_status knnssd_filtered_probs(const float *logits_dev, int rows, int vocab
         !std::isfinite(top_p))
         return KNNSSD_ERR_INVALID_ARG;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
-    sampling::filtered_probs_kernel<<<rows, sampling::NT, 0, s>>>(logits_dev, vocab, 1.0f / temperature, top_p, probs_dev);
+    launch_filter(logits_dev, rows, vocab, 1.0f / temperature, top_p, probs_dev, s);
     return cudaGetLastError() == cudaSuccess ? KNNSSD_OK : KNNSSD_ERR_CUDA;
 }
 
@@ -1563,7 +1578,7 @@ knnssd_status knnssd_sample_token(const float *weights_dev, int vocab, float u, 
     cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
     int *tok = nullptr;
     if (cudaMalloc(reinterpret_cast<void **>(&tok), sizeof(int)) != cudaSuccess) { cudaGetLastError(); return KNNSSD_ERR_CUDA; }
-    sampling::sample_kernel<<<1, sampling::NT, 0, s>>>(weights_dev, vocab, nullptr, u, tok);
+    sampling::sample_kernel<<<sampling::CL, sampling::NT, 0, s>>>(weights_dev, vocab, nullptr, u, tok);
     cudaError_t e = cudaMemcpyAsync(token_host, tok, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e == cudaSuccess) e = cudaGetLastError();
@@ -1594,7 +1609,7 @@ knnssd_status knnssd_spec_accept(const float *p_dev, const float *q_dev, const i
     }
     int host[2] = {0, 0};
     if (e == cudaSuccess) {
-        sampling::spec_accept_kernel<<<1, sampling::NT, 0, s>>>(p_dev, q_dev, d_dev, k, vocab, u_dev, nullptr, u_final, buf);
+        sampling::spec_accept_kernel<<<sampling::CL, sampling::NT, 0, s>>>(p_dev, q_dev, d_dev, k, vocab, u_dev, nullptr, u_final, buf);
         e = cudaMemcpyAsync(host, buf, sizeof(int) * 2, cudaMemcpyDeviceToHost, s);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);

@@ -8,37 +8,78 @@
 // more token is drawn from p.  Random numbers are inputs (one uniform per draw), consumed through the inverse CDF in
 // token-id order, so that the choices are reproducible.
 //
-// All three kernels run one block of 1024 threads per row: the work is a few passes over <= 152 k floats that sit in
-// L2, far below the cost of the pass that produced the logits.  Every sum has a fixed order.
+// A row is the work of a cluster of eight blocks, each with a contiguous eighth of the ids: a few passes over values that
+// stay in shared memory, bound by the meetings between the passes (~1.5 us each: block, then cluster).  Every sum has a
+// fixed order.
 #pragma once
+#include <cooperative_groups.h>
+
 #include "kernels.cuh"
 
 namespace knnssd {
 namespace sampling {
 
-constexpr int NT = 1024;
+namespace cg = cooperative_groups;
 
-// Sum over the block in a fixed order (thread partials -> warp trees -> warps in order); every thread gets the result.
-__device__ __forceinline__ float block_sum(float v, float *sh) {
-    v = warp_sum(v);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    float t = 0.f;
+constexpr int NT = 512;                    // at 1024 the meetings take twice as long (32 sums per warp to add up), at 256 long rows do
+constexpr int NW = NT / 32;
+constexpr int CL = 8;                      // blocks per row
+constexpr int NS = 32;                     // sums that one meeting adds up: one per lane, and per warp
+constexpr int SLICE_MAX = 49152;           // ids per block that fit in shared memory (192 KB)
+
+// Meeting place of the blocks of a row.  `slot` alternates: a block may still read the last meeting's sums while another
+// already writes the next one's.
+struct Meet {
+    float red[NW][NS + 1];
+    float slot[2][CL][NS];
+};
+
+// Sum (MAX: maximum of v[0]) over the threads of all blocks; lane j of every warp gets sum j, added in a fixed
+// order: lanes, warps, blocks.  `turn` counts the meetings.
+template <bool MAX>
+__device__ __forceinline__ float meet(Meet &sh, int &turn, float (&v)[NS]) {
+    cg::cluster_group cluster = cg::this_cluster();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, par = turn & 1;
+    ++turn;
+    if (MAX) {
+        const float m = warp_max(v[0]);
+        if (lane == 0) sh.red[warp][0] = m;
+    } else {
+        // each step halves the sums a lane is in charge of: 31 exchanges instead of 5 for every sum
 #pragma unroll
-    for (int w = 0; w < NT / 32; ++w) t += sh[w];
+        for (int h = NS / 2, bit = 16; h >= 1; h >>= 1, bit >>= 1) {
+            const bool up = lane & bit;
+#pragma unroll
+            for (int i = 0; i < h; ++i) {
+                const float give = up ? v[i] : v[i + h], keep = up ? v[i + h] : v[i];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, give, bit);
+            }
+        }
+        sh.red[warp][lane] = v[0];
+    }
+    __syncthreads();
+    // lanes r NW .. r NW + NW - 1 of warp w add up sum w PW + r of the NW warps
+    constexpr int PW = NS / NW;
+    static_assert(CL <= NW && NW <= 32 && NS == 32, "a lane per block in every group of lanes");
+    float t0 = sh.red[lane % NW][MAX ? 0 : warp * PW + lane / NW];
+#pragma unroll
+    for (int o = NW / 2; o > 0; o >>= 1) {
+        const float other = __shfl_xor_sync(0xffffffffu, t0, o);
+        t0 = MAX ? fmaxf(t0, other) : t0 + other;
+    }
+    if (lane % NW < CL && (!MAX || (warp == 0 && lane < NW)))
+        cluster.map_shared_rank(&sh, lane % NW)->slot[par][cluster.block_rank()][MAX ? 0 : warp * PW + lane / NW] = t0;
+    cluster.sync();
+    float t = sh.slot[par][0][MAX ? 0 : lane];
+#pragma unroll
+    for (int r = 1; r < CL; ++r) {
+        const float o = sh.slot[par][r][MAX ? 0 : lane];
+        t = MAX ? fmaxf(t, o) : t + o;
+    }
     return t;
 }
-__device__ __forceinline__ float block_max(float v, float *sh) {
-    v = warp_max(v);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    float t = sh[0];
-#pragma unroll
-    for (int w = 1; w < NT / 32; ++w) t = fmaxf(t, sh[w]);
-    return t;
-}
+
+// Count over one block.
 __device__ __forceinline__ int block_count(int v, int *sh) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -47,175 +88,275 @@ __device__ __forceinline__ int block_count(int v, int *sh) {
     __syncthreads();
     int t = 0;
 #pragma unroll
-    for (int w = 0; w < NT / 32; ++w) t += sh[w];
+    for (int w = 0; w < NW; ++w) t += sh[w];
     return t;
+}
+
+// Ids per block of a row of V: [rank S, rank S + S).
+__host__ __device__ __forceinline__ int slice_len(int V) { return (V + CL - 1) / CL; }
+// Shared memory of filtered_probs_kernel: the slice's values and, where it fits as well, the candidates among them.
+inline size_t probs_smem(int V) {
+    const size_t S = slice_len(V), padded = (S + NT - 1) / NT * NT;
+    return sizeof(float) * (S + padded <= SLICE_MAX ? S + padded : S <= SLICE_MAX ? S : 0);
 }
 
 // probs[row] = nucleus-filtered softmax(logits[row] / temperature), renormalised.  A token is kept iff the probability
 // mass of the tokens ranked before it (higher probability first, lower id first among equals) is below top_p.
-// The mass above a value is a decreasing step function of the value, so the smallest kept probability x0 is found by
-// bisection over the bit patterns of positive floats; tokens whose probability equals x0 are ranked by id.
-// grid = rows, NT threads.  probs doubles as scratch for the unfiltered probabilities.
-__global__ void __launch_bounds__(NT) filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_temperature, float top_p,
-                                                            float *__restrict__ probs) {
-    __shared__ float shf[NT / 32];
-    __shared__ int shi[NT / 32];
-    const float *l = logits + (size_t)blockIdx.x * V;
-    float *p = probs + (size_t)blockIdx.x * V;
-    const int tid = threadIdx.x;
+// The mass above a value is a decreasing step function of the value, so the smallest kept probability x0 is found in
+// the bit patterns of positive floats, 32 candidates at a time (five bits per pass; one candidate per pass, by one block
+// that re-read its row from L2 each time, took 65 us for 5 rows of 32000 and 241 us for one of 152064; this takes 20 and 35).  The first pass leaves
+// a few per cent of the values between its bounds; a thread keeps those of its own aside for the others.
+// Tokens whose probability equals x0 are ranked by id.
+// grid = (CL, rows), NT threads, probs_smem(V) of shared memory; rows too long for it keep their values in `probs`.
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT)
+filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_temperature, float top_p, float *__restrict__ probs) {
+    extern __shared__ float probs_slice[];
+    __shared__ Meet sh;
+    __shared__ int shi[NW];
+    __shared__ int s_cut;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int S = slice_len(V), rank = (int)cluster.block_rank(), tid = threadIdx.x;
+    const int id0 = min(V, rank * S), n = min(V, id0 + S) - id0;
+    const float *l = logits + (size_t)blockIdx.y * V + id0;
+    float *out = probs + (size_t)blockIdx.y * V + id0;
+    float *p = S <= SLICE_MAX ? probs_slice : out;               // a thread only ever touches its own entries, except where ids count
+    int turn = 0;
+    float v[NS];
+    cluster.barrier_arrive();                                    // every block has to run before another writes to its shared memory
     float m = -INFINITY;
-    for (int i = tid; i < V; i += NT) m = fmaxf(m, l[i]);
-    m = block_max(m, shf);
-    float s = 0.f;
-    for (int i = tid; i < V; i += NT) {
-        const float e = expf((l[i] - m) * inv_temperature);
+#pragma unroll 8
+    for (int i = tid; i < n; i += NT) { const float x = l[i]; p[i] = x; m = fmaxf(m, x); }
+    v[0] = m;
+    cluster.barrier_wait();
+    m = meet<true>(sh, turn, v);
+#pragma unroll
+    for (int j = 0; j < NS; ++j) v[j] = 0.f;
+    for (int i = tid; i < n; i += NT) {
+        const float e = expf((p[i] - m) * inv_temperature);
         p[i] = e;
-        s += e;
+        v[0] += e;
     }
-    s = block_sum(s, shf);
-    float pmax = 0.f;
-    for (int i = tid; i < V; i += NT) {
-        const float v = p[i] / s;
-        p[i] = v;
-        pmax = fmaxf(pmax, v);
-    }
-    pmax = block_max(pmax, shf);
-    auto mass_above = [&](float x) {
-        float a = 0.f;
-        for (int i = tid; i < V; i += NT) { const float v = p[i]; a += v > x ? v : 0.f; }
-        return block_sum(a, shf);
-    };
-    // smallest x (as a bit pattern) with mass_above(x) < top_p; mass_above(pmax) = 0
-    unsigned lo = 0u, hi = __float_as_uint(pmax);
-    if (mass_above(0.f) < top_p) hi = 0u;
-    while (hi > lo + 1u) {
-        const unsigned mid = lo + (hi - lo) / 2u;
-        if (mass_above(__uint_as_float(mid)) < top_p) hi = mid; else lo = mid;
+    const float s = __shfl_sync(0xffffffffu, meet<false>(sh, turn, v), 0);
+    for (int i = tid; i < n; i += NT) p[i] = p[i] / s;
+    // smallest x (as a bit pattern) in [lo, hi] with mass above x < top_p.  The largest probability is 1 / s (its exponent
+    // is zero), nothing lies above it.  Below (1 - top_p) / (2 V) there is less than half of 1 - top_p in all, so the mass above
+    // that is not below top_p: a sum of V terms is not off by the other half unless top_p is 1 to four digits.
+    unsigned lo = 0u, hi = __float_as_uint(fmaxf(0.f, 1.0f / s));
+    if (1.0f - top_p > 1e-4f) lo = min(hi, __float_as_uint(0.5f * (1.0f - top_p) / (float)V));
+    float *list = S + (S + NT - 1) / NT * NT <= SLICE_MAX ? probs_slice + S + tid : nullptr;
+    int n_list = 0;
+    float above = 0.f;                                           // this thread's values that lie above all candidates
+    for (bool first = true; first || hi > lo + 1u; first = false) {
+        const unsigned step = (hi - lo + NS - 1) / NS;           // candidates lo, lo + step, ..: lo itself only counts in the first pass
+        float x[NS];
+#pragma unroll
+        for (int j = 0; j < NS; ++j) { v[j] = above; x[j] = __uint_as_float(min(hi, lo + j * step)); }
+        const bool listed = list && !first;
+        const float *src = listed ? list : p + tid;
+        for (int i = 0, m_own = listed ? n_list : (n - tid + NT - 1) / NT; i < m_own; ++i) {
+            const float y = src[i * NT];
+#pragma unroll
+            for (int j = 0; j < NS; ++j) v[j] += y > x[j] ? y : 0.f;
+        }
+        const float mass = meet<false>(sh, turn, v);
+        const unsigned below = __ballot_sync(0xffffffffu, mass < top_p);
+        int j = below ? __ffs(below) - 1 : NS;                   // the first candidate with less than top_p above it
+        if (j == 0) {
+            if (first) { hi = lo; break; }
+            j = 1;                                               // lo was ruled out before, by sums in another order
+        }
+        const unsigned nhi = j < NS ? min(hi, lo + j * step) : hi;
+        lo = min(hi, lo + (j - 1) * step);
+        hi = nhi;
+        if (first && list) {
+            const float xl = __uint_as_float(lo), xh = __uint_as_float(hi);
+            for (int i = tid; i < n; i += NT) {
+                const float y = p[i];
+                if (y > xh) above += y;
+                else if (y > xl) list[NT * n_list++] = y;
+            }
+        }
     }
     const float x0 = __uint_as_float(hi);
-    // tokens at exactly x0: the n-th of them by id (n = 0, 1, ..) is kept iff mass_above(x0) + n x0 < top_p
-    const float a0 = mass_above(x0);
-    int c = 0;
-    for (int i = tid; i < V; i += NT) c += p[i] == x0 ? 1 : 0;
-    c = block_count(c, shi);
-    int nk = 0;
-    for (int n = tid; n < c; n += NT) nk += (a0 + (float)n * x0 < top_p) ? 1 : 0;
-    nk = block_count(nk, shi);
-    if (nk < 1) nk = 1;                       // the first token at x0 is kept by the definition of x0
-    int id_cut = V;                           // tokens at x0 with id < id_cut are kept
-    if (nk < c) {
-        int jl = 0, jh = V;                   // smallest J with #{j < J : p_j == x0} >= nk
-        while (jh > jl + 1) {
-            const int jm = jl + (jh - jl) / 2;
-            int g = 0;
-            for (int i = tid; i < jm; i += NT) g += p[i] == x0 ? 1 : 0;
-            g = block_count(g, shi);
-            if (g >= nk) jh = jm; else jl = jm;
+    // tokens at exactly x0: the n-th of them by id (n = 0, 1, ..) is kept iff mass above x0 + n x0 < top_p
+#pragma unroll
+    for (int j = 0; j < NS; ++j) v[j] = 0.f;
+    for (int i = tid; i < n; i += NT) {
+        const float y = p[i];
+        v[0] += y > x0 ? y : 0.f;
+        if (y == x0) v[1] += 1.f;                                // counts are exact up to 2^24 tokens
+    }
+    const float own_c = v[1];
+    float tot = meet<false>(sh, turn, v);
+    const float a0 = __shfl_sync(0xffffffffu, tot, 0);
+    const int c = (int)__shfl_sync(0xffffffffu, tot, 1);
+    int nk = 1, id_cut = V;                                      // tokens at x0 with id < id_cut are kept; the first one always is
+    if (c > 1) {
+        nk = 0;
+        for (int i = tid; i < c; i += NT) nk += (a0 + (float)i * x0 < top_p) ? 1 : 0;
+        nk = max(1, block_count(nk, shi));
+        if (nk < c) {                                            // which of them: the block that has the nk-th looks for its id
+            // sum r of this meeting: the tokens at x0 in block r
+#pragma unroll
+            for (int j = 0; j < NS; ++j) v[j] = j == rank ? own_c : 0.f;
+            tot = meet<false>(sh, turn, v);
+            int before = 0, holder = 0;
+            for (int r = 0; r < CL; ++r) {
+                const int cr = (int)__shfl_sync(0xffffffffu, tot, r);
+                if (before + cr >= nk) { holder = r; break; }
+                before += cr;
+            }
+            if (rank == holder) {
+                __syncthreads();
+                int jl = 0, jh = n;                              // smallest J with #{j < J : p_j == x0} >= nk - before
+                while (jh > jl + 1) {
+                    const int jm = jl + (jh - jl) / 2;
+                    int g = 0;
+                    for (int i = tid; i < jm; i += NT) g += p[i] == x0 ? 1 : 0;
+                    g = block_count(g, shi);
+                    if (g >= nk - before) jh = jm; else jl = jm;
+                }
+                if (tid < CL) *cluster.map_shared_rank(&s_cut, tid) = id0 + jh;
+            }
+            cluster.sync();
+            id_cut = s_cut;
         }
-        id_cut = jh;
     }
-    float z = 0.f;
-    for (int i = tid; i < V; i += NT) {
-        const float v = p[i];
-        z += (v > x0 || (v == x0 && i < id_cut)) ? v : 0.f;
+    const float z = a0 + (float)min(nk, c) * x0;
+    for (int i = tid; i < n; i += NT) {
+        const float y = p[i];
+        out[i] = (y > x0 || (y == x0 && id0 + i < id_cut)) ? y / z : 0.f;
     }
-    z = block_sum(z, shf);
-    for (int i = tid; i < V; i += NT) {
-        const float v = p[i];
-        p[i] = (v > x0 || (v == x0 && i < id_cut)) ? v / z : 0.f;
-    }
+    cluster.sync();                                              // nobody leaves while its shared memory may still be written to
 }
 
 // Inverse CDF in token-id order: the smallest id x with w_0 + .. + w_x > u * sum(w); w_i = a_i (b == nullptr) or
-// max(a_i - b_i, 0), falling back to a if that is zero everywhere.  Thread t owns the ids [t C, (t + 1) C).
-// Called by all NT threads of a block; every thread returns the token.
-__device__ __forceinline__ int block_sample(const float *__restrict__ a, const float *__restrict__ b, int V, float u, float *shf, int *shi) {
-    __shared__ float part[NT];
-    __shared__ int s_tok, s_last;
-    const int tid = threadIdx.x, C = (V + NT - 1) / NT, i0 = tid * C, i1 = min(V, i0 + C);
+// max(a_i - b_i, 0), falling back to a if that is zero everywhere.  Called by all threads of a cluster; block r has the ids
+// [r S, (r + 1) S), its warp w a contiguous run of them, read 32 at a time; the warp whose run holds the crossing walks it
+// again with a running sum.  Block 0's thread 0 returns the token (-1: no weight anywhere).
+// One block with a run of ids per thread and a serial scan of 1024 sums took 41 us for 152064 ids, this takes 8.5.
+struct Draw {
+    Meet m;
+    float warp_sum[NW];
+    int last[CL];
+    int token;
+};
+__device__ __forceinline__ int cluster_sample(const float *__restrict__ a, const float *__restrict__ b, int V, float u, Draw &sh) {
+    cg::cluster_group cluster = cg::this_cluster();
+    const int S = slice_len(V), rank = (int)cluster.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int run = (S + NW - 1) / NW, lim = min(V, rank * S + S);
+    const int i0 = min(lim, rank * S + warp * run), i1 = min(lim, i0 + run);
     bool use_b = b != nullptr;
-    for (int attempt = 0; attempt < 2; ++attempt) {
-        float s = 0.f;
+    int turn = 0;
+    if (tid == 0) sh.token = -1;
+    cluster.barrier_arrive();                                    // every block has to run before another writes to its shared memory
+    for (bool first = true;; first = false) {
+        auto weight = [&](int i) { return use_b ? fmaxf(a[i] - b[i], 0.f) : a[i]; };
+        float w = 0.f;
         int last = -1;
-        for (int i = i0; i < i1; ++i) {
-            const float w = use_b ? fmaxf(a[i] - b[i], 0.f) : a[i];
-            if (w > 0.f) last = i;
-            s += w;
+#pragma unroll 8
+        for (int i = i0 + lane; i < i1; i += 32) {
+            const float x = weight(i);
+            if (x > 0.f) last = i;
+            w += x;
         }
-        part[tid] = s;
-        // last id with weight, over the block
-        int lm = last;
+        w = warp_sum(w);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) lm = max(lm, __shfl_xor_sync(0xffffffffu, lm, o));
+        for (int o = 16; o > 0; o >>= 1) last = max(last, __shfl_xor_sync(0xffffffffu, last, o));
+        if (first) cluster.barrier_wait();
         __syncthreads();
-        if ((tid & 31) == 0) shi[tid >> 5] = lm;
+        if (lane == 0) { sh.warp_sum[warp] = w; sh.m.red[warp][NS] = __int_as_float(last); }
         __syncthreads();
-        if (tid == 0) {
-            int t = -1;
-            for (int w = 0; w < NT / 32; ++w) t = max(t, shi[w]);
-            s_last = t;
-            // exclusive scan of the thread sums in thread order
-            float run = 0.f;
-            for (int k = 0; k < NT; ++k) { const float v = part[k]; part[k] = run; run += v; }
-            shf[0] = run;
-            s_tok = -1;
+        // sum r of the meeting: block r's weights, its warps added in order
+        float v[NS], mine = 0.f;
+        if (tid == 0)
+            for (int k = 0; k < NW; ++k) mine += sh.warp_sum[k];
+        if (warp == 0) {
+            int lb = lane < NW ? __float_as_int(sh.m.red[lane][NS]) : -1;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) lb = max(lb, __shfl_xor_sync(0xffffffffu, lb, o));
+            if (lane == 0) cluster.map_shared_rank(&sh, 0)->last[rank] = lb;
         }
-        __syncthreads();
-        const float total = shf[0];
-        if (use_b && !(total > 0.f)) { use_b = false; __syncthreads(); continue; }
+#pragma unroll
+        for (int j = 0; j < NS; ++j) v[j] = j == rank ? mine : 0.f;
+        const float per_block = meet<false>(sh.m, turn, v);
+        float total = 0.f, before = 0.f, through = 0.f;
+#pragma unroll
+        for (int r = 0; r < CL; ++r) {
+            if (r == rank) before = total;
+            total += __shfl_sync(0xffffffffu, per_block, r);
+            if (r == rank) through = total;
+        }
+        if (use_b && !(total > 0.f)) { use_b = false; continue; }
         const float target = u * total;
-        const float excl = part[tid], incl = tid + 1 < NT ? part[tid + 1] : total;
-        // the chunk in which the running sum first exceeds the target
-        if (excl <= target && incl > target && i0 < i1) {
+        // runs of this block up to and including this warp's (the last warp ends where the block does)
+        float excl = before;
+        for (int k = 0; k < warp; ++k) excl += sh.warp_sum[k];
+        const float incl = warp == NW - 1 ? through : excl + sh.warp_sum[warp];
+        if (before <= target && through > target && excl <= target && incl > target) {
             float acc = excl;
-            int tok = -1;
-            for (int i = i0; i < i1; ++i) {
-                acc += use_b ? fmaxf(a[i] - b[i], 0.f) : a[i];
-                if (acc > target) { tok = i; break; }
+            int tok = -1, pos = -1;                              // pos: the last id with weight, if rounding hides the crossing
+            constexpr int B = 8;                                 // ids in flight: 8 x 32
+            for (int ib = i0; ib < i1 && tok < 0; ib += 32 * B) {
+                float xs[B];
+#pragma unroll
+                for (int e = 0; e < B; ++e) xs[e] = ib + 32 * e + lane < i1 ? weight(ib + 32 * e + lane) : 0.f;
+#pragma unroll
+                for (int e = 0; e < B; ++e) {
+                    const float x = xs[e];
+                    float sc = x;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const float t = __shfl_up_sync(0xffffffffu, sc, o);
+                        if (lane >= o) sc += t;
+                    }
+                    const unsigned over = __ballot_sync(0xffffffffu, x > 0.f && acc + sc > target), has = __ballot_sync(0xffffffffu, x > 0.f);
+                    if (over && tok < 0) tok = ib + 32 * e + __ffs(over) - 1;
+                    if (has) pos = ib + 32 * e + 31 - __clz(has);
+                    acc += __shfl_sync(0xffffffffu, sc, 31);
+                }
             }
-            if (tok >= 0) atomicMax(&s_tok, tok);       // at most one chunk qualifies; atomic only for safety
+            if (tok < 0) tok = pos;
+            if (lane == 0 && tok >= 0) atomicMax(&cluster.map_shared_rank(&sh, 0)->token, tok);
         }
-        __syncthreads();
-        const int tok = s_tok >= 0 ? s_tok : s_last;     // target rounded up to the total: the last id with weight
-        __syncthreads();
-        return tok;
+        break;
     }
-    return 0;
+    cluster.sync();
+    int tok = sh.token;
+    if (rank == 0 && tok < 0)                                    // target rounded up to the total: the last id with weight
+        for (int r = 0; r < CL; ++r) tok = max(tok, sh.last[r]);
+    return tok;
 }
 
-// token <- draw from weights w[V] with the uniform *u_ptr (u_val if u_ptr is null).  One block.
-__global__ void __launch_bounds__(NT) sample_kernel(const float *__restrict__ w, int V, const float *__restrict__ u_ptr, float u_val,
-                                                    int *__restrict__ token) {
-    __shared__ float shf[NT / 32];
-    __shared__ int shi[NT / 32];
-    const int tok = block_sample(w, nullptr, V, u_ptr ? *u_ptr : u_val, shf, shi);
-    if (threadIdx.x == 0) *token = tok < 0 ? 0 : tok;
+// token <- draw from weights w[V] with the uniform *u_ptr (u_val if u_ptr is null).  One cluster.
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT)
+sample_kernel(const float *__restrict__ w, int V, const float *__restrict__ u_ptr, float u_val, int *__restrict__ token) {
+    __shared__ Draw sh;
+    const int tok = cluster_sample(w, nullptr, V, u_ptr ? *u_ptr : u_val, sh);
+    if (threadIdx.x == 0 && blockIdx.x == 0) *token = tok < 0 ? 0 : tok;
 }
 
 // One verification round of speculative sampling.  p [k+1][V], q [k][V] filtered distributions, drafts [k] (device),
 // u_accept [k] (device), u_final (*u_final_ptr if given).  out[0] = number of drafts kept, out[1] = the token emitted
-// after them.  One block.
-__global__ void __launch_bounds__(NT) spec_accept_kernel(const float *__restrict__ p, const float *__restrict__ q, const int *__restrict__ drafts,
-                                                         int k, int V, const float *__restrict__ u_accept,
-                                                         const float *__restrict__ u_final_ptr, float u_final, int *__restrict__ out) {
+// after them.  One cluster.
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT)
+spec_accept_kernel(const float *__restrict__ p, const float *__restrict__ q, const int *__restrict__ drafts, int k, int V,
+                   const float *__restrict__ u_accept, const float *__restrict__ u_final_ptr, float u_final, int *__restrict__ out) {
+    __shared__ Draw sh;
     if (u_final_ptr) u_final = *u_final_ptr;
-    __shared__ float shf[NT / 32];
-    __shared__ int shi[NT / 32];
-    __shared__ int s_rej;
-    if (threadIdx.x == 0) {
-        int j = 0;
-        for (; j < k; ++j) {
-            int d = drafts[j];
-            if (d < 0 || d >= V) break;                          // a token outside the vocabulary is never kept
-            if (!(u_accept[j] * q[(size_t)j * V + d] < p[(size_t)j * V + d])) break;
-        }
-        s_rej = j;
+    // every warp tests all drafts, one per lane: the first that is not kept ends the round
+    const int lane = threadIdx.x & 31;
+    bool keep = false;
+    if (lane < k) {
+        const int d = drafts[lane];
+        // a token outside the vocabulary is never kept
+        keep = d >= 0 && d < V && u_accept[lane] * q[(size_t)lane * V + d] < p[(size_t)lane * V + d];
     }
-    __syncthreads();
-    const int j = s_rej;
-    const int tok = j < k ? block_sample(p + (size_t)j * V, q + (size_t)j * V, V, u_final, shf, shi)
-                          : block_sample(p + (size_t)k * V, nullptr, V, u_final, shf, shi);
-    if (threadIdx.x == 0) { out[0] = j; out[1] = tok < 0 ? 0 : tok; }
+    const unsigned lost = ~__ballot_sync(0xffffffffu, keep) & ((1u << k) - 1u);
+    const int j = lost ? __ffs(lost) - 1 : k;
+    const int tok = j < k ? cluster_sample(p + (size_t)j * V, q + (size_t)j * V, V, u_final, sh)
+                          : cluster_sample(p + (size_t)k * V, nullptr, V, u_final, sh);
+    if (threadIdx.x == 0 && blockIdx.x == 0) { out[0] = j; out[1] = tok < 0 ? 0 : tok; }
 }
 
 // The round's result into the session (one thread): res[0] = drafts kept, res[1] = the token after them; chain[1 .. k]
