@@ -540,6 +540,9 @@ __global__ void anchor_inv_norm_kernel(const float *__restrict__ anchors, int n,
     }
 }
 
+// One word of the session's state, in stream order.
+__global__ void set_word_kernel(int *word, int value) { *word = value; }
+
 __global__ void set_state_kernel(DeviceState *st, int len, int produced) {
     st->len = len; st->produced = produced; st->last_accept = 0; st->last_next = -1;
 }

@@ -120,6 +120,84 @@ template <typename T> cudaError_t dev_alloc(T **p, size_t count) {
     return cudaMalloc(reinterpret_cast<void **>(p), count * sizeof(T));
 }
 
+// ---- scratch of the stand-alone operators --------------------------------------------------------------------------
+// One memory pool per device that keeps at most kPoolKeep bytes between calls (what it holds beyond that goes back to the
+// driver at every synchronisation, all of it when a context is destroyed): a cudaMalloc / cudaFree pair cost 100 .. 1000 us
+// a call, next to kernels of 10 .. 50 us.  Allocations are ordered on the caller's stream, so any number of threads and
+// streams may call at once.
+constexpr unsigned long long kPoolKeep = 64ull << 20;
+
+struct DevicePools {
+    std::mutex mu;
+    cudaMemPool_t pool[64] = {};
+    bool tried[64] = {};
+    // The pool of the current device; nullptr where the device has none.
+    cudaMemPool_t current() {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+        std::lock_guard<std::mutex> lock(mu);
+        if (!tried[dev]) {
+            tried[dev] = true;
+            int has = 0;
+            cudaMemPoolProps props{};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            unsigned long long keep = kPoolKeep;
+            if (cudaDeviceGetAttribute(&has, cudaDevAttrMemoryPoolsSupported, dev) != cudaSuccess || !has ||
+                cudaMemPoolCreate(&pool[dev], &props) != cudaSuccess)
+                pool[dev] = nullptr;
+            else
+                cudaMemPoolSetAttribute(pool[dev], cudaMemPoolAttrReleaseThreshold, &keep);
+            cudaGetLastError();
+        }
+        return pool[dev];
+    }
+};
+DevicePools &device_pools() {
+    static DevicePools *pools = new DevicePools();      // never destroyed: a thread may still call at process exit
+    return *pools;
+}
+
+// The buffers of one call.  They are given back in stream order when it ends, whichever way it ends.
+struct Scratch {
+    cudaStream_t s;
+    cudaMemPool_t pool;
+    std::vector<void *> held;
+    explicit Scratch(cudaStream_t stream) : s(stream), pool(device_pools().current()) {}
+    Scratch(const Scratch &) = delete;
+    template <typename T> bool get(T **p, size_t count) {
+        void *q = nullptr;
+        const cudaError_t e = pool ? cudaMallocFromPoolAsync(&q, count * sizeof(T), pool, s) : cudaMalloc(&q, count * sizeof(T));
+        if (e != cudaSuccess) { cudaGetLastError(); return false; }
+        held.push_back(q);
+        *p = static_cast<T *>(q);
+        return true;
+    }
+    ~Scratch() {
+        for (void *q : held) {
+            if (pool) cudaFreeAsync(q, s);
+            else cudaFree(q);
+        }
+    }
+};
+
+// A few words of pinned memory per host thread, which kernels read arguments from and write results to: the calls that
+// use them synchronise before they return.  nullptr if they cannot be had.
+constexpr int kHostWords = 64;
+int *host_words() {
+    struct Words {
+        int *p = nullptr;
+        ~Words() { if (p) cudaFreeHost(p); }
+    };
+    static thread_local Words w;
+    if (!w.p && cudaHostAlloc(reinterpret_cast<void **>(&w.p), kHostWords * sizeof(int), cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        w.p = nullptr;
+    }
+    return w.p;
+}
+
 int pick_mt(int M) {
     static const int opts[] = {1, 2, 3, 4, 5, 6, 7, 8, 9, 16};
     for (int o : opts)
@@ -468,6 +546,19 @@ knnssd_status sync_check(knnssd_ctx *c, const char *what) {
     return KNNSSD_OK;
 }
 
+// A word of the session's state, written in stream order without waiting.  Refused while the stream is being captured, as
+// every call that changes the session is: the host's copy of the state would run ahead of the device's.
+knnssd_status set_word(knnssd_ctx *c, int *word, int value, const char *what) {
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(c->stream, &capturing);
+    if (e == cudaSuccess && capturing != cudaStreamCaptureStatusNone) e = cudaErrorStreamCaptureUnsupported;
+    if (e == cudaSuccess) {
+        set_word_kernel<<<1, 1, 0, c->stream>>>(word, value);
+        e = cudaGetLastError();
+    }
+    return e == cudaSuccess ? KNNSSD_OK : fail(c, KNNSSD_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
+}
+
 // What a non-zero device error word means.  Whatever it was, the pass that raised it did not finish: the session's
 // cache and pending token are no longer trustworthy, so the caller has to prefill again.
 knnssd_status fail_device_code(knnssd_ctx *c, const char *what, int code) {
@@ -480,6 +571,16 @@ knnssd_status fail_device_code(knnssd_ctx *c, const char *what, int code) {
         return fail(c, KNNSSD_ERR_INVALID_ARG, std::string(what) + ": a token id on the device was out of range (prefill again)");
     return fail(c, KNNSSD_ERR_TIMEOUT, std::string(what) + ": a device-side wait gave up (code " + std::to_string(code) +
                                        "); prefill again");
+}
+
+// Enqueue the read-back of the device error word with a call's other results; after the synchronisation that follows,
+// checked_err reports it once and clears it.
+constexpr int kErrWord = 32;           // its place in the pinned words
+cudaError_t read_err_word(knnssd_ctx *c) {
+    return cudaMemcpyAsync(c->pinned + kErrWord, c->err_word, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
+}
+knnssd_status checked_err(knnssd_ctx *c, const char *what) {
+    return c->pinned[kErrWord] ? fail_device_code(c, what, c->pinned[kErrWord]) : KNNSSD_OK;
 }
 
 // Read the device error word (synchronises); reports it once and clears it.
@@ -632,8 +733,9 @@ knnssd_status do_prefill(knnssd_ctx *c, const int *tokens_host, int n, float *po
     cudaEventRecord(c->ev1, s);
     if (pooled_dev) CUDA_TRY(c, cudaMemcpyAsync(pooled_dev, c->pooled, sizeof(float) * d, cudaMemcpyDeviceToDevice, s));
     CUDA_TRY(c, cudaMemcpyAsync(c->pinned, c->chain, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(c, read_err_word(c));
     knnssd_status st = sync_check(c, "prefill");
-    if (st == KNNSSD_OK) st = check_stream_err(c, "prefill");
+    if (st == KNNSSD_OK) st = checked_err(c, "prefill");
     if (st != KNNSSD_OK) return st;
     c->len = n;
     c->pending = c->pinned[0];
@@ -859,6 +961,7 @@ void knnssd_destroy(knnssd_ctx *c) {
     DeviceGuard dg(c->device);
     cudaStreamSynchronize(c->stream);
     free_all(c);
+    if (cudaMemPool_t pool = device_pools().current()) cudaMemPoolTrimTo(pool, 0);
     delete c;
 }
 
@@ -904,8 +1007,9 @@ knnssd_status knnssd_draft(knnssd_ctx *c, int k, int *draft_tokens_host, float *
     }
     cudaEventRecord(c->ev1, s);
     CUDA_TRY(c, cudaMemcpyAsync(c->pinned, c->chain + 1, sizeof(int) * k, cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(c, read_err_word(c));
     knnssd_status st = sync_check(c, "draft");
-    if (st == KNNSSD_OK) st = check_stream_err(c, "draft");
+    if (st == KNNSSD_OK) st = checked_err(c, "draft");
     if (st != KNNSSD_OK) return st;
     for (int j = 0; j < k; ++j) draft_tokens_host[j] = c->pinned[j];
     c->stats.ms_draft += elapsed_ms(c);
@@ -935,8 +1039,9 @@ knnssd_status knnssd_verify(knnssd_ctx *c, const int *draft_tokens_host, int k, 
         CUDA_TRY(c, cudaMemcpyAsync(hidden_dev_or_null, c->hfinal, sizeof(float) * (size_t)(k + 1) * g.d_model,
                                     cudaMemcpyDeviceToDevice, s));
     CUDA_TRY(c, cudaMemcpyAsync(c->pinned, c->state, sizeof(DeviceState), cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(c, read_err_word(c));
     knnssd_status st = sync_check(c, "verify");
-    if (st == KNNSSD_OK) st = check_stream_err(c, "verify");
+    if (st == KNNSSD_OK) st = checked_err(c, "verify");
     if (st != KNNSSD_OK) return st;
     const DeviceState *hs = reinterpret_cast<const DeviceState *>(c->pinned);
     c->len = hs->len;
@@ -1049,9 +1154,10 @@ knnssd_status knnssd_decode_sampled(knnssd_ctx *c, int max_new, int k, float tem
     cudaStream_t s = c->stream;
     float *u_dev = nullptr;
     const size_t n_u = (size_t)(max_new > 1 ? (max_new - 1) * stride : 1);
-    if (dev_alloc(&u_dev, n_u) != cudaSuccess) { cudaGetLastError(); return fail(c, KNNSSD_ERR_CUDA, "decode_sampled: cannot allocate the uniforms"); }
+    Scratch mem(s);
+    if (!mem.get(&u_dev, n_u)) return fail(c, KNNSSD_ERR_CUDA, "decode_sampled: cannot allocate the uniforms");
     knnssd_status st = KNNSSD_OK;
-    auto finish = [&](knnssd_status r) { cudaStreamSynchronize(s); cudaFree(u_dev); return r; };
+    auto finish = [&](knnssd_status r) { cudaStreamSynchronize(s); return r; };
     if (max_new > 1 && cudaMemcpyAsync(u_dev, uniforms_host, sizeof(float) * n_u, cudaMemcpyHostToDevice, s) != cudaSuccess)
         return finish(fail(c, KNNSSD_ERR_CUDA, "decode_sampled: cannot copy the uniforms"));
     emit_first_token_kernel<<<1, 1, 0, s>>>(c->chain, c->state, c->out_tokens, c->len);
@@ -1140,8 +1246,7 @@ knnssd_status knnssd_set_length(knnssd_ctx *c, int new_len) {
     DeviceGuard dg(c->device);
     if (!c->prefilled) return fail(c, KNNSSD_ERR_STATE, "set_length: prefill first");
     if (new_len < 1 || new_len > c->len) return fail(c, KNNSSD_ERR_INVALID_ARG, "set_length: can only roll back (1 <= new_len <= length)");
-    CUDA_TRY(c, cudaMemcpyAsync(&c->state->len, &new_len, sizeof(int), cudaMemcpyHostToDevice, c->stream));
-    knnssd_status st = sync_check(c, "set_length");
+    knnssd_status st = set_word(c, &c->state->len, new_len, "set_length");
     if (st != KNNSSD_OK) return st;
     c->len = new_len;
     return KNNSSD_OK;
@@ -1152,8 +1257,7 @@ knnssd_status knnssd_set_pending(knnssd_ctx *c, int token) {
     DeviceGuard dg(c->device);
     if (!c->prefilled) return fail(c, KNNSSD_ERR_STATE, "set_pending: prefill first");
     if (token < 0 || token >= c->cfg.vocab) return fail(c, KNNSSD_ERR_INVALID_ARG, "set_pending: token id out of range");
-    CUDA_TRY(c, cudaMemcpyAsync(c->chain, &token, sizeof(int), cudaMemcpyHostToDevice, c->stream));
-    knnssd_status st = sync_check(c, "set_pending");
+    knnssd_status st = set_word(c, c->chain, token, "set_pending");
     if (st != KNNSSD_OK) return st;
     c->pending = token;
     return KNNSSD_OK;
@@ -1377,17 +1481,10 @@ knnssd_status knnssd_gemm_split(const void *W0_dev, const void *W1_dev, int n_ou
     bf16_t *planes = nullptr, *outp = nullptr;
     prefill::GemmScratch scratch{};
     const size_t plane = (size_t)cap * n_in, oplane = (size_t)T * n_out;
-    auto cleanup = [&]() {
-        void *ptrs[] = {planes, outp, scratch.part, scratch.piece_cnt};
-        for (void *p : ptrs)
-            if (p) cudaFree(p);
-    };
-    if (dev_alloc(&planes, 2 * plane) != cudaSuccess || (mode == 2 && dev_alloc(&outp, 2 * oplane) != cudaSuccess) ||
-        dev_alloc(&scratch.part, (size_t)prefill::MAX_PIECES * prefill::PIECE_FLOATS) != cudaSuccess || dev_alloc(&scratch.piece_cnt, (size_t)prefill::PIECE_COUNTERS) != cudaSuccess) {
-        cudaGetLastError();
-        cleanup();
+    Scratch mem(s);
+    if (!mem.get(&planes, 2 * plane) || (mode == 2 && !mem.get(&outp, 2 * oplane)) ||
+        !mem.get(&scratch.part, (size_t)prefill::MAX_PIECES * prefill::PIECE_FLOATS) || !mem.get(&scratch.piece_cnt, (size_t)prefill::PIECE_COUNTERS))
         return KNNSSD_ERR_CUDA;
-    }
     cudaMemsetAsync(scratch.piece_cnt, 0, prefill::PIECE_COUNTERS * sizeof(int), s);
     knnssd_status st = KNNSSD_OK;
     cudaMemsetAsync(planes, 0, 2 * plane * sizeof(bf16_t), s);
@@ -1406,7 +1503,6 @@ knnssd_status knnssd_gemm_split(const void *W0_dev, const void *W1_dev, int n_ou
         if (cudaMemcpy(&code, stream_err_ptr(), sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) st = KNNSSD_ERR_CUDA;
         else if (code) { cudaMemset(stream_err_ptr(), 0, sizeof(int)); st = KNNSSD_ERR_TIMEOUT; }
     }
-    cleanup();
     return st;
 }
 
@@ -1430,11 +1526,10 @@ knnssd_status knnssd_linear_tc(const void *W_dev, int n_out, int n_in, const flo
     float *part = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     const size_t plane_elems = (size_t)2 * lintc::TN * n_in, part_elems = (size_t)kc * M * n_out;
-    bool ok = dev_alloc(&planes, plane_elems) == cudaSuccess && dev_alloc(&part, part_elems) == cudaSuccess &&
-              cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess;
+    Scratch mem(s);
+    bool ok = mem.get(&planes, plane_elems) && mem.get(&part, part_elems) && cudaEventCreate(&e0) == cudaSuccess &&
+              cudaEventCreate(&e1) == cudaSuccess;
     auto cleanup = [&]() {
-        if (planes) cudaFree(planes);
-        if (part) cudaFree(part);
         if (e0) cudaEventDestroy(e0);
         if (e1) cudaEventDestroy(e1);
     };
@@ -1494,15 +1589,11 @@ knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int 
     int *labels = nullptr, *small = nullptr, *out = nullptr;     // small: [0] changed, [1 .. n] counts
     unsigned char *taken = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    bool ok = dev_alloc(&mu, (size_t)n * d) == cudaSuccess && dev_alloc(&dist, (size_t)N) == cudaSuccess &&
-              dev_alloc(&part, (size_t)S * n * d) == cudaSuccess && dev_alloc(&labels, (size_t)N) == cudaSuccess &&
-              dev_alloc(&small, (size_t)n + 1) == cudaSuccess && dev_alloc(&out, (size_t)n * k) == cudaSuccess &&
-              dev_alloc(&taken, (size_t)N) == cudaSuccess && cudaEventCreate(&e0) == cudaSuccess &&
-              cudaEventCreate(&e1) == cudaSuccess;
+    Scratch mem(s);
+    bool ok = mem.get(&mu, (size_t)n * d) && mem.get(&dist, (size_t)N) && mem.get(&part, (size_t)S * n * d) && mem.get(&labels, (size_t)N) &&
+              mem.get(&small, (size_t)n + 1) && mem.get(&out, (size_t)n * k) && mem.get(&taken, (size_t)N) &&
+              cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess;
     auto cleanup = [&]() {
-        void *ptrs[] = {mu, dist, part, labels, small, out, taken};
-        for (void *p : ptrs)
-            if (p) cudaFree(p);
         if (e0) cudaEventDestroy(e0);
         if (e1) cudaEventDestroy(e1);
     };
@@ -1576,14 +1667,14 @@ knnssd_status knnssd_filtered_probs(const float *logits_dev, int rows, int vocab
 knnssd_status knnssd_sample_token(const float *weights_dev, int vocab, float u, int *token_host, void *cuda_stream) {
     if (!weights_dev || !token_host || vocab < 1 || !(u >= 0.f) || !(u < 1.f)) return KNNSSD_ERR_INVALID_ARG;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
-    int *tok = nullptr;
-    if (cudaMalloc(reinterpret_cast<void **>(&tok), sizeof(int)) != cudaSuccess) { cudaGetLastError(); return KNNSSD_ERR_CUDA; }
+    int *tok = host_words();
+    if (!tok) return KNNSSD_ERR_CUDA;
     sampling::sample_kernel<<<sampling::CL, sampling::NT, 0, s>>>(weights_dev, vocab, nullptr, u, tok);
-    cudaError_t e = cudaMemcpyAsync(token_host, tok, sizeof(int), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaError_t e = cudaStreamSynchronize(s);
     if (e == cudaSuccess) e = cudaGetLastError();
-    cudaFree(tok);
-    return e == cudaSuccess ? KNNSSD_OK : KNNSSD_ERR_CUDA;
+    if (e != cudaSuccess) return KNNSSD_ERR_CUDA;
+    *token_host = *static_cast<volatile int *>(tok);
+    return KNNSSD_OK;
 }
 
 knnssd_status knnssd_spec_accept(const float *p_dev, const float *q_dev, const int *drafts_host, int k, int vocab,
@@ -1595,29 +1686,18 @@ knnssd_status knnssd_spec_accept(const float *p_dev, const float *q_dev, const i
         if (drafts_host[j] < 0 || drafts_host[j] >= vocab || !(u_accept_host[j] >= 0.f) || !(u_accept_host[j] < 1.f))
             return KNNSSD_ERR_INVALID_ARG;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
-    int *buf = nullptr;                       // [0..1] result, [2 .. 2 + k) drafts, then k floats of uniforms
-    if (cudaMalloc(reinterpret_cast<void **>(&buf), sizeof(int) * (2 + 2 * (size_t)kMaxRows)) != cudaSuccess) {
-        cudaGetLastError();
-        return KNNSSD_ERR_CUDA;
-    }
-    int *d_dev = buf + 2;
-    float *u_dev = reinterpret_cast<float *>(buf + 2 + kMaxRows);
-    cudaError_t e = cudaSuccess;
-    if (k > 0) {
-        e = cudaMemcpyAsync(d_dev, drafts_host, sizeof(int) * k, cudaMemcpyHostToDevice, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(u_dev, u_accept_host, sizeof(float) * k, cudaMemcpyHostToDevice, s);
-    }
-    int host[2] = {0, 0};
-    if (e == cudaSuccess) {
-        sampling::spec_accept_kernel<<<sampling::CL, sampling::NT, 0, s>>>(p_dev, q_dev, d_dev, k, vocab, u_dev, nullptr, u_final, buf);
-        e = cudaMemcpyAsync(host, buf, sizeof(int) * 2, cudaMemcpyDeviceToHost, s);
-    }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    int *buf = host_words();                  // [0..1] result, [2 .. 2 + k) drafts, then k floats of uniforms
+    if (!buf) return KNNSSD_ERR_CUDA;
+    static_assert(2 + 2 * kMaxRows <= kHostWords, "the round's words");
+    float *u_pinned = reinterpret_cast<float *>(buf + 2 + kMaxRows);
+    for (int j = 0; j < k; ++j) { buf[2 + j] = drafts_host[j]; u_pinned[j] = u_accept_host[j]; }
+    sampling::spec_accept_kernel<<<sampling::CL, sampling::NT, 0, s>>>(p_dev, q_dev, buf + 2, k, vocab, u_pinned, nullptr, u_final, buf);
+    cudaError_t e = cudaStreamSynchronize(s);
     if (e == cudaSuccess) e = cudaGetLastError();
-    cudaFree(buf);
     if (e != cudaSuccess) return KNNSSD_ERR_CUDA;
-    *n_accepted = host[0];
-    *next_token = host[1];
+    const volatile int *res = buf;
+    *n_accepted = res[0];
+    *next_token = res[1];
     return KNNSSD_OK;
 }
 
@@ -1627,16 +1707,14 @@ knnssd_status knnssd_cosine_top1(const float *query_dev, const float *anchors_de
     cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
     float *cos_dev = nullptr;
     int *small = nullptr;  // [0..1] result, [2] flag
-    if (cudaMalloc(reinterpret_cast<void **>(&cos_dev), sizeof(float) * n) != cudaSuccess) return KNNSSD_ERR_CUDA;
-    if (cudaMalloc(reinterpret_cast<void **>(&small), sizeof(int) * 4) != cudaSuccess) { cudaFree(cos_dev); return KNNSSD_ERR_CUDA; }
+    Scratch scratch(s);
+    if (!scratch.get(&cos_dev, (size_t)n) || !scratch.get(&small, 4)) return KNNSSD_ERR_CUDA;
     cudaMemsetAsync(small, 0, sizeof(int) * 4, s);
     cosine_scores_kernel<<<(n + 7) / 8, 256, 0, s>>>(query_dev, anchors_dev, nullptr, n, d, cos_dev, small + 2);
     cosine_argmax_kernel<<<1, 256, 0, s>>>(cos_dev, n, small);
     int host[4] = {0, 0, 0, 0};
     cudaError_t e = cudaMemcpyAsync(host, small, sizeof(int) * 4, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(cos_dev);
-    cudaFree(small);
     if (e != cudaSuccess) return KNNSSD_ERR_CUDA;
     if (host[2]) return KNNSSD_ERR_DEGENERATE;
     if (best) *best = host[0];
