@@ -445,7 +445,12 @@ void run_pass_mega(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const 
     if (pr.merge_op) bars += n_attn;
     if (M > pass::BLKM) bars += n_attn;
     cudaError_t e;
-    if (M > 12) e = c->cfg.head_dim == 128 ? launch_pass_t<128, 2, 0>(c, pr) : launch_pass_t<64, 2, 0>(c, pr);
+    // 13..16 rows: where a CTA's share of the d_model-wide maps is more than two groups of 16 units, the packed form with
+    // four groups per batch fetches the activations half as often (16 rows, 8 layers of the 13B / Qwen widths 1.93 -> 1.75 /
+    // 2.17 -> 1.97 ms); with two groups there is one batch either way and its larger loop only costs (7B widths 1.31 -> 1.33)
+    const bool wide = c->cfg.d_model > 2 * stream::WROWS * c->n_sms;
+    if (M > 12 && wide) e = c->cfg.head_dim == 128 ? launch_pass_t<128, 2, 4>(c, pr) : launch_pass_t<64, 2, 4>(c, pr);
+    else if (M > 12) e = c->cfg.head_dim == 128 ? launch_pass_t<128, 2, 0>(c, pr) : launch_pass_t<64, 2, 0>(c, pr);
     else if (M > pass::BLKM) e = c->cfg.head_dim == 128 ? launch_pass_t<128, 2, 3>(c, pr) : launch_pass_t<64, 2, 3>(c, pr);
     else if (M > pass::BLKM / 2) e = c->cfg.head_dim == 128 ? launch_pass_t<128, 1, 0>(c, pr) : launch_pass_t<64, 1, 0>(c, pr);
     else e = c->cfg.head_dim == 128 ? launch_pass_t<128, 1, 1>(c, pr) : launch_pass_t<64, 1, 1>(c, pr);

@@ -9,7 +9,8 @@
 // NB = row blocks of eight: 1 for passes of up to 8 rows, 2 for 9..16 rows (the second block is a second 8-column
 // operand for the same weight fragments; every row is computed exactly as it would be in a one-row pass).
 //
-// NP > 0 (the paired form; NP = 1: passes of up to 4 rows - every draft step; NP = 3: passes of 9..12 rows): the rows
+// NP > 0 (the paired form; NP = 1: passes of up to 4 rows - every draft step; NP = 3: passes of 9..12 rows; NP = 4: of
+// 13..16 rows on wide models): the rows
 // are taken four at a time and the two bf16 terms of a row sit in neighbouring columns of ONE 8-column operand
 // (column 2 r = hi term of row 4 b + r, 2 r + 1 = its lo term), so a weight fragment takes one MMA per four rows
 // instead of two per eight: 1 instead of 2 for up to 4 rows, 3 instead of 4 for 9..12.  A consumer that is faster
@@ -29,7 +30,7 @@ namespace stream {
 __device__ __forceinline__ uint4 ld_frag4(const uint32_t *p) { return __ldcg(reinterpret_cast<const uint4 *>(p)); }
 
 // Column groups (of 16 units) a batch of the consumer takes, by kernel form; LinPhase::gb carries it to the producer.
-template <int NB, int NP> __host__ __device__ constexpr int groups_per_batch() { return NP == 3 ? GB : GB / NB; }
+template <int NB, int NP> __host__ __device__ constexpr int groups_per_batch() { return NP >= 3 ? GB : GB / NB; }
 
 template <int NB, int NP>
 __device__ __forceinline__ void consume_linear_pre(const LinPhase &p, const Ring &r, int cta, int n_cta, int warp, int lane,
@@ -40,7 +41,7 @@ __device__ __forceinline__ void consume_linear_pre(const LinPhase &p, const Ring
     constexpr int NTM = PAIRED ? 1 : NTERM;                 // operand sets (MMAs) per weight fragment and operand block
     // groups per batch: the tile loop is unrolled over them and has to stay small (instruction cache), so two row
     // blocks of eight take half as many groups; the producer is told the same number through LinPhase::gb.  The
-    // activation fragments of a column tile are fetched from L2 once per batch, so the 9..12-row form keeps four
+    // activation fragments of a column tile are fetched from L2 once per batch, so the 9..12-row and the packed 13..16-row form keep four
     // groups: at two it would pull 0.75 bytes of activations per byte of weights.
     constexpr int GBN = groups_per_batch<NB, NP>();
     constexpr int RW = PAIRED ? 2 : 4;                      // floats a lane leaves per (warp, group, block) for the batch-end sums

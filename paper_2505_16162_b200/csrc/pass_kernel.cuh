@@ -104,14 +104,16 @@ __device__ __forceinline__ bool grid_barrier(const Model &md, const Ring &r, uns
         atomicAdd(md.bar, 1ULL);
         unsigned spins = 0;
         while (ld_acquire_u64(md.bar) < target) {
-            if (*r.abort_flag || *reinterpret_cast<volatile int *>(md.gabort)) { *r.abort_flag = 1; break; }
+            // the abort words are looked at every 64 polls: a second trip to L2 per poll doubled the time between polls
+            // (8 layers of the 13B widths, one row: 0.6255 -> 0.6237 ms)
+            if ((spins & 63u) == 63u && (*r.abort_flag || *reinterpret_cast<volatile int *>(md.gabort))) { *r.abort_flag = 1; break; }
             if (++spins > spin_limit) {
                 *r.abort_flag = 1;
                 atomicExch(md.gabort, 1);
                 atomicExch(md.err, 7);
                 break;
             }
-            __nanosleep(32);
+            __nanosleep(20);
         }
     }
     asm volatile("bar.sync 1, %0;" ::"n"(NCW * 32) : "memory");
@@ -689,7 +691,7 @@ __device__ __forceinline__ void attn_merge_phase(const Model &md, const Op &op, 
 // ---- the pass ---------------------------------------------------------------------------------------------------
 // NB = 1: passes of up to BLKM rows; NB = 2: 9..16 rows (a kernel of its own, so that the common one stays small).
 // NP > 0: the linear maps take the rows four at a time with both terms in one operand (NP = 1: passes of up to 4 rows -
-// every draft step; NP = 3 with NB = 2: passes of 9..12 rows); NP = 0: eight at a time, one operand per term.
+// every draft step; NP = 3, 4 with NB = 2: passes of 9..12 and 13..16 rows); NP = 0: eight at a time, one operand per term.
 template <int HD, int NB, int NP>
 __global__ void __launch_bounds__(stream::NTHREADS, 1) pass_kernel(const Model md, const Params pr) {
     extern __shared__ __align__(128) unsigned char smem[];
