@@ -289,7 +289,7 @@ knnssd_status knnssd_linear_tc(const void *W_dev, int n_out, int n_in, const flo
  *   anchors_host        HOST int32 [n_clusters][k]: point indices, nearest first, lowest index first among equal
  *                       distances; -1 where a cluster has fewer than k members
  *   rounds_host         HOST: assignment rounds done (NULL: not wanted)
- *   ms_rounds_host      HOST: device time of all rounds' kernels, CUDA events on the stream (NULL: not wanted)
+ *   ms_rounds_host      HOST: device time of all rounds, CUDA events on the stream (NULL: not wanted)
  * Allocates and frees its scratch; synchronises the stream.
  */
 knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int n_clusters,

@@ -21,23 +21,44 @@ namespace anchors {
 constexpr int MAXC = 16;       // most clusters (domains)
 constexpr int CHUNK = 256;     // columns of the centroids staged in shared memory per step
 constexpr int PTS = 16;        // points per block of assign_kernel: two per warp
+constexpr int RING = 3;        // steps of columns a block of assign_kernel has in flight or in use: three blocks per SM
 
-// For each point: the squared distances to all n centroids; relabel != 0: labels[p] <- the nearest centroid (lowest
-// index among equal distances), *changed set if that differs from the old label, counts[c] incremented; in both modes
-// dist[p] <- the distance to the centroid of labels[p].  grid = ceil(N / PTS), 256 threads: a warp owns two points, the
-// block shares the staged columns of the centroids.  Per step of 256 columns a lane holds 8 columns of each of its
-// points (VEC: two 16-byte loads per point, d % 4 == 0), fetched one step ahead; the centroids' next columns are
-// fetched into registers under the arithmetic as well.  In shared memory the centroid values are ordered
-// [cluster][i][lane] (i = which of the lane's 8 columns), so that a warp reads consecutive words.
-// NC = the cluster count rounded up to 4, 8 or 16: the per-cluster registers (and with them the CTAs per SM) follow it.
+// What the rounds of a call leave on the device, so that several rounds can be enqueued without the host looking at the
+// outcome of each: the kernels of a round do nothing once an earlier round changed no assignment.
+struct Progress {
+    int done;                  // a round changed nothing
+    int rounds;                // assignment rounds done
+    int changed[2];            // by round parity: the round changed an assignment
+    int counts[2][MAXC];       // by round parity: members per cluster
+};
+
+// One 16-byte (VEC) or 4-byte piece on its way into shared memory; zeros where there is nothing to read.
+template <bool VEC> __device__ __forceinline__ void copy_piece(float *dst, const float *src, bool live) {
+    const unsigned to = (unsigned)__cvta_generic_to_shared(dst);
+    if (VEC) {
+        const int n = live ? 16 : 0;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(src), "r"(n) : "memory");
+    } else {
+        const int n = live ? 4 : 0;
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(to), "l"(src), "r"(n) : "memory");
+    }
+}
+
+// For each point: the squared distances to all n centroids, labels[p] <- the nearest centroid (lowest index among equal
+// distances); the round's `changed` is set if that differs from the old label, its counts[c] incremented.  mu32 holds the
+// centroids rounded to fp32, rows of stride ld (a multiple of 4).  grid = ceil(N / PTS), 256 threads: a warp owns two
+// points, the block shares the columns of the centroids.  Per step of 256 columns a lane holds 8 columns of each of its
+// points (VEC, d % 4 == 0: two runs of four).  Points and centroids come through a ring of RING steps of asynchronous
+// copies: what bounds the kernel is how much of the points is in flight (5000 x 5120: one step ahead in registers 58 us, with the ring 35).
+// NC = the cluster count rounded up to 4, 8 or 16: the per-cluster registers follow it.
+template <int NC> constexpr int assign_smem() { return RING * (PTS + NC) * CHUNK * (int)sizeof(float); }
 template <bool VEC, int NC>
-__global__ void __launch_bounds__(256, NC <= 8 ? 3 : 2) assign_kernel(const float *__restrict__ x, int N, int d, const double *__restrict__ mu, int n,
-                                                     int relabel, int *__restrict__ labels, double *__restrict__ dist,
-                                                     int *__restrict__ counts, int *__restrict__ changed) {
-    __shared__ float smu[NC][8][32];
+__global__ void __launch_bounds__(256, NC <= 8 ? 3 : 2) assign_kernel(const float *__restrict__ x, int N, int d, const float *__restrict__ mu32, int ld, int n,
+                                                     int parity, int *__restrict__ labels, Progress *__restrict__ pg) {
+    extern __shared__ __align__(16) float as_smem[];             // [RING][PTS points, then NC centroids][CHUNK]
+    if (pg->done) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int pa = blockIdx.x * PTS + 2 * warp, pb = pa + 1;
-    const bool la = pa < N, lb = pb < N;
+    const int p0 = blockIdx.x * PTS, pa = p0 + 2 * warp;
     // running sums as unevaluated pairs of floats (hi + lo, hi the rounded sum, lo the rounding errors collected by
     // the error-free two-sum): ~48 bits without touching the fp64 pipe in the loop
     float hi[2][NC], lo[2][NC];
@@ -49,68 +70,76 @@ __global__ void __launch_bounds__(256, NC <= 8 ? 3 : 2) assign_kernel(const floa
         l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(v, bb)));
         h = s;
     };
-    const float *xa = x + (size_t)(la ? pa : 0) * d, *xb = x + (size_t)(lb ? pb : 0) * d;
-    // the lane's i-th column within a step: VEC: (i / 4) 128 + 4 lane + i % 4; else lane + 32 i
-    auto col_of = [&](int i, int ln) { return VEC ? (i >> 2) * 128 + 4 * ln + (i & 3) : ln + 32 * i; };
-    auto fetch = [&](const float *xr, bool live, int col0, float (&v)[8]) {
-        if (VEC) {
+    const int steps = (d + CHUNK - 1) / CHUNK;
+    constexpr int W = VEC ? 4 : 1;                               // columns per piece
+    auto fetch = [&](int step) {
+        if (step < steps) {
+            const int col0 = step * CHUNK;
+            float *st = as_smem + (step % RING) * (PTS + NC) * CHUNK;
+            // rows of this warp: its two points, and every eighth centroid
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int c0 = col0 + h * 128 + 4 * lane;
-                const float4 t = (live && c0 < d) ? __ldg(reinterpret_cast<const float4 *>(xr + c0)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                v[4 * h] = t.x; v[4 * h + 1] = t.y; v[4 * h + 2] = t.z; v[4 * h + 3] = t.w;
+            for (int q = 0; q < 2; ++q) {
+                const int p = pa + q;
+                const float *src = x + (size_t)min(p, N - 1) * d;
+#pragma unroll
+                for (int j = lane * W; j < CHUNK; j += 32 * W) {
+                    const bool live = p < N && col0 + j < d;
+                    copy_piece<VEC>(st + (2 * warp + q) * CHUNK + j, src + (live ? col0 + j : 0), live);
+                }
             }
-        } else {
+            for (int c = warp; c < n; c += 8)
 #pragma unroll
-            for (int i = 0; i < 8; ++i) v[i] = (live && col0 + lane + 32 * i < d) ? __ldg(xr + col0 + lane + 32 * i) : 0.f;
+                for (int j = lane * 4; j < CHUNK; j += 128) {
+                    const bool live = col0 + j < ld;
+                    copy_piece<true>(st + (PTS + c) * CHUNK + j, mu32 + (size_t)c * ld + (live ? col0 + j : 0), live);
+                }
         }
+        asm volatile("cp.async.commit_group;" ::: "memory");     // empty groups keep the count of groups equal to that of steps
     };
-    // this thread stages slot (i, ln) = (threadIdx.x / 32, threadIdx.x % 32) of every cluster
-    const int my_col = col_of(warp, lane);
-    auto fetch_mu = [&](int col0, float (&m)[NC]) {
 #pragma unroll
-        for (int c = 0; c < NC; ++c) m[c] = (c < n && col0 + my_col < d) ? (float)mu[(size_t)c * d + col0 + my_col] : 0.f;
-    };
-    float ca[8], cb[8], na[8], nb[8];
-    float mreg[NC];
-    fetch(xa, la, 0, ca);
-    fetch(xb, lb, 0, cb);
-    fetch_mu(0, mreg);
-    for (int col0 = 0; col0 < d; col0 += CHUNK) {
+    for (int i = 0; i < RING - 1; ++i) fetch(i);
+    for (int step = 0; step < steps; ++step) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(RING - 2) : "memory");
+        __syncthreads();                                         // this step has arrived for all; the one before has been read by all
+        fetch(step + RING - 1);
+        const float *st = as_smem + (step % RING) * (PTS + NC) * CHUNK;
+        auto row = [&](int r, float (&v)[8]) {
+            if (VEC) {
 #pragma unroll
-        for (int c = 0; c < NC; ++c)
-            if (c < n) smu[c][warp][lane] = mreg[c];
-        __syncthreads();
-        if (col0 + CHUNK < d) {
-            fetch(xa, la, col0 + CHUNK, na);
-            fetch(xb, lb, col0 + CHUNK, nb);
-            fetch_mu(col0 + CHUNK, mreg);
-        }
+                for (int h = 0; h < 2; ++h) {
+                    const float4 t = *reinterpret_cast<const float4 *>(st + r * CHUNK + h * 128 + 4 * lane);
+                    v[4 * h] = t.x; v[4 * h + 1] = t.y; v[4 * h + 2] = t.z; v[4 * h + 3] = t.w;
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) v[i] = st[r * CHUNK + lane + 32 * i];
+            }
+        };
+        float ca[8], cb[8];
+        row(2 * warp, ca);
+        row(2 * warp + 1, cb);
 #pragma unroll
         for (int c = 0; c < NC; ++c)
             if (c < n) {
                 // columns past the end hold zeros on both sides: they add nothing
-                float sa = 0.f, sb = 0.f;
+                float m[8], sa = 0.f, sb = 0.f;
+                row(PTS + c, m);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    const float m = smu[c][i][lane];
-                    const float da = ca[i] - m, db = cb[i] - m;
+                    const float da = ca[i] - m[i], db = cb[i] - m[i];
                     sa = fmaf(da, da, sa);
                     sb = fmaf(db, db, sb);
                 }
                 add_pair(hi[0][c], lo[0][c], sa);
                 add_pair(hi[1][c], lo[1][c], sb);
             }
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < 8; ++i) { ca[i] = na[i]; cb[i] = nb[i]; }
     }
     double acc[2][NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) { acc[0][c] = (double)hi[0][c] + (double)lo[0][c]; acc[1][c] = (double)hi[1][c] + (double)lo[1][c]; }
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-        const int p = q ? pb : pa;
+        const int p = pa + q;
         if (p >= N) continue;                                  // warp-uniform
 #pragma unroll
         for (int c = 0; c < NC; ++c)
@@ -119,29 +148,24 @@ __global__ void __launch_bounds__(256, NC <= 8 ? 3 : 2) assign_kernel(const floa
                 for (int o = 16; o > 0; o >>= 1) acc[q][c] += __shfl_xor_sync(0xffffffffu, acc[q][c], o);
             }
         if (lane == 0) {
-            int best = labels[p];
-            if (relabel) {
-                best = 0;
-                double bv = acc[q][0];
-#pragma unroll
-                for (int c = 1; c < NC; ++c)
-                    if (c < n && acc[q][c] < bv) { bv = acc[q][c]; best = c; }
-                if (best != labels[p]) { labels[p] = best; atomicOr(changed, 1); }
-                atomicAdd(counts + best, 1);
-            }
-            double own = acc[q][0];
+            int best = 0;
+            double bv = acc[q][0];
 #pragma unroll
             for (int c = 1; c < NC; ++c)
-                if (c == best) own = acc[q][c];
-            dist[p] = sqrt(own);
+                if (c < n && acc[q][c] < bv) { bv = acc[q][c]; best = c; }
+            if (best != labels[p]) { labels[p] = best; atomicOr(pg->changed + parity, 1); }
+            atomicAdd(pg->counts[parity] + best, 1);
         }
     }
 }
 
 // part[s][c][j] = sum of x[p][j] over the points p of slice s (S slices of `per` consecutive points) labelled c, added
-// in index order.  grid = (ceil(d / 256), S), 256 threads: a thread owns one column.
+// in index order.  grid = (ceil(d / 256), S), 256 threads: a thread owns one column.  Bound by the fp64 pipe, which issues
+// about 4 lanes per clock and SM: 29 us for 5000 x 5120, the time of its 26 million additions.
 __global__ void __launch_bounds__(256) partial_sums_kernel(const float *__restrict__ x, int N, int d, const int *__restrict__ labels,
-                                                           int n, int per, double *__restrict__ part) {
+                                                           int n, int per, double *__restrict__ part, int parity,
+                                                           const Progress *__restrict__ pg) {
+    if (pg->done || !pg->changed[parity]) return;
     __shared__ double acc[MAXC][256];
     const int j = blockIdx.x * 256 + threadIdx.x, s = blockIdx.y;
     for (int c = 0; c < n; ++c) acc[c][threadIdx.x] = 0.0;
@@ -162,12 +186,21 @@ __global__ void __launch_bounds__(256) partial_sums_kernel(const float *__restri
         for (int c = 0; c < n; ++c) part[((size_t)s * n + c) * d + j] = acc[c][threadIdx.x];
 }
 
-// mu[c][j] = (sum over slices, in slice order, of part[s][c][j]) / counts[c]; a cluster without members keeps its
-// centroid.  grid = (ceil(d / 256), n), 256 threads.
-__global__ void fold_centroids_kernel(const double *__restrict__ part, const int *__restrict__ counts, int n, int d, int S,
-                                      double *__restrict__ mu) {
+// The end of a round.  If it changed an assignment: mu[c][j] = (sum over slices, in slice order, of part[s][c][j]) /
+// counts[c], in mu32 rounded to fp32; a cluster without members keeps its centroid.  Otherwise the iteration is done.  Clears
+// the counters of the next round.  grid = (ceil(d / 256), n), 256 threads.
+__global__ void fold_centroids_kernel(const double *__restrict__ part, int n, int d, int S, double *__restrict__ mu, float *__restrict__ mu32,
+                                      int ld, int parity, Progress *__restrict__ pg) {
+    const bool changed = pg->changed[parity] != 0;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && !pg->done) {
+        // the other blocks act on this round's `changed` and `counts` alone, which stay as they are until the next round's end
+        pg->rounds += 1;
+        pg->changed[parity ^ 1] = 0;
+        for (int c = 0; c < MAXC; ++c) pg->counts[parity ^ 1][c] = 0;
+        if (!changed) pg->done = 1;
+    }
     const int j = blockIdx.x * 256 + threadIdx.x, c = blockIdx.y;
-    if (j >= d || counts[c] == 0) return;
+    if (!changed || j >= d || pg->counts[parity][c] == 0) return;
     double s = 0.0;
     int i = 0;
     for (; i + 8 <= S; i += 8) {                              // eight loads in flight, added in slice order
@@ -178,7 +211,18 @@ __global__ void fold_centroids_kernel(const double *__restrict__ part, const int
         for (int e = 0; e < 8; ++e) s += v[e];
     }
     for (; i < S; ++i) s += part[((size_t)i * n + c) * d + j];
-    mu[(size_t)c * d + j] = s / (double)counts[c];
+    s /= (double)pg->counts[parity][c];
+    mu[(size_t)c * d + j] = s;
+    mu32[(size_t)c * ld + j] = (float)s;
+}
+
+// The starting centroids in both precisions (mu32's padding and the progress start at zero).  grid = (ceil(d / 256), n).
+__global__ void start_centroids_kernel(const float *__restrict__ start, int d, double *__restrict__ mu, float *__restrict__ mu32, int ld) {
+    const int j = blockIdx.x * 256 + threadIdx.x, c = blockIdx.y;
+    if (j >= d) return;
+    const float v = start[(size_t)c * d + j];
+    mu[(size_t)c * d + j] = (double)v;
+    mu32[(size_t)c * ld + j] = v;
 }
 
 // dist[p] = ||x_p - mu_{labels[p]}|| with every difference, square and sum in fp64 against the fp64 centroid: the
@@ -202,31 +246,52 @@ __global__ void __launch_bounds__(256) member_dist_kernel(const float *__restric
 }
 
 // Eq. (2) for cluster c = blockIdx.x: k times, the not yet taken member with the smallest (distance, index);
-// out[c][r] = its index, -1 once the cluster has run out of members.  taken[N] starts at zero.  256 threads.
-__global__ void __launch_bounds__(256) select_anchors_kernel(const double *__restrict__ dist, const int *__restrict__ labels, int N, int k,
-                                                             unsigned char *__restrict__ taken, int *__restrict__ out) {
-    __shared__ double sv[256];
-    __shared__ int si[256];
-    const int c = blockIdx.x, tid = threadIdx.x;
+// out[c][r] = its index, -1 once the cluster has run out of members.  A copy of the distances in shared memory (staged != 0:
+// N doubles) serves all k searches, with -1 for points that are no member or taken; longer lists are read from global memory
+// each time, taken[N] starting at zero.  SEL_NT threads.  (5 x 10 of 5000 points: 17 us; 256 threads
+// re-reading labels and distances took 38.)
+constexpr int SEL_NT = 1024, SEL_STAGED = 25600;
+__global__ void __launch_bounds__(SEL_NT) select_anchors_kernel(const double *__restrict__ dist, const int *__restrict__ labels, int N, int k,
+                                                                int staged, unsigned char *__restrict__ taken, int *__restrict__ out) {
+    extern __shared__ double sel_dist[];
+    __shared__ double sv[SEL_NT / 32];
+    __shared__ int si[SEL_NT / 32];
+    const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // does (ov, oi) come before (v, i)?  -1: nothing there
+    auto before = [](double ov, int oi, double v, int i) { return oi >= 0 && (i < 0 || ov < v || (ov == v && oi < i)); };
+    if (staged)
+        for (int p = tid; p < N; p += SEL_NT) sel_dist[p] = labels[p] == c ? dist[p] : -1.0;
     for (int r = 0; r < k; ++r) {
         double bv = INFINITY;
         int bi = -1;
-        for (int p = tid; p < N; p += 256)
-            if (labels[p] == c && !taken[p] && (bi < 0 || dist[p] < bv)) { bv = dist[p]; bi = p; }   // ascending p: first of equals wins
-        sv[tid] = bv;
-        si[tid] = bi;
-        __syncthreads();
-        for (int o = 128; o > 0; o >>= 1) {
-            if (tid < o) {
-                const double ov = sv[tid + o];
-                const int oi = si[tid + o];
-                if (oi >= 0 && (si[tid] < 0 || ov < sv[tid] || (ov == sv[tid] && oi < si[tid]))) { sv[tid] = ov; si[tid] = oi; }
-            }
-            __syncthreads();
+        for (int p = tid; p < N; p += SEL_NT) {                  // ascending p: the first of equals wins
+            const double v = staged ? sel_dist[p] : (labels[p] == c && !taken[p] ? dist[p] : -1.0);
+            if (v != -1.0 && (bi < 0 || v < bv)) { bv = v; bi = p; }
         }
-        if (tid == 0) {
-            out[c * k + r] = si[0];
-            if (si[0] >= 0) taken[si[0]] = 1;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+            if (before(ov, oi, bv, bi)) { bv = ov; bi = oi; }
+        }
+        if (lane == 0) { sv[warp] = bv; si[warp] = bi; }
+        __syncthreads();
+        if (warp == 0) {
+            bv = sv[lane];
+            bi = si[lane];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
+                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+                if (before(ov, oi, bv, bi)) { bv = ov; bi = oi; }
+            }
+            if (lane == 0) {
+                out[c * k + r] = bi;
+                if (bi >= 0) {
+                    if (staged) sel_dist[bi] = -1.0;
+                    else taken[bi] = 1;
+                }
+            }
         }
         __syncthreads();
     }

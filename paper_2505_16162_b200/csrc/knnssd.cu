@@ -1569,13 +1569,6 @@ knnssd_status knnssd_linear_tc(const void *W_dev, int n_out, int n_in, const flo
     return st;
 }
 
-namespace {
-__global__ void widen_kernel(const float *__restrict__ a, size_t n, double *__restrict__ b) {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) b[i] = (double)a[i];
-}
-}  // namespace
-
 knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int n_clusters,
                                    const float *init_centroids_dev, int max_rounds, int k, int *labels_host,
                                    double *centroids_out_dev, int *anchors_host, int *rounds_host, float *ms_rounds_host,
@@ -1590,61 +1583,66 @@ knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int 
     int S = (N + 63) / 64;                        // slices of the centroid sums: at least 64 points each, at most 64 slices
     if (S > 64) S = 64;
     const int per = (N + S - 1) / S;
+    const int ld = (d + 3) / 4 * 4;                 // row stride of the fp32 centroids
     double *mu = nullptr, *dist = nullptr, *part = nullptr;
-    int *labels = nullptr, *small = nullptr, *out = nullptr;     // small: [0] changed, [1 .. n] counts
+    float *mu32 = nullptr;
+    int *labels = nullptr, *out = nullptr;
+    anchors::Progress *progress = nullptr;
     unsigned char *taken = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     Scratch mem(s);
-    bool ok = mem.get(&mu, (size_t)n * d) && mem.get(&dist, (size_t)N) && mem.get(&part, (size_t)S * n * d) && mem.get(&labels, (size_t)N) &&
-              mem.get(&small, (size_t)n + 1) && mem.get(&out, (size_t)n * k) && mem.get(&taken, (size_t)N) &&
+    bool ok = mem.get(&mu, (size_t)n * d) && mem.get(&mu32, (size_t)n * ld) && mem.get(&dist, (size_t)N) && mem.get(&part, (size_t)S * n * d) &&
+              mem.get(&labels, (size_t)N) && mem.get(&progress, 1) && mem.get(&out, (size_t)n * k) && mem.get(&taken, (size_t)N) &&
               cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess;
     auto cleanup = [&]() {
         if (e0) cudaEventDestroy(e0);
         if (e1) cudaEventDestroy(e1);
     };
-    if (!ok) { cudaGetLastError(); cleanup(); return KNNSSD_ERR_CUDA; }
-    widen_kernel<<<(unsigned)(((size_t)n * d + 255) / 256), 256, 0, s>>>(init_centroids_dev, (size_t)n * d, mu);
-    cudaMemsetAsync(labels, 0xFF, sizeof(int) * N, s);           // -1: the first round changes every assignment
-    const dim3 cols((d + 255) / 256);
-    const int agrid = (N + anchors::PTS - 1) / anchors::PTS;
     const bool vec = d % 4 == 0;                                 // rows stay 16-byte aligned
-    auto launch_assign = [&](int relabel) {
-#define KNNSSD_ASSIGN(V, NC) anchors::assign_kernel<V, NC><<<agrid, 256, 0, s>>>(x_dev, N, d, mu, n, relabel, labels, dist, small + 1, small)
-        if (vec) { if (n <= 4) KNNSSD_ASSIGN(true, 4); else if (n <= 8) KNNSSD_ASSIGN(true, 8); else KNNSSD_ASSIGN(true, 16); }
-        else { if (n <= 4) KNNSSD_ASSIGN(false, 4); else if (n <= 8) KNNSSD_ASSIGN(false, 8); else KNNSSD_ASSIGN(false, 16); }
-#undef KNNSSD_ASSIGN
-    };
-    int rounds = 0, changed = 1;
+    typedef void (*AssignFn)(const float *, int, int, const float *, int, int, int, int *, anchors::Progress *);
+    const AssignFn assign = vec ? (n <= 4 ? anchors::assign_kernel<true, 4> : n <= 8 ? anchors::assign_kernel<true, 8> : anchors::assign_kernel<true, 16>)
+                                : (n <= 4 ? anchors::assign_kernel<false, 4> : n <= 8 ? anchors::assign_kernel<false, 8> : anchors::assign_kernel<false, 16>);
+    const int assign_smem = n <= 4 ? anchors::assign_smem<4>() : n <= 8 ? anchors::assign_smem<8>() : anchors::assign_smem<16>();
+    const int staged = N <= anchors::SEL_STAGED, sel_smem = staged ? N * (int)sizeof(double) : 0;
+    ok = ok && cudaFuncSetAttribute(assign, cudaFuncAttributeMaxDynamicSharedMemorySize, assign_smem) == cudaSuccess &&
+         cudaFuncSetAttribute(anchors::select_anchors_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              anchors::SEL_STAGED * (int)sizeof(double)) == cudaSuccess;
+    if (!ok) { cudaGetLastError(); cleanup(); return KNNSSD_ERR_CUDA; }
+    const dim3 cols((d + 255) / 256, n);
+    cudaMemsetAsync(mu32, 0, sizeof(float) * n * ld, s);
+    cudaMemsetAsync(progress, 0, sizeof(anchors::Progress), s);
+    cudaMemsetAsync(labels, 0xFF, sizeof(int) * N, s);           // -1: the first round changes every assignment
+    anchors::start_centroids_kernel<<<cols, 256, 0, s>>>(init_centroids_dev, d, mu, mu32, ld);
+    // rounds are enqueued four at a time: the kernels of rounds after the last one return at once (~2 us each), a look at the
+    // outcome of every round cost ~35 us of waiting and copies per round
+    int rounds = 0;
     float ms_total = 0.f;
     cudaError_t e = cudaSuccess;
-    while (rounds < max_rounds && e == cudaSuccess) {
-        cudaMemsetAsync(small, 0, sizeof(int) * (n + 1), s);
+    for (int r0 = 0; r0 < max_rounds && e == cudaSuccess; r0 += 4) {
         cudaEventRecord(e0, s);
-        launch_assign(1);
+        for (int r = r0; r < max_rounds && r < r0 + 4; ++r) {
+            assign<<<(N + anchors::PTS - 1) / anchors::PTS, 256, assign_smem, s>>>(x_dev, N, d, mu32, ld, n, r & 1, labels, progress);
+            anchors::partial_sums_kernel<<<dim3(cols.x, S), 256, 0, s>>>(x_dev, N, d, labels, n, per, part, r & 1, progress);
+            anchors::fold_centroids_kernel<<<cols, 256, 0, s>>>(part, n, d, S, mu, mu32, ld, r & 1, progress);
+        }
         cudaEventRecord(e1, s);
-        e = cudaMemcpyAsync(&changed, small, sizeof(int), cudaMemcpyDeviceToHost, s);
+        int seen[2] = {0, 0};                                    // done, rounds
+        e = cudaMemcpyAsync(seen, progress, sizeof(seen), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) break;
         float ms = 0.f;
         cudaEventElapsedTime(&ms, e0, e1);
         ms_total += ms;
-        ++rounds;
-        if (!changed) break;
-        cudaEventRecord(e0, s);
-        anchors::partial_sums_kernel<<<dim3(cols.x, S), 256, 0, s>>>(x_dev, N, d, labels, n, per, part);
-        anchors::fold_centroids_kernel<<<dim3(cols.x, n), 256, 0, s>>>(part, small + 1, n, d, S, mu);
-        cudaEventRecord(e1, s);
-        e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) break;
-        cudaEventElapsedTime(&ms, e0, e1);
-        ms_total += ms;
+        rounds = seen[1];
+        if (seen[0]) break;
     }
     if (e == cudaSuccess) {
         // the anchors are ranked by fp64 distances to the final fp64 centroids (which moved after the last assignment
         // if the round limit ended the iteration)
         anchors::member_dist_kernel<<<(N + 7) / 8, 256, 0, s>>>(x_dev, N, d, mu, labels, dist);
-        cudaMemsetAsync(taken, 0, (size_t)N, s);
-        anchors::select_anchors_kernel<<<n, 256, 0, s>>>(dist, labels, N, k, taken, out);
+        if (!staged) cudaMemsetAsync(taken, 0, (size_t)N, s);
+        anchors::select_anchors_kernel<<<n, anchors::SEL_NT, sel_smem, s>>>(dist, labels, N, k, staged, taken, out);
         e = cudaMemcpyAsync(anchors_host, out, sizeof(int) * n * k, cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess && labels_host) e = cudaMemcpyAsync(labels_host, labels, sizeof(int) * N, cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess && centroids_out_dev)
