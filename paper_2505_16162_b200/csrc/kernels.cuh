@@ -395,6 +395,47 @@ __global__ void pool_accumulate_kernel(const float *__restrict__ h, int M, int d
     for (int m = 0; m < M; ++m) s += (double)h[(size_t)m * d + i];
     sum[i] = s;
 }
+
+// The same for many rows, without writing the normalised rows out: part[s][i] = fp64 sum, in row order, of the rows of slice s
+// (`per` rows each), every term the row's value times its RMSNorm scale times the gain, rounded as rmsnorm_rows_kernel does;
+// pool_fold_kernel adds the slices in order.  The fp64 additions (about 4 lanes per clock and SM) want all SMs: one thread per
+// column walking 1024 rows took 83 us, this 16 with the scales.  grid = (ceil(d / 256), slices), 256 threads.
+__global__ void __launch_bounds__(256) pool_partial_kernel(const float *__restrict__ x, const float *__restrict__ rinv, const float *__restrict__ gain,
+                                                           int M, int d, int per, double *__restrict__ part) {
+    const int i = blockIdx.x * 256 + threadIdx.x, m0 = blockIdx.y * per, m1 = min(M, m0 + per);
+    if (i >= d) return;
+    const float g = gain[i];
+    double s = 0.0;
+#pragma unroll 8
+    for (int m = m0; m < m1; ++m) s += (double)(x[(size_t)m * d + i] * rinv[m] * g);
+    part[(size_t)blockIdx.y * d + i] = s;
+}
+__global__ void pool_fold_kernel(const double *__restrict__ part, int slices, int d, double *__restrict__ sum, int overwrite) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= d) return;
+    double s = overwrite ? 0.0 : sum[i];
+#pragma unroll 8
+    for (int k = 0; k < slices; ++k) s += part[(size_t)k * d + i];
+    sum[i] = s;
+}
+// rinv[m] = RMSNorm's scale of row m, summed as rmsnorm_rows_kernel does.  grid = M, 256 threads.
+__global__ void __launch_bounds__(256) row_scale_kernel(const float *__restrict__ x, int d, float eps, float *__restrict__ rinv) {
+    __shared__ float s_red[8];
+    const int m = blockIdx.x, tid = threadIdx.x;
+    const float *xr = x + (size_t)m * d;
+    float s = 0.f;
+    for (int i = tid * 4; i < d; i += 1024) {
+        const float4 v = *reinterpret_cast<const float4 *>(xr + i);
+        s = fmaf(v.x, v.x, s); s = fmaf(v.y, v.y, s); s = fmaf(v.z, v.z, s); s = fmaf(v.w, v.w, s);
+    }
+    s = warp_sum(s);
+    if ((tid & 31) == 0) s_red[tid >> 5] = s;
+    __syncthreads();
+    if (tid) return;
+    float tot = 0.f;
+    for (int w = 0; w < 8; ++w) tot += s_red[w];
+    rinv[m] = 1.0f / sqrtf(tot / (float)d + eps);
+}
 __global__ void pool_finish_kernel(const double *__restrict__ sum, int d, double inv_count, float *__restrict__ v) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < d) v[i] = (float)(sum[i] * inv_count);
@@ -478,40 +519,49 @@ __global__ void accept_kernel(int *__restrict__ chain, const int *__restrict__ t
 }
 
 // ---------------------------------------------------------------------------------------------
-// Cosine top-1 over the anchors.  One warp per anchor: dot(v, a) / (|v| |a|) with the anchor's
-// inverse norm precomputed (or computed here when inv_norm == nullptr).  Then one block folds the
-// n cosines to the arg-max, lowest index on ties.  A zero / non-finite norm sets *flag.
+// Cosine top-1 over the anchors
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) cosine_scores_kernel(const float *__restrict__ v, const float *__restrict__ anchors,
-                                                            const float *__restrict__ inv_norm, int n, int d,
-                                                            float *__restrict__ cosines, int *__restrict__ flag) {
-    const int lane = threadIdx.x & 31, a = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (a >= n) return;
-    const float *ar = anchors + (size_t)a * d;
-    float dot = 0.f, vv = 0.f, aa = 0.f;
-    for (int i = lane; i < d; i += 32) {
-        const float x = v[i], y = ar[i];
-        dot = fmaf(x, y, dot);
-        vv = fmaf(x, x, vv);
-        aa = fmaf(y, y, aa);
-    }
-    dot = warp_sum(dot); vv = warp_sum(vv); aa = warp_sum(aa);
-    if (lane == 0) {
-        const bool bad = !(vv > 0.f) || !isfinite(vv) || !(aa > 0.f) || !isfinite(aa);
-        if (bad) { *flag = 1; cosines[a] = -INFINITY; return; }
-        const float ia = inv_norm ? inv_norm[a] : 1.0f / sqrtf(aa);
-        cosines[a] = dot * (1.0f / sqrtf(vv)) * ia;
-    }
-}
 
-// out[0] = best flat index (as int bits), out[1] = cosine bits.
-__global__ void cosine_argmax_kernel(const float *__restrict__ cosines, int n, int *__restrict__ out) {
+// Eq. (4) in one launch: a warp per anchor, dot(v, a) / (|v| |a|) with the anchor's reciprocal norm given or, inv_norm ==
+// nullptr, computed here; then the block that finishes last takes the arg-max of all n, lowest index on ties.  cosines[n] and
+// work[2] (blocks done, a zero or non-finite norm was met) are scratch; work is zero between launches.  out[0] = best flat
+// index, out[1] = its cosine's bits, out[2] = the flag; it may be pinned host memory.  Bound by latencies: 9 us at 50 x 5120,
+// as the two launches before it, but one launch, a memset and two copies less make 28 us of a call of 40.
+// grid = ceil(n / 8), 256 threads.
+__global__ void __launch_bounds__(256) cosine_top1_kernel(const float *__restrict__ v, const float *__restrict__ anchors,
+                                                          const float *__restrict__ inv_norm, int n, int d, float *__restrict__ cosines,
+                                                          int *__restrict__ work, int *__restrict__ out) {
     __shared__ float s_v[8];
     __shared__ int s_i[8];
-    const int tid = threadIdx.x;
+    __shared__ int s_last;
+    const int tid = threadIdx.x, lane = tid & 31, a = blockIdx.x * 8 + (tid >> 5);
+    if (a < n) {
+        const float *ar = anchors + (size_t)a * d;
+        float dot = 0.f, vv = 0.f, aa = 0.f;
+#pragma unroll 16
+        for (int i = lane; i < d; i += 32) {
+            const float x = v[i], y = ar[i];
+            dot = fmaf(x, y, dot);
+            vv = fmaf(x, x, vv);
+            aa = fmaf(y, y, aa);
+        }
+        dot = warp_sum(dot); vv = warp_sum(vv); aa = warp_sum(aa);
+        if (lane == 0) {
+            const bool bad = !(vv > 0.f) || !isfinite(vv) || !(aa > 0.f) || !isfinite(aa);
+            const float ia = inv_norm ? inv_norm[a] : 1.0f / sqrtf(aa);
+            __stcg(cosines + a, bad ? -INFINITY : dot * (1.0f / sqrtf(vv)) * ia);
+            if (bad) atomicExch(work + 1, 1);
+        }
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(work, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
     float bv = -INFINITY;
     int bi = 0x7fffffff;
-    for (int i = tid; i < n; i += 256) argmax_fold(bv, bi, cosines[i], i);
+    for (int i = tid; i < n; i += 256) argmax_fold(bv, bi, __ldcg(cosines + i), i);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
@@ -522,8 +572,11 @@ __global__ void cosine_argmax_kernel(const float *__restrict__ cosines, int n, i
     __syncthreads();
     if (tid == 0) {
         for (int w = 1; w < 8; ++w) argmax_fold(bv, bi, s_v[w], s_i[w]);
+        const int bad = atomicExch(work + 1, 0);
         out[0] = bi;
         out[1] = __float_as_int(bv);
+        out[2] = bad;
+        work[0] = 0;
     }
 }
 

@@ -52,7 +52,7 @@ struct knnssd_ctx {
     float2 *part_ml = nullptr, *rope_cs = nullptr;
     double *pool_sum = nullptr, *inv_freq = nullptr;
     int *chain = nullptr, *target = nullptr, *prompt = nullptr, *out_tokens = nullptr, *accept_log = nullptr;
-    int *amax_i = nullptr, *flag = nullptr, *knn_out = nullptr;
+    int *amax_i = nullptr, *flag = nullptr, *knn_work = nullptr;
     DeviceState *state = nullptr;
     float *samp_p = nullptr, *samp_q = nullptr;   // sampled decoding: filtered distributions [kMaxRows][vocab], made on first use
     int *samp_res = nullptr;                      // [2] result of a keep-or-resample round
@@ -600,7 +600,7 @@ knnssd_status check_stream_err(knnssd_ctx *c, const char *what) {
 void free_all(knnssd_ctx *c) {
     void *ptrs[] = {c->kcache, c->vcache, c->x, c->qkv, c->attn, c->act, c->logits, c->hfinal, c->part_o, c->pooled,
                     c->anchor_inv_norm, c->cosines, c->amax_v, c->part_ml, c->rope_cs, c->pool_sum, c->inv_freq, c->chain,
-                    c->target, c->prompt, c->out_tokens, c->accept_log, c->amax_i, c->flag, c->knn_out, c->state,
+                    c->target, c->prompt, c->out_tokens, c->accept_log, c->amax_i, c->flag, c->knn_work, c->state,
                     c->ops_full, c->ops_draft, c->bar, c->gabort, c->attn_cnt, c->amax_cnt, c->mpart_o, c->mamax_v, c->mpart_ml,
                     c->mamax_i, c->trace, c->xs_x, c->xs_attn, c->xs_act, c->ssp, c->pf_x, c->pf_qkv, c->pf_ad, c->pf_aq, c->pf_af, c->pf_cs, c->pf_rinv, c->pf_part, c->pf_cnt,
                     c->samp_p, c->samp_q, c->samp_res};
@@ -669,7 +669,7 @@ bool prefill_tensor(knnssd_ctx *c, int n) {
                 ok = ok && prefill::launch_gemm(map_d, scratch, cap, ly.wv, nullptr, nkv, d, T, prefill::PF_STORE, c->pf_qkv, ldq, nq + nkv,
                                                 nullptr, nullptr, 0, err, c->n_sms, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
             }
-            if (!heads_done) prefill::rope_kv_rows_kernel<<<T, 256, 0, s>>>(c->pf_qkv, H, Hkv, HD, c->pf_cs, kc, vc, g.max_seq, t0);
+            if (!heads_done) prefill::rope_kv_rows_kernel<<<dim3(T, prefill::ROPE_PARTS), 256, 0, s>>>(c->pf_qkv, H, Hkv, HD, c->pf_cs, kc, vc, g.max_seq, t0);
             prefill::attn_prompt_kernel<HD><<<dim3(H, (T + 63) / 64), 128, prefill::attn_smem_bytes<HD>(), s>>>(
                 c->pf_qkv, H, Hkv, kc, vc, g.max_seq, t0, T, c->pf_aq, c->pf_aq + (size_t)cap * nq);
             ok = ok && prefill::launch_gemm(map_q, scratch, cap, ly.wo, nullptr, d, nq, T, prefill::PF_ADD, c->pf_x, d, 0, nullptr, nullptr, 0,
@@ -683,9 +683,12 @@ bool prefill_tensor(knnssd_ctx *c, int n) {
         }
         // pooled numerator: every row's final hidden state (mean pooling) or the last row's
         if (g.pool_mode == 0) {
-            rmsnorm_rows_kernel<<<T, 256, 0, s>>>(c->pf_x, c->final_norm, d, g.rms_eps, c->pf_qkv);     // [T][d] scratch
-            pool_accumulate_kernel<<<(d + 255) / 256, 256, 0, s>>>(c->pf_qkv, T, d, c->pool_sum, t0 == 0);
-            c->launches += 2;
+            const int per = 32, slices = (T + per - 1) / per;
+            double *part = reinterpret_cast<double *>(c->pf_qkv);                // [slices][d]: less than the projections' T rows
+            row_scale_kernel<<<T, 256, 0, s>>>(c->pf_x, d, g.rms_eps, c->pf_rinv);
+            pool_partial_kernel<<<dim3((d + 255) / 256, slices), 256, 0, s>>>(c->pf_x, c->pf_rinv, c->final_norm, T, d, per, part);
+            pool_fold_kernel<<<(d + 255) / 256, 256, 0, s>>>(part, slices, d, c->pool_sum, t0 == 0);
+            c->launches += 3;
         } else if (last) {
             rmsnorm_rows_kernel<<<1, 256, 0, s>>>(c->pf_x + (size_t)(T - 1) * d, c->final_norm, d, g.rms_eps, c->hfinal);
             pool_accumulate_kernel<<<(d + 255) / 256, 256, 0, s>>>(c->hfinal, 1, d, c->pool_sum, 1);
@@ -758,14 +761,11 @@ knnssd_status do_select(knnssd_ctx *c, const float *query_dev, int *domain, int 
     if (!query_dev && !c->prefilled) return fail(c, KNNSSD_ERR_STATE, "select_skipset: no pooled vector (prefill first)");
     const int n = g.n_domains * g.anchors_per_domain;
     cudaStream_t s = c->stream;
-    CUDA_TRY(c, cudaMemsetAsync(c->flag, 0, sizeof(int), s));
     cudaEventRecord(c->ev0, s);
-    cosine_scores_kernel<<<(n + 7) / 8, 256, 0, s>>>(query_dev ? query_dev : c->pooled, c->anchors, c->anchor_inv_norm, n,
-                                                     g.d_model, c->cosines, c->flag);
-    cosine_argmax_kernel<<<1, 256, 0, s>>>(c->cosines, n, c->knn_out);
+    cosine_top1_kernel<<<(n + 7) / 8, 256, 0, s>>>(query_dev ? query_dev : c->pooled, c->anchors, c->anchor_inv_norm, n, g.d_model, c->cosines,
+                                                   c->knn_work, c->pinned);
+    CUDA_TRY(c, cudaGetLastError());
     cudaEventRecord(c->ev1, s);
-    CUDA_TRY(c, cudaMemcpyAsync(c->pinned, c->knn_out, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(c, cudaMemcpyAsync(c->pinned + 2, c->flag, sizeof(int), cudaMemcpyDeviceToHost, s));
     knnssd_status st = sync_check(c, "select_skipset");
     if (st != KNNSSD_OK) return st;
     if (c->pinned[2]) return fail(c, KNNSSD_ERR_DEGENERATE, "select_skipset: query has zero or non-finite norm");
@@ -873,7 +873,7 @@ knnssd_status knnssd_init(const knnssd_config *cfg, const knnssd_weights *w, con
     ok &= dev_alloc(&c->out_tokens, (size_t)g.max_seq) == cudaSuccess;
     ok &= dev_alloc(&c->accept_log, (size_t)g.max_seq) == cudaSuccess;
     ok &= dev_alloc(&c->flag, 1) == cudaSuccess;
-    ok &= dev_alloc(&c->knn_out, 2) == cudaSuccess;
+    ok &= dev_alloc(&c->knn_work, 2) == cudaSuccess;
     ok &= dev_alloc(&c->state, 1) == cudaSuccess;
     ok &= dev_alloc(&c->cosines, (size_t)(na > 0 ? na : 1)) == cudaSuccess;
     ok &= dev_alloc(&c->anchor_inv_norm, (size_t)(na > 0 ? na : 1)) == cudaSuccess;
@@ -889,6 +889,7 @@ knnssd_status knnssd_init(const knnssd_config *cfg, const knnssd_weights *w, con
     cudaMemcpyAsync(c->inv_freq, inv_freq.data(), sizeof(double) * inv_freq.size(), cudaMemcpyHostToDevice, c->stream);
     set_state_kernel<<<1, 1, 0, c->stream>>>(c->state, 0, 0);
     cudaMemsetAsync(c->flag, 0, sizeof(int), c->stream);
+    cudaMemsetAsync(c->knn_work, 0, 2 * sizeof(int), c->stream);
     // token buffers start at a valid id, so that a pass that ends early never leaves garbage ids behind
     cudaMemsetAsync(c->chain, 0, sizeof(int) * (kMaxRows + 1), c->stream);
     cudaMemsetAsync(c->target, 0, sizeof(int) * kMaxRows, c->stream);
@@ -1709,15 +1710,13 @@ knnssd_status knnssd_cosine_top1(const float *query_dev, const float *anchors_de
     if (!query_dev || !anchors_dev || n < 1 || d < 1) return KNNSSD_ERR_INVALID_ARG;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
     float *cos_dev = nullptr;
-    int *small = nullptr;  // [0..1] result, [2] flag
+    int *work = nullptr, *host = host_words();
     Scratch scratch(s);
-    if (!scratch.get(&cos_dev, (size_t)n) || !scratch.get(&small, 4)) return KNNSSD_ERR_CUDA;
-    cudaMemsetAsync(small, 0, sizeof(int) * 4, s);
-    cosine_scores_kernel<<<(n + 7) / 8, 256, 0, s>>>(query_dev, anchors_dev, nullptr, n, d, cos_dev, small + 2);
-    cosine_argmax_kernel<<<1, 256, 0, s>>>(cos_dev, n, small);
-    int host[4] = {0, 0, 0, 0};
-    cudaError_t e = cudaMemcpyAsync(host, small, sizeof(int) * 4, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (!host || !scratch.get(&cos_dev, (size_t)n) || !scratch.get(&work, 2)) return KNNSSD_ERR_CUDA;
+    cudaMemsetAsync(work, 0, sizeof(int) * 2, s);
+    cosine_top1_kernel<<<(n + 7) / 8, 256, 0, s>>>(query_dev, anchors_dev, nullptr, n, d, cos_dev, work, host);
+    cudaError_t e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return KNNSSD_ERR_CUDA;
     if (host[2]) return KNNSSD_ERR_DEGENERATE;
     if (best) *best = host[0];
@@ -1728,11 +1727,11 @@ knnssd_status knnssd_cosine_top1(const float *query_dev, const float *anchors_de
 }  // extern "C"
 
 // ---- cosine top-1 without any allocation ------------------------------------------------------------------------
-// Scratch of knnssd_cosine_top1_static: the per-anchor cosines, then four result words (best index, cosine bits,
+// Scratch of knnssd_cosine_top1_static: the per-anchor cosines, then result words and counters (best index, cosine bits,
 // degenerate-input flag, spare).  It lives in the library's device image, one copy per GPU that loads the library.
 // In host code the name below is only a handle for cudaGetSymbolAddress; kernels get the address that call returns.
 namespace {
-constexpr int kStaticWords = KNNSSD_STATIC_MAX_ANCHORS + 4;
+constexpr int kStaticWords = KNNSSD_STATIC_MAX_ANCHORS + 8;
 }  // namespace
 static __device__ __align__(256) float g_top1_static_scratch[kStaticWords];
 
@@ -1763,11 +1762,10 @@ extern "C" knnssd_status knnssd_cosine_top1_static(const float *query_dev, const
     if (static_scratch_address(dev, &scratch) != cudaSuccess) { cudaGetLastError(); return KNNSSD_ERR_CUDA; }
     cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
     float *cos_dev = scratch;
-    int *small = reinterpret_cast<int *>(scratch + KNNSSD_STATIC_MAX_ANCHORS);   // [0..1] result, [2] flag
-    // the array still holds the previous call's result and flag: the words that must start at zero are cleared here
-    if (cudaMemsetAsync(small, 0, sizeof(int) * 4, s) != cudaSuccess) return KNNSSD_ERR_CUDA;
-    cosine_scores_kernel<<<(n + 7) / 8, 256, 0, s>>>(query_dev, anchors_dev, nullptr, n, d, cos_dev, small + 2);
-    cosine_argmax_kernel<<<1, 256, 0, s>>>(cos_dev, n, small);
+    int *small = reinterpret_cast<int *>(scratch + KNNSSD_STATIC_MAX_ANCHORS);   // [0..2] result and flag, [4..5] the kernel's counters
+    // the array still holds what the previous call left: the words that must start at zero are cleared here
+    if (cudaMemsetAsync(small, 0, sizeof(int) * 6, s) != cudaSuccess) return KNNSSD_ERR_CUDA;
+    cosine_top1_kernel<<<(n + 7) / 8, 256, 0, s>>>(query_dev, anchors_dev, nullptr, n, d, cos_dev, small + 4, small);
     int host[4] = {0, 0, 0, 0};
     cudaError_t e = cudaMemcpyAsync(host, small, sizeof(int) * 4, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);

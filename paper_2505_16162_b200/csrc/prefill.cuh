@@ -552,11 +552,17 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant_
 // Row-wise kernels around the contractions
 // ---------------------------------------------------------------------------------------------
 
-// x[t][:] = embedding row of token t (bf16 -> fp32).  grid = T.
+// x[t][:] = embedding row of token t (bf16 -> fp32), eight values per thread and step (d is a multiple of 8).  grid = T.
 __global__ void embed_rows_kernel(const bf16_t *__restrict__ table, const int *__restrict__ tok, int d, float *__restrict__ x) {
     const bf16_t *row = table + (size_t)tok[blockIdx.x] * d;
     float *xr = x + (size_t)blockIdx.x * d;
-    for (int i = threadIdx.x; i < d; i += blockDim.x) xr[i] = bf16_bits_to_float(row[i]);
+    for (int i = threadIdx.x * 8; i < d; i += blockDim.x * 8) {
+        const uint4 w = __ldg(reinterpret_cast<const uint4 *>(row + i));
+        const uint32_t p[4] = {w.x, w.y, w.z, w.w};
+        float4 *dst = reinterpret_cast<float4 *>(xr + i);
+        dst[0] = make_float4(__uint_as_float(p[0] << 16), __uint_as_float(p[0] & 0xFFFF0000u), __uint_as_float(p[1] << 16), __uint_as_float(p[1] & 0xFFFF0000u));
+        dst[1] = make_float4(__uint_as_float(p[2] << 16), __uint_as_float(p[2] & 0xFFFF0000u), __uint_as_float(p[3] << 16), __uint_as_float(p[3] & 0xFFFF0000u));
+    }
 }
 
 // RMSNorm of row t (gain g, epsilon eps) for the contraction that follows: the planes hold v = x g WITHOUT the row's
@@ -604,13 +610,15 @@ __global__ void rope_table_kernel(const double *__restrict__ inv_freq, int pos0,
 }
 
 // Rotary embedding of the q and k heads of row t at position pos0 + t (q in place, fp32); K and V rows rounded to
-// bf16 into the cache.  grid = T, 256 threads: a thread walks pairs (i, i + hd / 2) of the row's H + 2 Hkv head slots.
+// bf16 into the cache.  grid = (T, ROPE_PARTS), 256 threads: a thread walks pairs (i, i + hd / 2) of the row's H + 2 Hkv head
+// slots (in one part, 77 rows of the 13B width took 13 us: 30 steps of dependent latencies, in eight 4).
+constexpr int ROPE_PARTS = 8;
 __global__ void __launch_bounds__(256) rope_kv_rows_kernel(float *__restrict__ qkv, int H, int Hkv, int hd,
                                                            const float2 *__restrict__ table, bf16_t *__restrict__ kc,
                                                            bf16_t *__restrict__ vc, int max_seq, int pos0) {
     const int t = blockIdx.x, half = hd / 2, pos = pos0 + t;
     float *trow = qkv + (size_t)t * (H + 2 * Hkv) * hd;
-    for (int idx = threadIdx.x; idx < (H + 2 * Hkv) * half; idx += 256) {
+    for (int idx = blockIdx.y * 256 + threadIdx.x; idx < (H + 2 * Hkv) * half; idx += 256 * ROPE_PARTS) {
         const int slot = idx / half, i = idx % half;
         float *row = trow + (size_t)slot * hd;
         const float a = row[i], b = row[i + half];
