@@ -14,6 +14,26 @@ namespace knnssd {
 
 typedef unsigned short bf16_t;  // raw bf16 bit pattern
 
+// Kernels that follow one another closely are launched with programmatic stream serialisation: a kernel may be set up on
+// the SMs while the one before it still runs.  Each of them lets its successor come and then waits until the one before it
+// has finished and its writes are visible, before it touches any memory; with an ordinary launch both do nothing.
+// (The fp32 verification pass of 36 kernels of 2 .. 10 us: 279 -> 217 us; a prompt of 77 rows, 8 layers of the 7B widths:
+// 1.68 -> 1.62 ms.)
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// Launch of a kernel that calls chain_wait() before it touches memory.
+template <typename... P, typename... A>
+void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s; cfg.attrs = &attr; cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Codes a kernel may leave in the device error word (besides the codes of bounded waits that gave up, all < 100).
 enum { ERR_BAD_TOKEN = 101, ERR_BAD_LOGITS = 102 };
 
@@ -88,6 +108,7 @@ template <typename WT>
 __global__ void embed_rope_kernel(const WT *__restrict__ E, const int *__restrict__ tok, int d, float *__restrict__ x,
                                   const DeviceState *__restrict__ st, int pos_off, const double *__restrict__ inv_freq,
                                   int half, float2 *__restrict__ cs, int vocab, int *__restrict__ err) {
+    chain_wait();
     const int m = blockIdx.x;
     int t = tok[m];
     if (t < 0 || t >= vocab) {                 // never gather outside the table: report and read row 0 instead
@@ -133,6 +154,7 @@ struct LinearArgs {
 
 template <typename WT, int MT>
 __global__ void __launch_bounds__(256) linear_kernel(const LinearArgs a) {
+    chain_wait();
     __shared__ float s_red[8][MT];
     __shared__ float s_rinv[MT];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -252,6 +274,7 @@ template <typename WT>
 __global__ void rope_kv_kernel(float *__restrict__ qkv, int H, int Hkv, int hd, const float2 *__restrict__ cs,
                                WT *__restrict__ kc, WT *__restrict__ vc, int max_seq,
                                const DeviceState *__restrict__ st, int pos_off) {
+    chain_wait();
     const int head = blockIdx.x, m = blockIdx.y, i = threadIdx.x, half = hd >> 1;
     const int pos = st->len + pos_off + m;
     float *base = qkv + (size_t)m * (H + 2 * Hkv) * hd + (size_t)head * hd;
@@ -288,6 +311,7 @@ __global__ void __launch_bounds__(128) attn_partial_kernel(const float *__restri
                                                             int max_seq, const DeviceState *__restrict__ st, int pos_off,
                                                             float *__restrict__ part_o, float2 *__restrict__ part_ml,
                                                             int n_splits) {
+    chain_wait();
     const int head = blockIdx.x, m = blockIdx.y, split = blockIdx.z;
     const int T = st->len + pos_off + m + 1;           // positions attended: [0, T)
     const int t0 = split * ATT_CHUNK;
@@ -348,6 +372,7 @@ template <int HD>
 __global__ void attn_merge_kernel(const float *__restrict__ part_o, const float2 *__restrict__ part_ml, int H,
                                   const DeviceState *__restrict__ st, int pos_off, int n_splits,
                                   float *__restrict__ out) {
+    chain_wait();
     const int head = blockIdx.x, m = blockIdx.y, e = threadIdx.x;
     const int T = st->len + pos_off + m + 1;
     const int ns = min(n_splits, (T + ATT_CHUNK - 1) / ATT_CHUNK);
@@ -370,6 +395,7 @@ __global__ void attn_merge_kernel(const float *__restrict__ part_o, const float2
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) rmsnorm_rows_kernel(const float *__restrict__ x, const float *__restrict__ gain,
                                                            int d, float eps, float *__restrict__ h) {
+    chain_wait();
     __shared__ float s_red[8];
     const int m = blockIdx.x, tid = threadIdx.x;
     const float *xr = x + (size_t)m * d;
@@ -457,6 +483,7 @@ __device__ __forceinline__ int argmax_checked(int bi, int V, int *err) {
 
 __global__ void __launch_bounds__(256) argmax_partial_kernel(const float *__restrict__ logits, int V, int NB,
                                                              float *__restrict__ pv, int *__restrict__ pi) {
+    chain_wait();
     __shared__ float s_v[8];
     __shared__ int s_i[8];
     const int b = blockIdx.x, m = blockIdx.y, tid = threadIdx.x;
@@ -482,6 +509,7 @@ __global__ void __launch_bounds__(256) argmax_partial_kernel(const float *__rest
 
 __global__ void argmax_final_kernel(const float *__restrict__ pv, const int *__restrict__ pi, int NB, int *__restrict__ out,
                                     int V, int *__restrict__ err) {
+    chain_wait();
     const int m = blockIdx.x, lane = threadIdx.x;
     float bv = -INFINITY;
     int bi = 0x7fffffff;
@@ -503,6 +531,7 @@ __global__ void argmax_final_kernel(const float *__restrict__ pv, const int *__r
 // ---------------------------------------------------------------------------------------------
 __global__ void accept_kernel(int *__restrict__ chain, const int *__restrict__ target, int k, DeviceState *__restrict__ st,
                               int *__restrict__ out_tokens, int out_cap, int *__restrict__ accept_log, int round_idx) {
+    chain_wait();
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     int a = 0;
     while (a < k && target[a] == chain[a + 1]) ++a;

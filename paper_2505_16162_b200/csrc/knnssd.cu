@@ -207,16 +207,16 @@ int pick_mt(int M) {
 
 template <typename WT> void launch_linear_t(const LinearArgs &a, int grid, cudaStream_t s) {
     switch (pick_mt(a.M)) {
-        case 1: linear_kernel<WT, 1><<<grid, 256, 0, s>>>(a); break;
-        case 2: linear_kernel<WT, 2><<<grid, 256, 0, s>>>(a); break;
-        case 3: linear_kernel<WT, 3><<<grid, 256, 0, s>>>(a); break;
-        case 4: linear_kernel<WT, 4><<<grid, 256, 0, s>>>(a); break;
-        case 5: linear_kernel<WT, 5><<<grid, 256, 0, s>>>(a); break;
-        case 6: linear_kernel<WT, 6><<<grid, 256, 0, s>>>(a); break;
-        case 7: linear_kernel<WT, 7><<<grid, 256, 0, s>>>(a); break;
-        case 8: linear_kernel<WT, 8><<<grid, 256, 0, s>>>(a); break;
-        case 9: linear_kernel<WT, 9><<<grid, 256, 0, s>>>(a); break;
-        default: linear_kernel<WT, 16><<<grid, 256, 0, s>>>(a); break;
+        case 1: launch_chained(linear_kernel<WT, 1>, dim3(grid), dim3(256), 0, s, a); break;
+        case 2: launch_chained(linear_kernel<WT, 2>, dim3(grid), dim3(256), 0, s, a); break;
+        case 3: launch_chained(linear_kernel<WT, 3>, dim3(grid), dim3(256), 0, s, a); break;
+        case 4: launch_chained(linear_kernel<WT, 4>, dim3(grid), dim3(256), 0, s, a); break;
+        case 5: launch_chained(linear_kernel<WT, 5>, dim3(grid), dim3(256), 0, s, a); break;
+        case 6: launch_chained(linear_kernel<WT, 6>, dim3(grid), dim3(256), 0, s, a); break;
+        case 7: launch_chained(linear_kernel<WT, 7>, dim3(grid), dim3(256), 0, s, a); break;
+        case 8: launch_chained(linear_kernel<WT, 8>, dim3(grid), dim3(256), 0, s, a); break;
+        case 9: launch_chained(linear_kernel<WT, 9>, dim3(grid), dim3(256), 0, s, a); break;
+        default: launch_chained(linear_kernel<WT, 16>, dim3(grid), dim3(256), 0, s, a); break;
     }
 }
 
@@ -481,7 +481,7 @@ void run_pass_t(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const uns
     const int d = g.d_model, H = g.n_heads, Hkv = g.n_kv_heads, hd = g.head_dim, F = g.d_ff, V = g.vocab;
     const int nq = H * hd, nkv = Hkv * hd;
     cudaStream_t s = c->stream;
-    embed_rope_kernel<WT><<<M, 256, 0, s>>>(reinterpret_cast<const WT *>(c->tok_embed), tok_dev, d, c->x, c->state, pos_off,
+    launch_chained(embed_rope_kernel<WT>, dim3(M), dim3(256), 0, s, reinterpret_cast<const WT *>(c->tok_embed), tok_dev, d, c->x, c->state, pos_off,
                                             c->inv_freq, hd / 2, c->rope_cs, g.vocab, c->err_word);
     c->launches++;
     const size_t layer_stride = (size_t)Hkv * g.max_seq * hd;
@@ -493,18 +493,18 @@ void run_pass_t(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const uns
             ctx_linear(c, a);
             WT *kc = reinterpret_cast<WT *>(c->kcache) + (size_t)l * layer_stride;
             WT *vc = reinterpret_cast<WT *>(c->vcache) + (size_t)l * layer_stride;
-            rope_kv_kernel<WT><<<dim3(H + 2 * Hkv, M), hd / 2, 0, s>>>(c->qkv, H, Hkv, hd, c->rope_cs, kc, vc, g.max_seq,
+            launch_chained(rope_kv_kernel<WT>, dim3(H + 2 * Hkv, M), dim3(hd / 2), 0, s, c->qkv, H, Hkv, hd, c->rope_cs, kc, vc, g.max_seq,
                                                                       c->state, pos_off);
             const dim3 ag(H, M, c->n_splits);
             if (hd == 128) {
-                attn_partial_kernel<WT, 128><<<ag, 128, 0, s>>>(c->qkv, H, Hkv, kc, vc, g.max_seq, c->state, pos_off,
+                launch_chained(attn_partial_kernel<WT, 128>, ag, dim3(128), 0, s, c->qkv, H, Hkv, kc, vc, g.max_seq, c->state, pos_off,
                                                                  c->part_o, c->part_ml, c->n_splits);
-                attn_merge_kernel<128><<<dim3(H, M), 128, 0, s>>>(c->part_o, c->part_ml, H, c->state, pos_off, c->n_splits,
+                launch_chained(attn_merge_kernel<128>, dim3(H, M), dim3(128), 0, s, c->part_o, c->part_ml, H, c->state, pos_off, c->n_splits,
                                                                    c->attn);
             } else {
-                attn_partial_kernel<WT, 64><<<ag, 128, 0, s>>>(c->qkv, H, Hkv, kc, vc, g.max_seq, c->state, pos_off,
+                launch_chained(attn_partial_kernel<WT, 64>, ag, dim3(128), 0, s, c->qkv, H, Hkv, kc, vc, g.max_seq, c->state, pos_off,
                                                                 c->part_o, c->part_ml, c->n_splits);
-                attn_merge_kernel<64><<<dim3(H, M), 64, 0, s>>>(c->part_o, c->part_ml, H, c->state, pos_off, c->n_splits,
+                launch_chained(attn_merge_kernel<64>, dim3(H, M), dim3(64), 0, s, c->part_o, c->part_ml, H, c->state, pos_off, c->n_splits,
                                                                  c->attn);
             }
             c->launches += 3;
@@ -518,16 +518,16 @@ void run_pass_t(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const uns
         }
     }
     if (want_hidden) {
-        rmsnorm_rows_kernel<<<M, 256, 0, s>>>(c->x, c->final_norm, d, g.rms_eps, c->hfinal);
+        launch_chained(rmsnorm_rows_kernel, dim3(M), dim3(256), 0, s, c->x, c->final_norm, d, g.rms_eps, c->hfinal);
         c->launches++;
     }
     if (head_row0 < M) {
         const int hm = M - head_row0;
         ctx_linear(c, make_args(c->lm_head, V, d, c->x + (size_t)head_row0 * d, c->final_norm, g.rms_eps,
                                 c->logits + (size_t)head_row0 * V, EPI_STORE, hm));
-        argmax_partial_kernel<<<dim3(kArgmaxBlocks, hm), 256, 0, s>>>(c->logits + (size_t)head_row0 * V, V, kArgmaxBlocks,
+        launch_chained(argmax_partial_kernel, dim3(kArgmaxBlocks, hm), dim3(256), 0, s, c->logits + (size_t)head_row0 * V, V, kArgmaxBlocks,
                                                                       c->amax_v, c->amax_i);
-        argmax_final_kernel<<<hm, 32, 0, s>>>(c->amax_v, c->amax_i, kArgmaxBlocks, argmax_out, V, c->err_word);
+        launch_chained(argmax_final_kernel, dim3(hm), dim3(32), 0, s, c->amax_v, c->amax_i, kArgmaxBlocks, argmax_out, V, c->err_word);
         c->launches += 2;
     }
 }
@@ -654,7 +654,7 @@ bool prefill_tensor(knnssd_ctx *c, int n) {
             const Layer &ly = c->layers[l];
             bf16_t *kc = reinterpret_cast<bf16_t *>(c->kcache) + (size_t)l * layer_stride;
             bf16_t *vc = reinterpret_cast<bf16_t *>(c->vcache) + (size_t)l * layer_stride;
-            prefill::norm_split_kernel<<<T, 256, 0, s>>>(c->pf_x, d, ly.attn_norm, g.rms_eps, c->pf_ad, c->pf_ad + (size_t)cap * d, c->pf_rinv);
+            launch_chained(prefill::norm_split_kernel, dim3(T), dim3(256), 0, s, c->pf_x, d, ly.attn_norm, g.rms_eps, c->pf_ad, c->pf_ad + (size_t)cap * d, c->pf_rinv);
             bool heads_done = false;     // rotary embedding and K / V rows done by the q / k / v launch's epilogue
             if (nq % prefill::BOX_N == 0 && nkv % prefill::BOX_N == 0) {
                 // q, k and v in one launch over the stacked units (their columns of the projection buffer are adjacent)
@@ -669,12 +669,11 @@ bool prefill_tensor(knnssd_ctx *c, int n) {
                 ok = ok && prefill::launch_gemm(map_d, scratch, cap, ly.wv, nullptr, nkv, d, T, prefill::PF_STORE, c->pf_qkv, ldq, nq + nkv,
                                                 nullptr, nullptr, 0, err, c->n_sms, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
             }
-            if (!heads_done) prefill::rope_kv_rows_kernel<<<dim3(T, prefill::ROPE_PARTS), 256, 0, s>>>(c->pf_qkv, H, Hkv, HD, c->pf_cs, kc, vc, g.max_seq, t0);
-            prefill::attn_prompt_kernel<HD><<<dim3(H, (T + 63) / 64), 128, prefill::attn_smem_bytes<HD>(), s>>>(
-                c->pf_qkv, H, Hkv, kc, vc, g.max_seq, t0, T, c->pf_aq, c->pf_aq + (size_t)cap * nq);
+            if (!heads_done) launch_chained(prefill::rope_kv_rows_kernel, dim3(T, prefill::ROPE_PARTS), dim3(256), 0, s, c->pf_qkv, H, Hkv, HD, c->pf_cs, kc, vc, g.max_seq, t0);
+            launch_chained(prefill::attn_prompt_kernel<HD>, dim3(H, (T + 63) / 64), dim3(128), prefill::attn_smem_bytes<HD>(), s, c->pf_qkv, H, Hkv, kc, vc, g.max_seq, t0, T, c->pf_aq, c->pf_aq + (size_t)cap * nq);
             ok = ok && prefill::launch_gemm(map_q, scratch, cap, ly.wo, nullptr, d, nq, T, prefill::PF_ADD, c->pf_x, d, 0, nullptr, nullptr, 0,
                                             err, c->n_sms, s);
-            prefill::norm_split_kernel<<<T, 256, 0, s>>>(c->pf_x, d, ly.mlp_norm, g.rms_eps, c->pf_ad, c->pf_ad + (size_t)cap * d, c->pf_rinv);
+            launch_chained(prefill::norm_split_kernel, dim3(T), dim3(256), 0, s, c->pf_x, d, ly.mlp_norm, g.rms_eps, c->pf_ad, c->pf_ad + (size_t)cap * d, c->pf_rinv);
             ok = ok && prefill::launch_gemm(map_d, scratch, cap, ly.w_gate, ly.w_up, F, d, T, prefill::PF_SWIGLU, nullptr, 0, 0, c->pf_af,
                                             c->pf_af + (size_t)cap * F, F, err, c->n_sms, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
             ok = ok && prefill::launch_gemm(map_f, scratch, cap, ly.w_down, nullptr, d, F, T, prefill::PF_ADD, c->pf_x, d, 0, nullptr, nullptr,
@@ -791,7 +790,7 @@ void enqueue_draft(knnssd_ctx *c, int k) {
 // Enqueue the verification pass over chain[0..k] and the accept/rollback step.
 void enqueue_verify(knnssd_ctx *c, int k, bool want_hidden, int round_idx) {
     run_pass(c, k + 1, c->chain, 0, nullptr, 0, c->target, want_hidden);
-    accept_kernel<<<1, 32, 0, c->stream>>>(c->chain, c->target, k, c->state, c->out_tokens, c->cfg.max_seq, c->accept_log,
+    launch_chained(accept_kernel, dim3(1), dim3(32), 0, c->stream, c->chain, c->target, k, c->state, c->out_tokens, c->cfg.max_seq, c->accept_log,
                                            round_idx);
     c->launches++;
 }

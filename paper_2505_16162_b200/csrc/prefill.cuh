@@ -263,6 +263,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    chain_wait();                            // barriers and tensor memory are set up under the end of the kernel before
 
     if (warp == 0) {
         if (lane == 0) {
@@ -571,6 +572,7 @@ __global__ void embed_rows_kernel(const bf16_t *__restrict__ table, const int *_
 // bf16 terms - embedding rows with unit gains - stay exact.  grid = T, 256 threads.
 __global__ void __launch_bounds__(256) norm_split_kernel(const float *__restrict__ x, int d, const float *__restrict__ gain, float eps,
                                                          bf16_t *__restrict__ hi, bf16_t *__restrict__ lo, float *__restrict__ rinv_out) {
+    chain_wait();
     __shared__ float part[8];
     const float *xr = x + (size_t)blockIdx.x * d;
     bf16_t *hr = hi + (size_t)blockIdx.x * d, *lr = lo + (size_t)blockIdx.x * d;
@@ -616,6 +618,7 @@ constexpr int ROPE_PARTS = 8;
 __global__ void __launch_bounds__(256) rope_kv_rows_kernel(float *__restrict__ qkv, int H, int Hkv, int hd,
                                                            const float2 *__restrict__ table, bf16_t *__restrict__ kc,
                                                            bf16_t *__restrict__ vc, int max_seq, int pos0) {
+    chain_wait();
     const int t = blockIdx.x, half = hd / 2, pos = pos0 + t;
     float *trow = qkv + (size_t)t * (H + 2 * Hkv) * hd;
     for (int idx = blockIdx.y * 256 + threadIdx.x; idx < (H + 2 * Hkv) * half; idx += 256 * ROPE_PARTS) {
@@ -710,6 +713,7 @@ template <int HD>
 __global__ void __launch_bounds__(128, 2) attn_prompt_kernel(const float *__restrict__ qkv, int H, int Hkv, const bf16_t *__restrict__ kc,
                                                              const bf16_t *__restrict__ vc, int max_seq, int pos0, int T,
                                                              bf16_t *__restrict__ out_hi, bf16_t *__restrict__ out_lo) {
+    chain_wait();
     constexpr int SEG = ATTN_SEG, NT = SEG / 8, KS = HD / 16, VJ = HD / 8, KP = SEG / 16, RB = 64;
     constexpr int CH = HD / 8;                               // 16-byte pieces per row
     constexpr int TILE = SEG * HD * 2;                       // bytes of one K (or V) segment

@@ -157,11 +157,11 @@ inline bool launch_gemm(const CUtensorMap &planes, const GemmScratch &scratch, i
     const bool fuse_heads = heads && bn == 256;
     if (fuse_heads) {
         g.rope = fuse->rope; g.kc = fuse->kc; g.vc = fuse->vc; g.max_seq = fuse->max_seq; g.pos0 = fuse->pos0;
-        gemm_split_kernel<PF_QKV><<<grid, GEMM_THREADS, smem, s>>>(planes, tb0, tb1, tb2, g, cap);
+        launch_chained(gemm_split_kernel<PF_QKV>, grid, dim3(GEMM_THREADS), smem, s, planes, tb0, tb1, tb2, g, cap);
         if (fused) *fused = true;
-    } else if (epi == PF_STORE) gemm_split_kernel<PF_STORE><<<grid, GEMM_THREADS, smem, s>>>(planes, tb0, tb1, tb2, g, cap);
-    else if (epi == PF_ADD) gemm_split_kernel<PF_ADD><<<grid, GEMM_THREADS, smem, s>>>(planes, tb0, tb1, tb2, g, cap);
-    else gemm_split_kernel<PF_SWIGLU><<<grid, GEMM_THREADS, smem, s>>>(planes, tb0, tb1, tb2, g, cap);
+    } else if (epi == PF_STORE) launch_chained(gemm_split_kernel<PF_STORE>, grid, dim3(GEMM_THREADS), smem, s, planes, tb0, tb1, tb2, g, cap);
+    else if (epi == PF_ADD) launch_chained(gemm_split_kernel<PF_ADD>, grid, dim3(GEMM_THREADS), smem, s, planes, tb0, tb1, tb2, g, cap);
+    else launch_chained(gemm_split_kernel<PF_SWIGLU>, grid, dim3(GEMM_THREADS), smem, s, planes, tb0, tb1, tb2, g, cap);
     return true;
 }
 
