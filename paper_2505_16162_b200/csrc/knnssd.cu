@@ -93,7 +93,6 @@ struct knnssd_ctx {
     bf16_t *pf_ad = nullptr, *pf_aq = nullptr, *pf_af = nullptr;   // hi / lo planes [2][cap][d], [2][cap][nq], [2][cap][d_ff]
     CUtensorMap pf_map_d{}, pf_map_q{}, pf_map_f{};
     float *pf_part = nullptr;                                // sums of the pieces of tiles that several CTAs share
-    int *pf_cnt = nullptr;                                   // pieces done so far, zero between launches
 
     // instrumentation
     long long launches = 0;
@@ -465,7 +464,6 @@ void reset_mega_state(knnssd_ctx *c) {
     cudaMemset(c->gabort, 0, sizeof(int));
     cudaMemset(c->attn_cnt, 0, sizeof(int) * pass::MAXM * c->cfg.n_heads);
     cudaMemset(c->amax_cnt, 0, sizeof(int));
-    if (c->pf_cnt) cudaMemset(c->pf_cnt, 0, prefill::PIECE_COUNTERS * sizeof(int));
     c->bar_total = 0;
 }
 
@@ -602,7 +600,7 @@ void free_all(knnssd_ctx *c) {
                     c->anchor_inv_norm, c->cosines, c->amax_v, c->part_ml, c->rope_cs, c->pool_sum, c->inv_freq, c->chain,
                     c->target, c->prompt, c->out_tokens, c->accept_log, c->amax_i, c->flag, c->knn_work, c->state,
                     c->ops_full, c->ops_draft, c->bar, c->gabort, c->attn_cnt, c->amax_cnt, c->mpart_o, c->mamax_v, c->mpart_ml,
-                    c->mamax_i, c->trace, c->xs_x, c->xs_attn, c->xs_act, c->ssp, c->pf_x, c->pf_qkv, c->pf_ad, c->pf_aq, c->pf_af, c->pf_cs, c->pf_rinv, c->pf_part, c->pf_cnt,
+                    c->mamax_i, c->trace, c->xs_x, c->xs_attn, c->xs_act, c->ssp, c->pf_x, c->pf_qkv, c->pf_ad, c->pf_aq, c->pf_af, c->pf_cs, c->pf_rinv, c->pf_part,
                     c->samp_p, c->samp_q, c->samp_res};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -636,8 +634,12 @@ bool prefill_tensor(knnssd_ctx *c, int n) {
     cudaStream_t s = c->stream;
     int *err = c->err_word;
     const size_t layer_stride = (size_t)Hkv * g.max_seq * HD;
-    const prefill::GemmScratch scratch{c->pf_part, c->pf_cnt};
     bool ok = true;
+    auto contract = [&](auto... a) {
+        const int n_launched = prefill::launch_gemm(a...);
+        c->launches += n_launched;
+        return n_launched > 0;
+    };
     for (int t0 = 0; t0 < n && ok; t0 += cap) {
         const int T = n - t0 < cap ? n - t0 : cap;
         const bool last = t0 + T == n;
@@ -659,26 +661,26 @@ bool prefill_tensor(knnssd_ctx *c, int n) {
             if (nq % prefill::BOX_N == 0 && nkv % prefill::BOX_N == 0) {
                 // q, k and v in one launch over the stacked units (their columns of the projection buffer are adjacent)
                 const prefill::QkvFuse fuse{c->pf_cs, kc, vc, g.max_seq, t0, HD};
-                ok = ok && prefill::launch_gemm(map_d, scratch, cap, ly.wq, ly.wk, ldq, d, T, prefill::PF_STORE, c->pf_qkv, ldq, 0, nullptr,
+                ok = ok && contract(map_d, c->pf_part, cap, ly.wq, ly.wk, ldq, d, T, prefill::PF_STORE, c->pf_qkv, ldq, 0, nullptr,
                                                 nullptr, 0, err, c->n_sms, s, ly.wv, nq, nkv, &fuse, &heads_done, c->pf_rinv);
             } else {
-                ok = ok && prefill::launch_gemm(map_d, scratch, cap, ly.wq, nullptr, nq, d, T, prefill::PF_STORE, c->pf_qkv, ldq, 0, nullptr,
+                ok = ok && contract(map_d, c->pf_part, cap, ly.wq, nullptr, nq, d, T, prefill::PF_STORE, c->pf_qkv, ldq, 0, nullptr,
                                                 nullptr, 0, err, c->n_sms, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
-                ok = ok && prefill::launch_gemm(map_d, scratch, cap, ly.wk, nullptr, nkv, d, T, prefill::PF_STORE, c->pf_qkv, ldq, nq, nullptr,
+                ok = ok && contract(map_d, c->pf_part, cap, ly.wk, nullptr, nkv, d, T, prefill::PF_STORE, c->pf_qkv, ldq, nq, nullptr,
                                                 nullptr, 0, err, c->n_sms, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
-                ok = ok && prefill::launch_gemm(map_d, scratch, cap, ly.wv, nullptr, nkv, d, T, prefill::PF_STORE, c->pf_qkv, ldq, nq + nkv,
+                ok = ok && contract(map_d, c->pf_part, cap, ly.wv, nullptr, nkv, d, T, prefill::PF_STORE, c->pf_qkv, ldq, nq + nkv,
                                                 nullptr, nullptr, 0, err, c->n_sms, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
             }
             if (!heads_done) launch_chained(prefill::rope_kv_rows_kernel, dim3(T, prefill::ROPE_PARTS), dim3(256), 0, s, c->pf_qkv, H, Hkv, HD, c->pf_cs, kc, vc, g.max_seq, t0);
             launch_chained(prefill::attn_prompt_kernel<HD>, dim3(H, (T + 63) / 64), dim3(128), prefill::attn_smem_bytes<HD>(), s, c->pf_qkv, H, Hkv, kc, vc, g.max_seq, t0, T, c->pf_aq, c->pf_aq + (size_t)cap * nq);
-            ok = ok && prefill::launch_gemm(map_q, scratch, cap, ly.wo, nullptr, d, nq, T, prefill::PF_ADD, c->pf_x, d, 0, nullptr, nullptr, 0,
+            ok = ok && contract(map_q, c->pf_part, cap, ly.wo, nullptr, d, nq, T, prefill::PF_ADD, c->pf_x, d, 0, nullptr, nullptr, 0,
                                             err, c->n_sms, s);
             launch_chained(prefill::norm_split_kernel, dim3(T), dim3(256), 0, s, c->pf_x, d, ly.mlp_norm, g.rms_eps, c->pf_ad, c->pf_ad + (size_t)cap * d, c->pf_rinv);
-            ok = ok && prefill::launch_gemm(map_d, scratch, cap, ly.w_gate, ly.w_up, F, d, T, prefill::PF_SWIGLU, nullptr, 0, 0, c->pf_af,
+            ok = ok && contract(map_d, c->pf_part, cap, ly.w_gate, ly.w_up, F, d, T, prefill::PF_SWIGLU, nullptr, 0, 0, c->pf_af,
                                             c->pf_af + (size_t)cap * F, F, err, c->n_sms, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
-            ok = ok && prefill::launch_gemm(map_f, scratch, cap, ly.w_down, nullptr, d, F, T, prefill::PF_ADD, c->pf_x, d, 0, nullptr, nullptr,
+            ok = ok && contract(map_f, c->pf_part, cap, ly.w_down, nullptr, d, F, T, prefill::PF_ADD, c->pf_x, d, 0, nullptr, nullptr,
                                             0, err, c->n_sms, s);
-            c->launches += ((nq % prefill::BOX_N == 0 && nkv % prefill::BOX_N == 0) ? 9 : 11) - (heads_done ? 1 : 0);
+            c->launches += heads_done ? 3 : 4;                   // besides the contractions
         }
         // pooled numerator: every row's final hidden state (mean pooling) or the last row's
         if (g.pool_mode == 0) {
@@ -934,9 +936,7 @@ knnssd_status knnssd_init(const knnssd_config *cfg, const knnssd_weights *w, con
             ok3 &= dev_alloc(&c->pf_aq, 2 * cap * nq) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_af, 2 * cap * g.d_ff) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_part, (size_t)prefill::MAX_PIECES * prefill::PIECE_FLOATS) == cudaSuccess;
-            ok3 &= dev_alloc(&c->pf_cnt, (size_t)prefill::PIECE_COUNTERS) == cudaSuccess;
             if (!ok3) { cudaGetLastError(); return bail(KNNSSD_ERR_CUDA); }
-            cudaMemsetAsync(c->pf_cnt, 0, prefill::PIECE_COUNTERS * sizeof(int), c->stream);
             cudaMemsetAsync(c->pf_ad, 0, 2 * cap * d * sizeof(bf16_t), c->stream);
             cudaMemsetAsync(c->pf_aq, 0, 2 * cap * nq * sizeof(bf16_t), c->stream);
             cudaMemsetAsync(c->pf_af, 0, 2 * cap * g.d_ff * sizeof(bf16_t), c->stream);
@@ -1484,19 +1484,18 @@ knnssd_status knnssd_gemm_split(const void *W0_dev, const void *W1_dev, int n_ou
     cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev);
     const int cap = (T + prefill::BM - 1) / prefill::BM * prefill::BM;
     bf16_t *planes = nullptr, *outp = nullptr;
-    prefill::GemmScratch scratch{};
+    float *part = nullptr;
     const size_t plane = (size_t)cap * n_in, oplane = (size_t)T * n_out;
     Scratch mem(s);
     if (!mem.get(&planes, 2 * plane) || (mode == 2 && !mem.get(&outp, 2 * oplane)) ||
-        !mem.get(&scratch.part, (size_t)prefill::MAX_PIECES * prefill::PIECE_FLOATS) || !mem.get(&scratch.piece_cnt, (size_t)prefill::PIECE_COUNTERS))
+        !mem.get(&part, (size_t)prefill::MAX_PIECES * prefill::PIECE_FLOATS))
         return KNNSSD_ERR_CUDA;
-    cudaMemsetAsync(scratch.piece_cnt, 0, prefill::PIECE_COUNTERS * sizeof(int), s);
     knnssd_status st = KNNSSD_OK;
     cudaMemsetAsync(planes, 0, 2 * plane * sizeof(bf16_t), s);
     prefill::split_rows_kernel<<<T, 256, 0, s>>>(x_dev, n_in, planes, planes + plane);
     CUtensorMap ta;
     if (!prefill::make_map(&ta, planes, (size_t)2 * cap, (size_t)n_in, prefill::act_box_rows(T)) ||
-        !prefill::launch_gemm(ta, scratch, cap, W0_dev, W1_dev, n_out, n_in, T, mode, y_dev, n_out, 0, outp, outp ? outp + oplane : nullptr,
+        !prefill::launch_gemm(ta, part, cap, W0_dev, W1_dev, n_out, n_in, T, mode, y_dev, n_out, 0, outp, outp ? outp + oplane : nullptr,
                               n_out, stream_err_ptr(), n_sms, s))
         st = KNNSSD_ERR_CUDA;
     if (st == KNNSSD_OK && mode == 2) prefill::join_planes_kernel<<<T, 256, 0, s>>>(outp, outp + oplane, n_out, y_dev);

@@ -68,8 +68,8 @@ struct GemmArgs {
                        // whatever its height: 0.75 -> 0.6 us per k-block of 256 columns for the copies alone)
     int a_rows;        // rows of an activation box (the maps' box height): BM, or T rounded up to 8 where T < BM
     int whole;         // tiles [0, whole) are done whole by one CTA each, the others in pieces (see Jobs below)
-    float *part;       // the chunk sums of the tiles done in pieces, [tiles_x tiles_y - whole][chunks][PIECE_FLOATS]
-    int *piece_cnt;    // [tiles done in pieces][8 epilogue warps], zero between launches
+    float *part;       // the chunk sums of the tiles done in pieces, [tiles_x tiles_y - whole][chunks][PIECE_FLOATS]: what
+                       // gemm_split_kernel leaves and fold_pieces_kernel picks up
     int nA, nB;        // STORE over stacked matrices (q, k, v in one launch): units [0, nA) are rows of map tb0,
                        // [nA, nA + nB) rows of tb1, the rest rows of tb2; all multiples of BOX_N.  One matrix: nA = N
     // PF_QKV (stacked q, k, v; head dimension 128, bn = 256: an epilogue thread holds one head of its token): the q
@@ -151,12 +151,6 @@ __device__ __forceinline__ bool pf_wait(uint64_t *b, uint32_t parity, volatile i
     return true;
 }
 
-__device__ __forceinline__ int ld_acquire_int(const int *p) {
-    int v;
-    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
 // 32 bytes, a sector: in one access at a 32-byte boundary (whole), else in two at a 16-byte boundary.
 __device__ __forceinline__ void ld_sector(const float *p, float (&v)[8], bool whole) {
     if (whole) {
@@ -184,11 +178,9 @@ __device__ __forceinline__ uint32_t pack_bf16(uint32_t lo16, uint32_t hi16) { re
 // tiles each instead cost 1.05 us per k-block against 0.81: the weights of all column tiles in flight at once).  The
 // chunks (CHUNK_KB k-blocks) of the tiles that are left, fewer than the CTAs, are dealt out evenly, CTA c of P getting
 // chunks [c U / P, (c + 1) U / P): a last round that would leave most of the chip idle takes the time its work takes.
-// A piece's chunk sums go to `part` one by one; once all of a tile's are there (every CTA has left all of its
-// own before it waits for others, and nothing it waits for waits for it; the wait is bounded) the tile's CTAs take an eighth
-// of its columns each and add them up from the first chunk to the last, the order of a tile done whole: a row's
-// numbers do not depend on how the launch was dealt out.  Epilogue warp w of every CTA has the same 32 rows x half of
-// the columns of a tile, so counting and waiting are per warp.
+// A piece's chunk sums go to `part` one by one, and fold_pieces_kernel, launched behind, adds a tile's up from the first chunk
+// to the last, the order of a tile done whole: a row's numbers do not depend on how the launch was dealt out.  No CTA waits
+// for another: a launch that is not cooperative may run in parts, with another stream's launch on the SMs between them.
 struct Jobs {
     int G, P, cta, whole, nchunks, n_whole, r0;      // P: the CTAs that get pieces, one chunk each at least
     long long units, u0, u1;
@@ -212,9 +204,96 @@ struct Jobs {
         c1 = (int)min((long long)nchunks, u1 - first);
         return true;
     }
-    __device__ __forceinline__ int cta_of(long long u) const { return (int)(((u + 1) * P - 1) / units); }   // the CTA that has unit u
 };
 constexpr int PIECE_FLOATS = BM * BN_MAX;      // a chunk's sums, by register group and thread (coalesced): 32 x 256 float4
+
+// Tile column of register group gi (32 columns) of an epilogue thread, or -1 if the group is not in use.  Store / add: half
+// hsel of the columns in groups of 32; SwiGLU: groups 0 and 1 a quarter of them in the gate columns, 2 and 3 the up columns of
+// the same units.
+template <int EPI> __device__ __forceinline__ int group_col(int gi, int hsel, int bn) {
+    if (EPI == PF_SWIGLU) {
+        const int gg = gi & 1, qtr = bn / 4;
+        return 32 * gg < qtr ? (gi >= 2 ? bn / 2 : 0) + hsel * qtr + 32 * gg : -1;
+    }
+    return 32 * gi < bn / 2 ? hsel * (bn / 2) + 32 * gi : -1;
+}
+
+// What becomes of 16 sums of token t of a tile: register k8 .. k8 + 7 in v[0 .. 7], 64 + k8 .. in v[8 .. 15] (k8 = 8 k).
+// SwiGLU: gate and up columns of eight units; q / k / v heads: eight pairs (j, j + 64) of one head; else columns.
+// y32: y lies at a 32-byte boundary (ldy, col0 and the columns are multiples of 8).
+template <int EPI>
+__device__ __forceinline__ void finish_sums(const GemmArgs &g, int tile, int t, int hsel, int k8, bool y32, float (&v)[16]) {
+    const int half = g.bn / 2, qtr = g.bn / 4;
+    const int n0 = (tile / g.tiles_x) * (EPI == PF_SWIGLU ? half : g.bn);
+    if (g.row_scale) {
+        const float rs = g.row_scale[t];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] *= rs;
+    }
+    if (EPI == PF_SWIGLU) {
+        const int u = n0 + hsel * qtr + k8;
+        if (k8 >= qtr || u >= g.N) return;
+        uint32_t hi[4], lo[4];
+#pragma unroll
+        for (int i = 0; i < 8; i += 2) {
+            uint32_t h2[2], l2[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float gt = v[i + e], up = v[8 + i + e];
+                const float a = gt / (1.0f + expf(-gt)) * up;
+                h2[e] = float_to_bf16_rne(a);
+                l2[e] = float_to_bf16_rne(a - __uint_as_float(h2[e] << 16));
+            }
+            hi[i >> 1] = pack_bf16(h2[0], h2[1]);
+            lo[i >> 1] = pack_bf16(l2[0], l2[1]);
+        }
+        *reinterpret_cast<uint4 *>(g.out_hi + (size_t)t * g.ldo + u) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        *reinterpret_cast<uint4 *>(g.out_lo + (size_t)t * g.ldo + u) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    } else if (EPI == PF_QKV) {
+        const int u0 = n0 + hsel * 128;                  // the head's first unit of the stacked q / k / v units
+        if (u0 >= g.N) return;
+        if (u0 < g.nA + g.nB) {                          // a q or a k head: rotary embedding
+            const float2 *cs = g.rope + (size_t)t * 64 + k8;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float2 c = cs[i];
+                const float a = v[i], b = v[8 + i];
+                v[i] = a * c.x - b * c.y;
+                v[8 + i] = b * c.x + a * c.y;
+            }
+        }
+        const bool is_k = u0 < g.nA + g.nB;
+        const int kvh = (u0 - g.nA - (is_k ? 0 : g.nB)) >> 7;
+#pragma unroll
+        for (int e = 0; e < 16; e += 8) {
+            if (u0 < g.nA) {
+                float *yp = g.y + (size_t)t * g.ldy + g.col0 + u0 + 8 * e + k8;
+                float o[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) o[i] = v[e + i];
+                st_sector(yp, o, y32);
+            } else {
+                bf16_t *dst = (is_k ? g.kc : g.vc) + ((size_t)kvh * g.max_seq + g.pos0 + t) * 128 + 8 * e + k8;
+                uint32_t w[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) w[i] = pack_bf16(float_to_bf16_rne(v[e + 2 * i]), float_to_bf16_rne(v[e + 2 * i + 1]));
+                *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < 16; e += 8) {
+            const int r = 8 * e + k8, n = n0 + hsel * half + r;
+            if (r >= half || n >= g.N) continue;         // N is a multiple of 8
+            float *yp = g.y + (size_t)t * g.ldy + g.col0 + n;
+            float o[8], x[8];
+            if (EPI == PF_ADD) ld_sector(yp, x, y32);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) o[i] = EPI == PF_ADD ? v[e + i] + x[i] : v[e + i];
+            st_sector(yp, o, y32);
+        }
+    }
+}
 
 // Tiles of 128 tokens x bn accumulator columns, dealt out to one CTA per SM (Jobs).  EPI = PF_SWIGLU: columns [0, bn / 2) are units n0 .. of
 // the gate matrix (map tb0) and columns [bn / 2, bn) the same units of the up matrix (map tb1); otherwise the columns
@@ -342,100 +421,17 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant_
         //      [hsel bn / 4, + bn / 4), acc[64 .. 127] the up columns of the same units ----
         const int q = warp & 3, hsel = (warp - 2) >> 2;
         const uint32_t trow = tmem + ((uint32_t)(32 * q) << 16);
-        const int half = bn / 2, qtr = bn / 4;
+        const int half = bn / 2;
         const bool y32 = (reinterpret_cast<uintptr_t>(g.y) & 31u) == 0;      // ldy, col0 and the columns are multiples of 8
-        // tile column of register group gi (32 columns), or -1 if the group is not in use
-        auto group_col = [&](int gi) -> int {
-            if (EPI == PF_SWIGLU) {
-                const int gg = gi & 1;
-                if (32 * gg >= qtr) return -1;
-                return (gi >= 2 ? per : 0) + hsel * qtr + 32 * gg;
-            }
-            return 32 * gi < half ? hsel * half + 32 * gi : -1;
-        };
         bool ok = true;
         int cg = 0;                          // chunks taken so far, over all of this CTA's tiles
         const int et = threadIdx.x - 64;     // this thread among the epilogue threads
-        // the sums of piece r's chunk c as this thread's float4s, 256 apart; its counter
+        // the sums of piece r's chunk c as this thread's float4s, 256 apart
         auto part_of = [&](int r, int c) { return reinterpret_cast<float4 *>(g.part + ((size_t)r * nchunks + c) * PIECE_FLOATS) + et; };
-        auto counter = [&](int r) { return g.piece_cnt + (size_t)r * EPI_WARPS + (warp - 2); };
-        // What becomes of 16 sums of token t of a tile: register k8 .. k8 + 7 in v[0 .. 7], 64 + k8 .. in v[8 .. 15] (k8 = 8 k).
-        // SwiGLU: gate and up columns of eight units; q / k / v heads: eight pairs (j, j + 64) of one head; else columns.
-        auto finish = [&](int tile, int t, int k8, float (&v)[16]) {
-            const int n0 = (tile / g.tiles_x) * per;
-            if (g.row_scale) {
-                const float rs = g.row_scale[t];
-#pragma unroll
-                for (int i = 0; i < 16; ++i) v[i] *= rs;
-            }
-            if (EPI == PF_SWIGLU) {
-                const int u = n0 + hsel * qtr + k8;
-                if (k8 >= qtr || u >= g.N) return;
-                uint32_t hi[4], lo[4];
-#pragma unroll
-                for (int i = 0; i < 8; i += 2) {
-                    uint32_t h2[2], l2[2];
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const float gt = v[i + e], up = v[8 + i + e];
-                        const float a = gt / (1.0f + expf(-gt)) * up;
-                        h2[e] = float_to_bf16_rne(a);
-                        l2[e] = float_to_bf16_rne(a - __uint_as_float(h2[e] << 16));
-                    }
-                    hi[i >> 1] = pack_bf16(h2[0], h2[1]);
-                    lo[i >> 1] = pack_bf16(l2[0], l2[1]);
-                }
-                *reinterpret_cast<uint4 *>(g.out_hi + (size_t)t * g.ldo + u) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-                *reinterpret_cast<uint4 *>(g.out_lo + (size_t)t * g.ldo + u) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-            } else if (EPI == PF_QKV) {
-                const int u0 = n0 + hsel * 128;                  // the head's first unit of the stacked q / k / v units
-                if (u0 >= g.N) return;
-                if (u0 < g.nA + g.nB) {                          // a q or a k head: rotary embedding
-                    const float2 *cs = g.rope + (size_t)t * 64 + k8;
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const float2 c = cs[i];
-                        const float a = v[i], b = v[8 + i];
-                        v[i] = a * c.x - b * c.y;
-                        v[8 + i] = b * c.x + a * c.y;
-                    }
-                }
-                const bool is_k = u0 < g.nA + g.nB;
-                const int kvh = (u0 - g.nA - (is_k ? 0 : g.nB)) >> 7;
-#pragma unroll
-                for (int e = 0; e < 16; e += 8) {
-                    if (u0 < g.nA) {
-                        float *yp = g.y + (size_t)t * g.ldy + g.col0 + u0 + 8 * e + k8;
-                        float o[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) o[i] = v[e + i];
-                        st_sector(yp, o, y32);
-                    } else {
-                        bf16_t *dst = (is_k ? g.kc : g.vc) + ((size_t)kvh * g.max_seq + g.pos0 + t) * 128 + 8 * e + k8;
-                        uint32_t w[4];
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) w[i] = pack_bf16(float_to_bf16_rne(v[e + 2 * i]), float_to_bf16_rne(v[e + 2 * i + 1]));
-                        *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int e = 0; e < 16; e += 8) {
-                    const int r = 8 * e + k8, n = n0 + hsel * half + r;
-                    if (r >= half || n >= g.N) continue;         // N is a multiple of 8
-                    float *yp = g.y + (size_t)t * g.ldy + g.col0 + n;
-                    float o[8], x[8];
-                    if (EPI == PF_ADD) ld_sector(yp, x, y32);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) o[i] = EPI == PF_ADD ? v[e + i] + x[i] : v[e + i];
-                    st_sector(yp, o, y32);
-                }
-            }
-        };
         int tile, c_begin, c_end, i = 0;
         for (; ok && jobs.get(i, tile, c_begin, c_end); ++i) {
         const int t = (tile % g.tiles_x) * BM + 32 * q + lane;
-        const bool piece = c_end - c_begin < nchunks;
+        const bool piece = tile >= g.whole;
         float acc[128];
 #pragma unroll
         for (int i = 0; i < 128; ++i) acc[i] = 0.f;
@@ -447,7 +443,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant_
             tc_fence_after();
 #pragma unroll
             for (int gi = 0; gi < 4; ++gi) {
-                const int col = group_col(gi);
+                const int col = group_col<EPI>(gi, hsel, bn);
                 if (col >= 0) {                          // warp-uniform
                     float v[32];
                     tmem_ld32(trow + (uint32_t)(b * BN_MAX + col), v);
@@ -468,11 +464,8 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant_
             if (lane == 0) stream::mbar_arrive(&acc_empty[b]);
         }
         if (!ok) break;
-        if (piece) {
-            __threadfence();
-            __syncwarp();
-            if (lane == 0) atomicAdd(counter(tile - g.whole), c_end - c_begin);
-        } else if (t < g.T && (EPI == PF_STORE || EPI == PF_ADD)) {
+        if (piece) continue;                 // fold_pieces_kernel goes on from here
+        if (t < g.T && (EPI == PF_STORE || EPI == PF_ADD)) {
             // columns: 32 at a time, in 32-byte accesses (a sector each), the old values of a group fetched together
             const float rs = g.row_scale ? g.row_scale[t] : 1.0f;
 #pragma unroll
@@ -502,44 +495,10 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant_
                 float v[16];
 #pragma unroll
                 for (int e = 0; e < 8; ++e) { v[e] = acc[8 * k + e]; v[8 + e] = acc[64 + 8 * k + e]; }
-                finish(tile, t, 8 * k, v);
+                finish_sums<EPI>(g, tile, t, hsel, 8 * k, y32, v);
             }
         }
         }                                    // next job: its first chunks are already accumulating in tensor memory
-        // ---- this CTA's share of the tiles it has a piece of (at most two: its range is no longer than a tile's) ----
-        for (i = jobs.n_whole; ok && jobs.get(i, tile, c_begin, c_end); ++i) {
-            if (c_end - c_begin == nchunks) continue;
-            const int r = tile - g.whole, t = (tile % g.tiles_x) * BM + 32 * q + lane;
-            const int first = jobs.cta_of((long long)r * nchunks), n_ctas = min(8, jobs.cta_of((long long)(r + 1) * nchunks - 1) - first + 1);
-            if (jobs.cta - first >= n_ctas) continue;
-            int *cnt = counter(r), seen = 0;
-            unsigned spins = 0;
-            while (((seen = ld_acquire_int(cnt)) & 0xFFFF) < nchunks && !*cta_abort)
-                if (++spins > WAIT_LIMIT) { *cta_abort = 1; atomicExch(g.err, 25); }
-            ok = __all_sync(0xffffffffu, (seen & 0xFFFF) >= nchunks);
-            if (!ok) break;
-            for (int k = jobs.cta - first; k < 8; k += n_ctas) {
-                // registers 8 k .. and 64 + 8 k ..: not all are in use in tiles of fewer columns
-                const bool two = group_col(2 + (k >> 2)) >= 0;
-                if (group_col(k >> 2) < 0 || t >= g.T) continue;
-                float v[16];
-#pragma unroll
-                for (int e = 0; e < 16; ++e) v[e] = 0.f;
-#pragma unroll 8
-                for (int c = 0; c < nchunks; ++c) {
-                    const float4 *src = part_of(r, c) + 2 * k * 256;
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        if (e >= 2 && !two) continue;
-                        const float4 x = __ldcg(src + ((e & 1) + 16 * (e >> 1)) * 256);
-                        v[4 * e] += x.x; v[4 * e + 1] += x.y; v[4 * e + 2] += x.z; v[4 * e + 3] += x.w;
-                    }
-                }
-                finish(tile, t, 8 * k, v);
-            }
-            __syncwarp();
-            if (lane == 0 && (atomicAdd(cnt, 0x10000) >> 16) == n_ctas - 1) *cnt = 0;      // the last of them: idle again
-        }
     }
     tc_fence_before();
     __syncthreads();
@@ -547,6 +506,42 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant_
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
     }
+}
+
+// The tiles of a launch that were done in pieces: adds up the chunk sums of each, first chunk to last, and finishes them as
+// gemm_split_kernel finishes a tile done whole.  grid = 8 (tiles - whole), 256 threads: block 8 r + k has registers 8 k ..
+// and 64 + 8 k .. of piece r's epilogue threads.  Bound by reading the sums back from L2, which all SMs share here; taken by the
+// contraction's own CTAs, each waiting for its tile's last, a prompt of 77 rows (8 layers, 7B widths) took 1.62 ms, so 1.51.
+template <int EPI>
+__global__ void __launch_bounds__(256) fold_pieces_kernel(const GemmArgs g) {
+    chain_wait();
+    const int r = blockIdx.x >> 3, k = blockIdx.x & 7, tile = g.whole + r, warp = threadIdx.x >> 5;
+    const int hsel = warp >> 2, t = (tile % g.tiles_x) * BM + 32 * ((warp + 2) & 3) + (threadIdx.x & 31);
+    // not all registers are in use in tiles of fewer columns
+    const bool one = group_col<EPI>(k >> 2, hsel, g.bn) >= 0, two = group_col<EPI>(2 + (k >> 2), hsel, g.bn) >= 0;
+    if (!one || t >= g.T) return;
+    const int nchunks = (g.K / BK + CHUNK_KB - 1) / CHUNK_KB;
+    const float4 *src = reinterpret_cast<const float4 *>(g.part + (size_t)r * nchunks * PIECE_FLOATS) + 2 * k * 256 + threadIdx.x;
+    float v[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) v[e] = 0.f;
+    constexpr int B = 8;                                     // chunks in flight: 16 KB a warp
+    for (int c0 = 0; c0 < nchunks; c0 += B) {
+        float4 x[B][4];
+#pragma unroll
+        for (int c = 0; c < B; ++c)
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (c0 + c < nchunks && (e < 2 || two)) x[c][e] = __ldcg(src + (size_t)(c0 + c) * (PIECE_FLOATS / 4) + ((e & 1) + 16 * (e >> 1)) * 256);
+#pragma unroll
+        for (int c = 0; c < B; ++c)
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (c0 + c < nchunks && (e < 2 || two)) {
+                    v[4 * e] += x[c][e].x; v[4 * e + 1] += x[c][e].y; v[4 * e + 2] += x[c][e].z; v[4 * e + 3] += x[c][e].w;
+                }
+    }
+    finish_sums<EPI>(g, tile, t, hsel, 8 * k, (reinterpret_cast<uintptr_t>(g.y) & 31u) == 0, v);
 }
 
 // ---------------------------------------------------------------------------------------------

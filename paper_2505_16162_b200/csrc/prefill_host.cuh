@@ -70,7 +70,7 @@ struct Deal { int bn, grid, whole; };
 //   whole tiles: 8 us + rounds x k-blocks x 0.5 / 0.62 / 0.73 us - the products of a k-block take that long (both terms'
 //     operands leave shared memory at ~64 bytes per clock), copies and sums run under them.  5120 units x 1024 rows, 256
 //     columns: two rounds 144 us, of which the second has 12 tiles.
-//   pieces: 14 us for the two meetings and the last sums, 1.3 x the products' time (pieces are not in step, so they share
+//   pieces: 14 us for a launch, the fold behind it and the last sums, 1.3 x the products' time (pieces are not in step, so they share
 //     less through L2), and per chunk sum 0.012 us + 0.036 us per 128 KB to write and read it.  The same launch: one
 //     round + 12 tiles in 120 pieces, 93 us; at 77 rows, 20 tiles in 200 pieces 33 us against 63 us.
 // `heads`: 256 columns let the launch finish the heads itself; else a kernel of its own does.
@@ -105,17 +105,10 @@ inline Deal deal_out(int T, int N, int K, bool swiglu, bool heads, int n_sms) {
 // whatever the stage held before; they meet no live row).
 inline int act_box_rows(int T) { return T >= BM ? BM : (T + 7) / 8 * 8; }
 
-// Scratch of one launch: a launch finds the counters at zero and leaves them at zero.
-struct GemmScratch {
-    float *part;           // MAX_PIECES * PIECE_FLOATS
-    int *piece_cnt;        // PIECE_COUNTERS
-};
-constexpr int PIECE_COUNTERS = MAX_PIECES * (GEMM_THREADS / 32 - 2);
-
 // One contraction over T rows.  `planes` = the activation map (hi rows [0, cap), lo rows [cap, 2 cap)); W0 (and W1 for
 // SwiGLU: W0 = gate, W1 = up) are [N][K] bf16.  STORE with W1 and W2 given: the three matrices (nA, nB and nC rows, all
 // multiples of BOX_N) are stacked along the output units, N = nA + nB + nC, one launch for q, k and v.
-// Returns false if a tensor map could not be made.
+// `part`: scratch of MAX_PIECES * PIECE_FLOATS.  Returns the number of kernels launched, 0 if a tensor map could not be made.
 // What the q / k / v launch needs to finish the heads in its epilogue (rotary embedding, K / V rows into the cache).
 struct QkvFuse {
     const float2 *rope;    // [T][64]
@@ -126,12 +119,12 @@ struct QkvFuse {
 // `fuse` (stacked q, k, v only): if the head dimension is 128 and the launch takes 256-column tiles, the epilogue does
 // the rotary embedding and writes K / V to the cache itself; *fused says whether it did (otherwise the caller runs
 // rope_kv_rows_kernel on y).
-inline bool launch_gemm(const CUtensorMap &planes, const GemmScratch &scratch, int cap, const void *W0, const void *W1, int N, int K, int T, int epi, float *y,
+inline int launch_gemm(const CUtensorMap &planes, float *part, int cap, const void *W0, const void *W1, int N, int K, int T, int epi, float *y,
                         int ldy, int col0, bf16_t *out_hi, bf16_t *out_lo, int ldo, int *err, int n_sms, cudaStream_t s,
                         const void *W2 = nullptr, int nA = 0, int nB = 0, const QkvFuse *fuse = nullptr, bool *fused = nullptr,
                         const float *row_scale = nullptr) {
     if (fused) *fused = false;
-    if (!gemm_attrs_once()) return false;
+    if (!gemm_attrs_once()) return 0;
     const bool stacked = epi == PF_STORE && W1 && W2;
     const bool heads = stacked && fuse && fuse->head_dim == 128 && nA % 128 == 0 && nB % 128 == 0 && N % 128 == 0;
     const Deal deal = deal_out(T, N, K, epi == PF_SWIGLU, heads, n_sms);
@@ -139,30 +132,33 @@ inline bool launch_gemm(const CUtensorMap &planes, const GemmScratch &scratch, i
     const int per = epi == PF_SWIGLU ? bn / 2 : bn;
     const int box = per % 128 == 0 && (!stacked || (nA % 128 == 0 && nB % 128 == 0)) ? 128 : BOX_N;
     CUtensorMap tb0, tb1, tb2;
-    if (!make_map(&tb0, W0, (size_t)(stacked ? nA : N), (size_t)K, box)) return false;
+    if (!make_map(&tb0, W0, (size_t)(stacked ? nA : N), (size_t)K, box)) return 0;
     if (epi == PF_SWIGLU) {
-        if (!make_map(&tb1, W1, (size_t)N, (size_t)K, box)) return false;
+        if (!make_map(&tb1, W1, (size_t)N, (size_t)K, box)) return 0;
         tb2 = tb1;
     } else if (stacked) {
-        if (!make_map(&tb1, W1, (size_t)nB, (size_t)K, box) || !make_map(&tb2, W2, (size_t)(N - nA - nB), (size_t)K, box)) return false;
+        if (!make_map(&tb1, W1, (size_t)nB, (size_t)K, box) || !make_map(&tb2, W2, (size_t)(N - nA - nB), (size_t)K, box)) return 0;
     } else {
         tb1 = tb0;
         tb2 = tb0;
     }
     const int tiles_x = (T + BM - 1) / BM, tiles_y = (N + per - 1) / per;
-    GemmArgs g{T, K, N, bn, y, ldy, col0, out_hi, out_lo, ldo, err, tiles_x, tiles_y, box, act_box_rows(T), deal.whole, scratch.part, scratch.piece_cnt,
-               stacked ? nA : N, stacked ? nB : 0, row_scale, nullptr, nullptr, nullptr, 0, 0};
+    GemmArgs g{T, K, N, bn, y, ldy, col0, out_hi, out_lo, ldo, err, tiles_x, tiles_y, box, act_box_rows(T), deal.whole, part, stacked ? nA : N, stacked ? nB : 0, row_scale, nullptr, nullptr, nullptr, 0, 0};
     const dim3 grid(deal.grid);
     const int smem = gemm_smem(g.a_rows, bn);
-    const bool fuse_heads = heads && bn == 256;
-    if (fuse_heads) {
+    const int pieces = tiles_x * tiles_y - deal.whole;
+    auto run = [&](auto *contract, auto *fold) {
+        launch_chained(contract, grid, dim3(GEMM_THREADS), smem, s, planes, tb0, tb1, tb2, g, cap);
+        if (pieces) launch_chained(fold, dim3(8 * pieces), dim3(256), 0, s, g);
+    };
+    if (heads && bn == 256) {
         g.rope = fuse->rope; g.kc = fuse->kc; g.vc = fuse->vc; g.max_seq = fuse->max_seq; g.pos0 = fuse->pos0;
-        launch_chained(gemm_split_kernel<PF_QKV>, grid, dim3(GEMM_THREADS), smem, s, planes, tb0, tb1, tb2, g, cap);
+        run(gemm_split_kernel<PF_QKV>, fold_pieces_kernel<PF_QKV>);
         if (fused) *fused = true;
-    } else if (epi == PF_STORE) launch_chained(gemm_split_kernel<PF_STORE>, grid, dim3(GEMM_THREADS), smem, s, planes, tb0, tb1, tb2, g, cap);
-    else if (epi == PF_ADD) launch_chained(gemm_split_kernel<PF_ADD>, grid, dim3(GEMM_THREADS), smem, s, planes, tb0, tb1, tb2, g, cap);
-    else launch_chained(gemm_split_kernel<PF_SWIGLU>, grid, dim3(GEMM_THREADS), smem, s, planes, tb0, tb1, tb2, g, cap);
-    return true;
+    } else if (epi == PF_STORE) run(gemm_split_kernel<PF_STORE>, fold_pieces_kernel<PF_STORE>);
+    else if (epi == PF_ADD) run(gemm_split_kernel<PF_ADD>, fold_pieces_kernel<PF_ADD>);
+    else run(gemm_split_kernel<PF_SWIGLU>, fold_pieces_kernel<PF_SWIGLU>);
+    return pieces ? 2 : 1;
 }
 
 }  // namespace prefill

@@ -1,0 +1,59 @@
+"""Two sessions on two streams of one device, each driven by its own thread: their launches share the SMs in any mixture, and
+what a session computes must not depend on it."""
+import threading
+
+import pytest
+import torch
+
+import synthetic_inputs as si
+
+pytestmark = pytest.mark.gpu
+
+# wide enough that the last tiles of most maps of a prompt pass are done in pieces
+SHAPE = si.ModelShape("pieces", 2, 1536, 12, 4, 128, 4224, 2003, "bf16", 1e-5, 10000.0)
+LENGTHS = (77, 300, 17, 129, 500, 64, 256, 411)
+
+
+@pytest.fixture(scope="module")
+def kb():
+    from paper_2505_16162_b200 import build
+    build.build()
+    from paper_2505_16162_b200 import binding
+    return binding
+
+
+def _prompts(sess, seed, rounds):
+    """Prompts of all lengths, several times over: first token and pooled state of each."""
+    return [sess.prefill(si.uniform_tokens(seed, r, n, SHAPE.vocab).numpy(), want_pooled=True) for r in range(rounds) for n in LENGTHS]
+
+
+def _after(sess, seed):
+    """What the last prompt left in the K/V cache, as the logits of one pass."""
+    return sess.verify(si.uniform_tokens(seed, 100, 3, SHAPE.vocab).numpy(), want_logits=True)["logits"]
+
+
+def test_prompts_of_two_sessions_at_once_equal_the_serial_ones(kb):
+    w = si.make_model_weights(SHAPE, 4, device="cuda", gain_spread=0.1)
+    streams = [torch.cuda.Stream(priority=0), torch.cuda.Stream(priority=-1)]
+    torch.cuda.synchronize()
+    sess = [kb.Session.from_shape(SHAPE, w, 600, max_draft=4, stream=s) for s in streams]
+    rounds = 6
+    want = [(_prompts(sess[i], i, rounds), _after(sess[i], i)) for i in range(2)]
+    got, errors = [None, None], []
+
+    def work(i):
+        try:
+            with torch.cuda.stream(streams[i]):
+                got[i] = _prompts(sess[i], i, rounds)
+        except Exception as e:                                   # reported by the thread that started this one
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for i in range(2):
+        assert all(f0 == f1 and torch.equal(p0, p1) for (f0, p0), (f1, p1) in zip(want[i][0], got[i], strict=True))
+        assert torch.equal(want[i][1], _after(sess[i], i))
