@@ -56,7 +56,7 @@ struct knnssd_ctx {
     DeviceState *state = nullptr;
     float *samp_p = nullptr, *samp_q = nullptr;   // sampled decoding: filtered distributions [kMaxRows][vocab], made on first use
     int *samp_res = nullptr;                      // [2] result of a keep-or-resample round
-    int *err_word = nullptr;   // this device's error word (bounded waits that gave up, bad token ids, non-finite logits)
+    int *err_word = nullptr;   // bounded waits that gave up, bad token ids, non-finite logits: of this session's launches alone
     bool enqueue_failed = false;   // a pass could not be enqueued (its operation list did not reach the device)
     unsigned bar_spin_limit = 0;   // grid-barrier poll limit handed to the pass kernel (0 = its default)
     int *pinned = nullptr;  // host, pinned: small read-backs
@@ -219,7 +219,7 @@ template <typename WT> void launch_linear_t(const LinearArgs &a, int grid, cudaS
     }
 }
 
-// Set by the streaming kernel if one of its bounded waits ever gives up (never in normal operation).
+// Set by the streaming kernel of knnssd_linear if one of its bounded waits ever gives up (never in normal operation).
 __device__ int g_stream_err;
 
 constexpr int kMaxDevices = 64;
@@ -231,7 +231,9 @@ int current_device_slot() {
     return dev;
 }
 
-// Address of the error word on the CURRENT device (every device that loads the library has its own copy).
+// Address of the word on the CURRENT device that the launches of knnssd_linear report to (every device that loads the library has
+// its own copy).  Sessions and the operators that synchronise have words of their own: a word that several callers read and clear
+// tells one of them what another's launch met.
 int *stream_err_ptr() {
     static int *addr[kMaxDevices] = {};
     static std::mutex mu;
@@ -252,18 +254,18 @@ stream::LinPhase to_phase(const LinearArgs &a) {
     return p;
 }
 
-void launch_stream(const LinearArgs &a, int n_sms, cudaStream_t s) {
+void launch_stream(const LinearArgs &a, int n_sms, int *err, cudaStream_t s) {
     static bool configured[kMaxDevices] = {};          // function attributes are per device
     const int dev = current_device_slot();
     if (!configured[dev]) {
         cudaFuncSetAttribute(stream::linear_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, stream::SMEM_BYTES);
         configured[dev] = true;
     }
-    stream::linear_stream_kernel<<<n_sms, stream::NTHREADS, stream::SMEM_BYTES, s>>>(to_phase(a), stream_err_ptr());
+    stream::linear_stream_kernel<<<n_sms, stream::NTHREADS, stream::SMEM_BYTES, s>>>(to_phase(a), err);
 }
 
-void launch_linear(int dtype, const LinearArgs &a, int n_sms, cudaStream_t s) {
-    if (stream_eligible(dtype, a)) { launch_stream(a, n_sms, s); return; }
+void launch_linear(int dtype, const LinearArgs &a, int n_sms, int *err, cudaStream_t s) {
+    if (stream_eligible(dtype, a)) { launch_stream(a, n_sms, err, s); return; }
     // generic kernel: enough warps that every SM holds 8 blocks of 8 warps, but never more warps than units
     long long blocks = (long long)n_sms * 8;
     const long long max_blocks = (a.units + 7) / 8;
@@ -283,7 +285,7 @@ void ctx_linear(knnssd_ctx *c, const LinearArgs &a) {
         }
         cudaEventRecord(c->lin_events[c->lin_used], c->stream);
     }
-    launch_linear(c->cfg.dtype, a, c->n_sms, c->stream);
+    launch_linear(c->cfg.dtype, a, c->n_sms, c->err_word, c->stream);
     if (c->time_linear) {
         cudaEventRecord(c->lin_events[c->lin_used + 1], c->stream);
         c->lin_used += 2;
@@ -598,7 +600,7 @@ knnssd_status check_stream_err(knnssd_ctx *c, const char *what) {
 void free_all(knnssd_ctx *c) {
     void *ptrs[] = {c->kcache, c->vcache, c->x, c->qkv, c->attn, c->act, c->logits, c->hfinal, c->part_o, c->pooled,
                     c->anchor_inv_norm, c->cosines, c->amax_v, c->part_ml, c->rope_cs, c->pool_sum, c->inv_freq, c->chain,
-                    c->target, c->prompt, c->out_tokens, c->accept_log, c->amax_i, c->flag, c->knn_work, c->state,
+                    c->target, c->prompt, c->out_tokens, c->accept_log, c->amax_i, c->flag, c->knn_work, c->err_word, c->state,
                     c->ops_full, c->ops_draft, c->bar, c->gabort, c->attn_cnt, c->amax_cnt, c->mpart_o, c->mamax_v, c->mpart_ml,
                     c->mamax_i, c->trace, c->xs_x, c->xs_attn, c->xs_act, c->ssp, c->pf_x, c->pf_qkv, c->pf_ad, c->pf_aq, c->pf_af, c->pf_cs, c->pf_rinv, c->pf_part,
                     c->samp_p, c->samp_q, c->samp_res};
@@ -845,8 +847,6 @@ knnssd_status knnssd_init(const knnssd_config *cfg, const knnssd_weights *w, con
     auto bail = [&](knnssd_status s) { free_all(c); delete c; return s; };
     if (cudaGetDevice(&c->device) != cudaSuccess) return bail(KNNSSD_ERR_CUDA);
     cudaDeviceGetAttribute(&c->n_sms, cudaDevAttrMultiProcessorCount, c->device);
-    c->err_word = stream_err_ptr();
-    if (!c->err_word) return bail(KNNSSD_ERR_CUDA);
     const int d = g.d_model, hd = g.head_dim, nq = g.n_heads * hd, nkv = g.n_kv_heads * hd;
     const size_t cache_elems = (size_t)g.n_layers * g.n_kv_heads * g.max_seq * hd;
     c->n_splits = (g.max_seq + ATT_CHUNK - 1) / ATT_CHUNK;
@@ -875,6 +875,7 @@ knnssd_status knnssd_init(const knnssd_config *cfg, const knnssd_weights *w, con
     ok &= dev_alloc(&c->accept_log, (size_t)g.max_seq) == cudaSuccess;
     ok &= dev_alloc(&c->flag, 1) == cudaSuccess;
     ok &= dev_alloc(&c->knn_work, 2) == cudaSuccess;
+    ok &= dev_alloc(&c->err_word, 1) == cudaSuccess;
     ok &= dev_alloc(&c->state, 1) == cudaSuccess;
     ok &= dev_alloc(&c->cosines, (size_t)(na > 0 ? na : 1)) == cudaSuccess;
     ok &= dev_alloc(&c->anchor_inv_norm, (size_t)(na > 0 ? na : 1)) == cudaSuccess;
@@ -891,6 +892,7 @@ knnssd_status knnssd_init(const knnssd_config *cfg, const knnssd_weights *w, con
     set_state_kernel<<<1, 1, 0, c->stream>>>(c->state, 0, 0);
     cudaMemsetAsync(c->flag, 0, sizeof(int), c->stream);
     cudaMemsetAsync(c->knn_work, 0, 2 * sizeof(int), c->stream);
+    cudaMemsetAsync(c->err_word, 0, sizeof(int), c->stream);
     // token buffers start at a valid id, so that a pass that ends early never leaves garbage ids behind
     cudaMemsetAsync(c->chain, 0, sizeof(int) * (kMaxRows + 1), c->stream);
     cudaMemsetAsync(c->target, 0, sizeof(int) * kMaxRows, c->stream);
@@ -1466,7 +1468,7 @@ knnssd_status knnssd_linear(const void *W_dev, int dtype, int n_out, int n_in, c
     if (cudaGetDevice(&dev) != cudaSuccess) return KNNSSD_ERR_CUDA;
     cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev);
     LinearArgs a = make_args(W_dev, n_out, n_in, x_dev, nullptr, 0.f, y_dev, EPI_STORE, M);
-    launch_linear(dtype, a, n_sms, reinterpret_cast<cudaStream_t>(cuda_stream));
+    launch_linear(dtype, a, n_sms, stream_err_ptr(), reinterpret_cast<cudaStream_t>(cuda_stream));
     return cudaGetLastError() == cudaSuccess ? KNNSSD_OK : KNNSSD_ERR_CUDA;
 }
 
@@ -1485,18 +1487,20 @@ knnssd_status knnssd_gemm_split(const void *W0_dev, const void *W1_dev, int n_ou
     const int cap = (T + prefill::BM - 1) / prefill::BM * prefill::BM;
     bf16_t *planes = nullptr, *outp = nullptr;
     float *part = nullptr;
+    int *err = nullptr;
     const size_t plane = (size_t)cap * n_in, oplane = (size_t)T * n_out;
     Scratch mem(s);
     if (!mem.get(&planes, 2 * plane) || (mode == 2 && !mem.get(&outp, 2 * oplane)) ||
-        !mem.get(&part, (size_t)prefill::MAX_PIECES * prefill::PIECE_FLOATS))
+        !mem.get(&part, (size_t)prefill::MAX_PIECES * prefill::PIECE_FLOATS) || !mem.get(&err, 1))
         return KNNSSD_ERR_CUDA;
+    cudaMemsetAsync(err, 0, sizeof(int), s);
     knnssd_status st = KNNSSD_OK;
     cudaMemsetAsync(planes, 0, 2 * plane * sizeof(bf16_t), s);
     prefill::split_rows_kernel<<<T, 256, 0, s>>>(x_dev, n_in, planes, planes + plane);
     CUtensorMap ta;
     if (!prefill::make_map(&ta, planes, (size_t)2 * cap, (size_t)n_in, prefill::act_box_rows(T)) ||
         !prefill::launch_gemm(ta, part, cap, W0_dev, W1_dev, n_out, n_in, T, mode, y_dev, n_out, 0, outp, outp ? outp + oplane : nullptr,
-                              n_out, stream_err_ptr(), n_sms, s))
+                              n_out, err, n_sms, s))
         st = KNNSSD_ERR_CUDA;
     if (st == KNNSSD_OK && mode == 2) prefill::join_planes_kernel<<<T, 256, 0, s>>>(outp, outp + oplane, n_out, y_dev);
     cudaError_t e = cudaStreamSynchronize(s);
@@ -1504,8 +1508,8 @@ knnssd_status knnssd_gemm_split(const void *W0_dev, const void *W1_dev, int n_ou
     if (e != cudaSuccess) st = KNNSSD_ERR_CUDA;
     if (st == KNNSSD_OK) {
         int code = 0;
-        if (cudaMemcpy(&code, stream_err_ptr(), sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) st = KNNSSD_ERR_CUDA;
-        else if (code) { cudaMemset(stream_err_ptr(), 0, sizeof(int)); st = KNNSSD_ERR_TIMEOUT; }
+        if (cudaMemcpy(&code, err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) st = KNNSSD_ERR_CUDA;
+        else if (code) st = KNNSSD_ERR_TIMEOUT;
     }
     return st;
 }
@@ -1528,10 +1532,11 @@ knnssd_status knnssd_linear_tc(const void *W_dev, int n_out, int n_in, const flo
     kc = (nkb + kb_per - 1) / kb_per;
     bf16_t *planes = nullptr;
     float *part = nullptr;
+    int *err = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     const size_t plane_elems = (size_t)2 * lintc::TN * n_in, part_elems = (size_t)kc * M * n_out;
     Scratch mem(s);
-    bool ok = mem.get(&planes, plane_elems) && mem.get(&part, part_elems) && cudaEventCreate(&e0) == cudaSuccess &&
+    bool ok = mem.get(&planes, plane_elems) && mem.get(&part, part_elems) && mem.get(&err, 1) && cudaEventCreate(&e0) == cudaSuccess &&
               cudaEventCreate(&e1) == cudaSuccess;
     auto cleanup = [&]() {
         if (e0) cudaEventDestroy(e0);
@@ -1549,7 +1554,8 @@ knnssd_status knnssd_linear_tc(const void *W_dev, int n_out, int n_in, const flo
     }
     cudaMemsetAsync(planes, 0, plane_elems * sizeof(bf16_t), s);
     lintc::split_x_kernel<<<M, 256, 0, s>>>(x_dev, n_in, planes);
-    lintc::Args a{M, n_in, n_out, kc, kb_per, part, stream_err_ptr()};
+    cudaMemsetAsync(err, 0, sizeof(int), s);
+    lintc::Args a{M, n_in, n_out, kc, kb_per, part, err};
     cudaEventRecord(e0, s);
     lintc::linear_tc_kernel<<<dim3(tiles, kc), lintc::THREADS, lintc::SMEM, s>>>(tw, tx, a);
     const size_t n = (size_t)M * n_out;
@@ -1560,8 +1566,8 @@ knnssd_status knnssd_linear_tc(const void *W_dev, int n_out, int n_in, const flo
     if (e != cudaSuccess) st = KNNSSD_ERR_CUDA;
     if (st == KNNSSD_OK) {
         int code = 0;
-        if (cudaMemcpy(&code, stream_err_ptr(), sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) st = KNNSSD_ERR_CUDA;
-        else if (code) { cudaMemset(stream_err_ptr(), 0, sizeof(int)); st = KNNSSD_ERR_TIMEOUT; }
+        if (cudaMemcpy(&code, err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) st = KNNSSD_ERR_CUDA;
+        else if (code) st = KNNSSD_ERR_TIMEOUT;
     }
     if (st == KNNSSD_OK && ms_kernels_host) cudaEventElapsedTime(ms_kernels_host, e0, e1);
     cleanup();

@@ -57,3 +57,40 @@ def test_prompts_of_two_sessions_at_once_equal_the_serial_ones(kb):
     for i in range(2):
         assert all(f0 == f1 and torch.equal(p0, p1) for (f0, p0), (f1, p1) in zip(want[i][0], got[i], strict=True))
         assert torch.equal(want[i][1], _after(sess[i], i))
+
+
+def test_an_error_is_reported_to_the_session_that_met_it(kb):
+    """One session's logits hold no finite value, another's are sound: every call of the first says so, none of the second does."""
+    shape = si.SHAPES["tiny"]
+    sound = si.make_model_weights(shape, 0, device="cuda")
+    bad = dict(sound, final_norm=torch.full_like(sound["final_norm"], float("nan")))
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    torch.cuda.synchronize()
+    sess = [kb.Session.from_shape(shape, w, 96, max_draft=4, stream=s) for w, s in zip((bad, sound), streams)]
+    prompt = si.uniform_tokens(0, 0, 20, shape.vocab).numpy()
+    first = sess[1].prefill(prompt)
+    seen, errors = [], []
+
+    def sick():
+        for _ in range(150):
+            try:
+                sess[0].prefill(prompt)
+                seen.append(0)
+            except kb.KnnssdError as e:
+                seen.append(e.status)
+
+    def well():
+        for _ in range(150):
+            try:
+                if sess[1].prefill(prompt) != first:
+                    errors.append("another token")
+            except kb.KnnssdError as e:
+                errors.append(str(e))
+
+    threads = [threading.Thread(target=f) for f in (sick, well)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[:3]
+    assert seen == [5] * 150
