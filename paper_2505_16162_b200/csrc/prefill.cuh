@@ -207,6 +207,14 @@ struct Jobs {
 };
 constexpr int PIECE_FLOATS = BM * BN_MAX;      // a chunk's sums, by register group and thread (coalesced): 32 x 256 float4
 
+// Rotary embedding of a pair by (cos, sin) = c.  The rounding is spelled out: left to the compiler, the contraction's epilogue and
+// rope_kv_rows_kernel fused other products of the second sum, and a row's K depended on which of them a launch's sizes chose.
+__device__ __forceinline__ void rotate_pair(float &a, float &b, float2 c) {
+    const float ra = __fmaf_rn(a, c.x, -__fmul_rn(b, c.y));
+    b = __fmaf_rn(b, c.x, __fmul_rn(a, c.y));
+    a = ra;
+}
+
 // Tile column of register group gi (32 columns) of an epilogue thread, or -1 if the group is not in use.  Store / add: half
 // hsel of the columns in groups of 32; SwiGLU: groups 0 and 1 a quarter of them in the gate columns, 2 and 3 the up columns of
 // the same units.
@@ -255,12 +263,7 @@ __device__ __forceinline__ void finish_sums(const GemmArgs &g, int tile, int t, 
         if (u0 < g.nA + g.nB) {                          // a q or a k head: rotary embedding
             const float2 *cs = g.rope + (size_t)t * 64 + k8;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const float2 c = cs[i];
-                const float a = v[i], b = v[8 + i];
-                v[i] = a * c.x - b * c.y;
-                v[8 + i] = b * c.x + a * c.y;
-            }
+            for (int i = 0; i < 8; ++i) rotate_pair(v[i], v[8 + i], cs[i]);
         }
         const bool is_k = u0 < g.nA + g.nB;
         const int kvh = (u0 - g.nA - (is_k ? 0 : g.nB)) >> 7;
@@ -619,18 +622,16 @@ __global__ void __launch_bounds__(256) rope_kv_rows_kernel(float *__restrict__ q
     for (int idx = blockIdx.y * 256 + threadIdx.x; idx < (H + 2 * Hkv) * half; idx += 256 * ROPE_PARTS) {
         const int slot = idx / half, i = idx % half;
         float *row = trow + (size_t)slot * hd;
-        const float a = row[i], b = row[i + half];
+        float a = row[i], b = row[i + half];
         if (slot < H + Hkv) {
-            const float2 cs2 = table[(size_t)t * half + i];
-            const float c = cs2.x, s = cs2.y;
-            const float ra = a * c - b * s, rb = b * c + a * s;
+            rotate_pair(a, b, table[(size_t)t * half + i]);
             if (slot < H) {
-                row[i] = ra;
-                row[i + half] = rb;
+                row[i] = a;
+                row[i + half] = b;
             } else {
                 bf16_t *dst = kc + ((size_t)(slot - H) * max_seq + pos) * hd;
-                dst[i] = float_to_bf16_rne(ra);
-                dst[i + half] = float_to_bf16_rne(rb);
+                dst[i] = float_to_bf16_rne(a);
+                dst[i + half] = float_to_bf16_rne(b);
             }
         } else {
             bf16_t *dst = vc + ((size_t)(slot - H - Hkv) * max_seq + pos) * hd;
