@@ -317,6 +317,13 @@ __device__ __forceinline__ int cluster_sample(const float *__restrict__ a, const
                 }
             }
             if (tok < 0) tok = pos;
+            if (tok < 0) {
+                // the last warp, without weight of its own: the block's sum, added at once, ends an ulp past the running sum of its
+                // warps, and the target lies between.  The crossing is in this block all the same: its last id with weight
+                tok = lane < NW ? __float_as_int(sh.m.red[lane][NS]) : -1;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) tok = max(tok, __shfl_xor_sync(0xffffffffu, tok, o));
+            }
             if (lane == 0 && tok >= 0) atomicMax(&cluster.map_shared_rank(&sh, 0)->token, tok);
         }
         break;

@@ -84,3 +84,16 @@ def test_resample_falls_back_to_p_where_q_covers_it(kb):
     q[0, 3999] = 1.0
     q[0, 7] = 1.0
     assert kb.knnssd_spec_accept(p, q, [7], [0.5], 0.3) == (0, 3999)
+
+
+def test_a_draw_between_two_roundings_stays_in_its_block():
+    """512 ids: a block has 64, its warps four each.  1 + 2^-24 + 2^-24 is 1 when added one by one and 1 + 2^-23 when block 1's
+    two ids are added first, so a target of exactly 1 lies past all of the block's running sums and below its end."""
+    from paper_2505_16162_b200 import binding as kb
+    w = torch.zeros(512)
+    w[0], w[64], w[68], w[511] = 1.0, 2.0 ** -24, 2.0 ** -24, 0.5
+    total = np.float32(1.5 + 2.0 ** -23)
+    us = [u for u in (np.float32(2.0 / 3.0) + np.arange(-8, 9, dtype=np.float32) * np.float32(2.0 ** -24)) if u * total == np.float32(1.0)]
+    assert us
+    for u in us:
+        assert kb.knnssd_sample_token(w.cuda(), float(u)) in (64, 68)
