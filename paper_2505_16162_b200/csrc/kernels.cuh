@@ -423,12 +423,13 @@ __global__ void pool_accumulate_kernel(const float *__restrict__ h, int M, int d
 }
 
 // The same for many rows, without writing the normalised rows out: part[s][i] = fp64 sum, in row order, of the rows of slice s
-// (`per` rows each), every term the row's value times its RMSNorm scale times the gain, rounded as rmsnorm_rows_kernel does;
+// (POOL_ROWS rows each), every term the row's value times its RMSNorm scale times the gain, rounded as rmsnorm_rows_kernel does;
 // pool_fold_kernel adds the slices in order.  The fp64 additions (about 4 lanes per clock and SM) want all SMs: one thread per
 // column walking 1024 rows took 83 us, this 16 with the scales.  grid = (ceil(d / 256), slices), 256 threads.
+constexpr int POOL_ROWS = 32;
 __global__ void __launch_bounds__(256) pool_partial_kernel(const float *__restrict__ x, const float *__restrict__ rinv, const float *__restrict__ gain,
-                                                           int M, int d, int per, double *__restrict__ part) {
-    const int i = blockIdx.x * 256 + threadIdx.x, m0 = blockIdx.y * per, m1 = min(M, m0 + per);
+                                                           int M, int d, double *__restrict__ part) {
+    const int i = blockIdx.x * 256 + threadIdx.x, m0 = blockIdx.y * POOL_ROWS, m1 = min(M, m0 + POOL_ROWS);
     if (i >= d) return;
     const float g = gain[i];
     double s = 0.0;

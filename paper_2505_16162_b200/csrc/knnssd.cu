@@ -686,10 +686,10 @@ bool prefill_tensor(knnssd_ctx *c, int n) {
         }
         // pooled numerator: every row's final hidden state (mean pooling) or the last row's
         if (g.pool_mode == 0) {
-            const int per = 32, slices = (T + per - 1) / per;
-            double *part = reinterpret_cast<double *>(c->pf_qkv);                // [slices][d]: less than the projections' T rows
+            const int slices = (T + POOL_ROWS - 1) / POOL_ROWS;
+            double *part = reinterpret_cast<double *>(c->pf_qkv);                // [slices][d]: knnssd_init makes room for both uses
             row_scale_kernel<<<T, 256, 0, s>>>(c->pf_x, d, g.rms_eps, c->pf_rinv);
-            pool_partial_kernel<<<dim3((d + 255) / 256, slices), 256, 0, s>>>(c->pf_x, c->pf_rinv, c->final_norm, T, d, per, part);
+            pool_partial_kernel<<<dim3((d + 255) / 256, slices), 256, 0, s>>>(c->pf_x, c->pf_rinv, c->final_norm, T, d, part);
             pool_fold_kernel<<<(d + 255) / 256, 256, 0, s>>>(part, slices, d, c->pool_sum, t0 == 0);
             c->launches += 3;
         } else if (last) {
@@ -931,7 +931,9 @@ knnssd_status knnssd_init(const knnssd_config *cfg, const knnssd_weights *w, con
             const size_t cap = (size_t)c->pf_cap;
             bool ok3 = true;
             ok3 &= dev_alloc(&c->pf_x, cap * d) == cudaSuccess;
-            ok3 &= dev_alloc(&c->pf_qkv, cap * (nq + 2 * nkv)) == cudaSuccess;
+            // the projections, and behind the last layer the slices of the pooled sum: few heads on a wide model make those the larger
+            const size_t n_proj = cap * (nq + 2 * nkv), n_pool = 2 * ((cap + POOL_ROWS - 1) / POOL_ROWS) * d;
+            ok3 &= dev_alloc(&c->pf_qkv, n_proj > n_pool ? n_proj : n_pool) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_cs, cap * (hd / 2)) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_rinv, cap) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_ad, 2 * cap * d) == cudaSuccess;
