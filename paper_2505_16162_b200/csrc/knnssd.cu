@@ -939,7 +939,8 @@ knnssd_status knnssd_init(const knnssd_config *cfg, const knnssd_weights *w, con
             ok3 &= dev_alloc(&c->pf_ad, 2 * cap * d) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_aq, 2 * cap * nq) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_af, 2 * cap * g.d_ff) == cudaSuccess;
-            ok3 &= dev_alloc(&c->pf_part, (size_t)prefill::MAX_PIECES * prefill::PIECE_FLOATS) == cudaSuccess;
+            const int sums = prefill::most_sums(c->pf_cap, d, nq, nkv, g.d_ff, hd, c->n_sms);
+            ok3 &= sums == 0 || dev_alloc(&c->pf_part, (size_t)sums * prefill::PIECE_FLOATS) == cudaSuccess;
             if (!ok3) { cudaGetLastError(); return bail(KNNSSD_ERR_CUDA); }
             cudaMemsetAsync(c->pf_ad, 0, 2 * cap * d * sizeof(bf16_t), c->stream);
             cudaMemsetAsync(c->pf_aq, 0, 2 * cap * nq * sizeof(bf16_t), c->stream);
@@ -1490,10 +1491,11 @@ knnssd_status knnssd_gemm_split(const void *W0_dev, const void *W1_dev, int n_ou
     bf16_t *planes = nullptr, *outp = nullptr;
     float *part = nullptr;
     int *err = nullptr;
+    const int sums = prefill::deal_out(T, n_out, n_in, mode == 2, false, n_sms).sums;
     const size_t plane = (size_t)cap * n_in, oplane = (size_t)T * n_out;
     Scratch mem(s);
     if (!mem.get(&planes, 2 * plane) || (mode == 2 && !mem.get(&outp, 2 * oplane)) ||
-        !mem.get(&part, (size_t)prefill::MAX_PIECES * prefill::PIECE_FLOATS) || !mem.get(&err, 1))
+        (sums > 0 && !mem.get(&part, (size_t)sums * prefill::PIECE_FLOATS)) || !mem.get(&err, 1))
         return KNNSSD_ERR_CUDA;
     cudaMemsetAsync(err, 0, sizeof(int), s);
     knnssd_status st = KNNSSD_OK;

@@ -62,8 +62,8 @@ inline bool gemm_attrs_once() {
 // L2 to be worth it).  20 tiles of 27 chunks - 5120 units at 13824 input columns, up to 128 rows - are 540.
 constexpr int MAX_PIECES = 576;
 
-// Columns per tile, CTAs, and how many tiles are done whole (the rest in pieces).
-struct Deal { int bn, grid, whole; };
+// Columns per tile, CTAs, how many tiles are done whole (the rest in pieces), and the chunk sums that the pieces leave.
+struct Deal { int bn, grid, whole, sums; };
 
 // The cheapest of 128, 192 and 256 columns, tiles all whole or the last, incomplete round of them in pieces, by times measured
 // on the 13B widths (5120 / 13824 columns in, 77 .. 1024 rows):
@@ -76,7 +76,7 @@ struct Deal { int bn, grid, whole; };
 // `heads`: 256 columns let the launch finish the heads itself; else a kernel of its own does.
 inline Deal deal_out(int T, int N, int K, bool swiglu, bool heads, int n_sms) {
     const int row_tiles = (T + BM - 1) / BM, nkb = K / BK, nchunks = (nkb + CHUNK_KB - 1) / CHUNK_KB;
-    Deal best{0, 0, 0};
+    Deal best{0, 0, 0, 0};
     double best_us = 0.0;
     for (int bn = 128; bn <= BN_MAX; bn += 64) {
         if (swiglu && bn % 128) continue;
@@ -85,11 +85,12 @@ inline Deal deal_out(int T, int N, int K, bool swiglu, bool heads, int n_sms) {
         const double kb_us = bn == 256 ? 0.73 : bn == 192 ? 0.62 : 0.5, heads_us = heads && bn != 256 ? 12.0 + T * 0.02 : 0.0;
         const double round_us = nkb * kb_us;
         for (int pieces = 0; pieces < 2; ++pieces) {
-            Deal d{bn, (int)(tiles < n_sms ? tiles : n_sms), (int)tiles};
+            Deal d{bn, (int)(tiles < n_sms ? tiles : n_sms), (int)tiles, 0};
             double us = heads_us + 8.0 + (double)((tiles + n_sms - 1) / n_sms) * round_us;
             if (pieces) {
                 if (last_round == 0 || units > MAX_PIECES) continue;
                 d.whole = (int)(tiles - last_round);
+                d.sums = (int)units;
                 d.grid = d.whole == 0 && units < n_sms ? (int)units : n_sms;
                 const long long most = (units + d.grid - 1) / d.grid;
                 us = heads_us + 14.0 + (double)(d.whole / n_sms) * round_us + most * 1.3 * CHUNK_KB * kb_us +
@@ -105,10 +106,27 @@ inline Deal deal_out(int T, int N, int K, bool swiglu, bool heads, int n_sms) {
 // whatever the stage held before; they meet no live row).
 inline int act_box_rows(int T) { return T >= BM ? BM : (T + 7) / 8 * 8; }
 
+// Whether a stacked q / k / v launch may finish the heads in its epilogue (it does at 256 columns).
+inline bool heads_in_epilogue(int head_dim, int nA, int nB, int N) { return head_dim == 128 && nA % 128 == 0 && nB % 128 == 0 && N % 128 == 0; }
+
+// Most chunk sums that any launch of a prompt pass over up to `cap` rows leaves: what its scratch has to hold.
+inline int most_sums(int cap, int d, int nq, int nkv, int d_ff, int head_dim, int n_sms) {
+    const int ldq = nq + 2 * nkv;
+    const bool heads = heads_in_epilogue(head_dim, nq, nkv, ldq);
+    int most = 0;
+    for (int T = 1; T <= cap; ++T) {
+        const int sums[] = {deal_out(T, ldq, d, false, heads, n_sms).sums, deal_out(T, d, nq, false, false, n_sms).sums,
+                            deal_out(T, d_ff, d, true, false, n_sms).sums, deal_out(T, d, d_ff, false, false, n_sms).sums};
+        for (int n : sums)
+            if (n > most) most = n;
+    }
+    return most;
+}
+
 // One contraction over T rows.  `planes` = the activation map (hi rows [0, cap), lo rows [cap, 2 cap)); W0 (and W1 for
 // SwiGLU: W0 = gate, W1 = up) are [N][K] bf16.  STORE with W1 and W2 given: the three matrices (nA, nB and nC rows, all
 // multiples of BOX_N) are stacked along the output units, N = nA + nB + nC, one launch for q, k and v.
-// `part`: scratch of MAX_PIECES * PIECE_FLOATS.  Returns the number of kernels launched, 0 if a tensor map could not be made.
+// `part`: scratch of PIECE_FLOATS for every chunk sum that deal_out gives the launch.  Returns the number of kernels launched, 0 if a tensor map could not be made.
 // What the q / k / v launch needs to finish the heads in its epilogue (rotary embedding, K / V rows into the cache).
 struct QkvFuse {
     const float2 *rope;    // [T][64]
@@ -126,7 +144,7 @@ inline int launch_gemm(const CUtensorMap &planes, float *part, int cap, const vo
     if (fused) *fused = false;
     if (!gemm_attrs_once()) return 0;
     const bool stacked = epi == PF_STORE && W1 && W2;
-    const bool heads = stacked && fuse && fuse->head_dim == 128 && nA % 128 == 0 && nB % 128 == 0 && N % 128 == 0;
+    const bool heads = stacked && fuse && heads_in_epilogue(fuse->head_dim, nA, nB, N);
     const Deal deal = deal_out(T, N, K, epi == PF_SWIGLU, heads, n_sms);
     const int bn = deal.bn;
     const int per = epi == PF_SWIGLU ? bn / 2 : bn;
