@@ -459,13 +459,14 @@ void run_pass_mega(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const 
     c->launches++;
 }
 
-// After a pass kernel gave up: bring the barrier counter and the work counters back to their idle state.
+// After a pass kernel gave up: bring the barrier counter and the work counters back to their idle state.  On the session's stream:
+// it need not be one that waits for the legacy stream, and the next pass would run into a cudaMemset on its way.
 void reset_mega_state(knnssd_ctx *c) {
     if (!c->mega_ok) return;
-    cudaMemset(c->bar, 0, sizeof(unsigned long long));
-    cudaMemset(c->gabort, 0, sizeof(int));
-    cudaMemset(c->attn_cnt, 0, sizeof(int) * pass::MAXM * c->cfg.n_heads);
-    cudaMemset(c->amax_cnt, 0, sizeof(int));
+    cudaMemsetAsync(c->bar, 0, sizeof(unsigned long long), c->stream);
+    cudaMemsetAsync(c->gabort, 0, sizeof(int), c->stream);
+    cudaMemsetAsync(c->attn_cnt, 0, sizeof(int) * pass::MAXM * c->cfg.n_heads, c->stream);
+    cudaMemsetAsync(c->amax_cnt, 0, sizeof(int), c->stream);
     c->bar_total = 0;
 }
 
@@ -567,7 +568,7 @@ knnssd_status set_word(knnssd_ctx *c, int *word, int value, const char *what) {
 // What a non-zero device error word means.  Whatever it was, the pass that raised it did not finish: the session's
 // cache and pending token are no longer trustworthy, so the caller has to prefill again.
 knnssd_status fail_device_code(knnssd_ctx *c, const char *what, int code) {
-    cudaMemset(c->err_word, 0, sizeof(int));
+    cudaMemsetAsync(c->err_word, 0, sizeof(int), c->stream);
     reset_mega_state(c);
     c->prefilled = false;
     if (code == ERR_BAD_LOGITS)

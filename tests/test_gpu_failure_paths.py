@@ -93,3 +93,23 @@ def test_logits_without_a_finite_value_are_reported_not_followed(kb, shape_name)
     ok.set_skipmask(mask)
     got = ok.generate(prompt, 8, 2)
     assert np.array_equal(got["tokens"], want["tokens"])
+
+
+def test_recovery_on_a_stream_of_the_sessions_own(kb):
+    """What a failed pass left is cleared in the order of the session's stream, which does not wait for the default one."""
+    shape = si.SHAPES["stream-bf16"]
+    mask = si.skip_mask(0, 2 * shape.n_layers, 3)
+    w = _to_dev(si.make_model_weights(shape, 0, gain_spread=0.1))
+    prompt = si.uniform_tokens(0, 0, 12, shape.vocab).numpy()        # one pass of the persistent kernel
+    torch.cuda.synchronize()
+    sess = kb.Session.from_shape(shape, w, 160, max_draft=4, stream=torch.cuda.Stream())
+    sess.set_skipmask(mask)
+    want = sess.generate(prompt, 24, 4)
+    busy = torch.empty(1 << 28, dtype=torch.uint8, device="cuda")
+    for _ in range(20):
+        busy.fill_(1)                                                # keeps the default stream at work
+        with pytest.raises(kb.KnnssdError) as e:
+            sess.debug_barrier_timeout(2000)
+        assert e.value.status == 7
+        got = sess.generate(prompt, 24, 4)
+        assert np.array_equal(got["tokens"], want["tokens"]) and np.array_equal(got["accepts"], want["accepts"])
