@@ -124,7 +124,9 @@ template <typename T> cudaError_t dev_alloc(T **p, size_t count) {
 // driver at every synchronisation, all of it when a context is destroyed): a cudaMalloc / cudaFree pair cost 100 .. 1000 us
 // a call, next to kernels of 10 .. 50 us.  Allocations are ordered on the caller's stream, so any number of threads and
 // streams may call at once.
-constexpr unsigned long long kPoolKeep = 64ull << 20;
+// 96 MB hold the largest scratch of a contraction in pieces (prefill_host.cuh: 72 MB of chunk sums) and the planes of its rows: with
+// 64, knnssd_gemm_split over 5120 x 13824 weights mapped memory on every call (77 rows 336 us, with 96 129; 1024 rows 488, 275).
+constexpr unsigned long long kPoolKeep = 96ull << 20;
 
 struct DevicePools {
     std::mutex mu;
