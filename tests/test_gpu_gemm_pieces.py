@@ -27,10 +27,11 @@ def _inputs(n_out, n_in, T):
 @pytest.mark.parametrize("n_out,n_in", [(5120, 13824), (1032, 4416), (4936, 5120), (264, 512), (5000, 320)])
 def test_rows_are_the_same_bits_however_the_launch_is_dealt_out(kb, n_out, n_in):
     W, x = _inputs(n_out, n_in, 1024)
-    full = {0: kb.knnssd_gemm_split(W, x, 0), 2: kb.knnssd_gemm_split(W, x, 2, W1=W)}
+    y0 = si.normal_f32(21, 10, torch.arange(1024 * n_out, device="cuda"), 1.0).view(1024, n_out)
+    full = {0: kb.knnssd_gemm_split(W, x, 0), 1: kb.knnssd_gemm_split(W, x, 1, y=y0.clone()), 2: kb.knnssd_gemm_split(W, x, 2, W1=W)}
     for T in (1, 77, 128, 129, 300, 1000):
         for mode, want in full.items():
-            got = kb.knnssd_gemm_split(W, x[1024 - T:].contiguous(), mode, W1=W if mode == 2 else None)
+            got = kb.knnssd_gemm_split(W, x[1024 - T:].contiguous(), mode, W1=W if mode == 2 else None, y=y0[1024 - T:].clone() if mode == 1 else None)
             assert torch.equal(got, want[1024 - T:]), (T, mode)
 
 

@@ -94,3 +94,48 @@ def test_an_error_is_reported_to_the_session_that_met_it(kb):
         t.join()
     assert not errors, errors[:3]
     assert seen == [5] * 150
+
+
+def test_stand_alone_operators_from_several_threads(kb):
+    """Scratch from the shared pool, words of pinned memory per thread: what a call returns must not depend on the others'."""
+    g = torch.Generator(device="cuda").manual_seed(3)
+    def rand(*shape):
+        return torch.randn(*shape, generator=g, device="cuda")
+
+    jobs = []
+    for i in range(4):
+        logits = 1.4 * rand(5, 3000 + 517 * i)
+        p = kb.knnssd_filtered_probs(logits, 1.0, 0.95)
+        q = kb.knnssd_filtered_probs(logits[:4] + 0.3 * rand(4, logits.shape[1]), 1.0, 0.95)
+        x = rand(200 + 40 * i, 96)
+        jobs.append({"p": p, "q": q, "drafts": q.argmax(dim=1).cpu().numpy(), "anchors": rand(30 + i, 256), "query": rand(256), "x": x, "start": x[:3].contiguous(),
+                     "W": rand(640, 2048).bfloat16(), "rows": rand(40 + 30 * i, 2048)})
+
+    def once(j, r):
+        u = [((7 * r + e) % 31) / 31 for e in range(5)]
+        a = kb.knnssd_build_anchors(j["x"], j["start"], 20, 4)
+        return (kb.knnssd_sample_token(j["p"][0], u[0]), kb.knnssd_spec_accept(j["p"], j["q"], j["drafts"], u[:4], u[4]), kb.knnssd_cosine_top1(j["query"], j["anchors"]),
+                a["labels"].tolist(), a["anchors"].tolist(), a["centroids"], kb.knnssd_gemm_split(j["W"], j["rows"]))
+
+    rounds = 12
+    want = [[once(j, r) for r in range(rounds)] for j in jobs]
+    got, errors = [None] * len(jobs), []
+    torch.cuda.synchronize()
+
+    def work(i):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                got[i] = [once(jobs[i], r) for r in range(rounds)]
+                torch.cuda.current_stream().synchronize()
+        except Exception as e:
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(len(jobs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for w, h in zip(want, got):
+        for a, b in zip(w, h, strict=True):
+            assert a[:5] == b[:5] and torch.equal(a[5], b[5]) and torch.equal(a[6], b[6])
