@@ -12,7 +12,15 @@
  * Nothing aborts or throws across the boundary, and knnssd_last_error() gives a
  * one-line reason.  A context is bound to the CUDA
  * device that was current at knnssd_init and to the stream passed there; calls on
- * one context must not overlap (not thread-safe per context).
+ * one context must not overlap (not thread-safe per context).  Several contexts, on
+ * streams of their own, may be used at once from several threads: they share
+ * nothing but the model's weights.
+ *
+ * The stand-alone operators below take their scratch from a memory pool of the
+ * library, one per device, in the order of the caller's stream.  It keeps up to 96 MB
+ * between calls (more than that goes back at the next synchronisation) and is emptied
+ * by knnssd_destroy.  Their small arguments and results pass through 256 bytes of pinned
+ * memory per host thread, made by the thread's first such call.
  *
  * Notation follows the paper: L decoder layers = 2L sublayers; a skip mask
  * z in {0,1}^{2L} with z[j] = 1 meaning "sublayer j is skipped while drafting"
@@ -171,7 +179,9 @@ knnssd_status knnssd_decode(knnssd_ctx *ctx, int max_new, int k, int use_selecti
 long long knnssd_get_launch_count(const knnssd_ctx *ctx);
 
 /* Committed context length (positions whose K/V are valid), and explicit rollback to a shorter length
- * (new_len <= current length; the pending token is unchanged, so this is meant for tests and benchmarks). */
+ * (new_len <= current length; the pending token is unchanged, so this is meant for tests and benchmarks).
+ * knnssd_set_length and knnssd_set_pending are asynchronous: the new value is enqueued on the context's stream, and a failure of
+ * the device is reported by the next call that waits.  Both are refused (KNNSSD_ERR_CUDA) while the stream is being captured. */
 int knnssd_get_length(const knnssd_ctx *ctx);
 knnssd_status knnssd_set_length(knnssd_ctx *ctx, int new_len);
 
@@ -240,6 +250,7 @@ knnssd_status knnssd_debug_barrier_timeout(knnssd_ctx *ctx, unsigned spin_limit)
 /*
  * y[m][o] = sum_i W[o][i] * x[m][i] for m < M <= 16: the weight-streaming linear kernel.
  *   W DEVICE [n_out][n_in] (dtype as above), x DEVICE fp32 [M][n_in], y DEVICE fp32 [M][n_out]; n_in % 8 == 0.
+ *   Asynchronous on the stream; should a bounded wait in it give up, y is left incomplete and nothing reports it.
  */
 knnssd_status knnssd_linear(const void *W_dev, int dtype, int n_out, int n_in, const float *x_dev, int M,
                             float *y_dev, void *cuda_stream);
@@ -253,7 +264,7 @@ knnssd_status knnssd_linear(const void *W_dev, int dtype, int n_out, int n_in, c
  *            the prompt pass hands it to the next map
  *   W0, W1 DEVICE bf16 [n_out][n_in], 16-byte aligned (W1 only for mode 2); x DEVICE fp32 [T][n_in];
  *   y DEVICE fp32 [T][n_out]; n_in % 64 == 0, n_out % 8 == 0, T >= 1.
- * Allocates and frees its temporary planes, and synchronises the stream before it returns.  KNNSSD_ERR_SHAPE for
+ * Scratch from the pool (planes, chunk sums); synchronises the stream before it returns.  KNNSSD_ERR_SHAPE for
  * sizes outside the rules above, KNNSSD_ERR_TIMEOUT if a device-side wait gave up.
  */
 knnssd_status knnssd_gemm_split(const void *W0_dev, const void *W1_dev, int n_out, int n_in, const float *x_dev, int T,
@@ -267,7 +278,7 @@ knnssd_status knnssd_gemm_split(const void *W0_dev, const void *W1_dev, int n_ou
  * rows.
  *   W DEVICE bf16 [n_out][n_in], 16-byte aligned; x DEVICE fp32 [M][n_in]; y DEVICE fp32 [M][n_out]; n_in % 64 == 0;
  *   M > 16: KNNSSD_ERR_CAPACITY.  ms_kernels_host: HOST, device time of the contraction + the chunk sum (CUDA
- *   events), or NULL.  Allocates and frees its scratch; synchronises the stream.
+ *   events), or NULL.  Scratch from the pool; synchronises the stream.
  */
 knnssd_status knnssd_linear_tc(const void *W_dev, int n_out, int n_in, const float *x_dev, int M, float *y_dev,
                                float *ms_kernels_host, void *cuda_stream);
@@ -290,7 +301,7 @@ knnssd_status knnssd_linear_tc(const void *W_dev, int n_out, int n_in, const flo
  *                       distances; -1 where a cluster has fewer than k members
  *   rounds_host         HOST: assignment rounds done (NULL: not wanted)
  *   ms_rounds_host      HOST: device time of all rounds, CUDA events on the stream (NULL: not wanted)
- * Allocates and frees its scratch; synchronises the stream.
+ * Scratch from the pool; synchronises the stream.
  */
 knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int n_clusters,
                                    const float *init_centroids_dev, int max_rounds, int k, int *labels_host,
@@ -359,10 +370,10 @@ knnssd_status knnssd_cosine_top1(const float *query_dev, const float *anchors_de
  * deployment variant of the call above, same arithmetic, same results.)
  *
  * Who needs it: code that runs where cudaMalloc / cudaFree are off limits - inside a serving loop whose memory pool
- * was sized and handed out at start-up, in a process that shares the GPU under a fixed memory reservation, or in a
- * latency path where the implicit device synchronisation of cudaFree is not acceptable.  knnssd_cosine_top1 makes two
- * small cudaMalloc / cudaFree pairs per call for its per-anchor cosines and its result words; this variant keeps that
- * scratch in a fixed array inside the library's device image instead, and calls no allocating routine at all.
+ * was sized and handed out at start-up, or in a process that shares the GPU under a fixed memory reservation.
+ * knnssd_cosine_top1 takes its per-anchor cosines from the library's pool, which grows on the first call and after it was
+ * emptied, and its result through the thread's pinned words; this variant keeps both in a fixed array inside the library's
+ * device image instead, and calls no allocating routine at all.
  *
  *   arguments   as knnssd_cosine_top1 (query_dev, anchors_dev DEVICE fp32; best, cosine HOST outputs)
  *   limit       n <= KNNSSD_STATIC_MAX_ANCHORS; a larger n returns KNNSSD_ERR_CAPACITY and touches nothing

@@ -10,7 +10,9 @@
 //                       the decode passes), accumulator fp32.  Epilogues: store, add to the residual stream,
 //                       SwiGLU of a gate tile and an up tile.
 //   norm_split_kernel   RMSNorm of each row, written as the two bf16 planes the next map reads.
-//   rope_kv_kernel      rotary embedding of q and k, K/V rows rounded to bf16 into the cache.
+//   fold_pieces_kernel  the sums of the tiles that a launch did in pieces, and their epilogue.
+//   rope_kv_rows_kernel rotary embedding of q and k, K/V rows rounded to bf16 into the cache, where the contraction's epilogue
+//                       has not done it.
 //   attn_prompt_kernel  causal attention of 64 query rows per CTA (16 per warp) over the cached K/V, staged segment by
 //                       segment in shared memory, on mma.sync (the sizes are small next to the linear maps), output
 //                       written as bf16 planes for the O projection.
@@ -31,7 +33,7 @@ using stream::mbar_try_wait;
 using stream::smem_u32;
 
 constexpr int BM = 128;                               // tokens per tile: rows of the accumulator = lanes of tensor memory
-constexpr int BN_MAX = 256;                           // most accumulator columns per tile (a launch picks 64, 128, 192 or 256)
+constexpr int BN_MAX = 256;                           // most accumulator columns per tile (a launch picks 128, 192 or 256)
 constexpr int BOX_N = 64;                             // weight rows per TMA box
 constexpr int BK = 64;                                // input columns per stage: 128 bytes of bf16 = one swizzle row
 // The ring of stages.  A stage is what a k-block of the launch needs: two boxes of a_rows activation rows (hi and lo plane)
@@ -301,7 +303,7 @@ __device__ __forceinline__ void finish_sums(const GemmArgs &g, int tile, int t, 
 // Tiles of 128 tokens x bn accumulator columns, dealt out to one CTA per SM (Jobs).  EPI = PF_SWIGLU: columns [0, bn / 2) are units n0 .. of
 // the gate matrix (map tb0) and columns [bn / 2, bn) the same units of the up matrix (map tb1); otherwise the columns
 // are units n0 .. n0 + bn - 1 of one matrix (tb0 = tb1).  ta covers both activation planes: rows [0, Tpad) the hi
-// terms, rows [Tpad, 2 Tpad) the lo terms.  The weight maps are read in boxes of BOX_N rows.
+// terms, rows [Tpad, 2 Tpad) the lo terms.  The weight maps are read in boxes of g.box rows.
 //
 // Accumulation.  The tensor core adds every 16-column product into its fp32 accumulator by truncation, so a sum that
 // stays in tensor memory over all of K collects an error that grows with the number of steps (measured: ~4e-5 relative

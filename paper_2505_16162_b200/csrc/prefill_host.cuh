@@ -54,8 +54,8 @@ inline bool gemm_attrs_once() {
     return ok;
 }
 
-// Most chunk sums a launch may leave in the scratch of the pieces (PIECE_FLOATS each, 72 MB in all: they have to stay in
-// L2 to be worth it).  20 tiles of 27 chunks - 5120 units at 13824 input columns, up to 128 rows - are 540.
+// Most chunk sums a launch may leave in the scratch of the pieces: PIECE_FLOATS each, 72 MB in all of the 126 MB of L2, which they
+// have to stay in to be worth it while weights and activations pass through it.
 constexpr int MAX_PIECES = 576;
 
 // Columns per tile, CTAs, how many tiles are done whole (the rest in pieces), and the chunk sums that the pieces leave.
@@ -68,7 +68,9 @@ struct Deal { int bn, grid, whole, sums; };
 //     columns: two rounds 144 us, of which the second has 12 tiles.
 //   pieces: 14 us for a launch, the fold behind it and the last sums, 1.3 x the products' time (pieces are not in step, so they share
 //     less through L2), and per chunk sum 0.012 us + 0.036 us per 128 KB to write and read it.  The same launch: one
-//     round + 12 tiles in 120 pieces, 93 us; at 77 rows, 20 tiles in 200 pieces 33 us against 63 us.
+//     round + 12 tiles in 120 pieces, 93 us; at 77 rows, 27 tiles in 270 pieces 29 us against 63 us.
+// Sums of a layer's four maps on other widths, measured launch by launch (modelled), us at 77 / 300 / 512 / 1024 rows: 7B 163 (179), 316
+// (290), 395 (383), 642 (578); 13B 213 (225), 432 (434), 548 (508), 934 (883); Qwen 14B 192 (202), 399 (390), 480 (449).
 // `heads`: 256 columns let the launch finish the heads itself; else a kernel of its own does.
 inline Deal deal_out(int T, int N, int K, bool swiglu, bool heads, int n_sms) {
     const int row_tiles = (T + BM - 1) / BM, nkb = K / BK, nchunks = (nkb + CHUNK_KB - 1) / CHUNK_KB;
