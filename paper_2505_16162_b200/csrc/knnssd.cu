@@ -91,7 +91,6 @@ struct knnssd_ctx {
     float2 *pf_cs = nullptr;                                 // rotary (cos, sin) of the chunk's rows [cap][hd / 2]
     float *pf_rinv = nullptr;                                // RMSNorm scale of the chunk's rows [cap]
     bf16_t *pf_ad = nullptr, *pf_aq = nullptr, *pf_af = nullptr;   // hi / lo planes [2][cap][d], [2][cap][nq], [2][cap][d_ff]
-    CUtensorMap pf_map_d{}, pf_map_q{}, pf_map_f{};
     float *pf_part = nullptr;                                // sums of the pieces of tiles that several CTAs share
 
     // instrumentation
@@ -640,20 +639,14 @@ bool prefill_tensor(knnssd_ctx *c, int n) {
     int *err = c->err_word;
     const size_t layer_stride = (size_t)Hkv * g.max_seq * HD;
     bool ok = true;
-    auto contract = [&](auto... a) {
-        const int n_launched = prefill::launch_gemm(a...);
+    auto contract = [&](const bf16_t *planes, const void *W0, const void *W1, int N, int K, int T, int epi, auto... a) {
+        const int n_launched = prefill::launch_gemm(prefill::deal_out(T, N, K, epi == prefill::PF_SWIGLU, c->n_sms), planes, c->pf_part, cap, W0, W1, N, K, T, epi, a...);
         c->launches += n_launched;
         return n_launched > 0;
     };
     for (int t0 = 0; t0 < n && ok; t0 += cap) {
         const int T = n - t0 < cap ? n - t0 : cap;
         const bool last = t0 + T == n;
-        CUtensorMap map_d = c->pf_map_d, map_q = c->pf_map_q, map_f = c->pf_map_f;
-        if (T < prefill::BM) {               // fewer rows than a tile: boxes of the live rows only
-            const int box = prefill::act_box_rows(T);
-            ok = prefill::make_map(&map_d, c->pf_ad, 2 * (size_t)cap, (size_t)d, box) && prefill::make_map(&map_q, c->pf_aq, 2 * (size_t)cap, (size_t)nq, box) &&
-                 prefill::make_map(&map_f, c->pf_af, 2 * (size_t)cap, (size_t)F, box);
-        }
         prefill::embed_rows_kernel<<<T, 256, 0, s>>>(reinterpret_cast<const bf16_t *>(c->tok_embed), c->prompt + t0, d, c->pf_x);
         prefill::rope_table_kernel<<<T, HD / 2, 0, s>>>(c->inv_freq, t0, c->pf_cs);
         c->launches += 2;
@@ -666,25 +659,25 @@ bool prefill_tensor(knnssd_ctx *c, int n) {
             if (nq % prefill::BOX_N == 0 && nkv % prefill::BOX_N == 0) {
                 // q, k and v in one launch over the stacked units (their columns of the projection buffer are adjacent)
                 const prefill::QkvFuse fuse{c->pf_cs, kc, vc, g.max_seq, t0, HD};
-                ok = ok && contract(map_d, c->pf_part, cap, ly.wq, ly.wk, ldq, d, T, prefill::PF_STORE, c->pf_qkv, ldq, 0, nullptr,
-                                                nullptr, 0, err, c->n_sms, s, ly.wv, nq, nkv, &fuse, &heads_done, c->pf_rinv);
+                ok = ok && contract(c->pf_ad, ly.wq, ly.wk, ldq, d, T, prefill::PF_STORE, c->pf_qkv, ldq, 0, nullptr,
+                                                nullptr, 0, err, s, ly.wv, nq, nkv, &fuse, &heads_done, c->pf_rinv);
             } else {
-                ok = ok && contract(map_d, c->pf_part, cap, ly.wq, nullptr, nq, d, T, prefill::PF_STORE, c->pf_qkv, ldq, 0, nullptr,
-                                                nullptr, 0, err, c->n_sms, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
-                ok = ok && contract(map_d, c->pf_part, cap, ly.wk, nullptr, nkv, d, T, prefill::PF_STORE, c->pf_qkv, ldq, nq, nullptr,
-                                                nullptr, 0, err, c->n_sms, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
-                ok = ok && contract(map_d, c->pf_part, cap, ly.wv, nullptr, nkv, d, T, prefill::PF_STORE, c->pf_qkv, ldq, nq + nkv,
-                                                nullptr, nullptr, 0, err, c->n_sms, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
+                ok = ok && contract(c->pf_ad, ly.wq, nullptr, nq, d, T, prefill::PF_STORE, c->pf_qkv, ldq, 0, nullptr,
+                                                nullptr, 0, err, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
+                ok = ok && contract(c->pf_ad, ly.wk, nullptr, nkv, d, T, prefill::PF_STORE, c->pf_qkv, ldq, nq, nullptr,
+                                                nullptr, 0, err, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
+                ok = ok && contract(c->pf_ad, ly.wv, nullptr, nkv, d, T, prefill::PF_STORE, c->pf_qkv, ldq, nq + nkv,
+                                                nullptr, nullptr, 0, err, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
             }
             if (!heads_done) launch_chained(prefill::rope_kv_rows_kernel, dim3(T, prefill::ROPE_PARTS), dim3(256), 0, s, c->pf_qkv, H, Hkv, HD, c->pf_cs, kc, vc, g.max_seq, t0);
             launch_chained(prefill::attn_prompt_kernel<HD>, dim3(H, (T + 63) / 64), dim3(128), prefill::attn_smem_bytes<HD>(), s, c->pf_qkv, H, Hkv, kc, vc, g.max_seq, t0, T, c->pf_aq, c->pf_aq + (size_t)cap * nq);
-            ok = ok && contract(map_q, c->pf_part, cap, ly.wo, nullptr, d, nq, T, prefill::PF_ADD, c->pf_x, d, 0, nullptr, nullptr, 0,
-                                            err, c->n_sms, s);
+            ok = ok && contract(c->pf_aq, ly.wo, nullptr, d, nq, T, prefill::PF_ADD, c->pf_x, d, 0, nullptr, nullptr, 0,
+                                            err, s);
             launch_chained(prefill::norm_split_kernel, dim3(T), dim3(256), 0, s, c->pf_x, d, ly.mlp_norm, g.rms_eps, c->pf_ad, c->pf_ad + (size_t)cap * d, c->pf_rinv);
-            ok = ok && contract(map_d, c->pf_part, cap, ly.w_gate, ly.w_up, F, d, T, prefill::PF_SWIGLU, nullptr, 0, 0, c->pf_af,
-                                            c->pf_af + (size_t)cap * F, F, err, c->n_sms, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
-            ok = ok && contract(map_f, c->pf_part, cap, ly.w_down, nullptr, d, F, T, prefill::PF_ADD, c->pf_x, d, 0, nullptr, nullptr,
-                                            0, err, c->n_sms, s);
+            ok = ok && contract(c->pf_ad, ly.w_gate, ly.w_up, F, d, T, prefill::PF_SWIGLU, nullptr, 0, 0, c->pf_af,
+                                            c->pf_af + (size_t)cap * F, F, err, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
+            ok = ok && contract(c->pf_af, ly.w_down, nullptr, d, F, T, prefill::PF_ADD, c->pf_x, d, 0, nullptr, nullptr,
+                                            0, err, s);
             c->launches += heads_done ? 3 : 4;                   // besides the contractions
         }
         // pooled numerator: every row's final hidden state (mean pooling) or the last row's
@@ -929,7 +922,7 @@ knnssd_status knnssd_init(const knnssd_config *cfg, const knnssd_weights *w, con
         if (!ok2) { cudaGetLastError(); return bail(KNNSSD_ERR_CUDA); }
         // tensor-core prompt pass: needs the driver's tensor-map encoder; without it prompts go through the pass kernel
         if (prefill::encode_tiled_fn() && prefill::gemm_attrs_once()) {
-            const int cap_seq = (g.max_seq + prefill::BM - 1) / prefill::BM * prefill::BM;
+            const int cap_seq = (g.max_seq + prefill::ROW_PAD - 1) / prefill::ROW_PAD * prefill::ROW_PAD;
             c->pf_cap = cap_seq < 1024 ? cap_seq : 1024;
             const size_t cap = (size_t)c->pf_cap;
             bool ok3 = true;
@@ -942,15 +935,13 @@ knnssd_status knnssd_init(const knnssd_config *cfg, const knnssd_weights *w, con
             ok3 &= dev_alloc(&c->pf_ad, 2 * cap * d) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_aq, 2 * cap * nq) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_af, 2 * cap * g.d_ff) == cudaSuccess;
-            const int sums = prefill::most_sums(c->pf_cap, d, nq, nkv, g.d_ff, hd, c->n_sms);
-            ok3 &= sums == 0 || dev_alloc(&c->pf_part, (size_t)sums * prefill::PIECE_FLOATS) == cudaSuccess;
+            const size_t sums = prefill::most_sums(c->pf_cap, d, nq, nkv, g.d_ff, c->n_sms);
+            ok3 &= sums == 0 || dev_alloc(&c->pf_part, sums) == cudaSuccess;
             if (!ok3) { cudaGetLastError(); return bail(KNNSSD_ERR_CUDA); }
             cudaMemsetAsync(c->pf_ad, 0, 2 * cap * d * sizeof(bf16_t), c->stream);
             cudaMemsetAsync(c->pf_aq, 0, 2 * cap * nq * sizeof(bf16_t), c->stream);
             cudaMemsetAsync(c->pf_af, 0, 2 * cap * g.d_ff * sizeof(bf16_t), c->stream);
-            c->pf_ok = prefill::make_map(&c->pf_map_d, c->pf_ad, 2 * cap, (size_t)d, prefill::BM) &&
-                       prefill::make_map(&c->pf_map_q, c->pf_aq, 2 * cap, (size_t)nq, prefill::BM) &&
-                       prefill::make_map(&c->pf_map_f, c->pf_af, 2 * cap, (size_t)g.d_ff, prefill::BM);
+            c->pf_ok = true;
         }
         pass::Model &md = c->model;
         md.tok_embed = reinterpret_cast<const bf16_t *>(c->tok_embed); md.final_norm = c->final_norm; md.rms_eps = g.rms_eps;
@@ -1490,24 +1481,22 @@ knnssd_status knnssd_gemm_split(const void *W0_dev, const void *W1_dev, int n_ou
     int dev = 0, n_sms = 148;
     if (cudaGetDevice(&dev) != cudaSuccess) return KNNSSD_ERR_CUDA;
     cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev);
-    const int cap = (T + prefill::BM - 1) / prefill::BM * prefill::BM;
+    const int cap = (T + prefill::ROW_PAD - 1) / prefill::ROW_PAD * prefill::ROW_PAD;
     bf16_t *planes = nullptr, *outp = nullptr;
     float *part = nullptr;
     int *err = nullptr;
-    const int sums = prefill::deal_out(T, n_out, n_in, mode == 2, false, n_sms).sums;
+    const prefill::Deal deal = prefill::deal_out(T, n_out, n_in, mode == 2, n_sms);
     const size_t plane = (size_t)cap * n_in, oplane = (size_t)T * n_out;
     Scratch mem(s);
     if (!mem.get(&planes, 2 * plane) || (mode == 2 && !mem.get(&outp, 2 * oplane)) ||
-        (sums > 0 && !mem.get(&part, (size_t)sums * prefill::PIECE_FLOATS)) || !mem.get(&err, 1))
+        (deal.sums > 0 && !mem.get(&part, deal.sums)) || !mem.get(&err, 1))
         return KNNSSD_ERR_CUDA;
     cudaMemsetAsync(err, 0, sizeof(int), s);
     knnssd_status st = KNNSSD_OK;
     cudaMemsetAsync(planes, 0, 2 * plane * sizeof(bf16_t), s);
     prefill::split_rows_kernel<<<T, 256, 0, s>>>(x_dev, n_in, planes, planes + plane);
-    CUtensorMap ta;
-    if (!prefill::make_map(&ta, planes, (size_t)2 * cap, (size_t)n_in, prefill::act_box_rows(T)) ||
-        !prefill::launch_gemm(ta, part, cap, W0_dev, W1_dev, n_out, n_in, T, mode, y_dev, n_out, 0, outp, outp ? outp + oplane : nullptr,
-                              n_out, err, n_sms, s))
+    if (!prefill::launch_gemm(deal, planes, part, cap, W0_dev, W1_dev, n_out, n_in, T, mode, y_dev, n_out, 0, outp, outp ? outp + oplane : nullptr,
+                              n_out, err, s))
         st = KNNSSD_ERR_CUDA;
     if (st == KNNSSD_OK && mode == 2) prefill::join_planes_kernel<<<T, 256, 0, s>>>(outp, outp + oplane, n_out, y_dev);
     cudaError_t e = cudaStreamSynchronize(s);

@@ -18,9 +18,6 @@ namespace knnssd {
 namespace lintc {
 
 using prefill::pf_wait;
-using prefill::tma_load_2d;
-using prefill::umma_bf16;
-using prefill::umma_commit;
 using prefill::umma_desc;
 using prefill::umma_idesc;
 using stream::mbar_init;
@@ -36,6 +33,27 @@ constexpr int STAGE_BYTES = W_BYTES + 2 * X_BYTES;
 constexpr int THREADS = 192;                // warp 0: TMA; warp 1: MMA issue + tensor-memory owner; warps 2..5: epilogue
 constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + 256;
 constexpr int TMEM_COLS = 32;               // smallest allocation; 16 columns are used
+
+__device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar) {
+    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(
+                     smem_u32(dst)),
+                 "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y)
+                 : "memory");
+}
+__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t"
+        ".reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
+        "}\n" ::"r"(tmem_d),
+        "l"(da), "l"(db), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// The barrier gets one arrival once every MMA this thread issued before has finished.
+__device__ __forceinline__ void umma_commit(uint64_t *bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
 
 struct Args {
     int M;          // live rows (1..16)
@@ -102,7 +120,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap tw, const __grid_constant__
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            const uint32_t idesc = umma_idesc(TN);
+            const uint32_t idesc = umma_idesc(TM, TN);
             for (int kb = 0; kb < nkb; ++kb) {
                 const int s = kb % STAGES;
                 const uint32_t ph = (uint32_t)(kb / STAGES) & 1u;

@@ -32,24 +32,29 @@ using stream::mbar_init;
 using stream::mbar_try_wait;
 using stream::smem_u32;
 
-constexpr int BM = 128;                               // tokens per tile: rows of the accumulator = lanes of tensor memory
-constexpr int BN_MAX = 256;                           // most accumulator columns per tile (a launch picks 128, 192 or 256)
+constexpr int ROW_PAD = 128;                          // the activation planes' rows are padded to a multiple of this
+constexpr int PAIR_UNITS = 256;                       // weight rows per tile: 128 in each CTA of a pair = lanes of its tensor memory
+constexpr int TT_MAX = 256, TT_STEP = 32;             // most tokens per tile = accumulator columns; a launch picks a multiple of 32
 constexpr int BOX_N = 64;                             // weight rows per TMA box
 constexpr int BK = 64;                                // input columns per stage: 128 bytes of bf16 = one swizzle row
-// The ring of stages.  A stage is what a k-block of the launch needs: two boxes of a_rows activation rows (hi and lo plane)
-// and bn weight rows, 64 KB at 128 rows and 256 columns (three stages), 56 KB at 192 columns (four).  A launch takes no
-// more shared memory than its stages: the add epilogue reads 32 bytes of a row at a time and lives on what is left as L1.
-constexpr int RING_BYTES = 224 * 1024;
+constexpr int W_BYTES = 128 * BK * 2;                 // a CTA's weight rows of a stage
+// The ring of stages.  A stage is what a CTA holds of a k-block: 128 weight rows and half of the tile's token rows of either
+// plane, 48 KB at 256 tokens (four stages), 26 KB at 80 (seven).
+constexpr int RING_BYTES = 192 * 1024;
 constexpr int MAX_STAGES = 10;
-__host__ __device__ constexpr int ring_stages(int a_rows, int bn) {
-    return RING_BYTES / ((2 * a_rows + bn) * BK * 2) < MAX_STAGES ? RING_BYTES / ((2 * a_rows + bn) * BK * 2) : MAX_STAGES;
+__host__ __device__ constexpr int stage_bytes_of(int tt) { return W_BYTES + tt * BK * 2; }
+__host__ __device__ constexpr int ring_stages(int tt) {
+    return RING_BYTES / stage_bytes_of(tt) < MAX_STAGES ? RING_BYTES / stage_bytes_of(tt) : MAX_STAGES;
 }
-constexpr int TMEM_COLS = 512;                        // columns of tensor memory a CTA takes: two accumulators of BN_MAX columns
+constexpr int TURN_TOKENS = 16;                       // tokens that a group of epilogue warps turns at a time (see below)
+constexpr int TURN_BYTES = 2 * 2 * TURN_TOKENS * 128 * 4;      // two groups, two buffers each
+constexpr int TMEM_COLS = 512;                        // columns of tensor memory a CTA takes: two accumulators of TT_MAX columns
 constexpr int CHUNK_KB = 8;                           // k-blocks accumulated in tensor memory before the sum moves to registers
 constexpr int GEMM_THREADS = 320;                     // warp 0: TMA; warp 1: MMA issue + tensor-memory owner; warps 2..9: epilogue
-__host__ __device__ constexpr int gemm_smem(int a_rows, int bn) {     // + slack to align the tiles to 1024 bytes + barriers
-    return ring_stages(a_rows, bn) * (2 * a_rows + bn) * BK * 2 + 1024 + 256;
+__host__ __device__ constexpr int gemm_smem(int tt) {          // + slack to align the tiles to 1024 bytes + barriers
+    return TURN_BYTES + ring_stages(tt) * stage_bytes_of(tt) + 1024 + 256;
 }
+constexpr int GEMM_SMEM_MAX = TURN_BYTES + RING_BYTES + 1024 + 256;
 constexpr unsigned WAIT_LIMIT = 4000000u;           // polls of one wait (a whole tile takes well under a millisecond)
 
 enum { PF_STORE = 0, PF_ADD = 1, PF_SWIGLU = 2, PF_QKV = 3 };
@@ -58,37 +63,47 @@ struct GemmArgs {
     int T;             // live rows
     int K;             // input width, a multiple of BK
     int N;             // output units (per matrix)
-    int bn;            // accumulator columns per tile: a multiple of 64 (SwiGLU: of 128), at most BN_MAX
-    float *y;          // STORE: y[t * ldy + col0 + n] = sum;  ADD: y[t * ldy + n] += sum
+    int tt;            // tokens per tile: a multiple of TT_STEP, at most TT_MAX
+    float *y;          // STORE: y[t * ldy + col0 + n] = sum;  ADD: y[t * ldy + col0 + n] += sum
     int ldy, col0;
     bf16_t *out_hi;    // SWIGLU: silu(gate) * up as two bf16 planes, [t * ldo + n]
     bf16_t *out_lo;
     int ldo;
     int *err;          // set non-zero if a bounded wait gave up
-    int tiles_x, tiles_y;   // row tiles and column tiles of the launch (tile = ty tiles_x + tx)
-    int box;           // weight rows per box: BOX_N, or 128 where tiles and matrices allow it (a box costs the copy engine ~0.13 us
-                       // whatever its height: 0.75 -> 0.6 us per k-block of 256 columns for the copies alone)
-    int a_rows;        // rows of an activation box (the maps' box height): BM, or T rounded up to 8 where T < BM
-    int whole;         // tiles [0, whole) are done whole by one CTA each, the others in pieces (see Jobs below)
-    float *part;       // the chunk sums of the tiles done in pieces, [tiles_x tiles_y - whole][chunks][PIECE_FLOATS]: what
+    int tiles_x, tiles_y;   // token tiles and unit tiles of the launch (tile = ty tiles_x + tx)
+    int box;           // weight rows per box: BOX_N, or 128 where the matrices allow it
+    int whole;         // tiles [0, whole) are done whole by one pair each, the others in pieces (see Jobs below)
+    float *part;       // the chunk sums of the tiles done in pieces, [tiles - whole][chunks][CTA of the pair][tt][128]: what
                        // gemm_split_kernel leaves and fold_pieces_kernel picks up
     int nA, nB;        // STORE over stacked matrices (q, k, v in one launch): units [0, nA) are rows of map tb0,
                        // [nA, nA + nB) rows of tb1, the rest rows of tb2; all multiples of BOX_N.  One matrix: nA = N
-    // PF_QKV (stacked q, k, v; head dimension 128, bn = 256: an epilogue thread holds one head of its token): the q
-    // heads are rotated and stored to y, the k heads rotated, the k and v heads rounded to bf16 into the cache rows
-    // of position pos0 + t
     const float *row_scale;   // if given: every sum of row t is multiplied by row_scale[t] before the epilogue (the RMSNorm
                               // scale of the row whose gain-weighted, un-normalised values the planes hold)
+    // PF_QKV (stacked q, k, v; head dimension 128, so that a CTA's 128 weight rows are one head): the q heads are rotated
+    // and stored to y, the k heads rotated, the k and v heads rounded to bf16 into the cache rows of position pos0 + t
     const float2 *rope;    // [T][64] (cos, sin) of the rows' positions
     bf16_t *kc, *vc;       // this layer's K and V cache, [kv head][max_seq][128]
     int max_seq, pos0;
 };
 
-__device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar) {
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(
-                     smem_u32(dst)),
-                 "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y)
+// What one thread of a warp issues - copies, products, commits - takes its operands in uniform registers.  Inside a branch on the lane
+// the compiler has to move each of them there first (46 clocks per product of any size, 0.08 us per copy), so the warp
+// runs these loops as a whole and the instructions are predicated: `one` is 1 in the thread that issues them.
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t one;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one));
+    return one;
+}
+// A TMA load into this CTA's shared memory (dst) whose bytes are counted by a barrier of the pair's first CTA (`bar`: its address
+// in the cluster's window).
+__device__ __forceinline__ void tma_load_pair(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar, uint64_t policy, uint32_t one) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %6, 0;\n\t"
+                 "@p cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5;\n\t}" ::"r"(dst),
+                 "l"(map), "r"(bar), "r"(x), "r"(y), "l"(policy), "r"(one)
                  : "memory");
+}
+__device__ __forceinline__ void expect_tx_if(uint32_t bar, uint32_t bytes, uint32_t one) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}" ::"r"(bar), "r"(bytes), "r"(one) : "memory");
 }
 
 // Shared-memory operand descriptor of tcgen05.mma for a K-major tile whose rows are 128 bytes, written by TMA with the
@@ -101,26 +116,48 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t saddr) {
 }
 // Instruction descriptor, kind::f16: fp32 accumulator (bits 4..5 = 1), A and B bf16 (bits 7..9 and 10..12 = 1), both
 // K-major (bits 15, 16 = 0), N / 8 in bits 17..22, M / 16 in bits 24..28.
-__device__ __forceinline__ uint32_t umma_idesc(int n) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+__device__ __forceinline__ uint32_t umma_idesc(int m, int n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t"
-        ".reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
-        "}\n" ::"r"(tmem_d),
-        "l"(da), "l"(db), "r"(idesc), "r"(accumulate)
-        : "memory");
+// One instruction for the pair, issued by its first CTA: the 256 rows of A are 128 rows of either CTA's shared memory, the
+// columns of B half of either's, at the same addresses; a CTA's tensor memory takes the sums of its own 128 rows.  a, b: the
+// operands' descriptors without their constant upper halves.  The weights of a k-step meet the hi and the lo terms: FIRST reads them
+// from shared memory, the product behind it takes them from where the first left them.
+constexpr uint32_t DESC_UPPER = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t desc_lower(uint32_t saddr) { return (saddr >> 4) | (1u << 16); }
+template <bool FIRST>
+__device__ __forceinline__ void umma_pair(uint32_t tmem_d, uint32_t a, uint32_t b, uint32_t idesc, uint32_t accumulate, uint32_t one) {
+#define KNNSSD_UMMA_PAIR(COLLECT) \
+    asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\tmov.b64 da, {%1, %6};\n\tmov.b64 db, {%2, %6};\n\t" \
+                 "@q tcgen05.mma.cta_group::2.kind::f16.collector::a::" COLLECT " [%0], da, db, %3, p;\n\t}\n" \
+                 ::"r"(tmem_d), "r"(a), "r"(b), "r"(idesc), "r"(accumulate), "r"(one), "r"(DESC_UPPER) : "memory")
+    if (FIRST) KNNSSD_UMMA_PAIR("fill");
+    else KNNSSD_UMMA_PAIR("lastuse");
+#undef KNNSSD_UMMA_PAIR
 }
-// The barrier gets one arrival once every MMA this thread issued before has finished.
-__device__ __forceinline__ void umma_commit(uint64_t *bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+// The barrier at this address in both CTAs gets one arrival once every MMA this thread issued before has finished.
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint32_t one) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}" ::"r"(bar),
+                 "h"((uint16_t)3), "r"(one)
+                 : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+
+// The address of the pair's first CTA's copy of a shared-memory word.
+__device__ __forceinline__ uint32_t first_cta_addr(const void *p) {
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(smem_u32(p)));
+    return a;
+}
+__device__ __forceinline__ void pair_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void pair_sync() {
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
 
 // 32 consecutive accumulator columns of this thread's lane (lane = 32 * (warp % 4) + lane id).
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
@@ -139,10 +176,18 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// mbar_try_wait for a barrier whose other CTA's arrivals have to be seen with what they release.
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t *b, uint32_t parity) {
+    uint32_t done;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(done) : "r"(smem_u32(b)), "r"(parity) : "memory");
+    return done != 0;
+}
+
 // Bounded wait on an mbarrier phase; false once the limit is reached or another thread of the CTA has given up.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool pf_wait(uint64_t *b, uint32_t parity, volatile int *cta_abort, int *err, int code) {
     unsigned spins = 0;
-    while (!mbar_try_wait(b, parity)) {
+    while (!(CLUSTER ? mbar_try_wait_cluster(b, parity) : mbar_try_wait(b, parity))) {
         if (*cta_abort) return false;
         if (++spins > WAIT_LIMIT) {
             *cta_abort = 1;
@@ -153,40 +198,19 @@ __device__ __forceinline__ bool pf_wait(uint64_t *b, uint32_t parity, volatile i
     return true;
 }
 
-// 32 bytes, a sector: in one access at a 32-byte boundary (whole), else in two at a 16-byte boundary.
-__device__ __forceinline__ void ld_sector(const float *p, float (&v)[8], bool whole) {
-    if (whole) {
-        asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]) : "l"(p) : "memory");
-    } else {
-        const float4 a = *reinterpret_cast<const float4 *>(p), b = *reinterpret_cast<const float4 *>(p + 4);
-        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-    }
-}
-__device__ __forceinline__ void st_sector(float *p, const float (&v)[8], bool whole) {
-    if (whole) {
-        asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]),
-                     "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]) : "memory");
-    } else {
-        *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
-        *reinterpret_cast<float4 *>(p + 4) = make_float4(v[4], v[5], v[6], v[7]);
-    }
-}
-
 __device__ __forceinline__ uint32_t pack_bf16(uint32_t lo16, uint32_t hi16) { return lo16 | (hi16 << 16); }
 
-// How a launch's work is dealt out to its CTAs (one per SM).  Tiles [0, whole) go round: CTA c takes tiles c, c + G, ..,
-// so that all CTAs are at the same k-blocks of neighbouring tiles and share them through L2 (walking a contiguous run of
-// tiles each instead cost 1.05 us per k-block against 0.81: the weights of all column tiles in flight at once).  The
-// chunks (CHUNK_KB k-blocks) of the tiles that are left, fewer than the CTAs, are dealt out evenly, CTA c of P getting
-// chunks [c U / P, (c + 1) U / P): a last round that would leave most of the chip idle takes the time its work takes.
+// How a launch's work is dealt out to its pairs of CTAs (one CTA per SM).  Tiles [0, whole) go round: pair c takes tiles c,
+// c + G, .., so that all pairs are at the same k-blocks of neighbouring tiles and share them through L2.  The chunks (CHUNK_KB
+// k-blocks) of the tiles that are left, fewer than the pairs, are dealt out evenly, pair c of P getting chunks
+// [c U / P, (c + 1) U / P): a last round that would leave most of the chip idle takes the time its work takes.
 // A piece's chunk sums go to `part` one by one, and fold_pieces_kernel, launched behind, adds a tile's up from the first chunk
-// to the last, the order of a tile done whole: a row's numbers do not depend on how the launch was dealt out.  No CTA waits
+// to the last, the order of a tile done whole: a row's numbers do not depend on how the launch was dealt out.  No pair waits
 // for another: a launch that is not cooperative may run in parts, with another stream's launch on the SMs between them.
 struct Jobs {
-    int G, P, cta, whole, nchunks, n_whole, r0;      // P: the CTAs that get pieces, one chunk each at least
+    int G, P, cta, whole, nchunks, n_whole, r0;      // P: the pairs that get pieces, one chunk each at least
     long long units, u0, u1;
-    __device__ __forceinline__ Jobs(const GemmArgs &g) : G(gridDim.x), cta(blockIdx.x), whole(g.whole) {
+    __device__ __forceinline__ Jobs(const GemmArgs &g) : G(gridDim.x >> 1), cta(blockIdx.x >> 1), whole(g.whole) {
         nchunks = (g.K / BK + CHUNK_KB - 1) / CHUNK_KB;
         n_whole = cta < whole ? (whole - cta + G - 1) / G : 0;
         units = (long long)(g.tiles_x * g.tiles_y - whole) * nchunks;
@@ -195,7 +219,7 @@ struct Jobs {
         u1 = cta < P ? units * (cta + 1) / P : 0;
         r0 = (int)(u0 / nchunks);
     }
-    // job i of this CTA: chunks [c0, c1) of a tile; false when there is none
+    // job i of this pair: chunks [c0, c1) of a tile; false when there is none
     __device__ __forceinline__ bool get(int i, int &tile, int &c0, int &c1) const {
         if (i < n_whole) { tile = cta + i * G; c0 = 0; c1 = nchunks; return true; }
         const int r = r0 + i - n_whole;
@@ -207,7 +231,6 @@ struct Jobs {
         return true;
     }
 };
-constexpr int PIECE_FLOATS = BM * BN_MAX;      // a chunk's sums, by register group and thread (coalesced): 32 x 256 float4
 
 // Rotary embedding of a pair by (cos, sin) = c.  The rounding is spelled out: left to the compiler, the contraction's epilogue and
 // rope_kv_rows_kernel fused other products of the second sum, and a row's K depended on which of them a launch's sizes chose.
@@ -217,93 +240,82 @@ __device__ __forceinline__ void rotate_pair(float &a, float &b, float2 c) {
     a = ra;
 }
 
-// Tile column of register group gi (32 columns) of an epilogue thread, or -1 if the group is not in use.  Store / add: half
-// hsel of the columns in groups of 32; SwiGLU: groups 0 and 1 a quarter of them in the gate columns, 2 and 3 the up columns of
-// the same units.
-template <int EPI> __device__ __forceinline__ int group_col(int gi, int hsel, int bn) {
-    if (EPI == PF_SWIGLU) {
-        const int gg = gi & 1, qtr = bn / 4;
-        return 32 * gg < qtr ? (gi >= 2 ? bn / 2 : 0) + hsel * qtr + 32 * gg : -1;
-    }
-    return 32 * gi < bn / 2 ? hsel * (bn / 2) + 32 * gi : -1;
+// First unit of a CTA's 128 weight rows (SwiGLU: 64 gate rows, then the up rows of the same 64 units).
+template <int EPI> __device__ __forceinline__ int first_unit(int ty, int rank) {
+    return EPI == PF_SWIGLU ? ty * (PAIR_UNITS / 2) + 64 * rank : ty * PAIR_UNITS + 128 * rank;
 }
 
-// What becomes of 16 sums of token t of a tile: register k8 .. k8 + 7 in v[0 .. 7], 64 + k8 .. in v[8 .. 15] (k8 = 8 k).
-// SwiGLU: gate and up columns of eight units; q / k / v heads: eight pairs (j, j + 64) of one head; else columns.
-// y32: y lies at a 32-byte boundary (ldy, col0 and the columns are multiples of 8).
-template <int EPI>
-__device__ __forceinline__ void finish_sums(const GemmArgs &g, int tile, int t, int hsel, int k8, bool y32, float (&v)[16]) {
-    const int half = g.bn / 2, qtr = g.bn / 4;
-    const int n0 = (tile / g.tiles_x) * (EPI == PF_SWIGLU ? half : g.bn);
+// ADD: the old values of token t that finish_sums takes for weight rows j .. j + 3 and j + 64 .. j + 67.
+template <int EPI> __device__ __forceinline__ void old_values(const GemmArgs &g, int u0, int t, int j, float4 (&x)[2]) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        x[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (EPI == PF_ADD && t < g.T && u0 + j + 64 * e < g.N) x[e] = *reinterpret_cast<const float4 *>(g.y + (size_t)t * g.ldy + g.col0 + u0 + j + 64 * e);
+    }
+}
+
+// What becomes of the sums of token t for the weight rows j .. j + 3 (v[0 .. 3]) and j + 64 .. j + 67 (v[4 .. 7]) of a CTA whose
+// rows start at unit u0; j is a multiple of 4 below 64.  SwiGLU: gate and up of four units; q / k / v heads: four pairs of one
+// head; else units.  Products that meet a sum are rounded by themselves, whichever kernel this is part of.
+template <int EPI> __device__ __forceinline__ void finish_sums(const GemmArgs &g, int u0, int t, int j, float (&v)[8], const float4 (&x)[2]) {
     if (g.row_scale) {
         const float rs = g.row_scale[t];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] *= rs;
+        for (int i = 0; i < 8; ++i) v[i] = __fmul_rn(v[i], rs);
     }
     if (EPI == PF_SWIGLU) {
-        const int u = n0 + hsel * qtr + k8;
-        if (k8 >= qtr || u >= g.N) return;
-        uint32_t hi[4], lo[4];
+        if (u0 + j >= g.N) return;                       // N is a multiple of 8
+        uint32_t h[4], l[4];
 #pragma unroll
-        for (int i = 0; i < 8; i += 2) {
-            uint32_t h2[2], l2[2];
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const float gt = v[i + e], up = v[8 + i + e];
-                const float a = gt / (1.0f + expf(-gt)) * up;
-                h2[e] = float_to_bf16_rne(a);
-                l2[e] = float_to_bf16_rne(a - __uint_as_float(h2[e] << 16));
-            }
-            hi[i >> 1] = pack_bf16(h2[0], h2[1]);
-            lo[i >> 1] = pack_bf16(l2[0], l2[1]);
+        for (int i = 0; i < 4; ++i) {
+            const float a = __fmul_rn(v[i] / (1.0f + expf(-v[i])), v[4 + i]);
+            h[i] = float_to_bf16_rne(a);
+            l[i] = float_to_bf16_rne(a - __uint_as_float(h[i] << 16));
         }
-        *reinterpret_cast<uint4 *>(g.out_hi + (size_t)t * g.ldo + u) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-        *reinterpret_cast<uint4 *>(g.out_lo + (size_t)t * g.ldo + u) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+        const size_t at = (size_t)t * g.ldo + u0 + j;
+        *reinterpret_cast<uint2 *>(g.out_hi + at) = make_uint2(pack_bf16(h[0], h[1]), pack_bf16(h[2], h[3]));
+        *reinterpret_cast<uint2 *>(g.out_lo + at) = make_uint2(pack_bf16(l[0], l[1]), pack_bf16(l[2], l[3]));
     } else if (EPI == PF_QKV) {
-        const int u0 = n0 + hsel * 128;                  // the head's first unit of the stacked q / k / v units
         if (u0 >= g.N) return;
         if (u0 < g.nA + g.nB) {                          // a q or a k head: rotary embedding
-            const float2 *cs = g.rope + (size_t)t * 64 + k8;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) rotate_pair(v[i], v[8 + i], cs[i]);
+            const float4 *cs = reinterpret_cast<const float4 *>(g.rope + (size_t)t * 64 + j);
+            const float4 c0 = cs[0], c1 = cs[1];
+            rotate_pair(v[0], v[4], make_float2(c0.x, c0.y));
+            rotate_pair(v[1], v[5], make_float2(c0.z, c0.w));
+            rotate_pair(v[2], v[6], make_float2(c1.x, c1.y));
+            rotate_pair(v[3], v[7], make_float2(c1.z, c1.w));
         }
         const bool is_k = u0 < g.nA + g.nB;
         const int kvh = (u0 - g.nA - (is_k ? 0 : g.nB)) >> 7;
 #pragma unroll
-        for (int e = 0; e < 16; e += 8) {
+        for (int e = 0; e < 2; ++e) {
             if (u0 < g.nA) {
-                float *yp = g.y + (size_t)t * g.ldy + g.col0 + u0 + 8 * e + k8;
-                float o[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) o[i] = v[e + i];
-                st_sector(yp, o, y32);
+                *reinterpret_cast<float4 *>(g.y + (size_t)t * g.ldy + g.col0 + u0 + j + 64 * e) = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
             } else {
-                bf16_t *dst = (is_k ? g.kc : g.vc) + ((size_t)kvh * g.max_seq + g.pos0 + t) * 128 + 8 * e + k8;
-                uint32_t w[4];
+                bf16_t *dst = (is_k ? g.kc : g.vc) + ((size_t)kvh * g.max_seq + g.pos0 + t) * 128 + j + 64 * e;
+                uint32_t w[2];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) w[i] = pack_bf16(float_to_bf16_rne(v[e + 2 * i]), float_to_bf16_rne(v[e + 2 * i + 1]));
-                *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+                for (int i = 0; i < 2; ++i) w[i] = pack_bf16(float_to_bf16_rne(v[4 * e + 2 * i]), float_to_bf16_rne(v[4 * e + 2 * i + 1]));
+                *reinterpret_cast<uint2 *>(dst) = make_uint2(w[0], w[1]);
             }
         }
     } else {
 #pragma unroll
-        for (int e = 0; e < 16; e += 8) {
-            const int r = 8 * e + k8, n = n0 + hsel * half + r;
-            if (r >= half || n >= g.N) continue;         // N is a multiple of 8
-            float *yp = g.y + (size_t)t * g.ldy + g.col0 + n;
-            float o[8], x[8];
-            if (EPI == PF_ADD) ld_sector(yp, x, y32);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) o[i] = EPI == PF_ADD ? v[e + i] + x[i] : v[e + i];
-            st_sector(yp, o, y32);
+        for (int e = 0; e < 2; ++e) {
+            if (u0 + j + 64 * e >= g.N) continue;        // N is a multiple of 8
+            float4 o = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+            if (EPI == PF_ADD) { o.x += x[e].x; o.y += x[e].y; o.z += x[e].z; o.w += x[e].w; }
+            *reinterpret_cast<float4 *>(g.y + (size_t)t * g.ldy + g.col0 + u0 + j + 64 * e) = o;
         }
     }
 }
 
-// Tiles of 128 tokens x bn accumulator columns, dealt out to one CTA per SM (Jobs).  EPI = PF_SWIGLU: columns [0, bn / 2) are units n0 .. of
-// the gate matrix (map tb0) and columns [bn / 2, bn) the same units of the up matrix (map tb1); otherwise the columns
-// are units n0 .. n0 + bn - 1 of one matrix (tb0 = tb1).  ta covers both activation planes: rows [0, Tpad) the hi
-// terms, rows [Tpad, 2 Tpad) the lo terms.  The weight maps are read in boxes of g.box rows.
+// Tiles of 256 weight rows x tt tokens, dealt out to pairs of CTAs, one CTA per SM (Jobs).  The weights are the row operand of
+// the products, 128 rows in either CTA, and the tokens their columns, so that a tile takes any multiple of 32 tokens; each
+// CTA brings in half of the token rows of both planes, and the pair's tensor cores read both halves.  EPI = PF_SWIGLU: a CTA's
+// rows are 64 units of the gate matrix (map tb0) and the same units of the up matrix (map tb1); otherwise units of one
+// matrix (tb0 = tb1).  ta covers both activation planes: rows [0, Tpad) the hi terms, rows [Tpad, 2 Tpad) the lo terms, in boxes
+// of tt / 2 rows (rows past T are whatever the planes hold; they meet no live token).  Weight maps: boxes of g.box rows.
 //
 // Accumulation.  The tensor core adds every 16-column product into its fp32 accumulator by truncation, so a sum that
 // stays in tensor memory over all of K collects an error that grows with the number of steps (measured: ~4e-5 relative
@@ -311,242 +323,270 @@ __device__ __forceinline__ void finish_sums(const GemmArgs &g, int tile, int t, 
 // that showed as 2.4e-2 on the logits of a 40-layer model).  The sum over K is therefore cut into chunks of CHUNK_KB
 // k-blocks: a chunk accumulates in one of two accumulators in tensor memory while the eight epilogue warps move the
 // previous chunk's sum out and add it, rounded to nearest, to the running sums they keep in registers (a thread owns
-// one token row and half of the tile's columns).  The error left is that of the short chunks plus K / (64 CHUNK_KB)
+// one weight row and half of the tile's tokens).  The error left is that of the short chunks plus K / (64 CHUNK_KB)
 // ordinary fp32 additions.
+//
+// The sums of a tile done whole lie with their weight row's thread; what finishes them (rotary pairs, gate and up, rows of y)
+// wants four neighbouring units of a token in one thread, so a group of four warps turns 16 tokens at a time through shared memory.
 template <int EPI>
-__global__ void __launch_bounds__(GEMM_THREADS, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
 gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb0,
                   const __grid_constant__ CUtensorMap tb1, const __grid_constant__ CUtensorMap tb2, GemmArgs g, int Tpad) {
-    const int bn = g.bn, per = EPI == PF_SWIGLU ? bn / 2 : bn;      // units of a matrix per tile
-    const int a_bytes = g.a_rows * BK * 2, stage_bytes = 2 * a_bytes + bn * BK * 2, stages = ring_stages(g.a_rows, bn);
+    const int tt = g.tt, half = tt / 2, stage_bytes = stage_bytes_of(tt), stages = ring_stages(tt);
     extern __shared__ unsigned char pf_smem_raw[];
-    unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(pf_smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem + stages * stage_bytes);
-    uint64_t *empty = full + MAX_STAGES;
-    uint64_t *acc_full = empty + MAX_STAGES;      // [2]: a chunk's sum is complete in accumulator b
-    uint64_t *acc_empty = acc_full + 2;           // [2]: the epilogue warps have moved accumulator b's sum out
+    unsigned char *turn_smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(pf_smem_raw) + 1023) & ~(uintptr_t)1023);
+    unsigned char *smem = turn_smem + TURN_BYTES;
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem + stages * stage_bytes);      // in use in the first CTA: both CTAs' boxes have landed
+    uint64_t *empty = full + MAX_STAGES;          // in both: the MMAs that read the stage have finished
+    uint64_t *acc_full = empty + MAX_STAGES;      // [2], in both: a chunk's sum is complete in accumulator b
+    uint64_t *acc_empty = acc_full + 2;           // [2], in use in the first CTA: both CTAs' epilogue warps have moved accumulator b's sum out
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + 2);
     volatile int *cta_abort = reinterpret_cast<volatile int *>(tmem_slot + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const Jobs jobs(g);                                              // tiles: row tile fastest (tile = ty * tiles_x + tx)
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31, rank = blockIdx.x & 1;   // rank: of the pair
+    const Jobs jobs(g);                                              // tiles: token tile fastest (tile = ty * tiles_x + tx)
     const int nkb = g.K / BK, nchunks = jobs.nchunks;
     constexpr int EPI_WARPS = GEMM_THREADS / 32 - 2;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < stages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], EPI_WARPS); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 2 * EPI_WARPS); }
         *cta_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(TMEM_COLS) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(TMEM_COLS) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();
+    pair_sync();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    chain_wait();                            // barriers and tensor memory are set up under the end of the kernel before
 
     if (warp == 0) {
-        if (lane == 0) {
-            // ---- TMA producer: a stage is refilled once the MMAs that read it have finished ----
-            int armed = 0, s = 0;            // k-blocks armed so far, over all of this CTA's jobs; the next one's stage and phase
-            uint32_t ph = 0;
-            bool ok = true;
-            for (int i = 0, tile, c_begin, c_end; ok && jobs.get(i, tile, c_begin, c_end); ++i) {
-            const int t0 = (tile % g.tiles_x) * BM, n0 = (tile / g.tiles_x) * per, kb1 = min(nkb, c_end * CHUNK_KB);
-            for (int kb = c_begin * CHUNK_KB; kb < kb1; ++kb) {
-                if (!pf_wait(&empty[s], ph ^ 1u, cta_abort, g.err, 21)) { ok = false; break; }
-                unsigned char *st = smem + s * stage_bytes;
-                stream::mbar_expect_tx(&full[s], stage_bytes);
-                tma_load_2d(st, &ta, kb * BK, t0, &full[s]);
-                tma_load_2d(st + a_bytes, &ta, kb * BK, Tpad + t0, &full[s]);
-                for (int r = 0; r < bn; r += g.box) {        // accumulator column the box starts at
-                    const bool second = EPI == PF_SWIGLU && r >= per;
-                    const CUtensorMap *wm = second ? &tb1 : &tb0;
-                    int wrow = n0 + (second ? r - per : r);
-                    if (EPI != PF_SWIGLU && wrow >= g.nA) {          // stacked matrices: the box lies in the second or third one
-                        wm = &tb1; wrow -= g.nA;
-                        if (wrow >= g.nB) { wm = &tb2; wrow -= g.nB; }
-                    }
-                    tma_load_2d(st + 2 * a_bytes + r * BK * 2, wm, kb * BK, wrow, &full[s]);
+        // ---- TMA producer: a stage is refilled once the MMAs that read it have finished ----
+        const uint32_t one = elect_one(), arms = rank == 0 ? one : 0u;
+        const uint32_t ring = smem_u32(smem), full_here = smem_u32(full), full_first = first_cta_addr(full);
+        const int n_box = 128 / (EPI == PF_SWIGLU ? 64 : g.box);
+        uint64_t w_policy, a_policy;
+        // weights that a launch reads once (one token tile) go first when L2 needs room
+        if (g.tiles_x == 1) asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(w_policy));
+        else asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(w_policy));
+        asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(a_policy));
+        // a job's weight rows: the map and the row in it of either box
+        const CUtensorMap *w_map[2];
+        int w_row[2], t0;
+        auto locate = [&](int tile) {
+            const int u0 = first_unit<EPI>(tile / g.tiles_x, rank);
+            t0 = (tile % g.tiles_x) * tt + rank * half;
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                w_map[r] = EPI == PF_SWIGLU && r ? &tb1 : &tb0;
+                w_row[r] = EPI == PF_SWIGLU ? u0 : u0 + 64 * r;
+                if (EPI != PF_SWIGLU && w_row[r] >= g.nA) {          // stacked matrices: the box lies in the second or third one
+                    w_map[r] = &tb1; w_row[r] -= g.nA;
+                    if (w_row[r] >= g.nB) { w_map[r] = &tb2; w_row[r] -= g.nB; }
                 }
-                ++armed;
+            }
+        };
+        auto load_w = [&](int kb, int s) {
+            expect_tx_if(full_here + 8 * s, 2 * stage_bytes, arms);
+            tma_load_pair(ring + s * stage_bytes, w_map[0], kb * BK, w_row[0], full_first + 8 * s, w_policy, one);
+            if (n_box == 2) tma_load_pair(ring + s * stage_bytes + 64 * BK * 2, w_map[1], kb * BK, w_row[1], full_first + 8 * s, w_policy, one);
+        };
+        auto load_a = [&](int kb, int s) {
+            tma_load_pair(ring + s * stage_bytes + W_BYTES, &ta, kb * BK, t0, full_first + 8 * s, a_policy, one);
+            tma_load_pair(ring + s * stage_bytes + W_BYTES + half * BK * 2, &ta, kb * BK, Tpad + t0, full_first + 8 * s, a_policy, one);
+        };
+        int s = 0, ahead = 0, tile, c_begin, c_end;      // s, ph: the next k-block's stage and phase
+        uint32_t ph = 0;
+        bool ok = true;
+        // the weights are there before the kernel before this one has finished: the first stages' go out at once
+        if (jobs.get(0, tile, c_begin, c_end)) {
+            locate(tile);
+            ahead = min(stages, min(nkb, c_end * CHUNK_KB) - c_begin * CHUNK_KB);
+            for (int k = 0; k < ahead; ++k) load_w(c_begin * CHUNK_KB + k, k);
+            chain_wait();
+            for (int k = 0; k < ahead; ++k) load_a(c_begin * CHUNK_KB + k, k);
+            s = ahead == stages ? 0 : ahead;
+            ph = ahead == stages;
+        }
+        for (int i = 0; ok && jobs.get(i, tile, c_begin, c_end); ++i) {
+            locate(tile);
+            const int kb1 = min(nkb, c_end * CHUNK_KB);
+            for (int kb = c_begin * CHUNK_KB + (i == 0 ? ahead : 0); kb < kb1; ++kb) {
+                ok = __all_sync(0xffffffffu, pf_wait(&empty[s], ph ^ 1u, cta_abort, g.err, 21));
+                if (!ok) break;
+                load_w(kb, s);
+                load_a(kb, s);
                 if (++s == stages) { s = 0; ph ^= 1u; }
             }
-            }
-            if (*cta_abort) {
-                // copies in flight land in this CTA's shared memory: let them finish before the CTA goes away
-                for (int kb = (armed > stages ? armed - stages : 0); kb < armed; ++kb) {
-                    unsigned spins = 0;
-                    while (!mbar_try_wait(&full[kb % stages], (uint32_t)(kb / stages) & 1u) && ++spins < WAIT_LIMIT) {}
-                }
-            }
+        }
+        if (*cta_abort) {
+            // Copies in flight land in this CTA's shared memory, counted by a barrier that the other CTA may not have armed:
+            // they take microseconds, the CTA stays for some milliseconds (and the other one until this one is done).
+            for (int k = 0; k < 5000; ++k) __nanosleep(1000);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        chain_wait();
+        if (rank == 0) {
             // ---- MMA issue: chunk c goes to accumulator c & 1; per stage 4 k-steps of 16 columns, hi and lo term ----
             bool ok = true;
-            const uint32_t idesc = umma_idesc(bn);
-            int cg = 0, s = 0;               // chunks issued so far, over all of this CTA's jobs; stage and phase of the next k-block
+            const uint32_t one = elect_one(), idesc = umma_idesc(PAIR_UNITS, tt);
+            const uint32_t ring = smem_u32(smem), empty_at = smem_u32(empty), acc_full_at = smem_u32(acc_full);
+            int cg = 0, s = 0;               // chunks issued so far, over all of this pair's jobs; stage and phase of the next k-block
             uint32_t ph = 0;
             for (int i = 0, tile, c_begin, c_end; ok && jobs.get(i, tile, c_begin, c_end); ++i)
             for (int c = c_begin; c < c_end && ok; ++c, ++cg) {
                 const int b = cg & 1;
-                ok = pf_wait(&acc_empty[b], ((uint32_t)(cg >> 1) & 1u) ^ 1u, cta_abort, g.err, 24);
+                ok = __all_sync(0xffffffffu, pf_wait<true>(&acc_empty[b], ((uint32_t)(cg >> 1) & 1u) ^ 1u, cta_abort, g.err, 24));
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t acc_addr = tmem + (uint32_t)(b * BN_MAX);
+                const uint32_t acc_addr = tmem + (uint32_t)(b * TT_MAX);
                 const int kb1 = min(nkb, (c + 1) * CHUNK_KB);
-                for (int kb = c * CHUNK_KB; kb < kb1 && ok; ++kb) {
-                    ok = pf_wait(&full[s], ph, cta_abort, g.err, 22);
+                for (int kb = c * CHUNK_KB; kb < kb1; ++kb) {
+                    ok = __all_sync(0xffffffffu, pf_wait<true>(&full[s], ph, cta_abort, g.err, 22));
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t a_hi = smem_u32(smem + s * stage_bytes), a_lo = a_hi + a_bytes, bw = a_hi + 2 * a_bytes;   // fewer rows than a tile's: the rest of its rows is what follows, and meets no live token
+                    const uint32_t w = desc_lower(ring + s * stage_bytes), x_hi = w + (W_BYTES >> 4), x_lo = x_hi + (half * BK * 2 >> 4);
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k) {
-                        const uint32_t accum = (kb != c * CHUNK_KB || k != 0) ? 1u : 0u;
-                        const uint64_t db = umma_desc(bw + 32 * k);
-                        umma_bf16(acc_addr, umma_desc(a_hi + 32 * k), db, idesc, accum);
-                        umma_bf16(acc_addr, umma_desc(a_lo + 32 * k), db, idesc, 1u);
+                        umma_pair<true>(acc_addr, w + 2 * k, x_hi + 2 * k, idesc, kb != c * CHUNK_KB || k != 0, one);
+                        umma_pair<false>(acc_addr, w + 2 * k, x_lo + 2 * k, idesc, 1u, one);
                     }
-                    umma_commit(&empty[s]);
+                    umma_commit_pair(empty_at + 8 * s, one);
                     if (++s == stages) { s = 0; ph ^= 1u; }
                 }
-                umma_commit(&acc_full[b]);     // on the abort path too: it releases the epilogue warps' wait
+                umma_commit_pair(acc_full_at + 8 * b, one);     // on the abort path too: it releases the epilogue warps' wait
             }
-            if (!ok) { umma_commit(&acc_full[0]); umma_commit(&acc_full[1]); }
+            if (!ok) { umma_commit_pair(acc_full_at, one); umma_commit_pair(acc_full_at + 8, one); }
         }
     } else {
-        // ---- epilogue warps: warp w reads lanes 32 (w % 4) .. + 31 of tensor memory = tokens t0 + 32 (w % 4) + lane; the
-        //      two warps of a lane quarter split the tile's columns.  acc[] = this thread's running sums over the chunks:
-        //      store / add: columns [hsel bn / 2, + bn / 2) in groups of 32; SwiGLU: acc[0 .. 63] gate columns
-        //      [hsel bn / 4, + bn / 4), acc[64 .. 127] the up columns of the same units ----
-        const int q = warp & 3, hsel = (warp - 2) >> 2;
+        // ---- epilogue warps: warp w reads lanes 32 (w % 4) .. + 31 of tensor memory = this CTA's weight rows; the two groups of
+        //      four warps split the tile's tokens.  acc[] = this thread's running sums over the chunks, token half * hsel + i ----
+        chain_wait();
+        const int q = warp & 3, hsel = (warp - 2) >> 2, row = 32 * q + lane, gt = (threadIdx.x - 64) & 127;
         const uint32_t trow = tmem + ((uint32_t)(32 * q) << 16);
-        const int half = bn / 2;
-        const bool y32 = (reinterpret_cast<uintptr_t>(g.y) & 31u) == 0;      // ldy, col0 and the columns are multiples of 8
+        float *turn = reinterpret_cast<float *>(turn_smem) + hsel * (2 * TURN_TOKENS * 128);
+        const int f_tok = gt >> 4, f_j = 4 * (gt & 15);      // what this thread finishes: tokens f_tok and f_tok + 8 of 16, rows f_j ..
         bool ok = true;
-        int cg = 0;                          // chunks taken so far, over all of this CTA's tiles
-        const int et = threadIdx.x - 64;     // this thread among the epilogue threads
-        // the sums of piece r's chunk c as this thread's float4s, 256 apart
-        auto part_of = [&](int r, int c) { return reinterpret_cast<float4 *>(g.part + ((size_t)r * nchunks + c) * PIECE_FLOATS) + et; };
-        int tile, c_begin, c_end, i = 0;
-        for (; ok && jobs.get(i, tile, c_begin, c_end); ++i) {
-        const int t = (tile % g.tiles_x) * BM + 32 * q + lane;
-        const bool piece = tile >= g.whole;
-        float acc[128];
+        int cg = 0;                          // chunks taken so far, over all of this pair's jobs
+        int tile, c_begin, c_end;
+        for (int i = 0; jobs.get(i, tile, c_begin, c_end); ++i) {
+            const int t0 = (tile % g.tiles_x) * tt + hsel * half;
+            const bool piece = tile >= g.whole;
+            float acc[128];
 #pragma unroll
-        for (int i = 0; i < 128; ++i) acc[i] = 0.f;
-        for (int c = c_begin; c < c_end && ok; ++c, ++cg) {
-            const int b = cg & 1;
-            // the loads from tensor memory are warp-wide: the warp goes on only if all of its threads saw the accumulator
-            ok = __all_sync(0xffffffffu, pf_wait(&acc_full[b], (uint32_t)(cg >> 1) & 1u, cta_abort, g.err, 23) && !*cta_abort);
-            if (!ok) break;
-            tc_fence_after();
+            for (int e = 0; e < 128; ++e) acc[e] = 0.f;
+            for (int c = c_begin; c < c_end && ok; ++c, ++cg) {
+                const int b = cg & 1;
+                // the loads from tensor memory are warp-wide: the warp goes on only if all of its threads saw the accumulator
+                ok = __all_sync(0xffffffffu, pf_wait(&acc_full[b], (uint32_t)(cg >> 1) & 1u, cta_abort, g.err, 23) && !*cta_abort);
+                if (!ok) break;
+                tc_fence_after();
+                // the last group of 32 columns may reach into the other half's (or past them, inside the accumulators)
 #pragma unroll
-            for (int gi = 0; gi < 4; ++gi) {
-                const int col = group_col<EPI>(gi, hsel, bn);
-                if (col >= 0) {                          // warp-uniform
+                for (int gi = 0; gi < 4; ++gi) {
+                    if (32 * gi >= half) continue;
                     float v[32];
-                    tmem_ld32(trow + (uint32_t)(b * BN_MAX + col), v);
-                    if (piece) {                         // warp-uniform
-                        if (t < g.T) {
-                            float4 *dst = part_of(tile - g.whole, c) + 8 * gi * 256;
+                    tmem_ld32(trow + (uint32_t)(b * TT_MAX + hsel * half + 32 * gi), v);
+                    if (piece) {                             // warp-uniform
+                        float *dst = g.part + (((size_t)(tile - g.whole) * nchunks + c) * 2 + rank) * (tt * 128) + (size_t)(hsel * half + 32 * gi) * 128 + row;
+                        const int live = min(half, g.T - t0) - 32 * gi;
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) __stcg(dst + i * 256, make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
-                        }
+                        for (int e = 0; e < 32; ++e)
+                            if (e < live) __stcg(dst + e * 128, v[e]);
                     } else {
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) acc[32 * gi + i] += v[i];
+                        for (int e = 0; e < 32; ++e) acc[32 * gi + e] += v[e];
                     }
                 }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) pair_arrive(first_cta_addr(&acc_empty[b]));
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) stream::mbar_arrive(&acc_empty[b]);
-        }
-        if (!ok) break;
-        if (piece) continue;                 // fold_pieces_kernel goes on from here
-        if (t < g.T && (EPI == PF_STORE || EPI == PF_ADD)) {
-            // columns: 32 at a time, in 32-byte accesses (a sector each), the old values of a group fetched together
-            const float rs = g.row_scale ? g.row_scale[t] : 1.0f;
-#pragma unroll
-            for (int gi = 0; gi < 4; ++gi) {
-                const int n = (tile / g.tiles_x) * per + hsel * half + 32 * gi;
-                if (32 * gi >= half || n >= g.N) continue;
-                float *yp = g.y + (size_t)t * g.ldy + g.col0 + n;
-                const int live = min(4, (g.N - n) >> 3);         // N is a multiple of 8
-                float x[4][8];
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    if (EPI == PF_ADD && e < live) ld_sector(yp + 8 * e, x[e], y32);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    float o[8];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        o[j] = acc[32 * gi + 8 * e + j] * rs;
-                        if (EPI == PF_ADD) o[j] += x[e][j];
-                    }
-                    if (e < live) st_sector(yp + 8 * e, o, y32);
-                }
-            }
-        } else if (t < g.T) {
+            // a group's four warps go on together or not at all: they meet in what follows
+            asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.cta.red.and.pred q, %2, 128, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                         : "=r"(c_begin) : "r"((uint32_t)ok), "r"(1 + hsel) : "memory");
+            ok = c_begin != 0;
+            if (!ok) break;
+            if (piece) continue;             // fold_pieces_kernel goes on from here
+            const int u0 = first_unit<EPI>(tile / g.tiles_x, rank);
+            float4 x[2][2];
+            old_values<EPI>(g, u0, f_tok < half ? t0 + f_tok : g.T, f_j, x[0]);
+            old_values<EPI>(g, u0, f_tok + 8 < half ? t0 + f_tok + 8 : g.T, f_j, x[1]);
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
-                float v[16];
+                const int i0 = TURN_TOKENS * k;
+                if (i0 >= half) break;       // uniform
+                float *buf = turn + (k & 1) * (TURN_TOKENS * 128);
 #pragma unroll
-                for (int e = 0; e < 8; ++e) { v[e] = acc[8 * k + e]; v[8 + e] = acc[64 + 8 * k + e]; }
-                finish_sums<EPI>(g, tile, t, hsel, 8 * k, y32, v);
+                for (int e = 0; e < TURN_TOKENS; ++e) buf[e * 128 + row] = acc[i0 + e];
+                asm volatile("barrier.cta.sync %0, 128;" ::"r"(1 + hsel) : "memory");
+                float4 next[2][2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int it = i0 + TURN_TOKENS + f_tok + 8 * e;
+                    old_values<EPI>(g, u0, it < half ? t0 + it : g.T, f_j, next[e]);
+                }
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int tok = f_tok + 8 * e, t = t0 + i0 + tok;
+                    if (i0 + tok < half && t < g.T) {
+                        const float4 lo = *reinterpret_cast<const float4 *>(buf + tok * 128 + f_j), hi = *reinterpret_cast<const float4 *>(buf + tok * 128 + 64 + f_j);
+                        float v[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+                        finish_sums<EPI>(g, u0, t, f_j, v, x[e]);
+                    }
+                    x[e][0] = next[e][0];
+                    x[e][1] = next[e][1];
+                }
             }
-        }
         }                                    // next job: its first chunks are already accumulating in tensor memory
     }
     tc_fence_before();
+    __syncwarp();
     __syncthreads();
+    pair_sync();                             // neither CTA's barriers and tensor memory go away before the other is done with them
     if (warp == 1) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
     }
 }
 
 // The tiles of a launch that were done in pieces: adds up the chunk sums of each, first chunk to last, and finishes them as
-// gemm_split_kernel finishes a tile done whole.  grid = 8 (tiles - whole), 256 threads: block 8 r + k has registers 8 k ..
-// and 64 + 8 k .. of piece r's epilogue threads.  Bound by reading the sums back from L2, which all SMs share here; taken by the
-// contraction's own CTAs, each waiting for its tile's last, a prompt of 77 rows (8 layers, 7B widths) took 1.62 ms, so 1.51.
+// gemm_split_kernel finishes a tile done whole.  grid = (2 ceil(tt / 16), tiles - whole), 256 threads: block x has 16 tokens of one CTA's
+// 128 weight rows, a thread four rows and the four 64 further on of one token.  Bound by reading the sums back from L2, which
+// all SMs share here.
 template <int EPI>
 __global__ void __launch_bounds__(256) fold_pieces_kernel(const GemmArgs g) {
     chain_wait();
-    const int r = blockIdx.x >> 3, k = blockIdx.x & 7, tile = g.whole + r, warp = threadIdx.x >> 5;
-    const int hsel = warp >> 2, t = (tile % g.tiles_x) * BM + 32 * ((warp + 2) & 3) + (threadIdx.x & 31);
-    // not all registers are in use in tiles of fewer columns
-    const bool one = group_col<EPI>(k >> 2, hsel, g.bn) >= 0, two = group_col<EPI>(2 + (k >> 2), hsel, g.bn) >= 0;
-    if (!one || t >= g.T) return;
+    const int r = blockIdx.y, tile = g.whole + r, rank = blockIdx.x & 1, tok = 16 * (blockIdx.x >> 1) + (threadIdx.x >> 4), j = 4 * (threadIdx.x & 15);
+    const int t = (tile % g.tiles_x) * g.tt + tok, u0 = first_unit<EPI>(tile / g.tiles_x, rank);
+    if (t >= g.T || u0 >= g.N) return;
     const int nchunks = (g.K / BK + CHUNK_KB - 1) / CHUNK_KB;
-    const float4 *src = reinterpret_cast<const float4 *>(g.part + (size_t)r * nchunks * PIECE_FLOATS) + 2 * k * 256 + threadIdx.x;
-    float v[16];
+    const size_t stride = (size_t)2 * g.tt * (128 / 4);      // between chunks, in float4s
+    const float4 *src = reinterpret_cast<const float4 *>(g.part + (((size_t)r * nchunks * 2 + rank) * g.tt + tok) * 128 + j);
+    float4 x[2];
+    old_values<EPI>(g, u0, t, j, x);
+    float v[8];
 #pragma unroll
-    for (int e = 0; e < 16; ++e) v[e] = 0.f;
-    constexpr int B = 8;                                     // chunks in flight: 16 KB a warp
+    for (int e = 0; e < 8; ++e) v[e] = 0.f;
+    constexpr int B = 8;                                     // chunks in flight: 8 KB a warp
     for (int c0 = 0; c0 < nchunks; c0 += B) {
-        float4 x[B][4];
+        float4 p[B][2];
 #pragma unroll
         for (int c = 0; c < B; ++c)
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-                if (c0 + c < nchunks && (e < 2 || two)) x[c][e] = __ldcg(src + (size_t)(c0 + c) * (PIECE_FLOATS / 4) + ((e & 1) + 16 * (e >> 1)) * 256);
+            for (int e = 0; e < 2; ++e)
+                if (c0 + c < nchunks) p[c][e] = __ldcg(src + (size_t)(c0 + c) * stride + 16 * e);
 #pragma unroll
         for (int c = 0; c < B; ++c)
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-                if (c0 + c < nchunks && (e < 2 || two)) {
-                    v[4 * e] += x[c][e].x; v[4 * e + 1] += x[c][e].y; v[4 * e + 2] += x[c][e].z; v[4 * e + 3] += x[c][e].w;
-                }
+            for (int e = 0; e < 2; ++e)
+                if (c0 + c < nchunks) { v[4 * e] += p[c][e].x; v[4 * e + 1] += p[c][e].y; v[4 * e + 2] += p[c][e].z; v[4 * e + 3] += p[c][e].w; }
     }
-    finish_sums<EPI>(g, tile, t, hsel, 8 * k, (reinterpret_cast<uintptr_t>(g.y) & 31u) == 0, v);
+    finish_sums<EPI>(g, u0, t, j, v, x);
 }
 
 // ---------------------------------------------------------------------------------------------
