@@ -102,16 +102,18 @@ inline Deal deal_out(int T, int N, int K, bool swiglu, int n_sms) {
 // Whether a stacked q / k / v launch finishes the heads in its epilogue (a CTA's 128 weight rows are one head).
 inline bool heads_in_epilogue(int head_dim, int nA, int nB, int N) { return head_dim == 128 && nA % 128 == 0 && nB % 128 == 0 && N % 128 == 0; }
 
-// Most floats of chunk sums that any launch of a prompt pass over up to `cap` rows leaves: what its scratch has to hold.
+// At least the floats of chunk sums that any launch of a prompt pass over up to `cap` rows leaves: what its scratch has to hold.  (Going
+// through deal_out for every row count took a session's first call 25 ms.)
 inline size_t most_sums(int cap, int d, int nq, int nkv, int d_ff, int n_sms) {
+    const int units[] = {nq + 2 * nkv, d, 2 * d_ff, d}, width[] = {d, nq, d, d_ff};      // gate and up rows share a tile
     size_t most = 0;
-    for (int T = 1; T <= cap; ++T) {
-        const size_t sums[] = {deal_out(T, nq + 2 * nkv, d, false, n_sms).sums, deal_out(T, d, nq, false, n_sms).sums,
-                               deal_out(T, d_ff, d, true, n_sms).sums, deal_out(T, d, d_ff, false, n_sms).sums};
-        for (size_t n : sums)
-            if (n > most) most = n;
-    }
-    return most;
+    for (int i = 0; i < 4; ++i)
+        for (int tt = TT_STEP; tt <= TT_MAX && tt < cap + TT_STEP; tt += TT_STEP) {
+            const size_t tiles = (size_t)((cap + tt - 1) / tt) * ((units[i] + PAIR_UNITS - 1) / PAIR_UNITS), pairs = n_sms / 2;
+            const size_t sums = (tiles < pairs ? tiles : pairs - 1) * ((width[i] / BK + CHUNK_KB - 1) / CHUNK_KB) * PAIR_UNITS * tt;
+            if (sums > most) most = sums;
+        }
+    return most < MAX_SUMS ? most : MAX_SUMS;
 }
 
 // What the q / k / v launch needs to finish the heads in its epilogue (rotary embedding, K / V rows into the cache).
