@@ -552,40 +552,47 @@ __global__ void accept_kernel(int *__restrict__ chain, const int *__restrict__ t
 // Cosine top-1 over the anchors
 // ---------------------------------------------------------------------------------------------
 
-// Eq. (4) in one launch: a warp per anchor, dot(v, a) / (|v| |a|) with the anchor's reciprocal norm given or, inv_norm ==
-// nullptr, computed here; then the block that finishes last takes the arg-max of all n, lowest index on ties.  cosines[n] and
-// work[2] (blocks done, a zero or non-finite norm was met) are scratch; work is zero between launches.  out[0] = best flat
-// index, out[1] = its cosine's bits, out[2] = the flag; it may be pinned host memory.  Bound by latencies: 9 us at 50 x 5120,
-// as the two launches before it, but one launch, a memset and two copies less make 28 us of a call of 40.
-// grid = ceil(n / 8), 256 threads.
-__global__ void __launch_bounds__(256) cosine_top1_kernel(const float *__restrict__ v, const float *__restrict__ anchors,
-                                                          const float *__restrict__ inv_norm, int n, int d, float *__restrict__ cosines,
-                                                          int *__restrict__ work, int *__restrict__ out) {
+// Eq. (4) in one launch: dot(v, a) / (|v| |a|) by a block per anchor; then the block that finishes last takes the arg-max of all
+// n, lowest index on ties.  cosines[n] and work[2] (blocks done, a zero or non-finite norm was met) are scratch; work is zero
+// between launches.  out[0] = best flat index, out[1] = its cosine's bits, out[2] = the flag; it may be pinned host memory.
+// Bound by latencies: 16 bytes a load where query and rows allow it, 50 x 5120: 5 us (a warp per anchor, 4 bytes a load: 10).
+// grid = n, 256 threads.
+__global__ void __launch_bounds__(256) cosine_top1_kernel(const float *__restrict__ v, const float *__restrict__ anchors, int n, int d,
+                                                          float *__restrict__ cosines, int *__restrict__ work, int *__restrict__ out) {
     __shared__ float s_v[8];
     __shared__ int s_i[8];
+    __shared__ float s_sum[3][8];
     __shared__ int s_last;
-    const int tid = threadIdx.x, lane = tid & 31, a = blockIdx.x * 8 + (tid >> 5);
-    if (a < n) {
-        const float *ar = anchors + (size_t)a * d;
-        float dot = 0.f, vv = 0.f, aa = 0.f;
-#pragma unroll 16
-        for (int i = lane; i < d; i += 32) {
-            const float x = v[i], y = ar[i];
-            dot = fmaf(x, y, dot);
-            vv = fmaf(x, x, vv);
-            aa = fmaf(y, y, aa);
+    const int tid = threadIdx.x, a = blockIdx.x;
+    const float *ar = anchors + (size_t)a * d;
+    float dot = 0.f, vv = 0.f, aa = 0.f;
+    auto take = [&](float x, float y) {
+        dot = fmaf(x, y, dot);
+        vv = fmaf(x, x, vv);
+        aa = fmaf(y, y, aa);
+    };
+    if (((reinterpret_cast<uintptr_t>(v) | reinterpret_cast<uintptr_t>(anchors)) & 15u) == 0 && d % 4 == 0) {
+#pragma unroll 5
+        for (int i = tid; i < d / 4; i += 256) {
+            const float4 x = reinterpret_cast<const float4 *>(v)[i], y = reinterpret_cast<const float4 *>(ar)[i];
+            take(x.x, y.x); take(x.y, y.y); take(x.z, y.z); take(x.w, y.w);
         }
-        dot = warp_sum(dot); vv = warp_sum(vv); aa = warp_sum(aa);
-        if (lane == 0) {
-            const bool bad = !(vv > 0.f) || !isfinite(vv) || !(aa > 0.f) || !isfinite(aa);
-            const float ia = inv_norm ? inv_norm[a] : 1.0f / sqrtf(aa);
-            __stcg(cosines + a, bad ? -INFINITY : dot * (1.0f / sqrtf(vv)) * ia);
-            if (bad) atomicExch(work + 1, 1);
-        }
+    } else {
+#pragma unroll 4
+        for (int i = tid; i < d; i += 256) take(v[i], ar[i]);
     }
-    __threadfence();
+    dot = warp_sum(dot); vv = warp_sum(vv); aa = warp_sum(aa);
+    if ((tid & 31) == 0) { s_sum[0][tid >> 5] = dot; s_sum[1][tid >> 5] = vv; s_sum[2][tid >> 5] = aa; }
     __syncthreads();
-    if (tid == 0) s_last = atomicAdd(work, 1) == (int)gridDim.x - 1;
+    if (tid == 0) {
+#pragma unroll
+        for (int w = 1; w < 8; ++w) { dot += s_sum[0][w]; vv += s_sum[1][w]; aa += s_sum[2][w]; }
+        const bool bad = !(vv > 0.f) || !isfinite(vv) || !(aa > 0.f) || !isfinite(aa);
+        __stcg(cosines + a, bad ? -INFINITY : (float)((double)dot / sqrt((double)vv * (double)aa)));      // one rounding
+        if (bad) atomicExch(work + 1, 1);
+        __threadfence();
+        s_last = atomicAdd(work, 1) == (int)gridDim.x - 1;
+    }
     __syncthreads();
     if (!s_last) return;
     __threadfence();
@@ -610,17 +617,14 @@ __global__ void __launch_bounds__(256) cosine_top1_kernel(const float *__restric
     }
 }
 
-__global__ void anchor_inv_norm_kernel(const float *__restrict__ anchors, int n, int d, float *__restrict__ inv_norm,
-                                       int *__restrict__ flag) {
+// flag <- 1 if an anchor's norm is zero or not finite.
+__global__ void anchor_norm_check_kernel(const float *__restrict__ anchors, int n, int d, int *__restrict__ flag) {
     const int lane = threadIdx.x & 31, a = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (a >= n) return;
     float aa = 0.f;
     for (int i = lane; i < d; i += 32) { const float y = anchors[(size_t)a * d + i]; aa = fmaf(y, y, aa); }
     aa = warp_sum(aa);
-    if (lane == 0) {
-        if (!(aa > 0.f) || !isfinite(aa)) { *flag = 1; inv_norm[a] = 0.f; }
-        else inv_norm[a] = 1.0f / sqrtf(aa);
-    }
+    if (lane == 0 && (!(aa > 0.f) || !isfinite(aa))) *flag = 1;
 }
 
 // One word of the session's state, in stream order.

@@ -48,7 +48,7 @@ struct knnssd_ctx {
     // device buffers (owned)
     void *kcache = nullptr, *vcache = nullptr;
     float *x = nullptr, *qkv = nullptr, *attn = nullptr, *act = nullptr, *logits = nullptr, *hfinal = nullptr;
-    float *part_o = nullptr, *pooled = nullptr, *anchor_inv_norm = nullptr, *cosines = nullptr, *amax_v = nullptr;
+    float *part_o = nullptr, *pooled = nullptr, *cosines = nullptr, *amax_v = nullptr;
     float2 *part_ml = nullptr, *rope_cs = nullptr;
     double *pool_sum = nullptr, *inv_freq = nullptr;
     int *chain = nullptr, *target = nullptr, *prompt = nullptr, *out_tokens = nullptr, *accept_log = nullptr;
@@ -601,7 +601,7 @@ knnssd_status check_stream_err(knnssd_ctx *c, const char *what) {
 
 void free_all(knnssd_ctx *c) {
     void *ptrs[] = {c->kcache, c->vcache, c->x, c->qkv, c->attn, c->act, c->logits, c->hfinal, c->part_o, c->pooled,
-                    c->anchor_inv_norm, c->cosines, c->amax_v, c->part_ml, c->rope_cs, c->pool_sum, c->inv_freq, c->chain,
+                    c->cosines, c->amax_v, c->part_ml, c->rope_cs, c->pool_sum, c->inv_freq, c->chain,
                     c->target, c->prompt, c->out_tokens, c->accept_log, c->amax_i, c->flag, c->knn_work, c->err_word, c->state,
                     c->ops_full, c->ops_draft, c->bar, c->gabort, c->attn_cnt, c->amax_cnt, c->mpart_o, c->mamax_v, c->mpart_ml,
                     c->mamax_i, c->trace, c->xs_x, c->xs_attn, c->xs_act, c->ssp, c->pf_x, c->pf_qkv, c->pf_ad, c->pf_aq, c->pf_af, c->pf_cs, c->pf_rinv, c->pf_part,
@@ -761,7 +761,7 @@ knnssd_status do_select(knnssd_ctx *c, const float *query_dev, int *domain, int 
     const int n = g.n_domains * g.anchors_per_domain;
     cudaStream_t s = c->stream;
     cudaEventRecord(c->ev0, s);
-    cosine_top1_kernel<<<(n + 7) / 8, 256, 0, s>>>(query_dev ? query_dev : c->pooled, c->anchors, c->anchor_inv_norm, n, g.d_model, c->cosines,
+    cosine_top1_kernel<<<n, 256, 0, s>>>(query_dev ? query_dev : c->pooled, c->anchors, n, g.d_model, c->cosines,
                                                    c->knn_work, c->pinned);
     CUDA_TRY(c, cudaGetLastError());
     cudaEventRecord(c->ev1, s);
@@ -874,7 +874,6 @@ knnssd_status knnssd_init(const knnssd_config *cfg, const knnssd_weights *w, con
     ok &= dev_alloc(&c->err_word, 1) == cudaSuccess;
     ok &= dev_alloc(&c->state, 1) == cudaSuccess;
     ok &= dev_alloc(&c->cosines, (size_t)(na > 0 ? na : 1)) == cudaSuccess;
-    ok &= dev_alloc(&c->anchor_inv_norm, (size_t)(na > 0 ? na : 1)) == cudaSuccess;
     ok &= cudaMallocHost(reinterpret_cast<void **>(&c->pinned), 64 * sizeof(int)) == cudaSuccess;
     ok &= cudaEventCreate(&c->ev0) == cudaSuccess && cudaEventCreate(&c->ev1) == cudaSuccess &&
           cudaEventCreate(&c->ev2) == cudaSuccess;
@@ -892,7 +891,7 @@ knnssd_status knnssd_init(const knnssd_config *cfg, const knnssd_weights *w, con
     // token buffers start at a valid id, so that a pass that ends early never leaves garbage ids behind
     cudaMemsetAsync(c->chain, 0, sizeof(int) * (kMaxRows + 1), c->stream);
     cudaMemsetAsync(c->target, 0, sizeof(int) * kMaxRows, c->stream);
-    if (na > 0) anchor_inv_norm_kernel<<<(na + 7) / 8, 256, 0, c->stream>>>(c->anchors, na, d, c->anchor_inv_norm, c->flag);
+    if (na > 0) anchor_norm_check_kernel<<<(na + 7) / 8, 256, 0, c->stream>>>(c->anchors, na, d, c->flag);
     cudaMemcpyAsync(c->pinned, c->flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
     if (sync_check(c, "init") != KNNSSD_OK) return bail(KNNSSD_ERR_CUDA);
     if (c->pinned[0]) return bail(KNNSSD_ERR_DEGENERATE);
@@ -1714,7 +1713,7 @@ knnssd_status knnssd_cosine_top1(const float *query_dev, const float *anchors_de
     Scratch scratch(s);
     if (!host || !scratch.get(&cos_dev, (size_t)n) || !scratch.get(&work, 2)) return KNNSSD_ERR_CUDA;
     cudaMemsetAsync(work, 0, sizeof(int) * 2, s);
-    cosine_top1_kernel<<<(n + 7) / 8, 256, 0, s>>>(query_dev, anchors_dev, nullptr, n, d, cos_dev, work, host);
+    cosine_top1_kernel<<<n, 256, 0, s>>>(query_dev, anchors_dev, n, d, cos_dev, work, host);
     cudaError_t e = cudaStreamSynchronize(s);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return KNNSSD_ERR_CUDA;
@@ -1765,7 +1764,7 @@ extern "C" knnssd_status knnssd_cosine_top1_static(const float *query_dev, const
     int *small = reinterpret_cast<int *>(scratch + KNNSSD_STATIC_MAX_ANCHORS);   // [0..2] result and flag, [4..5] the kernel's counters
     // the array still holds what the previous call left: the words that must start at zero are cleared here
     if (cudaMemsetAsync(small, 0, sizeof(int) * 6, s) != cudaSuccess) return KNNSSD_ERR_CUDA;
-    cosine_top1_kernel<<<(n + 7) / 8, 256, 0, s>>>(query_dev, anchors_dev, nullptr, n, d, cos_dev, small + 4, small);
+    cosine_top1_kernel<<<n, 256, 0, s>>>(query_dev, anchors_dev, n, d, cos_dev, small + 4, small);
     int host[4] = {0, 0, 0, 0};
     cudaError_t e = cudaMemcpyAsync(host, small, sizeof(int) * 4, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
