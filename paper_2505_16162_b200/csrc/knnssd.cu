@@ -9,6 +9,7 @@
 #include "anchors.cuh"
 #include "linear_tc.cuh"
 #include "sampling.cuh"
+#include "small_pass.cuh"
 
 #include <cmath>
 #include <cstdio>
@@ -84,6 +85,11 @@ struct knnssd_ctx {
     uint32_t *xs_x = nullptr, *xs_attn = nullptr, *xs_act = nullptr;   // pre-split activations (see LinPhase::xs)
     float *ssp = nullptr;                                              // [MAXM][n_sms] partial sums of squares of x rows
 
+    // small models that the pass kernel does not take: a pass in one launch (small_pass.cuh)
+    bool small_ok = false;
+    small::LayerW *small_layers = nullptr;
+    unsigned *small_bar = nullptr;                           // [2]: the meetings of every second launch
+    int small_turn = 0;
     // tensor-core prompt pass (same eligibility as the pass kernel): activations of up to pf_cap rows
     bool pf_ok = false;
     int pf_cap = 0;                                          // rows per chunk, a multiple of 128
@@ -463,6 +469,7 @@ void run_pass_mega(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const 
 // After a pass kernel gave up: bring the barrier counter and the work counters back to their idle state.  On the session's stream:
 // it need not be one that waits for the legacy stream, and the next pass would run into a cudaMemset on its way.
 void reset_mega_state(knnssd_ctx *c) {
+    if (c->small_ok) cudaMemsetAsync(c->small_bar, 0, 2 * sizeof(unsigned), c->stream);       // either turn may go on from here
     if (!c->mega_ok) return;
     cudaMemsetAsync(c->bar, 0, sizeof(unsigned long long), c->stream);
     cudaMemsetAsync(c->gabort, 0, sizeof(int), c->stream);
@@ -534,9 +541,49 @@ void run_pass_t(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const uns
     }
 }
 
+// A model's pass is one launch of small_pass_kernel where a layer's weights are at most this much.  A kernel per operation has eight
+// times the warps on an SM to fetch them with, which is worth more than the launches from some 100 MB on.  Verification calls of 1 / 5
+// / 16 rows on four layers, one launch against a kernel per operation, us: fp32 3 MB a layer 113 / 136 / 180 against 176 / 246 / 420;
+// 48 MB 208 / 273 / 497 against 277 / 432 / 828; bf16 59 MB 331 / 419 / 935 against 326 / 586 / 1412, 190 MB 691 / 987 / 2141 against 503 / 1032 / 2700.
+constexpr size_t kSmallLayerBytes = (size_t)48 << 20;
+
+template <typename WT, int MT> cudaError_t launch_small_t(const small::Args &a, int grid, cudaStream_t s) {
+    void *args[] = {const_cast<small::Args *>(&a)};
+    return cudaLaunchCooperativeKernel(reinterpret_cast<void *>(small::small_pass_kernel<WT, MT>), dim3(grid), dim3(small::NT), args, 0, s);
+}
+template <typename WT> cudaError_t launch_small(const small::Args &a, int grid, cudaStream_t s) {
+    if (a.M <= 1) return launch_small_t<WT, 1>(a, grid, s);
+    if (a.M <= 3) return launch_small_t<WT, 3>(a, grid, s);
+    if (a.M <= 5) return launch_small_t<WT, 5>(a, grid, s);
+    if (a.M <= 9) return launch_small_t<WT, 9>(a, grid, s);
+    return launch_small_t<WT, kMaxRows>(a, grid, s);
+}
+
+// One pass of a small model.  Errors surface at the caller's next synchronisation.
+void run_pass_small(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const unsigned char *mask, int head_row0, int *argmax_out, bool want_hidden) {
+    const knnssd_config &g = c->cfg;
+    small::Args a{};
+    a.layers = c->small_layers; a.tok_embed = c->tok_embed; a.lm_head = c->lm_head; a.final_norm = c->final_norm;
+    a.n_layers = g.n_layers; a.d = g.d_model; a.H = g.n_heads; a.Hkv = g.n_kv_heads; a.hd = g.head_dim; a.F = g.d_ff; a.V = g.vocab; a.max_seq = g.max_seq;
+    a.eps = g.rms_eps; a.st = c->state; a.tok = tok_dev; a.M = M; a.pos_off = pos_off; a.head_row0 = head_row0; a.want_hidden = want_hidden ? 1 : 0;
+    a.argmax_out = argmax_out; a.inv_freq = c->inv_freq; a.x = c->x; a.qkv = c->qkv; a.attn = c->attn; a.act = c->act; a.logits = c->logits;
+    a.hfinal = c->hfinal; a.part_o = c->part_o; a.part_ml = c->part_ml; a.rope_cs = c->rope_cs; a.n_splits = c->n_splits; a.kc = c->kcache; a.vc = c->vcache;
+    a.bar = c->small_bar + c->small_turn; a.next_bar = c->small_bar + (c->small_turn ^ 1); a.err = c->err_word;
+    for (int j = 0; mask && j < 2 * g.n_layers; ++j)
+        if (mask[j]) a.skip[j >> 5] |= 1u << (j & 31);
+    // a warp per item of the widest map, as far as there are SMs
+    int items = (g.n_heads + 2 * g.n_kv_heads) * (g.head_dim / 2);
+    if (g.d_ff > items) items = g.d_ff;
+    if (head_row0 < M && (g.vocab + 1) / 2 > items) items = (g.vocab + 1) / 2;
+    const int blocks = (items + small::NW - 1) / small::NW, grid = blocks < c->n_sms ? blocks : c->n_sms;
+    if ((g.dtype ? launch_small<bf16_t>(a, grid, c->stream) : launch_small<float>(a, grid, c->stream)) == cudaSuccess) c->small_turn ^= 1;
+    c->launches++;
+}
+
 void run_pass(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const unsigned char *mask, int head_row0,
               int *argmax_out, bool want_hidden) {
     if (c->mega_ok && M <= pass::MAXM) { run_pass_mega(c, M, tok_dev, pos_off, mask, head_row0, argmax_out, want_hidden); return; }
+    if (c->small_ok) { run_pass_small(c, M, tok_dev, pos_off, mask, head_row0, argmax_out, want_hidden); return; }
     if (c->cfg.dtype) run_pass_t<bf16_t>(c, M, tok_dev, pos_off, mask, head_row0, argmax_out, want_hidden);
     else run_pass_t<float>(c, M, tok_dev, pos_off, mask, head_row0, argmax_out, want_hidden);
 }
@@ -604,7 +651,7 @@ void free_all(knnssd_ctx *c) {
                     c->cosines, c->amax_v, c->part_ml, c->rope_cs, c->pool_sum, c->inv_freq, c->chain,
                     c->target, c->prompt, c->out_tokens, c->accept_log, c->amax_i, c->flag, c->knn_work, c->err_word, c->state,
                     c->ops_full, c->ops_draft, c->bar, c->gabort, c->attn_cnt, c->amax_cnt, c->mpart_o, c->mamax_v, c->mpart_ml,
-                    c->mamax_i, c->trace, c->xs_x, c->xs_attn, c->xs_act, c->ssp, c->pf_x, c->pf_qkv, c->pf_ad, c->pf_aq, c->pf_af, c->pf_cs, c->pf_rinv, c->pf_part,
+                    c->mamax_i, c->trace, c->xs_x, c->xs_attn, c->xs_act, c->ssp, c->pf_x, c->pf_qkv, c->pf_ad, c->pf_aq, c->pf_af, c->pf_cs, c->pf_rinv, c->pf_part, c->small_layers, c->small_bar,
                     c->samp_p, c->samp_q, c->samp_res};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -954,6 +1001,17 @@ knnssd_status knnssd_init(const knnssd_config *cfg, const knnssd_weights *w, con
         const std::vector<pass::Op> ops = build_ops(c, nullptr, &c->bar_full, &c->attn_full);
         c->n_ops_full = (int)ops.size();
         if (upload_ops(c, ops, c->ops_full) != KNNSSD_OK) return bail(KNNSSD_ERR_CUDA);
+    }
+    // small models that the pass kernel does not take
+    const size_t layer_bytes = c->wbytes * ((size_t)2 * d * (nq + nkv) + (size_t)3 * d * g.d_ff);
+    if (!c->mega_ok && coop && 2 * g.n_layers <= 32 * small::MASK_WORDS && layer_bytes <= kSmallLayerBytes) {
+        std::vector<small::LayerW> ls;
+        for (const Layer &ly : c->layers) ls.push_back({ly.wq, ly.wk, ly.wv, ly.wo, ly.w_gate, ly.w_up, ly.w_down, ly.attn_norm, ly.mlp_norm});
+        if (dev_alloc(&c->small_layers, ls.size()) != cudaSuccess || dev_alloc(&c->small_bar, 2) != cudaSuccess) { cudaGetLastError(); return bail(KNNSSD_ERR_CUDA); }
+        cudaMemcpyAsync(c->small_layers, ls.data(), ls.size() * sizeof(small::LayerW), cudaMemcpyHostToDevice, c->stream);
+        cudaMemsetAsync(c->small_bar, 0, 2 * sizeof(unsigned), c->stream);
+        c->small_ok = true;
+        if (sync_check(c, "init") != KNNSSD_OK) return bail(KNNSSD_ERR_CUDA);
     }
     *out = c;
     return KNNSSD_OK;

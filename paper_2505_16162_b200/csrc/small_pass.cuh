@@ -1,0 +1,376 @@
+// A decoder pass of a small model in one launch (sm_100a).
+//
+// Models that the streaming pass kernel does not take (fp32 weights, widths that are no multiples of 128) run kernel by kernel.
+// Where a layer's weights are a few MB the work of such a kernel is a microsecond and what it costs is the way from one to
+// the next: 7 launches a layer, ~4.3 us each.  Here the pass is one cooperative launch of at most one block per SM that walks the
+// same operations with a grid-wide meeting between dependent ones, five a layer: the rotary embedding and the K / V rows are
+// written by the warps that compute the projections (a warp owns the two units of a rotary pair), and a row whose context is one
+// split leaves its attention output without a merge.  Bound by the meetings and the trips to L2 behind them, 3.8 us from one to the
+// next: fp32 tiny shape (4 layers, d 256), five rows: 170 -> 84 us on the device.
+//
+// Rows are independent of how many the pass carries.  Every wait is bounded: a block that gives up reports to the session's error
+// word and all blocks fall through to the end.
+#pragma once
+
+#include "kernels.cuh"
+
+namespace knnssd {
+namespace small {
+
+constexpr int NT = 256, NW = NT / 32;
+constexpr int MASK_WORDS = 16;                 // sublayers of at most 256 layers
+constexpr unsigned POLL_LIMIT = 4000000u;      // polls of one meeting
+static_assert(NT == ATT_CHUNK, "a thread per position of a split");
+
+struct LayerW {
+    const void *wq, *wk, *wv, *wo, *w_gate, *w_up, *w_down;
+    const float *attn_norm, *mlp_norm;
+};
+struct Args {
+    const LayerW *layers;                      // [n_layers], device
+    const void *tok_embed, *lm_head;
+    const float *final_norm;
+    int n_layers, d, H, Hkv, hd, F, V, max_seq;
+    float eps;
+    const DeviceState *st;
+    const int *tok;                            // [M] device
+    int M, pos_off, head_row0, want_hidden;    // rows from head_row0 on get logits and an arg-max (== M: none)
+    int *argmax_out;
+    const double *inv_freq;
+    float *x, *qkv, *attn, *act, *logits, *hfinal, *part_o;
+    float2 *part_ml, *rope_cs;
+    int n_splits;
+    void *kc, *vc;                             // [layer][kv head][max_seq][hd]
+    unsigned *bar, *next_bar;                  // arrivals of this launch's meetings, zero at its start; the next launch's, zeroed by this one
+    int *err;
+    unsigned skip[MASK_WORDS];                 // bit j: sublayer j is left out
+};
+
+__device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// All blocks have come this far and see one another's writes.  target: arrivals up to and including this meeting.
+__device__ __forceinline__ bool meet_grid(const Args &a, unsigned &target, int *s_abort) {
+    target += gridDim.x;
+    __syncthreads();
+    if (threadIdx.x == 0 && !*s_abort) {
+        __threadfence();                       // cumulative: covers the writes of the block's other threads ordered by the barrier
+        atomicAdd(a.bar, 1u);
+        unsigned polls = 0;
+        while (ld_acquire_u32(a.bar) < target)
+            if (++polls > POLL_LIMIT) { *s_abort = 1; atomicExch(a.err, 8); break; }
+    }
+    __syncthreads();
+    return !*s_abort;
+}
+
+// What the blocks of this launch write is read past the read-only path, from L2.
+__device__ __forceinline__ float4 ld_row4(const float *p) { return __ldcg(reinterpret_cast<const float4 *>(p)); }
+
+// RMSNorm scales of M rows of width d, a warp per row.
+__device__ __forceinline__ void norm_scales(const float *x, int M, int d, float eps, float *s_rinv) {
+    const int lane = threadIdx.x & 31;
+    for (int m = threadIdx.x >> 5; m < M; m += NW) {
+        float s = 0.f;
+#pragma unroll 4
+        for (int i = 4 * lane; i < d; i += 128) {
+            const float4 v = ld_row4(x + (size_t)m * d + i);
+            s = fmaf(v.x, v.x, s); s = fmaf(v.y, v.y, s); s = fmaf(v.z, v.z, s); s = fmaf(v.w, v.w, s);
+        }
+        s = warp_sum(s);
+        if (lane == 0) s_rinv[m] = 1.0f / sqrtf(s / (float)d + eps);
+    }
+    __syncthreads();
+}
+
+// A linear map over M <= MT rows of width K: a warp takes items gw, gw + (warps of the grid), ..; rows(item, w0, w1) names the two
+// weight rows of an item, early(item, m) fetches what row m's end needs, done(item, m, v0, v1, fetched) gets the products with row m,
+// in lane m.  NORM: of the rows times `gain`, scaled by their RMSNorm (every warp reads the rows whole: it sums the squares on the
+// way, where a pass of its own over them took 0.8 us).  The order of a sum depends on K alone.
+template <typename WT, int MT, bool NORM, typename Rows, typename Early, typename Done>
+__device__ __forceinline__ void map_rows(const float *x, int M, int K, const float *gain, float eps, int n_items, Rows rows, Early early, Done done) {
+    const int lane = threadIdx.x & 31;
+    for (int item = blockIdx.x * NW + (threadIdx.x >> 5); item < n_items; item += gridDim.x * NW) {
+        const WT *r0, *r1;
+        rows(item, r0, r1);
+        float2 fetched = make_float2(0.f, 0.f);
+        if (lane < M) fetched = early(item, lane);
+        float acc[2][MT], ss[MT];
+#pragma unroll
+        for (int m = 0; m < MT; ++m) acc[0][m] = acc[1][m] = ss[m] = 0.f;
+        for (int e = 8 * lane; e < K; e += 256) {
+            float w0[8], w1[8];
+            WeightLoad<WT>::load8(r0, e, w0);
+            WeightLoad<WT>::load8(r1, e, w1);
+            if (NORM) {
+                const float4 g0 = __ldg(reinterpret_cast<const float4 *>(gain + e)), g1 = __ldg(reinterpret_cast<const float4 *>(gain + e + 4));
+                const float g[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
+#pragma unroll
+                for (int j = 0; j < 8; ++j) { w0[j] *= g[j]; w1[j] *= g[j]; }
+            }
+#pragma unroll
+            for (int m = 0; m < MT; ++m) {
+                const float *xr = x + (size_t)min(m, M - 1) * K + e;
+                const float4 x0 = ld_row4(xr), x1 = ld_row4(xr + 4);
+                const float xv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    acc[0][m] = fmaf(w0[j], xv[j], acc[0][m]);
+                    acc[1][m] = fmaf(w1[j], xv[j], acc[1][m]);
+                    if (NORM) ss[m] = fmaf(xv[j], xv[j], ss[m]);
+                }
+            }
+        }
+        float v0 = 0.f, v1 = 0.f, sq = 0.f;
+#pragma unroll
+        for (int m = 0; m < MT; ++m) {
+            const float s0 = warp_sum(acc[0][m]), s1 = warp_sum(acc[1][m]), s2 = NORM ? warp_sum(ss[m]) : 0.f;
+            if (lane == m) { v0 = s0; v1 = s1; sq = s2; }
+        }
+        if (NORM) {
+            const float rinv = 1.0f / sqrtf(sq / (float)K + eps);
+            v0 = __fmul_rn(v0, rinv);
+            v1 = __fmul_rn(v1, rinv);
+        }
+        if (lane < M) done(item, lane, v0, v1, fetched);
+    }
+}
+
+// Attention of one (head, row, split of ATT_CHUNK positions) by a block: a thread per position for the scores, then threads by
+// dimension, the positions in NT / hd interleaved runs, whose first PRE values are fetched along with the K rows.  single: the row's
+// context is this split, its output is written at once.
+template <typename WT>
+__device__ __forceinline__ void attend(const Args &a, const WT *kc, const WT *vc, int T, int head, int m, int split, bool single, float *s_p, float *s_red) {
+    const int t0 = split * ATT_CHUNK;
+    if (t0 >= T) return;                                     // uniform over the block
+    constexpr int PRE = 32;
+    const int nt = min(T - t0, ATT_CHUNK), tid = threadIdx.x, hd = a.hd, warp = tid >> 5, lane = tid & 31;
+    const size_t row0 = (size_t)(head / (a.H / a.Hkv)) * a.max_seq + t0;
+    const int runs = NT / hd, e = tid % hd, run = tid / hd;
+    const WT *vr = vc + row0 * hd + e;
+    WT v_pre[PRE];
+#pragma unroll
+    for (int i = 0; i < PRE; ++i) v_pre[i] = run + i * runs < nt ? __ldcg(vr + (size_t)(run + i * runs) * hd) : WT(0);
+    const float *q = a.qkv + (size_t)m * (a.H + 2 * a.Hkv) * hd + (size_t)head * hd;
+    float s = -INFINITY;
+    if (tid < nt) {
+        const WT *kr = kc + (row0 + tid) * hd;
+        float dot = 0.f;
+        if (sizeof(WT) == 4) {
+#pragma unroll 16
+            for (int i = 0; i < hd; i += 4) {
+                const float4 k4 = ld_row4(reinterpret_cast<const float *>(kr) + i), q4 = ld_row4(q + i);
+                dot = fmaf(q4.x, k4.x, dot); dot = fmaf(q4.y, k4.y, dot); dot = fmaf(q4.z, k4.z, dot); dot = fmaf(q4.w, k4.w, dot);
+            }
+        } else {
+#pragma unroll 8
+            for (int i = 0; i < hd; i += 8) {
+                const uint4 k8 = __ldcg(reinterpret_cast<const uint4 *>(kr + i));
+                const float4 qa = ld_row4(q + i), qb = ld_row4(q + i + 4);
+                const uint32_t w[4] = {k8.x, k8.y, k8.z, k8.w};
+                const float qv[8] = {qa.x, qa.y, qa.z, qa.w, qb.x, qb.y, qb.z, qb.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    dot = fmaf(qv[2 * j], __uint_as_float(w[j] << 16), dot);
+                    dot = fmaf(qv[2 * j + 1], __uint_as_float(w[j] & 0xFFFF0000u), dot);
+                }
+            }
+        }
+        s = __fmul_rn(dot, 1.0f / sqrtf((float)hd));
+    }
+    const float wm = warp_max(s);
+    if (lane == 0) s_red[warp] = wm;
+    __syncthreads();
+    float mx = s_red[0];
+#pragma unroll
+    for (int w = 1; w < NW; ++w) mx = fmaxf(mx, s_red[w]);
+    const float p = tid < nt ? expf(s - mx) : 0.f;
+    s_p[tid] = p;
+    const float ws = warp_sum(p);
+    if (lane == 0) s_red[NW + warp] = ws;
+    __syncthreads();
+    float sum = 0.f;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) sum += s_red[NW + w];
+    float o = 0.f;
+#pragma unroll
+    for (int i = 0; i < PRE; ++i)
+        if (run + i * runs < nt) o = fmaf(s_p[run + i * runs], WeightLoad<WT>::load1(v_pre + i), o);
+#pragma unroll 16
+    for (int t = run + PRE * runs; t < nt; t += runs) {
+        const WT v = __ldcg(vr + (size_t)t * hd);
+        o = fmaf(s_p[t], WeightLoad<WT>::load1(&v), o);
+    }
+    __syncthreads();                                         // s_p has been read
+    s_p[tid] = o;
+    __syncthreads();
+    if (tid < hd) {
+        for (int r = 1; r < runs; ++r) o += s_p[r * hd + tid];
+        if (single) {
+            a.attn[(size_t)m * a.H * hd + (size_t)head * hd + tid] = o / sum;
+        } else {
+            const size_t at = ((size_t)m * a.H + head) * a.n_splits + split;
+            a.part_o[at * hd + tid] = o;
+            if (tid == 0) a.part_ml[at] = make_float2(mx, sum);
+        }
+    }
+    __syncthreads();                                         // the next task's
+}
+
+template <typename WT, int MT>
+__global__ void __launch_bounds__(NT, 1) small_pass_kernel(const __grid_constant__ Args a) {
+    __shared__ float s_rinv[MT], s_p[NT], s_red[2 * NW];
+    __shared__ int s_red_i[NW], s_abort;
+    const int tid = threadIdx.x, M = a.M, d = a.d, hd = a.hd, half = hd / 2, slots = a.H + 2 * a.Hkv, nq = a.H * hd;
+    unsigned met = 0;
+    if (tid == 0) {
+        s_abort = 0;
+        if (blockIdx.x == 0) *a.next_bar = 0u;
+    }
+    const int pos0 = a.st->len + a.pos_off;
+
+    // embedding rows, and (from the last block on) the rows' rotary angles, in fp64
+    for (int m = blockIdx.x; m < M; m += gridDim.x) {
+        int t = a.tok[m];
+        if (t < 0 || t >= a.V) {                             // never gather outside the table: report and read row 0 instead
+            if (tid == 0) atomicExch(a.err, ERR_BAD_TOKEN);
+            t = 0;
+        }
+        const WT *row = reinterpret_cast<const WT *>(a.tok_embed) + (size_t)t * d;
+        for (int i = tid; i < d; i += NT) a.x[(size_t)m * d + i] = WeightLoad<WT>::load1(row + i);
+    }
+    for (int m = gridDim.x - 1 - blockIdx.x; m < M; m += gridDim.x)
+        for (int i = tid; i < half; i += NT) {
+            double s, c;
+            sincos((double)(pos0 + m) * a.inv_freq[i], &s, &c);
+            a.rope_cs[m * half + i] = make_float2((float)c, (float)s);
+        }
+    if (!meet_grid(a, met, &s_abort)) return;
+
+    const int n_split = (pos0 + M + ATT_CHUNK - 1) / ATT_CHUNK;      // of the pass's last row
+    auto pair_rows = [&](const void *W, int K, int n, int item, const WT *&r0, const WT *&r1) {      // units 2 item and 2 item + 1 of n
+        r0 = reinterpret_cast<const WT *>(W) + (size_t)(2 * item) * K;
+        r1 = reinterpret_cast<const WT *>(W) + (size_t)min(2 * item + 1, n - 1) * K;
+    };
+    // d is even
+    auto old_pair = [&](int item, int m) { return __ldcg(reinterpret_cast<const float2 *>(a.x + (size_t)m * d + 2 * item)); };
+    auto add_pair = [&](int item, int m, float v0, float v1, float2 old) {
+        *reinterpret_cast<float2 *>(a.x + (size_t)m * d + 2 * item) = make_float2(old.x + v0, old.y + v1);
+    };
+    auto nothing = [&](int, int) { return make_float2(0.f, 0.f); };
+    for (int l = 0; l < a.n_layers; ++l) {
+        const LayerW &ly = a.layers[l];
+        if (!(a.skip[l >> 4] >> (2 * (l & 15)) & 1u)) {
+            WT *kc = reinterpret_cast<WT *>(a.kc) + (size_t)l * a.Hkv * a.max_seq * hd, *vc = reinterpret_cast<WT *>(a.vc) + (size_t)l * a.Hkv * a.max_seq * hd;
+            map_rows<WT, MT, true>(a.x, M, d, ly.attn_norm, a.eps, slots * half,
+                             [&](int item, const WT *&r0, const WT *&r1) {
+                                 int slot = item / half;
+                                 const void *W = ly.wq;
+                                 if (slot >= a.H) { W = ly.wk; slot -= a.H; if (slot >= a.Hkv) { W = ly.wv; slot -= a.Hkv; } }
+                                 r0 = reinterpret_cast<const WT *>(W) + (size_t)(slot * hd + item % half) * d;
+                                 r1 = r0 + (size_t)half * d;
+                             },
+                             [&](int item, int m) { return __ldcg(a.rope_cs + m * half + item % half); },
+                             [&](int item, int m, float p, float q, float2 c) {
+                                 const int slot = item / half, i = item % half;
+                                 if (slot < a.H + a.Hkv) {
+                                     // the rounding is spelled out, so that it is the same in every instance of the kernel
+                                     const float rp = __fmaf_rn(p, c.x, -__fmul_rn(q, c.y));
+                                     q = __fmaf_rn(q, c.x, __fmul_rn(p, c.y));
+                                     p = rp;
+                                 }
+                                 if (slot < a.H) {
+                                     float *dst = a.qkv + (size_t)m * slots * hd + (size_t)slot * hd + i;
+                                     dst[0] = p;
+                                     dst[half] = q;
+                                 } else {
+                                     const bool is_k = slot < a.H + a.Hkv;
+                                     WT *dst = (is_k ? kc : vc) + ((size_t)(slot - a.H - (is_k ? 0 : a.Hkv)) * a.max_seq + pos0 + m) * hd + i;
+                                     WeightLoad<WT>::store1(dst, p);
+                                     WeightLoad<WT>::store1(dst + half, q);
+                                 }
+                             });
+            if (!meet_grid(a, met, &s_abort)) return;
+            for (int task = blockIdx.x; task < a.H * M * n_split; task += gridDim.x)
+                attend<WT>(a, kc, vc, pos0 + task / a.H % M + 1, task % a.H, task / a.H % M, task / (a.H * M), n_split == 1, s_p, s_red);
+            if (!meet_grid(a, met, &s_abort)) return;
+            if (n_split > 1) {
+                for (int task = blockIdx.x; task < a.H * M; task += gridDim.x) {
+                    const int m = task / a.H, ns = (pos0 + m + ATT_CHUNK) / ATT_CHUNK;
+                    if (tid < hd) {
+                        const size_t at = (size_t)task * a.n_splits;     // task = m H + head
+                        float mx = -INFINITY, den = 0.f, o = 0.f;
+                        for (int s = 0; s < ns; ++s) mx = fmaxf(mx, __ldcg(a.part_ml + at + s).x);
+                        for (int s = 0; s < ns; ++s) {
+                            const float2 ml = __ldcg(a.part_ml + at + s);
+                            const float w = expf(ml.x - mx);
+                            den = fmaf(ml.y, w, den);
+                            o = fmaf(__ldcg(a.part_o + (at + s) * hd + tid), w, o);
+                        }
+                        a.attn[(size_t)task * hd + tid] = o / den;
+                    }
+                }
+                if (!meet_grid(a, met, &s_abort)) return;
+            }
+            map_rows<WT, MT, false>(a.attn, M, nq, nullptr, 0.f, d / 2, [&](int item, const WT *&r0, const WT *&r1) { pair_rows(ly.wo, nq, d, item, r0, r1); }, old_pair, add_pair);
+            if (!meet_grid(a, met, &s_abort)) return;
+        }
+        if (!(a.skip[l >> 4] >> (2 * (l & 15) + 1) & 1u)) {
+            map_rows<WT, MT, true>(a.x, M, d, ly.mlp_norm, a.eps, a.F,
+                             [&](int item, const WT *&r0, const WT *&r1) {
+                                 r0 = reinterpret_cast<const WT *>(ly.w_gate) + (size_t)item * d;
+                                 r1 = reinterpret_cast<const WT *>(ly.w_up) + (size_t)item * d;
+                             },
+                             nothing,
+                             [&](int item, int m, float g, float u, float2) {
+                                 a.act[(size_t)m * a.F + item] = g / (1.0f + expf(-g)) * u;
+                             });
+            if (!meet_grid(a, met, &s_abort)) return;
+            map_rows<WT, MT, false>(a.act, M, a.F, nullptr, 0.f, d / 2, [&](int item, const WT *&r0, const WT *&r1) { pair_rows(ly.w_down, a.F, d, item, r0, r1); }, old_pair, add_pair);
+            if (!meet_grid(a, met, &s_abort)) return;
+        }
+    }
+    const int hm = M - a.head_row0;
+    if (!a.want_hidden && hm <= 0) return;
+    if (a.want_hidden && (int)blockIdx.x < M) {
+        norm_scales(a.x, M, d, a.eps, s_rinv);
+        for (int m = blockIdx.x; m < M; m += gridDim.x)
+            for (int i = tid; i < d; i += NT) a.hfinal[(size_t)m * d + i] = __ldcg(a.x + (size_t)m * d + i) * s_rinv[m] * a.final_norm[i];
+    }
+    if (hm <= 0) return;
+    map_rows<WT, MT, true>(a.x + (size_t)a.head_row0 * d, hm, d, a.final_norm, a.eps, (a.V + 1) / 2,
+                     [&](int item, const WT *&r0, const WT *&r1) { pair_rows(a.lm_head, d, a.V, item, r0, r1); },
+                     nothing,
+                     [&](int item, int m, float v0, float v1, float2) {
+                         float *dst = a.logits + (size_t)(a.head_row0 + m) * a.V + 2 * item;
+                         dst[0] = v0;
+                         if (2 * item + 1 < a.V) dst[1] = v1;
+                     });
+    if (!meet_grid(a, met, &s_abort)) return;
+    for (int j = blockIdx.x; j < hm; j += gridDim.x) {               // arg-max of a row by a block, lowest index among equals
+        const float *row = a.logits + (size_t)(a.head_row0 + j) * a.V;
+        float bv = -INFINITY;
+        int bi = 0x7fffffff;
+#pragma unroll 4
+        for (int i = tid; i < a.V; i += NT) argmax_fold(bv, bi, __ldcg(row + i), i);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+            argmax_fold(bv, bi, ov, oi);
+        }
+        __syncthreads();
+        if ((tid & 31) == 0) { s_red[tid >> 5] = bv; s_red_i[tid >> 5] = bi; }
+        __syncthreads();
+        if (tid == 0) {
+            for (int w = 1; w < NW; ++w) argmax_fold(bv, bi, s_red[w], s_red_i[w]);
+            a.argmax_out[j] = argmax_checked(bi, a.V, a.err);
+        }
+    }
+}
+
+}  // namespace small
+}  // namespace knnssd
