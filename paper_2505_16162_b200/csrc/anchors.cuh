@@ -20,7 +20,7 @@ namespace anchors {
 
 constexpr int MAXC = 16;       // most clusters (domains)
 constexpr int CHUNK = 256;     // columns of the centroids staged in shared memory per step
-constexpr int PTS = 16;        // points per block of assign_kernel: two per warp
+constexpr int MAX_WARPS = 8;   // most warps of a block of assign_kernel, two points each
 constexpr int RING = 3;        // steps of columns a block of assign_kernel has in flight or in use: three blocks per SM
 
 // What the rounds of a call leave on the device, so that several rounds can be enqueued without the host looking at the
@@ -46,19 +46,31 @@ template <bool VEC> __device__ __forceinline__ void copy_piece(float *dst, const
 
 // For each point: the squared distances to all n centroids, labels[p] <- the nearest centroid (lowest index among equal
 // distances); the round's `changed` is set if that differs from the old label, its counts[c] incremented.  mu32 holds the
-// centroids rounded to fp32, rows of stride ld (a multiple of 4).  grid = ceil(N / PTS), 256 threads: a warp owns two
-// points, the block shares the columns of the centroids.  Per step of 256 columns a lane holds 8 columns of each of its
+// centroids rounded to fp32, rows of stride ld (a multiple of 4).  4 .. 8 warps a block (assign_warps), grid = ceil(N / (2 warps)): a
+// warp owns two points, the block shares the columns of the centroids.  Per step of 256 columns a lane holds 8 columns of each of its
 // points (VEC, d % 4 == 0: two runs of four).  Points and centroids come through a ring of RING steps of asynchronous
-// copies: what bounds the kernel is how much of the points is in flight (5000 x 5120: one step ahead in registers 58 us, with the ring 35).
+// copies: what bounds the kernel is how much of the points is in flight (5000 x 5120: one step ahead in registers 58 us, with the ring 35) and
+// the SM with most of the points (blocks of 8 warps leave 48 points on some SMs for 34 on average, of 6 warps 36: 30 us).
 // NC = the cluster count rounded up to 4, 8 or 16: the per-cluster registers follow it.
-template <int NC> constexpr int assign_smem() { return RING * (PTS + NC) * CHUNK * (int)sizeof(float); }
+template <int NC> constexpr int assign_smem(int warps) { return RING * (2 * warps + NC) * CHUNK * (int)sizeof(float); }
+// Warps per block: the fewest points on the fullest SM, blocks dealt out evenly; the larger block among equals.
+inline int assign_warps(int N, int n_sms) {
+    int best = MAX_WARPS;
+    long long least = -1;
+    for (int w = MAX_WARPS; w >= 4; --w) {
+        const long long blocks = (N + 2 * w - 1) / (2 * w), most = (blocks + n_sms - 1) / n_sms * 2 * w;
+        if (least < 0 || most < least) { least = most; best = w; }
+    }
+    return best;
+}
 template <bool VEC, int NC>
 __global__ void __launch_bounds__(256, NC <= 8 ? 3 : 2) assign_kernel(const float *__restrict__ x, int N, int d, const float *__restrict__ mu32, int ld, int n,
                                                      int parity, int *__restrict__ labels, Progress *__restrict__ pg) {
-    extern __shared__ __align__(16) float as_smem[];             // [RING][PTS points, then NC centroids][CHUNK]
+    extern __shared__ __align__(16) float as_smem[];             // [RING][pts points, then NC centroids][CHUNK]
+    chain_wait();
     if (pg->done) return;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int p0 = blockIdx.x * PTS, pa = p0 + 2 * warp;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5, pts = 2 * warps;
+    const int p0 = blockIdx.x * pts, pa = p0 + 2 * warp;
     // running sums as unevaluated pairs of floats (hi + lo, hi the rounded sum, lo the rounding errors collected by
     // the error-free two-sum): ~48 bits without touching the fp64 pipe in the loop
     float hi[2][NC], lo[2][NC];
@@ -75,8 +87,8 @@ __global__ void __launch_bounds__(256, NC <= 8 ? 3 : 2) assign_kernel(const floa
     auto fetch = [&](int step) {
         if (step < steps) {
             const int col0 = step * CHUNK;
-            float *st = as_smem + (step % RING) * (PTS + NC) * CHUNK;
-            // rows of this warp: its two points, and every eighth centroid
+            float *st = as_smem + (step % RING) * (pts + NC) * CHUNK;
+            // rows of this warp: its two points, and its share of the centroids
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 const int p = pa + q;
@@ -87,11 +99,11 @@ __global__ void __launch_bounds__(256, NC <= 8 ? 3 : 2) assign_kernel(const floa
                     copy_piece<VEC>(st + (2 * warp + q) * CHUNK + j, src + (live ? col0 + j : 0), live);
                 }
             }
-            for (int c = warp; c < n; c += 8)
+            for (int c = warp; c < n; c += warps)
 #pragma unroll
                 for (int j = lane * 4; j < CHUNK; j += 128) {
                     const bool live = col0 + j < ld;
-                    copy_piece<true>(st + (PTS + c) * CHUNK + j, mu32 + (size_t)c * ld + (live ? col0 + j : 0), live);
+                    copy_piece<true>(st + (pts + c) * CHUNK + j, mu32 + (size_t)c * ld + (live ? col0 + j : 0), live);
                 }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");     // empty groups keep the count of groups equal to that of steps
@@ -102,7 +114,7 @@ __global__ void __launch_bounds__(256, NC <= 8 ? 3 : 2) assign_kernel(const floa
         asm volatile("cp.async.wait_group %0;" ::"n"(RING - 2) : "memory");
         __syncthreads();                                         // this step has arrived for all; the one before has been read by all
         fetch(step + RING - 1);
-        const float *st = as_smem + (step % RING) * (PTS + NC) * CHUNK;
+        const float *st = as_smem + (step % RING) * (pts + NC) * CHUNK;
         auto row = [&](int r, float (&v)[8]) {
             if (VEC) {
 #pragma unroll
@@ -123,7 +135,7 @@ __global__ void __launch_bounds__(256, NC <= 8 ? 3 : 2) assign_kernel(const floa
             if (c < n) {
                 // columns past the end hold zeros on both sides: they add nothing
                 float m[8], sa = 0.f, sb = 0.f;
-                row(PTS + c, m);
+                row(pts + c, m);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const float da = ca[i] - m[i], db = cb[i] - m[i];
@@ -165,6 +177,7 @@ __global__ void __launch_bounds__(256, NC <= 8 ? 3 : 2) assign_kernel(const floa
 __global__ void __launch_bounds__(256) partial_sums_kernel(const float *__restrict__ x, int N, int d, const int *__restrict__ labels,
                                                            int n, int per, double *__restrict__ part, int parity,
                                                            const Progress *__restrict__ pg) {
+    chain_wait();
     if (pg->done || !pg->changed[parity]) return;
     __shared__ double acc[MAXC][256];
     const int j = blockIdx.x * 256 + threadIdx.x, s = blockIdx.y;
@@ -191,6 +204,7 @@ __global__ void __launch_bounds__(256) partial_sums_kernel(const float *__restri
 // the counters of the next round.  grid = (ceil(d / 256), n), 256 threads.
 __global__ void fold_centroids_kernel(const double *__restrict__ part, int n, int d, int S, double *__restrict__ mu, float *__restrict__ mu32,
                                       int ld, int parity, Progress *__restrict__ pg) {
+    chain_wait();
     const bool changed = pg->changed[parity] != 0;
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && !pg->done) {
         // the other blocks act on this round's `changed` and `counts` alone, which stay as they are until the next round's end
@@ -231,6 +245,7 @@ __global__ void start_centroids_kernel(const float *__restrict__ start, int d, d
 // stride over the columns, fixed-order reduction.  Runs once per call.  grid = ceil(N / 8), 256 threads.
 __global__ void __launch_bounds__(256) member_dist_kernel(const float *__restrict__ x, int N, int d, const double *__restrict__ mu,
                                                           const int *__restrict__ labels, double *__restrict__ dist) {
+    chain_wait();
     const int lane = threadIdx.x & 31, p = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (p >= N) return;
     const float *xr = x + (size_t)p * d;
@@ -246,50 +261,94 @@ __global__ void __launch_bounds__(256) member_dist_kernel(const float *__restric
 }
 
 // Eq. (2) for cluster c = blockIdx.x: k times, the not yet taken member with the smallest (distance, index);
-// out[c][r] = its index, -1 once the cluster has run out of members.  A copy of the distances in shared memory (staged != 0:
-// N doubles) serves all k searches, with -1 for points that are no member or taken; longer lists are read from global memory
-// each time, taken[N] starting at zero.  SEL_NT threads.  (5 x 10 of 5000 points: 17 us; 256 threads
-// re-reading labels and distances took 38.)
-constexpr int SEL_NT = 1024, SEL_STAGED = 25600;
+// out[c][r] = its index, -1 once the cluster has run out of members.  Distances are compared as the bit patterns of non-negative
+// doubles: the fp64 pipe takes eight clocks for a warp's comparison.  A copy of them in shared memory (staged != 0: N words), NO_KEY for
+// points that are no member or taken, serves all k searches; longer lists are read from global memory each time, taken[N]
+// starting at zero.  SEL_NT threads.  Staged and k <= SEL_K: every warp takes the k first of its own points, without
+// meeting the others, and one warp merges the lists (5 x 10 of 5000 points: 15 us; a meeting of the block per anchor and fp64
+// comparisons 17).
+constexpr int SEL_NT = 1024, SEL_STAGED = 25600, SEL_K = 32;
+constexpr unsigned long long NO_KEY = ~0ull;
+// The smallest (key, i) of the lanes, in every lane.
+__device__ __forceinline__ void first_of_warp(unsigned long long &key, int &i) {
+    const unsigned hi = (unsigned)(key >> 32), mh = __reduce_min_sync(0xffffffffu, hi);
+    const unsigned lo = (unsigned)key, ml = __reduce_min_sync(0xffffffffu, hi == mh ? lo : ~0u);
+    i = __reduce_min_sync(0xffffffffu, hi == mh && lo == ml ? i : 0x7fffffff);
+    key = (unsigned long long)mh << 32 | ml;
+}
 __global__ void __launch_bounds__(SEL_NT) select_anchors_kernel(const double *__restrict__ dist, const int *__restrict__ labels, int N, int k,
                                                                 int staged, unsigned char *__restrict__ taken, int *__restrict__ out) {
-    extern __shared__ double sel_dist[];
-    __shared__ double sv[SEL_NT / 32];
-    __shared__ int si[SEL_NT / 32];
+    chain_wait();
+    extern __shared__ unsigned long long sel_key[];
+    __shared__ unsigned long long list_key[SEL_NT / 32][SEL_K];
+    __shared__ int list_i[SEL_NT / 32][SEL_K];
     const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // does (ov, oi) come before (v, i)?  -1: nothing there
-    auto before = [](double ov, int oi, double v, int i) { return oi >= 0 && (i < 0 || ov < v || (ov == v && oi < i)); };
     if (staged)
-        for (int p = tid; p < N; p += SEL_NT) sel_dist[p] = labels[p] == c ? dist[p] : -1.0;
-    for (int r = 0; r < k; ++r) {
-        double bv = INFINITY;
-        int bi = -1;
-        for (int p = tid; p < N; p += SEL_NT) {                  // ascending p: the first of equals wins
-            const double v = staged ? sel_dist[p] : (labels[p] == c && !taken[p] ? dist[p] : -1.0);
-            if (v != -1.0 && (bi < 0 || v < bv)) { bv = v; bi = p; }
-        }
+        for (int p0 = tid; p0 < N; p0 += 8 * SEL_NT) {           // eight points' loads in flight
+            int l[8];
+            double v[8];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-            if (before(ov, oi, bv, bi)) { bv = ov; bi = oi; }
+            for (int e = 0; e < 8; ++e) {
+                const int p = min(p0 + e * SEL_NT, N - 1);
+                l[e] = labels[p];
+                v[e] = dist[p];
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (p0 + e * SEL_NT < N) sel_key[p0 + e * SEL_NT] = l[e] == c ? (unsigned long long)__double_as_longlong(v[e]) : NO_KEY;
         }
-        if (lane == 0) { sv[warp] = bv; si[warp] = bi; }
+    // this thread's first untaken point: ascending p, so the first of equals wins
+    auto own_first = [&](unsigned long long &key, int &i) {
+        key = NO_KEY;
+        i = 0x7ffffffe;
+        for (int p = tid; p < N; p += SEL_NT) {
+            const unsigned long long v = staged ? sel_key[p] : (labels[p] == c && !taken[p] ? (unsigned long long)__double_as_longlong(dist[p]) : NO_KEY);
+            if (v < key) { key = v; i = p; }
+        }
+    };
+    unsigned long long key;
+    int i;
+    if (staged && k <= SEL_K) {
+        unsigned long long own;
+        int own_i;
+        own_first(own, own_i);
+        for (int r = 0; r < k; ++r) {
+            key = own;
+            i = own_i;
+            first_of_warp(key, i);
+            if (lane == 0) { list_key[warp][r] = key; list_i[warp][r] = i; }
+            if (key != NO_KEY && i == own_i) {                   // only the owner of the point looks for its next one
+                sel_key[i] = NO_KEY;
+                own_first(own, own_i);
+            }
+        }
+        __syncthreads();
+        if (warp) return;
+        int at = 0;                                              // lane = list
+        for (int r = 0; r < k; ++r) {
+            const int mine = at < k ? list_i[lane][at] : 0x7ffffffe;
+            key = at < k ? list_key[lane][at] : NO_KEY;
+            i = mine;
+            first_of_warp(key, i);
+            if (key != NO_KEY && i == mine) ++at;
+            if (lane == 0) out[c * k + r] = key != NO_KEY ? i : -1;
+        }
+        return;
+    }
+    for (int r = 0; r < k; ++r) {
+        own_first(key, i);
+        first_of_warp(key, i);
+        if (lane == 0) { list_key[warp][0] = key; list_i[warp][0] = i; }
         __syncthreads();
         if (warp == 0) {
-            bv = sv[lane];
-            bi = si[lane];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
-                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-                if (before(ov, oi, bv, bi)) { bv = ov; bi = oi; }
-            }
+            key = list_key[lane][0];
+            i = list_i[lane][0];
+            first_of_warp(key, i);
             if (lane == 0) {
-                out[c * k + r] = bi;
-                if (bi >= 0) {
-                    if (staged) sel_dist[bi] = -1.0;
-                    else taken[bi] = 1;
+                out[c * k + r] = key != NO_KEY ? i : -1;
+                if (key != NO_KEY) {
+                    if (staged) sel_key[i] = NO_KEY;
+                    else taken[i] = 1;
                 }
             }
         }

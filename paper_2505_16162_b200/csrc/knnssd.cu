@@ -238,6 +238,13 @@ int current_device_slot() {
     return dev;
 }
 
+// Multiprocessors of the current device.
+int sm_count() {
+    int dev = 0, n = 148;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n;
+}
+
 // Address of the word on the CURRENT device that the launches of knnssd_linear report to (every device that loads the library has
 // its own copy).  Sessions and the operators that synchronise have words of their own: a word that several callers read and clear
 // tells one of them what another's launch met.
@@ -1660,7 +1667,8 @@ knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int 
     typedef void (*AssignFn)(const float *, int, int, const float *, int, int, int, int *, anchors::Progress *);
     const AssignFn assign = vec ? (n <= 4 ? anchors::assign_kernel<true, 4> : n <= 8 ? anchors::assign_kernel<true, 8> : anchors::assign_kernel<true, 16>)
                                 : (n <= 4 ? anchors::assign_kernel<false, 4> : n <= 8 ? anchors::assign_kernel<false, 8> : anchors::assign_kernel<false, 16>);
-    const int assign_smem = n <= 4 ? anchors::assign_smem<4>() : n <= 8 ? anchors::assign_smem<8>() : anchors::assign_smem<16>();
+    const int warps = anchors::assign_warps(N, sm_count());
+    const int assign_smem = n <= 4 ? anchors::assign_smem<4>(warps) : n <= 8 ? anchors::assign_smem<8>(warps) : anchors::assign_smem<16>(warps);
     const int staged = N <= anchors::SEL_STAGED, sel_smem = staged ? N * (int)sizeof(double) : 0;
     ok = ok && cudaFuncSetAttribute(assign, cudaFuncAttributeMaxDynamicSharedMemorySize, assign_smem) == cudaSuccess &&
          cudaFuncSetAttribute(anchors::select_anchors_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1679,9 +1687,9 @@ knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int 
     for (int r0 = 0; r0 < max_rounds && e == cudaSuccess; r0 += 4) {
         cudaEventRecord(e0, s);
         for (int r = r0; r < max_rounds && r < r0 + 4; ++r) {
-            assign<<<(N + anchors::PTS - 1) / anchors::PTS, 256, assign_smem, s>>>(x_dev, N, d, mu32, ld, n, r & 1, labels, progress);
-            anchors::partial_sums_kernel<<<dim3(cols.x, S), 256, 0, s>>>(x_dev, N, d, labels, n, per, part, r & 1, progress);
-            anchors::fold_centroids_kernel<<<cols, 256, 0, s>>>(part, n, d, S, mu, mu32, ld, r & 1, progress);
+            launch_chained(assign, dim3((N + 2 * warps - 1) / (2 * warps)), dim3(32 * warps), assign_smem, s, x_dev, N, d, mu32, ld, n, r & 1, labels, progress);
+            launch_chained(anchors::partial_sums_kernel, dim3(cols.x, S), dim3(256), 0, s, x_dev, N, d, labels, n, per, part, r & 1, progress);
+            launch_chained(anchors::fold_centroids_kernel, cols, dim3(256), 0, s, part, n, d, S, mu, mu32, ld, r & 1, progress);
         }
         cudaEventRecord(e1, s);
         int seen[2] = {0, 0};                                    // done, rounds
@@ -1700,7 +1708,7 @@ knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int 
         // if the round limit ended the iteration)
         anchors::member_dist_kernel<<<(N + 7) / 8, 256, 0, s>>>(x_dev, N, d, mu, labels, dist);
         if (!staged) cudaMemsetAsync(taken, 0, (size_t)N, s);
-        anchors::select_anchors_kernel<<<n, anchors::SEL_NT, sel_smem, s>>>(dist, labels, N, k, staged, taken, out);
+        launch_chained(anchors::select_anchors_kernel, dim3(n), dim3(anchors::SEL_NT), sel_smem, s, dist, labels, N, k, staged, taken, out);
         e = cudaMemcpyAsync(anchors_host, out, sizeof(int) * n * k, cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess && labels_host) e = cudaMemcpyAsync(labels_host, labels, sizeof(int) * N, cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess && centroids_out_dev)
