@@ -242,10 +242,13 @@ __global__ void start_centroids_kernel(const float *__restrict__ start, int d, d
 // dist[p] = ||x_p - mu_{labels[p]}|| with every difference, square and sum in fp64 against the fp64 centroid: the
 // distances Eq. (2) ranks the members by.  Points at equal distance in exact arithmetic (duplicates, or points mirrored
 // about their centroid) then get equal values, so the lowest index decides among them.  One warp per point, lanes
-// stride over the columns, fixed-order reduction.  Runs once per call.  grid = ceil(N / 8), 256 threads.
+// stride over the columns, fixed-order reduction.  Nothing happens while the rounds are
+// not done and these are not the last ones.  grid = ceil(N / 8), 256 threads.
 __global__ void __launch_bounds__(256) member_dist_kernel(const float *__restrict__ x, int N, int d, const double *__restrict__ mu,
-                                                          const int *__restrict__ labels, double *__restrict__ dist) {
+                                                          const int *__restrict__ labels, double *__restrict__ dist,
+                                                          const Progress *__restrict__ pg, int last) {
     chain_wait();
+    if (!pg->done && !last) return;
     const int lane = threadIdx.x & 31, p = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (p >= N) return;
     const float *xr = x + (size_t)p * d;
@@ -277,8 +280,10 @@ __device__ __forceinline__ void first_of_warp(unsigned long long &key, int &i) {
     key = (unsigned long long)mh << 32 | ml;
 }
 __global__ void __launch_bounds__(SEL_NT) select_anchors_kernel(const double *__restrict__ dist, const int *__restrict__ labels, int N, int k,
-                                                                int staged, unsigned char *__restrict__ taken, int *__restrict__ out) {
+                                                                int staged, unsigned char *__restrict__ taken, int *__restrict__ out,
+                                                                const Progress *__restrict__ pg, int last) {
     chain_wait();
+    if (!pg->done && !last) return;
     extern __shared__ unsigned long long sel_key[];
     __shared__ unsigned long long list_key[SEL_NT / 32][SEL_K];
     __shared__ int list_i[SEL_NT / 32][SEL_K];

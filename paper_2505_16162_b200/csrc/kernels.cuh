@@ -463,9 +463,13 @@ __global__ void __launch_bounds__(256) row_scale_kernel(const float *__restrict_
     for (int w = 0; w < 8; ++w) tot += s_red[w];
     rinv[m] = 1.0f / sqrtf(tot / (float)d + eps);
 }
-__global__ void pool_finish_kernel(const double *__restrict__ sum, int d, double inv_count, float *__restrict__ v) {
+// v <- the mean, and to the caller's buffer as well if there is one.
+__global__ void pool_finish_kernel(const double *__restrict__ sum, int d, double inv_count, float *__restrict__ v, float *__restrict__ also) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < d) v[i] = (float)(sum[i] * inv_count);
+    if (i >= d) return;
+    const float m = (float)(sum[i] * inv_count);
+    v[i] = m;
+    if (also) also[i] = m;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -530,10 +534,7 @@ __global__ void argmax_final_kernel(const float *__restrict__ pv, const int *__r
 // d_0..d_{a-1}, target[a] are appended to out_tokens; target[a] becomes the pending token; the committed
 // length grows by a + 1 (rows beyond it are dead).
 // ---------------------------------------------------------------------------------------------
-__global__ void accept_kernel(int *__restrict__ chain, const int *__restrict__ target, int k, DeviceState *__restrict__ st,
-                              int *__restrict__ out_tokens, int out_cap, int *__restrict__ accept_log, int round_idx) {
-    chain_wait();
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+__device__ __forceinline__ void accept_rows(int *chain, const int *target, int k, DeviceState *st, int *out_tokens, int out_cap, int *accept_log, int round_idx) {
     int a = 0;
     while (a < k && target[a] == chain[a + 1]) ++a;
     const int next = target[a];
@@ -546,6 +547,56 @@ __global__ void accept_kernel(int *__restrict__ chain, const int *__restrict__ t
     st->last_next = next;
     chain[0] = next;
     if (accept_log) accept_log[round_idx] = a;
+}
+__global__ void accept_kernel(int *__restrict__ chain, const int *__restrict__ target, int k, DeviceState *__restrict__ st,
+                              int *__restrict__ out_tokens, int out_cap, int *__restrict__ accept_log, int round_idx) {
+    chain_wait();
+    if (threadIdx.x == 0 && blockIdx.x == 0) accept_rows(chain, target, k, st, out_tokens, out_cap, accept_log, round_idx);
+}
+
+// What a call hands back, in one launch behind its last pass: rows of logits and hidden states to the caller's buffers, words and the
+// error word to pinned host memory (visible once the stream has been waited for).  ACCEPT: after accept_rows, the words are the
+// session's state.  Copies of their own between kernels and the wait cost ~5 us each.
+struct Delivery {
+    const float *src[2];
+    float *dst[2];
+    size_t n[2];                 // floats; 0: nothing
+    const int *words;
+    int n_words;
+    const int *err;
+    int *host, *host_err;        // pinned
+    // ACCEPT
+    int *chain;
+    const int *target;
+    int k;
+    DeviceState *st;
+    int *out_tokens, out_cap, *accept_log, round_idx;
+};
+template <bool ACCEPT> __global__ void __launch_bounds__(256) deliver_kernel(const Delivery a) {
+    chain_wait();
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
+        if (ACCEPT && threadIdx.x == 0) accept_rows(a.chain, a.target, a.k, a.st, a.out_tokens, a.out_cap, a.accept_log, a.round_idx);
+        __syncwarp();
+        for (int i = threadIdx.x; i < a.n_words; i += 32) a.host[i] = *reinterpret_cast<const volatile int *>(a.words + i);
+        if (threadIdx.x == 0) *a.host_err = *a.err;
+    }
+    const size_t first = (size_t)blockIdx.x * 256 + threadIdx.x, stride = (size_t)gridDim.x * 256;
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        if (a.n[r] == 0) continue;
+        if (((reinterpret_cast<uintptr_t>(a.src[r]) | reinterpret_cast<uintptr_t>(a.dst[r])) & 15u) == 0 && a.n[r] % 4 == 0) {
+#pragma unroll 4
+            for (size_t i = first; i < a.n[r] / 4; i += stride) reinterpret_cast<float4 *>(a.dst[r])[i] = reinterpret_cast<const float4 *>(a.src[r])[i];
+        } else {
+            for (size_t i = first; i < a.n[r]; i += stride) a.dst[r][i] = a.src[r][i];
+        }
+    }
+}
+
+// Up to 16 token ids, by value, into the session's chain.
+struct Tokens { int id[16]; };
+__global__ void put_tokens_kernel(const Tokens t, int n, int *__restrict__ chain) {
+    if (threadIdx.x < n) chain[threadIdx.x] = t.id[threadIdx.x];
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -633,8 +684,10 @@ __global__ void set_word_kernel(int *word, int value) { *word = value; }
 __global__ void set_state_kernel(DeviceState *st, int len, int produced) {
     st->len = len; st->produced = produced; st->last_accept = 0; st->last_next = -1;
 }
-__global__ void emit_first_token_kernel(const int *chain, DeviceState *st, int *out_tokens, int len) {
+// The first token of a generation; where `host` (pinned) is given the host gets it there, and the error word behind it.
+__global__ void emit_first_token_kernel(const int *chain, DeviceState *st, int *out_tokens, int len, const int *err, int *host, int *host_err) {
     out_tokens[0] = chain[0]; st->produced = 1; st->len = len;
+    if (host) { *host = chain[0]; *host_err = *err; }
 }
 
 }  // namespace knnssd

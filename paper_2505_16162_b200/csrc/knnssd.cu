@@ -188,18 +188,28 @@ struct Scratch {
     }
 };
 
-// A few words of pinned memory per host thread, which kernels read arguments from and write results to: the calls that
-// use them synchronise before they return.  nullptr if they cannot be had.
-constexpr int kHostWords = 64;
-int *host_words() {
+// `n` words of pinned memory per host thread, which kernels read arguments from and write results to: the calls that
+// use them synchronise before they return.  At least kHostWords are kept from call to call, at most 1 MB; nullptr if they cannot be
+// had or would be more.
+constexpr size_t kHostWords = 64, kMostHostWords = (size_t)1 << 18;
+int *host_words(size_t n = kHostWords) {
     struct Words {
         int *p = nullptr;
+        size_t n = 0;
         ~Words() { if (p) cudaFreeHost(p); }
     };
     static thread_local Words w;
-    if (!w.p && cudaHostAlloc(reinterpret_cast<void **>(&w.p), kHostWords * sizeof(int), cudaHostAllocPortable) != cudaSuccess) {
-        cudaGetLastError();
+    if (n > kMostHostWords) return nullptr;
+    if (w.n < n) {
+        if (w.p) cudaFreeHost(w.p);
         w.p = nullptr;
+        w.n = 0;
+        if (cudaHostAlloc(reinterpret_cast<void **>(&w.p), n * sizeof(int), cudaHostAllocPortable) != cudaSuccess) {
+            cudaGetLastError();
+            w.p = nullptr;
+            return nullptr;
+        }
+        w.n = n;
     }
     return w.p;
 }
@@ -634,12 +644,9 @@ knnssd_status fail_device_code(knnssd_ctx *c, const char *what, int code) {
                                        "); prefill again");
 }
 
-// Enqueue the read-back of the device error word with a call's other results; after the synchronisation that follows,
-// checked_err reports it once and clears it.
+// The last kernel of a call leaves the device error word in the pinned words with the call's other results; after the
+// synchronisation that follows, checked_err reports it once and clears it.
 constexpr int kErrWord = 32;           // its place in the pinned words
-cudaError_t read_err_word(knnssd_ctx *c) {
-    return cudaMemcpyAsync(c->pinned + kErrWord, c->err_word, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
-}
 knnssd_status checked_err(knnssd_ctx *c, const char *what) {
     return c->pinned[kErrWord] ? fail_device_code(c, what, c->pinned[kErrWord]) : KNNSSD_OK;
 }
@@ -667,6 +674,14 @@ void free_all(knnssd_ctx *c) {
     if (c->ev1) cudaEventDestroy(c->ev1);
     if (c->ev2) cudaEventDestroy(c->ev2);
     for (cudaEvent_t e : c->lin_events) cudaEventDestroy(e);
+}
+
+// Whether a kernel of this session may store floats to a caller's buffer.  What is elsewhere (another device, managed or host
+// memory) or not a multiple of four bytes is left to a copy.
+bool stores_reach(const knnssd_ctx *c, const void *p) {
+    cudaPointerAttributes at{};
+    if ((reinterpret_cast<uintptr_t>(p) & 3u) || cudaPointerGetAttributes(&at, p) != cudaSuccess) { cudaGetLastError(); return false; }
+    return at.type == cudaMemoryTypeDevice && at.device == c->device;
 }
 
 struct DeviceGuard {
@@ -789,12 +804,11 @@ knnssd_status do_prefill(knnssd_ctx *c, const int *tokens_host, int n, float *po
             pool_accumulate_kernel<<<(d + 255) / 256, 256, 0, s>>>(c->hfinal + (size_t)(M - 1) * d, 1, d, c->pool_sum, 1);
         }
     }
-    pool_finish_kernel<<<(d + 255) / 256, 256, 0, s>>>(c->pool_sum, d, g.pool_mode == 0 ? 1.0 / (double)n : 1.0, c->pooled);
-    emit_first_token_kernel<<<1, 1, 0, s>>>(c->chain, c->state, c->out_tokens, n);
+    const bool direct = pooled_dev && stores_reach(c, pooled_dev);
+    pool_finish_kernel<<<(d + 255) / 256, 256, 0, s>>>(c->pool_sum, d, g.pool_mode == 0 ? 1.0 / (double)n : 1.0, c->pooled, direct ? pooled_dev : nullptr);
+    if (pooled_dev && !direct) CUDA_TRY(c, cudaMemcpyAsync(pooled_dev, c->pooled, sizeof(float) * d, cudaMemcpyDeviceToDevice, s));
+    emit_first_token_kernel<<<1, 1, 0, s>>>(c->chain, c->state, c->out_tokens, n, c->err_word, c->pinned, c->pinned + kErrWord);
     cudaEventRecord(c->ev1, s);
-    if (pooled_dev) CUDA_TRY(c, cudaMemcpyAsync(pooled_dev, c->pooled, sizeof(float) * d, cudaMemcpyDeviceToDevice, s));
-    CUDA_TRY(c, cudaMemcpyAsync(c->pinned, c->chain, sizeof(int), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(c, read_err_word(c));
     knnssd_status st = sync_check(c, "prefill");
     if (st == KNNSSD_OK) st = checked_err(c, "prefill");
     if (st != KNNSSD_OK) return st;
@@ -837,6 +851,22 @@ knnssd_status do_select(knnssd_ctx *c, const float *query_dev, int *domain, int 
 }
 
 // Enqueue k draft steps: step j reads chain[j] at position len + j and writes chain[j + 1].
+// A call's results in one launch (see deliver_kernel); its words end up in c->pinned, the error word in its place there.
+template <bool ACCEPT> cudaError_t deliver(knnssd_ctx *c, Delivery out) {
+    cudaError_t e = cudaSuccess;
+    for (int r = 0; r < 2; ++r)
+        if (out.n[r] && !stores_reach(c, out.dst[r])) {
+            e = cudaMemcpyAsync(out.dst[r], out.src[r], out.n[r] * sizeof(float), cudaMemcpyDeviceToDevice, c->stream);
+            if (e != cudaSuccess) return e;
+            out.n[r] = 0;
+        }
+    out.err = c->err_word; out.host = c->pinned; out.host_err = c->pinned + kErrWord;
+    const size_t blocks = (out.n[0] + out.n[1]) / 4 / 256 + 1;       // four floats a thread and step
+    launch_chained(deliver_kernel<ACCEPT>, dim3((unsigned)(blocks < 2 * (size_t)c->n_sms ? blocks : 2 * c->n_sms)), dim3(256), 0, c->stream, out);
+    c->launches++;
+    return e;
+}
+
 void enqueue_draft(knnssd_ctx *c, int k) {
     for (int j = 0; j < k; ++j) run_pass(c, 1, c->chain + j, j, c->active_mask.data(), 0, c->chain + j + 1, false);
 }
@@ -1069,13 +1099,13 @@ knnssd_status knnssd_draft(knnssd_ctx *c, int k, int *draft_tokens_host, float *
     cudaEventRecord(c->ev0, s);
     for (int j = 0; j < k; ++j) {
         run_pass(c, 1, c->chain + j, j, c->active_mask.data(), 0, c->chain + j + 1, false);
-        if (logits_dev_or_null)
-            CUDA_TRY(c, cudaMemcpyAsync(logits_dev_or_null + (size_t)j * c->cfg.vocab, c->logits, sizeof(float) * c->cfg.vocab,
-                                        cudaMemcpyDeviceToDevice, s));
+        if (!logits_dev_or_null && j + 1 < k) continue;
+        Delivery out{};
+        if (logits_dev_or_null) { out.src[0] = c->logits; out.dst[0] = logits_dev_or_null + (size_t)j * c->cfg.vocab; out.n[0] = c->cfg.vocab; }
+        if (j + 1 == k) { out.words = c->chain + 1; out.n_words = k; }
+        CUDA_TRY(c, deliver<false>(c, out));
     }
     cudaEventRecord(c->ev1, s);
-    CUDA_TRY(c, cudaMemcpyAsync(c->pinned, c->chain + 1, sizeof(int) * k, cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(c, read_err_word(c));
     knnssd_status st = sync_check(c, "draft");
     if (st == KNNSSD_OK) st = checked_err(c, "draft");
     if (st != KNNSSD_OK) return st;
@@ -1096,18 +1126,21 @@ knnssd_status knnssd_verify(knnssd_ctx *c, const int *draft_tokens_host, int k, 
         if (draft_tokens_host[j] < 0 || draft_tokens_host[j] >= g.vocab)
             return fail(c, KNNSSD_ERR_INVALID_ARG, "verify: draft token id out of range");
     cudaStream_t s = c->stream;
-    if (k > 0) CUDA_TRY(c, cudaMemcpyAsync(c->chain + 1, draft_tokens_host, sizeof(int) * k, cudaMemcpyHostToDevice, s));
+    if (k > 0) {
+        Tokens t{};
+        for (int j = 0; j < k; ++j) t.id[j] = draft_tokens_host[j];
+        put_tokens_kernel<<<1, 32, 0, s>>>(t, k, c->chain + 1);
+    }
     cudaEventRecord(c->ev0, s);
-    enqueue_verify(c, k, hidden_dev_or_null != nullptr, c->stats.rounds % g.max_seq);
+    run_pass(c, k + 1, c->chain, 0, nullptr, 0, c->target, hidden_dev_or_null != nullptr);
+    Delivery out{};
+    if (logits_dev_or_null) { out.src[0] = c->logits; out.dst[0] = logits_dev_or_null; out.n[0] = (size_t)(k + 1) * g.vocab; }
+    if (hidden_dev_or_null) { out.src[1] = c->hfinal; out.dst[1] = hidden_dev_or_null; out.n[1] = (size_t)(k + 1) * g.d_model; }
+    out.words = reinterpret_cast<const int *>(c->state); out.n_words = sizeof(DeviceState) / sizeof(int);
+    out.chain = c->chain; out.target = c->target; out.k = k; out.st = c->state; out.out_tokens = c->out_tokens; out.out_cap = g.max_seq;
+    out.accept_log = c->accept_log; out.round_idx = c->stats.rounds % g.max_seq;
+    CUDA_TRY(c, deliver<true>(c, out));
     cudaEventRecord(c->ev1, s);
-    if (logits_dev_or_null)
-        CUDA_TRY(c, cudaMemcpyAsync(logits_dev_or_null, c->logits, sizeof(float) * (size_t)(k + 1) * g.vocab,
-                                    cudaMemcpyDeviceToDevice, s));
-    if (hidden_dev_or_null)
-        CUDA_TRY(c, cudaMemcpyAsync(hidden_dev_or_null, c->hfinal, sizeof(float) * (size_t)(k + 1) * g.d_model,
-                                    cudaMemcpyDeviceToDevice, s));
-    CUDA_TRY(c, cudaMemcpyAsync(c->pinned, c->state, sizeof(DeviceState), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(c, read_err_word(c));
     knnssd_status st = sync_check(c, "verify");
     if (st == KNNSSD_OK) st = checked_err(c, "verify");
     if (st != KNNSSD_OK) return st;
@@ -1141,7 +1174,7 @@ static knnssd_status do_decode(knnssd_ctx *c, int max_new, int k, int use_select
     }
     cudaStream_t s = c->stream;
     // the pending token is the first token of this call's output
-    emit_first_token_kernel<<<1, 1, 0, s>>>(c->chain, c->state, c->out_tokens, c->len);
+    emit_first_token_kernel<<<1, 1, 0, s>>>(c->chain, c->state, c->out_tokens, c->len, nullptr, nullptr, nullptr);
     c->launches++;
     int produced = 1, round = 0;
     c->stats.rounds = c->stats.drafted = c->stats.accepted = 0;
@@ -1228,7 +1261,7 @@ knnssd_status knnssd_decode_sampled(knnssd_ctx *c, int max_new, int k, float tem
     auto finish = [&](knnssd_status r) { cudaStreamSynchronize(s); return r; };
     if (max_new > 1 && cudaMemcpyAsync(u_dev, uniforms_host, sizeof(float) * n_u, cudaMemcpyHostToDevice, s) != cudaSuccess)
         return finish(fail(c, KNNSSD_ERR_CUDA, "decode_sampled: cannot copy the uniforms"));
-    emit_first_token_kernel<<<1, 1, 0, s>>>(c->chain, c->state, c->out_tokens, c->len);
+    emit_first_token_kernel<<<1, 1, 0, s>>>(c->chain, c->state, c->out_tokens, c->len, nullptr, nullptr, nullptr);
     c->launches++;
     int produced = 1, round = 0;
     c->stats.rounds = c->stats.drafted = c->stats.accepted = 0;
@@ -1651,14 +1684,19 @@ knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int 
     const int ld = (d + 3) / 4 * 4;                 // row stride of the fp32 centroids
     double *mu = nullptr, *dist = nullptr, *part = nullptr;
     float *mu32 = nullptr;
-    int *labels = nullptr, *out = nullptr;
-    anchors::Progress *progress = nullptr;
     unsigned char *taken = nullptr;
+    // what the host gets, in one piece: progress, anchors, labels
+    constexpr size_t kProgressWords = sizeof(anchors::Progress) / sizeof(int);
+    const size_t n_words = kProgressWords + (size_t)n * k + N;
+    int *words = nullptr, *host = host_words(n_words);
+    std::vector<int> pageable;
+    if (!host) { pageable.resize(n_words); host = pageable.data(); }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     Scratch mem(s);
     bool ok = mem.get(&mu, (size_t)n * d) && mem.get(&mu32, (size_t)n * ld) && mem.get(&dist, (size_t)N) && mem.get(&part, (size_t)S * n * d) &&
-              mem.get(&labels, (size_t)N) && mem.get(&progress, 1) && mem.get(&out, (size_t)n * k) && mem.get(&taken, (size_t)N) &&
-              cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess;
+              mem.get(&words, n_words) && mem.get(&taken, (size_t)N) && cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess;
+    anchors::Progress *progress = reinterpret_cast<anchors::Progress *>(words);
+    int *out = words + kProgressWords, *labels = out + (size_t)n * k;
     auto cleanup = [&]() {
         if (e0) cudaEventDestroy(e0);
         if (e1) cudaEventDestroy(e1);
@@ -1692,29 +1730,26 @@ knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int 
             launch_chained(anchors::fold_centroids_kernel, cols, dim3(256), 0, s, part, n, d, S, mu, mu32, ld, r & 1, progress);
         }
         cudaEventRecord(e1, s);
-        int seen[2] = {0, 0};                                    // done, rounds
-        e = cudaMemcpyAsync(seen, progress, sizeof(seen), cudaMemcpyDeviceToHost, s);
+        // The anchors are ranked by fp64 distances to the final fp64 centroids (which moved after the last assignment if the round
+        // limit ended the iteration).  The ranking goes out behind the rounds: it does nothing while they are not done.
+        const int last = r0 + 4 >= max_rounds;
+        if (!staged) cudaMemsetAsync(taken, 0, (size_t)N, s);
+        launch_chained(anchors::member_dist_kernel, dim3((N + 7) / 8), dim3(256), 0, s, x_dev, N, d, mu, labels, dist, progress, last);
+        launch_chained(anchors::select_anchors_kernel, dim3(n), dim3(anchors::SEL_NT), sel_smem, s, dist, labels, N, k, staged, taken, out, progress, last);
+        if (centroids_out_dev) e = cudaMemcpyAsync(centroids_out_dev, mu, sizeof(double) * n * d, cudaMemcpyDeviceToDevice, s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(host, words, n_words * sizeof(int), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) break;
         float ms = 0.f;
         cudaEventElapsedTime(&ms, e0, e1);
         ms_total += ms;
-        rounds = seen[1];
-        if (seen[0]) break;
+        rounds = host[1];
+        if (host[0]) break;
     }
     if (e == cudaSuccess) {
-        // the anchors are ranked by fp64 distances to the final fp64 centroids (which moved after the last assignment
-        // if the round limit ended the iteration)
-        anchors::member_dist_kernel<<<(N + 7) / 8, 256, 0, s>>>(x_dev, N, d, mu, labels, dist);
-        if (!staged) cudaMemsetAsync(taken, 0, (size_t)N, s);
-        launch_chained(anchors::select_anchors_kernel, dim3(n), dim3(anchors::SEL_NT), sel_smem, s, dist, labels, N, k, staged, taken, out);
-        e = cudaMemcpyAsync(anchors_host, out, sizeof(int) * n * k, cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess && labels_host) e = cudaMemcpyAsync(labels_host, labels, sizeof(int) * N, cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess && centroids_out_dev)
-            e = cudaMemcpyAsync(centroids_out_dev, mu, sizeof(double) * n * d, cudaMemcpyDeviceToDevice, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e == cudaSuccess) e = cudaGetLastError();
+        std::memcpy(anchors_host, host + kProgressWords, sizeof(int) * n * k);
+        if (labels_host) std::memcpy(labels_host, host + kProgressWords + (size_t)n * k, sizeof(int) * N);
     }
     cleanup();
     if (e != cudaSuccess) { cudaGetLastError(); return KNNSSD_ERR_CUDA; }
