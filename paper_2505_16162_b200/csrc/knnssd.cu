@@ -96,6 +96,7 @@ struct knnssd_ctx {
     float *pf_x = nullptr, *pf_qkv = nullptr;                // residual stream [cap][d]; q, k, v [cap][nq + 2 nkv]
     float2 *pf_cs = nullptr;                                 // rotary (cos, sin) of the chunk's rows [cap][hd / 2]
     float *pf_rinv = nullptr;                                // RMSNorm scale of the chunk's rows [cap]
+    float *pf_ss = nullptr;                                  // their sums of squares by 128 columns [d / 128][cap]
     bf16_t *pf_ad = nullptr, *pf_aq = nullptr, *pf_af = nullptr;   // hi / lo planes [2][cap][d], [2][cap][nq], [2][cap][d_ff]
     float *pf_part = nullptr;                                // sums of the pieces of tiles that several CTAs share
 
@@ -665,7 +666,7 @@ void free_all(knnssd_ctx *c) {
                     c->cosines, c->amax_v, c->part_ml, c->rope_cs, c->pool_sum, c->inv_freq, c->chain,
                     c->target, c->prompt, c->out_tokens, c->accept_log, c->amax_i, c->flag, c->knn_work, c->err_word, c->state,
                     c->ops_full, c->ops_draft, c->bar, c->gabort, c->attn_cnt, c->amax_cnt, c->mpart_o, c->mamax_v, c->mpart_ml,
-                    c->mamax_i, c->trace, c->xs_x, c->xs_attn, c->xs_act, c->ssp, c->pf_x, c->pf_qkv, c->pf_ad, c->pf_aq, c->pf_af, c->pf_cs, c->pf_rinv, c->pf_part, c->small_layers, c->small_bar,
+                    c->mamax_i, c->trace, c->xs_x, c->xs_attn, c->xs_act, c->ssp, c->pf_x, c->pf_qkv, c->pf_ad, c->pf_aq, c->pf_af, c->pf_cs, c->pf_rinv, c->pf_ss, c->pf_part, c->small_layers, c->small_bar,
                     c->samp_p, c->samp_q, c->samp_res};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -718,36 +719,42 @@ bool prefill_tensor(knnssd_ctx *c, int n) {
         const bool last = t0 + T == n;
         prefill::embed_rows_kernel<<<T, 256, 0, s>>>(reinterpret_cast<const bf16_t *>(c->tok_embed), c->prompt + t0, d, c->pf_x);
         prefill::rope_table_kernel<<<T, HD / 2, 0, s>>>(c->inv_freq, t0, c->pf_cs);
-        c->launches += 2;
+        launch_chained(prefill::norm_split_kernel, dim3(T), dim3(256), 0, s, c->pf_x, d, c->layers[0].attn_norm, c->pf_ad, c->pf_ad + (size_t)cap * d, c->pf_ss, cap);
+        c->launches += 3;
+        prefill::Norms normed;                       // of the rows a map reads, and below of those it has added to
+        normed.ss = c->pf_ss; normed.rows = cap; normed.eps = g.rms_eps;
+        auto norm_next = [&](const float *gain) {
+            prefill::Norms n;
+            n.rows = cap; n.next_gain = gain; n.next_hi = c->pf_ad; n.next_lo = c->pf_ad + (size_t)cap * d; n.ss_out = c->pf_ss;
+            return n;
+        };
         for (int l = 0; l < g.n_layers && ok; ++l) {
             const Layer &ly = c->layers[l];
             bf16_t *kc = reinterpret_cast<bf16_t *>(c->kcache) + (size_t)l * layer_stride;
             bf16_t *vc = reinterpret_cast<bf16_t *>(c->vcache) + (size_t)l * layer_stride;
-            launch_chained(prefill::norm_split_kernel, dim3(T), dim3(256), 0, s, c->pf_x, d, ly.attn_norm, g.rms_eps, c->pf_ad, c->pf_ad + (size_t)cap * d, c->pf_rinv);
             bool heads_done = false;     // rotary embedding and K / V rows done by the q / k / v launch's epilogue
             if (nq % prefill::BOX_N == 0 && nkv % prefill::BOX_N == 0) {
                 // q, k and v in one launch over the stacked units (their columns of the projection buffer are adjacent)
                 const prefill::QkvFuse fuse{c->pf_cs, kc, vc, g.max_seq, t0, HD};
                 ok = ok && contract(c->pf_ad, ly.wq, ly.wk, ldq, d, T, prefill::PF_STORE, c->pf_qkv, ldq, 0, nullptr,
-                                                nullptr, 0, err, s, ly.wv, nq, nkv, &fuse, &heads_done, c->pf_rinv);
+                                                nullptr, 0, err, s, ly.wv, nq, nkv, &fuse, &heads_done, normed);
             } else {
                 ok = ok && contract(c->pf_ad, ly.wq, nullptr, nq, d, T, prefill::PF_STORE, c->pf_qkv, ldq, 0, nullptr,
-                                                nullptr, 0, err, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
+                                                nullptr, 0, err, s, nullptr, 0, 0, nullptr, nullptr, normed);
                 ok = ok && contract(c->pf_ad, ly.wk, nullptr, nkv, d, T, prefill::PF_STORE, c->pf_qkv, ldq, nq, nullptr,
-                                                nullptr, 0, err, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
+                                                nullptr, 0, err, s, nullptr, 0, 0, nullptr, nullptr, normed);
                 ok = ok && contract(c->pf_ad, ly.wv, nullptr, nkv, d, T, prefill::PF_STORE, c->pf_qkv, ldq, nq + nkv,
-                                                nullptr, nullptr, 0, err, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
+                                                nullptr, nullptr, 0, err, s, nullptr, 0, 0, nullptr, nullptr, normed);
             }
             if (!heads_done) launch_chained(prefill::rope_kv_rows_kernel, dim3(T, prefill::ROPE_PARTS), dim3(256), 0, s, c->pf_qkv, H, Hkv, HD, c->pf_cs, kc, vc, g.max_seq, t0);
             launch_chained(prefill::attn_prompt_kernel<HD>, dim3(H, (T + 63) / 64), dim3(128), prefill::attn_smem_bytes<HD>(), s, c->pf_qkv, H, Hkv, kc, vc, g.max_seq, t0, T, c->pf_aq, c->pf_aq + (size_t)cap * nq);
             ok = ok && contract(c->pf_aq, ly.wo, nullptr, d, nq, T, prefill::PF_ADD, c->pf_x, d, 0, nullptr, nullptr, 0,
-                                            err, s);
-            launch_chained(prefill::norm_split_kernel, dim3(T), dim3(256), 0, s, c->pf_x, d, ly.mlp_norm, g.rms_eps, c->pf_ad, c->pf_ad + (size_t)cap * d, c->pf_rinv);
+                                            err, s, nullptr, 0, 0, nullptr, nullptr, norm_next(ly.mlp_norm));
             ok = ok && contract(c->pf_ad, ly.w_gate, ly.w_up, F, d, T, prefill::PF_SWIGLU, nullptr, 0, 0, c->pf_af,
-                                            c->pf_af + (size_t)cap * F, F, err, s, nullptr, 0, 0, nullptr, nullptr, c->pf_rinv);
+                                            c->pf_af + (size_t)cap * F, F, err, s, nullptr, 0, 0, nullptr, nullptr, normed);
             ok = ok && contract(c->pf_af, ly.w_down, nullptr, d, F, T, prefill::PF_ADD, c->pf_x, d, 0, nullptr, nullptr,
-                                            0, err, s);
-            c->launches += heads_done ? 3 : 4;                   // besides the contractions
+                                            0, err, s, nullptr, 0, 0, nullptr, nullptr, l + 1 < g.n_layers ? norm_next(c->layers[l + 1].attn_norm) : prefill::Norms());
+            c->launches += heads_done ? 1 : 2;                   // besides the contractions
         }
         // pooled numerator: every row's final hidden state (mean pooling) or the last row's
         if (g.pool_mode == 0) {
@@ -1015,6 +1022,7 @@ knnssd_status knnssd_init(const knnssd_config *cfg, const knnssd_weights *w, con
             ok3 &= dev_alloc(&c->pf_qkv, n_proj > n_pool ? n_proj : n_pool) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_cs, cap * (hd / 2)) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_rinv, cap) == cudaSuccess;
+            ok3 &= dev_alloc(&c->pf_ss, cap * (d / 128)) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_ad, 2 * cap * d) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_aq, 2 * cap * nq) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_af, 2 * cap * g.d_ff) == cudaSuccess;

@@ -9,7 +9,7 @@
 //                       activation, so that the product with the bf16 weights carries 16 mantissa bits of A, as in
 //                       the decode passes), accumulator fp32.  Epilogues: store, add to the residual stream,
 //                       SwiGLU of a gate tile and an up tile.
-//   norm_split_kernel   RMSNorm of each row, written as the two bf16 planes the next map reads.
+//   norm_split_kernel   the embedding rows times the first gain, as the two bf16 planes the first map reads.
 //   fold_pieces_kernel  the sums of the tiles that a launch did in pieces, and their epilogue.
 //   rope_kv_rows_kernel rotary embedding of q and k, K/V rows rounded to bf16 into the cache, where the contraction's epilogue
 //                       has not done it.
@@ -47,7 +47,7 @@ __host__ __device__ constexpr int ring_stages(int tt) {
     return RING_BYTES / stage_bytes_of(tt) < MAX_STAGES ? RING_BYTES / stage_bytes_of(tt) : MAX_STAGES;
 }
 constexpr int TURN_TOKENS = 16;                       // tokens that a group of epilogue warps turns at a time (see below)
-constexpr int TURN_BYTES = 2 * 2 * TURN_TOKENS * 128 * 4;      // two groups, two buffers each
+constexpr int TURN_BYTES = 2 * 2 * TURN_TOKENS * 128 * 4 + 2 * 128 * 4;      // two groups: two buffers each, and the scales of their tokens
 constexpr int TMEM_COLS = 512;                        // columns of tensor memory a CTA takes: two accumulators of TT_MAX columns
 constexpr int CHUNK_KB = 8;                           // k-blocks accumulated in tensor memory before the sum moves to registers
 constexpr int GEMM_THREADS = 320;                     // warp 0: TMA; warp 1: MMA issue + tensor-memory owner; warps 2..9: epilogue
@@ -77,8 +77,16 @@ struct GemmArgs {
                        // gemm_split_kernel leaves and fold_pieces_kernel picks up
     int nA, nB;        // STORE over stacked matrices (q, k, v in one launch): units [0, nA) are rows of map tb0,
                        // [nA, nA + nB) rows of tb1, the rest rows of tb2; all multiples of BOX_N.  One matrix: nA = N
-    const float *row_scale;   // if given: every sum of row t is multiplied by row_scale[t] before the epilogue (the RMSNorm
-                              // scale of the row whose gain-weighted, un-normalised values the planes hold)
+    // If given: the sums of row t are multiplied, before the epilogue, by the RMSNorm scale of the row whose gain-weighted, un-normalised
+    // values the planes hold.  ss[slot * ss_rows + t] = the row's sum of squares over columns 128 slot .., K / 128 slots.
+    const float *ss;
+    int ss_rows;
+    float eps;
+    // ADD, if given: what the map that reads the new rows behind an RMSNorm needs of them: y times next_gain as two planes of row length
+    // N, and their sums of squares (N a multiple of 128)
+    const float *next_gain;
+    bf16_t *next_hi, *next_lo;
+    float *ss_out;
     // PF_QKV (stacked q, k, v; head dimension 128, so that a CTA's 128 weight rows are one head): the q heads are rotated
     // and stored to y, the k heads rotated, the k and v heads rounded to bf16 into the cache rows of position pos0 + t
     const float2 *rope;    // [T][64] (cos, sin) of the rows' positions
@@ -245,6 +253,14 @@ template <int EPI> __device__ __forceinline__ int first_unit(int ty, int rank) {
     return EPI == PF_SWIGLU ? ty * (PAIR_UNITS / 2) + 64 * rank : ty * PAIR_UNITS + 128 * rank;
 }
 
+// RMSNorm scale of row t.  The order of its sum is the same wherever it is taken.
+__device__ __forceinline__ float row_scale(const GemmArgs &g, int t) {
+    float s = 0.f;
+#pragma unroll 8
+    for (int i = 0; i < g.K / 128; ++i) s += __ldcg(g.ss + (size_t)i * g.ss_rows + t);
+    return 1.0f / sqrtf(s / (float)g.K + g.eps);
+}
+
 // ADD: the old values of token t that finish_sums takes for weight rows j .. j + 3 and j + 64 .. j + 67.
 template <int EPI> __device__ __forceinline__ void old_values(const GemmArgs &g, int u0, int t, int j, float4 (&x)[2]) {
 #pragma unroll
@@ -257,9 +273,10 @@ template <int EPI> __device__ __forceinline__ void old_values(const GemmArgs &g,
 // What becomes of the sums of token t for the weight rows j .. j + 3 (v[0 .. 3]) and j + 64 .. j + 67 (v[4 .. 7]) of a CTA whose
 // rows start at unit u0; j is a multiple of 4 below 64.  SwiGLU: gate and up of four units; q / k / v heads: four pairs of one
 // head; else units.  Products that meet a sum are rounded by themselves, whichever kernel this is part of.
-template <int EPI> __device__ __forceinline__ void finish_sums(const GemmArgs &g, int u0, int t, int j, float (&v)[8], const float4 (&x)[2]) {
-    if (g.row_scale) {
-        const float rs = g.row_scale[t];
+// rs: the row's scale (SwiGLU, q / k / v and store; 1: none).  ADD with next_gain: the 16 threads of a token, half a warp, call it
+// together.
+template <int EPI> __device__ __forceinline__ void finish_sums(const GemmArgs &g, int u0, int t, int j, float (&v)[8], const float4 (&x)[2], float rs) {
+    if (EPI != PF_ADD) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) v[i] = __fmul_rn(v[i], rs);
     }
@@ -306,6 +323,30 @@ template <int EPI> __device__ __forceinline__ void finish_sums(const GemmArgs &g
             float4 o = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
             if (EPI == PF_ADD) { o.x += x[e].x; o.y += x[e].y; o.z += x[e].z; o.w += x[e].w; }
             *reinterpret_cast<float4 *>(g.y + (size_t)t * g.ldy + g.col0 + u0 + j + 64 * e) = o;
+            if (EPI == PF_ADD) { v[4 * e] = o.x; v[4 * e + 1] = o.y; v[4 * e + 2] = o.z; v[4 * e + 3] = o.w; }
+        }
+        if (EPI == PF_ADD && g.next_gain && u0 < g.N) {
+            float ss = 0.f;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float4 gn = __ldg(reinterpret_cast<const float4 *>(g.next_gain + u0 + j + 64 * e));
+                const float w[4] = {gn.x, gn.y, gn.z, gn.w};
+                uint32_t h[4], l[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float a = __fmul_rn(v[4 * e + i], w[i]);
+                    ss = __fmaf_rn(v[4 * e + i], v[4 * e + i], ss);
+                    h[i] = float_to_bf16_rne(a);
+                    l[i] = float_to_bf16_rne(a - __uint_as_float(h[i] << 16));
+                }
+                const size_t at = (size_t)t * g.N + u0 + j + 64 * e;
+                *reinterpret_cast<uint2 *>(g.next_hi + at) = make_uint2(pack_bf16(h[0], h[1]), pack_bf16(h[2], h[3]));
+                *reinterpret_cast<uint2 *>(g.next_lo + at) = make_uint2(pack_bf16(l[0], l[1]), pack_bf16(l[2], l[3]));
+            }
+            const unsigned half_warp = 0xffffu << (threadIdx.x & 16);
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) ss += __shfl_xor_sync(half_warp, ss, o);
+            if (j == 0) g.ss_out[(size_t)(u0 >> 7) * g.ss_rows + t] = ss;
         }
     }
 }
@@ -469,6 +510,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant_
         const int q = warp & 3, hsel = (warp - 2) >> 2, row = 32 * q + lane, gt = (threadIdx.x - 64) & 127;
         const uint32_t trow = tmem + ((uint32_t)(32 * q) << 16);
         float *turn = reinterpret_cast<float *>(turn_smem) + hsel * (2 * TURN_TOKENS * 128);
+        float *scales = reinterpret_cast<float *>(turn_smem) + 2 * (2 * TURN_TOKENS * 128) + hsel * 128;
         const int f_tok = gt >> 4, f_j = 4 * (gt & 15);      // what this thread finishes: tokens f_tok and f_tok + 8 of 16, rows f_j ..
         bool ok = true;
         int cg = 0;                          // chunks taken so far, over all of this pair's jobs
@@ -476,6 +518,8 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant_
         for (int i = 0; jobs.get(i, tile, c_begin, c_end); ++i) {
             const int t0 = (tile % g.tiles_x) * tt + hsel * half;
             const bool piece = tile >= g.whole;
+            float own_scale = 1.0f;          // of the group's token gt, summed while the first chunk is under way
+            if (EPI != PF_ADD && g.ss && !piece && gt < half && t0 + gt < g.T) own_scale = row_scale(g, t0 + gt);
             float acc[128];
 #pragma unroll
             for (int e = 0; e < 128; ++e) acc[e] = 0.f;
@@ -512,6 +556,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant_
             ok = c_begin != 0;
             if (!ok) break;
             if (piece) continue;             // fold_pieces_kernel goes on from here
+            if (EPI != PF_ADD) scales[gt] = own_scale;       // the group is done with the job before
             const int u0 = first_unit<EPI>(tile / g.tiles_x, rank);
             float4 x[2][2];
             old_values<EPI>(g, u0, f_tok < half ? t0 + f_tok : g.T, f_j, x[0]);
@@ -536,7 +581,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant_
                     if (i0 + tok < half && t < g.T) {
                         const float4 lo = *reinterpret_cast<const float4 *>(buf + tok * 128 + f_j), hi = *reinterpret_cast<const float4 *>(buf + tok * 128 + 64 + f_j);
                         float v[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-                        finish_sums<EPI>(g, u0, t, f_j, v, x[e]);
+                        finish_sums<EPI>(g, u0, t, f_j, v, x[e], EPI != PF_ADD ? scales[i0 + tok] : 1.0f);
                     }
                     x[e][0] = next[e][0];
                     x[e][1] = next[e][1];
@@ -569,6 +614,7 @@ __global__ void __launch_bounds__(256) fold_pieces_kernel(const GemmArgs g) {
     const float4 *src = reinterpret_cast<const float4 *>(g.part + (((size_t)r * nchunks * 2 + rank) * g.tt + tok) * 128 + j);
     float4 x[2];
     old_values<EPI>(g, u0, t, j, x);
+    const float rs = EPI != PF_ADD && g.ss ? row_scale(g, t) : 1.0f;
     float v[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) v[e] = 0.f;
@@ -586,7 +632,7 @@ __global__ void __launch_bounds__(256) fold_pieces_kernel(const GemmArgs g) {
             for (int e = 0; e < 2; ++e)
                 if (c0 + c < nchunks) { v[4 * e] += p[c][e].x; v[4 * e + 1] += p[c][e].y; v[4 * e + 2] += p[c][e].z; v[4 * e + 3] += p[c][e].w; }
     }
-    finish_sums<EPI>(g, u0, t, j, v, x);
+    finish_sums<EPI>(g, u0, t, j, v, x, rs);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -606,22 +652,21 @@ __global__ void embed_rows_kernel(const bf16_t *__restrict__ table, const int *_
     }
 }
 
-// RMSNorm of row t (gain g, epsilon eps) for the contraction that follows: the planes hold v = x g WITHOUT the row's
-// scale, hi = bf16(v) and lo = bf16(v - hi), and rinv[t] = 1 / sqrt(mean(x^2) + eps) goes to the contraction's epilogue
-// (a linear map commutes with a per-row scale).  Same operands as the decode passes use: values that are exact in two
-// bf16 terms - embedding rows with unit gains - stay exact.  grid = T, 256 threads.
-__global__ void __launch_bounds__(256) norm_split_kernel(const float *__restrict__ x, int d, const float *__restrict__ gain, float eps,
-                                                         bf16_t *__restrict__ hi, bf16_t *__restrict__ lo, float *__restrict__ rinv_out) {
+// RMSNorm of row t (gain g) for the contraction that follows: the planes hold v = x g WITHOUT the row's scale, hi = bf16(v) and
+// lo = bf16(v - hi), and the row's sums of squares by 128 columns go to the contraction's epilogue (a linear map commutes with a per-row
+// scale).  Same operands as the decode passes use: values that are exact in two bf16 terms - embedding rows with unit gains -
+// stay exact.  For the embedding rows only: the maps that add to the residual stream leave the same for the rows they have changed
+// (as a launch of its own behind each of them it took 4.5 us at 77 rows, 10 at 1024).  grid = T, 256 threads; d a multiple of 128.
+__global__ void __launch_bounds__(256) norm_split_kernel(const float *__restrict__ x, int d, const float *__restrict__ gain, bf16_t *__restrict__ hi,
+                                                         bf16_t *__restrict__ lo, float *__restrict__ ss_out, int ss_rows) {
     chain_wait();
-    __shared__ float part[8];
     const float *xr = x + (size_t)blockIdx.x * d;
     bf16_t *hr = hi + (size_t)blockIdx.x * d, *lr = lo + (size_t)blockIdx.x * d;
-    float ss = 0.f;
-    // one walk over the row: the planes do not depend on the row's scale
-    for (int i = threadIdx.x * 4; i < d; i += 1024) {
+    for (int i = threadIdx.x * 4; i < d; i += 1024) {            // a warp has 128 columns
         const float4 v = *reinterpret_cast<const float4 *>(xr + i);
         const float4 g = *reinterpret_cast<const float4 *>(gain + i);
-        ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+        const float ss = warp_sum(v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w);
+        if ((threadIdx.x & 31) == 0) ss_out[(size_t)(i >> 7) * ss_rows + blockIdx.x] = ss;
         const float a[4] = {v.x * g.x, v.y * g.y, v.z * g.z, v.w * g.w};
         uint32_t h[4], l[4];
 #pragma unroll
@@ -631,15 +676,6 @@ __global__ void __launch_bounds__(256) norm_split_kernel(const float *__restrict
         }
         *reinterpret_cast<uint2 *>(hr + i) = make_uint2(pack_bf16(h[0], h[1]), pack_bf16(h[2], h[3]));
         *reinterpret_cast<uint2 *>(lr + i) = make_uint2(pack_bf16(l[0], l[1]), pack_bf16(l[2], l[3]));
-    }
-    ss = warp_sum(ss);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = ss;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float tot = 0.f;
-#pragma unroll
-        for (int w = 0; w < 8; ++w) tot += part[w];
-        rinv_out[blockIdx.x] = 1.0f / sqrtf(tot / (float)d + eps);
     }
 }
 
