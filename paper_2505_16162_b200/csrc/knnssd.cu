@@ -319,18 +319,27 @@ void ctx_linear(knnssd_ctx *c, const LinearArgs &a) {
 }
 
 // Rows are y blocks of the grid, at most 65535 per launch.
-void launch_filter(const float *logits, int rows, int V, float inv_t, float top_p, float *probs, cudaStream_t s) {
+template <int C> void launch_filter_t(const float *logits, int rows, int V, float inv_t, float top_p, float *probs, cudaStream_t s) {
     static bool configured[kMaxDevices] = {};          // function attributes are per device
     const int dev = current_device_slot();
     if (!configured[dev]) {
-        cudaFuncSetAttribute(sampling::filtered_probs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(float) * sampling::SLICE_MAX);
+        cudaFuncSetAttribute(sampling::filtered_probs_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(float) * sampling::SLICE_MAX);
+        if (C > 8) cudaFuncSetAttribute(sampling::filtered_probs_kernel<C>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         configured[dev] = true;
     }
     for (int r = 0; r < rows; r += 65535) {
         const int n = rows - r < 65535 ? rows - r : 65535;
-        sampling::filtered_probs_kernel<<<dim3(sampling::CL, n), sampling::NT, sampling::probs_smem(V), s>>>(
+        sampling::filtered_probs_kernel<C><<<dim3(C, n), sampling::NT, sampling::probs_smem(V, C), s>>>(
             logits + (size_t)r * V, V, inv_t, top_p, probs + (size_t)r * V);
     }
+}
+// Sixteen blocks per row for few long rows, and where eight have no room to keep values aside.  One row of 50000 / 65536 / 152064 ids:
+// 16.1 / 15.6 / 21.5 us against 16.8 / 18.1 / 29.7 with eight; nine rows of 152064 are two rounds of clusters of sixteen, 42.5 against
+// 29.8; 300000 ids 31 against 153, 48 rows of them 240 against 630.
+constexpr int kWideFilterVocab = 65536, kWideFilterRows = 5;
+void launch_filter(const float *logits, int rows, int V, float inv_t, float top_p, float *probs, cudaStream_t s) {
+    if ((V >= kWideFilterVocab && rows <= kWideFilterRows) || V > sampling::CL * (sampling::SLICE_MAX / 2)) launch_filter_t<sampling::CL_WIDE>(logits, rows, V, inv_t, top_p, probs, s);
+    else launch_filter_t<sampling::CL>(logits, rows, V, inv_t, top_p, probs, s);
 }
 
 LinearArgs make_args(const void *W0, int rows0, int n_in, const float *x, const float *gain, float eps, float *y,

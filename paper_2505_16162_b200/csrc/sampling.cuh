@@ -23,21 +23,25 @@ namespace cg = cooperative_groups;
 
 constexpr int NT = 512;                    // at 1024 the meetings take twice as long (32 sums per warp to add up), at 256 long rows do
 constexpr int NW = NT / 32;
-constexpr int CL = 8;                      // blocks per row
+constexpr int CL = 8;                      // blocks per row; the filter takes CL_WIDE for long rows
+constexpr int CL_WIDE = 16;
 constexpr int NS = 32;                     // sums that one meeting adds up: one per lane, and per warp
 constexpr int SLICE_MAX = 49152;           // ids per block that fit in shared memory (192 KB)
 
 // Meeting place of the blocks of a row.  `slot` alternates: a block may still read the last meeting's sums while another
 // already writes the next one's.
-struct Meet {
+template <int C> struct MeetOf {
+    static constexpr int BLOCKS = C;
     float red[NW][NS + 1];
-    float slot[2][CL][NS];
+    float slot[2][C][NS];
 };
+typedef MeetOf<CL> Meet;
 
 // Sum (MAX: maximum of v[0]) over the threads of all blocks; lane j of every warp gets sum j, added in a fixed
 // order: lanes, warps, blocks.  `turn` counts the meetings.
-template <bool MAX>
-__device__ __forceinline__ float meet(Meet &sh, int &turn, float (&v)[NS]) {
+template <bool MAX, typename M>
+__device__ __forceinline__ float meet(M &sh, int &turn, float (&v)[NS]) {
+    constexpr int CL = M::BLOCKS;
     cg::cluster_group cluster = cg::this_cluster();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, par = turn & 1;
     ++turn;
@@ -93,10 +97,10 @@ __device__ __forceinline__ int block_count(int v, int *sh) {
 }
 
 // Ids per block of a row of V: [rank S, rank S + S).
-__host__ __device__ __forceinline__ int slice_len(int V) { return (V + CL - 1) / CL; }
+__host__ __device__ __forceinline__ int slice_len(int V, int blocks = CL) { return (V + blocks - 1) / blocks; }
 // Shared memory of filtered_probs_kernel: the slice's values and, where it fits as well, the candidates among them.
-inline size_t probs_smem(int V) {
-    const size_t S = slice_len(V), padded = (S + NT - 1) / NT * NT;
+inline size_t probs_smem(int V, int blocks) {
+    const size_t S = slice_len(V, blocks), padded = (S + NT - 1) / NT * NT;
     return sizeof(float) * (S + padded <= SLICE_MAX ? S + padded : S <= SLICE_MAX ? S : 0);
 }
 
@@ -105,17 +109,23 @@ inline size_t probs_smem(int V) {
 // The mass above a value is a decreasing step function of the value, so the smallest kept probability x0 is found in
 // the bit patterns of positive floats, 32 candidates at a time (five bits per pass; one candidate per pass, by one block
 // that re-read its row from L2 each time, took 65 us for 5 rows of 32000 and 241 us for one of 152064; this takes 20 and 35).  The first pass leaves
-// a few per cent of the values between its bounds; a thread keeps those of its own aside for the others.
+// a few per cent of the values between its bounds; a thread keeps those of its own aside for the others.  Once no block has more than
+// GATHER values left between the bounds all blocks get them all, and each finds x0 for itself: a meeting instead of five.
 // Tokens whose probability equals x0 are ranked by id.
-// grid = (CL, rows), NT threads, probs_smem(V) of shared memory; rows too long for it keep their values in `probs`.
-__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT)
+// grid = (C, rows), NT threads, probs_smem(V, C) of shared memory; rows too long for it keep their values in `probs`.
+constexpr int GATHER = 32;
+template <int C> __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(NT)
 filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_temperature, float top_p, float *__restrict__ probs) {
     extern __shared__ float probs_slice[];
-    __shared__ Meet sh;
+    __shared__ MeetOf<C> sh;
     __shared__ int shi[NW];
     __shared__ int s_cut;
+    __shared__ float left[C][GATHER];                            // the blocks' values between the bounds
+    __shared__ int n_left[C];
+    __shared__ unsigned s_x0;
+    constexpr int CL = C;
     cg::cluster_group cluster = cg::this_cluster();
-    const int S = slice_len(V), rank = (int)cluster.block_rank(), tid = threadIdx.x;
+    const int S = slice_len(V, C), rank = (int)cluster.block_rank(), tid = threadIdx.x;
     const int id0 = min(V, rank * S), n = min(V, id0 + S) - id0;
     const float *l = logits + (size_t)blockIdx.y * V + id0;
     float *out = probs + (size_t)blockIdx.y * V + id0;
@@ -146,6 +156,8 @@ filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_tempera
     float *list = S + (S + NT - 1) / NT * NT <= SLICE_MAX ? probs_slice + S + tid : nullptr;
     int n_list = 0;
     float above = 0.f;                                           // this thread's values that lie above all candidates
+    float above_hi = 0.f;                                        // all threads' values above hi
+    int gathered = -1;                                           // values between the bounds, once all blocks have them
     for (bool first = true; first || hi > lo + 1u; first = false) {
         const unsigned step = (hi - lo + NS - 1) / NS;           // candidates lo, lo + step, ..: lo itself only counts in the first pass
         float x[NS];
@@ -153,18 +165,24 @@ filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_tempera
         for (int j = 0; j < NS; ++j) { v[j] = above; x[j] = __uint_as_float(min(hi, lo + j * step)); }
         const bool listed = list && !first;
         const float *src = listed ? list : p + tid;
-        for (int i = 0, m_own = listed ? n_list : (n - tid + NT - 1) / NT; i < m_own; ++i) {
-            const float y = src[i * NT];
+        const int m_own = listed ? n_list : (n - tid + NT - 1) / NT;
+        for (int i0 = 0; i0 < m_own; i0 += 4) {                  // four loads in flight: rows too long for shared memory come from L2
+            float y[4];
 #pragma unroll
-            for (int j = 0; j < NS; ++j) v[j] += y > x[j] ? y : 0.f;
+            for (int e = 0; e < 4; ++e) y[e] = i0 + e < m_own ? src[(i0 + e) * NT] : 0.f;
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+#pragma unroll
+                for (int j = 0; j < NS; ++j) v[j] += y[e] > x[j] ? y[e] : 0.f;
         }
         const float mass = meet<false>(sh, turn, v);
         const unsigned below = __ballot_sync(0xffffffffu, mass < top_p);
         int j = below ? __ffs(below) - 1 : NS;                   // the first candidate with less than top_p above it
         if (j == 0) {
-            if (first) { hi = lo; break; }
+            if (first) { hi = lo; above_hi = __shfl_sync(0xffffffffu, mass, 0); break; }
             j = 1;                                               // lo was ruled out before, by sums in another order
         }
+        if (j < NS && lo + j * step < hi) above_hi = __shfl_sync(0xffffffffu, mass, j);
         const unsigned nhi = j < NS ? min(hi, lo + j * step) : hi;
         lo = min(hi, lo + (j - 1) * step);
         hi = nhi;
@@ -175,21 +193,79 @@ filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_tempera
                 if (y > xh) above += y;
                 else if (y > xl) list[NT * n_list++] = y;
             }
+        } else if (list && hi > lo + 1u) {
+            // hand the values left to all blocks, in the order of blocks, threads and each thread's list
+            const float xl = __uint_as_float(lo), xh = __uint_as_float(hi);
+            int own = 0;
+            for (int i = 0; i < n_list; ++i) { const float y = list[NT * i]; own += y > xl && y <= xh ? 1 : 0; }
+            const int lane = tid & 31, warp = tid >> 5;
+            int upto = own;                                      // of the warp's lanes up to this one
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xffffffffu, upto, o); if (lane >= o) upto += t; }
+            if (lane == 31) shi[warp] = upto;
+            __syncthreads();
+            int before = 0, all = 0;
+#pragma unroll
+            for (int w = 0; w < NW; ++w) { if (w == warp) before = all; all += shi[w]; }
+            int at = before + upto - own;
+            for (int i = 0; i < n_list; ++i) {
+                const float y = list[NT * i];
+                if (y > xl && y <= xh) { if (at < GATHER) left[rank][at] = y; ++at; }
+            }
+            __syncthreads();
+            for (int t = tid; t < C * GATHER; t += NT) {
+                const int r = t / GATHER, i = t % GATHER;
+                if (r != rank && i < min(all, GATHER)) *cluster.map_shared_rank(&left[rank][i], r) = left[rank][i];
+                if (i == 0) *cluster.map_shared_rank(&n_left[rank], r) = all;
+            }
+            cluster.sync();
+            int most = 0, total = 0;
+#pragma unroll
+            for (int r = 0; r < C; ++r) { most = max(most, n_left[r]); total += n_left[r]; }
+            if (most <= GATHER) { gathered = total; break; }
+            cluster.sync();                                      // nobody writes the next values while others read these counts
         }
     }
-    const float x0 = __uint_as_float(hi);
-    // tokens at exactly x0: the n-th of them by id (n = 0, 1, ..) is kept iff mass above x0 + n x0 < top_p
+    float x0 = __uint_as_float(hi);
+    float a0 = above_hi;                                         // mass above x0
+    int c = 0, own_c = 0;                                        // tokens at x0: of all blocks, and this thread's share of its block's
+    if (gathered >= 0) {
+        // the smallest of the values left with less than top_p above it; if rounding has it that there is none, hi
+        if (tid == 0) s_x0 = hi;
+        __syncthreads();
+        for (int t = tid; t < C * GATHER; t += NT) {
+            const int r = t / GATHER, i = t % GATHER;
+            if (i < n_left[r]) {
+                const float y = left[r][i];
+                float m_above = above_hi;
+                for (int q = 0; q < C; ++q)
+                    for (int e = 0, n_q = n_left[q]; e < n_q; ++e) { const float o = left[q][e]; m_above += o > y ? o : 0.f; }
+                if (m_above < top_p) atomicMin(&s_x0, __float_as_uint(y));
+            }
+        }
+        __syncthreads();
+        x0 = __uint_as_float(s_x0);
+        for (int q = 0; q < C; ++q)
+            for (int e = 0, n_q = n_left[q]; e < n_q; ++e) {
+                const float o = left[q][e];
+                a0 += o > x0 ? o : 0.f;
+                if (o == x0) { ++c; own_c += q == rank && tid == 0 ? 1 : 0; }
+            }
+    } else {
+        // rows whose values are not kept aside, and bounds that met without it
 #pragma unroll
-    for (int j = 0; j < NS; ++j) v[j] = 0.f;
-    for (int i = tid; i < n; i += NT) {
-        const float y = p[i];
-        v[0] += y > x0 ? y : 0.f;
-        if (y == x0) v[1] += 1.f;                                // counts are exact up to 2^24 tokens
+        for (int j = 0; j < NS; ++j) v[j] = 0.f;
+        for (int i = tid; i < n; i += NT) {
+            const float y = p[i];
+            v[0] += y > x0 ? y : 0.f;
+            if (y == x0) v[1] += 1.f;                            // counts are exact up to 2^24 tokens
+        }
+        own_c = (int)v[1];
+        const float tot = meet<false>(sh, turn, v);
+        a0 = __shfl_sync(0xffffffffu, tot, 0);
+        c = (int)__shfl_sync(0xffffffffu, tot, 1);
     }
-    const float own_c = v[1];
-    float tot = meet<false>(sh, turn, v);
-    const float a0 = __shfl_sync(0xffffffffu, tot, 0);
-    const int c = (int)__shfl_sync(0xffffffffu, tot, 1);
+    // tokens at exactly x0: the n-th of them by id (n = 0, 1, ..) is kept iff mass above x0 + n x0 < top_p
     int nk = 1, id_cut = V;                                      // tokens at x0 with id < id_cut are kept; the first one always is
     if (c > 1) {
         nk = 0;
@@ -198,8 +274,8 @@ filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_tempera
         if (nk < c) {                                            // which of them: the block that has the nk-th looks for its id
             // sum r of this meeting: the tokens at x0 in block r
 #pragma unroll
-            for (int j = 0; j < NS; ++j) v[j] = j == rank ? own_c : 0.f;
-            tot = meet<false>(sh, turn, v);
+            for (int j = 0; j < NS; ++j) v[j] = j == rank ? (float)own_c : 0.f;
+            const float tot = meet<false>(sh, turn, v);
             int before = 0, holder = 0;
             for (int r = 0; r < CL; ++r) {
                 const int cr = (int)__shfl_sync(0xffffffffu, tot, r);
