@@ -237,20 +237,22 @@ filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_tempera
             const int r = t / GATHER, i = t % GATHER;
             if (i < n_left[r]) {
                 const float y = left[r][i];
-                float m_above = above_hi;
+                float m_above = 0.f;                             // the few small values by themselves, then one rounding at the size of the mass
                 for (int q = 0; q < C; ++q)
                     for (int e = 0, n_q = n_left[q]; e < n_q; ++e) { const float o = left[q][e]; m_above += o > y ? o : 0.f; }
-                if (m_above < top_p) atomicMin(&s_x0, __float_as_uint(y));
+                if (above_hi + m_above < top_p) atomicMin(&s_x0, __float_as_uint(y));
             }
         }
         __syncthreads();
         x0 = __uint_as_float(s_x0);
+        float left_above = 0.f;
         for (int q = 0; q < C; ++q)
             for (int e = 0, n_q = n_left[q]; e < n_q; ++e) {
                 const float o = left[q][e];
-                a0 += o > x0 ? o : 0.f;
+                left_above += o > x0 ? o : 0.f;
                 if (o == x0) { ++c; own_c += q == rank && tid == 0 ? 1 : 0; }
             }
+        a0 = above_hi + left_above;
     } else {
         // rows whose values are not kept aside, and bounds that met without it
 #pragma unroll
