@@ -30,6 +30,8 @@
  *
  * Session protocol:  init -> prefill -> (select_skipset | set_skipmask)
  *                    -> { draft -> verify }* ;  generate = all of it for one request.
+ * Calls that enqueue work for a session wait for it or, where they say so, leave it in stream order.  They cannot be recorded: while
+ * the context's stream is being captured they return KNNSSD_ERR_CUDA, and neither the session nor the capture has changed.
  */
 #ifndef KNNSSD_H
 #define KNNSSD_H
@@ -181,7 +183,7 @@ long long knnssd_get_launch_count(const knnssd_ctx *ctx);
 /* Committed context length (positions whose K/V are valid), and explicit rollback to a shorter length
  * (new_len <= current length; the pending token is unchanged, so this is meant for tests and benchmarks).
  * knnssd_set_length and knnssd_set_pending are asynchronous: the new value is enqueued on the context's stream, and a failure of
- * the device is reported by the next call that waits.  Both are refused (KNNSSD_ERR_CUDA) while the stream is being captured. */
+ * the device is reported by the next call that waits. */
 int knnssd_get_length(const knnssd_ctx *ctx);
 knnssd_status knnssd_set_length(knnssd_ctx *ctx, int new_len);
 

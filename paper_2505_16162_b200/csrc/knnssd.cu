@@ -627,16 +627,24 @@ knnssd_status sync_check(knnssd_ctx *c, const char *what) {
     return KNNSSD_OK;
 }
 
-// A word of the session's state, written in stream order without waiting.  Refused while the stream is being captured, as
-// every call that changes the session is: the host's copy of the state would run ahead of the device's.
-knnssd_status set_word(knnssd_ctx *c, int *word, int value, const char *what) {
+// Calls that change the session are refused, before anything on the host has moved, while its stream is being captured: their launches
+// would be recorded and not run, and the host's copy of the state (length, barrier counts, which counter a pass meets at) would run
+// ahead of the device's.
+knnssd_status refuse_capture(knnssd_ctx *c, const char *what) {
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(c->stream, &capturing);
     if (e == cudaSuccess && capturing != cudaStreamCaptureStatusNone) e = cudaErrorStreamCaptureUnsupported;
-    if (e == cudaSuccess) {
-        set_word_kernel<<<1, 1, 0, c->stream>>>(word, value);
-        e = cudaGetLastError();
-    }
+    if (e == cudaSuccess) return KNNSSD_OK;
+    cudaGetLastError();
+    return fail(c, KNNSSD_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
+}
+
+// A word of the session's state, written in stream order without waiting.
+knnssd_status set_word(knnssd_ctx *c, int *word, int value, const char *what) {
+    const knnssd_status st = refuse_capture(c, what);
+    if (st != KNNSSD_OK) return st;
+    set_word_kernel<<<1, 1, 0, c->stream>>>(word, value);
+    const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? KNNSSD_OK : fail(c, KNNSSD_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
@@ -795,6 +803,7 @@ knnssd_status do_prefill(knnssd_ctx *c, const int *tokens_host, int n, float *po
     for (int i = 0; i < n; ++i)
         if (tokens_host[i] < 0 || tokens_host[i] >= g.vocab)
             return fail(c, KNNSSD_ERR_INVALID_ARG, "prefill: token id out of range");
+    if (knnssd_status r = refuse_capture(c, "prefill"); r != KNNSSD_OK) return r;
     cudaStream_t s = c->stream;
     c->prefilled = false;
     CUDA_TRY(c, cudaMemcpyAsync(c->prompt, tokens_host, sizeof(int) * n, cudaMemcpyHostToDevice, s));
@@ -842,6 +851,7 @@ knnssd_status do_select(knnssd_ctx *c, const float *query_dev, int *domain, int 
     const knnssd_config &g = c->cfg;
     if (g.n_domains <= 0) return fail(c, KNNSSD_ERR_STATE, "select_skipset: the context has no anchors");
     if (!query_dev && !c->prefilled) return fail(c, KNNSSD_ERR_STATE, "select_skipset: no pooled vector (prefill first)");
+    if (knnssd_status r = refuse_capture(c, "select_skipset"); r != KNNSSD_OK) return r;
     const int n = g.n_domains * g.anchors_per_domain;
     cudaStream_t s = c->stream;
     cudaEventRecord(c->ev0, s);
@@ -1112,6 +1122,7 @@ knnssd_status knnssd_draft(knnssd_ctx *c, int k, int *draft_tokens_host, float *
     if (!c->prefilled) return fail(c, KNNSSD_ERR_STATE, "draft: prefill first");
     if (!c->has_mask) return fail(c, KNNSSD_ERR_STATE, "draft: no active skip mask (select_skipset or set_skipmask first)");
     if (c->len + k + 1 > c->cfg.max_seq) return fail(c, KNNSSD_ERR_CAPACITY, "draft: len + k + 1 exceeds max_seq");
+    if (knnssd_status r = refuse_capture(c, "draft"); r != KNNSSD_OK) return r;
     cudaStream_t s = c->stream;
     cudaEventRecord(c->ev0, s);
     for (int j = 0; j < k; ++j) {
@@ -1142,6 +1153,7 @@ knnssd_status knnssd_verify(knnssd_ctx *c, const int *draft_tokens_host, int k, 
     for (int j = 0; j < k; ++j)
         if (draft_tokens_host[j] < 0 || draft_tokens_host[j] >= g.vocab)
             return fail(c, KNNSSD_ERR_INVALID_ARG, "verify: draft token id out of range");
+    if (knnssd_status r = refuse_capture(c, "verify"); r != KNNSSD_OK) return r;
     cudaStream_t s = c->stream;
     if (k > 0) {
         Tokens t{};
@@ -1183,6 +1195,7 @@ static knnssd_status do_decode(knnssd_ctx *c, int max_new, int k, int use_select
     if (c->len + max_new + 1 > g.max_seq) return fail(c, KNNSSD_ERR_CAPACITY, "decode: length + max_new + 1 exceeds max_seq");
     const bool select = use_selection && g.n_domains > 0;
     if (!select && !c->has_mask) return fail(c, KNNSSD_ERR_STATE, "decode: no active skip mask and no selection");
+    if (knnssd_status r = refuse_capture(c, "decode"); r != KNNSSD_OK) return r;
     knnssd_status st;
     int domain = -1;
     if (select) {
@@ -1261,6 +1274,7 @@ knnssd_status knnssd_decode_sampled(knnssd_ctx *c, int max_new, int k, float tem
     if (!c->prefilled) return fail(c, KNNSSD_ERR_STATE, "decode_sampled: prefill first");
     if (!c->has_mask) return fail(c, KNNSSD_ERR_STATE, "decode_sampled: no active skip mask");
     if (c->len + max_new + 1 > g.max_seq) return fail(c, KNNSSD_ERR_CAPACITY, "decode_sampled: length + max_new + 1 exceeds max_seq");
+    if (knnssd_status r = refuse_capture(c, "decode_sampled"); r != KNNSSD_OK) return r;
     const size_t V = (size_t)g.vocab;
     if (!c->samp_p) {
         if (dev_alloc(&c->samp_p, (size_t)kMaxRows * V) != cudaSuccess || dev_alloc(&c->samp_q, (size_t)kMaxRows * V) != cudaSuccess ||
@@ -1445,6 +1459,7 @@ knnssd_status knnssd_time_pass(knnssd_ctx *c, int which, int k, int iters, float
     if (!c->prefilled) return fail(c, KNNSSD_ERR_STATE, "time_pass: prefill first");
     if (which == 0 && !c->has_mask) return fail(c, KNNSSD_ERR_STATE, "time_pass: no active skip mask");
     if (c->len + k + 1 > g.max_seq) return fail(c, KNNSSD_ERR_CAPACITY, "time_pass: len + k + 1 exceeds max_seq");
+    if (knnssd_status r = refuse_capture(c, "time_pass"); r != KNNSSD_OK) return r;
     cudaStream_t s = c->stream;
     // the chain must hold valid token ids for the rows a verify pass reads
     std::vector<int> fill(k + 1, c->pending);
@@ -1497,6 +1512,7 @@ knnssd_status knnssd_trace_pass(knnssd_ctx *c, int which, int k, int cap, int *o
     if (!c->prefilled) return fail(c, KNNSSD_ERR_STATE, "trace_pass: prefill first");
     if (which == 0 && !c->has_mask) return fail(c, KNNSSD_ERR_STATE, "trace_pass: no active skip mask");
     if (c->len + k + 1 > g.max_seq) return fail(c, KNNSSD_ERR_CAPACITY, "trace_pass: len + k + 1 exceeds max_seq");
+    if (knnssd_status r = refuse_capture(c, "trace_pass"); r != KNNSSD_OK) return r;
     cudaStream_t s = c->stream;
     std::vector<int> fill(k + 1, c->pending);
     CUDA_TRY(c, cudaMemcpyAsync(c->chain, fill.data(), sizeof(int) * (k + 1), cudaMemcpyHostToDevice, s));
@@ -1544,6 +1560,7 @@ knnssd_status knnssd_debug_barrier_timeout(knnssd_ctx *c, unsigned spin_limit) {
     DeviceGuard dg(c->device);
     if (spin_limit < 1 || spin_limit > 1000000u) return fail(c, KNNSSD_ERR_INVALID_ARG, "debug_barrier_timeout: spin_limit must be 1..1000000");
     if (!c->mega_ok) return fail(c, KNNSSD_ERR_SHAPE, "debug_barrier_timeout: this model does not run in the persistent kernel");
+    if (knnssd_status r = refuse_capture(c, "debug_barrier_timeout"); r != KNNSSD_OK) return r;
     // an operation list holding just the embedding (no linear map: the producer warp issues no copy) whose barrier
     // waits for one more round of arrivals than there are CTAs; every CTA runs out of polls, raises the abort word and
     // falls through to the end of the kernel
