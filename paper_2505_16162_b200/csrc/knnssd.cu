@@ -96,7 +96,7 @@ struct knnssd_ctx {
     float *pf_x = nullptr, *pf_qkv = nullptr;                // residual stream [cap][d]; q, k, v [cap][nq + 2 nkv]
     float2 *pf_cs = nullptr;                                 // rotary (cos, sin) of the chunk's rows [cap][hd / 2]
     float *pf_rinv = nullptr;                                // RMSNorm scale of the chunk's rows [cap]
-    float *pf_ss = nullptr;                                  // their sums of squares by 128 columns [d / 128][cap]
+    float *pf_ss = nullptr;                                  // their sums of squares by four columns [cap][d / 4]
     bf16_t *pf_ad = nullptr, *pf_aq = nullptr, *pf_af = nullptr;   // hi / lo planes [2][cap][d], [2][cap][nq], [2][cap][d_ff]
     float *pf_part = nullptr;                                // sums of the pieces of tiles that several CTAs share
 
@@ -736,14 +736,18 @@ bool prefill_tensor(knnssd_ctx *c, int n) {
         const bool last = t0 + T == n;
         prefill::embed_rows_kernel<<<T, 256, 0, s>>>(reinterpret_cast<const bf16_t *>(c->tok_embed), c->prompt + t0, d, c->pf_x);
         prefill::rope_table_kernel<<<T, HD / 2, 0, s>>>(c->inv_freq, t0, c->pf_cs);
-        launch_chained(prefill::norm_split_kernel, dim3(T), dim3(256), 0, s, c->pf_x, d, c->layers[0].attn_norm, c->pf_ad, c->pf_ad + (size_t)cap * d, c->pf_ss, cap);
+        launch_chained(prefill::norm_split_kernel, dim3(T), dim3(256), 0, s, c->pf_x, d, c->layers[0].attn_norm, g.rms_eps, c->pf_ad, c->pf_ad + (size_t)cap * d, c->pf_rinv);
         c->launches += 3;
         prefill::Norms normed;                       // of the rows a map reads, and below of those it has added to
-        normed.ss = c->pf_ss; normed.rows = cap; normed.eps = g.rms_eps;
+        normed.row_scale = c->pf_rinv;
         auto norm_next = [&](const float *gain) {
             prefill::Norms n;
-            n.rows = cap; n.next_gain = gain; n.next_hi = c->pf_ad; n.next_lo = c->pf_ad + (size_t)cap * d; n.ss_out = c->pf_ss;
+            n.next_gain = gain; n.next_hi = c->pf_ad; n.next_lo = c->pf_ad + (size_t)cap * d; n.ss_out = c->pf_ss;
             return n;
+        };
+        auto scales = [&]() {
+            launch_chained(prefill::scales_kernel, dim3(T), dim3(256), 0, s, c->pf_ss, d, g.rms_eps, c->pf_rinv);
+            c->launches++;
         };
         for (int l = 0; l < g.n_layers && ok; ++l) {
             const Layer &ly = c->layers[l];
@@ -767,10 +771,12 @@ bool prefill_tensor(knnssd_ctx *c, int n) {
             launch_chained(prefill::attn_prompt_kernel<HD>, dim3(H, (T + 63) / 64), dim3(128), prefill::attn_smem_bytes<HD>(), s, c->pf_qkv, H, Hkv, kc, vc, g.max_seq, t0, T, c->pf_aq, c->pf_aq + (size_t)cap * nq);
             ok = ok && contract(c->pf_aq, ly.wo, nullptr, d, nq, T, prefill::PF_ADD, c->pf_x, d, 0, nullptr, nullptr, 0,
                                             err, s, nullptr, 0, 0, nullptr, nullptr, norm_next(ly.mlp_norm));
+            scales();
             ok = ok && contract(c->pf_ad, ly.w_gate, ly.w_up, F, d, T, prefill::PF_SWIGLU, nullptr, 0, 0, c->pf_af,
                                             c->pf_af + (size_t)cap * F, F, err, s, nullptr, 0, 0, nullptr, nullptr, normed);
             ok = ok && contract(c->pf_af, ly.w_down, nullptr, d, F, T, prefill::PF_ADD, c->pf_x, d, 0, nullptr, nullptr,
                                             0, err, s, nullptr, 0, 0, nullptr, nullptr, l + 1 < g.n_layers ? norm_next(c->layers[l + 1].attn_norm) : prefill::Norms());
+            if (l + 1 < g.n_layers) scales();
             c->launches += heads_done ? 1 : 2;                   // besides the contractions
         }
         // pooled numerator: every row's final hidden state (mean pooling) or the last row's
@@ -1041,7 +1047,7 @@ knnssd_status knnssd_init(const knnssd_config *cfg, const knnssd_weights *w, con
             ok3 &= dev_alloc(&c->pf_qkv, n_proj > n_pool ? n_proj : n_pool) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_cs, cap * (hd / 2)) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_rinv, cap) == cudaSuccess;
-            ok3 &= dev_alloc(&c->pf_ss, cap * (d / 128)) == cudaSuccess;
+            ok3 &= dev_alloc(&c->pf_ss, cap * (d / 4)) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_ad, 2 * cap * d) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_aq, 2 * cap * nq) == cudaSuccess;
             ok3 &= dev_alloc(&c->pf_af, 2 * cap * g.d_ff) == cudaSuccess;

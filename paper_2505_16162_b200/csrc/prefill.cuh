@@ -9,7 +9,8 @@
 //                       activation, so that the product with the bf16 weights carries 16 mantissa bits of A, as in
 //                       the decode passes), accumulator fp32.  Epilogues: store, add to the residual stream,
 //                       SwiGLU of a gate tile and an up tile.
-//   norm_split_kernel   the embedding rows times the first gain, as the two bf16 planes the first map reads.
+//   norm_split_kernel   the embedding rows times the first gain, as the two bf16 planes the first map reads, and their RMSNorm scales.
+//   scales_kernel       the RMSNorm scales of rows that a map has added to.
 //   fold_pieces_kernel  the sums of the tiles that a launch did in pieces, and their epilogue.
 //   rope_kv_rows_kernel rotary embedding of q and k, K/V rows rounded to bf16 into the cache, where the contraction's epilogue
 //                       has not done it.
@@ -77,13 +78,10 @@ struct GemmArgs {
                        // gemm_split_kernel leaves and fold_pieces_kernel picks up
     int nA, nB;        // STORE over stacked matrices (q, k, v in one launch): units [0, nA) are rows of map tb0,
                        // [nA, nA + nB) rows of tb1, the rest rows of tb2; all multiples of BOX_N.  One matrix: nA = N
-    // If given: the sums of row t are multiplied, before the epilogue, by the RMSNorm scale of the row whose gain-weighted, un-normalised
-    // values the planes hold.  ss[slot * ss_rows + t] = the row's sum of squares over columns 128 slot .., K / 128 slots.
-    const float *ss;
-    int ss_rows;
-    float eps;
+    const float *row_scale;   // if given: every sum of row t is multiplied by row_scale[t] before the epilogue (the RMSNorm
+                              // scale of the row whose gain-weighted, un-normalised values the planes hold)
     // ADD, if given: what the map that reads the new rows behind an RMSNorm needs of them: y times next_gain as two planes of row length
-    // N, and their sums of squares (N a multiple of 128)
+    // N, and the sums of squares of every four of their columns, [t][N / 4] (N a multiple of 128)
     const float *next_gain;
     bf16_t *next_hi, *next_lo;
     float *ss_out;
@@ -253,12 +251,26 @@ template <int EPI> __device__ __forceinline__ int first_unit(int ty, int rank) {
     return EPI == PF_SWIGLU ? ty * (PAIR_UNITS / 2) + 64 * rank : ty * PAIR_UNITS + 128 * rank;
 }
 
-// RMSNorm scale of row t.  The order of its sum is the same wherever it is taken.
-__device__ __forceinline__ float row_scale(const GemmArgs &g, int t) {
-    float s = 0.f;
-#pragma unroll 8
-    for (int i = 0; i < g.K / 128; ++i) s += __ldcg(g.ss + (size_t)i * g.ss_rows + t);
-    return 1.0f / sqrtf(s / (float)g.K + g.eps);
+// The sum of four squares, as one order of roundings wherever it is taken.
+__device__ __forceinline__ float squares(float a, float b, float c, float d) {
+    return __fmaf_rn(d, d, __fmaf_rn(c, c, __fmaf_rn(a, a, __fmul_rn(b, b))));
+}
+// v = x g in two bf16 terms.
+__device__ __forceinline__ void split_product(float x, float g, uint32_t &hi, uint32_t &lo) {
+    const float v = __fmul_rn(x, g);
+    hi = float_to_bf16_rne(v);
+    lo = float_to_bf16_rne(v - __uint_as_float(hi << 16));
+}
+// RMSNorm's scale of a row.  ss: the squares of the columns 4 tid .. 4 tid + 3, 1024 further and so on, added up by 256 threads; here lanes and
+// then warps are.
+__device__ __forceinline__ float scale_of_row(float ss, float *part, int d, float eps) {
+    ss = warp_sum(ss);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = ss;
+    __syncthreads();
+    float tot = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) tot += part[w];
+    return 1.0f / sqrtf(tot / (float)d + eps);
 }
 
 // ADD: the old values of token t that finish_sums takes for weight rows j .. j + 3 and j + 64 .. j + 67.
@@ -273,8 +285,7 @@ template <int EPI> __device__ __forceinline__ void old_values(const GemmArgs &g,
 // What becomes of the sums of token t for the weight rows j .. j + 3 (v[0 .. 3]) and j + 64 .. j + 67 (v[4 .. 7]) of a CTA whose
 // rows start at unit u0; j is a multiple of 4 below 64.  SwiGLU: gate and up of four units; q / k / v heads: four pairs of one
 // head; else units.  Products that meet a sum are rounded by themselves, whichever kernel this is part of.
-// rs: the row's scale (SwiGLU, q / k / v and store; 1: none).  ADD with next_gain: the 16 threads of a token, half a warp, call it
-// together.
+// rs: the row's scale (SwiGLU, q / k / v and store; 1: none).
 template <int EPI> __device__ __forceinline__ void finish_sums(const GemmArgs &g, int u0, int t, int j, float (&v)[8], const float4 (&x)[2], float rs) {
     if (EPI != PF_ADD) {
 #pragma unroll
@@ -326,27 +337,18 @@ template <int EPI> __device__ __forceinline__ void finish_sums(const GemmArgs &g
             if (EPI == PF_ADD) { v[4 * e] = o.x; v[4 * e + 1] = o.y; v[4 * e + 2] = o.z; v[4 * e + 3] = o.w; }
         }
         if (EPI == PF_ADD && g.next_gain && u0 < g.N) {
-            float ss = 0.f;
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
                 const float4 gn = __ldg(reinterpret_cast<const float4 *>(g.next_gain + u0 + j + 64 * e));
                 const float w[4] = {gn.x, gn.y, gn.z, gn.w};
                 uint32_t h[4], l[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float a = __fmul_rn(v[4 * e + i], w[i]);
-                    ss = __fmaf_rn(v[4 * e + i], v[4 * e + i], ss);
-                    h[i] = float_to_bf16_rne(a);
-                    l[i] = float_to_bf16_rne(a - __uint_as_float(h[i] << 16));
-                }
+                for (int i = 0; i < 4; ++i) split_product(v[4 * e + i], w[i], h[i], l[i]);
                 const size_t at = (size_t)t * g.N + u0 + j + 64 * e;
                 *reinterpret_cast<uint2 *>(g.next_hi + at) = make_uint2(pack_bf16(h[0], h[1]), pack_bf16(h[2], h[3]));
                 *reinterpret_cast<uint2 *>(g.next_lo + at) = make_uint2(pack_bf16(l[0], l[1]), pack_bf16(l[2], l[3]));
+                g.ss_out[at >> 2] = squares(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
             }
-            const unsigned half_warp = 0xffffu << (threadIdx.x & 16);
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1) ss += __shfl_xor_sync(half_warp, ss, o);
-            if (j == 0) g.ss_out[(size_t)(u0 >> 7) * g.ss_rows + t] = ss;
         }
     }
 }
@@ -518,8 +520,8 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant_
         for (int i = 0; jobs.get(i, tile, c_begin, c_end); ++i) {
             const int t0 = (tile % g.tiles_x) * tt + hsel * half;
             const bool piece = tile >= g.whole;
-            float own_scale = 1.0f;          // of the group's token gt, summed while the first chunk is under way
-            if (EPI != PF_ADD && g.ss && !piece && gt < half && t0 + gt < g.T) own_scale = row_scale(g, t0 + gt);
+            float own_scale = 1.0f;          // of the group's token gt, fetched while the first chunk is under way
+            if (EPI != PF_ADD && g.row_scale && !piece && gt < half && t0 + gt < g.T) own_scale = g.row_scale[t0 + gt];
             float acc[128];
 #pragma unroll
             for (int e = 0; e < 128; ++e) acc[e] = 0.f;
@@ -614,7 +616,7 @@ __global__ void __launch_bounds__(256) fold_pieces_kernel(const GemmArgs g) {
     const float4 *src = reinterpret_cast<const float4 *>(g.part + (((size_t)r * nchunks * 2 + rank) * g.tt + tok) * 128 + j);
     float4 x[2];
     old_values<EPI>(g, u0, t, j, x);
-    const float rs = EPI != PF_ADD && g.ss ? row_scale(g, t) : 1.0f;
+    const float rs = EPI != PF_ADD && g.row_scale ? g.row_scale[t] : 1.0f;
     float v[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) v[e] = 0.f;
@@ -652,31 +654,48 @@ __global__ void embed_rows_kernel(const bf16_t *__restrict__ table, const int *_
     }
 }
 
-// RMSNorm of row t (gain g) for the contraction that follows: the planes hold v = x g WITHOUT the row's scale, hi = bf16(v) and
-// lo = bf16(v - hi), and the row's sums of squares by 128 columns go to the contraction's epilogue (a linear map commutes with a per-row
-// scale).  Same operands as the decode passes use: values that are exact in two bf16 terms - embedding rows with unit gains -
-// stay exact.  For the embedding rows only: the maps that add to the residual stream leave the same for the rows they have changed
-// (as a launch of its own behind each of them it took 4.5 us at 77 rows, 10 at 1024).  grid = T, 256 threads; d a multiple of 128.
-__global__ void __launch_bounds__(256) norm_split_kernel(const float *__restrict__ x, int d, const float *__restrict__ gain, bf16_t *__restrict__ hi,
-                                                         bf16_t *__restrict__ lo, float *__restrict__ ss_out, int ss_rows) {
+// RMSNorm of row t (gain g, epsilon eps) for the contraction that follows: the planes hold v = x g WITHOUT the row's
+// scale, hi = bf16(v) and lo = bf16(v - hi), and rinv[t] = 1 / sqrt(mean(x^2) + eps) goes to the contraction's epilogue
+// (a linear map commutes with a per-row scale).  Same operands as the decode passes use: values that are exact in two
+// bf16 terms - embedding rows with unit gains - stay exact.  For the embedding rows only: the maps that add to the residual stream leave
+// planes and squares of the rows they have changed, and scales_kernel does the rest.  grid = T, 256 threads.
+__global__ void __launch_bounds__(256) norm_split_kernel(const float *__restrict__ x, int d, const float *__restrict__ gain, float eps,
+                                                         bf16_t *__restrict__ hi, bf16_t *__restrict__ lo, float *__restrict__ rinv_out) {
     chain_wait();
+    __shared__ float part[8];
     const float *xr = x + (size_t)blockIdx.x * d;
     bf16_t *hr = hi + (size_t)blockIdx.x * d, *lr = lo + (size_t)blockIdx.x * d;
-    for (int i = threadIdx.x * 4; i < d; i += 1024) {            // a warp has 128 columns
+    float ss = 0.f;
+    // one walk over the row: the planes do not depend on the row's scale
+    for (int i = threadIdx.x * 4; i < d; i += 1024) {
         const float4 v = *reinterpret_cast<const float4 *>(xr + i);
         const float4 g = *reinterpret_cast<const float4 *>(gain + i);
-        const float ss = warp_sum(v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w);
-        if ((threadIdx.x & 31) == 0) ss_out[(size_t)(i >> 7) * ss_rows + blockIdx.x] = ss;
-        const float a[4] = {v.x * g.x, v.y * g.y, v.z * g.z, v.w * g.w};
+        ss += squares(v.x, v.y, v.z, v.w);
         uint32_t h[4], l[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            h[e] = float_to_bf16_rne(a[e]);
-            l[e] = float_to_bf16_rne(a[e] - __uint_as_float(h[e] << 16));
-        }
+        split_product(v.x, g.x, h[0], l[0]);
+        split_product(v.y, g.y, h[1], l[1]);
+        split_product(v.z, g.z, h[2], l[2]);
+        split_product(v.w, g.w, h[3], l[3]);
         *reinterpret_cast<uint2 *>(hr + i) = make_uint2(pack_bf16(h[0], h[1]), pack_bf16(h[2], h[3]));
         *reinterpret_cast<uint2 *>(lr + i) = make_uint2(pack_bf16(l[0], l[1]), pack_bf16(l[2], l[3]));
     }
+    const float rinv = scale_of_row(ss, part, d, eps);
+    if (threadIdx.x == 0) rinv_out[blockIdx.x] = rinv;
+}
+
+// rinv[t] of a row whose squares a contraction has left four columns at a time.  The order of the sum is norm_split_kernel's.  Summed by
+// 128 columns in the one epilogue and slot after slot in the next one, without this launch, a scale of 5120 columns had twice the error (1.0e-7 rms
+// against 64 bits for 5.1e-8), and the epilogues of long prompts took longer than the launch does (4 layers of the 7B widths, 77 / 300 / 1024
+// rows: 631 / 1251 / 2980 us so, 647 / 1209 / 2918 with it).  grid = T, 256 threads.
+__global__ void __launch_bounds__(256) scales_kernel(const float *__restrict__ squares4, int d, float eps, float *__restrict__ rinv_out) {
+    chain_wait();
+    __shared__ float part[8];
+    const float *sr = squares4 + (size_t)blockIdx.x * (d / 4);
+    float ss = 0.f;
+#pragma unroll 5
+    for (int i = threadIdx.x; i < d / 4; i += 256) ss += __ldcg(sr + i);
+    const float rinv = scale_of_row(ss, part, d, eps);
+    if (threadIdx.x == 0) rinv_out[blockIdx.x] = rinv;
 }
 
 // (cos, sin) of the rotary angles of rows t = 0 .. T-1 at positions pos0 + t, once per chunk: all layers and heads

@@ -123,12 +123,9 @@ struct QkvFuse {
     int max_seq, pos0, head_dim;
 };
 
-// RMSNorms around a contraction: of the rows it reads (ss, eps), and of the rows it has added to (gain, planes, ss_out); `rows` long each
-// slot of the sums of squares (GemmArgs).
+// RMSNorms around a contraction: the scales of the rows it reads; gain, planes and squares of the rows it has added to (GemmArgs).
 struct Norms {
-    const float *ss = nullptr;
-    int rows = 0;
-    float eps = 0.f;
+    const float *row_scale = nullptr;
     const float *next_gain = nullptr;
     bf16_t *next_hi = nullptr, *next_lo = nullptr;
     float *ss_out = nullptr;
@@ -156,7 +153,7 @@ inline int launch_gemm(const Deal &deal, const bf16_t *planes, float *part, int 
     if (stacked && (!make_map(&tb1, W1, (size_t)nB, (size_t)K, box) || !make_map(&tb2, W2, (size_t)(N - nA - nB), (size_t)K, box))) return 0;
     const int per = epi == PF_SWIGLU ? PAIR_UNITS / 2 : PAIR_UNITS;
     const int tiles_x = (T + deal.tt - 1) / deal.tt, tiles_y = (N + per - 1) / per, pieces = tiles_x * tiles_y - deal.whole;
-    GemmArgs g{T, K, N, deal.tt, y, ldy, col0, out_hi, out_lo, ldo, err, tiles_x, tiles_y, box, deal.whole, part, stacked ? nA : N, stacked ? nB : 0, norms.ss, norms.rows, norms.eps, norms.next_gain, norms.next_hi, norms.next_lo, norms.ss_out, nullptr, nullptr, nullptr, 0, 0};
+    GemmArgs g{T, K, N, deal.tt, y, ldy, col0, out_hi, out_lo, ldo, err, tiles_x, tiles_y, box, deal.whole, part, stacked ? nA : N, stacked ? nB : 0, norms.row_scale, norms.next_gain, norms.next_hi, norms.next_lo, norms.ss_out, nullptr, nullptr, nullptr, 0, 0};
     auto run = [&](auto *contract, auto *fold) {
         launch_chained(contract, dim3(2 * deal.pairs), dim3(GEMM_THREADS), gemm_smem(deal.tt), s, ta, tb0, tb1, tb2, g, cap);
         if (pieces) launch_chained(fold, dim3(2 * (deal.tt / 16), pieces), dim3(256), 0, s, g);

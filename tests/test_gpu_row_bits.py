@@ -27,3 +27,27 @@ def test_cache_rows_are_the_same_bits_whatever_follows_them(name):
         got = sess.verify(rows[1:], want_logits=True)["logits"]
         want = got if want is None else want
         assert torch.equal(got, want), n
+
+
+@pytest.mark.parametrize("rows", [20, 77, 300])
+def test_a_norm_is_the_same_bits_whichever_kernel_sums_it(rows):
+    """A layer whose maps back into the residual stream are zero changes nothing: the layer behind it finds the rows that the embedding left.
+    Its norms come from squares that the zero maps' epilogues left, those of the same layer at the bottom of a model from the rows."""
+    from paper_2505_16162_b200 import build
+    build.build()
+    from paper_2505_16162_b200 import binding as kb
+    two = si.ModelShape("norms", 2, 1536, 12, 4, 128, 2048, 1003, "bf16", 1e-5, 10000.0)
+    one = two.with_layers(1)
+    w = si.make_model_weights(two, 9, device="cuda", gain_spread=0.1)
+    w["wo"][0].zero_()
+    w["w_down"][0].zero_()
+    w1 = {k: (v[1:] if isinstance(v, list) else v) for k, v in w.items()}
+    prompt = si.uniform_tokens(9, 0, rows, two.vocab).numpy()
+    tokens = si.uniform_tokens(9, 1, 4, two.vocab).numpy()
+    got = []
+    for shape, weights in ((two, w), (one, w1)):
+        sess = kb.Session.from_shape(shape, weights, 400, max_draft=4)
+        first, pooled = sess.prefill(prompt, want_pooled=True)
+        sess.set_pending(int(tokens[0]))
+        got.append((first, pooled, sess.verify(tokens[1:], want_logits=True)["logits"]))
+    assert got[0][0] == got[1][0] and torch.equal(got[0][1], got[1][1]) and torch.equal(got[0][2], got[1][2])
