@@ -318,28 +318,58 @@ void ctx_linear(knnssd_ctx *c, const LinearArgs &a) {
     c->launches++;
 }
 
+// How many of the filter's clusters of sixteen blocks the current device has room for at a time: they are larger than what every device
+// takes at all.
+int wide_filter_clusters() {
+    static std::mutex mu;
+    static int room[kMaxDevices] = {};                 // one more than the answer; 0: not asked yet
+    const int dev = current_device_slot();
+    std::lock_guard<std::mutex> lock(mu);
+    if (!room[dev]) {
+        const auto kernel = sampling::filtered_probs_kernel<sampling::CL_WIDE, 1>;
+        const int smem = (int)sizeof(float) * sampling::SLICE_MAX;
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = sampling::CL_WIDE; attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(sampling::CL_WIDE); cfg.blockDim = dim3(sampling::NT); cfg.dynamicSmemBytes = smem; cfg.attrs = &attr; cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess)
+            n = 0;
+        cudaGetLastError();
+        room[dev] = n + 1;
+    }
+    return room[dev] - 1;
+}
+
 // Rows are y blocks of the grid, at most 65535 per launch.
-template <int C> void launch_filter_t(const float *logits, int rows, int V, float inv_t, float top_p, float *probs, cudaStream_t s) {
+template <int C, int SL> void launch_filter_t(const float *logits, int rows, int V, float inv_t, float top_p, float *probs, cudaStream_t s) {
     static bool configured[kMaxDevices] = {};          // function attributes are per device
     const int dev = current_device_slot();
     if (!configured[dev]) {
-        cudaFuncSetAttribute(sampling::filtered_probs_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(float) * sampling::SLICE_MAX);
-        if (C > 8) cudaFuncSetAttribute(sampling::filtered_probs_kernel<C>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        cudaFuncSetAttribute(sampling::filtered_probs_kernel<C, SL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(float) * sampling::SLICE_MAX);
+        if (C > 8) cudaFuncSetAttribute(sampling::filtered_probs_kernel<C, SL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         configured[dev] = true;
     }
     for (int r = 0; r < rows; r += 65535) {
         const int n = rows - r < 65535 ? rows - r : 65535;
-        sampling::filtered_probs_kernel<C><<<dim3(C, n), sampling::NT, sampling::probs_smem(V, C), s>>>(
+        sampling::filtered_probs_kernel<C, SL><<<dim3(C, n), sampling::NT, sampling::probs_smem(V, C, SL), s>>>(
             logits + (size_t)r * V, V, inv_t, top_p, probs + (size_t)r * V);
     }
 }
-// Sixteen blocks per row for few long rows, and where eight have no room to keep values aside.  One row of 50000 / 65536 / 152064 ids:
-// 16.1 / 15.6 / 21.5 us against 16.8 / 18.1 / 29.7 with eight; nine rows of 152064 are two rounds of clusters of sixteen, 42.5 against
-// 29.8; 300000 ids 31 against 153, 48 rows of them 240 against 630.
-constexpr int kWideFilterVocab = 65536, kWideFilterRows = 5;
+// From kWideFilterVocab ids on a row is cut into sixteen slices, whatever its company: its sums are the same.  A block has one of them where all
+// rows' clusters of sixteen run at a time (seven of them here) and where eight blocks have no room to keep values aside, else two.  Us a
+// launch of 1 / 7 / 8 / 16 rows, sixteen blocks, eight with two slices, eight with one: 65536 ids 23 / 23 / 39 / 60, 29 / 29 / 29 / 50, 25 / 25 /
+// 25 / 43; 100003 ids 27 / 27 / 46 / 71, 37 / 37 / 37 / 65, 31 / 31 / 32 / 56; 152064 ids 31 / 33 / 56 / 89, 46 / 48 / 48 / 84, 41 / 42 / 42 / 74;
+// 300000 ids in sixteen blocks 31 for 153, 48 rows of them 240 for 630.
+constexpr int kWideFilterVocab = 65536;
 void launch_filter(const float *logits, int rows, int V, float inv_t, float top_p, float *probs, cudaStream_t s) {
-    if ((V >= kWideFilterVocab && rows <= kWideFilterRows) || V > sampling::CL * (sampling::SLICE_MAX / 2)) launch_filter_t<sampling::CL_WIDE>(logits, rows, V, inv_t, top_p, probs, s);
-    else launch_filter_t<sampling::CL>(logits, rows, V, inv_t, top_p, probs, s);
+    if (V < kWideFilterVocab) { launch_filter_t<sampling::CL, 1>(logits, rows, V, inv_t, top_p, probs, s); return; }
+    const int room = wide_filter_clusters();
+    if (rows <= room || (room > 0 && V > sampling::CL * (sampling::SLICE_MAX / 2))) launch_filter_t<sampling::CL_WIDE, 1>(logits, rows, V, inv_t, top_p, probs, s);
+    else launch_filter_t<sampling::CL, 2>(logits, rows, V, inv_t, top_p, probs, s);
 }
 
 LinearArgs make_args(const void *W0, int rows0, int n_in, const float *x, const float *gain, float eps, float *y,

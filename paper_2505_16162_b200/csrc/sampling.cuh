@@ -8,9 +8,9 @@
 // more token is drawn from p.  Random numbers are inputs (one uniform per draw), consumed through the inverse CDF in
 // token-id order, so that the choices are reproducible.
 //
-// A row is the work of a cluster of eight blocks, each with a contiguous eighth of the ids: a few passes over values that
-// stay in shared memory, bound by the meetings between the passes (~1.5 us each: block, then cluster).  Every sum has a
-// fixed order.
+// A row is the work of a cluster of eight blocks, each with a contiguous eighth of the ids, or, where the filter has a long row, of
+// sixteen: a few passes over values that stay in shared memory, bound by the meetings between the passes (~1.5 us each: block, then
+// cluster).  Every sum has a fixed order, which the row's length alone decides.
 #pragma once
 #include <cooperative_groups.h>
 
@@ -23,31 +23,28 @@ namespace cg = cooperative_groups;
 
 constexpr int NT = 512;                    // at 1024 the meetings take twice as long (32 sums per warp to add up), at 256 long rows do
 constexpr int NW = NT / 32;
-constexpr int CL = 8;                      // blocks per row; the filter takes CL_WIDE for long rows
+constexpr int CL = 8;                      // blocks per row; the filter takes CL_WIDE for few long rows
 constexpr int CL_WIDE = 16;
 constexpr int NS = 32;                     // sums that one meeting adds up: one per lane, and per warp
 constexpr int SLICE_MAX = 49152;           // ids per block that fit in shared memory (192 KB)
 
-// Meeting place of the blocks of a row.  `slot` alternates: a block may still read the last meeting's sums while another
-// already writes the next one's.
-template <int C> struct MeetOf {
-    static constexpr int BLOCKS = C;
-    float red[NW][NS + 1];
-    float slot[2][C][NS];
+// Meeting place of the C blocks of a row, each with SL slices of it.  `slot` alternates: a block may still read the last meeting's sums
+// while another already writes the next one's.
+template <int C, int SL = 1> struct MeetOf {
+    static constexpr int BLOCKS = C, SLICES = SL;
+    float red[SL][NW][NS + 1];
+    float slot[2][C * SL][NS];
 };
 typedef MeetOf<CL> Meet;
 
-// Sum (MAX: maximum of v[0]) over the threads of all blocks; lane j of every warp gets sum j, added in a fixed
-// order: lanes, warps, blocks.  `turn` counts the meetings.
+// A meeting: sums (MAX: maximum of v[0]) over the threads of all blocks, in a fixed order: lanes, warps, slices.  First every warp brings
+// its share of each slice, then all of them join: lane j of every warp gets sum j.  `turn` counts the meetings.
 template <bool MAX, typename M>
-__device__ __forceinline__ float meet(M &sh, int &turn, float (&v)[NS]) {
-    constexpr int CL = M::BLOCKS;
-    cg::cluster_group cluster = cg::this_cluster();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, par = turn & 1;
-    ++turn;
+__device__ __forceinline__ void bring(M &sh, int slice, float (&v)[NS]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (MAX) {
         const float m = warp_max(v[0]);
-        if (lane == 0) sh.red[warp][0] = m;
+        if (lane == 0) sh.red[slice][warp][0] = m;
     } else {
         // each step halves the sums a lane is in charge of: 31 exchanges instead of 5 for every sum
 #pragma unroll
@@ -59,28 +56,44 @@ __device__ __forceinline__ float meet(M &sh, int &turn, float (&v)[NS]) {
                 v[i] = keep + __shfl_xor_sync(0xffffffffu, give, bit);
             }
         }
-        sh.red[warp][lane] = v[0];
+        sh.red[slice][warp][lane] = v[0];
     }
+}
+template <bool MAX, typename M>
+__device__ __forceinline__ float join(M &sh, int &turn) {
+    constexpr int CL = M::BLOCKS, SL = M::SLICES;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, par = turn & 1;
+    ++turn;
     __syncthreads();
     // lanes r NW .. r NW + NW - 1 of warp w add up sum w PW + r of the NW warps
     constexpr int PW = NS / NW;
     static_assert(CL <= NW && NW <= 32 && NS == 32, "a lane per block in every group of lanes");
-    float t0 = sh.red[lane % NW][MAX ? 0 : warp * PW + lane / NW];
 #pragma unroll
-    for (int o = NW / 2; o > 0; o >>= 1) {
-        const float other = __shfl_xor_sync(0xffffffffu, t0, o);
-        t0 = MAX ? fmaxf(t0, other) : t0 + other;
+    for (int slice = 0; slice < SL; ++slice) {
+        float t0 = sh.red[slice][lane % NW][MAX ? 0 : warp * PW + lane / NW];
+#pragma unroll
+        for (int o = NW / 2; o > 0; o >>= 1) {
+            const float other = __shfl_xor_sync(0xffffffffu, t0, o);
+            t0 = MAX ? fmaxf(t0, other) : t0 + other;
+        }
+        if (lane % NW < CL && (!MAX || (warp == 0 && lane < NW)))
+            cluster.map_shared_rank(&sh, lane % NW)->slot[par][cluster.block_rank() * SL + slice][MAX ? 0 : warp * PW + lane / NW] = t0;
     }
-    if (lane % NW < CL && (!MAX || (warp == 0 && lane < NW)))
-        cluster.map_shared_rank(&sh, lane % NW)->slot[par][cluster.block_rank()][MAX ? 0 : warp * PW + lane / NW] = t0;
     cluster.sync();
     float t = sh.slot[par][0][MAX ? 0 : lane];
 #pragma unroll
-    for (int r = 1; r < CL; ++r) {
+    for (int r = 1; r < CL * SL; ++r) {
         const float o = sh.slot[par][r][MAX ? 0 : lane];
         t = MAX ? fmaxf(t, o) : t + o;
     }
     return t;
+}
+template <bool MAX, typename M>
+__device__ __forceinline__ float meet(M &sh, int &turn, float (&v)[NS]) {
+    static_assert(M::SLICES == 1, "one slice a block");
+    bring<MAX>(sh, 0, v);
+    return join<MAX>(sh, turn);
 }
 
 // Count over one block.
@@ -96,86 +109,127 @@ __device__ __forceinline__ int block_count(int v, int *sh) {
     return t;
 }
 
-// Ids per block of a row of V: [rank S, rank S + S).
-__host__ __device__ __forceinline__ int slice_len(int V, int blocks = CL) { return (V + blocks - 1) / blocks; }
-// Shared memory of filtered_probs_kernel: the slice's values and, where it fits as well, the candidates among them.
-inline size_t probs_smem(int V, int blocks) {
-    const size_t S = slice_len(V, blocks), padded = (S + NT - 1) / NT * NT;
-    return sizeof(float) * (S + padded <= SLICE_MAX ? S + padded : S <= SLICE_MAX ? S : 0);
+// Ids per slice of a row of V cut into so many: [r S, r S + S).
+__host__ __device__ __forceinline__ int slice_len(int V, int slices = CL) { return (V + slices - 1) / slices; }
+// Shared memory of filtered_probs_kernel: the values of a block's slices and, where it fits as well, the candidates among them.
+inline size_t probs_smem(int V, int blocks, int slices) {
+    const size_t S = slice_len(V, blocks * slices), padded = (S + NT - 1) / NT * NT;
+    return sizeof(float) * (slices * (S + padded) <= SLICE_MAX ? slices * (S + padded) : slices * S <= SLICE_MAX ? slices * S : 0);
+}
+
+// use(i, p[i]) for this thread's entries i = tid, tid + NT, .. below n, U of them fetched together: the rest of an unrolled loop would
+// fetch one after the other.
+template <int U, typename F> __device__ __forceinline__ void each_entry(const float *p, int n, F use) {
+    for (int i0 = threadIdx.x; i0 < n; i0 += U * NT) {
+        float y[U];
+#pragma unroll
+        for (int e = 0; e < U; ++e) y[e] = i0 + e * NT < n ? p[i0 + e * NT] : 0.f;
+#pragma unroll
+        for (int e = 0; e < U; ++e)
+            if (i0 + e * NT < n) use(i0 + e * NT, y[e]);
+    }
 }
 
 // probs[row] = nucleus-filtered softmax(logits[row] / temperature), renormalised.  A token is kept iff the probability
 // mass of the tokens ranked before it (higher probability first, lower id first among equals) is below top_p.
 // The mass above a value is a decreasing step function of the value, so the smallest kept probability x0 is found in
 // the bit patterns of positive floats, 32 candidates at a time (five bits per pass; one candidate per pass, by one block
-// that re-read its row from L2 each time, took 65 us for 5 rows of 32000 and 241 us for one of 152064; this takes 20 and 35).  The first pass leaves
+// that re-read its row from L2 each time, took 65 us for 5 rows of 32000 and 241 us for one of 152064; this takes 15 and 21).  The first pass leaves
 // a few per cent of the values between its bounds; a thread keeps those of its own aside for the others.  Once no block has more than
 // GATHER values left between the bounds all blocks get them all, and each finds x0 for itself: a meeting instead of five.
 // Tokens whose probability equals x0 are ranked by id.
-// grid = (C, rows), NT threads, probs_smem(V, C) of shared memory; rows too long for it keep their values in `probs`.
+// A row is cut into C SL slices; what comes out depends on their number, not on how many blocks share them.
+// grid = (C, rows), NT threads, probs_smem(V, C, SL) of shared memory; rows too long for it keep their values in `probs`.
 constexpr int GATHER = 32;
-template <int C> __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(NT)
+template <int C, int SL> __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(NT)
 filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_temperature, float top_p, float *__restrict__ probs) {
+    constexpr int SLICES = C * SL;
+    static_assert(SLICES <= NS, "a sum per slice");
     extern __shared__ float probs_slice[];
-    __shared__ MeetOf<C> sh;
-    __shared__ int shi[NW];
+    __shared__ MeetOf<C, SL> sh;
+    __shared__ int shi[SL][NW];
     __shared__ int s_cut;
-    __shared__ float left[C][GATHER];                            // the blocks' values between the bounds
-    __shared__ int n_left[C];
+    __shared__ float left[SLICES][GATHER];                       // the slices' values between the bounds
+    __shared__ int n_left[SLICES];
     __shared__ unsigned s_x0;
-    constexpr int CL = C;
     cg::cluster_group cluster = cg::this_cluster();
-    const int S = slice_len(V, C), rank = (int)cluster.block_rank(), tid = threadIdx.x;
-    const int id0 = min(V, rank * S), n = min(V, id0 + S) - id0;
-    const float *l = logits + (size_t)blockIdx.y * V + id0;
-    float *out = probs + (size_t)blockIdx.y * V + id0;
-    float *p = S <= SLICE_MAX ? probs_slice : out;               // a thread only ever touches its own entries, except where ids count
+    const int S = slice_len(V, SLICES), padded = (S + NT - 1) / NT * NT, rank = (int)cluster.block_rank(), tid = threadIdx.x;
+    const bool keeps_list = SL * (S + padded) <= SLICE_MAX;
     int turn = 0;
+    // this block's slices
+    int id0[SL], n[SL], n_list[SL];
+    float *p[SL];                                                // a thread only ever touches its own entries, except where ids count
+    float above[SL];                                             // this thread's values that lie above all candidates
+#pragma unroll
+    for (int k = 0; k < SL; ++k) {
+        id0[k] = min(V, (rank * SL + k) * S);
+        n[k] = min(V, id0[k] + S) - id0[k];
+        p[k] = keeps_list ? probs_slice + k * (S + padded) : SL * S <= SLICE_MAX ? probs_slice + k * S : probs + (size_t)blockIdx.y * V + id0[k];
+        n_list[k] = 0;
+        above[k] = 0.f;
+    }
+    auto list = [&](int k) { return probs_slice + k * (S + padded) + S + tid; };
     float v[NS];
     cluster.barrier_arrive();                                    // every block has to run before another writes to its shared memory
     float m = -INFINITY;
-#pragma unroll 8
-    for (int i = tid; i < n; i += NT) { const float x = l[i]; p[i] = x; m = fmaxf(m, x); }
+#pragma unroll
+    for (int k = 0; k < SL; ++k) {
+        float *to = p[k];
+        each_entry<8>(logits + (size_t)blockIdx.y * V + id0[k], n[k], [&](int i, float x) { to[i] = x; m = fmaxf(m, x); });
+    }
     v[0] = m;
     cluster.barrier_wait();
-    m = meet<true>(sh, turn, v);
 #pragma unroll
-    for (int j = 0; j < NS; ++j) v[j] = 0.f;
-    for (int i = tid; i < n; i += NT) {
-        const float e = expf((p[i] - m) * inv_temperature);
-        p[i] = e;
-        v[0] += e;
+    for (int k = 0; k < SL; ++k) bring<true>(sh, k, v);
+    m = join<true>(sh, turn);
+#pragma unroll
+    for (int k = 0; k < SL; ++k) {
+#pragma unroll
+        for (int j = 0; j < NS; ++j) v[j] = 0.f;
+        float *to = p[k];
+        each_entry<4>(to, n[k], [&](int i, float x) {
+            const float e = expf((x - m) * inv_temperature);
+            to[i] = e;
+            v[0] += e;
+        });
+        bring<false>(sh, k, v);
     }
-    const float s = __shfl_sync(0xffffffffu, meet<false>(sh, turn, v), 0);
-    for (int i = tid; i < n; i += NT) p[i] = p[i] / s;
+    const float s = __shfl_sync(0xffffffffu, join<false>(sh, turn), 0);
+#pragma unroll
+    for (int k = 0; k < SL; ++k) {
+        float *to = p[k];
+        each_entry<4>(to, n[k], [&](int i, float x) { to[i] = x / s; });
+    }
     // smallest x (as a bit pattern) in [lo, hi] with mass above x < top_p.  The largest probability is 1 / s (its exponent
     // is zero), nothing lies above it.  Below (1 - top_p) / (2 V) there is less than half of 1 - top_p in all, so the mass above
     // that is not below top_p: a sum of V terms is not off by the other half unless top_p is 1 to four digits.
     unsigned lo = 0u, hi = __float_as_uint(fmaxf(0.f, 1.0f / s));
     if (1.0f - top_p > 1e-4f) lo = min(hi, __float_as_uint(0.5f * (1.0f - top_p) / (float)V));
-    float *list = S + (S + NT - 1) / NT * NT <= SLICE_MAX ? probs_slice + S + tid : nullptr;
-    int n_list = 0;
-    float above = 0.f;                                           // this thread's values that lie above all candidates
     float above_hi = 0.f;                                        // all threads' values above hi
     int gathered = -1;                                           // values between the bounds, once all blocks have them
     for (bool first = true; first || hi > lo + 1u; first = false) {
         const unsigned step = (hi - lo + NS - 1) / NS;           // candidates lo, lo + step, ..: lo itself only counts in the first pass
         float x[NS];
 #pragma unroll
-        for (int j = 0; j < NS; ++j) { v[j] = above; x[j] = __uint_as_float(min(hi, lo + j * step)); }
-        const bool listed = list && !first;
-        const float *src = listed ? list : p + tid;
-        const int m_own = listed ? n_list : (n - tid + NT - 1) / NT;
-        for (int i0 = 0; i0 < m_own; i0 += 4) {                  // four loads in flight: rows too long for shared memory come from L2
-            float y[4];
+        for (int j = 0; j < NS; ++j) x[j] = __uint_as_float(min(hi, lo + j * step));
+        const bool listed = keeps_list && !first;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) y[e] = i0 + e < m_own ? src[(i0 + e) * NT] : 0.f;
+        for (int k = 0; k < SL; ++k) {
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
+            for (int j = 0; j < NS; ++j) v[j] = above[k];
+            auto count = [&](float y) {
 #pragma unroll
-                for (int j = 0; j < NS; ++j) v[j] += y[e] > x[j] ? y[e] : 0.f;
+                for (int j = 0; j < NS; ++j) v[j] += y > x[j] ? y : 0.f;
+            };
+            if (listed) {                                        // hardly any thread has more than one left
+#pragma unroll 1
+                for (int i = 0; i < n_list[k]; ++i) count(list(k)[NT * i]);
+            } else {
+                each_entry<4>(p[k], n[k], [&](int, float y) { count(y); });
+            }
+            bring<false>(sh, k, v);
         }
-        const float mass = meet<false>(sh, turn, v);
+        const float mass = join<false>(sh, turn);
         const unsigned below = __ballot_sync(0xffffffffu, mass < top_p);
         int j = below ? __ffs(below) - 1 : NS;                   // the first candidate with less than top_p above it
         if (j == 0) {
@@ -186,59 +240,71 @@ filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_tempera
         const unsigned nhi = j < NS ? min(hi, lo + j * step) : hi;
         lo = min(hi, lo + (j - 1) * step);
         hi = nhi;
-        if (first && list) {
-            const float xl = __uint_as_float(lo), xh = __uint_as_float(hi);
-            for (int i = tid; i < n; i += NT) {
-                const float y = p[i];
-                if (y > xh) above += y;
-                else if (y > xl) list[NT * n_list++] = y;
-            }
-        } else if (list && hi > lo + 1u) {
-            // hand the values left to all blocks, in the order of blocks, threads and each thread's list
-            const float xl = __uint_as_float(lo), xh = __uint_as_float(hi);
-            int own = 0;
-            for (int i = 0; i < n_list; ++i) { const float y = list[NT * i]; own += y > xl && y <= xh ? 1 : 0; }
+        const float xl = __uint_as_float(lo), xh = __uint_as_float(hi);
+        if (first && keeps_list) {
+#pragma unroll
+            for (int k = 0; k < SL; ++k)
+                each_entry<4>(p[k], n[k], [&](int, float y) {
+                    if (y > xh) above[k] += y;
+                    else if (y > xl) list(k)[NT * n_list[k]++] = y;
+                });
+        } else if (keeps_list && hi > lo + 1u) {
+            // hand the values left to all blocks, in the order of slices, threads and each thread's list
             const int lane = tid & 31, warp = tid >> 5;
-            int upto = own;                                      // of the warp's lanes up to this one
+            int upto[SL], own[SL], all[SL];
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xffffffffu, upto, o); if (lane >= o) upto += t; }
-            if (lane == 31) shi[warp] = upto;
-            __syncthreads();
-            int before = 0, all = 0;
+            for (int k = 0; k < SL; ++k) {
+                own[k] = 0;
+                for (int i = 0; i < n_list[k]; ++i) { const float y = list(k)[NT * i]; own[k] += y > xl && y <= xh ? 1 : 0; }
+                upto[k] = own[k];                                // of the warp's lanes up to this one
 #pragma unroll
-            for (int w = 0; w < NW; ++w) { if (w == warp) before = all; all += shi[w]; }
-            int at = before + upto - own;
-            for (int i = 0; i < n_list; ++i) {
-                const float y = list[NT * i];
-                if (y > xl && y <= xh) { if (at < GATHER) left[rank][at] = y; ++at; }
+                for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xffffffffu, upto[k], o); if (lane >= o) upto[k] += t; }
+                if (lane == 31) shi[k][warp] = upto[k];
             }
             __syncthreads();
-            for (int t = tid; t < C * GATHER; t += NT) {
-                const int r = t / GATHER, i = t % GATHER;
-                if (r != rank && i < min(all, GATHER)) *cluster.map_shared_rank(&left[rank][i], r) = left[rank][i];
-                if (i == 0) *cluster.map_shared_rank(&n_left[rank], r) = all;
+#pragma unroll
+            for (int k = 0; k < SL; ++k) {
+                int before = 0;
+                all[k] = 0;
+#pragma unroll
+                for (int w = 0; w < NW; ++w) { if (w == warp) before = all[k]; all[k] += shi[k][w]; }
+                int at = before + upto[k] - own[k];
+                for (int i = 0; i < n_list[k]; ++i) {
+                    const float y = list(k)[NT * i];
+                    if (y > xl && y <= xh) { if (at < GATHER) left[rank * SL + k][at] = y; ++at; }
+                }
             }
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < SL; ++k)
+                for (int t = tid; t < C * GATHER; t += NT) {
+                    const int r = t / GATHER, i = t % GATHER;
+                    if (r != rank && i < min(all[k], GATHER)) *cluster.map_shared_rank(&left[rank * SL + k][i], r) = left[rank * SL + k][i];
+                    if (i == 0) *cluster.map_shared_rank(&n_left[rank * SL + k], r) = all[k];
+                }
             cluster.sync();
             int most = 0, total = 0;
 #pragma unroll
-            for (int r = 0; r < C; ++r) { most = max(most, n_left[r]); total += n_left[r]; }
+            for (int r = 0; r < SLICES; ++r) { most = max(most, n_left[r]); total += n_left[r]; }
             if (most <= GATHER) { gathered = total; break; }
             cluster.sync();                                      // nobody writes the next values while others read these counts
         }
     }
     float x0 = __uint_as_float(hi);
     float a0 = above_hi;                                         // mass above x0
-    int c = 0, own_c = 0;                                        // tokens at x0: of all blocks, and this thread's share of its block's
+    int c = 0, own_c[SL];                                        // tokens at x0: of all slices, and this thread's share of its block's
+#pragma unroll
+    for (int k = 0; k < SL; ++k) own_c[k] = 0;
     if (gathered >= 0) {
         // the smallest of the values left with less than top_p above it; if rounding has it that there is none, hi
         if (tid == 0) s_x0 = hi;
         __syncthreads();
-        for (int t = tid; t < C * GATHER; t += NT) {
+        for (int t = tid; t < SLICES * GATHER; t += NT) {
             const int r = t / GATHER, i = t % GATHER;
             if (i < n_left[r]) {
                 const float y = left[r][i];
                 float m_above = 0.f;                             // the few small values by themselves, then one rounding at the size of the mass
-                for (int q = 0; q < C; ++q)
+                for (int q = 0; q < SLICES; ++q)
                     for (int e = 0, n_q = n_left[q]; e < n_q; ++e) { const float o = left[q][e]; m_above += o > y ? o : 0.f; }
                 if (above_hi + m_above < top_p) atomicMin(&s_x0, __float_as_uint(y));
             }
@@ -246,24 +312,31 @@ filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_tempera
         __syncthreads();
         x0 = __uint_as_float(s_x0);
         float left_above = 0.f;
-        for (int q = 0; q < C; ++q)
+        for (int q = 0; q < SLICES; ++q)
             for (int e = 0, n_q = n_left[q]; e < n_q; ++e) {
                 const float o = left[q][e];
                 left_above += o > x0 ? o : 0.f;
-                if (o == x0) { ++c; own_c += q == rank && tid == 0 ? 1 : 0; }
+                if (o == x0) {
+                    ++c;
+#pragma unroll
+                    for (int k = 0; k < SL; ++k) own_c[k] += q == rank * SL + k && tid == 0 ? 1 : 0;
+                }
             }
         a0 = above_hi + left_above;
     } else {
         // rows whose values are not kept aside, and bounds that met without it
 #pragma unroll
-        for (int j = 0; j < NS; ++j) v[j] = 0.f;
-        for (int i = tid; i < n; i += NT) {
-            const float y = p[i];
-            v[0] += y > x0 ? y : 0.f;
-            if (y == x0) v[1] += 1.f;                            // counts are exact up to 2^24 tokens
+        for (int k = 0; k < SL; ++k) {
+#pragma unroll
+            for (int j = 0; j < NS; ++j) v[j] = 0.f;
+            each_entry<4>(p[k], n[k], [&](int, float y) {
+                v[0] += y > x0 ? y : 0.f;
+                if (y == x0) v[1] += 1.f;                        // counts are exact up to 2^24 tokens
+            });
+            own_c[k] = (int)v[1];
+            bring<false>(sh, k, v);
         }
-        own_c = (int)v[1];
-        const float tot = meet<false>(sh, turn, v);
+        const float tot = join<false>(sh, turn);
         a0 = __shfl_sync(0xffffffffu, tot, 0);
         c = (int)__shfl_sync(0xffffffffu, tot, 1);
     }
@@ -272,38 +345,45 @@ filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_tempera
     if (c > 1) {
         nk = 0;
         for (int i = tid; i < c; i += NT) nk += (a0 + (float)i * x0 < top_p) ? 1 : 0;
-        nk = max(1, block_count(nk, shi));
-        if (nk < c) {                                            // which of them: the block that has the nk-th looks for its id
-            // sum r of this meeting: the tokens at x0 in block r
+        nk = max(1, block_count(nk, shi[0]));
+        if (nk < c) {                                            // which of them: the slice that has the nk-th is searched for its id
+            // sum r of this meeting: the tokens at x0 in slice r
 #pragma unroll
-            for (int j = 0; j < NS; ++j) v[j] = j == rank ? (float)own_c : 0.f;
-            const float tot = meet<false>(sh, turn, v);
+            for (int k = 0; k < SL; ++k) {
+#pragma unroll
+                for (int j = 0; j < NS; ++j) v[j] = j == rank * SL + k ? (float)own_c[k] : 0.f;
+                bring<false>(sh, k, v);
+            }
+            const float tot = join<false>(sh, turn);
             int before = 0, holder = 0;
-            for (int r = 0; r < CL; ++r) {
+            for (int r = 0; r < SLICES; ++r) {
                 const int cr = (int)__shfl_sync(0xffffffffu, tot, r);
                 if (before + cr >= nk) { holder = r; break; }
                 before += cr;
             }
-            if (rank == holder) {
-                __syncthreads();
-                int jl = 0, jh = n;                              // smallest J with #{j < J : p_j == x0} >= nk - before
-                while (jh > jl + 1) {
-                    const int jm = jl + (jh - jl) / 2;
-                    int g = 0;
-                    for (int i = tid; i < jm; i += NT) g += p[i] == x0 ? 1 : 0;
-                    g = block_count(g, shi);
-                    if (g >= nk - before) jh = jm; else jl = jm;
+#pragma unroll
+            for (int k = 0; k < SL; ++k)
+                if (rank * SL + k == holder) {
+                    __syncthreads();
+                    int jl = 0, jh = n[k];                       // smallest J with #{j < J : p_j == x0} >= nk - before
+                    while (jh > jl + 1) {
+                        const int jm = jl + (jh - jl) / 2;
+                        int g = 0;
+                        for (int i = tid; i < jm; i += NT) g += p[k][i] == x0 ? 1 : 0;
+                        g = block_count(g, shi[0]);
+                        if (g >= nk - before) jh = jm; else jl = jm;
+                    }
+                    if (tid < C) *cluster.map_shared_rank(&s_cut, tid) = id0[k] + jh;
                 }
-                if (tid < CL) *cluster.map_shared_rank(&s_cut, tid) = id0 + jh;
-            }
             cluster.sync();
             id_cut = s_cut;
         }
     }
     const float z = a0 + (float)min(nk, c) * x0;
-    for (int i = tid; i < n; i += NT) {
-        const float y = p[i];
-        out[i] = (y > x0 || (y == x0 && id0 + i < id_cut)) ? y / z : 0.f;
+#pragma unroll
+    for (int k = 0; k < SL; ++k) {
+        float *out = probs + (size_t)blockIdx.y * V + id0[k];
+        each_entry<4>(p[k], n[k], [&](int i, float y) { out[i] = (y > x0 || (y == x0 && id0[k] + i < id_cut)) ? y / z : 0.f; });
     }
     cluster.sync();                                              // nobody leaves while its shared memory may still be written to
 }
@@ -343,14 +423,14 @@ __device__ __forceinline__ int cluster_sample(const float *__restrict__ a, const
         for (int o = 16; o > 0; o >>= 1) last = max(last, __shfl_xor_sync(0xffffffffu, last, o));
         if (first) cluster.barrier_wait();
         __syncthreads();
-        if (lane == 0) { sh.warp_sum[warp] = w; sh.m.red[warp][NS] = __int_as_float(last); }
+        if (lane == 0) { sh.warp_sum[warp] = w; sh.m.red[0][warp][NS] = __int_as_float(last); }
         __syncthreads();
         // sum r of the meeting: block r's weights, its warps added in order
         float v[NS], mine = 0.f;
         if (tid == 0)
             for (int k = 0; k < NW; ++k) mine += sh.warp_sum[k];
         if (warp == 0) {
-            int lb = lane < NW ? __float_as_int(sh.m.red[lane][NS]) : -1;
+            int lb = lane < NW ? __float_as_int(sh.m.red[0][lane][NS]) : -1;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) lb = max(lb, __shfl_xor_sync(0xffffffffu, lb, o));
             if (lane == 0) cluster.map_shared_rank(&sh, 0)->last[rank] = lb;
@@ -398,7 +478,7 @@ __device__ __forceinline__ int cluster_sample(const float *__restrict__ a, const
             if (tok < 0) {
                 // the last warp, without weight of its own: the block's sum, added at once, ends an ulp past the running sum of its
                 // warps, and the target lies between.  The crossing is in this block all the same: its last id with weight
-                tok = lane < NW ? __float_as_int(sh.m.red[lane][NS]) : -1;
+                tok = lane < NW ? __float_as_int(sh.m.red[0][lane][NS]) : -1;
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) tok = max(tok, __shfl_xor_sync(0xffffffffu, tok, o));
             }

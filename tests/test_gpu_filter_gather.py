@@ -1,5 +1,5 @@
-"""The nucleus filter's search: values so close together that more of them lie between the bounds than blocks hand to one another, until
-late or to the end; rows on either side of the sizes at which a row takes sixteen blocks instead of eight."""
+"""The nucleus filter: values so close together that more of them lie between the bounds than blocks hand to one another, until late or to
+the end; rows on either side of the sizes at which a row takes sixteen slices; a row alone and in company."""
 import numpy as np
 import pytest
 import torch
@@ -52,3 +52,22 @@ def test_values_close_together(kb, V, ulps):
 def test_rows_at_the_line_between_eight_and_sixteen_blocks(kb, V, rows):
     l = 1.4 * torch.randn(rows, V, generator=torch.Generator().manual_seed(V + rows))
     _compare(kb, l, 0.5, 0.9)
+
+
+@pytest.mark.parametrize("V", [32000, 65535, 65536, 100003, 152064, 8 * 24576, 8 * 24576 + 1])
+def test_a_row_does_not_depend_on_its_company(kb, V):
+    """A row by itself, among five and among nine: the blocks that share it are not the same, its bits are.  Rows with nothing special
+    about them, with many equal values at the cut, and with more values between the bounds than blocks hand to one another."""
+    g = torch.Generator().manual_seed(V)
+    l = 1.4 * torch.randn(9, V, generator=g)
+    l[1] = torch.round(4 * l[1]) / 4
+    l[2] = 1.0 + torch.randint(0, 41, (V,), generator=g).float() * 2.0 ** -23
+    l[3] = 0.0
+    l[4, V // 2:] = -float("inf")
+    l = l.cuda()
+    for temperature, top_p in ((0.2, 0.85), (1.0, 0.95), (0.7, 2.0)):
+        nine = kb.knnssd_filtered_probs(l, temperature, top_p)
+        five = kb.knnssd_filtered_probs(l[:5].contiguous(), temperature, top_p)
+        assert torch.equal(five, nine[:5])
+        for r in range(9):
+            assert torch.equal(kb.knnssd_filtered_probs(l[r:r + 1].contiguous(), temperature, top_p)[0], nine[r]), r
