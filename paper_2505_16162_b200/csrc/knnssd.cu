@@ -1776,9 +1776,11 @@ knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int 
     const AssignFn assign = vec ? (n <= 4 ? anchors::assign_kernel<true, 4> : n <= 8 ? anchors::assign_kernel<true, 8> : anchors::assign_kernel<true, 16>)
                                 : (n <= 4 ? anchors::assign_kernel<false, 4> : n <= 8 ? anchors::assign_kernel<false, 8> : anchors::assign_kernel<false, 16>);
     const int warps = anchors::assign_warps(N, sm_count());
-    const int assign_smem = n <= 4 ? anchors::assign_smem<4>(warps) : n <= 8 ? anchors::assign_smem<8>(warps) : anchors::assign_smem<16>(warps);
+    auto smem_of = [&](int w) { return n <= 4 ? anchors::assign_smem<4>(w) : n <= 8 ? anchors::assign_smem<8>(w) : anchors::assign_smem<16>(w); };
+    const int assign_smem = smem_of(warps);
     const int staged = N <= anchors::SEL_STAGED, sel_smem = staged ? N * (int)sizeof(double) : 0;
-    ok = ok && cudaFuncSetAttribute(assign, cudaFuncAttributeMaxDynamicSharedMemorySize, assign_smem) == cudaSuccess &&
+    // the limit belongs to the kernel, not to the call: one for all point counts, since other threads may be between their launches
+    ok = ok && cudaFuncSetAttribute(assign, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_of(anchors::MAX_WARPS)) == cudaSuccess &&
          cudaFuncSetAttribute(anchors::select_anchors_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               anchors::SEL_STAGED * (int)sizeof(double)) == cudaSuccess;
     if (!ok) { cudaGetLastError(); cleanup(); return KNNSSD_ERR_CUDA; }
@@ -1800,6 +1802,7 @@ knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int 
             launch_chained(anchors::fold_centroids_kernel, cols, dim3(256), 0, s, part, n, d, S, mu, mu32, ld, r & 1, progress);
         }
         cudaEventRecord(e1, s);
+        if ((e = cudaGetLastError()) != cudaSuccess) break;      // without all of its rounds' launches there are no labels to rank by
         // The anchors are ranked by fp64 distances to the final fp64 centroids (which moved after the last assignment if the round
         // limit ended the iteration).  The ranking goes out behind the rounds: it does nothing while they are not done.
         const int last = r0 + 4 >= max_rounds;

@@ -139,3 +139,35 @@ def test_stand_alone_operators_from_several_threads(kb):
     for w, h in zip(want, got):
         for a, b in zip(w, h, strict=True):
             assert a[:5] == b[:5] and torch.equal(a[5], b[5]) and torch.equal(a[6], b[6])
+
+
+def test_anchors_of_different_point_counts_from_several_threads(kb):
+    """5 clusters of 700 .. 2600 points: the assignment takes blocks of four to eight warps with 48 to 72 KB of shared memory, by one kernel."""
+    g = torch.Generator(device="cuda").manual_seed(5)
+    xs = [torch.randn(n, 260, generator=g, device="cuda") for n in (700, 1000, 1500, 2000, 2300, 2600)]
+
+    def once(x):
+        a = kb.knnssd_build_anchors(x, x[:5].contiguous(), 12, 4)
+        return a["labels"].tolist(), a["anchors"].tolist(), a["centroids"], a["rounds"]
+
+    want, got, errors = [once(x) for x in xs], [[] for _ in xs], []
+    torch.cuda.synchronize()
+
+    def work(i):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(40):
+                    got[i].append(once(xs[i]))
+                torch.cuda.current_stream().synchronize()
+        except Exception as e:
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(len(xs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[:2]
+    for w, hs in zip(want, got):
+        for h in hs:
+            assert w[:2] == h[:2] and torch.equal(w[2], h[2]) and w[3] == h[3]
