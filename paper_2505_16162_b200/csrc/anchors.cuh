@@ -361,5 +361,19 @@ __global__ void __launch_bounds__(SEL_NT) select_anchors_kernel(const double *__
     }
 }
 
+// What the host gets, into pinned memory, behind the ranking: the progress always, the other words (anchors, labels) and the centroids
+// (out_mu, if given) once the rounds are done or the last ones have been.  (All of it copied behind every four rounds, done or not: 36.5 ms for
+// 50 rounds of 300000 x 64, so 35.1.)
+__global__ void __launch_bounds__(256) hand_over_kernel(const int *__restrict__ words, int n_progress, size_t n_words, int *__restrict__ host,
+                                                        const double *__restrict__ mu, size_t n_mu, double *__restrict__ out_mu,
+                                                        const Progress *__restrict__ pg, int last) {
+    chain_wait();
+    const size_t first = (size_t)blockIdx.x * 256 + threadIdx.x, stride = (size_t)gridDim.x * 256;
+    const size_t n = pg->done || last ? n_words : n_progress;
+    for (size_t i = first; i < n; i += stride) host[i] = words[i];
+    if (out_mu && n == n_words)
+        for (size_t i = first; i < n_mu; i += stride) out_mu[i] = mu[i];
+}
+
 }  // namespace anchors
 }  // namespace knnssd

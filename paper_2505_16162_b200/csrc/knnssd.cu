@@ -724,12 +724,12 @@ void free_all(knnssd_ctx *c) {
     for (cudaEvent_t e : c->lin_events) cudaEventDestroy(e);
 }
 
-// Whether a kernel of this session may store floats to a caller's buffer.  What is elsewhere (another device, managed or host
-// memory) or not a multiple of four bytes is left to a copy.
-bool stores_reach(const knnssd_ctx *c, const void *p) {
+// Whether a kernel on `device` may store values of so many bytes to a caller's buffer.  What is elsewhere (another device, managed or
+// host memory) or not at a multiple of their size is left to a copy.
+bool stores_reach(int device, const void *p, size_t bytes) {
     cudaPointerAttributes at{};
-    if ((reinterpret_cast<uintptr_t>(p) & 3u) || cudaPointerGetAttributes(&at, p) != cudaSuccess) { cudaGetLastError(); return false; }
-    return at.type == cudaMemoryTypeDevice && at.device == c->device;
+    if ((reinterpret_cast<uintptr_t>(p) & (bytes - 1)) || cudaPointerGetAttributes(&at, p) != cudaSuccess) { cudaGetLastError(); return false; }
+    return at.type == cudaMemoryTypeDevice && at.device == device;
 }
 
 struct DeviceGuard {
@@ -865,7 +865,7 @@ knnssd_status do_prefill(knnssd_ctx *c, const int *tokens_host, int n, float *po
             pool_accumulate_kernel<<<(d + 255) / 256, 256, 0, s>>>(c->hfinal + (size_t)(M - 1) * d, 1, d, c->pool_sum, 1);
         }
     }
-    const bool direct = pooled_dev && stores_reach(c, pooled_dev);
+    const bool direct = pooled_dev && stores_reach(c->device, pooled_dev, sizeof(float));
     pool_finish_kernel<<<(d + 255) / 256, 256, 0, s>>>(c->pool_sum, d, g.pool_mode == 0 ? 1.0 / (double)n : 1.0, c->pooled, direct ? pooled_dev : nullptr);
     if (pooled_dev && !direct) CUDA_TRY(c, cudaMemcpyAsync(pooled_dev, c->pooled, sizeof(float) * d, cudaMemcpyDeviceToDevice, s));
     emit_first_token_kernel<<<1, 1, 0, s>>>(c->chain, c->state, c->out_tokens, n, c->err_word, c->pinned, c->pinned + kErrWord);
@@ -917,7 +917,7 @@ knnssd_status do_select(knnssd_ctx *c, const float *query_dev, int *domain, int 
 template <bool ACCEPT> cudaError_t deliver(knnssd_ctx *c, Delivery out) {
     cudaError_t e = cudaSuccess;
     for (int r = 0; r < 2; ++r)
-        if (out.n[r] && !stores_reach(c, out.dst[r])) {
+        if (out.n[r] && !stores_reach(c->device, out.dst[r], sizeof(float))) {
             e = cudaMemcpyAsync(out.dst[r], out.src[r], out.n[r] * sizeof(float), cudaMemcpyDeviceToDevice, c->stream);
             if (e != cudaSuccess) return e;
             out.n[r] = 0;
@@ -1758,9 +1758,10 @@ knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int 
     // what the host gets, in one piece: progress, anchors, labels
     constexpr size_t kProgressWords = sizeof(anchors::Progress) / sizeof(int);
     const size_t n_words = kProgressWords + (size_t)n * k + N;
-    int *words = nullptr, *host = host_words(n_words);
-    std::vector<int> pageable;
-    if (!host) { pageable.resize(n_words); host = pageable.data(); }
+    int *words = nullptr, *host = host_words(n_words);      // nullptr: more than is kept pinned, fetched by copies
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return KNNSSD_ERR_CUDA;
+    double *mu_direct = centroids_out_dev && stores_reach(dev, centroids_out_dev, sizeof(double)) ? centroids_out_dev : nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     Scratch mem(s);
     bool ok = mem.get(&mu, (size_t)n * d) && mem.get(&mu32, (size_t)n * ld) && mem.get(&dist, (size_t)N) && mem.get(&part, (size_t)S * n * d) &&
@@ -1775,7 +1776,7 @@ knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int 
     typedef void (*AssignFn)(const float *, int, int, const float *, int, int, int, int *, anchors::Progress *);
     const AssignFn assign = vec ? (n <= 4 ? anchors::assign_kernel<true, 4> : n <= 8 ? anchors::assign_kernel<true, 8> : anchors::assign_kernel<true, 16>)
                                 : (n <= 4 ? anchors::assign_kernel<false, 4> : n <= 8 ? anchors::assign_kernel<false, 8> : anchors::assign_kernel<false, 16>);
-    const int warps = anchors::assign_warps(N, sm_count());
+    const int sms = sm_count(), warps = anchors::assign_warps(N, sms);
     auto smem_of = [&](int w) { return n <= 4 ? anchors::assign_smem<4>(w) : n <= 8 ? anchors::assign_smem<8>(w) : anchors::assign_smem<16>(w); };
     const int assign_smem = smem_of(warps);
     const int staged = N <= anchors::SEL_STAGED, sel_smem = staged ? N * (int)sizeof(double) : 0;
@@ -1788,10 +1789,11 @@ knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int 
     cudaMemsetAsync(mu32, 0, sizeof(float) * n * ld, s);
     cudaMemsetAsync(progress, 0, sizeof(anchors::Progress), s);
     cudaMemsetAsync(labels, 0xFF, sizeof(int) * N, s);           // -1: the first round changes every assignment
+    if (!staged) cudaMemsetAsync(taken, 0, (size_t)N, s);
     anchors::start_centroids_kernel<<<cols, 256, 0, s>>>(init_centroids_dev, d, mu, mu32, ld);
     // rounds are enqueued four at a time: the kernels of rounds after the last one return at once (~2 us each), a look at the
     // outcome of every round cost ~35 us of waiting and copies per round
-    int rounds = 0;
+    anchors::Progress seen{};
     float ms_total = 0.f;
     cudaError_t e = cudaSuccess;
     for (int r0 = 0; r0 < max_rounds && e == cudaSuccess; r0 += 4) {
@@ -1806,27 +1808,37 @@ knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int 
         // The anchors are ranked by fp64 distances to the final fp64 centroids (which moved after the last assignment if the round
         // limit ended the iteration).  The ranking goes out behind the rounds: it does nothing while they are not done.
         const int last = r0 + 4 >= max_rounds;
-        if (!staged) cudaMemsetAsync(taken, 0, (size_t)N, s);
         launch_chained(anchors::member_dist_kernel, dim3((N + 7) / 8), dim3(256), 0, s, x_dev, N, d, mu, labels, dist, progress, last);
         launch_chained(anchors::select_anchors_kernel, dim3(n), dim3(anchors::SEL_NT), sel_smem, s, dist, labels, N, k, staged, taken, out, progress, last);
-        if (centroids_out_dev) e = cudaMemcpyAsync(centroids_out_dev, mu, sizeof(double) * n * d, cudaMemcpyDeviceToDevice, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(host, words, n_words * sizeof(int), cudaMemcpyDeviceToHost, s);
+        if (host) {
+            const size_t most = n_words > (size_t)n * d ? n_words : (size_t)n * d, blocks = (most + 255) / 256;
+            launch_chained(anchors::hand_over_kernel, dim3((unsigned)(blocks < (size_t)sms ? blocks : sms)), dim3(256), 0, s, words, (int)kProgressWords, n_words, host, mu,
+                           (size_t)n * d, mu_direct, progress, last);
+        } else {
+            e = cudaMemcpyAsync(&seen, progress, sizeof(seen), cudaMemcpyDeviceToHost, s);
+        }
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) break;
+        if (host) std::memcpy(&seen, host, sizeof(seen));
         float ms = 0.f;
         cudaEventElapsedTime(&ms, e0, e1);
         ms_total += ms;
-        rounds = host[1];
-        if (host[0]) break;
+        if (seen.done) break;
     }
-    if (e == cudaSuccess) {
+    if (e == cudaSuccess && host) {
         std::memcpy(anchors_host, host + kProgressWords, sizeof(int) * n * k);
         if (labels_host) std::memcpy(labels_host, host + kProgressWords + (size_t)n * k, sizeof(int) * N);
+    } else if (e == cudaSuccess) {
+        e = cudaMemcpyAsync(anchors_host, out, sizeof(int) * n * k, cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess && labels_host) e = cudaMemcpyAsync(labels_host, labels, sizeof(int) * N, cudaMemcpyDeviceToHost, s);
     }
+    if (e == cudaSuccess && centroids_out_dev && !(host && mu_direct))
+        e = cudaMemcpyAsync(centroids_out_dev, mu, sizeof(double) * n * d, cudaMemcpyDeviceToDevice, s);
+    if (e == cudaSuccess && !(host && (mu_direct || !centroids_out_dev))) e = cudaStreamSynchronize(s);
     cleanup();
     if (e != cudaSuccess) { cudaGetLastError(); return KNNSSD_ERR_CUDA; }
-    if (rounds_host) *rounds_host = rounds;
+    if (rounds_host) *rounds_host = seen.rounds;
     if (ms_rounds_host) *ms_rounds_host = ms_total;
     return KNNSSD_OK;
 }

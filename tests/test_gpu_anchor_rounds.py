@@ -46,3 +46,9 @@ def test_rounds_past_a_batch_and_limits_inside_one():
 def test_more_points_than_the_selection_stages():
     _run(25600, 8, 3, 4, 6, 14, 0.4)
     _run(25601, 8, 3, 4, 6, 14, 0.4)
+
+
+def test_more_results_than_are_kept_pinned():
+    """Labels and anchors of 262200 points are more words than a thread keeps pinned: they come by copies, done in one batch or several."""
+    for limit in (2, 6):
+        _run(262200, 4, 3, 4, limit, 15, 1.5)
