@@ -53,12 +53,13 @@ template <bool VEC> __device__ __forceinline__ void copy_piece(float *dst, const
 // the SM with most of the points (blocks of 8 warps leave 48 points on some SMs for 34 on average, of 6 warps 36: 30 us).
 // NC = the cluster count rounded up to 4, 8 or 16: the per-cluster registers follow it.
 template <int NC> constexpr int assign_smem(int warps) { return RING * (2 * warps + NC) * CHUNK * (int)sizeof(float); }
-// Warps per block: the fewest points on the fullest SM, blocks dealt out evenly; the larger block among equals.
-inline int assign_warps(int N, int n_sms) {
+// Warps per block: the fewest rows for the fullest SM, blocks dealt out evenly, each with its points and all n centroids; the larger block
+// among equals.  5 clusters: 5000 x 5120 six warps 67 us a round, eight 71; 300000 x 64 eight 600, six 624, five (the fewest points alone) 628.
+inline int assign_warps(int N, int n, int n_sms) {
     int best = MAX_WARPS;
     long long least = -1;
     for (int w = MAX_WARPS; w >= 4; --w) {
-        const long long blocks = (N + 2 * w - 1) / (2 * w), most = (blocks + n_sms - 1) / n_sms * 2 * w;
+        const long long blocks = (N + 2 * w - 1) / (2 * w), most = (blocks + n_sms - 1) / n_sms * (2 * w + n);
         if (least < 0 || most < least) { least = most; best = w; }
     }
     return best;

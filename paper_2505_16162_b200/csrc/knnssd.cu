@@ -1776,7 +1776,7 @@ knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int 
     typedef void (*AssignFn)(const float *, int, int, const float *, int, int, int, int *, anchors::Progress *);
     const AssignFn assign = vec ? (n <= 4 ? anchors::assign_kernel<true, 4> : n <= 8 ? anchors::assign_kernel<true, 8> : anchors::assign_kernel<true, 16>)
                                 : (n <= 4 ? anchors::assign_kernel<false, 4> : n <= 8 ? anchors::assign_kernel<false, 8> : anchors::assign_kernel<false, 16>);
-    const int sms = sm_count(), warps = anchors::assign_warps(N, sms);
+    const int sms = sm_count(), warps = anchors::assign_warps(N, n, sms);
     auto smem_of = [&](int w) { return n <= 4 ? anchors::assign_smem<4>(w) : n <= 8 ? anchors::assign_smem<8>(w) : anchors::assign_smem<16>(w); };
     const int assign_smem = smem_of(warps);
     const int staged = N <= anchors::SEL_STAGED, sel_smem = staged ? N * (int)sizeof(double) : 0;
@@ -1800,7 +1800,9 @@ knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int 
         cudaEventRecord(e0, s);
         for (int r = r0; r < max_rounds && r < r0 + 4; ++r) {
             launch_chained(assign, dim3((N + 2 * warps - 1) / (2 * warps)), dim3(32 * warps), assign_smem, s, x_dev, N, d, mu32, ld, n, r & 1, labels, progress);
-            launch_chained(anchors::partial_sums_kernel, dim3(cols.x, S), dim3(256), 0, s, x_dev, N, d, labels, n, per, part, r & 1, progress);
+            // not chained: set up under the end of the assignment, its few blocks all go to the SMs that are free first (50000 x 256: 135 us a
+            // round so, 97 .. 99 with all SMs free)
+            anchors::partial_sums_kernel<<<dim3(cols.x, S), 256, 0, s>>>(x_dev, N, d, labels, n, per, part, r & 1, progress);
             launch_chained(anchors::fold_centroids_kernel, cols, dim3(256), 0, s, part, n, d, S, mu, mu32, ld, r & 1, progress);
         }
         cudaEventRecord(e1, s);
