@@ -535,6 +535,17 @@ void reset_mega_state(knnssd_ctx *c) {
     c->bar_total = 0;
 }
 
+// Logits of the rows of x from head_row0 on, and their arg-max.
+void run_head(knnssd_ctx *c, int M, int head_row0, int *argmax_out) {
+    const knnssd_config &g = c->cfg;
+    const int d = g.d_model, V = g.vocab, hm = M - head_row0;
+    float *logits = c->logits + (size_t)head_row0 * V;
+    ctx_linear(c, make_args(c->lm_head, V, d, c->x + (size_t)head_row0 * d, c->final_norm, g.rms_eps, logits, EPI_STORE, hm));
+    launch_chained(argmax_partial_kernel, dim3(kArgmaxBlocks, hm), dim3(256), 0, c->stream, logits, V, kArgmaxBlocks, c->amax_v, c->amax_i);
+    launch_chained(argmax_final_kernel, dim3(hm), dim3(32), 0, c->stream, c->amax_v, c->amax_i, kArgmaxBlocks, argmax_out, V, c->err_word);
+    c->launches += 2;
+}
+
 // One decoder pass over M rows whose token ids are tok_dev[0..M) at positions state.len + pos_off + m.
 //   mask       nullptr = full model, else [2L] with 1 = skipped
 //   head_row0  first row that gets logits and an arg-max (M = no head at all)
@@ -544,7 +555,7 @@ template <typename WT>
 void run_pass_t(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const unsigned char *mask, int head_row0,
                 int *argmax_out, bool want_hidden) {
     const knnssd_config &g = c->cfg;
-    const int d = g.d_model, H = g.n_heads, Hkv = g.n_kv_heads, hd = g.head_dim, F = g.d_ff, V = g.vocab;
+    const int d = g.d_model, H = g.n_heads, Hkv = g.n_kv_heads, hd = g.head_dim, F = g.d_ff;
     const int nq = H * hd, nkv = Hkv * hd;
     cudaStream_t s = c->stream;
     launch_chained(embed_rope_kernel<WT>, dim3(M), dim3(256), 0, s, reinterpret_cast<const WT *>(c->tok_embed), tok_dev, d, c->x, c->state, pos_off,
@@ -587,15 +598,7 @@ void run_pass_t(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const uns
         launch_chained(rmsnorm_rows_kernel, dim3(M), dim3(256), 0, s, c->x, c->final_norm, d, g.rms_eps, c->hfinal);
         c->launches++;
     }
-    if (head_row0 < M) {
-        const int hm = M - head_row0;
-        ctx_linear(c, make_args(c->lm_head, V, d, c->x + (size_t)head_row0 * d, c->final_norm, g.rms_eps,
-                                c->logits + (size_t)head_row0 * V, EPI_STORE, hm));
-        launch_chained(argmax_partial_kernel, dim3(kArgmaxBlocks, hm), dim3(256), 0, s, c->logits + (size_t)head_row0 * V, V, kArgmaxBlocks,
-                                                                      c->amax_v, c->amax_i);
-        launch_chained(argmax_final_kernel, dim3(hm), dim3(32), 0, s, c->amax_v, c->amax_i, kArgmaxBlocks, argmax_out, V, c->err_word);
-        c->launches += 2;
-    }
+    if (head_row0 < M) run_head(c, M, head_row0, argmax_out);
 }
 
 // A model's pass is one launch of small_pass_kernel where a layer's weights are at most this much.  A kernel per operation has eight
@@ -603,6 +606,12 @@ void run_pass_t(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const uns
 // / 16 rows on four layers, one launch against a kernel per operation, us: fp32 3 MB a layer 113 / 136 / 180 against 176 / 246 / 420;
 // 48 MB 208 / 273 / 497 against 277 / 432 / 828; bf16 59 MB 331 / 419 / 935 against 326 / 586 / 1412, 190 MB 691 / 987 / 2141 against 503 / 1032 / 2700.
 constexpr size_t kSmallLayerBytes = (size_t)48 << 20;
+// A head of more ids than this is streamed by launches of its own behind the pass, for the same reason.  Verification calls of 1 / 5 / 9 / 16 rows
+// on two layers, head inside / behind / a kernel per operation, us: fp32, d 1024, 8192 ids 84 / 119 / 139 / 200, 87 / 121 / 161 / 231, 108 /
+// 167 / 276 / 361; 16384 ids 94 / 140 / 162 / 229, 88 / 123 / 164 / 236, 110 / 172 / 275 / 369; 152064 ids 295 / 504 / 566 / 768, 175 / 271 / 410 /
+// 639, 197 / 319 / 527 / 814; d 256, 64000 ids 109 / 125 / 146 / 179, 62 / 88 / 131 / 179, 81 / 122 / 195 / 281; bf16, d 1024, 16384 ids 99 / 137 /
+// 159 / 218, 92 / 111 / 161 / 231, 107 / 127 / 240 / 354.
+constexpr int kSmallHeadIds = 12288;
 
 template <typename WT, int MT> cudaError_t launch_small_t(const small::Args &a, int grid, cudaStream_t s) {
     void *args[] = {const_cast<small::Args *>(&a)};
@@ -628,13 +637,16 @@ void run_pass_small(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const
     a.bar = c->small_bar + c->small_turn; a.next_bar = c->small_bar + (c->small_turn ^ 1); a.err = c->err_word;
     for (int j = 0; mask && j < 2 * g.n_layers; ++j)
         if (mask[j]) a.skip[j >> 5] |= 1u << (j & 31);
+    const bool head_apart = head_row0 < M && g.vocab > kSmallHeadIds;
+    if (head_apart) a.head_row0 = M;
     // a warp per item of the widest map, as far as there are SMs
     int items = (g.n_heads + 2 * g.n_kv_heads) * (g.head_dim / 2);
     if (g.d_ff > items) items = g.d_ff;
-    if (head_row0 < M && (g.vocab + 1) / 2 > items) items = (g.vocab + 1) / 2;
+    if (a.head_row0 < M && (g.vocab + 1) / 2 > items) items = (g.vocab + 1) / 2;
     const int blocks = (items + small::NW - 1) / small::NW, grid = blocks < c->n_sms ? blocks : c->n_sms;
     if ((g.dtype ? launch_small<bf16_t>(a, grid, c->stream) : launch_small<float>(a, grid, c->stream)) == cudaSuccess) c->small_turn ^= 1;
     c->launches++;
+    if (head_apart) run_head(c, M, head_row0, argmax_out);
 }
 
 void run_pass(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const unsigned char *mask, int head_row0,

@@ -41,3 +41,40 @@ def test_rows_around_the_borders_of_a_split_match_the_oracle(name):
         logits = sess.draft(1, want_logits=True)[1]
         assert np.abs(logits.cpu().numpy() - om.forward(rows[:1], n, skip_mask=mask)["logits"]).max() < TOL[shape.dtype], n
         om.forward(rows, n)
+
+
+def _session(kb, shape, w, max_seq):
+    return kb.Session.from_shape(shape, {k: ([t.cuda() for t in v] if isinstance(v, list) else v.cuda()) for k, v in w.items()}, max_seq, max_draft=15)
+
+
+def _launches(sess, call):
+    before = sess.launch_count
+    call()
+    return sess.launch_count - before
+
+
+@pytest.mark.parametrize("name,own_head", [("tiny", False), ("ragged-bf16", False), ("gqa-fp32", False), ("wide-head", True)])
+def test_a_pass_is_one_launch(name, own_head):
+    """And what hands its results back; a large head takes three launches behind it, the arg-max among them."""
+    from paper_2505_16162_b200 import build
+    build.build()
+    from paper_2505_16162_b200 import binding as kb
+    # 61 MB of head
+    shape = si.SHAPES[name] if name in si.SHAPES else si.ModelShape(name, 2, 512, 8, 2, 64, 512, 30011, "fp32", 1e-5, 10000.0)
+    w = si.make_model_weights(shape, 6, gain_spread=0.1)
+    sess = _session(kb, shape, w, 64)
+    prompt = si.uniform_tokens(6, 0, 20, shape.vocab).numpy()
+    sess.prefill(prompt)
+    sess.set_skipmask(si.skip_mask(6, 2 * shape.n_layers, 2))
+    each = 4 if own_head else 1
+    assert _launches(sess, lambda: sess.draft(1)) == each + 1
+    assert _launches(sess, lambda: sess.draft(3)) == 3 * each + 1
+    rows = si.uniform_tokens(6, 1, 5, shape.vocab).numpy()
+    om = oracle.OracleModel(shape, w, 64)
+    om.prefill(prompt)
+    want = om.forward(rows, len(prompt), want_hidden=True)
+    sess.set_pending(int(rows[0]))
+    got = {}
+    assert _launches(sess, lambda: got.update(sess.verify(rows[1:], want_logits=True, want_hidden=True))) == each + 1
+    assert np.abs(got["logits"].cpu().numpy() - want["logits"]).max() < TOL[shape.dtype]
+    assert np.abs(got["hidden"].cpu().numpy() - want["hidden"]).max() < TOL[shape.dtype]
