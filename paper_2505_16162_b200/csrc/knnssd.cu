@@ -612,6 +612,11 @@ constexpr size_t kSmallLayerBytes = (size_t)48 << 20;
 // 639, 197 / 319 / 527 / 814; d 256, 64000 ids 109 / 125 / 146 / 179, 62 / 88 / 131 / 179, 81 / 122 / 195 / 281; bf16, d 1024, 16384 ids 99 / 137 /
 // 159 / 218, 92 / 111 / 161 / 231, 107 / 127 / 240 / 354.
 constexpr int kSmallHeadIds = 12288;
+// Attention of more (head, row, split) tasks than this per SM is a launch of its own in every layer: a block per SM takes them one after the
+// other.  A layer more costs ~8 us of launches.  Four layers, one launch / launches of its own / a kernel per operation, us: 8 heads of 128, fp32,
+// 5 rows at 1000 positions 260 / 262 / 482, at 4000 410 / 383 / 576, 16 rows at 8000 1500 / 1125 / 1125; 16 heads of 64, bf16, 5 rows at 1000
+// 269 / 266 / 331, 16 at 2000 721 / 511 / 740, 16 at 8000 2095 / 995 / 1350.
+constexpr int kSmallTasks = 4;
 
 template <typename WT, int MT> cudaError_t launch_small_t(const small::Args &a, int grid, cudaStream_t s) {
     void *args[] = {const_cast<small::Args *>(&a)};
@@ -634,7 +639,7 @@ void run_pass_small(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const
     a.eps = g.rms_eps; a.st = c->state; a.tok = tok_dev; a.M = M; a.pos_off = pos_off; a.head_row0 = head_row0; a.want_hidden = want_hidden ? 1 : 0;
     a.argmax_out = argmax_out; a.inv_freq = c->inv_freq; a.x = c->x; a.qkv = c->qkv; a.attn = c->attn; a.act = c->act; a.logits = c->logits;
     a.hfinal = c->hfinal; a.part_o = c->part_o; a.part_ml = c->part_ml; a.rope_cs = c->rope_cs; a.n_splits = c->n_splits; a.kc = c->kcache; a.vc = c->vcache;
-    a.bar = c->small_bar + c->small_turn; a.next_bar = c->small_bar + (c->small_turn ^ 1); a.err = c->err_word;
+    a.err = c->err_word;
     for (int j = 0; mask && j < 2 * g.n_layers; ++j)
         if (mask[j]) a.skip[j >> 5] |= 1u << (j & 31);
     const bool head_apart = head_row0 < M && g.vocab > kSmallHeadIds;
@@ -644,8 +649,25 @@ void run_pass_small(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const
     if (g.d_ff > items) items = g.d_ff;
     if (a.head_row0 < M && (g.vocab + 1) / 2 > items) items = (g.vocab + 1) / 2;
     const int blocks = (items + small::NW - 1) / small::NW, grid = blocks < c->n_sms ? blocks : c->n_sms;
-    if ((g.dtype ? launch_small<bf16_t>(a, grid, c->stream) : launch_small<float>(a, grid, c->stream)) == cudaSuccess) c->small_turn ^= 1;
-    c->launches++;
+    auto part = [&](int l_from, int l_to) {
+        a.l_from = l_from; a.l_to = l_to;
+        a.bar = c->small_bar + c->small_turn; a.next_bar = c->small_bar + (c->small_turn ^ 1);
+        if ((g.dtype ? launch_small<bf16_t>(a, grid, c->stream) : launch_small<float>(a, grid, c->stream)) == cudaSuccess) c->small_turn ^= 1;
+        c->launches++;
+    };
+    int l_from = -1;
+    const int end = (c->prefilled ? c->len : 0) + pos_off + M;           // a prompt pass starts from length 0
+    const int tasks = g.n_heads * M * ((end + ATT_CHUNK - 1) / ATT_CHUNK);
+    if (tasks > kSmallTasks * c->n_sms)
+        for (int l = 0; l < g.n_layers; ++l) {
+            if (mask && mask[2 * l]) continue;
+            part(l_from, l);
+            if (g.dtype) small::small_attend_kernel<bf16_t><<<tasks, small::NT, 0, c->stream>>>(a, l);
+            else small::small_attend_kernel<float><<<tasks, small::NT, 0, c->stream>>>(a, l);
+            c->launches++;
+            l_from = l;
+        }
+    part(l_from, g.n_layers);
     if (head_apart) run_head(c, M, head_row0, argmax_out);
 }
 

@@ -3,7 +3,7 @@
 // Models that the streaming pass kernel does not take (fp32 weights, widths that are no multiples of 128) run kernel by kernel.
 // Where a layer's weights are a few MB the work of such a kernel is a microsecond and what it costs is the way from one to
 // the next: 7 launches a layer, ~4.3 us each.  Here the pass is one cooperative launch of at most one block per SM that walks the
-// same operations with a grid-wide meeting between dependent ones, five a layer: the rotary embedding and the K / V rows are
+// same operations with a grid-wide meeting between dependent ones, five a layer (six where a row's context is more than one split): the rotary embedding and the K / V rows are
 // written by the warps that compute the projections (a warp owns the two units of a rotary pair), and a row whose context is one
 // split leaves its attention output without a merge.  Bound by the meetings and the trips to L2 behind them, 3.8 us from one to the
 // next: fp32 tiny shape (4 layers, d 256), five rows: 170 -> 84 us on the device.
@@ -44,6 +44,9 @@ struct Args {
     unsigned *bar, *next_bar;                  // arrivals of this launch's meetings, zero at its start; the next launch's, zeroed by this one
     int *err;
     unsigned skip[MASK_WORDS];                 // bit j: sublayer j is left out
+    // A pass whose attention has launches of its own (small_attend_kernel) comes in parts: from behind the attention of layer l_from
+    // (-1: from the embedding) up to that of layer l_to (n_layers: to the end).
+    int l_from, l_to;
 };
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p) {
@@ -140,13 +143,12 @@ __device__ __forceinline__ void map_rows(const float *x, int M, int K, const flo
 }
 
 // Attention of one (head, row, split of ATT_CHUNK positions) by a block: a thread per position for the scores, then threads by
-// dimension, the positions in NT / hd interleaved runs, whose first PRE values are fetched along with the K rows.  single: the row's
-// context is this split, its output is written at once.
-template <typename WT>
+// dimension, the positions in NT / hd interleaved runs, whose first PRE values are fetched along with the K rows (U float4s of one at a
+// time).  single: the row's context is this split, its output is written at once.
+template <typename WT, int PRE, int U>
 __device__ __forceinline__ void attend(const Args &a, const WT *kc, const WT *vc, int T, int head, int m, int split, bool single, float *s_p, float *s_red) {
     const int t0 = split * ATT_CHUNK;
     if (t0 >= T) return;                                     // uniform over the block
-    constexpr int PRE = 32;
     const int nt = min(T - t0, ATT_CHUNK), tid = threadIdx.x, hd = a.hd, warp = tid >> 5, lane = tid & 31;
     const size_t row0 = (size_t)(head / (a.H / a.Hkv)) * a.max_seq + t0;
     const int runs = NT / hd, e = tid % hd, run = tid / hd;
@@ -160,13 +162,13 @@ __device__ __forceinline__ void attend(const Args &a, const WT *kc, const WT *vc
         const WT *kr = kc + (row0 + tid) * hd;
         float dot = 0.f;
         if (sizeof(WT) == 4) {
-#pragma unroll 16
+#pragma unroll U
             for (int i = 0; i < hd; i += 4) {
                 const float4 k4 = ld_row4(reinterpret_cast<const float *>(kr) + i), q4 = ld_row4(q + i);
                 dot = fmaf(q4.x, k4.x, dot); dot = fmaf(q4.y, k4.y, dot); dot = fmaf(q4.z, k4.z, dot); dot = fmaf(q4.w, k4.w, dot);
             }
         } else {
-#pragma unroll 8
+#pragma unroll (U / 2)
             for (int i = 0; i < hd; i += 8) {
                 const uint4 k8 = __ldcg(reinterpret_cast<const uint4 *>(kr + i));
                 const float4 qa = ld_row4(q + i), qb = ld_row4(q + i + 4);
@@ -220,6 +222,23 @@ __device__ __forceinline__ void attend(const Args &a, const WT *kc, const WT *vc
     __syncthreads();                                         // the next task's
 }
 
+// Attention of layer l for the pass's rows, the first of them at position pos0, by all blocks of the launch.
+template <typename WT, int PRE, int U> __device__ __forceinline__ void attend_rows(const Args &a, int l, int pos0, float *s_p, float *s_red) {
+    const size_t layer = (size_t)l * a.Hkv * a.max_seq * a.hd;
+    const WT *kc = reinterpret_cast<const WT *>(a.kc) + layer, *vc = reinterpret_cast<const WT *>(a.vc) + layer;
+    const int M = a.M, n_split = (pos0 + M + ATT_CHUNK - 1) / ATT_CHUNK;      // of the pass's last row
+    for (int task = blockIdx.x; task < a.H * M * n_split; task += gridDim.x)
+        attend<WT, PRE, U>(a, kc, vc, pos0 + task / a.H % M + 1, task % a.H, task / a.H % M, task / (a.H * M), n_split == 1, s_p, s_red);
+}
+
+// The same as a launch of its own, for many tasks: four blocks on an SM, which hide their latencies in one another, where small_pass_kernel
+// has one with everything in flight that it can (two with the same: 16 rows at 8000 positions, four layers of 16 heads of 64, bf16, 1382 us; so 995).
+// Bit for bit what that leaves.
+template <typename WT> __global__ void __launch_bounds__(NT, 4) small_attend_kernel(const __grid_constant__ Args a, int l) {
+    __shared__ float s_p[NT], s_red[2 * NW];
+    attend_rows<WT, 8, 8>(a, l, a.st->len + a.pos_off, s_p, s_red);
+}
+
 template <typename WT, int MT>
 __global__ void __launch_bounds__(NT, 1) small_pass_kernel(const __grid_constant__ Args a) {
     __shared__ float s_rinv[MT], s_p[NT], s_red[2 * NW];
@@ -232,23 +251,25 @@ __global__ void __launch_bounds__(NT, 1) small_pass_kernel(const __grid_constant
     }
     const int pos0 = a.st->len + a.pos_off;
 
-    // embedding rows, and (from the last block on) the rows' rotary angles, in fp64
-    for (int m = blockIdx.x; m < M; m += gridDim.x) {
-        int t = a.tok[m];
-        if (t < 0 || t >= a.V) {                             // never gather outside the table: report and read row 0 instead
-            if (tid == 0) atomicExch(a.err, ERR_BAD_TOKEN);
-            t = 0;
+    if (a.l_from < 0) {
+        // embedding rows, and (from the last block on) the rows' rotary angles, in fp64
+        for (int m = blockIdx.x; m < M; m += gridDim.x) {
+            int t = a.tok[m];
+            if (t < 0 || t >= a.V) {                         // never gather outside the table: report and read row 0 instead
+                if (tid == 0) atomicExch(a.err, ERR_BAD_TOKEN);
+                t = 0;
+            }
+            const WT *row = reinterpret_cast<const WT *>(a.tok_embed) + (size_t)t * d;
+            for (int i = tid; i < d; i += NT) a.x[(size_t)m * d + i] = WeightLoad<WT>::load1(row + i);
         }
-        const WT *row = reinterpret_cast<const WT *>(a.tok_embed) + (size_t)t * d;
-        for (int i = tid; i < d; i += NT) a.x[(size_t)m * d + i] = WeightLoad<WT>::load1(row + i);
+        for (int m = gridDim.x - 1 - blockIdx.x; m < M; m += gridDim.x)
+            for (int i = tid; i < half; i += NT) {
+                double s, c;
+                sincos((double)(pos0 + m) * a.inv_freq[i], &s, &c);
+                a.rope_cs[m * half + i] = make_float2((float)c, (float)s);
+            }
+        if (!meet_grid(a, met, &s_abort)) return;
     }
-    for (int m = gridDim.x - 1 - blockIdx.x; m < M; m += gridDim.x)
-        for (int i = tid; i < half; i += NT) {
-            double s, c;
-            sincos((double)(pos0 + m) * a.inv_freq[i], &s, &c);
-            a.rope_cs[m * half + i] = make_float2((float)c, (float)s);
-        }
-    if (!meet_grid(a, met, &s_abort)) return;
 
     const int n_split = (pos0 + M + ATT_CHUNK - 1) / ATT_CHUNK;      // of the pass's last row
     auto pair_rows = [&](const void *W, int K, int n, int item, const WT *&r0, const WT *&r1) {      // units 2 item and 2 item + 1 of n
@@ -261,42 +282,44 @@ __global__ void __launch_bounds__(NT, 1) small_pass_kernel(const __grid_constant
         *reinterpret_cast<float2 *>(a.x + (size_t)m * d + 2 * item) = make_float2(old.x + v0, old.y + v1);
     };
     auto nothing = [&](int, int) { return make_float2(0.f, 0.f); };
-    for (int l = 0; l < a.n_layers; ++l) {
+    for (int l = max(a.l_from, 0); l < a.n_layers; ++l) {
         const LayerW &ly = a.layers[l];
         if (!(a.skip[l >> 4] >> (2 * (l & 15)) & 1u)) {
-            WT *kc = reinterpret_cast<WT *>(a.kc) + (size_t)l * a.Hkv * a.max_seq * hd, *vc = reinterpret_cast<WT *>(a.vc) + (size_t)l * a.Hkv * a.max_seq * hd;
-            map_rows<WT, MT, true>(a.x, M, d, ly.attn_norm, a.eps, slots * half,
-                             [&](int item, const WT *&r0, const WT *&r1) {
-                                 int slot = item / half;
-                                 const void *W = ly.wq;
-                                 if (slot >= a.H) { W = ly.wk; slot -= a.H; if (slot >= a.Hkv) { W = ly.wv; slot -= a.Hkv; } }
-                                 r0 = reinterpret_cast<const WT *>(W) + (size_t)(slot * hd + item % half) * d;
-                                 r1 = r0 + (size_t)half * d;
-                             },
-                             [&](int item, int m) { return __ldcg(a.rope_cs + m * half + item % half); },
-                             [&](int item, int m, float p, float q, float2 c) {
-                                 const int slot = item / half, i = item % half;
-                                 if (slot < a.H + a.Hkv) {
-                                     // the rounding is spelled out, so that it is the same in every instance of the kernel
-                                     const float rp = __fmaf_rn(p, c.x, -__fmul_rn(q, c.y));
-                                     q = __fmaf_rn(q, c.x, __fmul_rn(p, c.y));
-                                     p = rp;
-                                 }
-                                 if (slot < a.H) {
-                                     float *dst = a.qkv + (size_t)m * slots * hd + (size_t)slot * hd + i;
-                                     dst[0] = p;
-                                     dst[half] = q;
-                                 } else {
-                                     const bool is_k = slot < a.H + a.Hkv;
-                                     WT *dst = (is_k ? kc : vc) + ((size_t)(slot - a.H - (is_k ? 0 : a.Hkv)) * a.max_seq + pos0 + m) * hd + i;
-                                     WeightLoad<WT>::store1(dst, p);
-                                     WeightLoad<WT>::store1(dst + half, q);
-                                 }
-                             });
-            if (!meet_grid(a, met, &s_abort)) return;
-            for (int task = blockIdx.x; task < a.H * M * n_split; task += gridDim.x)
-                attend<WT>(a, kc, vc, pos0 + task / a.H % M + 1, task % a.H, task / a.H % M, task / (a.H * M), n_split == 1, s_p, s_red);
-            if (!meet_grid(a, met, &s_abort)) return;
+            if (l != a.l_from) {
+                WT *kc = reinterpret_cast<WT *>(a.kc) + (size_t)l * a.Hkv * a.max_seq * hd, *vc = reinterpret_cast<WT *>(a.vc) + (size_t)l * a.Hkv * a.max_seq * hd;
+                map_rows<WT, MT, true>(a.x, M, d, ly.attn_norm, a.eps, slots * half,
+                                 [&](int item, const WT *&r0, const WT *&r1) {
+                                     int slot = item / half;
+                                     const void *W = ly.wq;
+                                     if (slot >= a.H) { W = ly.wk; slot -= a.H; if (slot >= a.Hkv) { W = ly.wv; slot -= a.Hkv; } }
+                                     r0 = reinterpret_cast<const WT *>(W) + (size_t)(slot * hd + item % half) * d;
+                                     r1 = r0 + (size_t)half * d;
+                                 },
+                                 [&](int item, int m) { return __ldcg(a.rope_cs + m * half + item % half); },
+                                 [&](int item, int m, float p, float q, float2 c) {
+                                     const int slot = item / half, i = item % half;
+                                     if (slot < a.H + a.Hkv) {
+                                         // the rounding is spelled out, so that it is the same in every instance of the kernel
+                                         const float rp = __fmaf_rn(p, c.x, -__fmul_rn(q, c.y));
+                                         q = __fmaf_rn(q, c.x, __fmul_rn(p, c.y));
+                                         p = rp;
+                                     }
+                                     if (slot < a.H) {
+                                         float *dst = a.qkv + (size_t)m * slots * hd + (size_t)slot * hd + i;
+                                         dst[0] = p;
+                                         dst[half] = q;
+                                     } else {
+                                         const bool is_k = slot < a.H + a.Hkv;
+                                         WT *dst = (is_k ? kc : vc) + ((size_t)(slot - a.H - (is_k ? 0 : a.Hkv)) * a.max_seq + pos0 + m) * hd + i;
+                                         WeightLoad<WT>::store1(dst, p);
+                                         WeightLoad<WT>::store1(dst + half, q);
+                                     }
+                                 });
+                if (l == a.l_to) return;
+                if (!meet_grid(a, met, &s_abort)) return;
+                attend_rows<WT, 32, 16>(a, l, pos0, s_p, s_red);
+                if (!meet_grid(a, met, &s_abort)) return;
+            }
             if (n_split > 1) {
                 for (int task = blockIdx.x; task < a.H * M; task += gridDim.x) {
                     const int m = task / a.H, ns = (pos0 + m + ATT_CHUNK) / ATT_CHUNK;

@@ -78,3 +78,57 @@ def test_a_pass_is_one_launch(name, own_head):
     assert _launches(sess, lambda: got.update(sess.verify(rows[1:], want_logits=True, want_hidden=True))) == each + 1
     assert np.abs(got["logits"].cpu().numpy() - want["logits"]).max() < TOL[shape.dtype]
     assert np.abs(got["hidden"].cpu().numpy() - want["hidden"]).max() < TOL[shape.dtype]
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+def test_attention_launches_of_its_own_leave_the_same(dtype):
+    """Ten splits of context for 16 rows of 16 heads are more attention tasks than the one launch takes, for one row they are not: the
+    first row of either has the same bits, and all agree with the oracle."""
+    from paper_2505_16162_b200 import build
+    build.build()
+    from paper_2505_16162_b200 import binding as kb
+    shape = si.ModelShape("long", 2, 264, 16, 4, 64, 264, 515, dtype, 1e-5, 10000.0)
+    w = si.make_model_weights(shape, 8, gain_spread=0.1)
+    om = oracle.OracleModel(shape, w, 2600)
+    sess = _session(kb, shape, w, 2600)
+    prompt = si.uniform_tokens(8, 0, 2500, shape.vocab).numpy()
+    want_pooled = om.prefill(prompt)[0]
+    first, pooled = sess.prefill(prompt, want_pooled=True)
+    assert np.abs(pooled.cpu().numpy() - want_pooled).max() < TOL[dtype]
+    for n in (2500, 2304, 2303, 300):
+        rows = si.uniform_tokens(8, 100 + n, 16, shape.vocab).numpy()
+        want = om.forward(rows, n, want_hidden=True)
+        one = {}
+        for k in (15, 0):
+            sess.set_length(n)
+            sess.set_pending(int(rows[0]))
+            got = {}
+            n_launches = _launches(sess, lambda: got.update(sess.verify(rows[1:k + 1], want_logits=True, want_hidden=True)))
+            assert n_launches == (2 + 2 * shape.n_layers if k and n > 300 else 2), (n, k)
+            assert np.abs(got["logits"].cpu().numpy() - want["logits"][:k + 1]).max() < TOL[dtype], (n, k)
+            assert np.abs(got["hidden"].cpu().numpy() - want["hidden"][:k + 1]).max() < TOL[dtype], (n, k)
+            one[k] = got
+        assert torch.equal(one[15]["logits"][:1], one[0]["logits"]) and torch.equal(one[15]["hidden"][:1], one[0]["hidden"])
+
+
+def test_sublayers_left_out_of_a_pass_in_parts():
+    """120 heads: a draft step of one row at 1100 positions comes in parts too, whichever of its sublayers are left out."""
+    from paper_2505_16162_b200 import build
+    build.build()
+    from paper_2505_16162_b200 import binding as kb
+    shape = si.ModelShape("heads", 3, 136, 120, 4, 64, 136, 301, "fp32", 1e-5, 10000.0)
+    w = si.make_model_weights(shape, 9, gain_spread=0.1)
+    om = oracle.OracleModel(shape, w, 1160)
+    sess = _session(kb, shape, w, 1160)
+    prompt = si.uniform_tokens(9, 0, 1100, shape.vocab).numpy()
+    om.prefill(prompt)
+    sess.prefill(prompt)
+    rows = si.uniform_tokens(9, 1, 2, shape.vocab).numpy()
+    for mask in ([0, 0, 0, 0, 0, 0], [1, 0, 0, 1, 0, 0], [0, 1, 1, 0, 1, 0], [1, 1, 1, 1, 1, 1], [0, 0, 0, 0, 1, 1]):
+        mask = np.array(mask, np.uint8)
+        sess.set_skipmask(mask)
+        sess.set_pending(int(rows[0]))
+        got = []
+        n_launches = _launches(sess, lambda: got.append(sess.draft(1, want_logits=True)[1]))
+        assert n_launches == 2 + 2 * int((mask[::2] == 0).sum())
+        assert np.abs(got[0].cpu().numpy() - om.forward(rows[:1], len(prompt), skip_mask=mask)["logits"]).max() < TOL["fp32"], mask
