@@ -217,7 +217,8 @@ knnssd_status knnssd_mask_objective(knnssd_ctx *ctx, const unsigned char *masks_
  * step each (or verify passes over k+1 rows) without committing anything, bracketed by CUDA events on the context's
  * stream, and returns the mean milliseconds per pass.  which: 0 = draft step, 1 = verify pass over k+1 rows.
  * Also returns how many kernels one such pass launches and the mean device milliseconds spent per pass inside the
- * weight-streaming linear kernels alone (events around each of them in a separate, untimed replay).
+ * weight-streaming linear kernels alone (events around each of them in a separate, untimed replay).  Models whose pass is one launch
+ * are replayed with a kernel per operation; in the persistent pass kernel the linear maps have no launches, and both numbers are 0.
  */
 knnssd_status knnssd_time_pass(knnssd_ctx *ctx, int which, int k, int iters, float *ms_per_pass,
                                int *launches_per_pass, float *ms_linear_per_pass, int *linear_launches_per_pass);

@@ -671,12 +671,17 @@ void run_pass_small(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const
     if (head_apart) run_head(c, M, head_row0, argmax_out);
 }
 
+// One pass, a kernel per operation.
+void run_operations(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const unsigned char *mask, int head_row0, int *argmax_out, bool want_hidden) {
+    if (c->cfg.dtype) run_pass_t<bf16_t>(c, M, tok_dev, pos_off, mask, head_row0, argmax_out, want_hidden);
+    else run_pass_t<float>(c, M, tok_dev, pos_off, mask, head_row0, argmax_out, want_hidden);
+}
+
 void run_pass(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const unsigned char *mask, int head_row0,
               int *argmax_out, bool want_hidden) {
     if (c->mega_ok && M <= pass::MAXM) { run_pass_mega(c, M, tok_dev, pos_off, mask, head_row0, argmax_out, want_hidden); return; }
     if (c->small_ok) { run_pass_small(c, M, tok_dev, pos_off, mask, head_row0, argmax_out, want_hidden); return; }
-    if (c->cfg.dtype) run_pass_t<bf16_t>(c, M, tok_dev, pos_off, mask, head_row0, argmax_out, want_hidden);
-    else run_pass_t<float>(c, M, tok_dev, pos_off, mask, head_row0, argmax_out, want_hidden);
+    run_operations(c, M, tok_dev, pos_off, mask, head_row0, argmax_out, want_hidden);
 }
 
 knnssd_status sync_check(knnssd_ctx *c, const char *what) {
@@ -1550,10 +1555,12 @@ knnssd_status knnssd_time_pass(knnssd_ctx *c, int which, int k, int iters, float
     if (st != KNNSSD_OK) return st;
     if (ms_per_pass) *ms_per_pass = elapsed_ms(c) / (float)iters;
     if (launches_per_pass) *launches_per_pass = launches;
-    // separate replay with events around every linear kernel
+    // separate replay with events around every linear kernel; a model whose pass is one launch is replayed kernel by kernel
     c->time_linear = true;
     c->lin_used = 0;
-    one();
+    if (!c->small_ok) one();
+    else if (which == 0) run_operations(c, 1, c->chain, 0, c->active_mask.data(), 0, c->target, false);
+    else run_operations(c, k + 1, c->chain, 0, nullptr, 0, c->target, false);
     c->time_linear = false;
     st = sync_check(c, "time_pass linear replay");
     if (st != KNNSSD_OK) return st;

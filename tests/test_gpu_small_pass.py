@@ -78,6 +78,9 @@ def test_a_pass_is_one_launch(name, own_head):
     assert _launches(sess, lambda: got.update(sess.verify(rows[1:], want_logits=True, want_hidden=True))) == each + 1
     assert np.abs(got["logits"].cpu().numpy() - want["logits"]).max() < TOL[shape.dtype]
     assert np.abs(got["hidden"].cpu().numpy() - want["hidden"]).max() < TOL[shape.dtype]
+    timed = sess.time_pass(1, 4, 2)
+    assert timed["launches"] == each
+    assert timed["linear_launches"] == 4 * shape.n_layers + 1 and timed["ms_linear"] > 0        # replayed kernel by kernel
 
 
 @pytest.mark.parametrize("dtype", ["fp32", "bf16"])
