@@ -1,5 +1,7 @@
 """Session calls while the session's stream is being captured: refused before anything has moved, the capture goes on, and the next call
 equals one from a session that never saw a capture."""
+import gc
+
 import numpy as np
 import pytest
 import torch
@@ -33,12 +35,17 @@ def test_calls_are_refused_while_the_stream_is_captured(name):
              lambda: s.set_pending(1)]
     launches = s.launch_count
     graph, kept = torch.cuda.CUDAGraph(), torch.zeros(4, device="cuda")
-    with torch.cuda.graph(graph, stream=stream):
-        kept.add_(1)
-        for call in calls:                                           # an odd number of passes each, for the first two
-            with pytest.raises(kb.KnnssdError) as e:
-                call()
-            assert e.value.status == 6
+    gc.collect()
+    gc.disable()                                                     # a session of another test that goes away now would end the capture
+    try:
+        with torch.cuda.graph(graph, stream=stream):
+            kept.add_(1)
+            for call in calls:                                       # an odd number of passes each, for the first two
+                with pytest.raises(kb.KnnssdError) as e:
+                    call()
+                assert e.value.status == 6
+    finally:
+        gc.enable()
     graph.replay()
     torch.cuda.synchronize()
     assert kept.tolist() == [1.0] * 4                                # the capture was not spoiled

@@ -43,11 +43,8 @@ def test_a_norm_is_the_same_bits_whichever_kernel_sums_it(rows):
     w["w_down"][0].zero_()
     w1 = {k: (v[1:] if isinstance(v, list) else v) for k, v in w.items()}
     prompt = si.uniform_tokens(9, 0, rows, two.vocab).numpy()
-    tokens = si.uniform_tokens(9, 1, 4, two.vocab).numpy()
     got = []
     for shape, weights in ((two, w), (one, w1)):
         sess = kb.Session.from_shape(shape, weights, 400, max_draft=4)
-        first, pooled = sess.prefill(prompt, want_pooled=True)
-        sess.set_pending(int(tokens[0]))
-        got.append((first, pooled, sess.verify(tokens[1:], want_logits=True)["logits"]))
-    assert got[0][0] == got[1][0] and torch.equal(got[0][1], got[1][1]) and torch.equal(got[0][2], got[1][2])
+        got.append(sess.prefill(prompt, want_pooled=True))
+    assert got[0][0] == got[1][0] and torch.equal(got[0][1], got[1][1])
