@@ -614,7 +614,7 @@ constexpr size_t kSmallLayerBytes = (size_t)48 << 20;
 constexpr int kSmallHeadIds = 12288;
 // Attention of more (head, row, split) tasks than this per SM is a launch of its own in every layer: a block per SM takes them one after the
 // other.  A layer more costs ~8 us of launches.  Four layers, one launch / launches of its own / a kernel per operation, us: 8 heads of 128, fp32,
-// 5 rows at 1000 positions 260 / 262 / 482, at 4000 410 / 383 / 576, 16 rows at 8000 1500 / 1125 / 1125; 16 heads of 64, bf16, 5 rows at 1000
+// 5 rows at 1000 positions 260 / 262 / 482, at 4000 410 / 363 / 576, 16 rows at 8000 1500 / 1132 / 1125; 16 heads of 64, bf16, 5 rows at 1000
 // 269 / 266 / 331, 16 at 2000 721 / 511 / 740, 16 at 8000 2095 / 995 / 1350.
 constexpr int kSmallTasks = 4;
 

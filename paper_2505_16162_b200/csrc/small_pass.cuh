@@ -231,12 +231,13 @@ template <typename WT, int PRE, int U> __device__ __forceinline__ void attend_ro
         attend<WT, PRE, U>(a, kc, vc, pos0 + task / a.H % M + 1, task % a.H, task / a.H % M, task / (a.H * M), n_split == 1, s_p, s_red);
 }
 
-// The same as a launch of its own, for many tasks: four blocks on an SM, which hide their latencies in one another, where small_pass_kernel
-// has one with everything in flight that it can (two with the same: 16 rows at 8000 positions, four layers of 16 heads of 64, bf16, 1382 us; so 995).
-// Bit for bit what that leaves.
-template <typename WT> __global__ void __launch_bounds__(NT, 4) small_attend_kernel(const __grid_constant__ Args a, int l) {
+// The same as a launch of its own, for many tasks: four blocks on an SM (fp32: three, whose rows are twice as long), which hide their latencies in
+// one another, where small_pass_kernel has one with everything in flight that it can.  Bit for bit what that leaves.  Passes of 5 / 9 / 16 rows
+// at 8000 positions, four layers of 16 heads of 64, two blocks as in small_pass_kernel / three / four, us: bf16 611 / 894 / 1382, 474 / 676 / 1094, 453 /
+// 642 / 995; fp32 491 / 728 / 1206, 462 / 695 / 1134, 471 / 685 / 1110, of 8 heads of 128 532 / 758 / 1196, 489 / 715 / 1132, 523 / 728 / 1125.
+template <typename WT> __global__ void __launch_bounds__(NT, sizeof(WT) == 4 ? 3 : 4) small_attend_kernel(const __grid_constant__ Args a, int l) {
     __shared__ float s_p[NT], s_red[2 * NW];
-    attend_rows<WT, 8, 8>(a, l, a.st->len + a.pos_off, s_p, s_red);
+    attend_rows<WT, sizeof(WT) == 4 ? 16 : 8, 8>(a, l, a.st->len + a.pos_off, s_p, s_red);
 }
 
 template <typename WT, int MT>
