@@ -19,8 +19,10 @@
  * The stand-alone operators below take their scratch from a memory pool of the
  * library, one per device, in the order of the caller's stream.  It keeps up to 96 MB
  * between calls (more than that goes back at the next synchronisation) and is emptied
- * by knnssd_destroy.  Their small arguments and results pass through 256 bytes of pinned
- * memory per host thread, made by the thread's first such call.
+ * by knnssd_destroy.  Their small arguments and results pass through pinned memory, one piece per
+ * host thread: 256 bytes, made by the thread's first such call and kept until the thread ends.
+ * knnssd_build_anchors makes it anew, up to 1 MB, when a call's labels and anchors need more than
+ * the thread has; results that need more than 1 MB come by copies.
  *
  * Notation follows the paper: L decoder layers = 2L sublayers; a skip mask
  * z in {0,1}^{2L} with z[j] = 1 meaning "sublayer j is skipped while drafting"

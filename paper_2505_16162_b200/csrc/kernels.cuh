@@ -17,7 +17,7 @@ typedef unsigned short bf16_t;  // raw bf16 bit pattern
 // Kernels that follow one another closely are launched with programmatic stream serialisation: a kernel may be set up on
 // the SMs while the one before it still runs.  Each of them lets its successor come and then waits until the one before it
 // has finished and its writes are visible, before it touches any memory; with an ordinary launch both do nothing.
-// (The fp32 verification pass of 36 kernels of 2 .. 10 us: 279 -> 217 us; a prompt of 77 rows, 8 layers of the 7B widths:
+// (A verification pass of an fp32 model, run as 36 kernels of 2 .. 10 us: 279 -> 217 us; a prompt of 77 rows, 8 layers of the 7B widths:
 // 1.68 -> 1.62 ms.)
 __device__ __forceinline__ void chain_wait() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -951,7 +951,6 @@ knnssd_status do_select(knnssd_ctx *c, const float *query_dev, int *domain, int 
     return KNNSSD_OK;
 }
 
-// Enqueue k draft steps: step j reads chain[j] at position len + j and writes chain[j + 1].
 // A call's results in one launch (see deliver_kernel); its words end up in c->pinned, the error word in its place there.
 template <bool ACCEPT> cudaError_t deliver(knnssd_ctx *c, Delivery out) {
     cudaError_t e = cudaSuccess;
@@ -968,13 +967,14 @@ template <bool ACCEPT> cudaError_t deliver(knnssd_ctx *c, Delivery out) {
     return e;
 }
 
+// Enqueue k draft steps: step j reads chain[j] at position len + j and writes chain[j + 1].
 void enqueue_draft(knnssd_ctx *c, int k) {
     for (int j = 0; j < k; ++j) run_pass(c, 1, c->chain + j, j, c->active_mask.data(), 0, c->chain + j + 1, false);
 }
 
 // Enqueue the verification pass over chain[0..k] and the accept/rollback step.
-void enqueue_verify(knnssd_ctx *c, int k, bool want_hidden, int round_idx) {
-    run_pass(c, k + 1, c->chain, 0, nullptr, 0, c->target, want_hidden);
+void enqueue_verify(knnssd_ctx *c, int k, int round_idx) {
+    run_pass(c, k + 1, c->chain, 0, nullptr, 0, c->target, false);
     launch_chained(accept_kernel, dim3(1), dim3(32), 0, c->stream, c->chain, c->target, k, c->state, c->out_tokens, c->cfg.max_seq, c->accept_log,
                                            round_idx);
     c->launches++;
@@ -1290,7 +1290,7 @@ static knnssd_status do_decode(knnssd_ctx *c, int max_new, int k, int use_select
         cudaEventRecord(c->ev0, s);
         enqueue_draft(c, keff);
         cudaEventRecord(c->ev1, s);
-        enqueue_verify(c, keff, false, round);
+        enqueue_verify(c, keff, round);
         cudaEventRecord(c->ev2, s);
         CUDA_TRY(c, cudaMemcpyAsync(c->pinned, c->state, sizeof(DeviceState), cudaMemcpyDeviceToHost, s));
         CUDA_TRY(c, cudaMemcpyAsync(c->pinned + 8, c->err_word, sizeof(int), cudaMemcpyDeviceToHost, s));

@@ -40,7 +40,7 @@ constexpr int BOX_N = 64;                             // weight rows per TMA box
 constexpr int BK = 64;                                // input columns per stage: 128 bytes of bf16 = one swizzle row
 constexpr int W_BYTES = 128 * BK * 2;                 // a CTA's weight rows of a stage
 // The ring of stages.  A stage is what a CTA holds of a k-block: 128 weight rows and half of the tile's token rows of either
-// plane, 48 KB at 256 tokens (four stages), 26 KB at 80 (seven).
+// plane, 48 KB at 256 tokens (four stages), 28 KB at 96 (six).
 constexpr int RING_BYTES = 192 * 1024;
 constexpr int MAX_STAGES = 10;
 __host__ __device__ constexpr int stage_bytes_of(int tt) { return W_BYTES + tt * BK * 2; }
