@@ -606,44 +606,84 @@ __global__ void put_tokens_kernel(const Tokens t, int n, int *__restrict__ chain
 // Eq. (4) in one launch: dot(v, a) / (|v| |a|) by a block per anchor; then the block that finishes last takes the arg-max of all
 // n, lowest index on ties.  cosines[n] and work[2] (blocks done, a zero or non-finite norm was met) are scratch; work is zero
 // between launches.  out[0] = best flat index, out[1] = its cosine's bits, out[2] = the flag; it may be pinned host memory.
-// Bound by latencies: 16 bytes a load where query and rows allow it, 50 x 5120: 5 us (a warp per anchor, 4 bytes a load: 10).
-// grid = n, 256 threads.
-__global__ void __launch_bounds__(256) cosine_top1_kernel(const float *__restrict__ v, const float *__restrict__ anchors, int n, int d,
+// Bound by latencies: 16 bytes a load where query and rows allow it, 50 x 5120: 5 us (a warp per anchor, 4 bytes a load: 10).  More anchors than
+// blocks are resident, of rows that a block has one piece of per thread, go to a warp each, which takes the shares of the block's warps one
+// after the other (WARPS): the sums are the same.  A call of 4096 x 640 / 20000 x 640 / 100000 x 64 / 100000 x 1024: a block per anchor 35 / 61 /
+// 191 / 237 us, so 31 / 43 / 79 / 139.  grid = n, or ceil(n / 8) of WARPS, 256 threads.
+template <bool WARPS> __global__ void __launch_bounds__(256) cosine_top1_kernel(const float *__restrict__ v, const float *__restrict__ anchors, int n, int d,
                                                           float *__restrict__ cosines, int *__restrict__ work, int *__restrict__ out) {
     __shared__ float s_v[8];
     __shared__ int s_i[8];
     __shared__ float s_sum[3][8];
     __shared__ int s_last;
-    const int tid = threadIdx.x, a = blockIdx.x;
-    const float *ar = anchors + (size_t)a * d;
-    float dot = 0.f, vv = 0.f, aa = 0.f;
-    auto take = [&](float x, float y) {
-        dot = fmaf(x, y, dot);
-        vv = fmaf(x, x, vv);
-        aa = fmaf(y, y, aa);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool vec = ((reinterpret_cast<uintptr_t>(v) | reinterpret_cast<uintptr_t>(anchors)) & 15u) == 0 && d % 4 == 0;
+    const int cols = vec ? d / 4 : d;
+    auto take = [](float (&sum)[3], float x, float y) {          // dot, |v|^2, |a|^2
+        sum[0] = fmaf(x, y, sum[0]);
+        sum[1] = fmaf(x, x, sum[1]);
+        sum[2] = fmaf(y, y, sum[2]);
     };
-    if (((reinterpret_cast<uintptr_t>(v) | reinterpret_cast<uintptr_t>(anchors)) & 15u) == 0 && d % 4 == 0) {
-#pragma unroll 5
-        for (int i = tid; i < d / 4; i += 256) {
-            const float4 x = reinterpret_cast<const float4 *>(v)[i], y = reinterpret_cast<const float4 *>(ar)[i];
-            take(x.x, y.x); take(x.y, y.y); take(x.z, y.z); take(x.w, y.w);
-        }
-    } else {
-#pragma unroll 4
-        for (int i = tid; i < d; i += 256) take(v[i], ar[i]);
-    }
-    dot = warp_sum(dot); vv = warp_sum(vv); aa = warp_sum(aa);
-    if ((tid & 31) == 0) { s_sum[0][tid >> 5] = dot; s_sum[1][tid >> 5] = vv; s_sum[2][tid >> 5] = aa; }
-    __syncthreads();
-    if (tid == 0) {
-#pragma unroll
-        for (int w = 1; w < 8; ++w) { dot += s_sum[0][w]; vv += s_sum[1][w]; aa += s_sum[2][w]; }
+    auto take4 = [&](float (&sum)[3], const float *ar, int i) {
+        const float4 x = reinterpret_cast<const float4 *>(v)[i], y = reinterpret_cast<const float4 *>(ar)[i];
+        take(sum, x.x, y.x); take(sum, x.y, y.y); take(sum, x.z, y.z); take(sum, x.w, y.w);
+    };
+    auto finish = [&](int a, float dot, float vv, float aa) {
         const bool bad = !(vv > 0.f) || !isfinite(vv) || !(aa > 0.f) || !isfinite(aa);
         __stcg(cosines + a, bad ? -INFINITY : (float)((double)dot / sqrt((double)vv * (double)aa)));      // one rounding
         if (bad) atomicExch(work + 1, 1);
         __threadfence();
-        s_last = atomicAdd(work, 1) == (int)gridDim.x - 1;
+    };
+    if (!WARPS) {
+        const float *ar = anchors + (size_t)blockIdx.x * d;
+        float sum[3] = {0.f, 0.f, 0.f};
+        if (vec) {
+#pragma unroll 5
+            for (int i = tid; i < cols; i += 256) take4(sum, ar, i);
+        } else {
+#pragma unroll 4
+            for (int i = tid; i < cols; i += 256) take(sum, v[i], ar[i]);
+        }
+#pragma unroll
+        for (int e = 0; e < 3; ++e) { sum[e] = warp_sum(sum[e]); if (lane == 0) s_sum[e][warp] = sum[e]; }
+        __syncthreads();
+        if (tid == 0) {
+#pragma unroll
+            for (int w = 1; w < 8; ++w)
+#pragma unroll
+                for (int e = 0; e < 3; ++e) sum[e] += s_sum[e][w];
+            finish(blockIdx.x, sum[0], sum[1], sum[2]);
+        }
+    } else {
+        const int a = blockIdx.x * 8 + warp;
+        if (a < n) {
+            const float *ar = anchors + (size_t)a * d;
+            float tot[3] = {0.f, 0.f, 0.f};
+            for (int w0 = 0; 32 * w0 < cols; w0 += 4) {          // four warps' columns in flight, each summed as that warp would
+                float4 x[4], y[4];
+#pragma unroll
+                for (int w = 0; w < 4; ++w) {
+                    const int i = 32 * (w0 + w) + lane;
+                    x[w] = y[w] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (i < cols) {
+                        if (vec) { x[w] = reinterpret_cast<const float4 *>(v)[i]; y[w] = reinterpret_cast<const float4 *>(ar)[i]; }
+                        else { x[w].x = v[i]; y[w].x = ar[i]; }
+                    }
+                }
+#pragma unroll
+                for (int w = 0; w < 4; ++w) {
+                    if (32 * (w0 + w) >= cols) continue;         // uniform
+                    float sum[3] = {0.f, 0.f, 0.f};
+                    take(sum, x[w].x, y[w].x); take(sum, x[w].y, y[w].y); take(sum, x[w].z, y[w].z); take(sum, x[w].w, y[w].w);
+#pragma unroll
+                    for (int e = 0; e < 3; ++e) tot[e] += warp_sum(sum[e]);
+                }
+            }
+            if (lane == 0) finish(a, tot[0], tot[1], tot[2]);
+        }
+        __syncthreads();
     }
+    if (tid == 0) s_last = atomicAdd(work, 1) == (int)gridDim.x - 1;
     __syncthreads();
     if (!s_last) return;
     __threadfence();
@@ -666,6 +706,12 @@ __global__ void __launch_bounds__(256) cosine_top1_kernel(const float *__restric
         out[2] = bad;
         work[0] = 0;
     }
+}
+
+inline void launch_cosine_top1(const float *v, const float *anchors, int n, int d, int n_sms, float *cosines, int *work, int *out, cudaStream_t s) {
+    const bool vec = ((reinterpret_cast<uintptr_t>(v) | reinterpret_cast<uintptr_t>(anchors)) & 15u) == 0 && d % 4 == 0;
+    if (n <= 8 * n_sms || (vec ? d / 4 : d) > 256) cosine_top1_kernel<false><<<n, 256, 0, s>>>(v, anchors, n, d, cosines, work, out);
+    else cosine_top1_kernel<true><<<(n + 7) / 8, 256, 0, s>>>(v, anchors, n, d, cosines, work, out);
 }
 
 // flag <- 1 if an anchor's norm is zero or not finite.

@@ -930,8 +930,7 @@ knnssd_status do_select(knnssd_ctx *c, const float *query_dev, int *domain, int 
     const int n = g.n_domains * g.anchors_per_domain;
     cudaStream_t s = c->stream;
     cudaEventRecord(c->ev0, s);
-    cosine_top1_kernel<<<n, 256, 0, s>>>(query_dev ? query_dev : c->pooled, c->anchors, n, g.d_model, c->cosines,
-                                                   c->knn_work, c->pinned);
+    launch_cosine_top1(query_dev ? query_dev : c->pooled, c->anchors, n, g.d_model, c->n_sms, c->cosines, c->knn_work, c->pinned, s);
     CUDA_TRY(c, cudaGetLastError());
     cudaEventRecord(c->ev1, s);
     knnssd_status st = sync_check(c, "select_skipset");
@@ -1942,7 +1941,7 @@ knnssd_status knnssd_cosine_top1(const float *query_dev, const float *anchors_de
     Scratch scratch(s);
     if (!host || !scratch.get(&cos_dev, (size_t)n) || !scratch.get(&work, 2)) return KNNSSD_ERR_CUDA;
     cudaMemsetAsync(work, 0, sizeof(int) * 2, s);
-    cosine_top1_kernel<<<n, 256, 0, s>>>(query_dev, anchors_dev, n, d, cos_dev, work, host);
+    launch_cosine_top1(query_dev, anchors_dev, n, d, sm_count(), cos_dev, work, host, s);
     cudaError_t e = cudaStreamSynchronize(s);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return KNNSSD_ERR_CUDA;
@@ -1993,7 +1992,7 @@ extern "C" knnssd_status knnssd_cosine_top1_static(const float *query_dev, const
     int *small = reinterpret_cast<int *>(scratch + KNNSSD_STATIC_MAX_ANCHORS);   // [0..2] result and flag, [4..5] the kernel's counters
     // the array still holds what the previous call left: the words that must start at zero are cleared here
     if (cudaMemsetAsync(small, 0, sizeof(int) * 6, s) != cudaSuccess) return KNNSSD_ERR_CUDA;
-    cosine_top1_kernel<<<n, 256, 0, s>>>(query_dev, anchors_dev, n, d, cos_dev, small + 4, small);
+    launch_cosine_top1(query_dev, anchors_dev, n, d, sm_count(), cos_dev, small + 4, small, s);
     int host[4] = {0, 0, 0, 0};
     cudaError_t e = cudaMemcpyAsync(host, small, sizeof(int) * 4, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
