@@ -56,6 +56,25 @@ __device__ __forceinline__ bf16_t float_to_bf16_rne(float f) {
     return (bf16_t)((u & 0x7FFFFFFFu) > 0x7F800000u ? 0x7FC0u : r);
 }
 
+// (v0, v1) -> packed bf16 pair (v0 in the low half), round to nearest even; hi part and what is left of it
+__device__ __forceinline__ uint32_t cvt_bf16x2(float v0, float v1) {
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(v1), "f"(v0));
+    return r;
+}
+__device__ __forceinline__ void split_pair(float v0, float v1, uint32_t &hi, uint32_t &lo) {
+    hi = cvt_bf16x2(v0, v1);
+    lo = cvt_bf16x2(v0 - __uint_as_float(hi << 16), v1 - __uint_as_float(hi & 0xffff0000u));
+}
+
+// Rotary embedding of a pair by (cos, sin) = c.  The rounding is spelled out: left to the compiler, the prompt pass's contraction and
+// rope_kv_rows_kernel fused other products of the second sum, and a row's K depended on which of them a launch's sizes chose.
+__device__ __forceinline__ void rotate_pair(float &a, float &b, float2 c) {
+    const float ra = __fmaf_rn(a, c.x, -__fmul_rn(b, c.y));
+    b = __fmaf_rn(b, c.x, __fmul_rn(a, c.y));
+    a = ra;
+}
+
 // 16-byte streaming load of weights: read-only path, do not keep in L1.
 __device__ __forceinline__ uint4 ld_stream16(const void *p) {
     uint4 v;
@@ -137,7 +156,7 @@ __global__ void embed_rope_kernel(const WT *__restrict__ E, const int *__restric
 // One warp owns a unit: lanes stride over the row in 16-byte pieces, fp32 FMAs, shuffle reduction.
 // The FMA order of a given (u, m) depends only on n_in, never on M or on the grid.
 // ---------------------------------------------------------------------------------------------
-enum { EPI_STORE = 0, EPI_ADD = 1, EPI_SWIGLU = 2 };
+enum { EPI_STORE = 0, EPI_ADD = 1, EPI_SWIGLU = 2, EPI_HEADS = 3 };      // EPI_HEADS: the pass kernel's q / k / v maps (LinPhase)
 
 struct LinearArgs {
     const void *W[3];

@@ -403,21 +403,19 @@ std::vector<pass::Op> build_ops(const knnssd_ctx *c, const unsigned char *mask, 
     for (int l = 0; l < g.n_layers; ++l) {
         const Layer &ly = c->layers[l];
         if (!mask || !mask[2 * l]) {
-            pass::Op q = lin(ly.wq, nq, d, c->x, ly.attn_norm, c->qkv, EPI_STORE);
+            pass::Op q = lin(ly.wq, nq, d, c->x, ly.attn_norm, nullptr, EPI_HEADS);
             q.lin.W[1] = reinterpret_cast<const bf16_t *>(ly.wk); q.lin.rows[1] = nkv;
             q.lin.W[2] = reinterpret_cast<const bf16_t *>(ly.wv); q.lin.rows[2] = nkv;
-            q.lin.units = nq + 2 * nkv; q.layer = l;
+            q.lin.units = (nq + 2 * nkv) / 2; q.layer = l;
             q.lin.xs = c->xs_x; q.lin.ss_in = c->ssp;
+            q.lin.half = hd / 2; q.lin.n_heads = g.n_heads; q.lin.n_kv_heads = g.n_kv_heads; q.lin.max_seq = g.max_seq;
+            q.lin.q = c->model.q;
+            q.lin.kc = reinterpret_cast<bf16_t *>(c->kcache) + (size_t)l * layer_stride;
+            q.lin.vc = reinterpret_cast<bf16_t *>(c->vcache) + (size_t)l * layer_stride;
             ops.push_back(q);
-            pass::Op ap{};                               // runs (and its barrier counts) only in passes of > BLKM rows
-            ap.type = pass::OP_KV_APPEND; ap.barrier_after = 1; ap.layer = l;
-            ap.kc = reinterpret_cast<bf16_t *>(c->kcache) + (size_t)l * layer_stride;
-            ap.vc = reinterpret_cast<bf16_t *>(c->vcache) + (size_t)l * layer_stride;
-            ops.push_back(ap);
             pass::Op a{};
             a.type = pass::OP_ATTN; a.barrier_after = 1; a.layer = l;
-            a.kc = reinterpret_cast<bf16_t *>(c->kcache) + (size_t)l * layer_stride;
-            a.vc = reinterpret_cast<bf16_t *>(c->vcache) + (size_t)l * layer_stride;
+            a.kc = q.lin.kc; a.vc = q.lin.vc;
             a.lin.ys = c->xs_attn;
             ops.push_back(a);
             pass::Op mg{};                               // runs (and its barrier counts) only in passes of >= MERGE_ROWS rows
@@ -508,7 +506,6 @@ void run_pass_mega(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const 
     if (head_row0 < M) bars += 1;
     pr.merge_op = pass::merge_rows_separately(M, c->cfg.n_heads / c->cfg.n_kv_heads) ? 1 : 0;
     if (pr.merge_op) bars += n_attn;
-    if (M > pass::BLKM) bars += n_attn;
     cudaError_t e;
     // 13..16 rows: where a CTA's share of the d_model-wide maps is more than two groups of 16 units, the packed form with
     // four groups per batch fetches the activations half as often (16 rows, 8 layers of the 13B / Qwen widths 1.93 -> 1.75 /
@@ -1131,7 +1128,7 @@ knnssd_status knnssd_init(const knnssd_config *cfg, const knnssd_weights *w, con
         md.tok_embed = reinterpret_cast<const bf16_t *>(c->tok_embed); md.final_norm = c->final_norm; md.rms_eps = g.rms_eps;
         md.d_model = d; md.H = g.n_heads; md.Hkv = g.n_kv_heads; md.hd = hd; md.vocab = g.vocab; md.max_seq = g.max_seq;
         md.n_seg_max = n_seg_max; md.inv_freq = c->inv_freq;
-        md.x = c->x; md.qkv = c->qkv; md.attn = c->attn; md.logits = c->logits; md.hfinal = c->hfinal; md.rope_cs = c->rope_cs;
+        md.x = c->x; md.q = reinterpret_cast<bf16_t *>(c->qkv); md.logits = c->logits; md.hfinal = c->hfinal; md.rope_cs = c->rope_cs;
         md.part_o = c->mpart_o; md.part_ml = c->mpart_ml; md.attn_cnt = c->attn_cnt; md.amax_v = c->mamax_v; md.amax_i = c->mamax_i;
         md.amax_cnt = c->amax_cnt; md.state = c->state; md.bar = c->bar; md.gabort = c->gabort; md.err = c->err_word;
         c->mega_ok = true;
@@ -1617,7 +1614,7 @@ knnssd_status knnssd_trace_pass(knnssd_ctx *c, int which, int k, int cap, int *o
     for (int i = 0; i < n && out < cap; ++i) {
         if (t[2 * i] == 0) continue;
         if (prev == 0) prev = t[2 * i];          // the first operation's start is not stamped: its work reads as 0
-        op_types[out] = ops[i].type == pass::OP_LINEAR ? (ops[i].is_head ? 14 : 10 + ops[i].lin.epi) : ops[i].type;
+        op_types[out] = ops[i].type == pass::OP_LINEAR ? (ops[i].is_head ? 14 : ops[i].lin.epi == EPI_HEADS ? 10 : 10 + ops[i].lin.epi) : ops[i].type;
         op_layers[out] = ops[i].layer;
         us_work[out] = (float)((double)(t[2 * i] - prev) * 1e-3);
         us_barrier[out] = (float)((double)(t[2 * i + 1] - t[2 * i]) * 1e-3);

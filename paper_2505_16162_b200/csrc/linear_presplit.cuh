@@ -20,7 +20,8 @@
 //
 // The epilogue writes what the NEXT map needs: the fp32 result where something reads it as fp32 (projection buffer,
 // residual stream, logits) and, for the residual update and the SwiGLU product, the pre-split form (times the next
-// RMSNorm's gain) plus this CTA's partial sums of squares.
+// RMSNorm's gain) plus this CTA's partial sums of squares.  Behind q / k / v it finishes the heads: rotary embedding, q as two bf16
+// rows, K and V into the cache - once per value, where every attention task that reads a head did it again.
 #pragma once
 #include "linear_stream.cuh"
 
@@ -104,21 +105,27 @@ __device__ __forceinline__ void consume_linear_pre(const LinPhase &p, const Ring
             }
         }
         // this thread's epilogue items: (unit, token) pairs, token fastest among the M live tokens.  For a residual
-        // update the old value and the next gain are fetched now, long before the epilogue needs them.
+        // update the old value and the next gain, for a rotary pair its cosine and sine are fetched now, long before the epilogue needs them.
         static_assert(NCW * GBN * NX * 32 * RW * 4 <= RED_BYTES, "the batch-end sums fit the reduction buffer");
-        const int gshift = s.swiglu ? 3 : 4, total = (ng << gshift) * p.M;
+        const int gshift = s.twin ? 3 : 4, total = (ng << gshift) * p.M;
         constexpr int ITEMS = GBN * 16 * 8 * NB / (NCW * 32);
         float xold[ITEMS], gnext[ITEMS];
 #pragma unroll
         for (int it4 = 0; it4 < ITEMS; ++it4) {
             xold[it4] = 0.f; gnext[it4] = 1.f;
             const int idx = tid + it4 * (NCW * 32);
-            if (p.epi == EPI_ADD && alive && idx < total) {
+            if ((p.epi == EPI_ADD || p.epi == EPI_HEADS) && alive && idx < total) {
                 const int n = idx % p.M, ur = idx / p.M, gi = ur >> gshift, rr = ur & ((1 << gshift) - 1);
                 if (rr < s.group_size(g0 + gi)) {
                     const int u = s.u_lo + s.group_lo(g0 + gi) + rr;
-                    xold[it4] = __ldcg(p.y + (size_t)n * p.units + u);
-                    if (p.next_gain) gnext[it4] = __ldg(p.next_gain + u);
+                    if (p.epi == EPI_HEADS) {
+                        const float2 cs = p.rope[n * p.half + u % p.half];
+                        xold[it4] = cs.x;
+                        gnext[it4] = cs.y;
+                    } else {
+                        xold[it4] = __ldcg(p.y + (size_t)n * p.units + u);
+                        if (p.next_gain) gnext[it4] = __ldg(p.next_gain + u);
+                    }
                 }
             }
         }
@@ -205,19 +212,37 @@ __device__ __forceinline__ void consume_linear_pre(const LinPhase &p, const Ring
                 // (unit / 8) * 2 + token % 2; paired: lane (unit % 8, token), register unit / 8
                 const int nb = PAIRED ? n >> 2 : n >> 3, n8 = PAIRED ? (n & 3) : (n & 7);
                 const int src_lane = (rr & 7) * 4 + (PAIRED ? n8 : (n8 >> 1)), reg = PAIRED ? 0 : (n8 & 1);
-                const int e0 = PAIRED ? (s.swiglu ? 0 : (rr >> 3)) : (s.swiglu ? reg : (rr >> 3) * 2 + reg);
-                const int e1 = PAIRED ? 1 : 2 + reg;            // SwiGLU: the up row of the unit (tile rows 8..15)
+                const int e0 = PAIRED ? (s.twin ? 0 : (rr >> 3)) : (s.twin ? reg : (rr >> 3) * 2 + reg);
+                const int e1 = PAIRED ? 1 : 2 + reg;            // the second row of a twin unit (tile rows 8..15)
                 float s0 = 0.f, s1 = 0.f;
 #pragma unroll
                 for (int w = 0; w < NCW; ++w) {
                     const float *q = red + ((((w * GBN + gi) * NX + nb) * 32) + src_lane) * RW;
                     s0 += q[e0];
-                    if (s.swiglu) s1 += q[e1];
+                    if (s.twin) s1 += q[e1];
                 }
                 const float ri = normed ? red_ss[n] : 1.0f;
                 const int u = s.u_lo + s.group_lo(g0 + gi) + rr;
                 float *yp = p.y + (size_t)n * p.units + u;
-                if (s.swiglu) {
+                if (p.epi == EPI_HEADS) {
+                    float a = __fmul_rn(s0, ri), b = __fmul_rn(s1, ri);
+                    int slot = u / p.half;
+                    const int i = u - slot * p.half;
+                    if (slot < p.n_heads + p.n_kv_heads) rotate_pair(a, b, make_float2(xold[it4], gnext[it4]));
+                    if (slot < p.n_heads) {
+                        bf16_t *dst = p.q + ((size_t)n * p.n_heads + slot) * (4 * p.half) + i;
+                        uint32_t hi, lo;
+                        split_pair(a, b, hi, lo);
+                        __stcg(dst, (bf16_t)hi); __stcg(dst + p.half, (bf16_t)(hi >> 16));
+                        __stcg(dst + 2 * p.half, (bf16_t)lo); __stcg(dst + 3 * p.half, (bf16_t)(lo >> 16));
+                    } else {
+                        slot -= p.n_heads;
+                        const bool is_k = slot < p.n_kv_heads;
+                        bf16_t *dst = (is_k ? p.kc : p.vc) + ((size_t)(slot - (is_k ? 0 : p.n_kv_heads)) * p.max_seq + *r.pos0 + n) * (2 * p.half) + i;
+                        dst[0] = float_to_bf16_rne(a);
+                        dst[p.half] = float_to_bf16_rne(b);
+                    }
+                } else if (p.epi == EPI_SWIGLU) {
                     const float gt = s0 * ri, up = s1 * ri;
                     const float a = gt / (1.0f + expf(-gt)) * up;
                     if (p.ys) store_split(p.ys, p.units >> 7, n, u, a); else __stcg(yp, a);

@@ -40,7 +40,7 @@ constexpr int KSTEPS = SLOT / 16;
 constexpr int GB = 4;                        // groups per batch
 constexpr int NTHREADS = (NCW + 4) * 32;      // two consumer warpgroups + the producer's warpgroup (one warp of it works)
 constexpr int REGS_PRODUCER = 40, REGS_CONSUMER = 232;
-constexpr int RED_BYTES = NCW * 8 * 32 * 4 * 4;  // reduction buffer (sized for 8 groups; attention keeps its K/V stash here)
+constexpr int RED_BYTES = NCW * 8 * 32 * 4 * 4;  // reduction buffer: the batch-end sums, sized for 8 groups
 constexpr int SS_BYTES = NCW * 8 * 4;
 constexpr int BAR_BYTES = 1024;
 constexpr int MAX_SMEM = 232448;             // 227 KB
@@ -55,7 +55,7 @@ static_assert(WS >= 4 && 2 * WS * 8 + 16 <= BAR_BYTES, "ring layout");
 struct LinPhase {
     const bf16_t *W[3];
     int rows[3];
-    int units;          // outputs (SWIGLU: d_ff, each unit = one gate row + one up row)
+    int units;          // outputs (SWIGLU: d_ff, each unit = one gate row + one up row; HEADS: rotary pairs, two rows each)
     int K;              // n_in, multiple of 128
     const float *x;     // [M][K]
     const float *gain;  // [K] or nullptr
@@ -71,6 +71,12 @@ struct LinPhase {
     uint32_t *ys;            // output in the same form for the next map (EPI_ADD: y * next_gain, SWIGLU: y); or nullptr
     const float *next_gain;  // [units] RMSNorm gain of the next map that reads y (EPI_ADD); nullptr = none
     float *ss_out;           // [M][n_cta] this CTA's partial sum of squares of each y row (EPI_ADD); or nullptr
+    // EPI_HEADS (q, k, v stacked; persistent pass kernel): a unit is a rotary pair, dimensions i and i + half of a head, so that the
+    // epilogue has both in one thread: it rotates q and k, leaves q as two bf16 rows and puts the rows of K and V into the cache
+    int half, n_heads, n_kv_heads, max_seq;
+    bf16_t *q;               // [M][n_heads][2 terms][2 half]
+    bf16_t *kc, *vc;         // this layer's cache [n_kv_heads][max_seq][2 half]
+    const float2 *rope;      // [M][half] (cos, sin) of the pass's rows: this CTA's copy
 };
 
 // Word index of term 0 of column `col` of row m in a pre-split buffer with nslots = K / 128 column slots; the terms
@@ -90,6 +96,7 @@ struct Ring {
     float *red, *red_ss;
     uint64_t *full_w, *empty_w;
     volatile int *abort_flag;
+    int *pos0;          // the position of the pass's first row (persistent pass kernel)
     int *err;           // device int: set non-zero if a bounded wait gave up
 };
 
@@ -176,15 +183,15 @@ __device__ __forceinline__ void store_split(uint32_t *buf, int nslots, int m, in
 // most one (the first g_rem groups hold g_base + 1 units).
 struct Share {
     int u_lo, n_units, n_groups, g_base, g_rem, n_batches, n_kt, gsz, gb;
-    bool swiglu;
+    bool twin;          // a unit has two weight rows, rows rr and rr + 8 of its tile: gate and up, or the dimensions of a rotary pair
     __device__ __forceinline__ int group_lo(int g) const { return g * g_base + min(g, g_rem); }
     __device__ __forceinline__ int group_size(int g) const { return g_base + (g < g_rem ? 1 : 0); }
 };
 
 __device__ __forceinline__ Share make_share(const LinPhase &p, int cta, int n_cta) {
     Share s;
-    s.swiglu = p.epi == EPI_SWIGLU;
-    s.gsz = s.swiglu ? 8 : 16;
+    s.twin = p.epi == EPI_SWIGLU || p.epi == EPI_HEADS;
+    s.gsz = s.twin ? 8 : 16;
     s.u_lo = (int)(((long long)p.units * cta) / n_cta);
     const int u_hi = (int)(((long long)p.units * (cta + 1)) / n_cta);
     s.n_units = u_hi - s.u_lo;
@@ -205,6 +212,7 @@ __device__ __forceinline__ void ring_setup(Ring &r, unsigned char *smem, int *er
     r.full_w = bars;
     r.empty_w = bars + WS;
     r.abort_flag = reinterpret_cast<volatile int *>(bars + 2 * WS);
+    r.pos0 = reinterpret_cast<int *>(bars + 2 * WS) + 1;
     r.err = err;
     if (threadIdx.x == 0) {
         for (int s = 0; s < WS; ++s) { mbar_init(&r.full_w[s], 1); mbar_init(&r.empty_w[s], NCW); }
@@ -232,18 +240,24 @@ __device__ __forceinline__ void produce_linear(const LinPhase &p, const Ring &r,
             nrows[gi] = 0;
             if (gi < ng) {
                 const int lo = s.group_lo(g0 + gi), nu = s.group_size(g0 + gi);
-                nrows[gi] = s.swiglu ? 2 * nu : nu;
-                const int rr = s.swiglu ? (lane & 7) : lane;
+                nrows[gi] = s.twin ? 2 * nu : nu;
+                const int rr = s.twin ? (lane & 7) : lane;
                 if (lane < WROWS && rr < nu) {
                     int u = s.u_lo + lo + rr;
-                    if (s.swiglu) {
-                        src[gi] = p.W[lane >> 3] + (size_t)u * p.K;
+                    // (selected, not indexed: an index would put the whole of p into local memory)
+                    const bf16_t *w = p.W[0];
+                    if (p.epi == EPI_SWIGLU) {
+                        if (lane >> 3) w = p.W[1];
                     } else {
-                        int which = 0;
-                        if (u >= p.rows[0]) { u -= p.rows[0]; which = 1; }
-                        if (which == 1 && u >= p.rows[1]) { u -= p.rows[1]; which = 2; }
-                        src[gi] = p.W[which] + (size_t)u * p.K;
+                        // HEADS: pair u % half of head u / half, its dimensions `half` rows apart
+                        if (s.twin) u += (u / p.half + (lane >> 3)) * p.half;
+                        if (u >= p.rows[0]) {
+                            u -= p.rows[0];
+                            w = p.W[1];
+                            if (u >= p.rows[1]) { u -= p.rows[1]; w = p.W[2]; }
+                        }
                     }
+                    src[gi] = w + (size_t)u * p.K;
                 }
             }
         }
@@ -378,7 +392,7 @@ __device__ __forceinline__ void consume_linear(const LinPhase &p, const Ring &r,
 #pragma unroll
                 for (int w = 0; w < NCW; ++w) {
                     const float *q = red + ((w * GB + gi) * 32 + src_lane) * 4;
-                    if (s.swiglu) { s0 += q[reg]; s1 += q[2 + reg]; }
+                    if (s.twin) { s0 += q[reg]; s1 += q[2 + reg]; }
                     else s0 += q[(rr >> 3) * 2 + reg];
                 }
                 float ri = 1.0f;
@@ -389,7 +403,7 @@ __device__ __forceinline__ void consume_linear(const LinPhase &p, const Ring &r,
                     ri = 1.0f / sqrtf(tot / (float)p.K + p.eps);
                 }
                 float *yp = p.y + (size_t)n * p.units + (s.u_lo + s.group_lo(g0 + gi) + rr);
-                if (s.swiglu) {
+                if (s.twin) {
                     const float gt = s0 * ri, up = s1 * ri;
                     __stcg(yp, gt / (1.0f + expf(-gt)) * up);
                 } else if (p.epi == EPI_ADD) {

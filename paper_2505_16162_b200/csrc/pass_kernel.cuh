@@ -24,11 +24,11 @@ using stream::Ring;
 using stream::NCW;
 
 constexpr int MAXM = 16;           // rows per pass this kernel handles
-constexpr int BLKM = 8;            // rows per tensor-core row block (linear maps take two blocks at once, attention one at a time)
+constexpr int BLKM = 8;            // rows per tensor-core row block (linear maps take two blocks at once, an attention task has one)
 constexpr int SEGP = 64;           // attention: positions per segment (fixed absolute boundaries)
 constexpr unsigned BAR_SPIN_LIMIT = 4000000u;
 
-enum { OP_EMBED = 0, OP_LINEAR = 1, OP_ATTN = 2, OP_HIDDEN = 3, OP_ARGMAX = 4, OP_ATTN_MERGE = 5, OP_KV_APPEND = 6 };
+enum { OP_EMBED = 0, OP_LINEAR = 1, OP_ATTN = 2, OP_HIDDEN = 3, OP_ARGMAX = 4, OP_ATTN_MERGE = 5 };
 constexpr int MERGE_ROWS = 3;      // tasks with at least this many (row, head) pairs leave the merge to a separate operation
 
 struct Op {
@@ -46,7 +46,8 @@ struct Model {           // what does not change from pass to pass
     float rms_eps;
     int d_model, H, Hkv, hd, vocab, max_seq, n_seg_max;
     const double *inv_freq;    // [hd/2]
-    float *x, *qkv, *attn, *logits, *hfinal;
+    float *x, *logits, *hfinal;
+    bf16_t *q;                 // [MAXM][H][2 terms][hd] rotated, hi and lo
     float2 *rope_cs;           // [grid][MAXM][hd/2]: one copy per CTA, written and read by that CTA only
     float *part_o;             // [MAXM][H][n_seg_max][hd]
     float2 *part_ml;           // [MAXM][H][n_seg_max]
@@ -77,10 +78,8 @@ struct Params {
 };
 
 // Whether a pass of M rows merges its attention partials in the separate operation: when an attention task carries
-// at least MERGE_ROWS (row, head) pairs - all G query heads of a K/V head for passes of up to BLKM rows.
-__host__ __device__ inline bool merge_rows_separately(int M, int G);
-
-__host__ __device__ inline bool merge_rows_separately(int M, int G) { return M > BLKM || M * G >= MERGE_ROWS; }
+// at least MERGE_ROWS (row, head) pairs.
+__host__ __device__ inline bool merge_rows_separately(int M, int G) { return M * G >= MERGE_ROWS; }
 
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
     unsigned long long t;
@@ -126,6 +125,7 @@ __device__ __forceinline__ void embed_phase(const Model &md, const Op &op, const
     const int d = md.d_model, half = md.hd >> 1;
     {   // every CTA fills its own copy of the (cos, sin) table of all rows: 148 readers of one copy would queue up at L2
         const int p0 = md.state->len + pr.pos_off;
+        if (tid == 0) *r.pos0 = p0;
         float2 *mine = md.rope_cs + (size_t)cta * MAXM * half;
         for (int idx = tid; idx < pr.M * half; idx += NCW * 32) {
             const int m = idx / half, i = idx % half;
@@ -233,50 +233,29 @@ __device__ __forceinline__ void argmax_phase(const Model &md, const Params &pr, 
 }
 
 // ---- attention over the KV cache ------------------------------------------------------------------------------
-// Rows m = 0..M-1 sit at positions P0 + m; row m attends to positions [0, P0 + m].  The context is cut at fixed
-// absolute boundaries into segments of SEGP positions; one warp handles one (query head, segment) for all rows: it
-// reads each K and V row of the segment once, keeps the segment's scores in registers, takes a plain softmax over
-// the segment and writes an un-normalised partial (max, sum, o).  The warp that completes the last segment of a
-// (row, head) merges the partials in segment order and writes the result pre-split for the output projection.
-// K/V of the M new positions come from the projection buffer (rotated, rounded to bf16 exactly as they are stored,
-// staged in shared memory); the warp of the first query head of each KV group also writes them to the cache.
-template <int HD> struct KVVec;
-template <> struct KVVec<128> { typedef uint2 T; };
-template <> struct KVVec<64> { typedef uint32_t T; };
+// Rows m = 0..M-1 sit at positions P0 + m; row m attends to positions [0, P0 + m], all of them in the cache: the q / k / v map before
+// has put the pass's own rows there.  The context is cut at fixed absolute boundaries into segments of SEGP positions; a warp
+// handles one (K/V head, segment) for eight (query head, row) pairs: it reads each K and V row of the segment once, keeps the
+// segment's scores in registers, takes a plain softmax over the segment and writes an un-normalised partial (max, sum, o).  The
+// partials are merged in segment order and written pre-split for the output projection, by the warp that completes the last
+// segment of a (row, head) where a task has one or two of them, else by an operation of its own.
 
-template <int HD> __device__ __forceinline__ void kv_unpack(const typename KVVec<HD>::T &v, float (&f)[HD / 32]);
-template <> __device__ __forceinline__ void kv_unpack<128>(const uint2 &v, float (&f)[4]) {
-    f[0] = __uint_as_float(v.x << 16); f[1] = __uint_as_float(v.x & 0xFFFF0000u);
-    f[2] = __uint_as_float(v.y << 16); f[3] = __uint_as_float(v.y & 0xFFFF0000u);
-}
-template <> __device__ __forceinline__ void kv_unpack<64>(const uint32_t &v, float (&f)[2]) {
-    f[0] = __uint_as_float(v << 16); f[1] = __uint_as_float(v & 0xFFFF0000u);
-}
-template <int HD> __device__ __forceinline__ typename KVVec<HD>::T kv_pack(const float (&f)[HD / 32]);
-template <> __device__ __forceinline__ uint2 kv_pack<128>(const float (&f)[4]) {
-    return make_uint2((uint32_t)float_to_bf16_rne(f[0]) | ((uint32_t)float_to_bf16_rne(f[1]) << 16),
-                      (uint32_t)float_to_bf16_rne(f[2]) | ((uint32_t)float_to_bf16_rne(f[3]) << 16));
-}
-template <> __device__ __forceinline__ uint32_t kv_pack<64>(const float (&f)[2]) {
-    return (uint32_t)float_to_bf16_rne(f[0]) | ((uint32_t)float_to_bf16_rne(f[1]) << 16);
-}
-template <int HD> __device__ __forceinline__ typename KVVec<HD>::T kv_zero();
-template <> __device__ __forceinline__ uint2 kv_zero<128>() { return make_uint2(0u, 0u); }
-template <> __device__ __forceinline__ uint32_t kv_zero<64>() { return 0u; }
-
-__device__ __forceinline__ void mma_tf32(float (&c)[4], uint32_t a0, uint32_t a2, uint32_t b0, uint32_t b1) {
-    // rows 8..15 of the 16-row operand are not used: their registers are zero
-    asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a0), "r"(0u), "r"(a2), "r"(0u), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ void mma_bf16_top(float (&c)[4], uint32_t a0, uint32_t a2, uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a0), "r"(0u), "r"(a2), "r"(0u), "r"(b0), "r"(b1));
+// N 32-bit words of a q, K or V row.  STREAM: K and V, which come by once per pass: first to go when L2 needs room.
+template <int N, bool STREAM> __device__ __forceinline__ void ld_words(const void *p, uint32_t *w) {
+    if constexpr (N == 8 && STREAM)
+        asm volatile("ld.global.L1::no_allocate.L2::evict_first.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7]) : "l"(p) : "memory");
+    else if constexpr (N == 8)
+        asm volatile("ld.global.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7]) : "l"(p) : "memory");
+    else {
+        static_assert(N == 4, "16 or 32 bytes");
+        const uint4 v = STREAM ? __ldcs(reinterpret_cast<const uint4 *>(p)) : __ldcg(reinterpret_cast<const uint4 *>(p));
+        w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
+    }
 }
 
-// The same with both halves of the 16-row operand: rows 0..7 from (a0, a2), rows 8..15 from (a1, a3).
+// c += a . b (m16n8k16, bf16 operands, fp32 accumulation): rows 0..7 of a from (a0, a2), rows 8..15 from (a1, a3).
 __device__ __forceinline__ void mma_bf16_rows(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
@@ -327,239 +306,113 @@ __device__ __forceinline__ void attn_merge_row(const Model &md, const Op &op, in
 }
 
 
-// Tensor-core form.  Lane (g8, t4) = (lane / 4, lane % 4).  The pass's rows are the rows 0..7 of the 16-row MMA
-// operand (row m = g8), so the cost does not depend on how many rows the pass carries.
+// Tensor-core form.  Lane (g8, t4) = (lane / 4, lane % 4).  The task's eight (query head, row) pairs are both halves of the 16-row MMA
+// operand: rows 0..7 their hi terms, rows 8..15 their lo terms, so that one product does both.
 //   scores  S = Q K^T   m16n8k16 bf16: the 8 columns of a tile are 8 consecutive positions (column n = g8 of the K
 //           operand = position 8*nt + g8).  A dot product does not care in which order its terms are taken, so k-step
-//           s pairs k-indices with the dimensions (DL*t4 + 4s .. + 3): every lane then reads one contiguous run of
-//           DL = HD/4 dimensions of "its" K row (16-byte loads) and holds the same run of q, split into two bf16
-//           terms (hi + lo, 16-17 bits); products are exact.
+//           s pairs k-indices with words 2s, 2s + 1 of the lane's share of a row: dimensions [RUN t4, RUN t4 + RUN) of either half
+//           of the head, RUN = HD / 8, 32 bytes of either (HD = 128) - whole sectors.
 //   output  O += P V    m16n8k16 bf16 over pairs of tiles: k-indices 2t4, 2t4+1 stand for positions 2t4, 2t4+1 of the
 //           first tile and 2t4+8, 2t4+9 for the same positions of the second - exactly the four scores the lane already
 //           holds - and column n = g8 of V-tile j is dimension (HD/8)*g8 + j, so a lane reads HD/8 contiguous
 //           dimensions of four V rows; an operand register (two positions of one dimension) is one byte-permute of two
 //           loaded words.  p is split into two bf16 terms.
-// A lane ends up with output dimensions [DL*t4, DL*t4 + DL) of row g8, the run it holds of q.
-template <int HD, bool R16>
-__device__ __forceinline__ void attn_phase(const Model &md, const Op &op, const Params &pr, const Ring &r, int cta, int n_cta,
-                                           int warp, int lane, bool defer_merge, int row0, bool all_cached) {
-    constexpr int DL = HD / 4;         // dimensions of q / o per lane
-    constexpr int NW = HD / 8;         // 32-bit words of a K row per lane
+// A lane ends up with output dimensions [DL*t4, DL*t4 + DL) of row g8, DL = HD / 4.
+// Bound by the chain of latencies of one task (a warp has at most a few): q and half of the segment's K and V are on their way at once.
+// With the heads rotated and split by every task, the pass's own K / V rows staged beside it and K read in 16-byte pieces 64 bytes apart
+// (two requests a sector), attention and what follows it up to the output projection took 16.7 us a layer of the 13B widths at 1 row and
+// 1280 positions, 18.5 at 5 rows, 23.7 of the 7B widths at 9 rows and 640; so 12.3, 12.7 and 10.8.
+template <int HD>
+__device__ __forceinline__ void attn_phase(const Model &md, const Op &op, const Params &pr, const Ring &r, int cta, int n_cta, int warp, int lane) {
+    constexpr int DL = HD / 4;         // output dimensions per lane
+    constexpr int RUN = HD / 8;        // dimensions of q and K per lane and half of the head
+    constexpr int NW = HD / 8;         // 32-bit words of a q or K row per lane
     constexpr int VW = HD / 16;        // 32-bit words of a V row per lane
     constexpr int VJ = HD / 8;         // V tiles (8 dimensions each)
     constexpr int HALF = HD / 2;
     constexpr int NT = SEGP / 8;       // position tiles per segment
-    constexpr int NR = R16 ? 2 : 1;    // pass rows per lane: row0 + g8 and, with R16, row0 + g8 + 8 (rows 8..15 of the MMA operand)
+    constexpr int KR = 4;              // tiles in flight
     const int g8 = lane >> 2, t4 = lane & 3;
     const int M = pr.M, H = md.H, Hkv = md.Hkv, G = H / Hkv;
-    const int P0 = md.state->len + pr.pos_off, Ttot = P0 + M;
-    const int Pc = all_cached ? Ttot : P0;                   // positions below Pc are read from the cache
-    // A task = (segment, head group, block of 8 rows).  Passes of up to BLKM rows (all_cached false) take the G query
-    // heads that share a K/V head together: the rows of a group are the (head-in-group, pass row) pairs rr = hg M + m,
-    // eight per block, so that a K/V segment is read once per block instead of once per head and a GQA model has
-    // G times fewer tasks.  With all_cached a task is one head and the block is given by row0.
-    const int Gt = all_cached ? 1 : G;                       // query heads per group
-    const int n_grp = H / Gt;
-    const int R = all_cached ? M : M * Gt;                   // rows of a group
-    const int nblk = all_cached ? 1 : (R + BLKM - 1) / BLKM;
-    const int n_seg = (Ttot + SEGP - 1) / SEGP, n_tasks = n_grp * n_seg * nblk;
-    const int qstride = (H + 2 * Hkv) * HD;
+    const int P0 = *r.pos0, Ttot = P0 + M;
+    // A task = (segment, K/V head, block of 8 of the R = G M (query head of the group, row) pairs rr = hg M + m).
+    const int R = M * G, nblk = (R + BLKM - 1) / BLKM;
+    const int n_seg = (Ttot + SEGP - 1) / SEGP, n_tasks = Hkv * n_seg * nblk;
     const float scale = 1.0f / sqrtf((float)HD);
-    const bool upper = t4 >= 2;                              // this lane's run lies in the second half of the head
-    const int ci = DL * (t4 & 1);                            // its offset in the (cos, sin) table
-    bf16_t *stash_k = reinterpret_cast<bf16_t *>(r.red) + (size_t)warp * (2 * BLKM * HD);   // [BLKM][HD] new K rows
-    bf16_t *stash_v = stash_k + BLKM * HD;                                                  // [BLKM][HD] new V rows
-    const float2 *my_cs = md.rope_cs + (size_t)cta * MAXM * HALF;                           // this CTA's copy
 
     for (int t = warp * n_cta + cta; t < n_tasks; t += NCW * n_cta) {
-        const int blk = t % nblk, tt = t / nblk, seg = tt / n_grp, grp = tt % n_grp;
-        const int kvh = all_cached ? grp / G : grp;
-        const int rr = blk * BLKM + g8;                      // this lane's row of the group (grouped tasks)
-        const int rm = all_cached ? row0 + g8 : rr % M;      // the pass row this lane's MMA row stands for
-        const int h = all_cached ? grp : kvh * G + min(rr / M, G - 1);   // and its query head
-        const bool row_in = all_cached ? rm < M : rr < R;
-        const int rm2 = rm + BLKM;                           // R16: the lane's second row (MMA row g8 + 8), same head
+        const int blk = t % nblk, tt = t / nblk, seg = tt / Hkv, kvh = tt % Hkv;
+        const int rr = min(blk * BLKM + g8, R - 1);          // this lane's pair
+        const int rm = rr % M, h = kvh * G + rr / M;
         const int p_begin = seg * SEGP, p_end = min(p_begin + SEGP, Ttot);
-        const int m_first = max(0, p_begin - P0);           // first row that sees this segment
-        const bool writer = !all_cached && blk == 0;         // one task per (segment, K/V head) puts the new rows into the cache
-        bf16_t *kbase = op.kc + (size_t)kvh * md.max_seq * HD;
-        bf16_t *vbase = op.vc + (size_t)kvh * md.max_seq * HD;
-        if (all_cached && row0 + NR * BLKM <= m_first) continue;  // none of this block's rows sees the segment
-        // pass row g8's own position lies in this segment and is not in the cache yet: this lane rotates / rounds its K, V
-        const bool row_new = !all_cached && g8 < M && P0 + g8 >= p_begin && P0 + g8 < p_end;
-        const bool row_live = row_in && rm >= m_first;
-        const bool row_live2 = R16 && rm2 < M && rm2 >= m_first;
-        // ---- this lane's run of q (row g8), of the new K row and of the new V row: load, rotate, round / split ----
-        float qf[DL], kf[DL];
-        float qf2[R16 ? DL : 1];                             // R16: the second row's run of q, rotated like the first
-        {
-            const float *qraw = md.qkv + (size_t)min(rm, M - 1) * qstride + (size_t)h * HD + DL * t4;
-            const float *kraw = md.qkv + (size_t)min(g8, M - 1) * qstride + (size_t)(H + kvh) * HD + DL * t4;
+        const bool row_live = blk * BLKM + g8 < R && P0 + rm >= p_begin;         // it exists, and sees the segment
+        if (!__any_sync(0xffffffffu, row_live)) continue;
+        const bf16_t *kbase = op.kc + ((size_t)kvh * md.max_seq + p_begin + g8) * HD + RUN * t4;
+        const bf16_t *vbase = op.vc + ((size_t)kvh * md.max_seq + p_begin + 2 * t4) * HD + 2 * VW * g8;
+        auto load_k = [&](int nt, uint32_t (&dst)[NW]) {
+            if (p_begin + 8 * nt + g8 < p_end) {
+                ld_words<NW / 2, true>(kbase + 8 * nt * HD, dst);
+                ld_words<NW / 2, true>(kbase + 8 * nt * HD + HALF, dst + NW / 2);
+            } else {
 #pragma unroll
-            for (int e = 0; e < DL; e += 4) {
-                const float4 a = row_live ? __ldcg(reinterpret_cast<const float4 *>(qraw + e)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                const float4 b = row_new ? __ldcg(reinterpret_cast<const float4 *>(kraw + e)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                qf[e] = a.x; qf[e + 1] = a.y; qf[e + 2] = a.z; qf[e + 3] = a.w;
-                kf[e] = b.x; kf[e + 1] = b.y; kf[e + 2] = b.z; kf[e + 3] = b.w;
+                for (int w = 0; w < NW; ++w) dst[w] = 0u;
             }
-            if constexpr (R16) {
-                const float *qraw2 = md.qkv + (size_t)min(rm2, M - 1) * qstride + (size_t)h * HD + DL * t4;
-#pragma unroll
-                for (int e = 0; e < DL; e += 4) {
-                    const float4 a = row_live2 ? __ldcg(reinterpret_cast<const float4 *>(qraw2 + e)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                    qf2[e] = a.x; qf2[e + 1] = a.y; qf2[e + 2] = a.z; qf2[e + 3] = a.w;
-                }
-            }
-#pragma unroll
-            for (int e = 0; e < DL; ++e) {
-                const float qp = __shfl_xor_sync(0xffffffffu, qf[e], 2), kp = __shfl_xor_sync(0xffffffffu, kf[e], 2);
-                const float2 cq = row_live ? my_cs[rm * HALF + ci + e] : make_float2(1.f, 0.f);
-                const float2 ck = row_new ? my_cs[g8 * HALF + ci + e] : make_float2(1.f, 0.f);
-                qf[e] = upper ? (qf[e] * cq.x + qp * cq.y) : (qf[e] * cq.x - qp * cq.y);
-                kf[e] = upper ? (kf[e] * ck.x + kp * ck.y) : (kf[e] * ck.x - kp * ck.y);
-            }
-            if constexpr (R16) {
-#pragma unroll
-                for (int e = 0; e < DL; ++e) {
-                    const float qp = __shfl_xor_sync(0xffffffffu, qf2[e], 2);
-                    const float2 cq = row_live2 ? my_cs[rm2 * HALF + ci + e] : make_float2(1.f, 0.f);
-                    qf2[e] = upper ? (qf2[e] * cq.x + qp * cq.y) : (qf2[e] * cq.x - qp * cq.y);
-                }
-            }
-        }
-        __syncwarp();
-        if (row_new) {
-            const float *vraw = md.qkv + (size_t)g8 * qstride + (size_t)(H + Hkv + kvh) * HD + DL * t4;
-#pragma unroll
-            for (int e = 0; e < DL; e += 8) {
-                const float4 a = __ldcg(reinterpret_cast<const float4 *>(vraw + e)), b = __ldcg(reinterpret_cast<const float4 *>(vraw + e + 4));
-                uint4 kp, vp;
-                kp.x = (uint32_t)float_to_bf16_rne(kf[e]) | ((uint32_t)float_to_bf16_rne(kf[e + 1]) << 16);
-                kp.y = (uint32_t)float_to_bf16_rne(kf[e + 2]) | ((uint32_t)float_to_bf16_rne(kf[e + 3]) << 16);
-                kp.z = (uint32_t)float_to_bf16_rne(kf[e + 4]) | ((uint32_t)float_to_bf16_rne(kf[e + 5]) << 16);
-                kp.w = (uint32_t)float_to_bf16_rne(kf[e + 6]) | ((uint32_t)float_to_bf16_rne(kf[e + 7]) << 16);
-                vp.x = (uint32_t)float_to_bf16_rne(a.x) | ((uint32_t)float_to_bf16_rne(a.y) << 16);
-                vp.y = (uint32_t)float_to_bf16_rne(a.z) | ((uint32_t)float_to_bf16_rne(a.w) << 16);
-                vp.z = (uint32_t)float_to_bf16_rne(b.x) | ((uint32_t)float_to_bf16_rne(b.y) << 16);
-                vp.w = (uint32_t)float_to_bf16_rne(b.z) | ((uint32_t)float_to_bf16_rne(b.w) << 16);
-                *reinterpret_cast<uint4 *>(stash_k + g8 * HD + DL * t4 + e) = kp;
-                *reinterpret_cast<uint4 *>(stash_v + g8 * HD + DL * t4 + e) = vp;
-                if (writer) {
-                    *reinterpret_cast<uint4 *>(kbase + (size_t)(P0 + g8) * HD + DL * t4 + e) = kp;
-                    *reinterpret_cast<uint4 *>(vbase + (size_t)(P0 + g8) * HD + DL * t4 + e) = vp;
-                }
-            }
-        }
-        __syncwarp();
-        uint32_t qh[NW], ql[NW];                             // word w = dimensions (2w, 2w + 1) of the run; q = hi + lo
-#pragma unroll
-        for (int w = 0; w < NW; ++w) {
-            const uint32_t h0 = float_to_bf16_rne(qf[2 * w]), h1 = float_to_bf16_rne(qf[2 * w + 1]);
-            const uint32_t l0 = float_to_bf16_rne(qf[2 * w] - __uint_as_float(h0 << 16));
-            const uint32_t l1 = float_to_bf16_rne(qf[2 * w + 1] - __uint_as_float(h1 << 16));
-            qh[w] = h0 | (h1 << 16); ql[w] = l0 | (l1 << 16);
-        }
-        uint32_t qh2[R16 ? NW : 1], ql2[R16 ? NW : 1];       // R16: the second row's words
-        if constexpr (R16) {
-#pragma unroll
-            for (int w = 0; w < NW; ++w) {
-                const uint32_t h0 = float_to_bf16_rne(qf2[2 * w]), h1 = float_to_bf16_rne(qf2[2 * w + 1]);
-                const uint32_t l0 = float_to_bf16_rne(qf2[2 * w] - __uint_as_float(h0 << 16));
-                const uint32_t l1 = float_to_bf16_rne(qf2[2 * w + 1] - __uint_as_float(h1 << 16));
-                qh2[w] = h0 | (h1 << 16); ql2[w] = l0 | (l1 << 16);
-            }
-        }
-        // ---- scores: one tile = 8 positions; K rows are fetched two tiles ahead ----
-        auto load_k = [&](int nt, uint4 (&dst)[NW / 4]) {
-            const int p = p_begin + 8 * nt + g8;
-            const bf16_t *src = p < Pc ? kbase + (size_t)p * HD + DL * t4 : stash_k + (p - P0) * HD + DL * t4;
-#pragma unroll
-            for (int q = 0; q < NW / 4; ++q)
-                dst[q] = p < p_end ? (p < Pc ? __ldcs(reinterpret_cast<const uint4 *>(src + 8 * q)) : *reinterpret_cast<const uint4 *>(src + 8 * q)) : make_uint4(0u, 0u, 0u, 0u);
         };
-        float sc[NT][2 * NR];                                // scores of (row g8, positions 8*nt + 2*t4 + {0, 1}); R16: [2], [3] = row g8 + 8
-        {
-            constexpr int KR = NT < 4 ? NT : 4;              // tiles in flight
-            uint4 kb[KR][NW / 4];
+        auto load_v = [&](int nt, uint32_t (&dst)[2][VW]) {
 #pragma unroll
-            for (int i = 0; i < KR; ++i) load_k(i, kb[i]);
-#pragma unroll
-            for (int nt = 0; nt < NT; ++nt) {
-                uint4(&kq)[NW / 4] = kb[nt % KR];
-                float ch[4] = {}, cl[4] = {};
-#pragma unroll
-                for (int q = 0; q < NW / 4; ++q) {
-                    // words 4q .. 4q+3 of the run: k-steps 2q (x, y) and 2q + 1 (z, w)
-                    if constexpr (R16) {
-                        mma_bf16_rows(cl, ql[4 * q], ql2[4 * q], ql[4 * q + 1], ql2[4 * q + 1], kq[q].x, kq[q].y);
-                        mma_bf16_rows(ch, qh[4 * q], qh2[4 * q], qh[4 * q + 1], qh2[4 * q + 1], kq[q].x, kq[q].y);
-                        mma_bf16_rows(cl, ql[4 * q + 2], ql2[4 * q + 2], ql[4 * q + 3], ql2[4 * q + 3], kq[q].z, kq[q].w);
-                        mma_bf16_rows(ch, qh[4 * q + 2], qh2[4 * q + 2], qh[4 * q + 3], qh2[4 * q + 3], kq[q].z, kq[q].w);
-                    } else {
-                        mma_bf16_top(cl, ql[4 * q], ql[4 * q + 1], kq[q].x, kq[q].y);
-                        mma_bf16_top(ch, qh[4 * q], qh[4 * q + 1], kq[q].x, kq[q].y);
-                        mma_bf16_top(cl, ql[4 * q + 2], ql[4 * q + 3], kq[q].z, kq[q].w);
-                        mma_bf16_top(ch, qh[4 * q + 2], qh[4 * q + 3], kq[q].z, kq[q].w);
-                    }
-                }
-                sc[nt][0] = cl[0] + ch[0];
-                sc[nt][1] = cl[1] + ch[1];
-                if constexpr (R16) { sc[nt][2] = cl[2] + ch[2]; sc[nt][3] = cl[3] + ch[3]; }
-                if (nt + KR < NT) load_k(nt + KR, kq);
-            }
-        }
-        // ---- V rows of the first tiles start moving while the softmax runs ----
-        auto load_v = [&](int nt, uint4 (&dst)[2][(VW + 3) / 4]) {
-#pragma unroll
-            for (int rr = 0; rr < 2; ++rr) {
-                const int p = p_begin + 8 * nt + 2 * t4 + rr;
-                const bf16_t *src = p < Pc ? vbase + (size_t)p * HD + 2 * VW * g8 : stash_v + (p - P0) * HD + 2 * VW * g8;
-                if (VW >= 4) {
-#pragma unroll
-                    for (int q = 0; q < VW / 4; ++q)
-                        dst[rr][q] = p < p_end ? (p < Pc ? __ldcs(reinterpret_cast<const uint4 *>(src + 8 * q)) : *reinterpret_cast<const uint4 *>(src + 8 * q)) : make_uint4(0u, 0u, 0u, 0u);
+            for (int e = 0; e < 2; ++e)
+                if (p_begin + 8 * nt + 2 * t4 + e < p_end) {
+                    ld_words<VW, true>(vbase + (8 * nt + e) * HD, dst[e]);
                 } else {
-                    const uint2 v = p < p_end ? *reinterpret_cast<const uint2 *>(src) : make_uint2(0u, 0u);
-                    dst[rr][0] = make_uint4(v.x, v.y, 0u, 0u);
+#pragma unroll
+                    for (int w = 0; w < VW; ++w) dst[e][w] = 0u;
                 }
-            }
         };
-        constexpr int VR = NT < 4 ? NT : 4;                  // tiles in flight
-        uint4 vb[VR][2][(VW + 3) / 4];
-#pragma unroll
-        for (int i = 0; i < VR; ++i) load_v(i, vb[i]);
-        // ---- softmax over the segment for row g8 (the four lanes of a row share it); R16: and for row g8 + 8 ----
-        float mx_r[NR], lsum_r[NR];
-#pragma unroll
-        for (int r = 0; r < NR; ++r) {
-            const bool live_r = r == 0 ? row_live : row_live2;
-            const int rm_r = r == 0 ? rm : rm2;
-            float mx = -INFINITY;
-#pragma unroll
-            for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int p = p_begin + 8 * nt + 2 * t4 + e;
-                    const bool valid = live_r && p <= P0 + rm_r;             // causal; also excludes p >= p_end
-                    sc[nt][2 * r + e] = valid ? sc[nt][2 * r + e] * scale : -INFINITY;
-                    mx = fmaxf(mx, sc[nt][2 * r + e]);
-                }
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-            float lsum = 0.f;
-#pragma unroll
-            for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const float pj = sc[nt][2 * r + e] == -INFINITY ? 0.f : expf(sc[nt][2 * r + e] - mx);
-                    sc[nt][2 * r + e] = pj;
-                    lsum += pj;
-                }
-            lsum += __shfl_xor_sync(0xffffffffu, lsum, 1);
-            lsum += __shfl_xor_sync(0xffffffffu, lsum, 2);
-            mx_r[r] = mx; lsum_r[r] = lsum;
+        uint32_t qh[NW], ql[NW], kb[KR][NW], vb[KR][2][VW];
+        {
+            const bf16_t *q = md.q + ((size_t)rm * H + h) * (2 * HD) + RUN * t4;
+            ld_words<NW / 2, false>(q, qh);
+            ld_words<NW / 2, false>(q + HALF, qh + NW / 2);
+            ld_words<NW / 2, false>(q + HD, ql);
+            ld_words<NW / 2, false>(q + HD + HALF, ql + NW / 2);
         }
-        const float mx = mx_r[0], lsum = lsum_r[0];
+#pragma unroll
+        for (int i = 0; i < KR; ++i) load_k(i, kb[i]);
+#pragma unroll
+        for (int i = 0; i < KR; ++i) load_v(i, vb[i]);
+        // ---- scores of pair g8, positions 8 nt + 2 t4 + {0, 1} ----
+        float sc[NT][2];
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+            uint32_t(&k)[NW] = kb[nt % KR];
+            float c[4] = {};
+#pragma unroll
+            for (int w = 0; w < NW; w += 2) mma_bf16_rows(c, qh[w], ql[w], qh[w + 1], ql[w + 1], k[w], k[w + 1]);
+            sc[nt][0] = c[2] + c[0];
+            sc[nt][1] = c[3] + c[1];
+            if (nt + KR < NT) load_k(nt + KR, k);
+        }
+        // ---- softmax over the segment (the four lanes of a pair share it) ----
+        float mx = -INFINITY, lsum = 0.f;
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const bool valid = row_live && p_begin + 8 * nt + 2 * t4 + e <= P0 + rm;     // causal; also excludes positions past p_end
+                sc[nt][e] = valid ? sc[nt][e] * scale : -INFINITY;
+                mx = fmaxf(mx, sc[nt][e]);
+            }
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                sc[nt][e] = sc[nt][e] == -INFINITY ? 0.f : expf(sc[nt][e] - mx);
+                lsum += sc[nt][e];
+            }
+        lsum += __shfl_xor_sync(0xffffffffu, lsum, 1);
+        lsum += __shfl_xor_sync(0xffffffffu, lsum, 2);
         // ---- o += p V ----
         float o[VJ][4];
 #pragma unroll
@@ -568,66 +421,30 @@ __device__ __forceinline__ void attn_phase(const Model &md, const Op &op, const 
         for (int np = 0; np < NT; np += 2) {
             // k-indices 2t4, 2t4+1 stand for this lane's two positions of tile np, 2t4+8, 2t4+9 for those of tile np + 1
             uint32_t ah[2], al[2];
-            uint32_t ah2[2] = {0u, 0u}, al2[2] = {0u, 0u};  // R16: the same for row g8 + 8
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const uint32_t h0 = float_to_bf16_rne(sc[np + i][0]), h1 = float_to_bf16_rne(sc[np + i][1]);
-                const uint32_t l0 = float_to_bf16_rne(sc[np + i][0] - __uint_as_float(h0 << 16));
-                const uint32_t l1 = float_to_bf16_rne(sc[np + i][1] - __uint_as_float(h1 << 16));
-                ah[i] = h0 | (h1 << 16); al[i] = l0 | (l1 << 16);
-                if constexpr (R16) {
-                    const uint32_t g0 = float_to_bf16_rne(sc[np + i][2]), g1 = float_to_bf16_rne(sc[np + i][3]);
-                    const uint32_t m0 = float_to_bf16_rne(sc[np + i][2] - __uint_as_float(g0 << 16));
-                    const uint32_t m1 = float_to_bf16_rne(sc[np + i][3] - __uint_as_float(g1 << 16));
-                    ah2[i] = g0 | (g1 << 16); al2[i] = m0 | (m1 << 16);
-                }
-            }
+            for (int i = 0; i < 2; ++i) split_pair(sc[np + i][0], sc[np + i][1], ah[i], al[i]);
 #pragma unroll
             for (int j = 0; j < VJ; ++j) {
-                const int wi = (j >> 1) & 3;
                 uint32_t b[2];
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    const uint4 &wa = vb[(np + i) % VR][0][j / 8], &wb = vb[(np + i) % VR][1][j / 8];
-                    const uint32_t xa = wi == 0 ? wa.x : wi == 1 ? wa.y : wi == 2 ? wa.z : wa.w;
-                    const uint32_t xb = wi == 0 ? wb.x : wi == 1 ? wb.y : wi == 2 ? wb.z : wb.w;
-                    b[i] = __byte_perm(xa, xb, (j & 1) ? 0x7632 : 0x5410);     // dimension j of the two positions' rows
-                }
-                if constexpr (R16) {
-                    mma_bf16_rows(o[j], al[0], al2[0], al[1], al2[1], b[0], b[1]);
-                    mma_bf16_rows(o[j], ah[0], ah2[0], ah[1], ah2[1], b[0], b[1]);
-                } else {
-                    mma_bf16_top(o[j], al[0], al[1], b[0], b[1]);
-                    mma_bf16_top(o[j], ah[0], ah[1], b[0], b[1]);
-                }
+                for (int i = 0; i < 2; ++i)                  // dimension j of the two positions' rows
+                    b[i] = __byte_perm(vb[(np + i) % KR][0][j / 2], vb[(np + i) % KR][1][j / 2], (j & 1) ? 0x7632 : 0x5410);
+                mma_bf16_rows(o[j], ah[0], al[0], ah[1], al[1], b[0], b[1]);
             }
-            if (np + VR < NT) load_v(np + VR, vb[np % VR]);
-            if (np + 1 + VR < NT) load_v(np + 1 + VR, vb[(np + 1) % VR]);
+            if (np + KR < NT) { load_v(np + KR, vb[np % KR]); load_v(np + 1 + KR, vb[(np + 1) % KR]); }
         }
-        // ---- partials out (row g8: dimensions DL*t4 + j and DL*t4 + VJ + j); the last warp of a (row, head) merges ----
+        // ---- partials out (pair g8: dimensions DL*t4 + j and DL*t4 + VJ + j); the last warp of a (row, head) merges ----
         if (row_live) {
             const size_t pidx = ((size_t)rm * H + h) * md.n_seg_max + seg;
             if (t4 == 0) __stcg(md.part_ml + pidx, make_float2(mx, lsum));
             float *po = md.part_o + pidx * HD + DL * t4;
 #pragma unroll
             for (int j = 0; j < VJ; j += 4) {
-                __stcg(reinterpret_cast<float4 *>(po + j), make_float4(o[j][0], o[j + 1][0], o[j + 2][0], o[j + 3][0]));
-                __stcg(reinterpret_cast<float4 *>(po + VJ + j), make_float4(o[j][1], o[j + 1][1], o[j + 2][1], o[j + 3][1]));
+                __stcg(reinterpret_cast<float4 *>(po + j), make_float4(o[j][2] + o[j][0], o[j + 1][2] + o[j + 1][0], o[j + 2][2] + o[j + 2][0], o[j + 3][2] + o[j + 3][0]));
+                __stcg(reinterpret_cast<float4 *>(po + VJ + j), make_float4(o[j][3] + o[j][1], o[j + 1][3] + o[j + 1][1], o[j + 2][3] + o[j + 2][1], o[j + 3][3] + o[j + 3][1]));
             }
         }
-        if constexpr (R16) {
-            if (row_live2) {                                  // row g8 + 8: accumulator registers 2, 3
-                const size_t pidx = ((size_t)rm2 * H + h) * md.n_seg_max + seg;
-                if (t4 == 0) __stcg(md.part_ml + pidx, make_float2(mx_r[NR - 1], lsum_r[NR - 1]));
-                float *po = md.part_o + pidx * HD + DL * t4;
-#pragma unroll
-                for (int j = 0; j < VJ; j += 4) {
-                    __stcg(reinterpret_cast<float4 *>(po + j), make_float4(o[j][2], o[j + 1][2], o[j + 2][2], o[j + 3][2]));
-                    __stcg(reinterpret_cast<float4 *>(po + VJ + j), make_float4(o[j][3], o[j + 1][3], o[j + 2][3], o[j + 3][3]));
-                }
-            }
-        }
-        if (defer_merge) continue;                            // a separate merge operation follows a grid barrier
+        if (pr.merge_op) continue;                            // a separate merge operation follows a grid barrier
         __threadfence();
         __syncwarp();
         bool last = false;
@@ -640,8 +457,7 @@ __device__ __forceinline__ void attn_phase(const Model &md, const Op &op, const 
             __threadfence();
             for (int g = 0; g < BLKM; ++g) {
                 if (!((last_mask >> (4 * g)) & 1u)) continue;
-                const int rg = blk * BLKM + g;
-                const int mg = all_cached ? row0 + g : rg % M, hg = all_cached ? grp : kvh * G + rg / M;
+                const int rg = blk * BLKM + g, mg = rg % M, hg = kvh * G + rg / M;
                 attn_merge_row<HD>(md, op, P0, mg, hg, lane);
                 if (lane == 0) md.attn_cnt[mg * H + hg] = 0;
             }
@@ -649,42 +465,12 @@ __device__ __forceinline__ void attn_phase(const Model &md, const Op &op, const 
     }
 }
 
-// Passes of more than BLKM rows first put the K/V rows of all their new positions into the cache (rotated, rounded),
-// one (row, KV head) per warp, so that the attention operation - which then takes the rows one block at a time - reads
-// every position from the cache.  Lane l holds dimensions [DPL*l, DPL*l + DPL); its rotation partner is lane l ^ 16.
-template <int HD>
-__device__ __forceinline__ void kv_append_phase(const Model &md, const Op &op, const Params &pr, int cta, int n_cta, int warp,
-                                                int lane) {
-    constexpr int DPL = HD / 32, HALF = HD / 2;
-    typedef typename KVVec<HD>::T VT;
-    const int H = md.H, Hkv = md.Hkv, P0 = md.state->len + pr.pos_off, jobs = pr.M * Hkv;
-    const int qstride = (H + 2 * Hkv) * HD, d0 = DPL * lane, ci = d0 % HALF;
-    const bool upper = d0 >= HALF;
-    const float2 *my_cs = md.rope_cs + (size_t)cta * MAXM * HALF;
-    for (int j = warp * n_cta + cta; j < jobs; j += NCW * n_cta) {
-        const int m = j / Hkv, kvh = j % Hkv;
-        const float *kraw = md.qkv + (size_t)m * qstride + (size_t)(H + kvh) * HD + d0;
-        const float *vraw = md.qkv + (size_t)m * qstride + (size_t)(H + Hkv + kvh) * HD + d0;
-        float kf[DPL], vf[DPL];
-#pragma unroll
-        for (int e = 0; e < DPL; ++e) { kf[e] = __ldcg(kraw + e); vf[e] = __ldcg(vraw + e); }
-#pragma unroll
-        for (int e = 0; e < DPL; ++e) {
-            const float partner = __shfl_xor_sync(0xffffffffu, kf[e], 16);
-            const float2 cs = my_cs[m * HALF + ci + e];
-            kf[e] = upper ? (kf[e] * cs.x + partner * cs.y) : (kf[e] * cs.x - partner * cs.y);
-        }
-        *reinterpret_cast<VT *>(op.kc + ((size_t)kvh * md.max_seq + P0 + m) * HD + d0) = kv_pack<HD>(kf);
-        *reinterpret_cast<VT *>(op.vc + ((size_t)kvh * md.max_seq + P0 + m) * HD + d0) = kv_pack<HD>(vf);
-    }
-}
-
 // With several rows the warp that finishes a head last would merge all its rows one after the other; the merges
 // then run as an operation of their own instead, one (row, head) per warp across the whole grid.
 template <int HD>
-__device__ __forceinline__ void attn_merge_phase(const Model &md, const Op &op, const Params &pr, int cta, int n_cta, int warp,
+__device__ __forceinline__ void attn_merge_phase(const Model &md, const Op &op, const Params &pr, const Ring &r, int cta, int n_cta, int warp,
                                                  int lane) {
-    const int P0 = md.state->len + pr.pos_off, jobs = pr.M * md.H;
+    const int P0 = *r.pos0, jobs = pr.M * md.H;
     for (int j = warp * n_cta + cta; j < jobs; j += NCW * n_cta) attn_merge_row<HD>(md, op, P0, j / md.H, j % md.H, lane);
 }
 
@@ -735,18 +521,12 @@ __global__ void __launch_bounds__(stream::NTHREADS, 1) pass_kernel(const Model m
                 lp.ss_in += (size_t)pr.head_row0 * n_cta;
                 lp.y += (size_t)(pr.out_row0 + pr.head_row0) * lp.units;
             }
+            lp.rope = md.rope_cs + (size_t)cta * MAXM * (HD / 2);
             if (ran) stream::consume_linear_pre<NB, NP>(lp, r, cta, n_cta, warp, lane, w_use, alive);
         } else if (alive) {
             if (op.type == OP_EMBED) embed_phase(md, op, pr, r, cta, n_cta, tid);
-            else if (op.type == OP_KV_APPEND) { if (NB > 1) kv_append_phase<HD>(md, op, pr, cta, n_cta, warp, lane); else ran = false; }
-            else if (op.type == OP_ATTN) {
-                if (NB == 1) {
-                    attn_phase<HD, false>(md, op, pr, r, cta, n_cta, warp, lane, pr.merge_op != 0, 0, false);
-                } else {
-                    attn_phase<HD, true>(md, op, pr, r, cta, n_cta, warp, lane, true, 0, true);
-                }
-            }
-            else if (op.type == OP_ATTN_MERGE) { if (pr.merge_op) attn_merge_phase<HD>(md, op, pr, cta, n_cta, warp, lane); else ran = false; }
+            else if (op.type == OP_ATTN) attn_phase<HD>(md, op, pr, r, cta, n_cta, warp, lane);
+            else if (op.type == OP_ATTN_MERGE) { if (pr.merge_op) attn_merge_phase<HD>(md, op, pr, r, cta, n_cta, warp, lane); else ran = false; }
             else if (op.type == OP_HIDDEN) { if (pr.want_hidden) hidden_phase(md, pr, r, cta, tid); else ran = false; }
             else if (op.type == OP_ARGMAX) { if (pr.head_row0 < pr.M) argmax_phase(md, pr, r, cta, n_cta, tid); else ran = false; }
         }

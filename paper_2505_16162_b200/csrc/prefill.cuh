@@ -238,14 +238,6 @@ struct Jobs {
     }
 };
 
-// Rotary embedding of a pair by (cos, sin) = c.  The rounding is spelled out: left to the compiler, the contraction's epilogue and
-// rope_kv_rows_kernel fused other products of the second sum, and a row's K depended on which of them a launch's sizes chose.
-__device__ __forceinline__ void rotate_pair(float &a, float &b, float2 c) {
-    const float ra = __fmaf_rn(a, c.x, -__fmul_rn(b, c.y));
-    b = __fmaf_rn(b, c.x, __fmul_rn(a, c.y));
-    a = ra;
-}
-
 // First unit of a CTA's 128 weight rows (SwiGLU: 64 gate rows, then the up rows of the same 64 units).
 template <int EPI> __device__ __forceinline__ int first_unit(int ty, int rank) {
     return EPI == PF_SWIGLU ? ty * (PAIR_UNITS / 2) + 64 * rank : ty * PAIR_UNITS + 128 * rank;
@@ -785,16 +777,6 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t &a0, u
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(a0), "=r"(a1), "=r"(a2), "=r"(a3) : "r"(addr));
 }
 
-// (v0, v1) -> packed bf16 pair (v0 in the low half), round to nearest even; hi part and what is left of it
-__device__ __forceinline__ uint32_t cvt_bf16x2(float v0, float v1) {
-    uint32_t r;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(v1), "f"(v0));
-    return r;
-}
-__device__ __forceinline__ void split_pair(float v0, float v1, uint32_t &hi, uint32_t &lo) {
-    hi = cvt_bf16x2(v0, v1);
-    lo = cvt_bf16x2(v0 - __uint_as_float(hi << 16), v1 - __uint_as_float(hi & 0xffff0000u));
-}
 // c += a . b (m16n8k16, bf16 operands, fp32 accumulation); a pure function of its registers, free to be scheduled
 __device__ __forceinline__ void mma_acc(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
