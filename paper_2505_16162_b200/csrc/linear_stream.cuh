@@ -192,9 +192,10 @@ __device__ __forceinline__ Share make_share(const LinPhase &p, int cta, int n_ct
     Share s;
     s.twin = p.epi == EPI_SWIGLU || p.epi == EPI_HEADS;
     s.gsz = s.twin ? 8 : 16;
-    s.u_lo = (int)(((long long)p.units * cta) / n_cta);
-    const int u_hi = (int)(((long long)p.units * (cta + 1)) / n_cta);
-    s.n_units = u_hi - s.u_lo;
+    // [units cta / n_cta, units (cta + 1) / n_cta), in 32 bits
+    const unsigned each = (unsigned)p.units / (unsigned)n_cta, rest = (unsigned)p.units - each * (unsigned)n_cta;
+    s.u_lo = (int)(each * cta + rest * cta / (unsigned)n_cta);
+    s.n_units = (int)(each * (cta + 1) + rest * (cta + 1) / (unsigned)n_cta) - s.u_lo;
     s.n_groups = (s.n_units + s.gsz - 1) / s.gsz;
     s.g_base = s.n_groups ? s.n_units / s.n_groups : 0;
     s.g_rem = s.n_groups ? s.n_units % s.n_groups : 0;

@@ -31,7 +31,7 @@ constexpr unsigned BAR_SPIN_LIMIT = 4000000u;
 enum { OP_EMBED = 0, OP_LINEAR = 1, OP_ATTN = 2, OP_HIDDEN = 3, OP_ARGMAX = 4, OP_ATTN_MERGE = 5 };
 constexpr int MERGE_ROWS = 3;      // tasks with at least this many (row, head) pairs leave the merge to a separate operation
 
-struct Op {
+struct alignas(16) Op {
     int type;
     int barrier_after;   // 1: all CTAs meet before the next operation starts
     int is_head;         // OP_LINEAR: the LM head (runs on rows head_row0.. only)
@@ -39,6 +39,8 @@ struct Op {
     LinPhase lin;        // OP_LINEAR; OP_EMBED and OP_ATTN use its ys / next_gain / ss_out fields for their output
     bf16_t *kc, *vc;     // OP_ATTN: this layer's cache [n_kv_heads][max_seq][head_dim]
 };
+constexpr int OP_SLOTS_AT = 256;   // where the ring's bytes for barriers hold the operation at work and the one behind it
+static_assert(OP_SLOTS_AT + 2 * sizeof(Op) <= stream::BAR_BYTES && 2 * stream::WS * 8 + 16 <= OP_SLOTS_AT, "two operations beside the ring's barriers");
 
 struct Model {           // what does not change from pass to pass
     const bf16_t *tok_embed;
@@ -507,8 +509,21 @@ __global__ void __launch_bounds__(stream::NTHREADS, 1) pass_kernel(const Model m
     stream::regs_inc<stream::REGS_CONSUMER>();
     const int tid = threadIdx.x;
     unsigned long long n_bar = 0;
+    // The operation behind the one at work is on its way into shared memory: read from L2 when its turn came (a barrier leaves nothing in
+    // L1), its type and then its fields took two trips of ~0.6 us, six times a layer.
+    Op *slots = reinterpret_cast<Op *>(reinterpret_cast<unsigned char *>(r.full_w) + OP_SLOTS_AT);
+    auto fetch_op = [&](int i) {
+        if (i < pr.n_ops && tid < (int)(sizeof(Op) / 16))
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(stream::smem_u32(slots + (i & 1)) + 16 * tid),
+                         "l"(reinterpret_cast<const unsigned char *>(pr.ops + i) + 16 * tid) : "memory");
+    };
+    auto op_arrived = [] { asm volatile("cp.async.wait_all;" ::: "memory"); };
+    fetch_op(0);
+    op_arrived();
+    asm volatile("bar.sync 1, %0;" ::"n"(NCW * 32) : "memory");
     for (int i = 0; i < pr.n_ops; ++i) {
-        const Op &op = pr.ops[i];
+        const Op &op = slots[i & 1];
+        fetch_op(i + 1);                       // over the operation before this one, which all have left
         bool ran = true;
         if (op.type == OP_LINEAR) {
             LinPhase lp = op.lin;
@@ -531,10 +546,13 @@ __global__ void __launch_bounds__(stream::NTHREADS, 1) pass_kernel(const Model m
             else if (op.type == OP_ARGMAX) { if (pr.head_row0 < pr.M) argmax_phase(md, pr, r, cta, n_cta, tid); else ran = false; }
         }
         if (md.trace && cta == 0 && tid == 0) md.trace[2 * i] = globaltimer_ns();
+        op_arrived();
         if (op.barrier_after && ran) {
             ++n_bar;
             alive = grid_barrier(md, r, pr.bar_base + n_bar * (unsigned long long)n_cta, tid, alive,
                                  pr.bar_spin_limit ? pr.bar_spin_limit : BAR_SPIN_LIMIT);
+        } else {
+            asm volatile("bar.sync 1, %0;" ::"n"(NCW * 32) : "memory");
         }
         if (md.trace && cta == 0 && tid == 0) md.trace[2 * i + 1] = globaltimer_ns();
     }
