@@ -73,7 +73,7 @@ struct knnssd_ctx {
     bool mega_ok = false;
     pass::Model model{};
     pass::Op *ops_full = nullptr, *ops_draft = nullptr;     // device op lists
-    int n_ops_full = 0, n_ops_draft = 0, bar_full = 0, bar_draft = 0;   // ops and barriers (without head / hidden parts)
+    int n_ops_full = 0, n_ops_draft = 0, bar_full = 0, bar_draft = 0;   // ops and barriers (without merge operations)
     int attn_full = 0, attn_draft = 0;                                  // attention sublayers in each list
     std::vector<unsigned char> ops_draft_mask;              // the mask ops_draft was built for
     unsigned long long *bar = nullptr, bar_total = 0;
@@ -381,8 +381,8 @@ LinearArgs make_args(const void *W0, int rows0, int n_in, const float *x, const 
 }
 
 // ---- persistent pass kernel: op lists and launch ----------------------------------------------------------------
-// The list of one pass under a skip mask (nullptr = full model).  n_bar receives the number of grid barriers of the
-// body; the head part (when rows get logits) adds one more.
+// The list of one pass under a skip mask (nullptr = full model).  n_bar receives the number of its grid barriers
+// (merge operations, which run in some passes, add one each).
 std::vector<pass::Op> build_ops(const knnssd_ctx *c, const unsigned char *mask, int *n_bar, int *n_attn) {
     const knnssd_config &g = c->cfg;
     const int d = g.d_model, hd = g.head_dim, nq = g.n_heads * hd, nkv = g.n_kv_heads * hd, F = g.d_ff, V = g.vocab;
@@ -444,7 +444,8 @@ std::vector<pass::Op> build_ops(const knnssd_ctx *c, const unsigned char *mask, 
     hdn.type = pass::OP_HIDDEN;                      // runs only when the pass wants hidden states; no barrier: reads x only
     ops.push_back(hdn);
     pass::Op head = lin(c->lm_head, V, d, c->x, c->final_norm, c->logits, EPI_STORE);
-    head.is_head = 1;                                // runs only when rows get logits; its barrier counts only then
+    head.is_head = 1;                                // runs only when rows get logits; the arg-max behind it starts from its CTA's own
+    head.barrier_after = 0;
     head.lin.xs = c->xs_x; head.lin.ss_in = c->ssp;
     ops.push_back(head);
     pass::Op am{};
@@ -503,7 +504,6 @@ void run_pass_mega(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const 
     pr.out_row0 = out_row0;
     pr.bar_spin_limit = c->bar_spin_limit;
     pr.bar_base = c->bar_total;
-    if (head_row0 < M) bars += 1;
     pr.merge_op = pass::merge_rows_separately(M, c->cfg.n_heads / c->cfg.n_kv_heads) ? 1 : 0;
     if (pr.merge_op) bars += n_attn;
     cudaError_t e;

@@ -188,14 +188,18 @@ struct Share {
     __device__ __forceinline__ int group_size(int g) const { return g_base + (g < g_rem ? 1 : 0); }
 };
 
+// The units of a CTA: [units cta / n_cta, units (cta + 1) / n_cta), in 32 bits.
+__device__ __forceinline__ void unit_range(int units, int cta, int n_cta, int &lo, int &n) {
+    const unsigned each = (unsigned)units / (unsigned)n_cta, rest = (unsigned)units - each * (unsigned)n_cta;
+    lo = (int)(each * cta + rest * cta / (unsigned)n_cta);
+    n = (int)(each * (cta + 1) + rest * (cta + 1) / (unsigned)n_cta) - lo;
+}
+
 __device__ __forceinline__ Share make_share(const LinPhase &p, int cta, int n_cta) {
     Share s;
     s.twin = p.epi == EPI_SWIGLU || p.epi == EPI_HEADS;
     s.gsz = s.twin ? 8 : 16;
-    // [units cta / n_cta, units (cta + 1) / n_cta), in 32 bits
-    const unsigned each = (unsigned)p.units / (unsigned)n_cta, rest = (unsigned)p.units - each * (unsigned)n_cta;
-    s.u_lo = (int)(each * cta + rest * cta / (unsigned)n_cta);
-    s.n_units = (int)(each * (cta + 1) + rest * (cta + 1) / (unsigned)n_cta) - s.u_lo;
+    unit_range(p.units, cta, n_cta, s.u_lo, s.n_units);
     s.n_groups = (s.n_units + s.gsz - 1) / s.gsz;
     s.g_base = s.n_groups ? s.n_units / s.n_groups : 0;
     s.g_rem = s.n_groups ? s.n_units % s.n_groups : 0;

@@ -96,13 +96,18 @@ __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long
     return v;
 }
 
-// Called by all 256 consumer threads.  Returns false once the pass has been aborted.
+// Called by all 256 consumer threads.  Returns false once the pass has been aborted.  meanwhile(): what the CTA has to do for itself, done
+// between its arrival and the wait for the others.
+template <typename F>
 __device__ __forceinline__ bool grid_barrier(const Model &md, const Ring &r, unsigned long long target, int tid, bool alive,
-                                             unsigned spin_limit) {
+                                             unsigned spin_limit, F meanwhile) {
     asm volatile("bar.sync 1, %0;" ::"n"(NCW * 32) : "memory");
     if (tid == 0 && alive) {
         __threadfence();                       // cumulative: covers the writes of the CTA's other threads ordered by the bar.sync
         atomicAdd(md.bar, 1ULL);
+    }
+    meanwhile();
+    if (tid == 0 && alive) {
         unsigned spins = 0;
         while (ld_acquire_u64(md.bar) < target) {
             // the abort words are looked at every 64 polls: a second trip to L2 per poll doubled the time between polls
@@ -121,24 +126,14 @@ __device__ __forceinline__ bool grid_barrier(const Model &md, const Ring &r, uns
     return alive && !*r.abort_flag;
 }
 
-// ---- embedding gather + rotary table ----------------------------------------------------------------------
-__device__ __forceinline__ void embed_phase(const Model &md, const Op &op, const Params &pr, const Ring &r, int cta, int n_cta,
+// What runs once a pass is kept out of line: inlined, it shifted the registers and the code of the linear maps by up to 1 % of a pass.
+// ---- embedding gather ----------------------------------------------------------------------------------------
+__device__ __noinline__ void embed_phase(const Model &md, const Op &op, const Params &pr, const Ring &r, int cta, int n_cta,
                                             int tid) {
-    const int d = md.d_model, half = md.hd >> 1;
-    {   // every CTA fills its own copy of the (cos, sin) table of all rows: 148 readers of one copy would queue up at L2
-        const int p0 = md.state->len + pr.pos_off;
-        if (tid == 0) *r.pos0 = p0;
-        float2 *mine = md.rope_cs + (size_t)cta * MAXM * half;
-        for (int idx = tid; idx < pr.M * half; idx += NCW * 32) {
-            const int m = idx / half, i = idx % half;
-            double s, c;
-            sincos((double)(p0 + m) * md.inv_freq[i], &s, &c);
-            mine[idx] = make_float2((float)c, (float)s);
-        }
-    }
+    if (tid == 0) *r.pos0 = md.state->len + pr.pos_off;
     if (cta >= pr.M) return;                               // whole CTAs only: the named barrier below is CTA-local
     // row m = cta: residual stream in fp32, its pre-split form times the first RMSNorm's gain, its sum of squares
-    const int m = cta, lane = tid & 31, warp = tid >> 5;
+    const int d = md.d_model, m = cta, lane = tid & 31, warp = tid >> 5;
     int t = pr.tok[m];
     if (t < 0 || t >= md.vocab) {                          // never gather outside the table: report and read row 0 instead
         if (tid == 0) atomicExch(md.err, ERR_BAD_TOKEN);
@@ -146,11 +141,23 @@ __device__ __forceinline__ void embed_phase(const Model &md, const Op &op, const
     }
     const bf16_t *row = md.tok_embed + (size_t)t * d;
     float ss = 0.f;
-    for (int i = tid; i < d; i += NCW * 32) {
-        const float v = bf16_bits_to_float(row[i]);
-        __stcg(md.x + (size_t)m * d + i, v);
-        stream::store_split(op.lin.ys, d >> 7, m, i, op.lin.next_gain ? v * __ldg(op.lin.next_gain + i) : v);
-        ss = fmaf(v, v, ss);
+    constexpr int U = 10;                                  // values in flight
+    for (int i0 = tid; i0 < d; i0 += U * NCW * 32) {
+        float v[U], g[U];
+#pragma unroll
+        for (int e = 0; e < U; ++e) {
+            const int i = i0 + e * NCW * 32;
+            v[e] = i < d ? bf16_bits_to_float(__ldg(row + i)) : 0.f;
+            g[e] = i < d && op.lin.next_gain ? __ldg(op.lin.next_gain + i) : 1.f;
+        }
+#pragma unroll
+        for (int e = 0; e < U; ++e) {
+            const int i = i0 + e * NCW * 32;
+            if (i >= d) break;
+            __stcg(md.x + (size_t)m * d + i, v[e]);
+            stream::store_split(op.lin.ys, d >> 7, m, i, v[e] * g[e]);
+            ss = fmaf(v[e], v[e], ss);
+        }
     }
     ss = warp_sum(ss);
     if (lane == 0) r.red_ss[32 + warp] = ss;
@@ -161,11 +168,22 @@ __device__ __forceinline__ void embed_phase(const Model &md, const Op &op, const
         __stcg(op.lin.ss_out + (size_t)m * n_cta, tot);
     }
     for (int c = 1 + tid; c < n_cta; c += NCW * 32) __stcg(op.lin.ss_out + (size_t)m * n_cta + c, 0.f);
-    asm volatile("bar.sync 1, %0;" ::"n"(NCW * 32) : "memory");
+}
+
+// The (cos, sin) of all rows' rotary angles, a copy for every CTA: 148 readers of one copy would queue up at L2.  Nobody else waits for it.
+__device__ __noinline__ void rope_table(const Model &md, const Params &pr, int cta, int tid) {
+    const int half = md.hd >> 1, p0 = md.state->len + pr.pos_off;
+    float2 *mine = md.rope_cs + (size_t)cta * MAXM * half;
+    for (int idx = tid; idx < pr.M * half; idx += NCW * 32) {
+        const int m = idx / half, i = idx % half;
+        double s, c;
+        sincos((double)(p0 + m) * md.inv_freq[i], &s, &c);
+        mine[idx] = make_float2((float)c, (float)s);
+    }
 }
 
 // ---- RMSNorm of the rows written out (hidden-state output) -------------------------------------------------
-__device__ __forceinline__ void hidden_phase(const Model &md, const Params &pr, const Ring &r, int cta, int tid) {
+__device__ __noinline__ void hidden_phase(const Model &md, const Params &pr, const Ring &r, int cta, int tid) {
     if (cta >= pr.M) return;          // whole CTAs only: the named barrier below is CTA-local
     const int d = md.d_model, m = cta, lane = tid & 31, warp = tid >> 5;
     const float *xr = md.x + (size_t)m * d;
@@ -181,57 +199,64 @@ __device__ __forceinline__ void hidden_phase(const Model &md, const Params &pr, 
     asm volatile("bar.sync 1, %0;" ::"n"(NCW * 32) : "memory");
 }
 
-// ---- greedy arg-max: every CTA scans a slice of each row, the last one to finish folds the partials --------
-__device__ __forceinline__ void argmax_phase(const Model &md, const Params &pr, const Ring &r, int cta, int n_cta, int tid) {
-    const int V = md.vocab, lane = tid & 31, warp = tid >> 5;
-    const int per = (V + n_cta - 1) / n_cta, i0 = cta * per, i1 = min(V, i0 + per);
-    float *s_v = r.red;
-    int *s_i = reinterpret_cast<int *>(r.red + 64);
-    int *s_last = reinterpret_cast<int *>(r.red + 128);
-    const int rows = pr.M - pr.head_row0;
-    for (int m = 0; m < rows; ++m) {
-        const float *row = md.logits + (size_t)(pr.out_row0 + pr.head_row0 + m) * V;
-        float bv = -INFINITY;
-        int bi = 0x7fffffff;
-        for (int i = i0 + tid; i < i1; i += NCW * 32) argmax_fold(bv, bi, __ldcg(row + i), i);
+// ---- greedy arg-max: every CTA scans the logits that it has just made (no barrier lies between), the last one folds the partials ----
+// All warps share a row's slice, two rows at a time.  Row after row behind a barrier of the grid, five rows took 7.2 us and nine 10.
+__device__ __noinline__ void argmax_phase(const Model &md, const Params &pr, const Ring &r, int cta, int n_cta, int tid) {
+    const int V = md.vocab, lane = tid & 31, warp = tid >> 5, rows = pr.M - pr.head_row0;
+    int i0, n;
+    stream::unit_range(V, cta, n_cta, i0, n);
+    float *s_v = r.red;                        // [rows][NCW]
+    int *s_i = reinterpret_cast<int *>(r.red + MAXM * NCW);
+    int *s_last = reinterpret_cast<int *>(r.red + 2 * MAXM * NCW);
+    auto fold_warp = [](float &bv, int &bi) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
             const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
             argmax_fold(bv, bi, ov, oi);
         }
-        if (lane == 0) { s_v[warp] = bv; s_i[warp] = bi; }
-        asm volatile("bar.sync 1, %0;" ::"n"(NCW * 32) : "memory");
-        if (tid == 0) {
-            for (int w = 1; w < NCW; ++w) argmax_fold(bv, bi, s_v[w], s_i[w]);
-            __stcg(md.amax_v + m * n_cta + cta, bv);
-            __stcg(md.amax_i + m * n_cta + cta, bi);
+    };
+    for (int m = 0; m < rows; m += 2) {
+        const float *row0 = md.logits + (size_t)(pr.out_row0 + pr.head_row0 + m) * V + i0, *row1 = row0 + (m + 1 < rows ? V : 0);
+        float v0 = -INFINITY, v1 = -INFINITY;
+        int k0 = 0x7fffffff, k1 = 0x7fffffff;
+#pragma unroll 5
+        for (int i = tid; i < n; i += NCW * 32) {
+            argmax_fold(v0, k0, __ldcg(row0 + i), i0 + i);
+            argmax_fold(v1, k1, __ldcg(row1 + i), i0 + i);
         }
-        asm volatile("bar.sync 1, %0;" ::"n"(NCW * 32) : "memory");
+        fold_warp(v0, k0);
+        fold_warp(v1, k1);
+        if (lane == 0) { s_v[m * NCW + warp] = v0; s_i[m * NCW + warp] = k0; s_v[(m + 1) * NCW + warp] = v1; s_i[(m + 1) * NCW + warp] = k1; }
     }
-    __threadfence();
     asm volatile("bar.sync 1, %0;" ::"n"(NCW * 32) : "memory");
-    if (tid == 0) *s_last = (atomicAdd(md.amax_cnt, 1) == n_cta - 1);
+    if (warp == 0) {
+        if (lane < rows) {
+            float bv = -INFINITY;
+            int bi = 0x7fffffff;
+            for (int w = 0; w < NCW; ++w) argmax_fold(bv, bi, s_v[lane * NCW + w], s_i[lane * NCW + w]);
+            __stcg(md.amax_v + lane * n_cta + cta, bv);
+            __stcg(md.amax_i + lane * n_cta + cta, bi);
+        }
+        __syncwarp();
+        if (lane == 0) {
+            __threadfence();
+            *s_last = atomicAdd(md.amax_cnt, 1) == n_cta - 1;
+        }
+    }
     asm volatile("bar.sync 1, %0;" ::"n"(NCW * 32) : "memory");
     if (*s_last) {
         __threadfence();
-        if (warp < rows && warp < NCW) {
-            for (int m = warp; m < rows; m += NCW) {
-                float bv = -INFINITY;
-                int bi = 0x7fffffff;
-                for (int b = lane; b < n_cta; b += 32) argmax_fold(bv, bi, __ldcg(md.amax_v + m * n_cta + b), __ldcg(md.amax_i + m * n_cta + b));
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
-                    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-                    argmax_fold(bv, bi, ov, oi);
-                }
-                if (lane == 0) pr.argmax_out[m] = argmax_checked(bi, V, md.err);
-            }
+        for (int m = warp; m < rows; m += NCW) {
+            float bv = -INFINITY;
+            int bi = 0x7fffffff;
+#pragma unroll 5
+            for (int b = lane; b < n_cta; b += 32) argmax_fold(bv, bi, __ldcg(md.amax_v + m * n_cta + b), __ldcg(md.amax_i + m * n_cta + b));
+            fold_warp(bv, bi);
+            if (lane == 0) pr.argmax_out[m] = argmax_checked(bi, V, md.err);
         }
         if (tid == 0) *md.amax_cnt = 0;
     }
-    asm volatile("bar.sync 1, %0;" ::"n"(NCW * 32) : "memory");
 }
 
 // ---- attention over the KV cache ------------------------------------------------------------------------------
@@ -481,7 +506,7 @@ __device__ __forceinline__ void attn_merge_phase(const Model &md, const Op &op, 
 // NP > 0: the linear maps take the rows four at a time with both terms in one operand (NP = 1: passes of up to 4 rows -
 // every draft step; NP = 3, 4 with NB = 2: passes of 9..12 and 13..16 rows); NP = 0: eight at a time, one operand per term.
 template <int HD, int NB, int NP>
-__global__ void __launch_bounds__(stream::NTHREADS, 1) pass_kernel(const Model md, const Params pr) {
+__global__ void __launch_bounds__(stream::NTHREADS, 1) pass_kernel(const __grid_constant__ Model md, const __grid_constant__ Params pr) {
     extern __shared__ __align__(128) unsigned char smem[];
     Ring r;
     stream::ring_setup(r, smem, md.err);
@@ -550,7 +575,8 @@ __global__ void __launch_bounds__(stream::NTHREADS, 1) pass_kernel(const Model m
         if (op.barrier_after && ran) {
             ++n_bar;
             alive = grid_barrier(md, r, pr.bar_base + n_bar * (unsigned long long)n_cta, tid, alive,
-                                 pr.bar_spin_limit ? pr.bar_spin_limit : BAR_SPIN_LIMIT);
+                                 pr.bar_spin_limit ? pr.bar_spin_limit : BAR_SPIN_LIMIT,
+                                 [&] { if (op.type == OP_EMBED) rope_table(md, pr, cta, tid); });
         } else {
             asm volatile("bar.sync 1, %0;" ::"n"(NCW * 32) : "memory");
         }
