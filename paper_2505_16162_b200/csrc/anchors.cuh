@@ -5,8 +5,8 @@
 // The points are fp32 [N][d] (d = the model width, N = domains x samples per domain: 5 x 1000 in the paper's
 // set-up, 100 MB at d = 5120).  Centroids and their sums are fp64.  A squared distance is formed from fp32
 // differences to the fp32-rounded centroid, squared and added eight at a time in fp32, and those short sums are
-// accumulated without loss in pairs of floats (fp64 only for the final reductions): the fp64 pipe of this GPU issues
-// a few lanes per clock per SM, so per-element fp64 arithmetic made the assignment 15x slower than its memory
+// accumulated without loss in pairs of floats (fp64 only for the final reductions): a float becomes a double at 15 lanes per clock and SM
+// (fp64 additions and products 58), so fp64 arithmetic for every element and cluster made the assignment 15x slower than its memory
 // traffic, while this form keeps ~1e-8 relative accuracy (error of a
 // distance^2 of ~1e3: ~1e-5, four orders below the gaps that decide nearest centroids and nearest members).  A round
 // reads the points twice (assignment, centroid sums).  Every reduction has a fixed order: results do not depend on
@@ -172,9 +172,19 @@ __global__ void __launch_bounds__(256, NC <= 8 ? 3 : 2) assign_kernel(const floa
     }
 }
 
+// Slices of the centroid sums: at least 64 points each, at most 64 slices, and as many as keep all blocks resident (six on an SM) if that is
+// fewer: then the sorted form runs.
+constexpr int SUM_BLOCKS = 6;
+inline int sum_slices(int N, int d, int n_sms, bool &sorted) {
+    int S = (N + 63) / 64;
+    if (S > 64) S = 64;
+    const int cols = (d + 255) / 256, most = SUM_BLOCKS * n_sms / cols;
+    sorted = S > most;
+    return !sorted ? S : most > 1 ? most : 1;
+}
 // part[s][c][j] = sum of x[p][j] over the points p of slice s (S slices of `per` consecutive points) labelled c, added
-// in index order.  grid = (ceil(d / 256), S), 256 threads: a thread owns one column.  Bound by the fp64 pipe, which issues
-// about 4 lanes per clock and SM: 29 us for 5000 x 5120, the time of its 26 million additions.
+// in index order.  grid = (ceil(d / 256), S), 256 threads: a thread owns one column.  Bound by the trips to memory, eight points at a
+// time.  (The fp64 pipe has room: 58 additions and 15 conversions per clock and SM, measured.)
 __global__ void __launch_bounds__(256) partial_sums_kernel(const float *__restrict__ x, int N, int d, const int *__restrict__ labels,
                                                            int n, int per, double *__restrict__ part, int parity,
                                                            const Progress *__restrict__ pg) {
@@ -200,10 +210,72 @@ __global__ void __launch_bounds__(256) partial_sums_kernel(const float *__restri
         for (int c = 0; c < n; ++c) part[((size_t)s * n + c) * d + j] = acc[c][threadIdx.x];
 }
 
+// The same where its blocks would not all be resident at once: fewer and longer slices (sum_slices), whose points are taken cluster by
+// cluster - a stable sort of at most 256 of them at a time -, so that a running sum stays in a register and only goes to shared memory
+// where the cluster changes.  5000 x 5120: 26 us for 32 in one and a half rounds of blocks, the call of four rounds 320 us for 341; 4000 x 4096 252
+// for 258.  Where all blocks of the plain form are resident the sort only costs: 120 x 1024 106 us for 101, 1200 x 2049 157 for 150.  (The
+// running sums in as much shared memory as there: another size has the SM's memory divided anew between kernels, 5 .. 7 us a round.)
+constexpr int SUM_LOADS = 8;
+__global__ void __launch_bounds__(256, 6) sorted_sums_kernel(const float *__restrict__ x, int N, int d, const int *__restrict__ labels,
+                                                              int n, int per, double *__restrict__ part, int parity,
+                                                              const Progress *__restrict__ pg) {
+    chain_wait();
+    if (pg->done || !pg->changed[parity]) return;
+    __shared__ double sum_acc[MAXC * 256];                     // [n][256]
+    __shared__ int order[256], first[MAXC + 1], in_warp[8][MAXC];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, j = blockIdx.x * 256 + tid, s = blockIdx.y;
+    const int p0 = s * per, p1 = min(N, p0 + per);
+    const float *col = x + min(j, d - 1);
+    for (int c = 0; c < n; ++c) sum_acc[c * 256 + tid] = 0.0;
+    for (int q0 = p0; q0 < p1; q0 += 256) {
+        const int len = min(256, p1 - q0), l = tid < len ? labels[q0 + tid] : -1;
+        unsigned mine = 0u;
+        for (int c = 0; c < n; ++c) {
+            const unsigned who = __ballot_sync(0xffffffffu, l == c);
+            if (l == c) mine = who;
+            if (lane == 0) in_warp[warp][c] = __popc(who);
+        }
+        __syncthreads();                                       // the counts are there, the order before has been read
+        if (l >= 0) {
+            int at = __popc(mine & ((1u << lane) - 1u));
+            for (int c = 0; c < l; ++c)
+#pragma unroll
+                for (int w = 0; w < 8; ++w) at += in_warp[w][c];
+            for (int w = 0; w < warp; ++w) at += in_warp[w][l];
+            order[at] = q0 + tid;
+        }
+        if (tid <= n) {
+            int at = 0;
+            for (int c = 0; c < tid; ++c)
+#pragma unroll
+                for (int w = 0; w < 8; ++w) at += in_warp[w][c];
+            first[tid] = at;
+        }
+        __syncthreads();
+        int c = 0, end = first[1];
+        double a = sum_acc[tid];
+        for (int i0 = 0; i0 < len; i0 += SUM_LOADS) {
+            float v[SUM_LOADS];
+#pragma unroll
+            for (int e = 0; e < SUM_LOADS; ++e) v[e] = __ldg(col + (size_t)order[min(i0 + e, len - 1)] * d);
+#pragma unroll
+            for (int e = 0; e < SUM_LOADS; ++e) {
+                if (i0 + e >= len) break;                      // uniform, as are the clusters' ends
+                while (i0 + e >= end) { sum_acc[c * 256 + tid] = a; ++c; a = sum_acc[c * 256 + tid]; end = first[c + 1]; }
+                a += (double)v[e];
+            }
+        }
+        sum_acc[c * 256 + tid] = a;
+    }
+    if (j < d)
+        for (int c = 0; c < n; ++c) part[((size_t)s * n + c) * d + j] = sum_acc[c * 256 + tid];
+}
+
 // The end of a round.  If it changed an assignment: mu[c][j] = (sum over slices, in slice order, of part[s][c][j]) /
 // counts[c], in mu32 rounded to fp32; a cluster without members keeps its centroid.  Otherwise the iteration is done.  Clears
-// the counters of the next round.  grid = (ceil(d / 256), n), 256 threads.
-__global__ void fold_centroids_kernel(const double *__restrict__ part, int n, int d, int S, double *__restrict__ mu, float *__restrict__ mu32,
+// the counters of the next round.  grid = (ceil(d / 128), n), 128 threads.  Bound by the trips to L2: twenty slices in flight (44 slices of
+// 5 x 5120 7.5 us; eight of 64 in flight took 9.3).
+__global__ void __launch_bounds__(128) fold_centroids_kernel(const double *__restrict__ part, int n, int d, int S, double *__restrict__ mu, float *__restrict__ mu32,
                                       int ld, int parity, Progress *__restrict__ pg) {
     chain_wait();
     const bool changed = pg->changed[parity] != 0;
@@ -214,18 +286,18 @@ __global__ void fold_centroids_kernel(const double *__restrict__ part, int n, in
         for (int c = 0; c < MAXC; ++c) pg->counts[parity ^ 1][c] = 0;
         if (!changed) pg->done = 1;
     }
-    const int j = blockIdx.x * 256 + threadIdx.x, c = blockIdx.y;
+    const int j = blockIdx.x * 128 + threadIdx.x, c = blockIdx.y;
     if (!changed || j >= d || pg->counts[parity][c] == 0) return;
     double s = 0.0;
-    int i = 0;
-    for (; i + 8 <= S; i += 8) {                              // eight loads in flight, added in slice order
-        double v[8];
+    constexpr int U = 20;                                     // loads in flight, added in slice order
+    for (int i = 0; i < S; i += U) {
+        double v[U];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = part[((size_t)(i + e) * n + c) * d + j];
+        for (int e = 0; e < U; ++e) v[e] = i + e < S ? __ldcg(part + ((size_t)(i + e) * n + c) * d + j) : 0.0;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) s += v[e];
+        for (int e = 0; e < U; ++e)
+            if (i + e < S) s += v[e];
     }
-    for (; i < S; ++i) s += part[((size_t)i * n + c) * d + j];
     s /= (double)pg->counts[parity][c];
     mu[(size_t)c * d + j] = s;
     mu32[(size_t)c * ld + j] = (float)s;
@@ -255,9 +327,30 @@ __global__ void __launch_bounds__(256) member_dist_kernel(const float *__restric
     const float *xr = x + (size_t)p * d;
     const double *m = mu + (size_t)labels[p] * d;
     double s = 0.0;
-    for (int j = lane; j < d; j += 32) {
-        const double df = (double)__ldg(xr + j) - m[j];
+    auto take = [&](float v, double c) {
+        const double df = (double)v - c;
         s = fma(df, df, s);
+    };
+    if (d % 4 == 0) {                                          // rows of both are aligned to what is read at once
+        constexpr int U = 4;                                   // 512 columns in flight
+        for (int j0 = 4 * lane; j0 < d; j0 += 128 * U) {
+            float4 v[U];
+            double2 a[U], b[U];
+#pragma unroll
+            for (int e = 0; e < U; ++e) {
+                const int j = min(j0 + 128 * e, d - 4);
+                const uint4 t = ld_stream16(xr + j);         // a point comes by once: L1 is left to the centroids
+                v[e] = make_float4(__uint_as_float(t.x), __uint_as_float(t.y), __uint_as_float(t.z), __uint_as_float(t.w));
+                a[e] = __ldg(reinterpret_cast<const double2 *>(m + j));
+                b[e] = __ldg(reinterpret_cast<const double2 *>(m + j) + 1);
+            }
+#pragma unroll
+            for (int e = 0; e < U; ++e)
+                if (j0 + 128 * e < d) { take(v[e].x, a[e].x); take(v[e].y, a[e].y); take(v[e].z, b[e].x); take(v[e].w, b[e].y); }
+        }
+    } else {
+#pragma unroll 8
+        for (int j = lane; j < d; j += 32) take(__ldg(xr + j), __ldg(m + j));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -266,7 +359,7 @@ __global__ void __launch_bounds__(256) member_dist_kernel(const float *__restric
 
 // Eq. (2) for cluster c = blockIdx.x: k times, the not yet taken member with the smallest (distance, index);
 // out[c][r] = its index, -1 once the cluster has run out of members.  Distances are compared as the bit patterns of non-negative
-// doubles: the fp64 pipe takes eight clocks for a warp's comparison.  A copy of them in shared memory (staged != 0: N words), NO_KEY for
+// doubles.  A copy of them in shared memory (staged != 0: N words), NO_KEY for
 // points that are no member or taken, serves all k searches; longer lists are read from global memory each time, taken[N]
 // starting at zero.  SEL_NT threads.  Staged and k <= SEL_K: every warp takes the k first of its own points, without
 // meeting the others, and one warp merges the lists (5 x 10 of 5000 points: 15 us; a meeting of the block per anchor and fp64

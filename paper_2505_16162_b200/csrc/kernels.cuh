@@ -443,7 +443,7 @@ __global__ void pool_accumulate_kernel(const float *__restrict__ h, int M, int d
 
 // The same for many rows, without writing the normalised rows out: part[s][i] = fp64 sum, in row order, of the rows of slice s
 // (POOL_ROWS rows each), every term the row's value times its RMSNorm scale times the gain, rounded as rmsnorm_rows_kernel does;
-// pool_fold_kernel adds the slices in order.  The fp64 additions (about 4 lanes per clock and SM) want all SMs: one thread per
+// pool_fold_kernel adds the slices in order.  The loads want all SMs: one thread per
 // column walking 1024 rows took 83 us, this 16 with the scales.  grid = (ceil(d / 256), slices), 256 threads.
 constexpr int POOL_ROWS = 32;
 __global__ void __launch_bounds__(256) pool_partial_kernel(const float *__restrict__ x, const float *__restrict__ rinv, const float *__restrict__ gain,

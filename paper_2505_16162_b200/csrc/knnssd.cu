@@ -1785,8 +1785,9 @@ knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int 
     if (reinterpret_cast<uintptr_t>(x_dev) & 15u) return KNNSSD_ERR_SHAPE;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
     const int N = n_points, n = n_clusters;
-    int S = (N + 63) / 64;                        // slices of the centroid sums: at least 64 points each, at most 64 slices
-    if (S > 64) S = 64;
+    const int sms = sm_count();
+    bool sorted = false;
+    const int S = anchors::sum_slices(N, d, sms, sorted);
     const int per = (N + S - 1) / S;
     const int ld = (d + 3) / 4 * 4;                 // row stride of the fp32 centroids
     double *mu = nullptr, *dist = nullptr, *part = nullptr;
@@ -1813,7 +1814,8 @@ knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int 
     typedef void (*AssignFn)(const float *, int, int, const float *, int, int, int, int *, anchors::Progress *);
     const AssignFn assign = vec ? (n <= 4 ? anchors::assign_kernel<true, 4> : n <= 8 ? anchors::assign_kernel<true, 8> : anchors::assign_kernel<true, 16>)
                                 : (n <= 4 ? anchors::assign_kernel<false, 4> : n <= 8 ? anchors::assign_kernel<false, 8> : anchors::assign_kernel<false, 16>);
-    const int sms = sm_count(), warps = anchors::assign_warps(N, n, sms);
+    const int warps = anchors::assign_warps(N, n, sms);
+    const auto sums = sorted ? anchors::sorted_sums_kernel : anchors::partial_sums_kernel;
     auto smem_of = [&](int w) { return n <= 4 ? anchors::assign_smem<4>(w) : n <= 8 ? anchors::assign_smem<8>(w) : anchors::assign_smem<16>(w); };
     const int assign_smem = smem_of(warps);
     const int staged = N <= anchors::SEL_STAGED, sel_smem = staged ? N * (int)sizeof(double) : 0;
@@ -1839,8 +1841,8 @@ knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int 
             launch_chained(assign, dim3((N + 2 * warps - 1) / (2 * warps)), dim3(32 * warps), assign_smem, s, x_dev, N, d, mu32, ld, n, r & 1, labels, progress);
             // not chained: set up under the end of the assignment, its few blocks all go to the SMs that are free first (50000 x 256: 135 us a
             // round so, 97 .. 99 with all SMs free)
-            anchors::partial_sums_kernel<<<dim3(cols.x, S), 256, 0, s>>>(x_dev, N, d, labels, n, per, part, r & 1, progress);
-            launch_chained(anchors::fold_centroids_kernel, cols, dim3(256), 0, s, part, n, d, S, mu, mu32, ld, r & 1, progress);
+            sums<<<dim3(cols.x, S), 256, 0, s>>>(x_dev, N, d, labels, n, per, part, r & 1, progress);
+            launch_chained(anchors::fold_centroids_kernel, dim3((d + 127) / 128, n), dim3(128), 0, s, part, n, d, S, mu, mu32, ld, r & 1, progress);
         }
         cudaEventRecord(e1, s);
         if ((e = cudaGetLastError()) != cudaSuccess) break;      // without all of its rounds' launches there are no labels to rank by

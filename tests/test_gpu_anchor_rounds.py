@@ -52,3 +52,10 @@ def test_more_results_than_are_kept_pinned():
     """Labels and anchors of 262200 points are more words than a thread keeps pinned: they come by copies, done in one batch or several."""
     for limit in (2, 6):
         _run(262200, 4, 3, 4, limit, 15, 1.5)
+
+
+@pytest.mark.parametrize("n_points,d,n", [(1301, 39999, 7), (900, 16388, 16), (1280, 3585, 1)])
+def test_sums_of_slices_that_are_sorted_by_cluster(n_points, d, n):
+    """More blocks of sums than are resident: longer slices, taken cluster by cluster - past 256 points, with clusters that have no point
+    in a slice, and all points in one."""
+    _run(n_points, d, n, 3, 4, 11 + n, 3.0)
