@@ -355,8 +355,8 @@ template <int C, int SL> void launch_filter_t(const float *logits, int rows, int
     }
     for (int r = 0; r < rows; r += 65535) {
         const int n = rows - r < 65535 ? rows - r : 65535;
-        sampling::filtered_probs_kernel<C, SL><<<dim3(C, n), sampling::NT, sampling::probs_smem(V, C, SL), s>>>(
-            logits + (size_t)r * V, V, inv_t, top_p, probs + (size_t)r * V);
+        launch_chained(sampling::filtered_probs_kernel<C, SL>, dim3(C, n), dim3(sampling::NT), sampling::probs_smem(V, C, SL), s,
+                       logits + (size_t)r * V, V, inv_t, top_p, probs + (size_t)r * V);
     }
 }
 // From kWideFilterVocab ids on a row is cut into sixteen slices, whatever its company: its sums are the same.  A block has one of them where all
@@ -1378,14 +1378,14 @@ knnssd_status knnssd_decode_sampled(knnssd_ctx *c, int max_new, int k, float tem
             // draft step j: the draft model's logits of the row, filtered into q_j, the draft drawn from it
             run_pass(c, 1, c->chain + j, j, c->active_mask.data(), 0, c->target, false);
             launch_filter(c->logits, 1, g.vocab, inv_t, top_p, c->samp_q + (size_t)j * V, s);
-            sampling::sample_kernel<<<sampling::CL, sampling::NT, 0, s>>>(c->samp_q + (size_t)j * V, g.vocab, u + j, 0.f, c->chain + j + 1);
+            launch_chained(sampling::sample_kernel, dim3(sampling::CL), dim3(sampling::NT), 0, s, c->samp_q + (size_t)j * V, g.vocab, u + j, 0.f, c->chain + j + 1);
             c->launches += 2;
         }
         cudaEventRecord(c->ev1, s);
         run_pass(c, keff + 1, c->chain, 0, nullptr, 0, c->target, false);
         launch_filter(c->logits, keff + 1, g.vocab, inv_t, top_p, c->samp_p, s);
-        sampling::spec_accept_kernel<<<sampling::CL, sampling::NT, 0, s>>>(c->samp_p, c->samp_q, c->chain + 1, keff, g.vocab, u + k, u + 2 * k, 0.f,
-                                                                c->samp_res);
+        launch_chained(sampling::spec_accept_kernel<sampling::DeviceRound>, dim3(sampling::CL), dim3(sampling::NT), 0, s, c->samp_p, c->samp_q,
+                       sampling::DeviceRound{c->chain + 1, u + k, u + 2 * k}, keff, g.vocab, c->samp_res);
         sampling::commit_sampled_kernel<<<1, 32, 0, s>>>(c->chain, c->samp_res, c->state, c->out_tokens, g.max_seq, c->accept_log, round);
         c->launches += 3;
         cudaEventRecord(c->ev2, s);
@@ -1899,7 +1899,7 @@ knnssd_status knnssd_sample_token(const float *weights_dev, int vocab, float u, 
     cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
     int *tok = host_words();
     if (!tok) return KNNSSD_ERR_CUDA;
-    sampling::sample_kernel<<<sampling::CL, sampling::NT, 0, s>>>(weights_dev, vocab, nullptr, u, tok);
+    launch_chained(sampling::sample_kernel, dim3(sampling::CL), dim3(sampling::NT), 0, s, weights_dev, vocab, nullptr, u, tok);
     cudaError_t e = cudaStreamSynchronize(s);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return KNNSSD_ERR_CUDA;
@@ -1916,12 +1916,13 @@ knnssd_status knnssd_spec_accept(const float *p_dev, const float *q_dev, const i
         if (drafts_host[j] < 0 || drafts_host[j] >= vocab || !(u_accept_host[j] >= 0.f) || !(u_accept_host[j] < 1.f))
             return KNNSSD_ERR_INVALID_ARG;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
-    int *buf = host_words();                  // [0..1] result, [2 .. 2 + k) drafts, then k floats of uniforms
+    int *buf = host_words();                  // [0..1] result
     if (!buf) return KNNSSD_ERR_CUDA;
-    static_assert(2 + 2 * kMaxRows <= kHostWords, "the round's words");
-    float *u_pinned = reinterpret_cast<float *>(buf + 2 + kMaxRows);
-    for (int j = 0; j < k; ++j) { buf[2 + j] = drafts_host[j]; u_pinned[j] = u_accept_host[j]; }
-    sampling::spec_accept_kernel<<<sampling::CL, sampling::NT, 0, s>>>(p_dev, q_dev, buf + 2, k, vocab, u_pinned, nullptr, u_final, buf);
+    sampling::GivenRound round{};
+    static_assert(kMaxRows <= 16, "a round's drafts go with its launch");
+    for (int j = 0; j < k; ++j) { round.drafts[j] = drafts_host[j]; round.u_accept[j] = u_accept_host[j]; }
+    round.u_final = u_final;
+    launch_chained(sampling::spec_accept_kernel<sampling::GivenRound>, dim3(sampling::CL), dim3(sampling::NT), 0, s, p_dev, q_dev, round, k, vocab, buf);
     cudaError_t e = cudaStreamSynchronize(s);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return KNNSSD_ERR_CUDA;

@@ -12,6 +12,7 @@
 // sixteen: a few passes over values that stay in shared memory, bound by the meetings between the passes (~1.5 us each: block, then
 // cluster).  Every sum has a fixed order, which the row's length alone decides.
 #pragma once
+#include <climits>
 #include <cooperative_groups.h>
 
 #include "kernels.cuh"
@@ -81,13 +82,14 @@ __device__ __forceinline__ float join(M &sh, int &turn) {
             cluster.map_shared_rank(&sh, lane % NW)->slot[par][cluster.block_rank() * SL + slice][MAX ? 0 : warp * PW + lane / NW] = t0;
     }
     cluster.sync();
-    float t = sh.slot[par][0][MAX ? 0 : lane];
+    float t[CL * SL];
 #pragma unroll
-    for (int r = 1; r < CL * SL; ++r) {
-        const float o = sh.slot[par][r][MAX ? 0 : lane];
-        t = MAX ? fmaxf(t, o) : t + o;
-    }
-    return t;
+    for (int r = 0; r < CL * SL; ++r) t[r] = sh.slot[par][r][MAX ? 0 : lane];
+#pragma unroll
+    for (int h = CL * SL / 2; h >= 1; h >>= 1)                   // by halves: fewer roundings than one after the other
+#pragma unroll
+        for (int r = 0; r < h; ++r) t[r] = MAX ? fmaxf(t[r], t[r + h]) : t[r] + t[r + h];
+    return t[0];
 }
 template <bool MAX, typename M>
 __device__ __forceinline__ float meet(M &sh, int &turn, float (&v)[NS]) {
@@ -137,12 +139,16 @@ template <int U, typename F> __device__ __forceinline__ void each_entry(const fl
 // that re-read its row from L2 each time, took 65 us for 5 rows of 32000 and 241 us for one of 152064; this takes 15 and 21).  The first pass leaves
 // a few per cent of the values between its bounds; a thread keeps those of its own aside for the others.  Once no block has more than
 // GATHER values left between the bounds all blocks get them all, and each finds x0 for itself: a meeting instead of five.
-// Tokens whose probability equals x0 are ranked by id.
+// Tokens whose probability equals x0 are ranked by id.  The sum of the row comes with the first pass, what is kept is scaled once at the end:
+// 5 rows of 32000 and their 4 filtered after them, with the keep-or-resample round behind: 64 us a call for 54 (kernels set up under the
+// end of the one before), 9 + 8 of 152064 165 for 136; one of 152064 and a draw 52 for 48.  Error against 64 bits, rms over 2200 rows: 8.1e-8 so far,
+// 7.0e-8 so.
 // A row is cut into C SL slices; what comes out depends on their number, not on how many blocks share them.
 // grid = (C, rows), NT threads, probs_smem(V, C, SL) of shared memory; rows too long for it keep their values in `probs`.
 constexpr int GATHER = 32;
 template <int C, int SL> __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(NT)
 filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_temperature, float top_p, float *__restrict__ probs) {
+    chain_wait();
     constexpr int SLICES = C * SL;
     static_assert(SLICES <= NS, "a sum per slice");
     extern __shared__ float probs_slice[];
@@ -182,33 +188,26 @@ filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_tempera
 #pragma unroll
     for (int k = 0; k < SL; ++k) bring<true>(sh, k, v);
     m = join<true>(sh, turn);
-#pragma unroll
-    for (int k = 0; k < SL; ++k) {
-#pragma unroll
-        for (int j = 0; j < NS; ++j) v[j] = 0.f;
-        float *to = p[k];
-        each_entry<4>(to, n[k], [&](int i, float x) {
-            const float e = expf((x - m) * inv_temperature);
-            to[i] = e;
-            v[0] += e;
-        });
-        bring<false>(sh, k, v);
-    }
-    const float s = __shfl_sync(0xffffffffu, join<false>(sh, turn), 0);
+    // From here on the values are e = exp((x - max) / temperature), softmax before its division by the sum, which the first pass brings along:
+    // a token's mass is compared with top_p times that sum.  (A pass of its own over the row for the sum and one for the division cost a
+    // meeting and 2 us.)  The largest value is 1, nothing lies above it.  Below (1 - top_p) / (2 V) there is less than half of 1 - top_p of the
+    // mass, which is at least 1, so what lies above that is not below top_p of it: a sum of V terms is not off by the other half
+    // unless top_p is 1 to four digits.
 #pragma unroll
     for (int k = 0; k < SL; ++k) {
         float *to = p[k];
-        each_entry<4>(to, n[k], [&](int i, float x) { to[i] = x / s; });
+        each_entry<4>(to, n[k], [&](int i, float x) { to[i] = expf((x - m) * inv_temperature); });
     }
-    // smallest x (as a bit pattern) in [lo, hi] with mass above x < top_p.  The largest probability is 1 / s (its exponent
-    // is zero), nothing lies above it.  Below (1 - top_p) / (2 V) there is less than half of 1 - top_p in all, so the mass above
-    // that is not below top_p: a sum of V terms is not off by the other half unless top_p is 1 to four digits.
-    unsigned lo = 0u, hi = __float_as_uint(fmaxf(0.f, 1.0f / s));
+    unsigned lo = 0u, hi = __float_as_uint(1.0f);
     if (1.0f - top_p > 1e-4f) lo = min(hi, __float_as_uint(0.5f * (1.0f - top_p) / (float)V));
-    float above_hi = 0.f;                                        // all threads' values above hi
+    // The largest value, 1, is counted and not added: the sums are of what lies below it, so that they are not rounded at its size.
+    float ones = 0.f, kept_mass = 0.f, kept_rest = 0.f;          // how often it occurs; top_p times the whole sum, and what that leaves for the rest
+    auto small = [](float y) { return y == 1.f ? 0.f : y; };
+    float above_hi = 0.f;                                        // the rest of all threads' values above hi
     int gathered = -1;                                           // values between the bounds, once all blocks have them
     for (bool first = true; first || hi > lo + 1u; first = false) {
-        const unsigned step = (hi - lo + NS - 1) / NS;           // candidates lo, lo + step, ..: lo itself only counts in the first pass
+        const int nc = first ? NS - 2 : NS;                      // candidates lo, lo + step, ..: lo itself only counts in the first pass, whose last
+        const unsigned step = (hi - lo + nc - 1) / nc;           // sums are the row's ones and the rest of it
         float x[NS];
 #pragma unroll
         for (int j = 0; j < NS; ++j) x[j] = __uint_as_float(min(hi, lo + j * step));
@@ -218,8 +217,16 @@ filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_tempera
 #pragma unroll
             for (int j = 0; j < NS; ++j) v[j] = above[k];
             auto count = [&](float y) {
+                const float r = small(y);
 #pragma unroll
-                for (int j = 0; j < NS; ++j) v[j] += y > x[j] ? y : 0.f;
+                for (int j = 0; j < NS - 2; ++j) v[j] += y > x[j] ? r : 0.f;
+                if (first) {
+                    v[NS - 2] += y == 1.f ? 1.f : 0.f;
+                    v[NS - 1] += r;
+                } else {
+                    v[NS - 2] += y > x[NS - 2] ? r : 0.f;
+                    v[NS - 1] += y > x[NS - 1] ? r : 0.f;
+                }
             };
             if (listed) {                                        // hardly any thread has more than one left
 #pragma unroll 1
@@ -230,14 +237,21 @@ filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_tempera
             bring<false>(sh, k, v);
         }
         const float mass = join<false>(sh, turn);
-        const unsigned below = __ballot_sync(0xffffffffu, mass < top_p);
-        int j = below ? __ffs(below) - 1 : NS;                   // the first candidate with less than top_p above it
+        if (first) {
+            const float rest = __shfl_sync(0xffffffffu, mass, NS - 1);
+            if (!(rest == rest)) { hi = lo = __float_as_uint(2.0f); break; }     // a NaN in the row: nothing is kept of it
+            ones = __shfl_sync(0xffffffffu, mass, NS - 2);
+            kept_mass = fmaf(top_p, rest, top_p * ones);
+            kept_rest = fmaf(top_p, rest, (top_p - 1.0f) * ones);
+        }
+        const unsigned below = __ballot_sync(0xffffffffu, mass < kept_rest) & (first ? 0x3fffffffu : 0xffffffffu);
+        int j = below ? __ffs(below) - 1 : nc;                   // the first candidate with less than top_p above it
         if (j == 0) {
             if (first) { hi = lo; above_hi = __shfl_sync(0xffffffffu, mass, 0); break; }
             j = 1;                                               // lo was ruled out before, by sums in another order
         }
-        if (j < NS && lo + j * step < hi) above_hi = __shfl_sync(0xffffffffu, mass, j);
-        const unsigned nhi = j < NS ? min(hi, lo + j * step) : hi;
+        if (j < nc && lo + j * step < hi) above_hi = __shfl_sync(0xffffffffu, mass, j);
+        const unsigned nhi = j < nc ? min(hi, lo + j * step) : hi;
         lo = min(hi, lo + (j - 1) * step);
         hi = nhi;
         const float xl = __uint_as_float(lo), xh = __uint_as_float(hi);
@@ -245,7 +259,7 @@ filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_tempera
 #pragma unroll
             for (int k = 0; k < SL; ++k)
                 each_entry<4>(p[k], n[k], [&](int, float y) {
-                    if (y > xh) above[k] += y;
+                    if (y > xh) above[k] += small(y);
                     else if (y > xl) list(k)[NT * n_list[k]++] = y;
                 });
         } else if (keeps_list && hi > lo + 1u) {
@@ -291,7 +305,7 @@ filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_tempera
         }
     }
     float x0 = __uint_as_float(hi);
-    float a0 = above_hi;                                         // mass above x0
+    float a0 = above_hi;                                         // the rest's mass above x0
     int c = 0, own_c[SL];                                        // tokens at x0: of all slices, and this thread's share of its block's
 #pragma unroll
     for (int k = 0; k < SL; ++k) own_c[k] = 0;
@@ -305,8 +319,8 @@ filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_tempera
                 const float y = left[r][i];
                 float m_above = 0.f;                             // the few small values by themselves, then one rounding at the size of the mass
                 for (int q = 0; q < SLICES; ++q)
-                    for (int e = 0, n_q = n_left[q]; e < n_q; ++e) { const float o = left[q][e]; m_above += o > y ? o : 0.f; }
-                if (above_hi + m_above < top_p) atomicMin(&s_x0, __float_as_uint(y));
+                    for (int e = 0, n_q = n_left[q]; e < n_q; ++e) { const float o = left[q][e]; m_above += o > y ? small(o) : 0.f; }
+                if (y == 1.f || above_hi + m_above < kept_rest) atomicMin(&s_x0, __float_as_uint(y));
             }
         }
         __syncthreads();
@@ -315,7 +329,7 @@ filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_tempera
         for (int q = 0; q < SLICES; ++q)
             for (int e = 0, n_q = n_left[q]; e < n_q; ++e) {
                 const float o = left[q][e];
-                left_above += o > x0 ? o : 0.f;
+                left_above += o > x0 ? small(o) : 0.f;
                 if (o == x0) {
                     ++c;
 #pragma unroll
@@ -330,7 +344,7 @@ filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_tempera
 #pragma unroll
             for (int j = 0; j < NS; ++j) v[j] = 0.f;
             each_entry<4>(p[k], n[k], [&](int, float y) {
-                v[0] += y > x0 ? y : 0.f;
+                v[0] += y > x0 ? small(y) : 0.f;
                 if (y == x0) v[1] += 1.f;                        // counts are exact up to 2^24 tokens
             });
             own_c[k] = (int)v[1];
@@ -340,11 +354,14 @@ filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_tempera
         a0 = __shfl_sync(0xffffffffu, tot, 0);
         c = (int)__shfl_sync(0xffffffffu, tot, 1);
     }
-    // tokens at exactly x0: the n-th of them by id (n = 0, 1, ..) is kept iff mass above x0 + n x0 < top_p
+    const bool at_top = x0 == 1.f;                               // the largest value's tokens are the last ones kept
+    if (at_top) a0 = 0.f;
+    const float enough = at_top ? kept_mass : kept_rest;
+    // tokens at exactly x0: the n-th of them by id (n = 0, 1, ..) is kept iff mass above x0 + n x0 < top_p of it all
     int nk = 1, id_cut = V;                                      // tokens at x0 with id < id_cut are kept; the first one always is
     if (c > 1) {
         nk = 0;
-        for (int i = tid; i < c; i += NT) nk += (a0 + (float)i * x0 < top_p) ? 1 : 0;
+        for (int i = tid; i < c; i += NT) nk += (a0 + (float)i * x0 < enough) ? 1 : 0;
         nk = max(1, block_count(nk, shi[0]));
         if (nk < c) {                                            // which of them: the slice that has the nk-th is searched for its id
             // sum r of this meeting: the tokens at x0 in slice r
@@ -379,24 +396,27 @@ filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_tempera
             id_cut = s_cut;
         }
     }
-    const float z = a0 + (float)min(nk, c) * x0;
+    // one over what is kept in all, in two floats: a product with both is rounded once (and costs less than a division)
+    const double per_z = 1.0 / ((at_top ? 0.0 : (double)ones) + (double)a0 + (double)min(nk, c) * (double)x0);
+    const float z_hi = (float)per_z, z_lo = (float)(per_z - (double)z_hi);
 #pragma unroll
     for (int k = 0; k < SL; ++k) {
         float *out = probs + (size_t)blockIdx.y * V + id0[k];
-        each_entry<4>(p[k], n[k], [&](int i, float y) { out[i] = (y > x0 || (y == x0 && id0[k] + i < id_cut)) ? y / z : 0.f; });
+        each_entry<4>(p[k], n[k], [&](int i, float y) { out[i] = (y > x0 || (y == x0 && id0[k] + i < id_cut)) ? fmaf(y, z_hi, y * z_lo) : 0.f; });
     }
     cluster.sync();                                              // nobody leaves while its shared memory may still be written to
 }
 
 // Inverse CDF in token-id order: the smallest id x with w_0 + .. + w_x > u * sum(w); w_i = a_i (b == nullptr) or
 // max(a_i - b_i, 0), falling back to a if that is zero everywhere.  Called by all threads of a cluster; block r has the ids
-// [r S, (r + 1) S), its warp w a contiguous run of them, read 32 at a time; the warp whose run holds the crossing walks it
-// again with a running sum.  Block 0's thread 0 returns the token (-1: no weight anywhere).
-// One block with a run of ids per thread and a serial scan of 1024 sums took 41 us for 152064 ids, this takes 8.5.
+// [r S, (r + 1) S), its warp w a contiguous run of them, read 32 at a time; the block whose ids hold the crossing walks the run of the warp
+// that does with all its threads.  Block 0's thread 0 returns the token (-1: no weight anywhere).
+// (One block with a run of ids per thread and a serial scan of 1024 sums took 41 us for 152064 ids, the run walked by its own warp 8.5.)
 struct Draw {
     Meet m;
-    float warp_sum[NW];
+    float warp_sum[NW], tot[4 * NW];
     int last[CL];
+    int first, seen;                                             // of the ids that the block walks: where the sum crosses, the last with weight
     int token;
 };
 __device__ __forceinline__ int cluster_sample(const float *__restrict__ a, const float *__restrict__ b, int V, float u, Draw &sh) {
@@ -447,42 +467,55 @@ __device__ __forceinline__ int cluster_sample(const float *__restrict__ a, const
         }
         if (use_b && !(total > 0.f)) { use_b = false; continue; }
         const float target = u * total;
-        // runs of this block up to and including this warp's (the last warp ends where the block does)
-        float excl = before;
-        for (int k = 0; k < warp; ++k) excl += sh.warp_sum[k];
-        const float incl = warp == NW - 1 ? through : excl + sh.warp_sum[warp];
-        if (before <= target && through > target && excl <= target && incl > target) {
-            float acc = excl;
-            int tok = -1, pos = -1;                              // pos: the last id with weight, if rounding hides the crossing
-            constexpr int B = 8;                                 // ids in flight: 8 x 32
-            for (int ib = i0; ib < i1 && tok < 0; ib += 32 * B) {
-                float xs[B];
+        if (before <= target && through > target) {              // uniform: the crossing is in this block
+            // the warp whose run holds it (the last one ends where the block does); the whole block walks that run, 4 NT ids at a time
+            int w = 0;
+            float excl = before;
+            while (w < NW - 1 && !(excl + sh.warp_sum[w] > target)) excl += sh.warp_sum[w++];
+            const int j0 = min(lim, rank * S + w * run), j1 = min(lim, j0 + run);
+            if (tid == 0) { sh.first = INT_MAX; sh.seen = -1; }
+            __syncthreads();
+            int tok = -1;
+            for (int jb = j0; jb < j1 && tok < 0; jb += 4 * NT) {
+                float x[4], sc[4];
 #pragma unroll
-                for (int e = 0; e < B; ++e) xs[e] = ib + 32 * e + lane < i1 ? weight(ib + 32 * e + lane) : 0.f;
+                for (int e = 0; e < 4; ++e) { const int i = jb + e * NT + tid; x[e] = i < j1 ? weight(i) : 0.f; }
 #pragma unroll
-                for (int e = 0; e < B; ++e) {
-                    const float x = xs[e];
-                    float sc = x;
+                for (int e = 0; e < 4; ++e) {
+                    sc[e] = x[e];
 #pragma unroll
                     for (int o = 1; o < 32; o <<= 1) {
-                        const float t = __shfl_up_sync(0xffffffffu, sc, o);
-                        if (lane >= o) sc += t;
+                        const float t = __shfl_up_sync(0xffffffffu, sc[e], o);
+                        if (lane >= o) sc[e] += t;
                     }
-                    const unsigned over = __ballot_sync(0xffffffffu, x > 0.f && acc + sc > target), has = __ballot_sync(0xffffffffu, x > 0.f);
-                    if (over && tok < 0) tok = ib + 32 * e + __ffs(over) - 1;
-                    if (has) pos = ib + 32 * e + 31 - __clz(has);
-                    acc += __shfl_sync(0xffffffffu, sc, 31);
+                    if (lane == 31) sh.tot[e * NW + warp] = sc[e];
                 }
-            }
-            if (tok < 0) tok = pos;
-            if (tok < 0) {
-                // the last warp, without weight of its own: the block's sum, added at once, ends an ulp past the running sum of its
-                // warps, and the target lies between.  The crossing is in this block all the same: its last id with weight
-                tok = lane < NW ? __float_as_int(sh.m.red[0][lane][NS]) : -1;
+                __syncthreads();
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) tok = max(tok, __shfl_xor_sync(0xffffffffu, tok, o));
+                for (int e = 0; e < 4; ++e) {
+                    if (jb + e * NT >= j1) break;                // uniform
+                    float acc = excl;                            // before this thread's warp, and before the next NT ids
+#pragma unroll
+                    for (int k = 0; k < NW; ++k) {
+                        const float t = sh.tot[e * NW + k];
+                        if (k < warp) acc += t;
+                        excl += t;
+                    }
+                    const int i = jb + e * NT + tid;
+                    if (x[e] > 0.f) {
+                        if (acc + sc[e] > target) atomicMin(&sh.first, i);
+                        atomicMax(&sh.seen, i);
+                    }
+                }
+                __syncthreads();
+                if (sh.first != INT_MAX) tok = sh.first;
             }
-            if (lane == 0 && tok >= 0) atomicMax(&cluster.map_shared_rank(&sh, 0)->token, tok);
+            if (tok < 0) tok = sh.seen;                          // the last id with weight, if rounding hides the crossing
+            // no weight in the run: the block's sum, added at once, ends an ulp past the running sum of its warps, and the target lies between.
+            // The crossing is in this block all the same: its last id with weight
+            if (tok < 0)
+                for (int k = 0; k < NW; ++k) tok = max(tok, __float_as_int(sh.m.red[0][k][NS]));
+            if (tid == 0 && tok >= 0) atomicMax(&cluster.map_shared_rank(&sh, 0)->token, tok);
         }
         break;
     }
@@ -496,26 +529,43 @@ __device__ __forceinline__ int cluster_sample(const float *__restrict__ a, const
 // token <- draw from weights w[V] with the uniform *u_ptr (u_val if u_ptr is null).  One cluster.
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT)
 sample_kernel(const float *__restrict__ w, int V, const float *__restrict__ u_ptr, float u_val, int *__restrict__ token) {
+    chain_wait();
     __shared__ Draw sh;
     const int tok = cluster_sample(w, nullptr, V, u_ptr ? *u_ptr : u_val, sh);
     if (threadIdx.x == 0 && blockIdx.x == 0) *token = tok < 0 ? 0 : tok;
 }
 
-// One verification round of speculative sampling.  p [k+1][V], q [k][V] filtered distributions, drafts [k] (device),
-// u_accept [k] (device), u_final (*u_final_ptr if given).  out[0] = number of drafts kept, out[1] = the token emitted
-// after them.  One cluster.
+// The drafts of a round and their uniforms: on the device, or with the launch (read from pinned host memory they were a trip across the bus).
+struct DeviceRound {
+    const int *drafts;
+    const float *u_accept, *u_final;
+    __device__ __forceinline__ int draft(int j) const { return drafts[j]; }
+    __device__ __forceinline__ float accept(int j) const { return u_accept[j]; }
+    __device__ __forceinline__ float last() const { return *u_final; }
+};
+struct GivenRound {
+    int drafts[16];
+    float u_accept[16], u_final;
+    __device__ __forceinline__ int draft(int j) const { return drafts[j]; }
+    __device__ __forceinline__ float accept(int j) const { return u_accept[j]; }
+    __device__ __forceinline__ float last() const { return u_final; }
+};
+
+// One verification round of speculative sampling.  p [k+1][V], q [k][V] filtered distributions, k <= 16.  out[0] = number of drafts kept,
+// out[1] = the token emitted after them.  One cluster.
+template <typename Round>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT)
-spec_accept_kernel(const float *__restrict__ p, const float *__restrict__ q, const int *__restrict__ drafts, int k, int V,
-                   const float *__restrict__ u_accept, const float *__restrict__ u_final_ptr, float u_final, int *__restrict__ out) {
+spec_accept_kernel(const float *__restrict__ p, const float *__restrict__ q, const __grid_constant__ Round round, int k, int V, int *__restrict__ out) {
+    chain_wait();
     __shared__ Draw sh;
-    if (u_final_ptr) u_final = *u_final_ptr;
+    const float u_final = round.last();
     // every warp tests all drafts, one per lane: the first that is not kept ends the round
     const int lane = threadIdx.x & 31;
     bool keep = false;
     if (lane < k) {
-        const int d = drafts[lane];
+        const int d = round.draft(lane);
         // a token outside the vocabulary is never kept
-        keep = d >= 0 && d < V && u_accept[lane] * q[(size_t)lane * V + d] < p[(size_t)lane * V + d];
+        keep = d >= 0 && d < V && round.accept(lane) * q[(size_t)lane * V + d] < p[(size_t)lane * V + d];
     }
     const unsigned lost = ~__ballot_sync(0xffffffffu, keep) & ((1u << k) - 1u);
     const int j = lost ? __ffs(lost) - 1 : k;

@@ -97,3 +97,31 @@ def test_a_draw_between_two_roundings_stays_in_its_block():
     assert us
     for u in us:
         assert kb.knnssd_sample_token(w.cuda(), float(u)) in (64, 68)
+
+
+@pytest.mark.parametrize("V", [9, 4100, 70000])
+@pytest.mark.parametrize("top,top_p", [(1, 0.3), (1, 0.999), (3, 0.3), (3, 0.6), (3, 0.95), (3, 2.0)])
+def test_largest_values_alone_among_equals_and_beside_others(kb, V, top, top_p):
+    """The largest value is counted apart from the sums: the cut falls on it, among its equals, and past them."""
+    g = torch.Generator().manual_seed(V + top)
+    l = torch.randn(2, V, generator=g).clamp_(max=2.0) - 6.0
+    at = torch.randperm(V, generator=g)[:top]
+    l[:, at] = 7.0
+    l[1, 0] = float("nan")
+    got = kb.knnssd_filtered_probs(l.cuda(), 1.0, top_p).cpu().numpy().astype(np.float64)
+    want = orc.filtered_distribution(l[0].numpy(), 1.0, top_p)
+    edge = (got[0] > 0) != (want > 0)
+    assert (got[0] + want)[edge].sum() < 4e-6 and np.abs(got[0] - want).max() < 2e-6
+    assert not got[1].any()                                            # a NaN in the row: nothing is kept of it
+
+
+@pytest.mark.parametrize("V", [8 * 16 * 2048, 8 * 16 * 2048 + 1, 600001])
+def test_draws_from_runs_of_several_steps(kb, V):
+    """A warp's run of more ids than the block walks at once: every draw against the exact cumulative sum."""
+    w = torch.rand(V, generator=torch.Generator().manual_seed(3)).cuda()
+    cdf = w.double().cumsum(0)
+    for u in np.linspace(0.0005, 0.9995, 40).astype(np.float32):
+        x = kb.knnssd_sample_token(w, float(u))
+        t = float(u) * float(cdf[-1])
+        # 32-bit partial sums: a few ulps of the total
+        assert float(cdf[x]) > t * (1 - 2e-6) and (x == 0 or float(cdf[x - 1]) <= t * (1 + 2e-6))
