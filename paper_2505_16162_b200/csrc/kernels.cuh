@@ -34,6 +34,14 @@ void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cu
     cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// The GPU's nanosecond timer.  Calls that return a device time have it stamped by their first and their last kernel, into pinned words: two
+// events and their difference took 7.3 us of a call, next to 9.3 for a launch and the wait for it.
+__device__ __forceinline__ unsigned long long globaltimer_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+    return t;
+}
+
 // Codes a kernel may leave in the device error word (besides the codes of bounded waits that gave up, all < 100).
 enum { ERR_BAD_TOKEN = 101, ERR_BAD_LOGITS = 102 };
 
@@ -126,9 +134,10 @@ __device__ __forceinline__ float warp_max(float v) {
 template <typename WT>
 __global__ void embed_rope_kernel(const WT *__restrict__ E, const int *__restrict__ tok, int d, float *__restrict__ x,
                                   const DeviceState *__restrict__ st, int pos_off, const double *__restrict__ inv_freq,
-                                  int half, float2 *__restrict__ cs, int vocab, int *__restrict__ err) {
+                                  int half, float2 *__restrict__ cs, int vocab, int *__restrict__ err, unsigned long long *stamp) {
     chain_wait();
     const int m = blockIdx.x;
+    if (stamp && m == 0 && threadIdx.x == 0) *stamp = globaltimer_ns();
     int t = tok[m];
     if (t < 0 || t >= vocab) {                 // never gather outside the table: report and read row 0 instead
         if (threadIdx.x == 0) atomicExch(err, ERR_BAD_TOKEN);
@@ -584,6 +593,7 @@ struct Delivery {
     int n_words;
     const int *err;
     int *host, *host_err;        // pinned
+    unsigned long long *stamp;   // pinned: when the call's last pass was done
     // ACCEPT
     int *chain;
     const int *target;
@@ -597,7 +607,7 @@ template <bool ACCEPT> __global__ void __launch_bounds__(256) deliver_kernel(con
         if (ACCEPT && threadIdx.x == 0) accept_rows(a.chain, a.target, a.k, a.st, a.out_tokens, a.out_cap, a.accept_log, a.round_idx);
         __syncwarp();
         for (int i = threadIdx.x; i < a.n_words; i += 32) a.host[i] = *reinterpret_cast<const volatile int *>(a.words + i);
-        if (threadIdx.x == 0) *a.host_err = *a.err;
+        if (threadIdx.x == 0) { *a.host_err = *a.err; *a.stamp = globaltimer_ns(); }
     }
     const size_t first = (size_t)blockIdx.x * 256 + threadIdx.x, stride = (size_t)gridDim.x * 256;
 #pragma unroll
@@ -615,6 +625,7 @@ template <bool ACCEPT> __global__ void __launch_bounds__(256) deliver_kernel(con
 // Up to 16 token ids, by value, into the session's chain.
 struct Tokens { int id[16]; };
 __global__ void put_tokens_kernel(const Tokens t, int n, int *__restrict__ chain) {
+    chain_wait();
     if (threadIdx.x < n) chain[threadIdx.x] = t.id[threadIdx.x];
 }
 
@@ -630,7 +641,9 @@ __global__ void put_tokens_kernel(const Tokens t, int n, int *__restrict__ chain
 // after the other (WARPS): the sums are the same.  A call of 4096 x 640 / 20000 x 640 / 100000 x 64 / 100000 x 1024: a block per anchor 35 / 61 /
 // 191 / 237 us, so 31 / 43 / 79 / 139.  grid = n, or ceil(n / 8) of WARPS, 256 threads.
 template <bool WARPS> __global__ void __launch_bounds__(256) cosine_top1_kernel(const float *__restrict__ v, const float *__restrict__ anchors, int n, int d,
-                                                          float *__restrict__ cosines, int *__restrict__ work, int *__restrict__ out) {
+                                                          float *__restrict__ cosines, int *__restrict__ work, int *__restrict__ out,
+                                                          unsigned long long *__restrict__ stamps) {
+    if (stamps && blockIdx.x == 0 && threadIdx.x == 0) stamps[0] = globaltimer_ns();
     __shared__ float s_v[8];
     __shared__ int s_i[8];
     __shared__ float s_sum[3][8];
@@ -723,14 +736,17 @@ template <bool WARPS> __global__ void __launch_bounds__(256) cosine_top1_kernel(
         out[0] = bi;
         out[1] = __float_as_int(bv);
         out[2] = bad;
+        if (stamps) stamps[1] = globaltimer_ns();
         work[0] = 0;
     }
 }
 
-inline void launch_cosine_top1(const float *v, const float *anchors, int n, int d, int n_sms, float *cosines, int *work, int *out, cudaStream_t s) {
+// stamps: if given, when the first block began and the last one was done.
+inline void launch_cosine_top1(const float *v, const float *anchors, int n, int d, int n_sms, float *cosines, int *work, int *out, cudaStream_t s,
+                               unsigned long long *stamps = nullptr) {
     const bool vec = ((reinterpret_cast<uintptr_t>(v) | reinterpret_cast<uintptr_t>(anchors)) & 15u) == 0 && d % 4 == 0;
-    if (n <= 8 * n_sms || (vec ? d / 4 : d) > 256) cosine_top1_kernel<false><<<n, 256, 0, s>>>(v, anchors, n, d, cosines, work, out);
-    else cosine_top1_kernel<true><<<(n + 7) / 8, 256, 0, s>>>(v, anchors, n, d, cosines, work, out);
+    if (n <= 8 * n_sms || (vec ? d / 4 : d) > 256) cosine_top1_kernel<false><<<n, 256, 0, s>>>(v, anchors, n, d, cosines, work, out, stamps);
+    else cosine_top1_kernel<true><<<(n + 7) / 8, 256, 0, s>>>(v, anchors, n, d, cosines, work, out, stamps);
 }
 
 // flag <- 1 if an anchor's norm is zero or not finite.
@@ -744,15 +760,17 @@ __global__ void anchor_norm_check_kernel(const float *__restrict__ anchors, int 
 }
 
 // One word of the session's state, in stream order.
-__global__ void set_word_kernel(int *word, int value) { *word = value; }
+__global__ void set_word_kernel(int *word, int value) { chain_wait(); *word = value; }
 
-__global__ void set_state_kernel(DeviceState *st, int len, int produced) {
+__global__ void set_state_kernel(DeviceState *st, int len, int produced, unsigned long long *stamp) {
+    if (stamp) *stamp = globaltimer_ns();
     st->len = len; st->produced = produced; st->last_accept = 0; st->last_next = -1;
 }
-// The first token of a generation; where `host` (pinned) is given the host gets it there, and the error word behind it.
-__global__ void emit_first_token_kernel(const int *chain, DeviceState *st, int *out_tokens, int len, const int *err, int *host, int *host_err) {
+// The first token of a generation; where `host` (pinned) is given the host gets it there, the error word behind it, and when that was.
+__global__ void emit_first_token_kernel(const int *chain, DeviceState *st, int *out_tokens, int len, const int *err, int *host, int *host_err,
+                                        unsigned long long *stamp) {
     out_tokens[0] = chain[0]; st->produced = 1; st->len = len;
-    if (host) { *host = chain[0]; *host_err = *err; }
+    if (host) { *host = chain[0]; *host_err = *err; *stamp = globaltimer_ns(); }
 }
 
 }  // namespace knnssd

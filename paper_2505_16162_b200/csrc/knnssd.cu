@@ -67,6 +67,7 @@ struct knnssd_ctx {
     int len = 0, pending = -1;
     knnssd_stats stats{};
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr;
+    bool stamp_pass = false;       // the next pass leaves the time it began in the pinned words
     std::string err;
 
     // persistent pass kernel (bf16 models whose widths are multiples of 128)
@@ -482,6 +483,20 @@ template <int HD, int NB, int NP> cudaError_t launch_pass_t(knnssd_ctx *c, const
                                        dim3(stream::NTHREADS), args, stream::SMEM_BYTES, c->stream);
 }
 
+// Device times of a call, in pinned words that are 8-byte aligned: when it began and when it was done.
+constexpr int kStampWord = 40;
+unsigned long long *stamps_of(knnssd_ctx *c) { return reinterpret_cast<unsigned long long *>(c->pinned + kStampWord); }
+float stamped_ms(knnssd_ctx *c) {
+    const unsigned long long *t = stamps_of(c);
+    return t[1] > t[0] ? (float)((double)(t[1] - t[0]) * 1e-6) : 0.f;
+}
+// Where the pass that is being enqueued stamps its begin: once after stamp_pass was set, else nowhere.
+unsigned long long *pass_stamp(knnssd_ctx *c) {
+    unsigned long long *at = c->stamp_pass ? stamps_of(c) : nullptr;
+    c->stamp_pass = false;
+    return at;
+}
+
 // One pass through the persistent kernel.  Errors surface at the caller's next synchronisation.
 void run_pass_mega(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const unsigned char *mask, int head_row0,
                    int *argmax_out, bool want_hidden, int out_row0 = 0) {
@@ -502,6 +517,7 @@ void run_pass_mega(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const 
     pr.M = M; pr.tok = tok_dev; pr.pos_off = pos_off; pr.head_row0 = head_row0; pr.argmax_out = argmax_out;
     pr.want_hidden = want_hidden ? 1 : 0;
     pr.out_row0 = out_row0;
+    pr.stamp = pass_stamp(c);
     pr.bar_spin_limit = c->bar_spin_limit;
     pr.bar_base = c->bar_total;
     pr.merge_op = pass::merge_rows_separately(M, c->cfg.n_heads / c->cfg.n_kv_heads) ? 1 : 0;
@@ -556,7 +572,7 @@ void run_pass_t(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const uns
     const int nq = H * hd, nkv = Hkv * hd;
     cudaStream_t s = c->stream;
     launch_chained(embed_rope_kernel<WT>, dim3(M), dim3(256), 0, s, reinterpret_cast<const WT *>(c->tok_embed), tok_dev, d, c->x, c->state, pos_off,
-                                            c->inv_freq, hd / 2, c->rope_cs, g.vocab, c->err_word);
+                                            c->inv_freq, hd / 2, c->rope_cs, g.vocab, c->err_word, pass_stamp(c));
     c->launches++;
     const size_t layer_stride = (size_t)Hkv * g.max_seq * hd;
     for (int l = 0; l < g.n_layers; ++l) {
@@ -636,7 +652,7 @@ void run_pass_small(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const
     a.eps = g.rms_eps; a.st = c->state; a.tok = tok_dev; a.M = M; a.pos_off = pos_off; a.head_row0 = head_row0; a.want_hidden = want_hidden ? 1 : 0;
     a.argmax_out = argmax_out; a.inv_freq = c->inv_freq; a.x = c->x; a.qkv = c->qkv; a.attn = c->attn; a.act = c->act; a.logits = c->logits;
     a.hfinal = c->hfinal; a.part_o = c->part_o; a.part_ml = c->part_ml; a.rope_cs = c->rope_cs; a.n_splits = c->n_splits; a.kc = c->kcache; a.vc = c->vcache;
-    a.err = c->err_word;
+    a.err = c->err_word; a.stamp = pass_stamp(c);
     for (int j = 0; mask && j < 2 * g.n_layers; ++j)
         if (mask[j]) a.skip[j >> 5] |= 1u << (j & 31);
     const bool head_apart = head_row0 < M && g.vocab > kSmallHeadIds;
@@ -709,7 +725,7 @@ knnssd_status refuse_capture(knnssd_ctx *c, const char *what) {
 knnssd_status set_word(knnssd_ctx *c, int *word, int value, const char *what) {
     const knnssd_status st = refuse_capture(c, what);
     if (st != KNNSSD_OK) return st;
-    set_word_kernel<<<1, 1, 0, c->stream>>>(word, value);
+    launch_chained(set_word_kernel, dim3(1), dim3(1), 0, c->stream, word, value);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? KNNSSD_OK : fail(c, KNNSSD_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
@@ -879,8 +895,7 @@ knnssd_status do_prefill(knnssd_ctx *c, const int *tokens_host, int n, float *po
     cudaStream_t s = c->stream;
     c->prefilled = false;
     CUDA_TRY(c, cudaMemcpyAsync(c->prompt, tokens_host, sizeof(int) * n, cudaMemcpyHostToDevice, s));
-    set_state_kernel<<<1, 1, 0, s>>>(c->state, 0, 0);
-    cudaEventRecord(c->ev0, s);
+    set_state_kernel<<<1, 1, 0, s>>>(c->state, 0, 0, stamps_of(c));
     const int d = g.d_model;
     const int chunk = c->mega_ok ? pass::MAXM : kMaxRows;   // rows per pass: what the faster path takes
     // prompts longer than one pass's rows go through the tensor-core prompt pass where the model is eligible for it
@@ -904,8 +919,7 @@ knnssd_status do_prefill(knnssd_ctx *c, const int *tokens_host, int n, float *po
     const bool direct = pooled_dev && stores_reach(c->device, pooled_dev, sizeof(float));
     pool_finish_kernel<<<(d + 255) / 256, 256, 0, s>>>(c->pool_sum, d, g.pool_mode == 0 ? 1.0 / (double)n : 1.0, c->pooled, direct ? pooled_dev : nullptr);
     if (pooled_dev && !direct) CUDA_TRY(c, cudaMemcpyAsync(pooled_dev, c->pooled, sizeof(float) * d, cudaMemcpyDeviceToDevice, s));
-    emit_first_token_kernel<<<1, 1, 0, s>>>(c->chain, c->state, c->out_tokens, n, c->err_word, c->pinned, c->pinned + kErrWord);
-    cudaEventRecord(c->ev1, s);
+    emit_first_token_kernel<<<1, 1, 0, s>>>(c->chain, c->state, c->out_tokens, n, c->err_word, c->pinned, c->pinned + kErrWord, stamps_of(c) + 1);
     knnssd_status st = sync_check(c, "prefill");
     if (st == KNNSSD_OK) st = checked_err(c, "prefill");
     if (st != KNNSSD_OK) return st;
@@ -914,7 +928,7 @@ knnssd_status do_prefill(knnssd_ctx *c, const int *tokens_host, int n, float *po
     c->prefilled = true;
     c->stats = knnssd_stats{};
     c->stats.tokens = 1;
-    c->stats.ms_prefill = elapsed_ms(c);
+    c->stats.ms_prefill = stamped_ms(c);
     if (first_token) *first_token = c->pending;
     return KNNSSD_OK;
 }
@@ -926,10 +940,8 @@ knnssd_status do_select(knnssd_ctx *c, const float *query_dev, int *domain, int 
     if (knnssd_status r = refuse_capture(c, "select_skipset"); r != KNNSSD_OK) return r;
     const int n = g.n_domains * g.anchors_per_domain;
     cudaStream_t s = c->stream;
-    cudaEventRecord(c->ev0, s);
-    launch_cosine_top1(query_dev ? query_dev : c->pooled, c->anchors, n, g.d_model, c->n_sms, c->cosines, c->knn_work, c->pinned, s);
+    launch_cosine_top1(query_dev ? query_dev : c->pooled, c->anchors, n, g.d_model, c->n_sms, c->cosines, c->knn_work, c->pinned, s, stamps_of(c));
     CUDA_TRY(c, cudaGetLastError());
-    cudaEventRecord(c->ev1, s);
     knnssd_status st = sync_check(c, "select_skipset");
     if (st != KNNSSD_OK) return st;
     if (c->pinned[2]) return fail(c, KNNSSD_ERR_DEGENERATE, "select_skipset: query has zero or non-finite norm");
@@ -940,7 +952,7 @@ knnssd_status do_select(knnssd_ctx *c, const float *query_dev, int *domain, int 
     c->active_mask.assign(c->domain_masks.begin() + (size_t)dom * 2 * g.n_layers,
                           c->domain_masks.begin() + (size_t)(dom + 1) * 2 * g.n_layers);
     c->has_mask = true;
-    c->stats.ms_select = elapsed_ms(c);
+    c->stats.ms_select = stamped_ms(c);
     if (domain) *domain = dom;
     if (anchor) *anchor = best % g.anchors_per_domain;
     if (cosine) *cosine = cs;
@@ -956,7 +968,7 @@ template <bool ACCEPT> cudaError_t deliver(knnssd_ctx *c, Delivery out) {
             if (e != cudaSuccess) return e;
             out.n[r] = 0;
         }
-    out.err = c->err_word; out.host = c->pinned; out.host_err = c->pinned + kErrWord;
+    out.err = c->err_word; out.host = c->pinned; out.host_err = c->pinned + kErrWord; out.stamp = stamps_of(c) + 1;
     const size_t blocks = (out.n[0] + out.n[1]) / 4 / 256 + 1;       // four floats a thread and step
     launch_chained(deliver_kernel<ACCEPT>, dim3((unsigned)(blocks < 2 * (size_t)c->n_sms ? blocks : 2 * c->n_sms)), dim3(256), 0, c->stream, out);
     c->launches++;
@@ -1065,7 +1077,7 @@ knnssd_status knnssd_init(const knnssd_config *cfg, const knnssd_weights *w, con
     std::vector<double> inv_freq(hd / 2);
     for (int i = 0; i < hd / 2; ++i) inv_freq[i] = std::pow((double)g.rope_theta, -2.0 * (double)i / (double)hd);
     cudaMemcpyAsync(c->inv_freq, inv_freq.data(), sizeof(double) * inv_freq.size(), cudaMemcpyHostToDevice, c->stream);
-    set_state_kernel<<<1, 1, 0, c->stream>>>(c->state, 0, 0);
+    set_state_kernel<<<1, 1, 0, c->stream>>>(c->state, 0, 0, nullptr);
     cudaMemsetAsync(c->flag, 0, sizeof(int), c->stream);
     cudaMemsetAsync(c->knn_work, 0, 2 * sizeof(int), c->stream);
     cudaMemsetAsync(c->err_word, 0, sizeof(int), c->stream);
@@ -1194,8 +1206,7 @@ knnssd_status knnssd_draft(knnssd_ctx *c, int k, int *draft_tokens_host, float *
     if (!c->has_mask) return fail(c, KNNSSD_ERR_STATE, "draft: no active skip mask (select_skipset or set_skipmask first)");
     if (c->len + k + 1 > c->cfg.max_seq) return fail(c, KNNSSD_ERR_CAPACITY, "draft: len + k + 1 exceeds max_seq");
     if (knnssd_status r = refuse_capture(c, "draft"); r != KNNSSD_OK) return r;
-    cudaStream_t s = c->stream;
-    cudaEventRecord(c->ev0, s);
+    c->stamp_pass = true;
     for (int j = 0; j < k; ++j) {
         run_pass(c, 1, c->chain + j, j, c->active_mask.data(), 0, c->chain + j + 1, false);
         if (!logits_dev_or_null && j + 1 < k) continue;
@@ -1204,12 +1215,11 @@ knnssd_status knnssd_draft(knnssd_ctx *c, int k, int *draft_tokens_host, float *
         if (j + 1 == k) { out.words = c->chain + 1; out.n_words = k; }
         CUDA_TRY(c, deliver<false>(c, out));
     }
-    cudaEventRecord(c->ev1, s);
     knnssd_status st = sync_check(c, "draft");
     if (st == KNNSSD_OK) st = checked_err(c, "draft");
     if (st != KNNSSD_OK) return st;
     for (int j = 0; j < k; ++j) draft_tokens_host[j] = c->pinned[j];
-    c->stats.ms_draft += elapsed_ms(c);
+    c->stats.ms_draft += stamped_ms(c);
     return KNNSSD_OK;
 }
 
@@ -1229,9 +1239,9 @@ knnssd_status knnssd_verify(knnssd_ctx *c, const int *draft_tokens_host, int k, 
     if (k > 0) {
         Tokens t{};
         for (int j = 0; j < k; ++j) t.id[j] = draft_tokens_host[j];
-        put_tokens_kernel<<<1, 32, 0, s>>>(t, k, c->chain + 1);
+        launch_chained(put_tokens_kernel, dim3(1), dim3(32), 0, s, t, k, c->chain + 1);
     }
-    cudaEventRecord(c->ev0, s);
+    c->stamp_pass = true;
     run_pass(c, k + 1, c->chain, 0, nullptr, 0, c->target, hidden_dev_or_null != nullptr);
     Delivery out{};
     if (logits_dev_or_null) { out.src[0] = c->logits; out.dst[0] = logits_dev_or_null; out.n[0] = (size_t)(k + 1) * g.vocab; }
@@ -1240,7 +1250,6 @@ knnssd_status knnssd_verify(knnssd_ctx *c, const int *draft_tokens_host, int k, 
     out.chain = c->chain; out.target = c->target; out.k = k; out.st = c->state; out.out_tokens = c->out_tokens; out.out_cap = g.max_seq;
     out.accept_log = c->accept_log; out.round_idx = c->stats.rounds % g.max_seq;
     CUDA_TRY(c, deliver<true>(c, out));
-    cudaEventRecord(c->ev1, s);
     knnssd_status st = sync_check(c, "verify");
     if (st == KNNSSD_OK) st = checked_err(c, "verify");
     if (st != KNNSSD_OK) return st;
@@ -1251,7 +1260,7 @@ knnssd_status knnssd_verify(knnssd_ctx *c, const int *draft_tokens_host, int k, 
     c->stats.drafted += k;
     c->stats.accepted += hs->last_accept;
     c->stats.tokens += hs->last_accept + 1;
-    c->stats.ms_verify += elapsed_ms(c);
+    c->stats.ms_verify += stamped_ms(c);
     if (n_accepted) *n_accepted = hs->last_accept;
     if (next_token) *next_token = hs->last_next;
     return KNNSSD_OK;
@@ -1275,7 +1284,7 @@ static knnssd_status do_decode(knnssd_ctx *c, int max_new, int k, int use_select
     }
     cudaStream_t s = c->stream;
     // the pending token is the first token of this call's output
-    emit_first_token_kernel<<<1, 1, 0, s>>>(c->chain, c->state, c->out_tokens, c->len, nullptr, nullptr, nullptr);
+    emit_first_token_kernel<<<1, 1, 0, s>>>(c->chain, c->state, c->out_tokens, c->len, nullptr, nullptr, nullptr, nullptr);
     c->launches++;
     int produced = 1, round = 0;
     c->stats.rounds = c->stats.drafted = c->stats.accepted = 0;
@@ -1363,7 +1372,7 @@ knnssd_status knnssd_decode_sampled(knnssd_ctx *c, int max_new, int k, float tem
     auto finish = [&](knnssd_status r) { cudaStreamSynchronize(s); return r; };
     if (max_new > 1 && cudaMemcpyAsync(u_dev, uniforms_host, sizeof(float) * n_u, cudaMemcpyHostToDevice, s) != cudaSuccess)
         return finish(fail(c, KNNSSD_ERR_CUDA, "decode_sampled: cannot copy the uniforms"));
-    emit_first_token_kernel<<<1, 1, 0, s>>>(c->chain, c->state, c->out_tokens, c->len, nullptr, nullptr, nullptr);
+    emit_first_token_kernel<<<1, 1, 0, s>>>(c->chain, c->state, c->out_tokens, c->len, nullptr, nullptr, nullptr, nullptr);
     c->launches++;
     int produced = 1, round = 0;
     c->stats.rounds = c->stats.drafted = c->stats.accepted = 0;

@@ -76,18 +76,13 @@ struct Params {
     int out_row0;              // row of the logits / hidden-state buffers that this pass's row 0 goes to
     unsigned long long bar_base;   // value of *bar when this launch starts
     int merge_op;              // the attention partials are merged by the separate merge operation (merge_rows_separately)
+    unsigned long long *stamp; // if given: when the pass began (pinned host memory)
     unsigned bar_spin_limit;   // polls a grid-barrier wait may take before the pass is aborted (0 = BAR_SPIN_LIMIT)
 };
 
 // Whether a pass of M rows merges its attention partials in the separate operation: when an attention task carries
 // at least MERGE_ROWS (row, head) pairs.
 __host__ __device__ inline bool merge_rows_separately(int M, int G) { return M * G >= MERGE_ROWS; }
-
-__device__ __forceinline__ unsigned long long globaltimer_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-    return t;
-}
 
 // ---- grid-wide barrier among the consumer warps of all CTAs -----------------------------------------------
 __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long *p) {
@@ -131,6 +126,7 @@ __device__ __forceinline__ bool grid_barrier(const Model &md, const Ring &r, uns
 __device__ __noinline__ void embed_phase(const Model &md, const Op &op, const Params &pr, const Ring &r, int cta, int n_cta,
                                             int tid) {
     if (tid == 0) *r.pos0 = md.state->len + pr.pos_off;
+    if (tid == 0 && cta == 0 && pr.stamp) *pr.stamp = globaltimer_ns();
     if (cta >= pr.M) return;                               // whole CTAs only: the named barrier below is CTA-local
     // row m = cta: residual stream in fp32, its pre-split form times the first RMSNorm's gain, its sum of squares
     const int d = md.d_model, m = cta, lane = tid & 31, warp = tid >> 5;

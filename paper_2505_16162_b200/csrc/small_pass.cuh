@@ -41,6 +41,7 @@ struct Args {
     float2 *part_ml, *rope_cs;
     int n_splits;
     void *kc, *vc;                             // [layer][kv head][max_seq][hd]
+    unsigned long long *stamp;                 // if given: when the pass began (pinned host memory)
     unsigned *bar, *next_bar;                  // arrivals of this launch's meetings, zero at its start; the next launch's, zeroed by this one
     int *err;
     unsigned skip[MASK_WORDS];                 // bit j: sublayer j is left out
@@ -248,7 +249,10 @@ __global__ void __launch_bounds__(NT, 1) small_pass_kernel(const __grid_constant
     unsigned met = 0;
     if (tid == 0) {
         s_abort = 0;
-        if (blockIdx.x == 0) *a.next_bar = 0u;
+        if (blockIdx.x == 0) {
+            *a.next_bar = 0u;
+            if (a.stamp && a.l_from < 0) *a.stamp = globaltimer_ns();
+        }
     }
     const int pos0 = a.st->len + a.pos_off;
 

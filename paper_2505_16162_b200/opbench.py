@@ -116,7 +116,7 @@ def bench_prompt(shape_name: str, layers: int, rows: int, iters: int, seed: int 
     ms = []
     for _ in range(iters + 2):
         sess.prefill(prompt)
-        ms.append(sess.get_stats()["ms_prefill"])         # CUDA events around the pass, on its stream
+        ms.append(sess.get_stats()["ms_prefill"])         # device time of the pass
     ms = sorted(ms[2:])
     d, hd = shape.d_model, shape.head_dim
     weights = layers * (2 * d * shape.n_heads * hd + 2 * d * shape.n_kv_heads * hd + 3 * d * shape.d_ff)
