@@ -632,8 +632,14 @@ constexpr int kSmallHeadIds = 12288;
 constexpr int kSmallTasks = 4;
 
 template <typename WT, int MT> cudaError_t launch_small_t(const small::Args &a, int grid, cudaStream_t s) {
+    static bool configured[kMaxDevices] = {};          // function attributes are per device
+    const int dev = current_device_slot();
+    if (!configured[dev]) {
+        cudaFuncSetAttribute(small::small_pass_kernel<WT, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, small::SMEM_BYTES);
+        configured[dev] = true;
+    }
     void *args[] = {const_cast<small::Args *>(&a)};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<void *>(small::small_pass_kernel<WT, MT>), dim3(grid), dim3(small::NT), args, 0, s);
+    return cudaLaunchCooperativeKernel(reinterpret_cast<void *>(small::small_pass_kernel<WT, MT>), dim3(grid), dim3(small::NT), args, small::SMEM_BYTES, s);
 }
 template <typename WT> cudaError_t launch_small(const small::Args &a, int grid, cudaStream_t s) {
     if (a.M <= 1) return launch_small_t<WT, 1>(a, grid, s);

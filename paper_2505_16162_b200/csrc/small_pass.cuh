@@ -5,8 +5,11 @@
 // the next: 7 launches a layer, ~4.3 us each.  Here the pass is one cooperative launch of at most one block per SM that walks the
 // same operations with a grid-wide meeting between dependent ones, five a layer (six where a row's context is more than one split): the rotary embedding and the K / V rows are
 // written by the warps that compute the projections (a warp owns the two units of a rotary pair), and a row whose context is one
-// split leaves its attention output without a merge.  Bound by the meetings and the trips to L2 behind them, 3.8 us from one to the
-// next: fp32 tiny shape (4 layers, d 256), five rows: 170 -> 84 us on the device.
+// split leaves its attention output without a merge.  Bound by the meetings and the trips to L2 behind them.  What a block can have before a
+// meeting is over - the layers' pointers, its warps' first weight rows of the next map, the gains - is on its way into shared memory
+// between its arrival and the others', and the rows of a map are brought in once for all warps.  Calls, us, before and with that: fp32 tiny
+// shape (4 layers, d 256) at 96 positions, 1 / 5 / 16 rows 97 / 113 / 159, 93 / 108 / 151; bf16 d 1000, two layers 118 / 150 / 250, 86 / 112 / 187.
+// (The copies begun before the arrival: no gain on the tiny shape.)
 //
 // Rows are independent of how many the pass carries.  Every wait is bounded: a block that gives up reports to the session's error
 // word and all blocks fall through to the end.
@@ -56,13 +59,17 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p) {
     return v;
 }
 
-// All blocks have come this far and see one another's writes.  target: arrivals up to and including this meeting.
-__device__ __forceinline__ bool meet_grid(const Args &a, unsigned &target, int *s_abort) {
+// All blocks have come this far and see one another's writes.  target: arrivals up to and including this meeting.  meanwhile(): what a block
+// does for itself between its arrival and the others'.
+template <typename F> __device__ __forceinline__ bool meet_grid(const Args &a, unsigned &target, int *s_abort, F meanwhile) {
     target += gridDim.x;
     __syncthreads();
     if (threadIdx.x == 0 && !*s_abort) {
         __threadfence();                       // cumulative: covers the writes of the block's other threads ordered by the barrier
         atomicAdd(a.bar, 1u);
+    }
+    meanwhile();
+    if (threadIdx.x == 0 && !*s_abort) {
         unsigned polls = 0;
         while (ld_acquire_u32(a.bar) < target)
             if (++polls > POLL_LIMIT) { *s_abort = 1; atomicExch(a.err, 8); break; }
@@ -90,16 +97,117 @@ __device__ __forceinline__ void norm_scales(const float *x, int M, int d, float 
     __syncthreads();
 }
 
-// A linear map over M <= MT rows of width K: a warp takes items gw, gw + (warps of the grid), ..; rows(item, w0, w1) names the two
-// weight rows of an item, early(item, m) fetches what row m's end needs, done(item, m, v0, v1, fetched) gets the products with row m,
-// in lane m.  NORM: of the rows times `gain`, scaled by their RMSNorm (every warp reads the rows whole: it sums the squares on the
-// way, where a pass of its own over them took 0.8 us).  The order of a sum depends on K alone.
-template <typename WT, int MT, bool NORM, typename Rows, typename Early, typename Done>
-__device__ __forceinline__ void map_rows(const float *x, int M, int K, const float *gain, float eps, int n_items, Rows rows, Early early, Done done) {
-    const int lane = threadIdx.x & 31;
-    for (int item = blockIdx.x * NW + (threadIdx.x >> 5); item < n_items; item += gridDim.x * NW) {
+// What a block keeps in shared memory: the layers' pointers; the weight rows of every warp's first item of the next map and that map's
+// gains, on their way while the grid meets; the rows of the map at work.  What does not fit is read where it lies.
+constexpr int W_STAGE = 8192, G_STAGE = 8192, X_STAGE = 96 * 1024, LAYERS_STAGE = 16 * MASK_WORDS * (int)sizeof(LayerW);
+constexpr int SMEM_BYTES = NW * W_STAGE + G_STAGE + X_STAGE + LAYERS_STAGE;
+struct Stage {
+    unsigned char *w;                          // this warp's
+    float *g, *x;
+    LayerW *layers;
+};
+enum { MAP_HEADS = 0, MAP_O = 1, MAP_GATE_UP = 2, MAP_DOWN = 3, MAP_HEAD = 4, MAP_NONE = 5 };
+struct Map { int which, layer; };
+
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ bool skipped(const Args &a, int sublayer) { return a.skip[sublayer >> 5] >> (sublayer & 31) & 1u; }
+// The first map of layer l or of the layers behind it, then the head.
+__device__ __forceinline__ Map first_map(const Args &a, int l) {
+    for (; l < a.n_layers; ++l) {
+        if (!skipped(a, 2 * l)) return {MAP_HEADS, l};
+        if (!skipped(a, 2 * l + 1)) return {MAP_GATE_UP, l};
+    }
+    return {a.head_row0 < a.M ? MAP_HEAD : MAP_NONE, 0};
+}
+__device__ __forceinline__ Map next_map(const Args &a, Map m) {
+    if (m.which == MAP_HEADS) return {MAP_O, m.layer};
+    if (m.which == MAP_GATE_UP) return {MAP_DOWN, m.layer};
+    if (m.which == MAP_O && !skipped(a, 2 * m.layer + 1)) return {MAP_GATE_UP, m.layer};
+    return first_map(a, m.layer + 1);
+}
+__device__ __forceinline__ int map_width(const Args &a, int which) { return which == MAP_O ? a.H * a.hd : which == MAP_DOWN ? a.F : a.d; }
+__device__ __forceinline__ int map_items(const Args &a, int which) {
+    return which == MAP_HEADS ? (a.H + 2 * a.Hkv) * (a.hd / 2) : which == MAP_GATE_UP ? a.F : which == MAP_HEAD ? (a.V + 1) / 2 : a.d / 2;
+}
+__device__ __forceinline__ const float *map_gain(const Args &a, const Stage &st, Map m) {
+    return m.which == MAP_HEADS ? st.layers[m.layer].attn_norm : m.which == MAP_GATE_UP ? st.layers[m.layer].mlp_norm : m.which == MAP_HEAD ? a.final_norm : nullptr;
+}
+// The two weight rows of an item: the dimensions of a rotary pair, gate and up, or units 2 item and 2 item + 1.
+template <typename WT> __device__ __forceinline__ void map_rows_of(const Args &a, const Stage &st, Map m, int item, const WT *&r0, const WT *&r1) {
+    const LayerW &ly = st.layers[m.layer];
+    if (m.which == MAP_HEADS) {
+        const int half = a.hd / 2;
+        int slot = item / half;
+        const void *W = ly.wq;
+        if (slot >= a.H) { W = ly.wk; slot -= a.H; if (slot >= a.Hkv) { W = ly.wv; slot -= a.Hkv; } }
+        r0 = reinterpret_cast<const WT *>(W) + (size_t)(slot * a.hd + item % half) * a.d;
+        r1 = r0 + (size_t)half * a.d;
+    } else if (m.which == MAP_GATE_UP) {
+        r0 = reinterpret_cast<const WT *>(ly.w_gate) + (size_t)item * a.d;
+        r1 = reinterpret_cast<const WT *>(ly.w_up) + (size_t)item * a.d;
+    } else {
+        const int K = map_width(a, m.which), n = m.which == MAP_HEAD ? a.V : a.d;
+        const WT *W = reinterpret_cast<const WT *>(m.which == MAP_HEAD ? a.lm_head : m.which == MAP_O ? ly.wo : ly.w_down);
+        r0 = W + (size_t)(2 * item) * K;
+        r1 = W + (size_t)min(2 * item + 1, n - 1) * K;
+    }
+}
+template <typename WT> __device__ __forceinline__ bool weights_fit(int K) { return 2 * K * (int)sizeof(WT) <= W_STAGE; }
+// Starts the copies of what the blocks know of map m before they meet.  No warp is at a map with gains when another one's are fetched.
+template <typename WT> __device__ __forceinline__ void stage_map(const Args &a, const Stage &st, Map m) {
+    if (m.which == MAP_NONE) return;
+    const int lane = threadIdx.x & 31, K = map_width(a, m.which), item = blockIdx.x * NW + (threadIdx.x >> 5);
+    __syncwarp();                                                // the rows before have been read
+    if (weights_fit<WT>(K) && item < map_items(a, m.which)) {
         const WT *r0, *r1;
-        rows(item, r0, r1);
+        map_rows_of(a, st, m, item, r0, r1);
+        for (int e = lane * 16; e < K * (int)sizeof(WT); e += 512) {
+            cp_async16(st.w + e, reinterpret_cast<const unsigned char *>(r0) + e);
+            cp_async16(st.w + K * sizeof(WT) + e, reinterpret_cast<const unsigned char *>(r1) + e);
+        }
+    }
+    const float *gain = map_gain(a, st, m);
+    if (gain && K * (int)sizeof(float) <= G_STAGE)
+        for (int i = 4 * threadIdx.x; i < K; i += 4 * NT) cp_async16(st.g + i, gain + i);
+}
+// Eight weights from shared memory or from where they lie.
+__device__ __forceinline__ void load8_any(const float *row, int e, float (&w)[8]) {
+    const float4 p = *reinterpret_cast<const float4 *>(row + e), q = *reinterpret_cast<const float4 *>(row + e + 4);
+    w[0] = p.x; w[1] = p.y; w[2] = p.z; w[3] = p.w; w[4] = q.x; w[5] = q.y; w[6] = q.z; w[7] = q.w;
+}
+__device__ __forceinline__ void load8_any(const bf16_t *row, int e, float (&w)[8]) {
+    const uint4 v = *reinterpret_cast<const uint4 *>(row + e);
+    const uint32_t p[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { w[2 * i] = __uint_as_float(p[i] << 16); w[2 * i + 1] = __uint_as_float(p[i] & 0xFFFF0000u); }
+}
+
+// A linear map over M <= MT rows of width K: a warp takes items gw, gw + (warps of the grid), ..; early(item, m) fetches what row m's end
+// needs, done(item, m, v0, v1, fetched) gets the products with row m, in lane m.  NORM: of the rows times the map's gain, scaled by
+// their RMSNorm (every warp reads the rows whole: it sums the squares on the way, where a pass of its own over them took 0.8 us).  The
+// order of a sum depends on K alone.
+template <typename WT, int MT, bool NORM, typename Early, typename Done>
+__device__ __forceinline__ void map_rows(const Args &a, const Stage &st, Map map, const float *x, int M, Early early, Done done) {
+    const int lane = threadIdx.x & 31, K = map_width(a, map.which), n_items = map_items(a, map.which);
+    const float *gain = nullptr;
+    if (NORM) gain = K * (int)sizeof(float) <= G_STAGE ? st.g : map_gain(a, st, map);
+    if (M * K * (int)sizeof(float) <= X_STAGE) {                 // every warp of the block reads all rows
+#pragma unroll 4
+        for (int i = threadIdx.x; i < M * K / 4; i += NT) cp_async16(st.x + 4 * i, x + 4 * i);
+        x = st.x;
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    for (int first = blockIdx.x * NW + (threadIdx.x >> 5), item = first; item < n_items; item += gridDim.x * NW) {
+        const WT *r0, *r1;
+        if (item == first && weights_fit<WT>(K)) {
+            r0 = reinterpret_cast<const WT *>(st.w);
+            r1 = r0 + K;
+        } else {
+            map_rows_of(a, st, map, item, r0, r1);
+        }
         float2 fetched = make_float2(0.f, 0.f);
         if (lane < M) fetched = early(item, lane);
         float acc[2][MT], ss[MT];
@@ -107,10 +215,10 @@ __device__ __forceinline__ void map_rows(const float *x, int M, int K, const flo
         for (int m = 0; m < MT; ++m) acc[0][m] = acc[1][m] = ss[m] = 0.f;
         for (int e = 8 * lane; e < K; e += 256) {
             float w0[8], w1[8];
-            WeightLoad<WT>::load8(r0, e, w0);
-            WeightLoad<WT>::load8(r1, e, w1);
+            load8_any(r0, e, w0);
+            load8_any(r1, e, w1);
             if (NORM) {
-                const float4 g0 = __ldg(reinterpret_cast<const float4 *>(gain + e)), g1 = __ldg(reinterpret_cast<const float4 *>(gain + e + 4));
+                const float4 g0 = *reinterpret_cast<const float4 *>(gain + e), g1 = *reinterpret_cast<const float4 *>(gain + e + 4);
                 const float g[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
 #pragma unroll
                 for (int j = 0; j < 8; ++j) { w0[j] *= g[j]; w1[j] *= g[j]; }
@@ -118,7 +226,7 @@ __device__ __forceinline__ void map_rows(const float *x, int M, int K, const flo
 #pragma unroll
             for (int m = 0; m < MT; ++m) {
                 const float *xr = x + (size_t)min(m, M - 1) * K + e;
-                const float4 x0 = ld_row4(xr), x1 = ld_row4(xr + 4);
+                const float4 x0 = *reinterpret_cast<const float4 *>(xr), x1 = *reinterpret_cast<const float4 *>(xr + 4);
                 const float xv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
@@ -135,7 +243,7 @@ __device__ __forceinline__ void map_rows(const float *x, int M, int K, const flo
             if (lane == m) { v0 = s0; v1 = s1; sq = s2; }
         }
         if (NORM) {
-            const float rinv = 1.0f / sqrtf(sq / (float)K + eps);
+            const float rinv = 1.0f / sqrtf(sq / (float)K + a.eps);
             v0 = __fmul_rn(v0, rinv);
             v1 = __fmul_rn(v1, rinv);
         }
@@ -243,9 +351,10 @@ template <typename WT> __global__ void __launch_bounds__(NT, sizeof(WT) == 4 ? 3
 
 template <typename WT, int MT>
 __global__ void __launch_bounds__(NT, 1) small_pass_kernel(const __grid_constant__ Args a) {
+    extern __shared__ __align__(16) unsigned char small_smem[];
     __shared__ float s_rinv[MT], s_p[NT], s_red[2 * NW];
     __shared__ int s_red_i[NW], s_abort;
-    const int tid = threadIdx.x, M = a.M, d = a.d, hd = a.hd, half = hd / 2, slots = a.H + 2 * a.Hkv, nq = a.H * hd;
+    const int tid = threadIdx.x, M = a.M, d = a.d, hd = a.hd, half = hd / 2, slots = a.H + 2 * a.Hkv;
     unsigned met = 0;
     if (tid == 0) {
         s_abort = 0;
@@ -255,6 +364,16 @@ __global__ void __launch_bounds__(NT, 1) small_pass_kernel(const __grid_constant
         }
     }
     const int pos0 = a.st->len + a.pos_off;
+    auto nothing_more = [] {};
+    Stage st;
+    st.w = small_smem + (tid >> 5) * W_STAGE;
+    st.g = reinterpret_cast<float *>(small_smem + NW * W_STAGE);
+    st.x = st.g + G_STAGE / 4;
+    st.layers = reinterpret_cast<LayerW *>(st.x + X_STAGE / 4);
+    for (int i = tid; i < a.n_layers * (int)(sizeof(LayerW) / 8); i += NT)
+        reinterpret_cast<unsigned long long *>(st.layers)[i] = reinterpret_cast<const unsigned long long *>(a.layers)[i];
+    __syncthreads();
+    stage_map<WT>(a, st, a.l_from < 0 ? first_map(a, 0) : Map{MAP_O, a.l_from});
 
     if (a.l_from < 0) {
         // embedding rows, and (from the last block on) the rows' rotary angles, in fp64
@@ -273,14 +392,10 @@ __global__ void __launch_bounds__(NT, 1) small_pass_kernel(const __grid_constant
                 sincos((double)(pos0 + m) * a.inv_freq[i], &s, &c);
                 a.rope_cs[m * half + i] = make_float2((float)c, (float)s);
             }
-        if (!meet_grid(a, met, &s_abort)) return;
+        if (!meet_grid(a, met, &s_abort, nothing_more)) return;
     }
 
     const int n_split = (pos0 + M + ATT_CHUNK - 1) / ATT_CHUNK;      // of the pass's last row
-    auto pair_rows = [&](const void *W, int K, int n, int item, const WT *&r0, const WT *&r1) {      // units 2 item and 2 item + 1 of n
-        r0 = reinterpret_cast<const WT *>(W) + (size_t)(2 * item) * K;
-        r1 = reinterpret_cast<const WT *>(W) + (size_t)min(2 * item + 1, n - 1) * K;
-    };
     // d is even
     auto old_pair = [&](int item, int m) { return __ldcg(reinterpret_cast<const float2 *>(a.x + (size_t)m * d + 2 * item)); };
     auto add_pair = [&](int item, int m, float v0, float v1, float2 old) {
@@ -288,18 +403,10 @@ __global__ void __launch_bounds__(NT, 1) small_pass_kernel(const __grid_constant
     };
     auto nothing = [&](int, int) { return make_float2(0.f, 0.f); };
     for (int l = max(a.l_from, 0); l < a.n_layers; ++l) {
-        const LayerW &ly = a.layers[l];
-        if (!(a.skip[l >> 4] >> (2 * (l & 15)) & 1u)) {
+        if (!skipped(a, 2 * l)) {
             if (l != a.l_from) {
                 WT *kc = reinterpret_cast<WT *>(a.kc) + (size_t)l * a.Hkv * a.max_seq * hd, *vc = reinterpret_cast<WT *>(a.vc) + (size_t)l * a.Hkv * a.max_seq * hd;
-                map_rows<WT, MT, true>(a.x, M, d, ly.attn_norm, a.eps, slots * half,
-                                 [&](int item, const WT *&r0, const WT *&r1) {
-                                     int slot = item / half;
-                                     const void *W = ly.wq;
-                                     if (slot >= a.H) { W = ly.wk; slot -= a.H; if (slot >= a.Hkv) { W = ly.wv; slot -= a.Hkv; } }
-                                     r0 = reinterpret_cast<const WT *>(W) + (size_t)(slot * hd + item % half) * d;
-                                     r1 = r0 + (size_t)half * d;
-                                 },
+                map_rows<WT, MT, true>(a, st, {MAP_HEADS, l}, a.x, M,
                                  [&](int item, int m) { return __ldcg(a.rope_cs + m * half + item % half); },
                                  [&](int item, int m, float p, float q, float2 c) {
                                      const int slot = item / half, i = item % half;
@@ -321,9 +428,9 @@ __global__ void __launch_bounds__(NT, 1) small_pass_kernel(const __grid_constant
                                      }
                                  });
                 if (l == a.l_to) return;
-                if (!meet_grid(a, met, &s_abort)) return;
+                if (!meet_grid(a, met, &s_abort, [&] { stage_map<WT>(a, st, {MAP_O, l}); })) return;
                 attend_rows<WT, 32, 16>(a, l, pos0, s_p, s_red);
-                if (!meet_grid(a, met, &s_abort)) return;
+                if (!meet_grid(a, met, &s_abort, nothing_more)) return;
             }
             if (n_split > 1) {
                 for (int task = blockIdx.x; task < a.H * M; task += gridDim.x) {
@@ -341,24 +448,20 @@ __global__ void __launch_bounds__(NT, 1) small_pass_kernel(const __grid_constant
                         a.attn[(size_t)task * hd + tid] = o / den;
                     }
                 }
-                if (!meet_grid(a, met, &s_abort)) return;
+                if (!meet_grid(a, met, &s_abort, nothing_more)) return;
             }
-            map_rows<WT, MT, false>(a.attn, M, nq, nullptr, 0.f, d / 2, [&](int item, const WT *&r0, const WT *&r1) { pair_rows(ly.wo, nq, d, item, r0, r1); }, old_pair, add_pair);
-            if (!meet_grid(a, met, &s_abort)) return;
+            map_rows<WT, MT, false>(a, st, {MAP_O, l}, a.attn, M, old_pair, add_pair);
+            if (!meet_grid(a, met, &s_abort, [&] { stage_map<WT>(a, st, next_map(a, {MAP_O, l})); })) return;
         }
-        if (!(a.skip[l >> 4] >> (2 * (l & 15) + 1) & 1u)) {
-            map_rows<WT, MT, true>(a.x, M, d, ly.mlp_norm, a.eps, a.F,
-                             [&](int item, const WT *&r0, const WT *&r1) {
-                                 r0 = reinterpret_cast<const WT *>(ly.w_gate) + (size_t)item * d;
-                                 r1 = reinterpret_cast<const WT *>(ly.w_up) + (size_t)item * d;
-                             },
+        if (!skipped(a, 2 * l + 1)) {
+            map_rows<WT, MT, true>(a, st, {MAP_GATE_UP, l}, a.x, M,
                              nothing,
                              [&](int item, int m, float g, float u, float2) {
                                  a.act[(size_t)m * a.F + item] = g / (1.0f + expf(-g)) * u;
                              });
-            if (!meet_grid(a, met, &s_abort)) return;
-            map_rows<WT, MT, false>(a.act, M, a.F, nullptr, 0.f, d / 2, [&](int item, const WT *&r0, const WT *&r1) { pair_rows(ly.w_down, a.F, d, item, r0, r1); }, old_pair, add_pair);
-            if (!meet_grid(a, met, &s_abort)) return;
+            if (!meet_grid(a, met, &s_abort, [&] { stage_map<WT>(a, st, {MAP_DOWN, l}); })) return;
+            map_rows<WT, MT, false>(a, st, {MAP_DOWN, l}, a.act, M, old_pair, add_pair);
+            if (!meet_grid(a, met, &s_abort, [&] { stage_map<WT>(a, st, next_map(a, {MAP_DOWN, l})); })) return;
         }
     }
     const int hm = M - a.head_row0;
@@ -369,15 +472,14 @@ __global__ void __launch_bounds__(NT, 1) small_pass_kernel(const __grid_constant
             for (int i = tid; i < d; i += NT) a.hfinal[(size_t)m * d + i] = __ldcg(a.x + (size_t)m * d + i) * s_rinv[m] * a.final_norm[i];
     }
     if (hm <= 0) return;
-    map_rows<WT, MT, true>(a.x + (size_t)a.head_row0 * d, hm, d, a.final_norm, a.eps, (a.V + 1) / 2,
-                     [&](int item, const WT *&r0, const WT *&r1) { pair_rows(a.lm_head, d, a.V, item, r0, r1); },
+    map_rows<WT, MT, true>(a, st, {MAP_HEAD, 0}, a.x + (size_t)a.head_row0 * d, hm,
                      nothing,
                      [&](int item, int m, float v0, float v1, float2) {
                          float *dst = a.logits + (size_t)(a.head_row0 + m) * a.V + 2 * item;
                          dst[0] = v0;
                          if (2 * item + 1 < a.V) dst[1] = v1;
                      });
-    if (!meet_grid(a, met, &s_abort)) return;
+    if (!meet_grid(a, met, &s_abort, nothing_more)) return;
     for (int j = blockIdx.x; j < hm; j += gridDim.x) {               // arg-max of a row by a block, lowest index among equals
         const float *row = a.logits + (size_t)(a.head_row0 + j) * a.V;
         float bv = -INFINITY;

@@ -135,3 +135,33 @@ def test_sublayers_left_out_of_a_pass_in_parts():
         n_launches = _launches(sess, lambda: got.append(sess.draft(1, want_logits=True)[1]))
         assert n_launches == 2 + 2 * int((mask[::2] == 0).sum())
         assert np.abs(got[0].cpu().numpy() - om.forward(rows[:1], len(prompt), skip_mask=mask)["logits"]).max() < TOL["fp32"], mask
+
+
+@pytest.mark.parametrize("shape", [si.ModelShape("wide-bf16", 2, 2056, 8, 2, 64, 1032, 515, "bf16", 1e-5, 10000.0),
+                                   si.ModelShape("wide-fp32", 2, 1032, 4, 4, 64, 2056, 515, "fp32", 1e-5, 10000.0)], ids=lambda s: s.name)
+def test_widths_that_shared_memory_does_not_hold(shape):
+    """Weight rows, gains and (from some row count on) the rows of a map one step longer than what a block keeps of them."""
+    from paper_2505_16162_b200 import build
+    build.build()
+    from paper_2505_16162_b200 import binding as kb
+    w = si.make_model_weights(shape, 6, gain_spread=0.1)
+    om = oracle.OracleModel(shape, w, 64)
+    sess = kb.Session.from_shape(shape, {k: ([t.cuda() for t in v] if isinstance(v, list) else v.cuda()) for k, v in w.items()}, 64, max_draft=15)
+    prompt = si.uniform_tokens(6, 0, 30, shape.vocab).numpy()
+    om.prefill(prompt)
+    sess.prefill(prompt)
+    for mask in ([0, 1, 0, 0], [1, 0, 0, 1], [0, 0, 1, 1], [1, 1, 1, 1]):
+        sess.set_length(30)
+        sess.set_skipmask(np.array(mask, np.uint8))
+        sess.set_pending(int(prompt[3]))
+        logits = sess.draft(1, want_logits=True)[1]
+        want = om.forward(prompt[3:4], 30, skip_mask=np.array(mask, np.uint8))["logits"]
+        assert np.abs(logits.cpu().numpy() - want).max() < TOL[shape.dtype], mask
+    for k in (0, 4, 10, 11, 12, 15):
+        rows = si.uniform_tokens(6, 100 + k, k + 1, shape.vocab).numpy()
+        want = om.forward(rows, 30, want_hidden=True)
+        sess.set_length(30)
+        sess.set_pending(int(rows[0]))
+        got = sess.verify(rows[1:], want_logits=True, want_hidden=True)
+        assert np.abs(got["logits"].cpu().numpy() - want["logits"]).max() < TOL[shape.dtype], k
+        assert np.abs(got["hidden"].cpu().numpy() - want["hidden"]).max() < TOL[shape.dtype], k
