@@ -443,6 +443,7 @@ __global__ void __launch_bounds__(256) rmsnorm_rows_kernel(const float *__restri
 
 // Running fp64 sum of hidden rows in row order (the pooled vector's numerator).  grid = ceil(d/256).
 __global__ void pool_accumulate_kernel(const float *__restrict__ h, int M, int d, double *__restrict__ sum, int overwrite) {
+    chain_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= d) return;
     double s = overwrite ? 0.0 : sum[i];
@@ -457,6 +458,7 @@ __global__ void pool_accumulate_kernel(const float *__restrict__ h, int M, int d
 constexpr int POOL_ROWS = 32;
 __global__ void __launch_bounds__(256) pool_partial_kernel(const float *__restrict__ x, const float *__restrict__ rinv, const float *__restrict__ gain,
                                                            int M, int d, double *__restrict__ part) {
+    chain_wait();
     const int i = blockIdx.x * 256 + threadIdx.x, m0 = blockIdx.y * POOL_ROWS, m1 = min(M, m0 + POOL_ROWS);
     if (i >= d) return;
     const float g = gain[i];
@@ -466,6 +468,7 @@ __global__ void __launch_bounds__(256) pool_partial_kernel(const float *__restri
     part[(size_t)blockIdx.y * d + i] = s;
 }
 __global__ void pool_fold_kernel(const double *__restrict__ part, int slices, int d, double *__restrict__ sum, int overwrite) {
+    chain_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= d) return;
     double s = overwrite ? 0.0 : sum[i];
@@ -475,6 +478,7 @@ __global__ void pool_fold_kernel(const double *__restrict__ part, int slices, in
 }
 // rinv[m] = RMSNorm's scale of row m, summed as rmsnorm_rows_kernel does.  grid = M, 256 threads.
 __global__ void __launch_bounds__(256) row_scale_kernel(const float *__restrict__ x, int d, float eps, float *__restrict__ rinv) {
+    chain_wait();
     __shared__ float s_red[8];
     const int m = blockIdx.x, tid = threadIdx.x;
     const float *xr = x + (size_t)m * d;
@@ -493,6 +497,7 @@ __global__ void __launch_bounds__(256) row_scale_kernel(const float *__restrict_
 }
 // v <- the mean, and to the caller's buffer as well if there is one.
 __global__ void pool_finish_kernel(const double *__restrict__ sum, int d, double inv_count, float *__restrict__ v, float *__restrict__ also) {
+    chain_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= d) return;
     const float m = (float)(sum[i] * inv_count);
@@ -769,6 +774,7 @@ __global__ void set_state_kernel(DeviceState *st, int len, int produced, unsigne
 // The first token of a generation; where `host` (pinned) is given the host gets it there, the error word behind it, and when that was.
 __global__ void emit_first_token_kernel(const int *chain, DeviceState *st, int *out_tokens, int len, const int *err, int *host, int *host_err,
                                         unsigned long long *stamp) {
+    chain_wait();
     out_tokens[0] = chain[0]; st->produced = 1; st->len = len;
     if (host) { *host = chain[0]; *host_err = *err; *stamp = globaltimer_ns(); }
 }

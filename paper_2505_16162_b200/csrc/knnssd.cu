@@ -287,7 +287,7 @@ void launch_stream(const LinearArgs &a, int n_sms, int *err, cudaStream_t s) {
         cudaFuncSetAttribute(stream::linear_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, stream::SMEM_BYTES);
         configured[dev] = true;
     }
-    stream::linear_stream_kernel<<<n_sms, stream::NTHREADS, stream::SMEM_BYTES, s>>>(to_phase(a), err);
+    launch_chained(stream::linear_stream_kernel, dim3(n_sms), dim3(stream::NTHREADS), stream::SMEM_BYTES, s, to_phase(a), err);
 }
 
 void launch_linear(int dtype, const LinearArgs &a, int n_sms, int *err, cudaStream_t s) {
@@ -822,8 +822,8 @@ bool prefill_tensor(knnssd_ctx *c, int n) {
     for (int t0 = 0; t0 < n && ok; t0 += cap) {
         const int T = n - t0 < cap ? n - t0 : cap;
         const bool last = t0 + T == n;
-        prefill::embed_rows_kernel<<<T, 256, 0, s>>>(reinterpret_cast<const bf16_t *>(c->tok_embed), c->prompt + t0, d, c->pf_x);
-        prefill::rope_table_kernel<<<T, HD / 2, 0, s>>>(c->inv_freq, t0, c->pf_cs);
+        launch_chained(prefill::embed_rows_kernel, dim3(T), dim3(256), 0, s, reinterpret_cast<const bf16_t *>(c->tok_embed), c->prompt + t0, d, c->pf_x);
+        launch_chained(prefill::rope_table_kernel, dim3(T), dim3(HD / 2), 0, s, c->inv_freq, t0, c->pf_cs);
         launch_chained(prefill::norm_split_kernel, dim3(T), dim3(256), 0, s, c->pf_x, d, c->layers[0].attn_norm, g.rms_eps, c->pf_ad, c->pf_ad + (size_t)cap * d, c->pf_rinv);
         c->launches += 3;
         prefill::Norms normed;                       // of the rows a map reads, and below of those it has added to
@@ -871,19 +871,19 @@ bool prefill_tensor(knnssd_ctx *c, int n) {
         if (g.pool_mode == 0) {
             const int slices = (T + POOL_ROWS - 1) / POOL_ROWS;
             double *part = reinterpret_cast<double *>(c->pf_qkv);                // [slices][d]: knnssd_init makes room for both uses
-            row_scale_kernel<<<T, 256, 0, s>>>(c->pf_x, d, g.rms_eps, c->pf_rinv);
-            pool_partial_kernel<<<dim3((d + 255) / 256, slices), 256, 0, s>>>(c->pf_x, c->pf_rinv, c->final_norm, T, d, part);
-            pool_fold_kernel<<<(d + 255) / 256, 256, 0, s>>>(part, slices, d, c->pool_sum, t0 == 0);
+            launch_chained(row_scale_kernel, dim3(T), dim3(256), 0, s, c->pf_x, d, g.rms_eps, c->pf_rinv);
+            launch_chained(pool_partial_kernel, dim3((d + 255) / 256, slices), dim3(256), 0, s, c->pf_x, c->pf_rinv, c->final_norm, T, d, part);
+            launch_chained(pool_fold_kernel, dim3((d + 255) / 256), dim3(256), 0, s, part, slices, d, c->pool_sum, t0 == 0);
             c->launches += 3;
         } else if (last) {
-            rmsnorm_rows_kernel<<<1, 256, 0, s>>>(c->pf_x + (size_t)(T - 1) * d, c->final_norm, d, g.rms_eps, c->hfinal);
-            pool_accumulate_kernel<<<(d + 255) / 256, 256, 0, s>>>(c->hfinal, 1, d, c->pool_sum, 1);
+            launch_chained(rmsnorm_rows_kernel, dim3(1), dim3(256), 0, s, c->pf_x + (size_t)(T - 1) * d, c->final_norm, d, g.rms_eps, c->hfinal);
+            launch_chained(pool_accumulate_kernel, dim3((d + 255) / 256), dim3(256), 0, s, c->hfinal, 1, d, c->pool_sum, 1);
             c->launches += 2;
         }
         if (last) {
             ctx_linear(c, make_args(c->lm_head, V, d, c->pf_x + (size_t)(T - 1) * d, c->final_norm, g.rms_eps, c->logits, EPI_STORE, 1));
-            argmax_partial_kernel<<<dim3(kArgmaxBlocks, 1), 256, 0, s>>>(c->logits, V, kArgmaxBlocks, c->amax_v, c->amax_i);
-            argmax_final_kernel<<<1, 32, 0, s>>>(c->amax_v, c->amax_i, kArgmaxBlocks, c->chain, V, c->err_word);
+            launch_chained(argmax_partial_kernel, dim3(kArgmaxBlocks, 1), dim3(256), 0, s, c->logits, V, kArgmaxBlocks, c->amax_v, c->amax_i);
+            launch_chained(argmax_final_kernel, dim3(1), dim3(32), 0, s, c->amax_v, c->amax_i, kArgmaxBlocks, c->chain, V, c->err_word);
             c->launches += 2;
         }
     }
@@ -917,15 +917,15 @@ knnssd_status do_prefill(knnssd_ctx *c, const int *tokens_host, int n, float *po
         const bool hidden = g.pool_mode == 0 || last;
         run_pass(c, M, c->prompt + t0, t0, nullptr, last ? M - 1 : M, c->chain, hidden);
         if (g.pool_mode == 0) {
-            pool_accumulate_kernel<<<(d + 255) / 256, 256, 0, s>>>(c->hfinal, M, d, c->pool_sum, t0 == 0);
+            launch_chained(pool_accumulate_kernel, dim3((d + 255) / 256), dim3(256), 0, s, c->hfinal, M, d, c->pool_sum, t0 == 0);
         } else if (last) {
-            pool_accumulate_kernel<<<(d + 255) / 256, 256, 0, s>>>(c->hfinal + (size_t)(M - 1) * d, 1, d, c->pool_sum, 1);
+            launch_chained(pool_accumulate_kernel, dim3((d + 255) / 256), dim3(256), 0, s, c->hfinal + (size_t)(M - 1) * d, 1, d, c->pool_sum, 1);
         }
     }
     const bool direct = pooled_dev && stores_reach(c->device, pooled_dev, sizeof(float));
-    pool_finish_kernel<<<(d + 255) / 256, 256, 0, s>>>(c->pool_sum, d, g.pool_mode == 0 ? 1.0 / (double)n : 1.0, c->pooled, direct ? pooled_dev : nullptr);
+    launch_chained(pool_finish_kernel, dim3((d + 255) / 256), dim3(256), 0, s, c->pool_sum, d, g.pool_mode == 0 ? 1.0 / (double)n : 1.0, c->pooled, direct ? pooled_dev : nullptr);
     if (pooled_dev && !direct) CUDA_TRY(c, cudaMemcpyAsync(pooled_dev, c->pooled, sizeof(float) * d, cudaMemcpyDeviceToDevice, s));
-    emit_first_token_kernel<<<1, 1, 0, s>>>(c->chain, c->state, c->out_tokens, n, c->err_word, c->pinned, c->pinned + kErrWord, stamps_of(c) + 1);
+    launch_chained(emit_first_token_kernel, dim3(1), dim3(1), 0, s, c->chain, c->state, c->out_tokens, n, c->err_word, c->pinned, c->pinned + kErrWord, stamps_of(c) + 1);
     knnssd_status st = sync_check(c, "prefill");
     if (st == KNNSSD_OK) st = checked_err(c, "prefill");
     if (st != KNNSSD_OK) return st;

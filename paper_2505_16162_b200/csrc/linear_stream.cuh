@@ -422,8 +422,10 @@ __device__ __forceinline__ void consume_linear(const LinPhase &p, const Ring &r,
     }
 }
 
-// Stand-alone launch of one linear map: grid = one CTA per SM.
+// Stand-alone launch of one linear map: grid = one CTA per SM.  The weights, which no kernel of this library writes, are on their way while
+// the kernel before still runs; the activations are waited for.
 __global__ void __launch_bounds__(NTHREADS, 1) linear_stream_kernel(const LinPhase p, int *err) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     extern __shared__ __align__(128) unsigned char smem[];
     Ring r;
     ring_setup(r, smem, err);
@@ -439,6 +441,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) linear_stream_kernel(const LinPha
         }
     } else {
         regs_inc<REGS_CONSUMER>();
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         consume_linear(p, r, blockIdx.x, gridDim.x, warp, lane, w_use, alive);
     }
 }

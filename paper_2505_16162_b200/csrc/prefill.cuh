@@ -635,6 +635,7 @@ __global__ void __launch_bounds__(256) fold_pieces_kernel(const GemmArgs g) {
 
 // x[t][:] = embedding row of token t (bf16 -> fp32), eight values per thread and step (d is a multiple of 8).  grid = T.
 __global__ void embed_rows_kernel(const bf16_t *__restrict__ table, const int *__restrict__ tok, int d, float *__restrict__ x) {
+    chain_wait();
     const bf16_t *row = table + (size_t)tok[blockIdx.x] * d;
     float *xr = x + (size_t)blockIdx.x * d;
     for (int i = threadIdx.x * 8; i < d; i += blockDim.x * 8) {
@@ -693,6 +694,7 @@ __global__ void __launch_bounds__(256) scales_kernel(const float *__restrict__ s
 // (cos, sin) of the rotary angles of rows t = 0 .. T-1 at positions pos0 + t, once per chunk: all layers and heads
 // use the same table.  grid = T, hd / 2 threads.
 __global__ void rope_table_kernel(const double *__restrict__ inv_freq, int pos0, float2 *__restrict__ table) {
+    chain_wait();
     double sn, cs;
     sincos((double)(pos0 + (int)blockIdx.x) * inv_freq[threadIdx.x], &sn, &cs);
     table[(size_t)blockIdx.x * blockDim.x + threadIdx.x] = make_float2((float)cs, (float)sn);
