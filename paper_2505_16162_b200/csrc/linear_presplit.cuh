@@ -4,7 +4,7 @@
 // split into its bf16 terms and laid out fragment by fragment (LinPhase::xs), written once by whoever produced the
 // activation.  The consumer therefore spends no arithmetic on the split that every CTA would otherwise repeat:
 // per column tile a lane loads four 16-byte pieces per term and row block, one tile ahead of the tensor-core work.
-// RMSNorm's scalar comes from per-CTA partial sums of squares that the producer of the row left in LinPhase::ss_in.
+// RMSNorm's scalar comes from per-CTA partial sums of squares that the producer of the row left in LinPhase::ss_in (scale_rows).
 //
 // NB = row blocks of eight: 1 for passes of up to 8 rows, 2 for 9..16 rows (the second block is a second 8-column
 // operand for the same weight fragments; every row is computed exactly as it would be in a one-row pass).
@@ -30,6 +30,32 @@ namespace stream {
 
 __device__ __forceinline__ uint4 ld_frag4(const uint32_t *p) { return __ldcg(reinterpret_cast<const uint4 *>(p)); }
 
+// RMSNorm's scalars of a map's rows, from the partial sums that the producers of the rows left: by the warps of the producer's warpgroup that
+// have nothing to copy, while the consumers multiply.  Done by the consumers before their first tile they held it back by 0.8 us at one
+// row, 1.1 at five and 1.9 at nine, twice a layer; added up behind the first tile the registers they wait in cost as much as that at six
+// rows and more.  All consumers arrive at barrier 2 once the map's input is there, and meet the scales at barrier 3 where they meet
+// for the end of the first batch.
+constexpr int SCALE_WARPS = 3;
+// (The forms of 13 .. 16 rows have no registers to give to those warps: their consumers do it.)  How the registers are split: at 40 a thread the
+// producer's warpgroup spills with both jobs in it, and a producer that spills costs 2 .. 5 % of a pass; the consumers of up to 8 rows do with
+// 216, those of 9 .. 12 lose 3 % below 224.
+template <int NB, int NP> __host__ __device__ constexpr bool scales_apart() { return NB == 1 || NP == 3; }
+template <int NB, int NP> __host__ __device__ constexpr int regs_producer() { return NB == 1 ? 64 : NP == 3 ? 56 : REGS_PRODUCER; }
+template <int NB, int NP> __host__ __device__ constexpr int regs_consumer() { return NB == 1 ? 216 : NP == 3 ? 224 : REGS_CONSUMER; }
+__device__ __forceinline__ void rows_ready() { asm volatile("bar.arrive 2, %0;" ::"n"((NCW + SCALE_WARPS) * 32) : "memory"); }
+__device__ __forceinline__ void scale_rows(const float *ss_in, int M, int K, float eps, const Ring &r, int n_cta, int idle_warp, int lane) {
+    asm volatile("bar.sync 2, %0;" ::"n"((NCW + SCALE_WARPS) * 32) : "memory");
+#pragma unroll 1
+    for (int row = idle_warp; row < M; row += SCALE_WARPS) {
+        float tot = 0.f;                                         // lanes take CTAs lane, lane + 32, ..
+#pragma unroll 5
+        for (int c = lane; c < n_cta; c += 32) tot += __ldcg(ss_in + (size_t)row * n_cta + c);
+        tot = warp_sum(tot);
+        if (lane == 0) r.red_ss[row] = 1.0f / sqrtf(tot / (float)K + eps);
+    }
+    asm volatile("bar.arrive 3, %0;" ::"n"((NCW + SCALE_WARPS) * 32) : "memory");
+}
+
 // Column groups (of 16 units) a batch of the consumer takes, by kernel form; LinPhase::gb carries it to the producer.
 template <int NB, int NP> __host__ __device__ constexpr int groups_per_batch() { return NP >= 3 ? GB : GB / NB; }
 
@@ -45,6 +71,7 @@ __device__ __forceinline__ void consume_linear_pre(const LinPhase &p, const Ring
     // activation fragments of a column tile are fetched from L2 once per batch, so the 9..12-row and the packed 13..16-row form keep four
     // groups: at two it would pull 0.75 bytes of activations per byte of weights.
     constexpr int GBN = groups_per_batch<NB, NP>();
+    constexpr bool HELPED = scales_apart<NB, NP>();
     constexpr int RW = PAIRED ? 2 : 4;                      // floats a lane leaves per (warp, group, block) for the batch-end sums
     const Share s = make_share(p, cta, n_cta);
     const int tid = warp * 32 + lane;
@@ -90,9 +117,9 @@ __device__ __forceinline__ void consume_linear_pre(const LinPhase &p, const Ring
             }
         };
         fetch(0);
-        if (b == 0 && normed) {
-            // RMSNorm scalar of rows `warp` (and warp + 8) from the producers' partial sums (lanes take CTAs lane,
-            // lane + 32, ...); issued after the first fragment fetch so that both round trips to L2 overlap
+        if (!HELPED && b == 0 && normed) {
+            // RMSNorm scalar of rows `warp` (and warp + 8), lanes as in scale_rows; issued after the first fragment fetch so that both round
+            // trips to L2 overlap
 #pragma unroll
             for (int nb = 0; nb < NB; ++nb) {
                 const int row = nb * 8 + warp;
@@ -199,7 +226,8 @@ __device__ __forceinline__ void consume_linear_pre(const LinPhase &p, const Ring
                 if (PAIRED) *reinterpret_cast<float2 *>(dst) = make_float2(acc[gi][nb][0], acc[gi][nb][1]);
                 else *reinterpret_cast<float4 *>(dst) = make_float4(acc[gi][nb][0], acc[gi][nb][1], acc[gi][nb][2], acc[gi][nb][3]);
             }
-        asm volatile("bar.sync 1, %0;" ::"n"(NCW * 32) : "memory");
+        if (HELPED && b == 0 && normed) asm volatile("bar.sync 3, %0;" ::"n"((NCW + SCALE_WARPS) * 32) : "memory");      // and the rows' scales are there
+        else asm volatile("bar.sync 1, %0;" ::"n"(NCW * 32) : "memory");
         if (alive) {
 #pragma unroll
             for (int it4 = 0; it4 < ITEMS; ++it4) {
@@ -279,6 +307,7 @@ __device__ __forceinline__ void consume_linear_pre(const LinPhase &p, const Ring
         }
         asm volatile("bar.sync 1, %0;" ::"n"(NCW * 32) : "memory");
     }
+    if (HELPED && normed && s.n_batches == 0) asm volatile("bar.sync 3, %0;" ::"n"((NCW + SCALE_WARPS) * 32) : "memory");      // no units: the meeting all the same
     if (p.ss_out && alive && lane == 0) {
 #pragma unroll
         for (int nb = 0; nb < NB; ++nb)

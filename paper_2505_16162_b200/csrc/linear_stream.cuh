@@ -38,7 +38,7 @@ constexpr int NCW = 8;                       // consumer warps
 constexpr int SLOT = SEG / NCW;              // columns per consumer warp per tile (128 = 8 k16 steps)
 constexpr int KSTEPS = SLOT / 16;
 constexpr int GB = 4;                        // groups per batch
-constexpr int NTHREADS = (NCW + 4) * 32;      // two consumer warpgroups + the producer's warpgroup (one warp of it works)
+constexpr int NTHREADS = (NCW + 4) * 32;      // two consumer warpgroups + the producer's warpgroup (one warp of it copies)
 constexpr int REGS_PRODUCER = 40, REGS_CONSUMER = 232;
 constexpr int RED_BYTES = NCW * 8 * 32 * 4 * 4;  // reduction buffer: the batch-end sums, sized for 8 groups
 constexpr int SS_BYTES = NCW * 8 * 4;

@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(stream::NTHREADS, 1) pass_kernel(const __grid_
     int w_use = 0;
     bool alive = true;
     if (warp >= NCW) {
-        stream::regs_dec<stream::REGS_PRODUCER>();
+        stream::regs_dec<stream::regs_producer<NB, NP>()>();
         if (warp == NCW) {
             for (int i = 0; i < pr.n_ops && alive; ++i) {
                 const Op &op = pr.ops[i];
@@ -524,10 +524,18 @@ __global__ void __launch_bounds__(stream::NTHREADS, 1) pass_kernel(const __grid_
                 stream::produce_linear(lp, r, cta, n_cta, lane, w_use, alive);
             }
             if (!alive) stream::producer_drain_after_abort();
+        } else if (stream::scales_apart<NB, NP>()) {
+#pragma unroll 1
+            for (int i = 0; i < pr.n_ops; ++i) {
+                const Op &op = pr.ops[i];
+                if (op.type != OP_LINEAR || !op.lin.ss_in || (op.is_head && pr.head_row0 >= pr.M)) continue;
+                const int row0 = op.is_head ? pr.head_row0 : 0;
+                stream::scale_rows(op.lin.ss_in + (size_t)row0 * n_cta, pr.M - row0, op.lin.K, op.lin.eps, r, n_cta, warp - NCW - 1, lane);
+            }
         }
         return;
     }
-    stream::regs_inc<stream::REGS_CONSUMER>();
+    stream::regs_inc<stream::regs_consumer<NB, NP>()>();
     const int tid = threadIdx.x;
     unsigned long long n_bar = 0;
     // The operation behind the one at work is on its way into shared memory: read from L2 when its turn came (a barrier leaves nothing in
@@ -558,6 +566,7 @@ __global__ void __launch_bounds__(stream::NTHREADS, 1) pass_kernel(const __grid_
                 lp.y += (size_t)(pr.out_row0 + pr.head_row0) * lp.units;
             }
             lp.rope = md.rope_cs + (size_t)cta * MAXM * (HD / 2);
+            if (stream::scales_apart<NB, NP>() && ran && lp.ss_in) stream::rows_ready();
             if (ran) stream::consume_linear_pre<NB, NP>(lp, r, cta, n_cta, warp, lane, w_use, alive);
         } else if (alive) {
             if (op.type == OP_EMBED) embed_phase(md, op, pr, r, cta, n_cta, tid);
