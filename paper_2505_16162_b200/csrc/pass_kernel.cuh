@@ -285,27 +285,20 @@ __device__ __forceinline__ void mma_bf16_rows(float (&c)[4], uint32_t a0, uint32
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// Merge the segment partials of one (row m, head h) in segment order and write the result pre-split (one warp).
-template <int HD>
+// Merge the segment partials of one (row m, head h) in segment order and write the result pre-split (one warp).  Bound by the trips to L2: in
+// passes of up to 8 rows (NB = 1) the first 24 segments' outputs come along with the statistics, others follow 24 at a time.  8 layers, ms, with
+// 16 at a time behind the statistics and so: 13B 1 row at 1280 positions 0.5666 / 0.5626, 5 rows 1.0243 / 1.0164; Qwen 14B 5 rows at 2304 1.125 / 1.110.
+// (9 and more rows have more merges than CTAs, and lose 0.5 .. 1 % by it.)
+template <int HD, int NB>
 __device__ __forceinline__ void attn_merge_row(const Model &md, const Op &op, int P0, int m, int h, int lane) {
-    constexpr int DPL = HD / 32;
+    constexpr int DPL = HD / 32, AHEAD = NB == 1 ? 24 : 16;
     const int H = md.H, d0 = DPL * lane;
     const int n_seg_m = (P0 + m + SEGP) / SEGP;
     const size_t base = ((size_t)m * H + h) * md.n_seg_max;
-    // segment statistics: lane s holds segments s and s + 32 (contexts up to 4096); fixed-order warp reductions
-    const float2 ml0 = lane < n_seg_m ? __ldcg(md.part_ml + base + lane) : make_float2(-INFINITY, 0.f);
-    const float2 ml1 = lane + 32 < n_seg_m ? __ldcg(md.part_ml + base + lane + 32) : make_float2(-INFINITY, 0.f);
-    const float gm = warp_max(fmaxf(ml0.x, ml1.x));
-    const float w0 = ml0.x == -INFINITY ? 0.f : expf(ml0.x - gm), w1 = ml1.x == -INFINITY ? 0.f : expf(ml1.x - gm);
-    const float L = warp_sum(fmaf(ml1.y, w1, ml0.y * w0));
-    // weighted sum of the partial outputs in segment order, sixteen segments in flight at a time
-    float acc[DPL];
+    float pv[AHEAD][DPL];
+    auto fetch = [&](int s0) {
 #pragma unroll
-    for (int e = 0; e < DPL; ++e) acc[e] = 0.f;
-    for (int s0 = 0; s0 < n_seg_m; s0 += 16) {
-        float pv[16][DPL];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
+        for (int i = 0; i < AHEAD; ++i) {
             // one vector load per segment (DPL = 4: 16 bytes, DPL = 2: 8 bytes)
             const float *src = md.part_o + (base + s0 + i) * HD + d0;
             if (DPL == 4) {
@@ -316,8 +309,22 @@ __device__ __forceinline__ void attn_merge_row(const Model &md, const Op &op, in
                 pv[i][0] = v.x; pv[i][DPL - 1] = v.y;
             }
         }
+    };
+    // segment statistics: lane s holds segments s and s + 32 (contexts up to 4096); fixed-order warp reductions
+    const float2 ml0 = lane < n_seg_m ? __ldcg(md.part_ml + base + lane) : make_float2(-INFINITY, 0.f);
+    const float2 ml1 = lane + 32 < n_seg_m ? __ldcg(md.part_ml + base + lane + 32) : make_float2(-INFINITY, 0.f);
+    if (NB == 1) fetch(0);
+    const float gm = warp_max(fmaxf(ml0.x, ml1.x));
+    const float w0 = ml0.x == -INFINITY ? 0.f : expf(ml0.x - gm), w1 = ml1.x == -INFINITY ? 0.f : expf(ml1.x - gm);
+    const float L = warp_sum(fmaf(ml1.y, w1, ml0.y * w0));
+    // weighted sum of the partial outputs in segment order
+    float acc[DPL];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
+    for (int e = 0; e < DPL; ++e) acc[e] = 0.f;
+    for (int s0 = 0; s0 < n_seg_m; s0 += AHEAD) {
+        if (NB > 1 || s0) fetch(s0);
+#pragma unroll
+        for (int i = 0; i < AHEAD; ++i) {
             const int sg = s0 + i;
             const float w = __shfl_sync(0xffffffffu, sg < 32 ? w0 : w1, sg & 31);
 #pragma unroll
@@ -327,7 +334,6 @@ __device__ __forceinline__ void attn_merge_row(const Model &md, const Op &op, in
 #pragma unroll
     for (int e = 0; e < DPL; ++e) stream::store_split(op.lin.ys, (H * HD) >> 7, m, h * HD + d0 + e, acc[e] / L);
 }
-
 
 // Tensor-core form.  Lane (g8, t4) = (lane / 4, lane % 4).  The task's eight (query head, row) pairs are both halves of the 16-row MMA
 // operand: rows 0..7 their hi terms, rows 8..15 their lo terms, so that one product does both.
@@ -345,7 +351,7 @@ __device__ __forceinline__ void attn_merge_row(const Model &md, const Op &op, in
 // With the heads rotated and split by every task, the pass's own K / V rows staged beside it and K read in 16-byte pieces 64 bytes apart
 // (two requests a sector), attention and what follows it up to the output projection took 16.7 us a layer of the 13B widths at 1 row and
 // 1280 positions, 18.5 at 5 rows, 23.7 of the 7B widths at 9 rows and 640; so 12.3, 12.7 and 10.8.
-template <int HD>
+template <int HD, int NB>
 __device__ __forceinline__ void attn_phase(const Model &md, const Op &op, const Params &pr, const Ring &r, int cta, int n_cta, int warp, int lane) {
     constexpr int DL = HD / 4;         // output dimensions per lane
     constexpr int RUN = HD / 8;        // dimensions of q and K per lane and half of the head
@@ -481,7 +487,7 @@ __device__ __forceinline__ void attn_phase(const Model &md, const Op &op, const 
             for (int g = 0; g < BLKM; ++g) {
                 if (!((last_mask >> (4 * g)) & 1u)) continue;
                 const int rg = blk * BLKM + g, mg = rg % M, hg = kvh * G + rg / M;
-                attn_merge_row<HD>(md, op, P0, mg, hg, lane);
+                attn_merge_row<HD, NB>(md, op, P0, mg, hg, lane);
                 if (lane == 0) md.attn_cnt[mg * H + hg] = 0;
             }
         }
@@ -490,11 +496,11 @@ __device__ __forceinline__ void attn_phase(const Model &md, const Op &op, const 
 
 // With several rows the warp that finishes a head last would merge all its rows one after the other; the merges
 // then run as an operation of their own instead, one (row, head) per warp across the whole grid.
-template <int HD>
+template <int HD, int NB>
 __device__ __forceinline__ void attn_merge_phase(const Model &md, const Op &op, const Params &pr, const Ring &r, int cta, int n_cta, int warp,
                                                  int lane) {
     const int P0 = *r.pos0, jobs = pr.M * md.H;
-    for (int j = warp * n_cta + cta; j < jobs; j += NCW * n_cta) attn_merge_row<HD>(md, op, P0, j / md.H, j % md.H, lane);
+    for (int j = warp * n_cta + cta; j < jobs; j += NCW * n_cta) attn_merge_row<HD, NB>(md, op, P0, j / md.H, j % md.H, lane);
 }
 
 // ---- the pass ---------------------------------------------------------------------------------------------------
@@ -570,8 +576,8 @@ __global__ void __launch_bounds__(stream::NTHREADS, 1) pass_kernel(const __grid_
             if (ran) stream::consume_linear_pre<NB, NP>(lp, r, cta, n_cta, warp, lane, w_use, alive);
         } else if (alive) {
             if (op.type == OP_EMBED) embed_phase(md, op, pr, r, cta, n_cta, tid);
-            else if (op.type == OP_ATTN) attn_phase<HD>(md, op, pr, r, cta, n_cta, warp, lane);
-            else if (op.type == OP_ATTN_MERGE) { if (pr.merge_op) attn_merge_phase<HD>(md, op, pr, r, cta, n_cta, warp, lane); else ran = false; }
+            else if (op.type == OP_ATTN) attn_phase<HD, NB>(md, op, pr, r, cta, n_cta, warp, lane);
+            else if (op.type == OP_ATTN_MERGE) { if (pr.merge_op) attn_merge_phase<HD, NB>(md, op, pr, r, cta, n_cta, warp, lane); else ran = false; }
             else if (op.type == OP_HIDDEN) { if (pr.want_hidden) hidden_phase(md, pr, r, cta, tid); else ran = false; }
             else if (op.type == OP_ARGMAX) { if (pr.head_row0 < pr.M) argmax_phase(md, pr, r, cta, n_cta, tid); else ran = false; }
         }
