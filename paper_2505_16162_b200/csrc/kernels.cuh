@@ -639,8 +639,8 @@ __global__ void put_tokens_kernel(const Tokens t, int n, int *__restrict__ chain
 // ---------------------------------------------------------------------------------------------
 
 // Eq. (4) in one launch: dot(v, a) / (|v| |a|) by a block per anchor; then the block that finishes last takes the arg-max of all
-// n, lowest index on ties.  cosines[n] and work[2] (blocks done, a zero or non-finite norm was met) are scratch; work is zero
-// between launches.  out[0] = best flat index, out[1] = its cosine's bits, out[2] = the flag; it may be pinned host memory.
+// n, lowest index on ties.  cosines[n] and work[1] (blocks done) are scratch; work is zero between launches.  out[0] = best flat index,
+// out[1] = its cosine's bits, out[2] = whether a zero or non-finite norm was met; it may be pinned host memory.
 // Bound by latencies: 16 bytes a load where query and rows allow it, 50 x 5120: 5 us (a warp per anchor, 4 bytes a load: 10).  More anchors than
 // blocks are resident, of rows that a block has one piece of per thread, go to a warp each, which takes the shares of the block's warps one
 // after the other (WARPS): the sums are the same.  A call of 4096 x 640 / 20000 x 640 / 100000 x 64 / 100000 x 1024: a block per anchor 35 / 61 /
@@ -668,7 +668,6 @@ template <bool WARPS> __global__ void __launch_bounds__(256) cosine_top1_kernel(
     auto finish = [&](int a, float dot, float vv, float aa) {
         const bool bad = !(vv > 0.f) || !isfinite(vv) || !(aa > 0.f) || !isfinite(aa);
         __stcg(cosines + a, bad ? -INFINITY : (float)((double)dot / sqrt((double)vv * (double)aa)));      // one rounding
-        if (bad) atomicExch(work + 1, 1);
         __threadfence();
     };
     if (!WARPS) {
@@ -726,7 +725,12 @@ template <bool WARPS> __global__ void __launch_bounds__(256) cosine_top1_kernel(
     __threadfence();
     float bv = -INFINITY;
     int bi = 0x7fffffff;
-    for (int i = tid; i < n; i += 256) argmax_fold(bv, bi, __ldcg(cosines + i), i);
+    bool bad = false;                                            // only a vector without a norm has left -inf
+    for (int i = tid; i < n; i += 256) {
+        const float c = __ldcg(cosines + i);
+        bad |= c == -INFINITY;
+        argmax_fold(bv, bi, c, i);
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
@@ -734,13 +738,12 @@ template <bool WARPS> __global__ void __launch_bounds__(256) cosine_top1_kernel(
         argmax_fold(bv, bi, ov, oi);
     }
     if ((tid & 31) == 0) { s_v[tid >> 5] = bv; s_i[tid >> 5] = bi; }
-    __syncthreads();
+    const int any_bad = __syncthreads_or(bad);
     if (tid == 0) {
         for (int w = 1; w < 8; ++w) argmax_fold(bv, bi, s_v[w], s_i[w]);
-        const int bad = atomicExch(work + 1, 0);
         out[0] = bi;
         out[1] = __float_as_int(bv);
-        out[2] = bad;
+        out[2] = any_bad;
         if (stamps) stamps[1] = globaltimer_ns();
         work[0] = 0;
     }
