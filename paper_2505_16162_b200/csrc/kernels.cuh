@@ -23,7 +23,8 @@ __device__ __forceinline__ void chain_wait() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
-// Launch of a kernel that calls chain_wait() before it touches memory.
+// Launch of a kernel that calls chain_wait() before it touches memory.  (The prompt pass's contractions and its head fetch weights before: in a
+// chain that an ordinary launch has begun, nothing on the stream before the chain is still at work.)
 template <typename... P, typename... A>
 void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
     cudaLaunchConfig_t cfg{};

@@ -280,18 +280,23 @@ stream::LinPhase to_phase(const LinearArgs &a) {
     return p;
 }
 
-void launch_stream(const LinearArgs &a, int n_sms, int *err, cudaStream_t s) {
+template <bool EARLY> void launch_stream(const LinearArgs &a, int n_sms, int *err, cudaStream_t s) {
     static bool configured[kMaxDevices] = {};          // function attributes are per device
     const int dev = current_device_slot();
     if (!configured[dev]) {
-        cudaFuncSetAttribute(stream::linear_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, stream::SMEM_BYTES);
+        cudaFuncSetAttribute(stream::linear_stream_kernel<EARLY>, cudaFuncAttributeMaxDynamicSharedMemorySize, stream::SMEM_BYTES);
         configured[dev] = true;
     }
-    launch_chained(stream::linear_stream_kernel, dim3(n_sms), dim3(stream::NTHREADS), stream::SMEM_BYTES, s, to_phase(a), err);
+    launch_chained(stream::linear_stream_kernel<EARLY>, dim3(n_sms), dim3(stream::NTHREADS), stream::SMEM_BYTES, s, to_phase(a), err);
 }
 
-void launch_linear(int dtype, const LinearArgs &a, int n_sms, int *err, cudaStream_t s) {
-    if (stream_eligible(dtype, a)) { launch_stream(a, n_sms, err, s); return; }
+// early: linear_stream_kernel's EARLY, where its conditions hold.
+void launch_linear(int dtype, const LinearArgs &a, int n_sms, int *err, cudaStream_t s, bool early = false) {
+    if (stream_eligible(dtype, a)) {
+        if (early) launch_stream<true>(a, n_sms, err, s);
+        else launch_stream<false>(a, n_sms, err, s);
+        return;
+    }
     // generic kernel: enough warps that every SM holds 8 blocks of 8 warps, but never more warps than units
     long long blocks = (long long)n_sms * 8;
     const long long max_blocks = (a.units + 7) / 8;
@@ -300,7 +305,7 @@ void launch_linear(int dtype, const LinearArgs &a, int n_sms, int *err, cudaStre
     if (dtype) launch_linear_t<bf16_t>(a, (int)blocks, s); else launch_linear_t<float>(a, (int)blocks, s);
 }
 
-void ctx_linear(knnssd_ctx *c, const LinearArgs &a) {
+void ctx_linear(knnssd_ctx *c, const LinearArgs &a, bool early = false) {
     if (c->time_linear) {
         if (c->lin_used + 2 > c->lin_events.size()) {
             for (int i = 0; i < 2; ++i) {
@@ -311,7 +316,7 @@ void ctx_linear(knnssd_ctx *c, const LinearArgs &a) {
         }
         cudaEventRecord(c->lin_events[c->lin_used], c->stream);
     }
-    launch_linear(c->cfg.dtype, a, c->n_sms, c->err_word, c->stream);
+    launch_linear(c->cfg.dtype, a, c->n_sms, c->err_word, c->stream, early);
     if (c->time_linear) {
         cudaEventRecord(c->lin_events[c->lin_used + 1], c->stream);
         c->lin_used += 2;
@@ -881,7 +886,7 @@ bool prefill_tensor(knnssd_ctx *c, int n) {
             c->launches += 2;
         }
         if (last) {
-            ctx_linear(c, make_args(c->lm_head, V, d, c->pf_x + (size_t)(T - 1) * d, c->final_norm, g.rms_eps, c->logits, EPI_STORE, 1));
+            ctx_linear(c, make_args(c->lm_head, V, d, c->pf_x + (size_t)(T - 1) * d, c->final_norm, g.rms_eps, c->logits, EPI_STORE, 1), true);
             launch_chained(argmax_partial_kernel, dim3(kArgmaxBlocks, 1), dim3(256), 0, s, c->logits, V, kArgmaxBlocks, c->amax_v, c->amax_i);
             launch_chained(argmax_final_kernel, dim3(1), dim3(32), 0, s, c->amax_v, c->amax_i, kArgmaxBlocks, c->chain, V, c->err_word);
             c->launches += 2;

@@ -422,10 +422,13 @@ __device__ __forceinline__ void consume_linear(const LinPhase &p, const Ring &r,
     }
 }
 
-// Stand-alone launch of one linear map: grid = one CTA per SM.  The weights, which no kernel of this library writes, are on their way while
-// the kernel before still runs; the activations are waited for.
-__global__ void __launch_bounds__(NTHREADS, 1) linear_stream_kernel(const LinPhase p, int *err) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+// Launch of one linear map: grid = one CTA per SM.  EARLY: the weights are on their way while the kernel before still runs, the activations
+// are waited for.  Only for a launch in a chain that an ordinary launch has begun, with weights that no kernel of the chain writes (the
+// head at the end of a prompt pass: its set_state_kernel has waited for whatever the caller had on the stream).  The kernel before may
+// otherwise be the one that writes W, whoever launched it: its stores can be read once it has been waited for, and not earlier.
+template <bool EARLY> __global__ void __launch_bounds__(NTHREADS, 1) linear_stream_kernel(const LinPhase p, int *err) {
+    if (EARLY) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    else chain_wait();
     extern __shared__ __align__(128) unsigned char smem[];
     Ring r;
     ring_setup(r, smem, err);
@@ -441,7 +444,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) linear_stream_kernel(const LinPha
         }
     } else {
         regs_inc<REGS_CONSUMER>();
-        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (EARLY) asm volatile("griddepcontrol.wait;" ::: "memory");
         consume_linear(p, r, blockIdx.x, gridDim.x, warp, lane, w_use, alive);
     }
 }
