@@ -229,7 +229,10 @@ __device__ __forceinline__ void ring_setup(Ring &r, unsigned char *smem, int *er
 // ------------------------------------------------------------------------------------------------------------
 // Producer warp: streams this CTA's share of the weights of one linear map into the ring.  w_use counts the
 // stages this CTA has filled since the kernel began (the consumers keep the same count).
+// EARLY (linear_stream_kernel): the consumers may still wait for the kernel before.  Once the ring is full so does the producer, whose
+// bounded wait for a free stage would count the time that the other kernel takes.
 // ------------------------------------------------------------------------------------------------------------
+template <bool EARLY = false>
 __device__ __forceinline__ void produce_linear(const LinPhase &p, const Ring &r, int cta, int n_cta, int lane, int &w_use,
                                                bool &alive) {
     const Share s = make_share(p, cta, n_cta);
@@ -271,6 +274,7 @@ __device__ __forceinline__ void produce_linear(const LinPhase &p, const Ring &r,
 #pragma unroll
             for (int gi = 0; gi < GB; ++gi) {
                 if (gi >= ng || !alive) break;
+                if (EARLY && w_use == WS) asm volatile("griddepcontrol.wait;" ::: "memory");
                 if (it > 0) alive = mbar_wait(&r.empty_w[ws], (it - 1) & 1, r.abort_flag, r.err, 3);
                 if (!alive) break;
                 if (lane == 0) mbar_expect_tx(&r.full_w[ws], (uint32_t)nrows[gi] * segc * 2);
@@ -439,7 +443,7 @@ template <bool EARLY> __global__ void __launch_bounds__(NTHREADS, 1) linear_stre
     if (warp >= NCW) {
         regs_dec<REGS_PRODUCER>();
         if (warp == NCW) {
-            produce_linear(p, r, blockIdx.x, gridDim.x, lane, w_use, alive);
+            produce_linear<EARLY>(p, r, blockIdx.x, gridDim.x, lane, w_use, alive);
             if (!alive) producer_drain_after_abort();
         }
     } else {
