@@ -90,8 +90,8 @@ typedef struct {
     int drafted;   /* draft steps taken (sum of k_eff) */
     int accepted;  /* draft tokens accepted */
     int tokens;    /* tokens emitted */
-    float ms_prefill, ms_select, ms_draft, ms_verify; /* device time: stamped by the GPU's nanosecond timer in a call's kernels (first
-                                                         to last pass); in knnssd_decode and its kin CUDA events on the context's stream */
+    float ms_prefill, ms_select, ms_draft, ms_verify; /* device time: stamped by the GPU's nanosecond timer in a call's kernels (begin
+                                                         of the first pass to results handed over); in knnssd_decode and its kin CUDA events on the context's stream */
 } knnssd_stats;
 
 /*

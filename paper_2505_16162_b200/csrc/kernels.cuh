@@ -599,7 +599,8 @@ struct Delivery {
     int n_words;
     const int *err;
     int *host, *host_err;        // pinned
-    unsigned long long *stamp;   // pinned: when the call's last pass was done
+    unsigned long long *stamp;   // pinned: when all of it had been handed over
+    int *blocks_done;            // zero between launches
     // ACCEPT
     int *chain;
     const int *target;
@@ -613,7 +614,7 @@ template <bool ACCEPT> __global__ void __launch_bounds__(256) deliver_kernel(con
         if (ACCEPT && threadIdx.x == 0) accept_rows(a.chain, a.target, a.k, a.st, a.out_tokens, a.out_cap, a.accept_log, a.round_idx);
         __syncwarp();
         for (int i = threadIdx.x; i < a.n_words; i += 32) a.host[i] = *reinterpret_cast<const volatile int *>(a.words + i);
-        if (threadIdx.x == 0) { *a.host_err = *a.err; *a.stamp = globaltimer_ns(); }
+        if (threadIdx.x == 0) *a.host_err = *a.err;
     }
     const size_t first = (size_t)blockIdx.x * 256 + threadIdx.x, stride = (size_t)gridDim.x * 256;
 #pragma unroll
@@ -625,6 +626,11 @@ template <bool ACCEPT> __global__ void __launch_bounds__(256) deliver_kernel(con
         } else {
             for (size_t i = first; i < a.n[r]; i += stride) a.dst[r][i] = a.src[r][i];
         }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {                                          // the block that is done last has the time
+        __threadfence();
+        if (atomicAdd(a.blocks_done, 1) == (int)gridDim.x - 1) { *a.blocks_done = 0; *a.stamp = globaltimer_ns(); }
     }
 }
 

@@ -53,7 +53,7 @@ struct knnssd_ctx {
     float2 *part_ml = nullptr, *rope_cs = nullptr;
     double *pool_sum = nullptr, *inv_freq = nullptr;
     int *chain = nullptr, *target = nullptr, *prompt = nullptr, *out_tokens = nullptr, *accept_log = nullptr;
-    int *amax_i = nullptr, *flag = nullptr, *knn_work = nullptr;
+    int *amax_i = nullptr, *flag = nullptr, *knn_work = nullptr, *deliver_done = nullptr;
     DeviceState *state = nullptr;
     float *samp_p = nullptr, *samp_q = nullptr;   // sampled decoding: filtered distributions [kMaxRows][vocab], made on first use
     int *samp_res = nullptr;                      // [2] result of a keep-or-resample round
@@ -774,7 +774,7 @@ knnssd_status check_stream_err(knnssd_ctx *c, const char *what) {
 void free_all(knnssd_ctx *c) {
     void *ptrs[] = {c->kcache, c->vcache, c->x, c->qkv, c->attn, c->act, c->logits, c->hfinal, c->part_o, c->pooled,
                     c->cosines, c->amax_v, c->part_ml, c->rope_cs, c->pool_sum, c->inv_freq, c->chain,
-                    c->target, c->prompt, c->out_tokens, c->accept_log, c->amax_i, c->flag, c->knn_work, c->err_word, c->state,
+                    c->target, c->prompt, c->out_tokens, c->accept_log, c->amax_i, c->flag, c->knn_work, c->deliver_done, c->err_word, c->state,
                     c->ops_full, c->ops_draft, c->bar, c->gabort, c->attn_cnt, c->amax_cnt, c->mpart_o, c->mamax_v, c->mpart_ml,
                     c->mamax_i, c->trace, c->xs_x, c->xs_attn, c->xs_act, c->ssp, c->pf_x, c->pf_qkv, c->pf_ad, c->pf_aq, c->pf_af, c->pf_cs, c->pf_rinv, c->pf_ss, c->pf_part, c->small_layers, c->small_bar,
                     c->samp_p, c->samp_q, c->samp_res};
@@ -980,6 +980,7 @@ template <bool ACCEPT> cudaError_t deliver(knnssd_ctx *c, Delivery out) {
             out.n[r] = 0;
         }
     out.err = c->err_word; out.host = c->pinned; out.host_err = c->pinned + kErrWord; out.stamp = stamps_of(c) + 1;
+    out.blocks_done = c->deliver_done;
     const size_t blocks = (out.n[0] + out.n[1]) / 4 / 256 + 1;       // four floats a thread and step
     launch_chained(deliver_kernel<ACCEPT>, dim3((unsigned)(blocks < 2 * (size_t)c->n_sms ? blocks : 2 * c->n_sms)), dim3(256), 0, c->stream, out);
     c->launches++;
@@ -1074,7 +1075,8 @@ knnssd_status knnssd_init(const knnssd_config *cfg, const knnssd_weights *w, con
     ok &= dev_alloc(&c->out_tokens, (size_t)g.max_seq) == cudaSuccess;
     ok &= dev_alloc(&c->accept_log, (size_t)g.max_seq) == cudaSuccess;
     ok &= dev_alloc(&c->flag, 1) == cudaSuccess;
-    ok &= dev_alloc(&c->knn_work, 2) == cudaSuccess;
+    ok &= dev_alloc(&c->knn_work, 1) == cudaSuccess;
+    ok &= dev_alloc(&c->deliver_done, 1) == cudaSuccess;
     ok &= dev_alloc(&c->err_word, 1) == cudaSuccess;
     ok &= dev_alloc(&c->state, 1) == cudaSuccess;
     ok &= dev_alloc(&c->cosines, (size_t)(na > 0 ? na : 1)) == cudaSuccess;
@@ -1090,7 +1092,8 @@ knnssd_status knnssd_init(const knnssd_config *cfg, const knnssd_weights *w, con
     cudaMemcpyAsync(c->inv_freq, inv_freq.data(), sizeof(double) * inv_freq.size(), cudaMemcpyHostToDevice, c->stream);
     set_state_kernel<<<1, 1, 0, c->stream>>>(c->state, 0, 0, nullptr);
     cudaMemsetAsync(c->flag, 0, sizeof(int), c->stream);
-    cudaMemsetAsync(c->knn_work, 0, 2 * sizeof(int), c->stream);
+    cudaMemsetAsync(c->knn_work, 0, sizeof(int), c->stream);
+    cudaMemsetAsync(c->deliver_done, 0, sizeof(int), c->stream);
     cudaMemsetAsync(c->err_word, 0, sizeof(int), c->stream);
     // token buffers start at a valid id, so that a pass that ends early never leaves garbage ids behind
     cudaMemsetAsync(c->chain, 0, sizeof(int) * (kMaxRows + 1), c->stream);
