@@ -9,8 +9,8 @@
 // (fp64 additions and products 58), so fp64 arithmetic for every element and cluster made the assignment 15x slower than its memory
 // traffic, while this form keeps ~1e-8 relative accuracy (error of a
 // distance^2 of ~1e3: ~1e-5, four orders below the gaps that decide nearest centroids and nearest members).  A round
-// reads the points twice (assignment, centroid sums).  Every reduction has a fixed order: results do not depend on
-// timing.
+// reads the points twice (assignment, centroid sums).  Every reduction has a fixed order, given by the sizes: results depend neither on
+// timing nor on the device's share of SMs.
 #pragma once
 
 #include "kernels.cuh"
@@ -172,13 +172,14 @@ __global__ void __launch_bounds__(256, NC <= 8 ? 3 : 2) assign_kernel(const floa
     }
 }
 
-// Slices of the centroid sums: at least 64 points each, at most 64 slices, and as many as keep all blocks resident (six on an SM) if that is
-// fewer: then the sorted form runs.
-constexpr int SUM_BLOCKS = 6;
-inline int sum_slices(int N, int d, int n_sms, bool &sorted) {
+// Slices of the centroid sums: at least 64 points each, at most 64 slices, and as many as keep all blocks resident (six on each of 148 SMs) if
+// that is fewer: then the sorted form runs.  N and d decide, not the SMs that the process has got: the slices are the order of the
+// additions, and the centroids' last bits are the same on a part of a GPU.
+constexpr int SUM_BLOCKS = 6 * 148;
+inline int sum_slices(int N, int d, bool &sorted) {
     int S = (N + 63) / 64;
     if (S > 64) S = 64;
-    const int cols = (d + 255) / 256, most = SUM_BLOCKS * n_sms / cols;
+    const int cols = (d + 255) / 256, most = SUM_BLOCKS / cols;
     sorted = S > most;
     return !sorted ? S : most > 1 ? most : 1;
 }

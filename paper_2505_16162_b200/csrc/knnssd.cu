@@ -1810,7 +1810,7 @@ knnssd_status knnssd_build_anchors(const float *x_dev, int n_points, int d, int 
     const int N = n_points, n = n_clusters;
     const int sms = sm_count();
     bool sorted = false;
-    const int S = anchors::sum_slices(N, d, sms, sorted);
+    const int S = anchors::sum_slices(N, d, sorted);
     const int per = (N + S - 1) / S;
     const int ld = (d + 3) / 4 * 4;                 // row stride of the fp32 centroids
     double *mu = nullptr, *dist = nullptr, *part = nullptr;

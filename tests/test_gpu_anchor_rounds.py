@@ -59,3 +59,25 @@ def test_sums_of_slices_that_are_sorted_by_cluster(n_points, d, n):
     """More blocks of sums than are resident: longer slices, taken cluster by cluster - past 256 points, with clusters that have no point
     in a slice, and all points in one."""
     _run(n_points, d, n, 3, 4, 11 + n, 3.0)
+
+
+@pytest.mark.parametrize("n_points,d,n", [(1301, 3585, 3), (700, 130, 16), (1301, 20001, 3), (600, 60000, 1), (203, 230000, 4)])
+def test_order_of_the_sums(n_points, d, n):
+    """A centroid is the sum of its members by slices - the number of them a matter of n_points and d alone - in index order, the slices' sums
+    added in their order, over the count: to the last bit.  Both forms of the sums, the smallest and the largest slices."""
+    from paper_2505_16162_b200 import build
+    build.build()
+    from paper_2505_16162_b200 import binding as kb
+    rng = np.random.default_rng(d)
+    X = rng.normal(size=(n_points, d)).astype(np.float32)
+    got = kb.knnssd_build_anchors(torch.from_numpy(X).cuda(), torch.from_numpy(X[:n]).cuda(), 1, 1)
+    slices = min(64, -(-n_points // 64), max(1, 6 * 148 // -(-d // 256)))
+    per = -(-n_points // slices)
+    want = np.zeros((n, d))
+    for p0 in range(0, n_points, per):
+        part = np.zeros((n, d))
+        for p in range(p0, min(n_points, p0 + per)):
+            part[got["labels"][p]] += X[p]
+        want += part
+    want /= np.bincount(got["labels"], minlength=n)[:, None]
+    assert np.array_equal(got["centroids"].cpu().numpy(), want)
