@@ -54,7 +54,7 @@ def test_more_results_than_are_kept_pinned():
         _run(262200, 4, 3, 4, limit, 15, 1.5)
 
 
-@pytest.mark.parametrize("n_points,d,n", [(1301, 39999, 7), (900, 16388, 16), (1280, 3585, 1)])
+@pytest.mark.parametrize("n_points,d,n", [(1301, 39999, 7), (900, 16388, 16), (1301, 39999, 1)])
 def test_sums_of_slices_that_are_sorted_by_cluster(n_points, d, n):
     """More blocks of sums than are resident: longer slices, taken cluster by cluster - past 256 points, with clusters that have no point
     in a slice, and all points in one."""
