@@ -75,7 +75,9 @@ template <typename F> __device__ __forceinline__ bool meet_grid(const Args &a, u
             if (++polls > POLL_LIMIT) { *s_abort = 1; atomicExch(a.err, 8); break; }
     }
     __syncthreads();
-    return !*s_abort;
+    if (!*s_abort) return true;
+    asm volatile("cp.async.wait_all;" ::: "memory");      // the block leaves: its own copies have landed by then
+    return false;
 }
 
 // What the blocks of this launch write is read past the read-only path, from L2.
