@@ -342,7 +342,7 @@ def run_ours(args):
         "tokens_per_s_by_accepted_drafts": closed_form,
         "acceptance": {"mean_generated_length": M_len, "alpha": alpha, "rounds": stats["rounds"],
                        "expected_speedup_c_plain": metrics.expected_speedup(M_len, alpha, metrics.cost_coefficient(n_skip / (2 * shape.n_layers))) if alpha > 0 else None},
-        # the prompt pass inside the end-to-end steps (CUDA events around it): every linear map is one tensor-core
+        # the prompt pass inside the end-to-end steps (stamped by its first and last kernel): every linear map is one tensor-core
         # contraction over all prompt rows, activations as two bf16 terms, so 4 x rows x weights FLOP are executed
         # for the 2 x rows x weights the method asks for
         "prompt_pass": prompt_pass_report(shape, P, prefill_ms),

@@ -620,20 +620,22 @@ void run_pass_t(knnssd_ctx *c, int M, const int *tok_dev, int pos_off, const uns
 }
 
 // A model's pass is one launch of small_pass_kernel where a layer's weights are at most this much.  A kernel per operation has eight
-// times the warps on an SM to fetch them with, which is worth more than the launches from some 100 MB on.  Verification calls of 1 / 5
-// / 16 rows on four layers, one launch against a kernel per operation, us: fp32 3 MB a layer 113 / 136 / 180 against 176 / 246 / 420;
-// 48 MB 208 / 273 / 497 against 277 / 432 / 828; bf16 59 MB 331 / 419 / 935 against 326 / 586 / 1412, 190 MB 691 / 987 / 2141 against 503 / 1032 / 2700.
+// times the warps on an SM to fetch them with, which is worth more than the launches at one and five rows from somewhere above 100 MB on: the
+// line is on the safe side of that.  Verification calls of 1 / 5 / 16 rows on four layers at 96 positions, one launch against a kernel per
+// operation, us: fp32 3 MB a layer 80 / 96 / 138 against 125 / 186 / 357; 49 MB 174 / 222 / 364 against 230 / 370 / 774; bf16 45 MB 198 / 257 / 480
+// against 248 / 462 / 1087, 92 MB 293 / 407 / 818 against 311 / 469 / 1530, 184 MB 518 / 752 / 1543 against 416 / 634 / 2463.
 constexpr size_t kSmallLayerBytes = (size_t)48 << 20;
 // A head of more ids than this is streamed by launches of its own behind the pass, for the same reason.  Verification calls of 1 / 5 / 9 / 16 rows
-// on two layers, head inside / behind / a kernel per operation, us: fp32, d 1024, 8192 ids 84 / 119 / 139 / 200, 87 / 121 / 161 / 231, 108 /
-// 167 / 276 / 361; 16384 ids 94 / 140 / 162 / 229, 88 / 123 / 164 / 236, 110 / 172 / 275 / 369; 152064 ids 295 / 504 / 566 / 768, 175 / 271 / 410 /
-// 639, 197 / 319 / 527 / 814; d 256, 64000 ids 109 / 125 / 146 / 179, 62 / 88 / 131 / 179, 81 / 122 / 195 / 281; bf16, d 1024, 16384 ids 99 / 137 /
-// 159 / 218, 92 / 111 / 161 / 231, 107 / 127 / 240 / 354.
+// on two layers, head inside / behind / a kernel per operation, us: fp32, d 1024, 8192 ids 111 / 146 / 175 / 234, 118 / 155 / 203 / 270, 136 /
+// 215 / 342 / 452; 16384 ids 121 / 159 / 193 / 259, 122 / 160 / 206 / 281, 138 / 215 / 344 / 458; 152064 ids 310 / 452 / 544 / 737, 244 / 310 / 455 /
+// 690, 225 / 362 / 591 / 871; d 256, 64000 ids 93 / 120 / 144 / 186, 72 / 102 / 145 / 191, 95 / 142 / 208 / 293; bf16, d 1024, 8192 ids 80 / 112 /
+// 151 / 214, 82 / 110 / 179 / 258, 120 / 167 / 289 / 445; 16384 ids 96 / 132 / 170 / 250, 87 / 115 / 181 / 262, 125 / 173 / 292 / 450.
 constexpr int kSmallHeadIds = 12288;
 // Attention of more (head, row, split) tasks than this per SM is a launch of its own in every layer: a block per SM takes them one after the
 // other.  A layer more costs ~8 us of launches.  Four layers, one launch / launches of its own / a kernel per operation, us: 8 heads of 128, fp32,
-// 5 rows at 1000 positions 260 / 262 / 482, at 4000 410 / 363 / 576, 16 rows at 8000 1500 / 1132 / 1125; 16 heads of 64, bf16, 5 rows at 1000
-// 269 / 266 / 331, 16 at 2000 721 / 511 / 740, 16 at 8000 2095 / 995 / 1350.
+// 5 rows at 500 positions (0.5 tasks an SM) 266 / 298 / 491, at 1000 (1.1) 304 / 298 / 504, at 4000 (4.6) 447 / 397 / 647, 16 rows at 8000 (28)
+// 1522 / 1195 / 1269; 16 heads of 64, bf16, 5 rows at 500 (1.1) 255 / 251 / 348, at 1000 (2.2) 285 / 260 / 349, 16 at 2000 (14) 700 / 546 / 842,
+// 16 at 8000 (55) 1681 / 1021 / 1413.  (The two meet at one or two tasks an SM: between that and this line launches would be up to a fifth faster.)
 constexpr int kSmallTasks = 4;
 
 template <typename WT, int MT> cudaError_t launch_small_t(const small::Args &a, int grid, cudaStream_t s) {

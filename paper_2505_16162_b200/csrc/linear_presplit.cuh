@@ -38,7 +38,7 @@ __device__ __forceinline__ uint4 ld_frag4(const uint32_t *p) { return __ldcg(rei
 constexpr int SCALE_WARPS = 3;
 // (The forms of 13 .. 16 rows have no registers to give to those warps: their consumers do it.)  How the registers are split: at 40 a thread the
 // producer's warpgroup spills with both jobs in it, and a producer that spills costs 2 .. 5 % of a pass; the consumers of up to 8 rows do with
-// 216, those of 9 .. 12 lose 3 % below 224.
+// 216, those of 9 .. 12 lose 3 % below 224.  (What ptxas still spills up to 12 rows: 20 bytes in <128, 2, 3>, 4 stored and 40 read in <64, 1, 0>.)
 template <int NB, int NP> __host__ __device__ constexpr bool scales_apart() { return NB == 1 || NP == 3; }
 template <int NB, int NP> __host__ __device__ constexpr int regs_producer() { return NB == 1 ? 64 : NP == 3 ? 56 : REGS_PRODUCER; }
 template <int NB, int NP> __host__ __device__ constexpr int regs_consumer() { return NB == 1 ? 216 : NP == 3 ? 224 : REGS_CONSUMER; }
