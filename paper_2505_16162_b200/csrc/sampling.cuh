@@ -242,7 +242,8 @@ filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_tempera
             if (!(rest == rest)) { hi = lo = __float_as_uint(2.0f); break; }     // a NaN in the row: nothing is kept of it
             ones = __shfl_sync(0xffffffffu, mass, NS - 2);
             kept_mass = fmaf(top_p, rest, top_p * ones);
-            kept_rest = fmaf(top_p, rest, (top_p - 1.0f) * ones);
+            // (from 1 on nothing is left out: where the sums' rounding ends the nucleus is not searched for)
+            kept_rest = top_p >= 1.0f ? INFINITY : fmaf(top_p, rest, (top_p - 1.0f) * ones);
         }
         const unsigned below = __ballot_sync(0xffffffffu, mass < kept_rest) & (first ? 0x3fffffffu : 0xffffffffu);
         int j = below ? __ffs(below) - 1 : nc;                   // the first candidate with less than top_p above it

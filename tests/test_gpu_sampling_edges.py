@@ -43,6 +43,15 @@ def test_equal_logits_are_kept_by_lowest_id(kb, V, kept):
     assert torch.allclose(p[:kept], torch.full((kept,), 1.0 / kept, device="cuda"), rtol=1e-5)
 
 
+@pytest.mark.parametrize("V", [1000, 32000, 65536, 152064, 400000])
+def test_a_nucleus_of_everything_leaves_nothing_out(kb, V):
+    """top_p = 1: less than that is ranked before every token, however small it is next to the rounding of the sums."""
+    l = _rows(V, 3).cuda()
+    for temperature in (0.5, 1.0):
+        got = kb.knnssd_filtered_probs(l, temperature, 1.0)
+        assert bool((got > 0).all()) and torch.equal(got, kb.knnssd_filtered_probs(l, temperature, 2.0))
+
+
 def test_masked_and_unusable_rows(kb):
     l = _rows(1000, 4)
     l[1, 500:] = -float("inf")
