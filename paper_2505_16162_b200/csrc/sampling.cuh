@@ -143,9 +143,12 @@ template <int U, typename F> __device__ __forceinline__ void each_entry(const fl
 // 5 rows of 32000 and their 4 filtered after them, with the keep-or-resample round behind: 64 us a call for 54 (kernels set up under the
 // end of the one before), 9 + 8 of 152064 165 for 136; one of 152064 and a draw 52 for 48.  Error against 64 bits, rms over 2200 rows: 8.1e-8 so far,
 // 7.0e-8 so.
+// Every thread goes through the values left twice, ~35 ns each, where a pass leaves a thirtieth of them in 2 us: rows of sixteen slices, which may
+// have 512 of them, take another pass while there are more than GATHER_WIDE (one / five / nine rows of 65536 at temperature 1, top_p 0.95:
+// 28 / 34 / 44 us a call with up to 512, 23 / 24 / 32 so; 48 or 160 instead of 96: the same within 1 %, 0.2 .. 2 us more in some).
 // A row is cut into C SL slices; what comes out depends on their number, not on how many blocks share them.
 // grid = (C, rows), NT threads, probs_smem(V, C, SL) of shared memory; rows too long for it keep their values in `probs`.
-constexpr int GATHER = 32;
+constexpr int GATHER = 32, GATHER_WIDE = 96;
 template <int C, int SL> __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(NT)
 filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_temperature, float top_p, float *__restrict__ probs) {
     chain_wait();
@@ -301,7 +304,7 @@ filtered_probs_kernel(const float *__restrict__ logits, int V, float inv_tempera
             int most = 0, total = 0;
 #pragma unroll
             for (int r = 0; r < SLICES; ++r) { most = max(most, n_left[r]); total += n_left[r]; }
-            if (most <= GATHER) { gathered = total; break; }
+            if (most <= GATHER && (SLICES <= CL || total <= GATHER_WIDE)) { gathered = total; break; }
             cluster.sync();                                      // nobody writes the next values while others read these counts
         }
     }

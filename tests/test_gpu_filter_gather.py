@@ -54,6 +54,14 @@ def test_rows_at_the_line_between_eight_and_sixteen_blocks(kb, V, rows):
     _compare(kb, l, 0.5, 0.9)
 
 
+@pytest.mark.parametrize("V", [65536, 80000, 100003, 152064, 8 * 24576])
+@pytest.mark.parametrize("top_p", [0.8, 0.95])
+def test_flat_rows_of_sixteen_slices(kb, V, top_p):
+    """No block has more values left between the bounds than it may hand over, all of them together have more than are gone through."""
+    l = 1.4 * torch.randn(3, V, generator=torch.Generator().manual_seed(V))
+    _compare(kb, l, 1.0, top_p)
+
+
 @pytest.mark.parametrize("V", [32000, 65535, 65536, 100003, 152064, 8 * 24576, 8 * 24576 + 1])
 def test_a_row_does_not_depend_on_its_company(kb, V):
     """A row by itself, among five and among nine: the blocks that share it are not the same, its bits are.  Rows with nothing special
