@@ -733,10 +733,17 @@ template <bool WARPS> __global__ void __launch_bounds__(256) cosine_top1_kernel(
     float bv = -INFINITY;
     int bi = 0x7fffffff;
     bool bad = false;                                            // only a vector without a norm has left -inf
-    for (int i = tid; i < n; i += 256) {
-        const float c = __ldcg(cosines + i);
-        bad |= c == -INFINITY;
-        argmax_fold(bv, bi, c, i);
+    constexpr int U = WARPS ? 16 : 8;                            // scores in flight (no more registers than the loop above has taken)
+    for (int i0 = tid; i0 < n; i0 += U * 256) {
+        float c[U];
+#pragma unroll
+        for (int e = 0; e < U; ++e) c[e] = i0 + 256 * e < n ? __ldcg(cosines + i0 + 256 * e) : 0.f;
+#pragma unroll
+        for (int e = 0; e < U; ++e) {
+            if (i0 + 256 * e >= n) break;
+            bad |= c[e] == -INFINITY;
+            argmax_fold(bv, bi, c[e], i0 + 256 * e);
+        }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
